@@ -269,7 +269,23 @@ tt_status tt_split_check(int64_t extent, const int64_t* factors, size_t n_factor
 
 /* Run the workload once under the applied record (device pointers). */
 tt_status tt_run(tt_workload* w, const tt_tensors* t, void* cuda_stream);
-/* The same with HOST pointers: copies x, w, bias, residual to library-owned device buffers, runs, copies y back,
+
+/* One layer of a chained pass: a workload on its tensors, enqueued on stream number `lane`, after the layers whose
+ * positions in the chain are listed in `waits` (all of them in front of this one; layers on the same lane need no entry). */
+typedef struct tt_chain_step {
+    tt_workload* workload;
+    const tt_tensors* tensors;
+    const int32_t* waits;
+    int32_t n_waits;
+    int32_t lane;
+} tt_chain_step;
+/* Enqueue a whole pass of a model in one call: streams[0] is the caller's stream (a capturing one, too), the others are
+ * side streams that fork from it where they are first used and join it again at the end.  Nothing is synchronised.  On an
+ * error the layers in front of the failing one have been enqueued and the side streams joined; failed_at (may be NULL)
+ * receives its position.  Layers may share a workload; calls for the same workloads do not overlap in time (one handle,
+ * one thread), calls for different ones may run on different threads. */
+tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* streams, size_t n_streams, size_t* failed_at);
+/* tt_run with HOST pointers: copies x, w, bias, residual to library-owned device buffers, runs, copies y back,
  * synchronises.  bytes_h2d/bytes_d2h (may be NULL) receive the bytes copied. */
 tt_status tt_run_host(tt_workload* w, const tt_tensors* host, void* cuda_stream, int64_t* bytes_h2d, int64_t* bytes_d2h);
 /* The same without the final synchronisation: the copies and the kernel are only enqueued on `cuda_stream`, so calls

@@ -1,12 +1,15 @@
-"""ctypes binding of libtt.so: argument marshalling only.
+"""Python binding of libtt.so: argument marshalling only.
 
 Names mirror ``include/tt.h``.  Torch tensors supply device memory and the current
 stream; every step of the hot path runs inside the library's CUDA kernels.  There
 is no fallback: if the library is missing or no GPU is present the calls raise.
+The calls a program makes per kernel or per pass (``Workload.run``, ``run_chain``) go
+through the CPython module ``_ttcall``; the others through ctypes.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 
 from . import build as _build
@@ -65,6 +68,10 @@ class tt_tensors(C.Structure):
     _fields_ = [("x", C.c_void_p), ("w", C.c_void_p), ("bias", C.c_void_p), ("residual", C.c_void_p), ("y", C.c_void_p)]
 
 
+class tt_chain_step(C.Structure):
+    _fields_ = [("workload", C.c_void_p), ("tensors", C.POINTER(tt_tensors)), ("waits", C.POINTER(i32)), ("n_waits", i32), ("lane", i32)]
+
+
 class tt_gemm_view(C.Structure):
     _fields_ = [("batch", i32), ("gm", i32), ("gn", i32), ("gk", i32), ("flops", C.c_double), ("bytes", C.c_double)]
 
@@ -110,6 +117,7 @@ EXPORTS = {
     "tt_schedule_apply_ex": (i32, [C.c_void_p, C.POINTER(tt_schedule_record), i32, i32, C.POINTER(tt_apply_info)]),
     "tt_split_check": (i32, [C.c_int64, C.POINTER(C.c_int64), C.c_size_t, i32, C.POINTER(i32)]),
     "tt_run": (i32, [C.c_void_p, C.POINTER(tt_tensors), C.c_void_p]),
+    "tt_run_chain": (i32, [C.POINTER(tt_chain_step), C.c_size_t, C.POINTER(C.c_void_p), C.c_size_t, C.POINTER(C.c_size_t)]),
     "tt_run_host": (i32, [C.c_void_p, C.POINTER(tt_tensors), C.c_void_p, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]),
     "tt_run_host_async": (i32, [C.c_void_p, C.POINTER(tt_tensors), C.c_void_p, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]),
     "tt_workload_status": (i32, [C.c_void_p, C.c_void_p]),
@@ -145,11 +153,12 @@ EXPORTS = {
 }
 
 _lib = None
+_call = None        # the CPython module of the hot calls, loaded with the library
 
 
 def lib():
     """Load libtt.so (building it with nvcc first if the sources are newer).  Raises if that fails."""
-    global _lib
+    global _lib, _call
     if _lib is None:
         path = _build.LIB
         if _build.needs_build():
@@ -158,6 +167,11 @@ def lib():
         for name, (res, args) in EXPORTS.items():
             fn = getattr(handle, name)          # AttributeError if a declared symbol is missing
             fn.restype, fn.argtypes = res, args
+        spec = importlib.util.spec_from_file_location("_ttcall", _build.CALL_LIB)
+        call = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(call)
+        call.bind(C.cast(handle.tt_run, C.c_void_p).value, C.cast(handle.tt_run_chain, C.c_void_p).value)
+        _call = call
         _lib = handle
     return _lib
 
@@ -292,9 +306,27 @@ def tensors(x, w=None, bias=None, residual=None, y=None) -> tt_tensors:
     return t
 
 
+_torch = None
+
+
+def _raw_stream() -> int:
+    """The current stream of the current device as an integer (torch's own stream object costs a microsecond to make)."""
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch._C._cuda_getCurrentRawStream(_torch.cuda.current_device())
+
+
 def _stream():
-    import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(_raw_stream())
+
+
+def run_chain(wls, steps, tts, plan, streams):
+    """tt_run_chain over the nodes of a chain (workloads.run_chain): streams are torch streams."""
+    st, at = _call.run_chain(wls, steps, tts, plan, [s.cuda_stream for s in streams])
+    if st != TT_OK:
+        raise TTError(st, f"tt_run({wls[steps[at].kernel].name})" if at >= 0 else "tt_run_chain")
 
 
 class Workload:
@@ -304,12 +336,12 @@ class Workload:
         self.op, self.shapes, self.name, self.use_count = op, shapes, name, use_count
         h = C.c_void_p()
         _check(lib().tt_workload_create(op, C.byref(shapes), C.byref(h)), f"tt_workload_create({name})")
-        self.handle = h
+        self.handle, self.address = h, h.value
 
     def close(self):
         if getattr(self, "handle", None):
             lib().tt_workload_destroy(self.handle)
-            self.handle = None
+            self.handle = self.address = None
 
     __del__ = close
 
@@ -356,7 +388,9 @@ class Workload:
         return st, info
 
     def run(self, t: tt_tensors):
-        _check(lib().tt_run(self.handle, C.byref(t), _stream()), f"tt_run({self.name})")
+        st = _call.run(self.address or 0, t, _raw_stream())
+        if st != TT_OK:
+            raise TTError(st, f"tt_run({self.name})")
 
     def run_host(self, t: tt_tensors):
         up, down = C.c_int64(), C.c_int64()

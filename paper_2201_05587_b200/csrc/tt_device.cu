@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cstring>
+#include <mutex>
 #include <vector>
 #include "tt_internal.h"
 
@@ -122,6 +123,42 @@ tt_status encode_planes(void* out, const float* base, int W, int H, long long pl
 
 const void* pick(const tt_tensors* t, int which) { return which == 0 ? t->x : t->w; }
 
+// The events of chained passes.  A pass borrows its events and gives them back when it has been enqueued: a wait refers to
+// what was recorded when it was issued, so an event may be recorded again at once.  At most kKept stay for the next pass on
+// each device, the rest are destroyed; any thread may borrow.
+class EventLoan {
+public:
+    EventLoan() { if (cudaGetDevice(&dev_) != cudaSuccess || dev_ >= kDevices) dev_ = -1; }
+    ~EventLoan() {
+        if (taken_.empty()) return;
+        std::lock_guard<std::mutex> hold(lock());
+        for (cudaEvent_t e : taken_) {
+            if (kept()[dev_].size() < kKept) kept()[dev_].push_back(e);
+            else cudaEventDestroy(e);
+        }
+    }
+    EventLoan(const EventLoan&) = delete;
+    EventLoan& operator=(const EventLoan&) = delete;
+    cudaEvent_t get() {
+        if (dev_ < 0) return nullptr;
+        cudaEvent_t e = nullptr;
+        {
+            std::lock_guard<std::mutex> hold(lock());
+            if (!kept()[dev_].empty()) { e = kept()[dev_].back(); kept()[dev_].pop_back(); }
+        }
+        if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+        taken_.push_back(e);
+        return e;
+    }
+private:
+    static constexpr int kDevices = 64;
+    static constexpr size_t kKept = 128;
+    static std::mutex& lock() { static std::mutex m; return m; }
+    static std::vector<cudaEvent_t>* kept() { static std::vector<cudaEvent_t> k[kDevices]; return k; }
+    int dev_ = -1;
+    std::vector<cudaEvent_t> taken_;
+};
+
 }  // namespace
 
 void release_device(tt_workload* w) {
@@ -189,8 +226,13 @@ tt_status bind_device(tt_workload* w) {
 }
 
 static tt_status tensor_maps_for(tt_workload* w, const void* a_ptr, const void* b_ptr, const TmapPair** out) {
-    for (const TmapPair& e : w->tmaps)
-        if (e.a_ptr == a_ptr && e.b_ptr == b_ptr) { *out = &e; return TT_OK; }
+    // a pass calls a kernel's layers in the same order every time: the search begins behind the last hit
+    const size_t n_maps = w->tmaps.size();
+    for (size_t i = 0, at = w->tmap_next; i < n_maps; ++i, ++at) {
+        if (at >= n_maps) at = 0;
+        const TmapPair& e = w->tmaps[at];
+        if (e.a_ptr == a_ptr && e.b_ptr == b_ptr) { w->tmap_next = at + 1; *out = &e; return TT_OK; }
+    }
     const GemmArgs& g = w->plan.g;
     TmapPair e;
     std::memset(&e, 0, sizeof e);
@@ -467,6 +509,53 @@ tt_status tt_schedule_apply_ex(tt_workload* w, const tt_schedule_record* rec, in
 
 tt_status tt_run(tt_workload* w, const tt_tensors* t, void* cuda_stream) { return launch(w, t, cuda_stream); }
 
+tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* streams, size_t n_streams, size_t* failed_at) {
+    if (!steps || n_steps == 0 || !streams || n_streams == 0) return TT_ERR_INVALID_ARG;
+    // which layers some layer on another stream waits for
+    std::vector<cudaEvent_t> done(n_steps, nullptr);
+    std::vector<char> needed(n_steps, 0), used(n_streams, 0);
+    bool side = false;
+    for (size_t i = 0; i < n_steps; ++i) {
+        const tt_chain_step& s = steps[i];
+        if (failed_at) *failed_at = i;
+        if (s.lane < 0 || (size_t)s.lane >= n_streams || s.n_waits < 0 || (s.n_waits && !s.waits)) return TT_ERR_INVALID_ARG;
+        for (int32_t j = 0; j < s.n_waits; ++j) {
+            if (s.waits[j] < 0 || (size_t)s.waits[j] >= i) return TT_ERR_INVALID_ARG;
+            needed[(size_t)s.waits[j]] = 1;
+        }
+        side = side || s.lane != 0;
+    }
+    EventLoan events;
+    tt_status rc = TT_OK;
+    cudaEvent_t start = nullptr;
+    cudaStream_t main_stream = static_cast<cudaStream_t>(streams[0]);
+    if (side) {
+        start = events.get();
+        if (!start || cudaEventRecord(start, main_stream) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+    }
+    for (size_t i = 0; i < n_steps && rc == TT_OK; ++i) {
+        const tt_chain_step& s = steps[i];
+        if (failed_at) *failed_at = i;
+        cudaStream_t st = static_cast<cudaStream_t>(streams[s.lane]);
+        cudaError_t e = cudaSuccess;
+        if (s.lane != 0 && !used[(size_t)s.lane]) e = cudaStreamWaitEvent(st, start, 0);      // the side stream forks (a capture, or the caller's ordering)
+        used[(size_t)s.lane] = 1;
+        for (int32_t j = 0; j < s.n_waits && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(st, done[(size_t)s.waits[j]], 0);
+        if (e == cudaSuccess) rc = launch(s.workload, s.tensors, st);
+        if (e == cudaSuccess && rc == TT_OK && needed[i]) {
+            done[i] = events.get();
+            e = done[i] ? cudaEventRecord(done[i], st) : cudaErrorUnknown;
+        }
+        if (e != cudaSuccess) { cudaGetLastError(); rc = TT_ERR_CUDA; }
+    }
+    for (size_t l = 1; l < n_streams; ++l) {
+        if (!used[l]) continue;
+        cudaEvent_t end = events.get();
+        if (!end || cudaEventRecord(end, static_cast<cudaStream_t>(streams[l])) != cudaSuccess ||
+            cudaStreamWaitEvent(main_stream, end, 0) != cudaSuccess) { cudaGetLastError(); if (rc == TT_OK) rc = TT_ERR_CUDA; }
+    }
+    return rc;
+}
 
 tt_status tt_workload_set_constant_weights(tt_workload* w, int32_t on) {
     if (!w) return TT_ERR_INVALID_ARG;

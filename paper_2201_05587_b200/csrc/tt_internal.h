@@ -153,6 +153,7 @@ struct tt_workload {
     // device staging buffers of tt_run_host
     void* hbuf[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     size_t hbytes[5] = {0, 0, 0, 0, 0};
+    size_t tmap_next = 0;             // where the next look-up in tmaps begins
     std::vector<tt::TmapPair> tmaps;  // tensor maps encoded so far for the applied record, by operand pointers
 };
 

@@ -2867,25 +2867,41 @@ static cudaError_t launch_serialized(void (*kern)(KArgs...), dim3 grid, unsigned
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
+// How many CTAs of a kernel a device holds at once, remembered for the launch shape asked for last.
+struct ResidentCtas {
+    int dev = -1, threads = 0, smem = -1;
+    long long ctas = 0;
+    template <typename K>
+    cudaError_t get(K kern, int d, int t, int sm, long long* out) {
+        if (d != dev || t != threads || sm != smem) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+            if (e != cudaSuccess) return e;
+            int occ = 0, sm_count = 0;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, t, (size_t)sm)) != cudaSuccess) return e;
+            if ((e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, d)) != cudaSuccess) return e;
+            if (occ < 1) return cudaErrorLaunchOutOfResources;
+            dev = d; threads = t; smem = sm; ctas = (long long)sm_count * occ;
+        }
+        *out = ctas;
+        return cudaSuccess;
+    }
+};
+
 cudaError_t launch_dw_tma(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st) {
     CUtensorMap tx;
     memcpy(&tx, tmap_x, sizeof tx);
     dim3 grid(I.grid_x, 1, 1);
-    int sm_count = 148, dev_now = 0;
-    cudaGetDevice(&dev_now);
-    cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev_now);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    // resident CTAs of this instantiation, looked up once per launch shape (the query costs more than the launch)
 #define TT_DWT_CASE(RR, SS, RO, WI) \
     if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == WI) { \
-        static int attr_dev = -1; int dev = 0; cudaGetDevice(&dev); \
-        if (attr_dev != dev) { \
-            cudaError_t e = cudaFuncSetAttribute(tt_dwconv_tma_kernel<RR, SS, RO, WI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); \
-            if (e != cudaSuccess) return e; attr_dev = dev; } \
-        int occ = 0; \
-        cudaError_t eo = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, tt_dwconv_tma_kernel<RR, SS, RO, WI>, I.threads, (size_t)I.smem_bytes); \
-        if (eo != cudaSuccess) return eo; \
-        if (occ < 1) return cudaErrorLaunchOutOfResources; \
+        static thread_local ResidentCtas known; \
+        long long resident = 0; \
+        cudaError_t e = known.get(tt_dwconv_tma_kernel<RR, SS, RO, WI>, dev, I.threads, I.smem_bytes, &resident); \
+        if (e != cudaSuccess) return e; \
         /* persistent CTAs: never more than are resident at once (registers may allow fewer than shared memory does) */ \
-        grid.x = (unsigned)std::min<long long>(grid.x, (long long)sm_count * occ); \
+        grid.x = (unsigned)std::min<long long>(grid.x, resident); \
         return launch_serialized(tt_dwconv_tma_kernel<RR, SS, RO, WI>, grid, (unsigned)I.threads, (size_t)I.smem_bytes, st, tx, dw); }
     TT_DWT_CASE(3, 1, 1, 4) TT_DWT_CASE(3, 1, 2, 4) TT_DWT_CASE(3, 1, 4, 4) TT_DWT_CASE(3, 1, 1, 8) TT_DWT_CASE(3, 1, 2, 8)
     TT_DWT_CASE(3, 2, 1, 4) TT_DWT_CASE(3, 2, 2, 4) TT_DWT_CASE(3, 2, 4, 4) TT_DWT_CASE(3, 2, 1, 8) TT_DWT_CASE(3, 2, 2, 8)

@@ -446,28 +446,5 @@ def chain_lanes(steps, max_lanes=4, serial_kernels=()):
 
 def run_chain(wls, steps, tts, plan, streams):
     """Enqueue one pass of a chain: streams[0] is the caller's current stream (under stream capture: the capturing one),
-    the others are side streams that fork from it and join it again at the end."""
-    import torch
-    events, used = {}, set()
-    needed = {p for pl in plan if pl is not None for p in pl[1]}
-    start = torch.cuda.Event()
-    start.record(streams[0])
-    for i, (st, tt, pl) in enumerate(zip(steps, tts, plan)):
-        if pl is None:
-            continue
-        lane, waits = pl
-        s = streams[lane]
-        if lane != 0 and lane not in used:
-            s.wait_event(start)                           # the side stream joins (a capture, or the caller's ordering)
-        used.add(lane)
-        for p in waits:
-            s.wait_event(events[p])
-        with torch.cuda.stream(s):
-            wls[st.kernel].run(tt)
-        if i in needed:
-            events[i] = torch.cuda.Event()
-            events[i].record(s)
-    for lane in sorted(used - {0}):
-        e = torch.cuda.Event()
-        e.record(streams[lane])
-        streams[0].wait_event(e)
+    the others are side streams that fork from it and join it again at the end.  One native call walks the whole chain."""
+    B.run_chain(wls, steps, tts, plan, streams)

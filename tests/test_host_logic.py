@@ -574,3 +574,18 @@ def test_compensated_precision_is_kept_where_it_exists_and_reported_elsewhere():
     assert st == B.TT_OK and info.legal.precision == 1 and info.legal.persistent == 0 and info.changed & B.TT_CHG_FORM
     bad = B.make_record(B.TT_FAMILY_GEMM_TC, precision=2)
     assert dense.check(bad)[0] == B.TT_ERR_INVALID_SCHEDULE
+
+
+@pytest.mark.parametrize("lanes,waits,want", [
+    ((0, 0), ((), ()), B.TT_ERR_NOT_APPLIED),       # well formed: stops at the first layer, which has no record applied
+    ((0, 1), ((), (1,)), B.TT_ERR_INVALID_ARG),     # a layer that waits for itself
+    ((0, 2), ((), (0,)), B.TT_ERR_INVALID_ARG),     # a lane without a stream
+])
+def test_run_chain_checks_its_arguments(lanes, waits, want):
+    wl = W._dense(8, 16, 8).workload()
+    t = B.tt_tensors()
+    ws = [(ctypes.c_int32 * max(len(w), 1))(*w) for w in waits]
+    steps = (B.tt_chain_step * 2)(*[B.tt_chain_step(wl.handle, ctypes.pointer(t), w, len(ids), lane) for w, ids, lane in zip(ws, waits, lanes)])
+    at = ctypes.c_size_t(99)
+    assert B.lib().tt_run_chain(steps, 2, (ctypes.c_void_p * 2)(), 2, ctypes.byref(at)) == want
+    assert at.value == (0 if want == B.TT_ERR_NOT_APPLIED else 1)
