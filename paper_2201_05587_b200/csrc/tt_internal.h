@@ -107,6 +107,8 @@ struct DwArgs {
 struct RowArgs {
     const float* x; float* y; long long rows; int cols; float scale;
     int lanes_per_row, rows_per_cta, vec;
+    int aligned;       // x and y start on 16-byte boundaries
+    unsigned* status; unsigned long long wait_ns;   // the workload's status word and wait limit
 };
 
 // Host-side plan of an applied record.

@@ -951,3 +951,14 @@ def test_compensated_products_come_within_fp32_accumulation_of_the_exact_result(
         y3 = run_spec(spec, tc(precision=1, **kw), a, ref)
         e0, e3 = util.rel_l2(y0, ref), util.rel_l2(y3, ref)
         assert e3 <= 2e-5 and e3 * 20 <= e0, (spec.name, kw, e0, e3)
+
+
+@pytest.mark.parametrize("cols", [1, 2, 3, 5, 31, 33, 63, 127, 129, 197, 255, 257, 1023, 1025, 2045, 2047, 2049, 2051])
+def test_softmax_ragged_rows(cols):
+    """Rows that start at every offset inside a 16-byte group, up to the longest row that stays in registers and just
+    beyond it; lanes per row from 1 to 32; the last rows fill no whole chunk."""
+    spec = W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(5, 7, cols, scale=0.125), 1, f"softmax_35x{cols}", "bert")
+    a = W.make_inputs(spec, 11)
+    ref = util.oracle_ref(spec, a)
+    for bx in (1, 4, 16, 32):
+        run_spec(spec, B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=bx, block_y=8, vec_width=4), a, ref, ref_elem=ref)
