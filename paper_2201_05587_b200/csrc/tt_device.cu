@@ -16,11 +16,10 @@ cudaError_t launch_gemm(const tt_apply_info& I, const GemmArgs& g, const void* t
 cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st);
 cudaError_t launch_dw_tma(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st);
 cudaError_t launch_row(const tt_apply_info& I, const RowArgs& row, cudaStream_t st);
-cudaError_t gemm_cluster_fits(int smem_bytes, int cluster, int* fits);
+cudaError_t gemm_cluster_fits(const GemmArgs& g, int smem_bytes, int* fits);
 cudaError_t launch_repack(const float* w, float* out, int kout, int C, int RS, int CB, cudaStream_t st);
 cudaError_t launch_floor(const tt_apply_info& I, int cluster, cudaStream_t st);
-cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
-                           cudaStream_t st);
+cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const TmapPair& maps, cudaStream_t st);
 
 namespace {
 
@@ -72,20 +71,34 @@ tt_status encode_operand(void* out, const float* base, int K, int rows, int batc
     return r == CUDA_SUCCESS ? TT_OK : TT_ERR_CUDA;
 }
 
-// Row-contiguous operand [batch][K][rows] (element (row, k) at k * ks + row) -> 3-D tensor map without swizzle,
-// box = [box_rows, box_k, 1]: the staging boxes of the persistent kernel.
-tt_status encode_operand_mn(void* out, const float* base, int rows, int K, int batch, long long ks, long long bs, bool batched,
-                            int box_rows, int box_k) {
+// Row-contiguous operand [batch][K][rows] (element (row, k) at k * ks + row) -> 3-D tensor map, box = [32 rows, box_k, 1]: the
+// 128-byte lines of an MN-major tile, swizzled in 32-byte atoms as kind::tf32 reads them.
+tt_status encode_operand_mn(void* out, const float* base, int rows, int K, int batch, long long ks, long long bs, bool batched, int box_k) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return TT_ERR_CUDA;
     if ((reinterpret_cast<uintptr_t>(base) & 15u) != 0) return TT_ERR_INVALID_ARG;
     const cuuint64_t nb = batched ? (cuuint64_t)batch : 1;
     cuuint64_t dims[3] = {(cuuint64_t)rows, (cuuint64_t)K, nb};
     cuuint64_t strides[2] = {(cuuint64_t)ks * 4, (cuuint64_t)(batched ? bs : (long long)K * ks) * 4};
-    cuuint32_t box[3] = {(cuuint32_t)box_rows, (cuuint32_t)box_k, 1};
+    cuuint32_t box[3] = {32, (cuuint32_t)box_k, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = fn(reinterpret_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims,
-                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? TT_OK : TT_ERR_CUDA;
+}
+
+// A matrix [batch][rows][cols] (rows `pitch` elements apart) in 32 x 32 blocks: the read-out's stores and residual loads.
+tt_status encode_blocks(void* out, const float* base, int cols, int rows, int batch, long long pitch, long long bs, bool batched, bool swizzled) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return TT_ERR_CUDA;
+    const cuuint64_t nb = batched ? (cuuint64_t)batch : 1;
+    cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, nb};
+    cuuint64_t strides[2] = {(cuuint64_t)pitch * 4, (cuuint64_t)(batched ? bs : (long long)rows * pitch) * 4};
+    cuuint32_t box[3] = {32, 32, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(reinterpret_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims,
+                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzled ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? TT_OK : TT_ERR_CUDA;
 }
@@ -177,7 +190,7 @@ tt_status bind_device(tt_workload* w) {
     if (w->family == TT_FAMILY_GEMM_TC && w->plan.g.cluster) {
         // a cluster whose CTAs cannot be resident together can never launch: an invalid pair, not a device error
         int fits = 0;
-        if (gemm_cluster_fits(w->plan.info.smem_bytes, w->plan.g.cluster, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+        if (gemm_cluster_fits(w->plan.g, w->plan.info.smem_bytes, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
         if (!fits) return TT_ERR_RESOURCE;
     }
     const size_t need = (size_t)w->plan.info.workspace_bytes;
@@ -196,7 +209,7 @@ tt_status bind_device(tt_workload* w) {
         if (cudaMalloc(reinterpret_cast<void**>(&w->status_word), 512) != cudaSuccess) { cudaGetLastError(); return TT_ERR_OOM; }
         if (cudaMemset(w->status_word, 0, 512) != cudaSuccess) return TT_ERR_CUDA;
     }
-    if (w->op == TT_OP_CONV2D && !w->plan.g.tap_major && !w->plan.g.persistent) {
+    if (w->family == TT_FAMILY_GEMM_TC && (w->plan.g.a_mode == OPM_IM2COL || w->plan.g.b_mode == OPM_IM2COL)) {
         // reduction-index table of the applied record: byte offset of (c, r, s) inside the slab, channel counted
         // from 0 (the kernel rebases it per chunk); indices past K point at the last channel, whose products meet
         // zero-filled filter values
@@ -225,18 +238,19 @@ tt_status bind_device(tt_workload* w) {
     return TT_OK;
 }
 
-static tt_status tensor_maps_for(tt_workload* w, const void* a_ptr, const void* b_ptr, const TmapPair** out) {
+static tt_status tensor_maps_for(tt_workload* w, const GemmArgs& g, const void* a_ptr, const void* b_ptr, const TmapPair** out) {
+    const void* y_ptr = g.epi_tma ? g.y : nullptr;
+    const void* r_ptr = g.res_tma ? g.residual : nullptr;
     // a pass calls a kernel's layers in the same order every time: the search begins behind the last hit
     const size_t n_maps = w->tmaps.size();
     for (size_t i = 0, at = w->tmap_next; i < n_maps; ++i, ++at) {
         if (at >= n_maps) at = 0;
         const TmapPair& e = w->tmaps[at];
-        if (e.a_ptr == a_ptr && e.b_ptr == b_ptr) { w->tmap_next = at + 1; *out = &e; return TT_OK; }
+        if (e.a_ptr == a_ptr && e.b_ptr == b_ptr && e.y_ptr == y_ptr && e.r_ptr == r_ptr) { w->tmap_next = at + 1; *out = &e; return TT_OK; }
     }
-    const GemmArgs& g = w->plan.g;
     TmapPair e;
     std::memset(&e, 0, sizeof e);
-    e.a_ptr = a_ptr; e.b_ptr = b_ptr;
+    e.a_ptr = a_ptr; e.b_ptr = b_ptr; e.y_ptr = y_ptr; e.r_ptr = r_ptr;
     // A gathered operand keeps an all-zero map in its parameter slot; the kernel never issues a TMA load on it.
     tt_status st = TT_OK;
     if (g.a_mode == OPM_TMA)
@@ -249,11 +263,18 @@ static tt_status tensor_maps_for(tt_workload* w, const void* a_ptr, const void* 
     if (st != TT_OK) return st;
     if (g.a_mode == OPM_TMA_MN)
         st = encode_operand_mn(e.a, static_cast<const float*>(a_ptr), g.M, g.K, g.batch, g.a_ks, g.a_bs, g.a_tma_batched != 0,
-                               kHwTileM, g.tile_k);
+                               g.tile_k);
     if (st != TT_OK) return st;
     if (g.b_mode == OPM_TMA_MN)
         st = encode_operand_mn(e.b, static_cast<const float*>(b_ptr), g.N, g.K, g.batch, g.b_ks, g.b_bs, g.b_tma_batched != 0,
-                               g.b_rows_cta, g.tile_k);
+                               g.tile_k);
+    if (st != TT_OK) return st;
+    // the output (and the residual) in blocks: along the tile's columns, or, for a residual of outputs that are contiguous
+    // along its rows, transposed
+    if (y_ptr) st = encode_blocks(e.y, static_cast<const float*>(y_ptr), g.N, g.M, g.batch, g.y_ms, g.y_bs, g.y_tma_batched != 0, true);
+    if (st == TT_OK && r_ptr)
+        st = g.epi_tma ? encode_blocks(e.r, static_cast<const float*>(r_ptr), g.N, g.M, g.batch, g.y_ms, g.y_bs, g.y_tma_batched != 0, true)
+                       : encode_blocks(e.r, static_cast<const float*>(r_ptr), g.M, g.N, g.batch, g.y_ns, g.y_bs, g.y_tma_batched != 0, false);
     if (st != TT_OK) return st;
     if (g.slab_tma) {
         const float* img = static_cast<const float*>(g.a_mode == OPM_IM2COL ? a_ptr : b_ptr);
@@ -293,9 +314,6 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
             }
             a_ptr = w->workspace;
         }
-        const TmapPair* maps = nullptr;
-        tt_status s = tensor_maps_for(w, a_ptr, b_ptr, &maps);
-        if (s != TT_OK) return s;
         g.a = static_cast<const float*>(a_ptr);
         g.b = static_cast<const float*>(b_ptr);
         g.y = static_cast<float*>(t->y);
@@ -305,7 +323,8 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
         g.counters = reinterpret_cast<unsigned*>(static_cast<char*>(w->workspace) + p.partial_bytes);
         g.status = w->status_word;
         if ((reinterpret_cast<uintptr_t>(t->y) & 15u) != 0 ||
-            (g.residual && (reinterpret_cast<uintptr_t>(g.residual) & 15u) != 0)) g.vec_store = 0;
+            (g.residual && (reinterpret_cast<uintptr_t>(g.residual) & 15u) != 0)) g.vec_store = g.epi_tma = g.res_tma = 0;
+        if (!g.residual) g.res_tma = 0;
         if (g.bias && (reinterpret_cast<uintptr_t>(g.bias) & 15u) == 0) g.vec_store |= 2;
         g.ktab_dev = w->ktab_dev;
         g.wait_ns = w->wait_ns;
@@ -315,7 +334,10 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
             if (p.a_tensor == 1 && g.a_mode == OPM_TMA) g.w_operand = 1;
             else if (p.b_tensor == 1 && g.b_mode == OPM_TMA) g.w_operand = 2;
         }
-        e = g.persistent ? launch_gemm_ps(p.info, g, maps->a, maps->b, maps->x, st) : launch_gemm(p.info, g, maps->a, maps->b, maps->x, st);
+        const TmapPair* maps = nullptr;
+        const tt_status s = tensor_maps_for(w, g, a_ptr, b_ptr, &maps);
+        if (s != TT_OK) return s;
+        e = g.persistent ? launch_gemm_ps(p.info, g, *maps, st) : launch_gemm(p.info, g, maps->a, maps->b, maps->x, st);
     } else if (w->family == TT_FAMILY_DW_SIMT) {
         DwArgs d = p.dw;
         d.x = static_cast<const float*>(t->x); d.w = static_cast<const float*>(t->w);
@@ -971,7 +993,7 @@ extern "C" tt_status tt_dense_static_scratch(const void* x, const void* w, const
     if (plan.g.cluster) {
         // as in tt_schedule_apply: a split-K cluster whose CTAs cannot be resident together is an invalid pair
         int fits = 0;
-        if (gemm_cluster_fits(plan.info.smem_bytes, plan.g.cluster, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+        if (gemm_cluster_fits(plan.g, plan.info.smem_bytes, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
         if (!fits) return TT_ERR_RESOURCE;
     }
     unsigned char* base = nullptr;

@@ -21,6 +21,7 @@ uint64_t fnv1a(const void* data, size_t n, uint64_t h = 1469598103934665603ull) 
 }
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
+long long round_up64(long long v, long long m) { return (v + m - 1) / m * m; }
 int pow2_ceil(int v) { int p = 1; while (p < v) p <<= 1; return p; }
 int pow2_floor(int v) { int p = 1; while (p * 2 <= v) p <<= 1; return p; }
 
@@ -298,7 +299,10 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
             can = can && (o.nn % 4) == 0;
         if (persistent && !can) { if (strict) return TT_ERR_INVALID_SCHEDULE; persistent = false; changed |= TT_CHG_FORM; }
     }
-    const bool mn_operand = persistent && (w->op == TT_OP_CONV2D || (w->op == TT_OP_BATCH_MATMUL && !w->sh.trans_b));
+    // An operand whose row index is the contiguous one, in 16-byte steps: TMA boxes that the tensor core reads MN-major.
+    const bool mn_operand = w->op == TT_OP_CONV2D
+        ? w->sh.r == 1 && w->sh.s == 1 && w->sh.stride_h == 1 && w->sh.stride_w == 1 && w->sh.pad_h == 0 && w->sh.pad_w == 0 && ((long long)w->sh.h * w->sh.w) % 4 == 0
+        : w->op == TT_OP_BATCH_MATMUL && !w->sh.trans_b && w->sh.nn % 4 == 0;
     int cg = rec->cta_group == 2 ? 2 : 1;
     if (cg == 2 && (!persistent || mn_operand || tn < 32)) { if (strict) return TT_ERR_INVALID_SCHEDULE; cg = 1; changed |= TT_CHG_FORM; }
     L.persistent = persistent ? 1 : 0;
@@ -325,7 +329,8 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
 
     const int atom_k = std::min(tk, 32), n_atoms = tk / atom_k, row_bytes = atom_k * 4;
     const unsigned a_stage = (unsigned)n_atoms * kHwTileM * row_bytes;
-    const unsigned b_stage = (unsigned)n_atoms * (tn / cg) * row_bytes;
+    // an MN-major operand B takes whole boxes of 32 rows
+    const unsigned b_stage = swap || !mn_operand ? (unsigned)n_atoms * (tn / cg) * row_bytes : (unsigned)round_up(tn, 32) * tk * 4;
     if (persistent) {
         // ---- the persistent form: its own shared-memory plan, grid and arguments ----
         const tt_shapes& o = w->sh;
@@ -333,24 +338,36 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
         // logical operands U (rows i of the output) and V (columns j): which of them is row-contiguous
         const bool u_mn = false, v_mn = conv1 || nn;
         const bool a_mn = swap ? v_mn : u_mn, b_mn = swap ? u_mn : v_mn;
-        const unsigned stg_a = a_mn ? (unsigned)(tk * kHwTileM * 4) : 0u, stg_b = b_mn ? (unsigned)(tk * tn * 4) : 0u;
-        const long long epi = 4ll * 32 * 36 * 4;
-        // the staging ring of a row-contiguous operand has its own depth (record field slab_tiles; 0 = as deep as fits,
-        // at most 8): it is what is in flight from DRAM, while the K-major stages only decouple transposing from multiplying
+        // How many stages: the record's, or, with a row-contiguous operand (whose boxes come from memory one after the other),
+        // what the record field slab_tiles asks for; 0 = as many as fit, at most 8.
         if (rec->slab_tiles < 0) return TT_ERR_INVALID_SCHEDULE;
-        const bool any_stg = stg_a + stg_b > 0;
-        int sd = any_stg ? (rec->slab_tiles == 0 ? kMaxStages : std::min(kMaxStages, rec->slab_tiles)) : 0;
-        long long smem_p = 0;
-        for (;;) {
-            smem_p = (long long)st * (a_stage + b_stage) + (long long)sd * (stg_a + stg_b) + epi + 1024;
-            if (smem_p <= kDynSmemLimit) break;
-            if (any_stg && sd > 1 && (rec->slab_tiles == 0 || !strict) && (rec->slab_tiles == 0 || sd >= st)) { --sd; continue; }
-            if (strict || st <= 1) break;
-            --st; changed |= TT_CHG_STAGES;
+        const bool mn = a_mn || b_mn;
+        const long long stage = (long long)a_stage + b_stage;
+        // Read-out staging: eight warps with three (a residual passes through them) or two 32 x 32 blocks each, fewer where
+        // the record's stages need the room; never less than four warps with one block (5 KB, the width the unaligned
+        // read-out's transposition takes).
+        struct { int warps, bufs; } epi[] = {{8, 3}, {8, 2}, {4, 3}, {4, 2}, {8, 1}, {4, 1}};
+        auto warp_bytes = [](int bufs) { return bufs == 1 ? 5120ll : bufs * 4096ll; };
+        const bool res = w->sh.has_residual != 0;
+        int ew = 4, eb = 1;
+        const int want = !mn ? st : (rec->slab_tiles == 0 ? kMaxStages : std::min(kMaxStages, std::max(st, rec->slab_tiles)));
+        auto total = [&](int stages, int warps, int bufs) { return round_up64(stages * stage, 1024) + warps * warp_bytes(bufs) + 1024; };
+        while (!strict && st > 1 && total(st, 4, 1) > kDynSmemLimit) { --st; changed |= TT_CHG_STAGES; }
+        if (mn && rec->slab_tiles != 0 && want > st && total(want, 4, 1) > kDynSmemLimit) {
+            if (strict) return TT_ERR_INVALID_SCHEDULE;
+            changed |= TT_CHG_SLAB;
         }
-        if (any_stg && rec->slab_tiles != 0 && sd != rec->slab_tiles) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_SLAB; }
-        if (!any_stg && rec->slab_tiles != 0) changed |= TT_CHG_SLAB;
-        L.stages = st; L.split_k = 1; L.acc_split = 1; L.slab_tiles = (any_stg && rec->slab_tiles != 0) ? sd : 0; L.ctas_per_sm = 1;
+        // with a free depth the read-out's ring comes first, as long as three stages (or the record's) stay in flight
+        const int keep = rec->slab_tiles == 0 && mn ? std::max(st, 3) : std::max(want, st);
+        for (const auto& o : epi) {
+            if (!res && o.bufs == 3) continue;
+            if (total(keep, o.warps, o.bufs) <= kDynSmemLimit || (o.warps == 4 && o.bufs == 1)) { ew = o.warps; eb = o.bufs; break; }
+        }
+        int depth = std::max(want, st);
+        while (depth > st && total(depth, ew, eb) > kDynSmemLimit) --depth;
+        const long long smem_p = total(depth, ew, eb);
+        if (!mn && rec->slab_tiles != 0) changed |= TT_CHG_SLAB;
+        L.stages = st; L.split_k = 1; L.acc_split = 1; L.slab_tiles = (mn && rec->slab_tiles != 0) ? depth : 0; L.ctas_per_sm = 1;
         if (rec->ctas_per_sm == 2) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_FORM; }
         if (strict && (changed & ~TT_CHG_TILE_M)) return TT_ERR_INVALID_SCHEDULE;
         const int rows_m = kHwTileM * cg;
@@ -370,21 +387,19 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
         GemmArgs& g = plan->g;
         g = GemmArgs{};
         g.M = M; g.N = N; g.K = K; g.batch = B;
-        g.tile_n = tn; g.tile_k = tk; g.stages = st;
+        g.tile_n = tn; g.tile_k = tk; g.stages = depth;
         g.k_tiles = k_tiles; g.k_tiles_per_split = k_tiles; g.split_k = 1;
         g.tiles_m = tiles_m; g.tiles_n = tiles_n; g.raster = L.raster;
         g.atom_k = atom_k; g.n_atoms = n_atoms; g.row_bytes = row_bytes;
         g.swz_mask = row_bytes == 128 ? 7 : (row_bytes == 64 ? 3 : 1);
         g.a_stage_bytes = a_stage; g.b_stage_bytes = b_stage;
         g.tmem_cols = (unsigned)I.tmem_cols; g.n_acc = 1; g.cluster = 0;
-        g.idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(tn >> 3) << 17) | ((unsigned)(rows_m >> 4) << 24);
+        g.idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(tn >> 3) << 17) | ((unsigned)(rows_m >> 4) << 24) |
+                  (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u);          // (an MN-major operand is read transposed)
         g.persistent = 1; g.cta_group = cg; g.total_tiles = (int)units;
         g.a_mn = a_mn; g.b_mn = b_mn; g.b_rows_cta = tn / cg;
-        g.stg_depth = std::max(sd, 1);
-        g.a_stg_off = (unsigned)((long long)st * (a_stage + b_stage));
-        g.b_stg_off = g.a_stg_off + (unsigned)sd * stg_a;
-        g.stg_a_bytes = stg_a; g.stg_b_bytes = stg_b;
-        g.epi_off = g.b_stg_off + (unsigned)sd * stg_b;
+        g.epi_off = (unsigned)round_up64(depth * stage, 1024);
+        g.epi_warps = ew; g.epi_bufs = eb; g.epi_warp_bytes = (unsigned)warp_bytes(eb);
         struct Opnd { int mode; long long rs, ks, bs; int batched; } U{}, V{};
         long long y_is, y_js, y_bs;
         int bias_on;
@@ -413,8 +428,14 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
         g.y_ms = swap ? y_js : y_is; g.y_ns = swap ? y_is : y_js; g.y_bs = y_bs;
         g.bias_mode = o.has_bias ? (swap ? 3 - bias_on : bias_on) : 0;
         g.act = o.act;
-        g.tx_bytes = (a_mn ? 0 : a_stage) + (b_mn ? 0 : b_stage);
+        g.tx_bytes = a_stage + b_stage;
         g.vec_store = (g.y_ns == 1 && g.y_ms % 4 == 0 && g.y_bs % 4 == 0) ? 1 : 0;
+        // TMA read-out: 16-byte rows, whole 32-column blocks (a narrower last block would write its neighbour's columns), and
+        // two ring blocks per warp, so that one fills while the other is sent (with one the last tile's read-out, which nothing
+        // hides, took twice as long: dense 1854 x 680 -> 1248 14.3 -> 16.0 us)
+        g.y_tma_batched = y_bs != 0;
+        g.epi_tma = g.vec_store && tn % 32 == 0 && g.y_ms != 1 && eb >= 2;
+        g.res_tma = res && eb >= 2 && (g.epi_tma || (g.y_ms == 1 && g.y_ns % 4 == 0 && g.y_bs % 4 == 0));
         return TT_OK;
     }
     // Shared memory: pipeline buffers (reused by the epilogue as a 32 x 36-float staging area per warp), then for
@@ -435,7 +456,8 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
     // main loop): per OTHER split, this CTA's band of the tile -- rows x (tile_n + 4) or columns x 128 floats
     const long long red_bytes = cluster ? (4 * std::max<long long>((long long)(sk - 1) * ((kHwTileM + sk - 1) / sk) * (tn + 4),
                                                                     (long long)(sk - 1) * ((tn + sk - 1) / sk) * kHwTileM) + 127) / 128 * 128 : 0;
-    const bool conv = w->op == TT_OP_CONV2D;
+    // A pointwise convolution on images of 16-byte multiples needs no slab: its pixels are an MN-major operand.
+    const bool conv = w->op == TT_OP_CONV2D && !mn_operand;
     const long long ktab = conv ? (((long long)per_split * tk * 4 + 127) / 128) * 128 : 0;
     int sl_tiles = 0, sl_nbuf = 0, sl_wp = 0, sl_gap = 0, sl_chpitch = 0, sl_in_rows = 0, sl_rstep = 1;
     long long sl_buf_bytes = 0, chp = 0;
@@ -567,8 +589,8 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
     g.two_per_sm = L.ctas_per_sm == 2;
     g.x3 = x3 ? 1 : 0;
     g.b_rows_cta = tn; g.cta_group = 1;
-    // Instruction descriptor, kind::tf32: D = F32 (bits 4-5 = 1), A and B = TF32 (bits 7-9, 10-12 = 2), both
-    // K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28.
+    // Instruction descriptor, kind::tf32: D = F32 (bits 4-5 = 1), A and B = TF32 (bits 7-9, 10-12 = 2), K-major or
+    // (bits 15, 16 = 1) MN-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28.
     g.idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(tn >> 3) << 17) | ((unsigned)(kHwTileM >> 4) << 24);
     // Operands of the logical contraction Y[b][i][j] = sum_k U[b][i][k] V[b][j][k], then the optional swap.
     struct Opnd { int mode; long long rs, ks, bs; int batched; } U{}, V{};
@@ -576,8 +598,10 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
     int bias_on;   // 1: bias indexed by i, 2: by j
     const bool k4 = (K % 4) == 0;
     if (w->op == TT_OP_CONV2D) {
+        const long long hw = (long long)s.h * s.w;
         U = {k4 ? OPM_TMA : OPM_GATHER_K, K, 1, 0, 0};                         // filters [k][c*r*s], shared by images
-        V = {OPM_IM2COL, 0, 0, (long long)s.c * s.h * s.w, 1};                 // pixels x (c,r,s) gathered from NCHW
+        if (mn_operand) V = {OPM_TMA_MN, 1, hw, (long long)s.c * hw, 1};       // pixel index contiguous, channels hw apart
+        else V = {OPM_IM2COL, 0, 0, (long long)s.c * hw, 1};                   // pixels x (c,r,s) gathered from NCHW
         y_is = (long long)P * Q; y_js = 1; y_bs = (long long)s.k * P * Q; bias_on = 1;
     } else if (w->op == TT_OP_DENSE) {
         U = {k4 ? OPM_TMA : OPM_GATHER_K, K, 1, 0, 0};
@@ -586,7 +610,7 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
     } else {
         U = {k4 ? OPM_TMA : OPM_GATHER_K, K, 1, (long long)s.m * K, 1};
         if (s.trans_b) V = {k4 ? OPM_TMA : OPM_GATHER_K, K, 1, (long long)s.nn * K, 1};
-        else V = {OPM_GATHER_ROWS, 1, s.nn, (long long)s.nn * K, 1};           // w[b][k][j]: rows j are contiguous
+        else V = {mn_operand ? OPM_TMA_MN : OPM_GATHER_ROWS, 1, s.nn, (long long)s.nn * K, 1};   // w[b][k][j]: rows j are contiguous
         y_is = s.nn; y_js = 1; y_bs = (long long)s.m * s.nn; bias_on = 2;
     }
     const int u_tensor = w->op == TT_OP_CONV2D ? 1 : 0;       // conv: U is the filter tensor; dense/bmm: U is x
@@ -601,7 +625,8 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
     g.act = s.act;
     g.C = s.c; g.H = s.h; g.W = s.w; g.R = s.r; g.S = s.s; g.Q = Q;
     g.sh = s.stride_h; g.sw = s.stride_w; g.ph = s.pad_h; g.pw = s.pad_w;
-    g.tx_bytes = (A.mode == OPM_TMA ? a_stage : 0) + (Bo.mode == OPM_TMA ? b_stage : 0);
+    g.idesc |= (A.mode == OPM_TMA_MN ? 1u << 15 : 0u) | (Bo.mode == OPM_TMA_MN ? 1u << 16 : 0u);
+    g.tx_bytes = (A.mode == OPM_TMA || A.mode == OPM_TMA_MN ? a_stage : 0) + (Bo.mode == OPM_TMA || Bo.mode == OPM_TMA_MN ? b_stage : 0);
     g.vec_store = (g.y_ns == 1 && g.y_ms % 4 == 0 && g.y_bs % 4 == 0) ? 1 : 0;
     return TT_OK;
 }

@@ -23,8 +23,8 @@ enum OperandMode : int {
     OPM_IM2COL = 3,       // rows are output pixels, k = (c, r, s): expanded from a slab of NCHW input rows
     OPM_IM2COL_T = 4,     // rows are padded-linear output pixels, k = (32-channel block, tap, channel): every tap's tile
                           // is a shifted view of a pixel-major slab in shared memory (nothing is staged per tile)
-    OPM_TMA_MN = 5        // persistent kernel: the row index is the contiguous one in memory; [tile_k][rows] boxes arrive by
-                          // TMA in a staging ring and are transposed into the K-major stage by four warps
+    OPM_TMA_MN = 5        // the row index is the contiguous one in memory: [tile_k][32 rows] boxes by TMA, multiplied as
+                          // they lie (an MN-major tile)
 };
 
 // Device-side arguments of the GEMM_TC kernel (plain data, passed by value).
@@ -80,12 +80,16 @@ struct GemmArgs {
     // persistent kernel (record field persistent = 1)
     int persistent, cta_group;
     int total_tiles;                            // tiles_m * tiles_n * batch; tiles_m counts 128 * cta_group rows
-    int a_mn, b_mn;                             // operand arrives as [tile_k][rows] boxes and is transposed in shared memory
+    int a_mn, b_mn;                             // the operand's tiles are MN-major
     int b_rows_cta;                             // rows of operand B one CTA loads: tile_n / cta_group
-    unsigned a_stg_off, b_stg_off;              // staging rings: byte offsets from the aligned tile base
-    unsigned stg_a_bytes, stg_b_bytes;          // ... and bytes per box
-    int stg_depth;                              // boxes per staging ring (what is in flight from DRAM)
-    unsigned epi_off;                           // read-out staging area (one 32 x 36-float block per read-out warp)
+    int stg_depth;                              // tap-major: boxes per staging ring
+    unsigned epi_off;                           // read-out staging area: byte offset from the aligned tile base
+    int epi_warps;                              // read-out warps: 4 or 8
+    int epi_bufs;                               // 32 x 32 blocks in each read-out warp's ring
+    unsigned epi_warp_bytes;                    // ... and its bytes
+    int epi_tma;                                // outputs leave by TMA stores (contiguous along the tile's columns)
+    int res_tma;                                // the residual comes in by TMA, one block ahead
+    int y_tma_batched;                          // the output's tensor map has the batch as its third dimension
 };
 
 struct DwArgs {
@@ -127,8 +131,14 @@ struct Plan {
     RowArgs row{};
 };
 
+constexpr int kMaxEpiBufs = 3;
+
+// The tensor maps of a launch, cached by the pointers they were made for.
 struct TmapPair {
     const void* a_ptr; const void* b_ptr;
+    const void* y_ptr; const void* r_ptr;   // persistent form with TMA read-out; null elsewhere
+    alignas(64) unsigned char y[128];
+    alignas(64) unsigned char r[128];
     alignas(64) unsigned char a[128];
     alignas(64) unsigned char b[128];
     alignas(64) unsigned char x[128];   // conv2d: the image as a (W, H, C, N) tensor, for the slab

@@ -21,6 +21,7 @@
 #include <cstdint>
 #include <cstring>
 #include <algorithm>
+#include <atomic>
 #include <utility>
 #include "tt_internal.h"
 
@@ -124,6 +125,12 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, uint
         ::"r"(dst), "l"(tmap), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
 
+// An MN-major operand tile: one box [tile_k][32 rows] after the other.
+__device__ __forceinline__ void load_mn_boxes(uint32_t dst, const void* tmap, uint32_t bar, int row0, int rows, int k0, int tile_k, int bz) {
+#pragma unroll 1
+    for (int r = 0; r < rows; r += 32, dst += (uint32_t)tile_k * 128u) tma_load_3d(dst, tmap, bar, row0 + r, k0, bz);
+}
+
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2, int c3) {
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
@@ -162,6 +169,21 @@ __device__ __forceinline__ void issue_steps(uint32_t d_tmem, uint32_t d_hi, uint
         }
     }
 }
+// The same when an operand is MN-major: any number of steps, each operand with its own stride (k8_a, k8_b) per step inside
+// an atom of k8_n steps.
+__device__ __forceinline__ void issue_steps_any(uint32_t d_tmem, uint32_t a_hi, uint32_t b_hi, uint32_t a_lo, uint32_t b_lo, uint32_t k8_a,
+                                                uint32_t k8_b, uint32_t a_atom, uint32_t b_atom, int atoms, int k8_n, uint32_t idesc,
+                                                uint32_t accumulate) {
+#pragma unroll 1
+    for (int at = 0; at < atoms; ++at, a_lo += a_atom, b_lo += b_atom) {
+        uint32_t a = a_lo, b = b_lo;
+#pragma unroll 4
+        for (int k8 = 0; k8 < k8_n; ++k8, a += k8_a, b += k8_b) {
+            mma_tf32(d_tmem, ((uint64_t)a_hi << 32) | (uint64_t)a, ((uint64_t)b_hi << 32) | (uint64_t)b, idesc, accumulate);
+            accumulate = 1u;
+        }
+    }
+}
 
 // Arrive on an mbarrier once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
@@ -189,6 +211,30 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, int row_bytes) {
     d |= 1ull << 46;
     d |= swz << 61;
     return d;
+}
+
+// The same for an MN-major tile: the row index of the operand is the contiguous one in memory (the pixels of a 1x1
+// convolution, the columns of an NN batch_matmul's second operand), so a TMA box of 32 rows x tile_k is [k][32 rows] lines of
+// 128 bytes.  kind::tf32 reads that form with the 128-byte swizzle of 32-byte atoms (mode 1: the 32-byte chunk index is XORed
+// with the line index modulo 4; read out of the tensor core with an indexed tile): four lines make an atom of 512 bytes
+// (stride byte offset), and the next 32 rows begin a box further on (leading byte offset).
+__device__ __forceinline__ uint64_t make_desc_mn(uint32_t saddr, uint32_t box_bytes) {
+    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(box_bytes >> 4) << 16;
+    d |= (uint64_t)(512u >> 4) << 32;
+    d |= 1ull << 46;
+    d |= 1ull << 61;
+    return d;
+}
+// How far a descriptor's start address (in 16-byte units) moves per 8-wide reduction step and per swizzle atom of K.
+struct DescSteps { uint32_t lo, hi, k8, atom; };
+__device__ __forceinline__ DescSteps desc_steps(bool mn, int row_bytes, int rows, int tile_k, int atom_k) {
+    DescSteps s;
+    const uint64_t d = mn ? make_desc_mn(0u, (uint32_t)tile_k * 128u) : make_desc(0u, row_bytes);
+    s.lo = (uint32_t)d; s.hi = (uint32_t)(d >> 32);
+    s.k8 = mn ? 64u : 2u;                                // eight lines of 128 bytes; 32 bytes along a line
+    s.atom = mn ? 64u * (uint32_t)(atom_k >> 3) : (uint32_t)(rows * row_bytes) >> 4;
+    return s;
 }
 
 // GELU in its erf form, 0.5 x (1 + erf(x / sqrt 2)).  erf through the rational approximation 7.1.26 of Abramowitz and
@@ -716,7 +762,9 @@ __device__ __forceinline__ void epilogue_block(float (&v)[32], const EpiArgs& e,
 // ------------------------------------------------------------------------------------------------------------
 // GEMM_TC kernel.  grid = (tiles_m * tiles_n, split_k, batch), block = 320 threads:
 // warp 0 TMA producer, warp 1 MMA issuer + tensor-memory owner, warps 2-9 gather producers, then epilogue.
-// Two builds: MIN_CTAS = 1 (all registers), and MIN_CTAS = 2 (registers capped so that two CTAs share an SM when a
+// Built for each way its operands reach shared memory (GemmForm), so that a kernel carries only the code it runs: the
+// launches of a batch-1 model pass are a few microseconds long and meet a cold instruction cache.
+// Two builds of each: MIN_CTAS = 1 (all registers), and MIN_CTAS = 2 (registers capped so that two CTAs share an SM when a
 // record's shared memory and tensor memory allow it: one CTA's set-up and read-out then overlap the other's main loop).
 // ------------------------------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
@@ -757,7 +805,15 @@ __device__ __forceinline__ uint32_t red_band_bytes(const GemmArgs& g, int owner)
     return (uint32_t)red_band_extent(g, owner) * 4u * (uint32_t)(g.y_ns == 1 ? g.tile_n + 4 : kRedColPitch);
 }
 
-template <int MIN_CTAS>
+enum GemmForm {
+    kFormTma = 0,       // both operands K-major by TMA
+    kFormMn = 1,        // both by TMA, one of them (or both) MN-major
+    kFormIm2col = 2,    // one operand expanded from a slab of input rows, the other by TMA or gathered
+    kFormTap = 3,       // tap-major convolution
+    kFormGather = 4     // an operand gathered from global memory
+};
+
+template <int MIN_CTAS, int FORM>
 __global__ void __launch_bounds__(kGemmThreads, MIN_CTAS)
 tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                   const __grid_constant__ CUtensorMap tmap_x, const GemmArgs g) {
@@ -796,12 +852,15 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     // (error-compensated products: a stage holds the two operand tiles and, behind them, their remainders)
     const uint32_t lo_off = g.a_stage_bytes + g.b_stage_bytes;
-    const uint32_t stage_bytes = g.x3 ? 2u * lo_off : lo_off;
-    const bool a_tma = g.a_mode == OPM_TMA, b_tma = g.b_mode == OPM_TMA;
+    const uint32_t stage_bytes = FORM == kFormTma && g.x3 ? 2u * lo_off : lo_off;
+    // what the instantiation is made for (GemmForm); within it only the modes that its form leaves open are looked at
+    constexpr bool im2col = FORM == kFormIm2col, tapm = FORM == kFormTap;     // tapm: reduction walked by channel block and tap
+    const bool a_mn = FORM == kFormMn && g.a_mode == OPM_TMA_MN, b_mn = FORM == kFormMn && g.b_mode == OPM_TMA_MN;
+    const bool a_tma = FORM == kFormTma || FORM == kFormMn || FORM == kFormTap || g.a_mode == OPM_TMA;
+    const bool b_tma = FORM == kFormTma || FORM == kFormMn || (FORM != kFormTap && g.b_mode == OPM_TMA);
     const bool any_tma = a_tma || b_tma, any_gather = !a_tma || !b_tma;
-    const bool im2col = g.a_mode == OPM_IM2COL || g.b_mode == OPM_IM2COL;
-    const bool tapm = g.tap_major != 0;               // conv2d, reduction walked by channel block and tap
     const bool slab_tma = (im2col || tapm) && g.slab_tma != 0;
+    const bool x3 = FORM == kFormTma && g.x3 != 0;       // error-compensated products
     // im2col geometry of this CTA: first output row of its pixels, the image row its slab starts at, slab chunks
     int ic_p_first = 0, ic_ih_lo = 0, ic_chunks = 0;
     if (im2col) {
@@ -824,9 +883,9 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     if (threadIdx.x == 32) {
         // the tensor maps are fetched ahead of their first use (they are kernel parameters: nothing the previous
         // kernel of the stream could still be writing)
-        if (g.a_mode == OPM_TMA) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
-        if (g.b_mode == OPM_TMA) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_b) : "memory");
-        if (g.slab_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
+        if (a_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
+        if (b_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_b) : "memory");
+        if (slab_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
     }
     if (threadIdx.x == 0) {
         const uint32_t full_count = tapm ? 1u : (any_tma ? 1u : 0u) + (any_gather ? (uint32_t)wpg : 0u);
@@ -835,7 +894,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             mbar_init(smem_u32(&empty_bar[s]), 1u);
         }
         mbar_init(smem_u32(&accum_bar), 1u);
-        if (g.x3) for (int s = 0; s < g.stages; ++s) mbar_init(smem_u32(&lo_bar[s]), (uint32_t)kGatherWarps);
+        if (x3) for (int s = 0; s < g.stages; ++s) mbar_init(smem_u32(&lo_bar[s]), (uint32_t)kGatherWarps);
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&slab_full[b]), 1u);
             mbar_init(smem_u32(&slab_empty[b]), (uint32_t)kGatherWarps);
@@ -951,12 +1010,16 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                     if (a_here) {
                         uint32_t dst = a_stage;
                         int kc = k0;
+                        if (a_mn) load_mn_boxes(dst, &tmap_a, full_addr, m0, kHwTileM, k0, g.tile_k, a_bz);
+                        else
 #pragma unroll 1
                         for (int at = 0; at < g.n_atoms; ++at, dst += a_atom, kc += g.atom_k) tma_load_3d(dst, &tmap_a, full_addr, kc, m0, a_bz);
                     }
                     if (b_here) {
                         uint32_t dst = a_stage + g.a_stage_bytes;
                         int kc = k0;
+                        if (b_mn) load_mn_boxes(dst, &tmap_b, full_addr, n0, g.tile_n, k0, g.tile_k, b_bz);
+                        else
 #pragma unroll 1
                         for (int at = 0; at < g.n_atoms; ++at, dst += b_atom, kc += g.atom_k) tma_load_3d(dst, &tmap_b, full_addr, kc, n0, b_bz);
                     }
@@ -993,14 +1056,16 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             const uint32_t full0 = smem_u32(&full_bar[0]), empty0 = smem_u32(&empty_bar[0]);
             // descriptors differ only in their 14-bit start-address field: keep the constant upper word, step the
             // lower word by (bytes >> 4) per stage, per atom and per 8-wide K slice
-            const uint64_t d0 = make_desc(0u, g.row_bytes);
-            const uint32_t d_hi = (uint32_t)(d0 >> 32), d_lo = (uint32_t)d0;
+            const DescSteps da = desc_steps(a_mn, g.row_bytes, kHwTileM, g.tile_k, g.atom_k);
+            const DescSteps db = desc_steps(b_mn, g.row_bytes, g.tile_n, g.tile_k, g.atom_k);
+            const bool any_mn = a_mn || b_mn;
+            const uint32_t d_hi = da.hi, d_lo = da.lo;
             const uint32_t a_lo0 = d_lo + ((tiles_base & 0x3FFFFu) >> 4);
-            const uint32_t b_lo0 = a_lo0 + (g.a_stage_bytes >> 4);
+            const uint32_t b_lo0 = db.lo + (((tiles_base + g.a_stage_bytes) & 0x3FFFFu) >> 4);
             const uint32_t stage_step = stage_bytes >> 4;
-            const uint32_t a_atom = (uint32_t)(kHwTileM * g.row_bytes) >> 4, b_atom = (uint32_t)(g.tile_n * g.row_bytes) >> 4;
+            const uint32_t a_atom = da.atom, b_atom = db.atom;
             const int k8_per_atom = g.atom_k >> 3;
-            const uint32_t a_next_atom = a_atom - 2u * (uint32_t)k8_per_atom, b_next_atom = b_atom - 2u * (uint32_t)k8_per_atom;
+            const uint32_t a_next_atom = a_atom - da.k8 * (uint32_t)k8_per_atom, b_next_atom = b_atom - db.k8 * (uint32_t)k8_per_atom;
             const bool leader = elect_one();             // this lane issues every multiply-accumulate and every commit
             // accumulators: reduction steps are dealt round-robin; an accumulator's first step overwrites
             uint32_t d_tmem = tmem_base;
@@ -1044,13 +1109,15 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             } else
             for (int it = 0; it < iters; ++it) {
                 bool got = mbar_wait(full_addr, ph, abortp, g.status, 2u, g.wait_ns);
-                if (g.x3) got = mbar_wait(smem_u32(&lo_bar[st]), ph, abortp, g.status, 16u, g.wait_ns) && got;   // the remainders too
+                if (x3) got = mbar_wait(smem_u32(&lo_bar[st]), ph, abortp, g.status, 16u, g.wait_ns) && got;   // the remainders too
                 if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
                 tc_fence_after();
                 if (leader) {
                     // descriptors step by 2 (32 bytes = 8 TF32 along K) inside a swizzle atom, then to the next atom
                     uint32_t a_lo = a_stage, b_lo = b_stage;
-                    if (g.n_acc == 1) {
+                    if (any_mn && g.n_acc == 1) {
+                        issue_steps_any(tmem_base, da.hi, db.hi, a_lo, b_lo, da.k8, db.k8, a_atom, b_atom, g.n_atoms, k8_per_atom, g.idesc, it > 0 ? 1u : 0u);
+                    } else if (g.n_acc == 1) {
                         // one accumulator: nothing to rotate.  The common tile_k values are unrolled completely, so
                         // that an issue is two additions and the instruction.
                         auto issue_stage = [&](uint32_t a0, uint32_t b0, uint32_t accumulate) {
@@ -1061,7 +1128,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                             else issue_steps<1, 1>(tmem_base, d_hi, a0, b0, a_atom, b_atom, g.idesc, accumulate);
                         };
                         const uint32_t accumulate = it > 0 ? 1u : 0u;
-                        if (g.x3) {
+                        if (x3) {
                             // the two cross terms first (small), then the product of what the tensor core sees of a and b
                             const uint32_t lo = lo_off >> 4;
                             issue_stage(a_lo + lo, b_lo, accumulate);
@@ -1075,9 +1142,9 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                     for (int at = 0; at < g.n_atoms; ++at) {
 #pragma unroll 4
                         for (int k8 = 0; k8 < k8_per_atom; ++k8) {
-                            mma_tf32(d_tmem, ((uint64_t)d_hi << 32) | (uint64_t)a_lo, ((uint64_t)d_hi << 32) | (uint64_t)b_lo, g.idesc,
+                            mma_tf32(d_tmem, ((uint64_t)da.hi << 32) | (uint64_t)a_lo, ((uint64_t)db.hi << 32) | (uint64_t)b_lo, g.idesc,
                                      fresh > 0 ? 0u : 1u);
-                            a_lo += 2u; b_lo += 2u;
+                            a_lo += da.k8; b_lo += db.k8;
                             if (fresh > 0) --fresh;
                             d_tmem += (uint32_t)g.tile_n;
                             if (d_tmem == d_end) d_tmem = tmem_base;
@@ -1282,7 +1349,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 while (st >= g.stages) { st -= g.stages; ph ^= 1u; }
             }
         }
-        if (g.x3) {
+        if (x3) {
             // ---- error-compensated products: once a stage's operand tiles have landed, the eight warps write, 16 bytes
             // per thread and step, what the tensor core will NOT see of every value (x minus x truncated to TF32's ten
             // mantissa bits: exact in fp32) into the second half of the stage, in the same swizzled layout ----
@@ -1622,14 +1689,19 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
 // t = unit, unit + units, ... (a unit is a CTA, or a pair of CTAs when CG = 2) with
 //   - the operand pipeline running on across tile boundaries (the loads of the next tile are in flight while this
 //     tile's last multiply-accumulates run),
-//   - TWO accumulators in tensor memory, used alternately: the read-out warps drain tile t (bias, activation,
-//     stores) while the MMA warp already accumulates tile t + 1,
+//   - TWO accumulators in tensor memory, used alternately: the read-out warps drain tile t (bias, residual,
+//     activation, stores) while the MMA warp already accumulates tile t + 1,
 //   - barriers and tensor memory set up once per CTA instead of once per tile.
-// Operands: K-major tensors arrive by TMA straight into the swizzled pipeline stage.  Operands whose ROW index is
-// the contiguous one in memory (the image of a 1x1 convolution: pixels; the second operand of an NN batch_matmul)
-// arrive by TMA as [tile_k][rows] boxes in a staging ring and four warps transpose them into the K-major stage
-// (kind::tf32 has no MN-major operands on this part).  No split-K, one accumulator per tile.
-// Warps: 0 TMA producer, 1 MMA issuer + tensor-memory owner, 2-5 transposers, 6-9 read-out.
+// Operands arrive by TMA and are multiplied as they lie: K-major tensors in K-major tiles, operands whose ROW index is the
+// contiguous one in memory (the image of a 1x1 convolution: pixels; the second operand of an NN batch_matmul) in MN-major
+// tiles (make_desc_mn).  No split-K, one accumulator per tile.
+// Warps: 0 TMA producer, 1 MMA issuer + tensor-memory owner, 2-9 read-out (two per lane quadrant, alternate 32-column
+// blocks; only 6-9 when the record's stages leave shared memory for four staging areas).
+// Read-out.  Rows of the output that are contiguous along the tile's columns leave through a ring of `epi_bufs` 32 x 32
+// blocks per warp in shared memory (128-byte lines, swizzled so that a lane's 16-byte stores do not conflict) and TMA
+// stores, which also clip the ragged edges; a residual comes in through the same ring by TMA one block ahead, so no
+// lane waits on a global load.  1x1 convolution 64 -> 256 at 56 x 56 with residual, batch 32: 116 us with the residual
+// loaded by the lanes and the image transposed in shared memory, 41 us this way (bytes at the copy rate: 35 us).
 // CG = 2: two CTAs of a cluster work on one 256-row tile.  Each loads its own 128 rows of A and its half of B's
 // rows with ordinary (non-multicast) TMA; the CTA of rank 0 issues tcgen05.mma.cta_group::2, which reads both
 // CTAs' shared memory and writes each CTA's half of the accumulator into that CTA's tensor memory, so an SM reads
@@ -1680,86 +1752,29 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void* tmap,
         "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
         ::"r"(dst), "l"(tmap), "r"(bar_cluster), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
-__device__ __forceinline__ void tma_load_3d_plain(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2) {
-    tma_load_3d(dst, tmap, bar, c0, c1, c2);
+// One 3-D box from shared memory to a tensor (clipped at its extents); tracked by the issuing thread's bulk groups.
+__device__ __forceinline__ void tma_store_3d(const void* tmap, uint32_t src, int c0, int c1, int c2) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];"
+                 ::"l"(tmap), "r"(src), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
-
-constexpr int kPsTransposeWarps = 4;
-constexpr int kPsEpilogueWarps = 4;
-
-// Transpose one staged box [tile_k][rows] (row index contiguous) into the K-major swizzled stage tile.  A task is a
-// (32-row block, four consecutive reduction indices) pair: lanes walk rows (conflict-free 4-byte loads), each lane
-// assembles its row's four values and writes one 16-byte chunk.  What bounds this routine is its instruction count, so
-// a warp keeps a row block (or shares one with other warps, taking alternate chunks) and everything that depends on the
-// row is worked out once; per chunk there are four loads, one store and a few additions.
-template <int KB>
-__device__ __forceinline__ void ps_transpose_chunks(uint32_t src, uint32_t src_step, uint32_t dst_row, uint32_t swz, int c0, int step, int n_ch,
-                                                    uint32_t k_bytes, int atom_shift, int atom_k, uint32_t atom_bytes, bool in_tile) {
-    for (; c0 < n_ch; c0 += step * KB, src += src_step * KB) {
-        float val[KB][4];
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            const uint32_t a = src + (c0 + b * step < n_ch ? (uint32_t)b * src_step : 0u);
-            val[b][0] = ld_shared_f32(a);
-            val[b][1] = ld_shared_f32(a + k_bytes);
-            val[b][2] = ld_shared_f32(a + 2u * k_bytes);
-            val[b][3] = ld_shared_f32(a + 3u * k_bytes);
-        }
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            const int ci = c0 + b * step;
-            if (ci < n_ch && in_tile) {
-                const int kk = ci << 2;
-                st_shared_v4(dst_row + (uint32_t)(kk >> atom_shift) * atom_bytes + ((uint32_t)((kk & (atom_k - 1)) << 2) ^ swz),
-                             val[b][0], val[b][1], val[b][2], val[b][3]);
-            }
-        }
-    }
-}
-
-__device__ __forceinline__ void ps_transpose(uint32_t stg, uint32_t tile, int rows, int tile_k, int atom_k, int row_bytes,
-                                             int swz_mask, int tw, int nw, int lane) {
-    const int atom_shift = atom_k == 32 ? 5 : (atom_k == 16 ? 4 : 3);
-    const int shift = row_bytes == 128 ? 0 : (row_bytes == 64 ? 1 : 2);
-    const uint32_t atom_bytes = (uint32_t)rows * (uint32_t)row_bytes;
-    const int n_rb = (rows + 31) >> 5, n_ch = tile_k >> 2;
-    const uint32_t k_bytes = 4u * (uint32_t)rows;                  // distance between consecutive reduction indices in the box
-    // row blocks to the nw warps that work on this machine: with nw or more blocks (or a count that does not divide nw) a warp
-    // takes blocks tw, tw + nw, ... and every chunk of them; with fewer, nw / n_rb warps share a block and take alternate chunks
-    int rb_first, rb_step, c_first, c_step;
-    const bool shared_block = n_rb < nw && (nw % n_rb) == 0;
-    if (!shared_block) { rb_first = tw; rb_step = nw; c_first = 0; c_step = 1; }
-    else { rb_first = tw % n_rb; rb_step = n_rb; c_first = tw / n_rb; c_step = nw / n_rb; }   // (rb_step only ends the loop)
-    for (int rb = rb_first; rb < n_rb; rb += rb_step) {
-        const int row = rb * 32 + lane;
-        const bool in_tile = row < rows;
-        const uint32_t src = stg + 4u * (uint32_t)(in_tile ? row : rows - 1) + (uint32_t)c_first * 4u * k_bytes;
-        const uint32_t dst_row = tile + (uint32_t)row * (uint32_t)row_bytes;
-        const uint32_t swz = (uint32_t)((row >> shift) & swz_mask) << 4;
-        const int mine = (n_ch - c_first + c_step - 1) / c_step;
-        if (mine <= 2) ps_transpose_chunks<2>(src, (uint32_t)c_step * 4u * k_bytes, dst_row, swz, c_first, c_step, n_ch, k_bytes, atom_shift, atom_k, atom_bytes, in_tile);
-        else if (mine <= 4) ps_transpose_chunks<4>(src, (uint32_t)c_step * 4u * k_bytes, dst_row, swz, c_first, c_step, n_ch, k_bytes, atom_shift, atom_k, atom_bytes, in_tile);
-        else ps_transpose_chunks<8>(src, (uint32_t)c_step * 4u * k_bytes, dst_row, swz, c_first, c_step, n_ch, k_bytes, atom_shift, atom_k, atom_bytes, in_tile);
-        if (shared_block) break;                                     // this warp has no other block
-    }
-}
+__device__ __forceinline__ void bulk_stores_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// Wait until at most N of the store groups this thread committed have still to read their shared memory.
+template <int N>
+__device__ __forceinline__ void bulk_stores_pending() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 
 template <int CG>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
-                  const __grid_constant__ CUtensorMap tmap_x, const GemmArgs g) {
+                  const __grid_constant__ CUtensorMap tmap_y, const __grid_constant__ CUtensorMap tmap_r, const GemmArgs g) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[kMaxStages];     // a stage's operands are in place (TMA bytes and/or the transposer warps)
+    __shared__ uint64_t full_bar[kMaxStages];     // a stage's operands have landed
     __shared__ uint64_t empty_bar[kMaxStages];    // every multiply-accumulate that reads the stage has completed
-    __shared__ uint64_t stg_full[kMaxStages];     // a staging box has landed
-    __shared__ uint64_t stg_empty[kMaxStages];    // the transposer warps are done with it
-    __shared__ uint64_t pm_full[2];               // tap-major convolution: a pixel-major slab buffer has been written
-    __shared__ uint64_t pm_empty[2];              // ... and every multiply-accumulate that reads it has completed
     __shared__ uint64_t acc_full[2];              // an accumulator holds a finished tile
     __shared__ uint64_t acc_empty[2];             // the read-out warps (of both CTAs) have drained it
+    __shared__ uint64_t res_full[8 * kMaxEpiBufs];   // per read-out warp and ring buffer: a residual block has landed
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ __align__(16) float s_bias[2][256];
+    __shared__ __align__(16) float s_bias[8][32];   // per read-out warp: the bias of its current block
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     volatile int* abortp = &abort_flag;
@@ -1773,39 +1788,25 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t stage_bytes = g.a_stage_bytes + g.b_stage_bytes;
     const bool a_mn = g.a_mn != 0, b_mn = g.b_mn != 0;
-    // Tap-major convolution (see the one-tile kernel): operand A = re-packed filters by TMA; operand B = views of a
-    // pixel-major slab that the transposer warps write once per 32-channel block from a staged NCHW box.  Here the
-    // staging ring, the two slab buffers and the filter stages all run on across tile boundaries.
-    const bool tapm = g.tap_major != 0;
-    const bool any_mn = a_mn || b_mn, any_km = !a_mn || !b_mn;
-    const bool any_stg = any_mn || tapm;
     const int b_rows = g.b_rows_cta;
-    const int RS = g.R * g.S;
-    const int blocks_per_tile = tapm ? kt_n * g.n_atoms / RS : 0;     // 32-channel blocks
-    constexpr int tr_groups = 1;                                      // all transposer warps work on the same box
-    constexpr int tr_warps = kPsTransposeWarps / tr_groups;
+    const int epi_warps = g.epi_warps;
 
     if (threadIdx.x == 32) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
-        if (!tapm) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_b) : "memory");
-        else asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_b) : "memory");
+        if (g.epi_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_y) : "memory");
+        if (g.res_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_r) : "memory");
     }
     if (threadIdx.x == 0) {
-        const uint32_t full_count = tapm ? 1u : (any_km ? 1u : 0u) + (any_mn ? (uint32_t)tr_warps : 0u);
         for (int s = 0; s < g.stages; ++s) {
-            mbar_init(smem_u32(&full_bar[s]), full_count);
+            mbar_init(smem_u32(&full_bar[s]), 1u);
             mbar_init(smem_u32(&empty_bar[s]), 1u);
         }
-        for (int s = 0; s < g.stg_depth; ++s) {
-            mbar_init(smem_u32(&stg_full[s]), 1u);
-            mbar_init(smem_u32(&stg_empty[s]), (uint32_t)(tapm ? kPsTransposeWarps : tr_warps));
-        }
         for (int a = 0; a < 2; ++a) {
-            mbar_init(smem_u32(&pm_full[a]), (uint32_t)kPsTransposeWarps);
-            mbar_init(smem_u32(&pm_empty[a]), 1u);
             mbar_init(smem_u32(&acc_full[a]), 1u);
-            mbar_init(smem_u32(&acc_empty[a]), (uint32_t)(kPsEpilogueWarps * CG));
+            mbar_init(smem_u32(&acc_empty[a]), (uint32_t)(epi_warps * CG));
         }
+        if (g.res_tma) for (int b = 0; b < 8 * kMaxEpiBufs; ++b) mbar_init(smem_u32(&res_full[b]), 1u);
         abort_flag = 0;
         fence_mbar_init();
         fence_proxy_async_shared();
@@ -1840,18 +1841,388 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
-        // Two independent streams of requests, each with its own ring and cursor: boxes of a row-contiguous operand go
-        // to the staging ring (g.stg_depth deep: what is in flight from DRAM), K-major tiles to the pipeline stages.
-        // The warp polls both rings and serves whichever has a free slot, so the staging ring runs as far ahead as
-        // its depth allows, whatever the multiply-accumulates are doing.
         const bool leader = elect_one();
         const uint32_t a_atom = (uint32_t)(kHwTileM * g.row_bytes), b_atom = (uint32_t)(b_rows * g.row_bytes);
-        const uint32_t km_bytes = (a_mn ? 0u : g.a_stage_bytes) + ((b_mn || tapm) ? 0u : g.b_stage_bytes);
-        const uint32_t mn_bytes = (a_mn ? g.stg_a_bytes : 0u) + (b_mn ? g.stg_b_bytes : 0u);
+        bool ok = true;
+        uint32_t st = 0, ph = 0;
+        long long issued = 0;
+        for (int i = 0; i < my_tiles && ok; ++i) {
+            int m0, n0, bz;
+            decode(i, m0, n0, bz);
+            const int a_bz = g.a_tma_batched ? bz : 0, b_bz = g.b_tma_batched ? bz : 0;
+            const int nb0 = n0 + (int)rank * b_rows;      // CG 2: this CTA's half of the B rows
+            for (int kt = 0, k0 = 0; kt < kt_n; ++kt, k0 += g.tile_k) {
+                const bool got = mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1u, abortp, g.status, 1u, g.wait_ns);
+                if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+                if (leader) {
+                    uint32_t bar = smem_u32(&full_bar[st]);
+                    // (test facility: the first stage may be told to expect more than arrives, see tt_workload_test_stall)
+                    if (rank == 0) mbar_expect_tx(bar, (uint32_t)CG * stage_bytes + (issued == 0 ? g.extra_tx : 0u));
+                    if constexpr (CG == 2) bar = map_to_peer(bar, 0u);       // the pair's loads all report to rank 0
+                    uint32_t dst = tiles_base + st * stage_bytes;
+                    int kc = k0;
+                    if (a_mn) load_mn_boxes(dst, &tmap_a, bar, m0, kHwTileM, k0, g.tile_k, a_bz);
+                    else
+#pragma unroll 1
+                    for (int at = 0; at < g.n_atoms; ++at, dst += a_atom, kc += g.atom_k) {
+                        if constexpr (CG == 2) tma_load_3d_pair(dst, &tmap_a, bar, kc, m0, a_bz);
+                        else tma_load_3d(dst, &tmap_a, bar, kc, m0, a_bz);
+                    }
+                    dst = tiles_base + st * stage_bytes + g.a_stage_bytes;
+                    kc = k0;
+                    if (b_mn) load_mn_boxes(dst, &tmap_b, bar, nb0, b_rows, k0, g.tile_k, b_bz);
+                    else
+#pragma unroll 1
+                    for (int at = 0; at < g.n_atoms; ++at, dst += b_atom, kc += g.atom_k) {
+                        if constexpr (CG == 2) tma_load_3d_pair(dst, &tmap_b, bar, kc, nb0, b_bz);
+                        else tma_load_3d(dst, &tmap_b, bar, kc, nb0, b_bz);
+                    }
+                }
+                __syncwarp();
+                ++issued;
+                if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
+            }
+        }
+        if ((!ok || *abortp) && lane == 0) {
+            // let copies in flight land before shared memory is given back (bounded)
+            if (rank == 0) {
+                const long long first = issued > g.stages ? issued - g.stages : 0;
+                for (long long it = first; it < issued; ++it) {
+                    const unsigned long long t0 = global_timer_ns();
+                    while (!mbar_try_wait(smem_u32(&full_bar[it % g.stages]), (uint32_t)(it / g.stages) & 1u)) { if (global_timer_ns() - t0 > 2000000ull) break; }
+                }
+            } else {
+                // this CTA's loads report to rank 0's barriers: give them time to land instead (the pair leaves
+                // together, after rank 0 has seen the pair's bytes or given up on them)
+                const unsigned long long t0 = global_timer_ns();
+                while (global_timer_ns() - t0 < 200000ull) { }
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (of a pair: rank 0's) ----------------
+        const bool leader = elect_one();
+        uint32_t st = 0, ph = 0;
+        bool ok = true;
+        if (CG == 2 && rank != 0) {
+            // rank 0 issues for the pair
+        } else {
+            const DescSteps da = desc_steps(a_mn, g.row_bytes, kHwTileM, g.tile_k, g.atom_k);
+            const DescSteps db = desc_steps(b_mn, g.row_bytes, b_rows, g.tile_k, g.atom_k);
+            const uint32_t a_lo0 = da.lo + ((tiles_base & 0x3FFFFu) >> 4);
+            const uint32_t b_lo0 = db.lo + (((tiles_base + g.a_stage_bytes) & 0x3FFFFu) >> 4);
+            const uint32_t stage_step = stage_bytes >> 4;
+            const int k8n = g.atom_k >> 3;
+            for (int i = 0; i < my_tiles && ok; ++i) {
+                const uint32_t acc = (uint32_t)i & 1u, aph = ((uint32_t)i >> 1) & 1u;
+                // the read-out of the tile that used this accumulator two tiles ago has finished
+                const bool freed = CG == 2 ? mbar_wait_cluster(smem_u32(&acc_empty[acc]), aph ^ 1u, abortp, g.status, 12u, g.wait_ns)
+                                           : mbar_wait(smem_u32(&acc_empty[acc]), aph ^ 1u, abortp, g.status, 12u, g.wait_ns);
+                if (!__all_sync(0xffffffffu, freed)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + acc * (uint32_t)g.tile_n;
+                for (int kt = 0; kt < kt_n; ++kt) {
+                    const bool got = mbar_wait(smem_u32(&full_bar[st]), ph, abortp, g.status, 2u, g.wait_ns);
+                    if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+                    tc_fence_after();
+                    if (leader) {
+                        uint32_t a_lo = a_lo0 + st * stage_step, b_lo = b_lo0 + st * stage_step;
+                        uint32_t accumulate = kt > 0 ? 1u : 0u;
+#pragma unroll 1
+                        for (int at = 0; at < g.n_atoms; ++at, a_lo += da.atom, b_lo += db.atom) {
+                            if (k8n == 4 && !a_mn && !b_mn) {
+#pragma unroll
+                                for (uint32_t k8 = 0; k8 < 4; ++k8) {
+                                    mma_tf32_cg<CG>(d_tmem, ((uint64_t)da.hi << 32) | (uint64_t)(a_lo + 2u * k8), ((uint64_t)db.hi << 32) | (uint64_t)(b_lo + 2u * k8), g.idesc, accumulate);
+                                    accumulate = 1u;
+                                }
+                            } else {
+                                uint32_t a = a_lo, b = b_lo;
+#pragma unroll 4
+                                for (int k8 = 0; k8 < k8n; ++k8, a += da.k8, b += db.k8) {
+                                    mma_tf32_cg<CG>(d_tmem, ((uint64_t)da.hi << 32) | (uint64_t)a, ((uint64_t)db.hi << 32) | (uint64_t)b, g.idesc, accumulate);
+                                    accumulate = 1u;
+                                }
+                            }
+                        }
+                        mma_commit_cg<CG>(smem_u32(&empty_bar[st]));          // stage reusable once these MMAs have read it
+                    }
+                    __syncwarp();
+                    if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
+                }
+                if (ok && leader) mma_commit_cg<CG>(smem_u32(&acc_full[acc]));   // the tile's accumulator is complete
+                __syncwarp();
+            }
+        }
+    } else if (warp >= 10 - epi_warps) {
+        // ---------------- read-out: tensor memory -> bias, residual, activation -> global memory ----------------
+        const int ew = warp - (10 - epi_warps);
+        const int quad = warp & 3;                       // tensor-memory lane quadrant this warp may read
+        const int c_first = (ew >> 2) * 32, c_step = epi_warps * 8;      // the 32-column blocks of a tile that this warp takes
+        EpiArgs e;
+        e.y_ms = g.y_ms; e.y_ns = g.y_ns; e.M = g.M;
+        e.lo = g.act == TT_ACT_NONE || g.act == TT_ACT_GELU_ERF ? -INFINITY : 0.f;
+        e.hi = g.act == TT_ACT_RELU6 ? 6.f : INFINITY;
+        e.gelu = g.act == TT_ACT_GELU_ERF;
+        e.vec = (g.vec_store & 1) != 0;
+        e.lin_wp = 0; e.lin_q = 0; e.lin_p = 0;
+        const bool transposed = g.y_ns == 1 && g.y_ms != 1;
+        const bool tma_out = g.epi_tma != 0, res_in = g.res_tma != 0;
+        const uint32_t ring = tiles_base + g.epi_off + (uint32_t)ew * g.epi_warp_bytes;
+        const int bufs = g.epi_bufs;
+        const int per_tile = c_first < g.tile_n ? (g.tile_n - c_first + c_step - 1) / c_step : 0;    // blocks of a tile
+        bool ok = true;
+        // residual blocks are requested one ahead of their use: cursor of the next request
+        int ri = 0, rc = c_first, rb = 0, rm0 = 0, rn0 = 0, rbz = 0;
+        if (my_tiles > 0) decode(0, rm0, rn0, rbz);
+        auto request_residual = [&]() {                  // lane 0; the buffer is free
+            const uint32_t bar = smem_u32(&res_full[ew * kMaxEpiBufs + rb]);
+            mbar_expect_tx(bar, 4096u);
+            if (tma_out) tma_load_3d(ring + (uint32_t)rb * 4096u, &tmap_r, bar, rn0 + rc, rm0 + quad * 32, g.y_tma_batched ? rbz : 0);
+            else tma_load_3d(ring + (uint32_t)rb * 4096u, &tmap_r, bar, rm0 + quad * 32, rn0 + rc, g.y_tma_batched ? rbz : 0);
+        };
+        auto advance_request = [&]() {
+            if (++rb == bufs) rb = 0;
+            rc += c_step;
+            if (rc >= g.tile_n) { rc = c_first; if (++ri < my_tiles) decode(ri, rm0, rn0, rbz); }
+        };
+        int req_left = per_tile > 0 ? my_tiles : 0;      // (tiles; a warp without blocks requests nothing)
+        if (res_in && req_left > 0) {
+            if (lane == 0) request_residual();
+            advance_request();
+        }
+        int buf = 0;                                     // ring position of the current block
+        uint32_t rph = 0;                                // phase of the residual barriers at `buf`
+        for (int i = 0; i < my_tiles; ++i) {
+            int m0, n0, bz;
+            decode(i, m0, n0, bz);
+            const uint32_t acc = (uint32_t)i & 1u, aph = ((uint32_t)i >> 1) & 1u;
+            const int m_first = m0 + quad * 32, m = m_first + lane;
+            // bias of this warp's first block, fetched while the tile is still being accumulated; later ones a block ahead
+            float bias_col = (g.bias_mode == 2 && c_first < g.tile_n && n0 + c_first + lane < g.N) ? __ldg(g.bias + n0 + c_first + lane) : 0.f;
+            const float bias_row = (g.bias_mode == 1 && m < g.M) ? __ldg(g.bias + m) : 0.f;
+            // (each read-out warp walks on its own: a barrier over the eight of them per tile cost batch_matmul NT
+            // 3072 x 128 x 128 x 64 a tenth of its time, 73 us against 65 us)
+            ok = ok && mbar_wait(smem_u32(&acc_full[acc]), aph, abortp, g.status, 4u, g.wait_ns);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+            tc_fence_after();
+            e.ybase = g.y + (long long)bz * g.y_bs;
+            e.rbase = g.residual ? g.residual + (long long)bz * g.y_bs : nullptr;
+            const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * (uint32_t)g.tile_n;
+            uint32_t r[32];
+            if (per_tile > 0) tmem_ld32(t_row + (uint32_t)c_first, r);
+            else if (lane == 0) {
+                if (CG == 2) mbar_arrive_remote(smem_u32(&acc_empty[acc]), 0u);
+                else mbar_arrive(smem_u32(&acc_empty[acc]));
+            }
+#pragma unroll 1
+            for (int c0 = c_first; c0 < g.tile_n; c0 += c_step) {
+                float v[32];
+                const int nb = n0 + c0;
+                const int cnt = min(g.N - nb, g.tile_n - c0);
+                const uint32_t stg = ring + (uint32_t)buf * 4096u;
+                if (res_in) {
+                    // request the next block's residual: its buffer's last TMA store (if any) must have read it
+                    if (ri < my_tiles) {
+                        if (lane == 0) {
+                            if (tma_out) { if (bufs == 2) bulk_stores_pending<0>(); else bulk_stores_pending<1>(); }
+                            request_residual();
+                        }
+                        advance_request();
+                    }
+                } else if (tma_out) {
+                    if (lane == 0) { if (bufs == 1) bulk_stores_pending<0>(); else bulk_stores_pending<1>(); }   // this buffer's last store has read it
+                    __syncwarp();
+                }
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+                if (c0 + c_step < g.tile_n) tmem_ld32(t_row + (uint32_t)(c0 + c_step), r);
+                else {
+                    // every value of this warp's part of the accumulator is in registers: hand it back to the MMA warp
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (CG == 2) mbar_arrive_remote(smem_u32(&acc_empty[acc]), 0u);
+                        else mbar_arrive(smem_u32(&acc_empty[acc]));
+                    }
+                }
+                if (g.bias_mode == 1) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] += bias_row;
+                } else if (g.bias_mode == 2) {
+                    __syncwarp();                        // (the previous block's values have been read)
+                    s_bias[ew][lane] = bias_col;
+                    const int nc = c0 + c_step;
+                    bias_col = (nc < g.tile_n && n0 + nc + lane < g.N) ? __ldg(g.bias + n0 + nc + lane) : 0.f;
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4) {
+                        const float4 b = *reinterpret_cast<const float4*>(&s_bias[ew][j]);
+                        v[j] += b.x; v[j + 1] += b.y; v[j + 2] += b.z; v[j + 3] += b.w;
+                    }
+                }
+                if (res_in) {
+                    if (!mbar_wait(smem_u32(&res_full[ew * kMaxEpiBufs + buf]), rph, abortp, g.status, 17u, g.wait_ns)) ok = false;
+                    ok = __all_sync(0xffffffffu, ok); // (after a lost block nothing more is stored; the next tile ends the walk)
+                    if (tma_out) {
+#pragma unroll
+                        for (int j = 0; j < 32; j += 4) {
+                            const float4 q = ld_shared_v4f(stg + (uint32_t)lane * 128u + ((uint32_t)((j >> 2) ^ (lane & 7)) << 4));
+                            v[j] += q.x; v[j + 1] += q.y; v[j + 2] += q.z; v[j + 3] += q.w;
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] += ld_shared_f32(stg + (uint32_t)j * 128u + (uint32_t)lane * 4u);
+                        __syncwarp();                    // the buffer may be requested again after the next block
+                    }
+                }
+                if (tma_out || res_in || e.rbase == nullptr) {
+                    if (e.gelu) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] = gelu_erf(v[j]);
+                    } else if (g.act != TT_ACT_NONE) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] = fminf(fmaxf(v[j], e.lo), e.hi);
+                    }
+                }
+                if (!ok) continue;
+                if (tma_out) {
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4)
+                        st_shared_v4(stg + (uint32_t)lane * 128u + ((uint32_t)((j >> 2) ^ (lane & 7)) << 4), v[j], v[j + 1], v[j + 2], v[j + 3]);
+                    fence_proxy_async_shared();          // the lanes' stores -> visible to the TMA store
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (cnt > 0 && m_first < g.M) tma_store_3d(&tmap_y, stg, nb, m_first, g.y_tma_batched ? bz : 0);
+                        bulk_stores_commit();
+                    }
+                } else if (cnt > 0) {                    // (warp-uniform)
+                    const bool full = cnt >= 32 && m_first + 32 <= g.M && (e.vec || !transposed);
+                    if (res_in || e.rbase == nullptr) {
+                        if (full) epilogue_block<true, false>(v, e, m_first, nb, cnt, stg, lane, transposed);
+                        else epilogue_block<false, false>(v, e, m_first, nb, cnt, stg, lane, transposed);
+                    } else {
+                        if (full) epilogue_block<true, true>(v, e, m_first, nb, cnt, stg, lane, transposed);
+                        else epilogue_block<false, true>(v, e, m_first, nb, cnt, stg, lane, transposed);
+                    }
+                }
+                if (tma_out || res_in) { if (++buf == bufs) { buf = 0; rph ^= 1u; } }
+            }
+        }
+        if (tma_out && lane == 0) bulk_stores_pending<0>();      // shared memory stays until the last store has read it
+        if (!ok && res_in && lane == 0) {
+            // a residual block that was requested and not waited for (bounded)
+            const unsigned long long t0 = global_timer_ns();
+            while (global_timer_ns() - t0 < 200000ull) { }
+        }
+        __syncwarp();
+    }
+    tc_fence_before();
+    __syncthreads();
+    // a pair stays together until neither CTA touches the other's shared memory, barriers or tensor memory any more
+    if constexpr (CG == 2) cluster_sync_all();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        if constexpr (CG == 1) tmem_dealloc(tmem_base, g.tmem_cols);
+        else asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(g.tmem_cols) : "memory");
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------
+// GEMM_TC, persistent form of the tap-major convolution (records with k_order = 1 and persistent = 1): the same walk over
+// output tiles with two accumulators; operand A = re-packed filters by TMA, operand B = views of a pixel-major slab that
+// four transposer warps write once per 32-channel block from a staged NCHW box.
+// Warps: 0 TMA producer, 1 MMA issuer + tensor-memory owner, 2-5 transposers, 6-9 read-out.
+// ------------------------------------------------------------------------------------------------------------
+constexpr int kPsTransposeWarps = 4;
+constexpr int kPsEpilogueWarps = 4;
+
+__global__ void __launch_bounds__(kGemmThreads, 1)
+tt_gemm_ps_tap_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_x, const GemmArgs g) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t full_bar[kMaxStages];     // a stage's operands are in place (TMA bytes and/or the transposer warps)
+    __shared__ uint64_t empty_bar[kMaxStages];    // every multiply-accumulate that reads the stage has completed
+    __shared__ uint64_t stg_full[kMaxStages];     // a staging box has landed
+    __shared__ uint64_t stg_empty[kMaxStages];    // the transposer warps are done with it
+    __shared__ uint64_t pm_full[2];               // tap-major convolution: a pixel-major slab buffer has been written
+    __shared__ uint64_t pm_empty[2];              // ... and every multiply-accumulate that reads it has completed
+    __shared__ uint64_t acc_full[2];              // an accumulator holds a finished tile
+    __shared__ uint64_t acc_empty[2];             // the read-out warps (of both CTAs) have drained it
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+    __shared__ __align__(16) float s_bias[2][256];
+
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    volatile int* abortp = &abort_flag;
+    pdl_allow_next();
+    const int unit = (int)blockIdx.x, n_units = (int)gridDim.x;
+    const int my_tiles = g.total_tiles > unit ? (g.total_tiles - unit + n_units - 1) / n_units : 0;
+    const int tiles_per_batch = g.tiles_m * g.tiles_n;
+    const int kt_n = g.k_tiles;
+
+    const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t stage_bytes = g.a_stage_bytes + g.b_stage_bytes;
+    // Tap-major convolution (see the one-tile kernel): operand A = re-packed filters by TMA; operand B = views of a
+    // pixel-major slab that the transposer warps write once per 32-channel block from a staged NCHW box.  Here the
+    // staging ring, the two slab buffers and the filter stages all run on across tile boundaries.
+    const int RS = g.R * g.S;
+    const int blocks_per_tile = kt_n * g.n_atoms / RS;     // 32-channel blocks
+
+    if (threadIdx.x == 32) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
+    }
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < g.stages; ++s) {
+            mbar_init(smem_u32(&full_bar[s]), 1u);
+            mbar_init(smem_u32(&empty_bar[s]), 1u);
+        }
+        for (int s = 0; s < g.stg_depth; ++s) {
+            mbar_init(smem_u32(&stg_full[s]), 1u);
+            mbar_init(smem_u32(&stg_empty[s]), (uint32_t)kPsTransposeWarps);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(smem_u32(&pm_full[a]), (uint32_t)kPsTransposeWarps);
+            mbar_init(smem_u32(&pm_empty[a]), 1u);
+            mbar_init(smem_u32(&acc_full[a]), 1u);
+            mbar_init(smem_u32(&acc_empty[a]), (uint32_t)kPsEpilogueWarps);
+        }
+        abort_flag = 0;
+        fence_mbar_init();
+        fence_proxy_async_shared();
+    }
+    if (warp == 1) {
+        tmem_alloc(smem_u32(&tmem_slot), g.tmem_cols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *(volatile uint32_t*)&tmem_slot;
+    pdl_wait_prev();                                      // the set-up above touched no global memory
+
+    auto decode = [&](int i, int& m0, int& n0, int& bz) {
+        const int t = unit + i * n_units;
+        bz = t / tiles_per_batch;
+        const int r = t - bz * tiles_per_batch;
+        int tm, tn;
+        if (g.raster == 0) { tm = r % g.tiles_m; tn = r / g.tiles_m; }
+        else               { tn = r % g.tiles_n; tm = r / g.tiles_n; }
+        m0 = tm * kHwTileM;
+        n0 = tn * g.tile_n;
+    };
+
+    if (warp == 0) {
+        // ---------------- TMA producer ----------------
+        // Two independent streams of requests, each with its own ring and cursor: NCHW boxes of input rows go to the staging
+        // ring, filter tiles to the pipeline stages.  The warp polls both rings and serves whichever has a free slot.
+        const bool leader = elect_one();
+        const uint32_t a_atom = (uint32_t)(kHwTileM * g.row_bytes);
         struct Cursor { int i, kt, m0, n0, bz, slot; uint32_t ph; long long it; };
         const long long total_it = (long long)my_tiles * kt_n;
-        const int inner_s = tapm ? blocks_per_tile : kt_n;            // staging boxes per tile
-        const long long total_s = (long long)my_tiles * inner_s;
+        const long long total_s = (long long)my_tiles * blocks_per_tile;    // a staging box per 32-channel block
         auto cur_init = [&](Cursor& c) {
             c.i = 0; c.kt = 0; c.slot = 0; c.ph = 0; c.it = 0; c.m0 = c.n0 = c.bz = 0;
             if (my_tiles > 0) decode(0, c.m0, c.n0, c.bz);
@@ -1866,61 +2237,33 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         };
         Cursor cs, ck;
         cur_init(cs); cur_init(ck);
-        if (!any_stg) cs.it = total_s;
-        if (!any_km) ck.it = total_it;
         bool ok = true;
         unsigned long long t_last = global_timer_ns();
         unsigned idle = 0;
         while (cs.it < total_s || ck.it < total_it) {
             bool progressed = false;
             if (cs.it < total_s && mbar_test_wait(smem_u32(&stg_empty[cs.slot]), cs.ph ^ 1u)) {
-                if (leader && tapm) {
+                if (leader) {
                     // the input rows of 32-channel block cs.kt behind this tile's pixels: one box that starts `gap` columns
                     // left of the image and at the tile's first input row (zero fill supplies padding and gaps)
                     const uint32_t bar = smem_u32(&stg_full[cs.slot]);
                     mbar_expect_tx(bar, g.slab_box_bytes);
                     tma_load_4d(tiles_base + g.slab_off + (uint32_t)cs.slot * g.slab_buf_bytes, &tmap_x, bar, -g.slab_gap,
                                 cs.n0 / g.slab_wp - g.ph, cs.kt * 32, cs.bz);
-                } else if (leader) {
-                    const uint32_t bar = smem_u32(&stg_full[cs.slot]);
-                    const int k0 = cs.kt * g.tile_k;
-                    mbar_expect_tx(bar, mn_bytes);
-                    if (a_mn) tma_load_3d(tiles_base + g.a_stg_off + (uint32_t)cs.slot * g.stg_a_bytes, &tmap_a, bar, cs.m0, k0, g.a_tma_batched ? cs.bz : 0);
-                    if (b_mn) tma_load_3d(tiles_base + g.b_stg_off + (uint32_t)cs.slot * g.stg_b_bytes, &tmap_b, bar, cs.n0 + (int)rank * b_rows, k0,
-                                          g.b_tma_batched ? cs.bz : 0);
                 }
                 __syncwarp();
-                cur_next(cs, g.stg_depth, inner_s);
+                cur_next(cs, g.stg_depth, blocks_per_tile);
                 progressed = true;
             }
             if (ck.it < total_it && mbar_test_wait(smem_u32(&empty_bar[ck.slot]), ck.ph ^ 1u)) {
                 if (leader) {
-                    uint32_t bar = smem_u32(&full_bar[ck.slot]);
-                    const int k0 = ck.kt * g.tile_k;
-                    const int nb0 = ck.n0 + (int)rank * b_rows;       // CG 2: this CTA's half of the B rows
-                    const int a_bz = g.a_tma_batched ? ck.bz : 0, b_bz = g.b_tma_batched ? ck.bz : 0;
+                    const uint32_t bar = smem_u32(&full_bar[ck.slot]);
                     // (test facility: the first stage may be told to expect more than arrives, see tt_workload_test_stall)
-                    if (rank == 0) mbar_expect_tx(bar, (uint32_t)CG * km_bytes + (ck.it == 0 ? g.extra_tx : 0u));
-                    if constexpr (CG == 2) bar = map_to_peer(bar, 0u);       // the pair's loads all report to rank 0
-                    const uint32_t a_dst = tiles_base + (uint32_t)ck.slot * stage_bytes;
-                    if (!a_mn) {
-                        uint32_t dst = a_dst;
-                        int kc = k0;
+                    mbar_expect_tx(bar, g.a_stage_bytes + (ck.it == 0 ? g.extra_tx : 0u));
+                    uint32_t dst = tiles_base + (uint32_t)ck.slot * stage_bytes;
+                    int kc = ck.kt * g.tile_k;
 #pragma unroll 1
-                        for (int at = 0; at < g.n_atoms; ++at, dst += a_atom, kc += g.atom_k) {
-                            if constexpr (CG == 2) tma_load_3d_pair(dst, &tmap_a, bar, kc, ck.m0, a_bz);
-                            else tma_load_3d(dst, &tmap_a, bar, kc, ck.m0, a_bz);
-                        }
-                    }
-                    if (!b_mn && !tapm) {
-                        uint32_t dst = a_dst + g.a_stage_bytes;
-                        int kc = k0;
-#pragma unroll 1
-                        for (int at = 0; at < g.n_atoms; ++at, dst += b_atom, kc += g.atom_k) {
-                            if constexpr (CG == 2) tma_load_3d_pair(dst, &tmap_b, bar, kc, nb0, b_bz);
-                            else tma_load_3d(dst, &tmap_b, bar, kc, nb0, b_bz);
-                        }
-                    }
+                    for (int at = 0; at < g.n_atoms; ++at, dst += a_atom, kc += g.atom_k) tma_load_3d(dst, &tmap_a, bar, kc, ck.m0, 0);
                 }
                 __syncwarp();
                 cur_next(ck, g.stages, kt_n);
@@ -1944,7 +2287,6 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             for (int pass = 0; pass < 2; ++pass) {
                 const long long issued = pass == 0 ? ck.it : cs.it;
                 const int depth = pass == 0 ? g.stages : g.stg_depth;
-                if ((pass == 0 && (!any_km || rank != 0)) || (pass == 1 && !any_stg)) continue;
                 const long long first = issued > depth ? issued - depth : 0;
                 for (long long it = first; it < issued; ++it) {
                     const uint32_t bar = pass == 0 ? smem_u32(&full_bar[it % depth]) : smem_u32(&stg_full[it % depth]);
@@ -1953,38 +2295,28 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                     while (!mbar_try_wait(bar, par)) { if (global_timer_ns() - t0 > 2000000ull) break; }
                 }
             }
-            if (rank != 0) {
-                // this CTA's K-major loads report to rank 0's barriers: give them time to land instead (the pair leaves
-                // together, after rank 0 has seen the pair's bytes or given up on them)
-                const unsigned long long t0 = global_timer_ns();
-                while (global_timer_ns() - t0 < 200000ull) { }
-            }
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ---------------- MMA issuer (of a pair: rank 0's) ----------------
+        // ---------------- MMA issuer ----------------
         const bool leader = elect_one();
         uint32_t st = 0, ph = 0;
         bool ok = true;
-        if (CG == 2 && rank != 0) {
-            // rank 0 issues for the pair
-        } else {
+        {
             const uint64_t d0 = make_desc(0u, g.row_bytes);
             const uint32_t d_hi = (uint32_t)(d0 >> 32), d_lo = (uint32_t)d0;
             const uint32_t a_lo0 = d_lo + ((tiles_base & 0x3FFFFu) >> 4);
             const uint32_t stage_step = stage_bytes >> 4;
-            const uint32_t a_atom = (uint32_t)(kHwTileM * g.row_bytes) >> 4, b_atom = (uint32_t)(b_rows * g.row_bytes) >> 4;
-            const uint32_t b_off = g.a_stage_bytes >> 4;
+            const uint32_t a_atom = (uint32_t)(kHwTileM * g.row_bytes) >> 4;
             uint32_t gblock = 0;                         // tap-major: 32-channel blocks consumed so far, over all tiles
             for (int i = 0; i < my_tiles && ok; ++i) {
                 const uint32_t acc = (uint32_t)i & 1u, aph = ((uint32_t)i >> 1) & 1u;
                 // the read-out of the tile that used this accumulator two tiles ago has finished
-                const bool freed = CG == 2 ? mbar_wait_cluster(smem_u32(&acc_empty[acc]), aph ^ 1u, abortp, g.status, 12u, g.wait_ns)
-                                           : mbar_wait(smem_u32(&acc_empty[acc]), aph ^ 1u, abortp, g.status, 12u, g.wait_ns);
+                const bool freed = mbar_wait(smem_u32(&acc_empty[acc]), aph ^ 1u, abortp, g.status, 12u, g.wait_ns);
                 if (!__all_sync(0xffffffffu, freed)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)g.tile_n;
-                if (tapm) {
+                {
                     // the B tile of reduction tile kt = (channel block, taps) is the block's pixel-major slab read from row
                     // lin0 + r * wp + s on: only the descriptor's start address changes from tap to tap
                     int m0t, n0t, bzt;
@@ -2006,13 +2338,13 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                                 const uint32_t b_lo = d_lo + (((pm0 + (gblock & 1u) * g.pm_buf_bytes + row * 128u) & 0x3FFFFu) >> 4);
 #pragma unroll
                                 for (int k8 = 0; k8 < 4; ++k8)
-                                    mma_tf32_cg<CG>(d_tmem, ((uint64_t)d_hi << 32) | (uint64_t)(a_lo + 2u * (uint32_t)k8),
+                                    mma_tf32(d_tmem, ((uint64_t)d_hi << 32) | (uint64_t)(a_lo + 2u * (uint32_t)k8),
                                                     ((uint64_t)d_hi << 32) | (uint64_t)(b_lo + 2u * (uint32_t)k8), g.idesc,
                                                     (kt > 0 || t > 0 || k8 > 0) ? 1u : 0u);
                                 if (++s2 == g.S) { s2 = 0; ++r2; }
                             }
-                            mma_commit_cg<CG>(smem_u32(&empty_bar[st]));                           // filter stage reusable
-                            if (tap + g.n_atoms == RS) mma_commit_cg<CG>(smem_u32(&pm_empty[gblock & 1u]));   // slab buffer reusable
+                            mma_commit(smem_u32(&empty_bar[st]));                           // filter stage reusable
+                            if (tap + g.n_atoms == RS) mma_commit(smem_u32(&pm_empty[gblock & 1u]));   // slab buffer reusable
                         }
                         __syncwarp();
                         for (int t = 0; t < g.n_atoms; ++t) if (++fs == g.S) { fs = 0; ++fr; }
@@ -2020,35 +2352,14 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                         if (tap == RS) { tap = 0; fr = 0; fs = 0; ++gblock; }
                         if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
                     }
-                } else
-                for (int kt = 0; kt < kt_n; ++kt) {
-                    const bool got = mbar_wait(smem_u32(&full_bar[st]), ph, abortp, g.status, 2u, g.wait_ns);
-                    if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-                    tc_fence_after();
-                    if (leader) {
-                        const uint32_t a_lo = a_lo0 + st * stage_step, b_lo = a_lo + b_off;
-                        const uint32_t accumulate = kt > 0 ? 1u : 0u;
-#pragma unroll 1
-                        for (int at = 0; at < g.n_atoms; ++at) {
-                            const int k8n = g.atom_k >> 3;
-#pragma unroll 4
-                            for (int k8 = 0; k8 < k8n; ++k8)
-                                mma_tf32_cg<CG>(d_tmem, ((uint64_t)d_hi << 32) | (uint64_t)(a_lo + (uint32_t)at * a_atom + 2u * (uint32_t)k8),
-                                                ((uint64_t)d_hi << 32) | (uint64_t)(b_lo + (uint32_t)at * b_atom + 2u * (uint32_t)k8), g.idesc,
-                                                (at == 0 && k8 == 0) ? accumulate : 1u);
-                        }
-                        mma_commit_cg<CG>(smem_u32(&empty_bar[st]));          // stage reusable once these MMAs have read it
-                    }
-                    __syncwarp();
-                    if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
                 }
-                if (ok && leader) mma_commit_cg<CG>(smem_u32(&acc_full[acc]));   // the tile's accumulator is complete
+                if (ok && leader) mma_commit(smem_u32(&acc_full[acc]));   // the tile's accumulator is complete
                 __syncwarp();
             }
         }
     } else if (warp < 2 + kPsTransposeWarps) {
         // ---------------- transposers ----------------
-        if (tapm) {
+        {
             // staging box [32 channels][in_rows][wp] -> pixel-major slab: one 128-byte row per staged position (32
             // channels), 16-byte chunks swizzled by the row's absolute address like a TMA 128-byte tile.  Warp tw moves
             // the channel groups tw and tw + 4 of every position; lanes walk positions.
@@ -2105,28 +2416,6 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 }
                 if (++sst == (uint32_t)g.stg_depth) { sst = 0; sph ^= 1u; }
             }
-        } else if (any_mn) {
-            const int grp = (warp - 2) / tr_warps, tw = (warp - 2) - grp * tr_warps;
-            int st = grp % g.stages, sst = grp % g.stg_depth;
-            uint32_t ph = (uint32_t)(grp / g.stages) & 1u, sph = (uint32_t)(grp / g.stg_depth) & 1u;
-            const long long total_it = (long long)my_tiles * kt_n;
-            for (long long it = grp; it < total_it; it += tr_groups) {
-                if (!mbar_wait(smem_u32(&stg_full[sst]), sph, abortp, g.status, 6u, g.wait_ns) ||
-                    !mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1u, abortp, g.status, 3u, g.wait_ns)) break;
-                const uint32_t a_s = tiles_base + (uint32_t)st * stage_bytes, b_s = a_s + g.a_stage_bytes;
-                if (a_mn) ps_transpose(tiles_base + g.a_stg_off + (uint32_t)sst * g.stg_a_bytes, a_s, kHwTileM, g.tile_k, g.atom_k, g.row_bytes, g.swz_mask, tw, tr_warps, lane);
-                if (b_mn) ps_transpose(tiles_base + g.b_stg_off + (uint32_t)sst * g.stg_b_bytes, b_s, b_rows, g.tile_k, g.atom_k, g.row_bytes, g.swz_mask, tw, tr_warps, lane);
-                fence_proxy_async_shared();              // generic-proxy stores -> visible to the tensor core's reads
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(smem_u32(&full_bar[st]));
-                    mbar_arrive(smem_u32(&stg_empty[sst]));
-                }
-                st += tr_groups;
-                while (st >= g.stages) { st -= g.stages; ph ^= 1u; }
-                sst += tr_groups;
-                while (sst >= g.stg_depth) { sst -= g.stg_depth; sph ^= 1u; }
-            }
         }
     } else {
         // ---------------- read-out: tensor memory -> bias, residual, activation -> global memory ----------------
@@ -2139,7 +2428,7 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         e.hi = g.act == TT_ACT_RELU6 ? 6.f : INFINITY;
         e.gelu = g.act == TT_ACT_GELU_ERF;
         e.vec = (g.vec_store & 1) != 0;
-        e.lin_wp = tapm ? g.slab_wp : 0; e.lin_q = g.Q; e.lin_p = g.Pout;
+        e.lin_wp = g.slab_wp; e.lin_q = g.Q; e.lin_p = g.Pout;
         const bool transposed = g.y_ns == 1 && g.y_ms != 1;
         const uint32_t stg = tiles_base + g.epi_off + (uint32_t)ew * (uint32_t)kStageBytesPerWarp;
         bool ok = true;
@@ -2181,8 +2470,7 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) {
-                        if (CG == 2) mbar_arrive_remote(smem_u32(&acc_empty[acc]), 0u);
-                        else mbar_arrive(smem_u32(&acc_empty[acc]));
+                        mbar_arrive(smem_u32(&acc_empty[acc]));
                     }
                 }
                 if (cnt <= 0) continue;                  // warp-uniform
@@ -2196,7 +2484,6 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                         v[j] += b.x; v[j + 1] += b.y; v[j + 2] += b.z; v[j + 3] += b.w;
                     }
                 }
-                const bool full = !tapm && cnt >= 32 && m_first + 32 <= g.M && (e.vec || !transposed);
                 if (e.rbase == nullptr) {
                     if (e.gelu) {
 #pragma unroll
@@ -2205,24 +2492,19 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
 #pragma unroll
                         for (int j = 0; j < 32; ++j) v[j] = fminf(fmaxf(v[j], e.lo), e.hi);
                     }
-                    if (full) epilogue_block<true, false>(v, e, m_first, nb, cnt, stg, lane, transposed);
-                    else epilogue_block<false, false>(v, e, m_first, nb, cnt, stg, lane, transposed);
+                    epilogue_block<false, false>(v, e, m_first, nb, cnt, stg, lane, transposed);
                 } else {
-                    if (full) epilogue_block<true, true>(v, e, m_first, nb, cnt, stg, lane, transposed);
-                    else epilogue_block<false, true>(v, e, m_first, nb, cnt, stg, lane, transposed);
+                    epilogue_block<false, true>(v, e, m_first, nb, cnt, stg, lane, transposed);
                 }
             }
         }
     }
     tc_fence_before();
     __syncthreads();
-    // a pair stays together until neither CTA touches the other's shared memory, barriers or tensor memory any more
-    if constexpr (CG == 2) cluster_sync_all();
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
-        if constexpr (CG == 1) tmem_dealloc(tmem_base, g.tmem_cols);
-        else asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(g.tmem_cols) : "memory");
+        tmem_dealloc(tmem_base, g.tmem_cols);
     }
 }
 
@@ -2825,18 +3107,41 @@ __global__ void tt_floor_kernel() {
 // system's, plus the kernel's static part) and half of its 512 tensor-memory columns.
 static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <= 112 * 1024 && tmem_cols <= 256; }
 
-cudaError_t launch_gemm(const tt_apply_info& I, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
-                        cudaStream_t st) {
-    static int attr_set_for = -1;
+typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
+static const GemmKernel kGemmKernels[2][5] = {
+    {tt_gemm_tc_kernel<1, kFormTma>, tt_gemm_tc_kernel<1, kFormMn>, tt_gemm_tc_kernel<1, kFormIm2col>, tt_gemm_tc_kernel<1, kFormTap>, tt_gemm_tc_kernel<1, kFormGather>},
+    {tt_gemm_tc_kernel<2, kFormTma>, tt_gemm_tc_kernel<2, kFormMn>, tt_gemm_tc_kernel<2, kFormIm2col>, tt_gemm_tc_kernel<2, kFormTap>, tt_gemm_tc_kernel<2, kFormGather>}};
+
+static int gemm_form(const GemmArgs& g) {
+    if (g.tap_major) return kFormTap;
+    if (g.a_mode == OPM_IM2COL || g.b_mode == OPM_IM2COL) return kFormIm2col;
+    const bool a = g.a_mode == OPM_TMA || g.a_mode == OPM_TMA_MN, b = g.b_mode == OPM_TMA || g.b_mode == OPM_TMA_MN;
+    if (!a || !b) return kFormGather;
+    return g.a_mode == OPM_TMA && g.b_mode == OPM_TMA ? kFormTma : kFormMn;
+}
+
+// Which instantiation a plan runs; its shared-memory limit is raised once per device.  Which build (two CTAs per SM) is the
+// record's choice (ctas_per_sm), resolved by the legaliser.
+static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel* out) {
+    static std::atomic<uint64_t> raised[2][5];           // a bit per device
+    const int two = g.two_per_sm && gemm_two_per_sm(smem_bytes, g.tmem_cols), form = gemm_form(g);
     int dev = 0;
     cudaGetDevice(&dev);
-    if (attr_set_for != dev) {
-        cudaError_t e = cudaFuncSetAttribute(tt_gemm_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+    const uint64_t bit = 1ull << (dev & 63);
+    *out = kGemmKernels[two][form];
+    if (!(raised[two][form].load(std::memory_order_relaxed) & bit)) {
+        cudaError_t e = cudaFuncSetAttribute(*out, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(tt_gemm_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-        if (e != cudaSuccess) return e;
-        attr_set_for = dev;
+        raised[two][form].fetch_or(bit, std::memory_order_relaxed);
     }
+    return cudaSuccess;
+}
+
+cudaError_t launch_gemm(const tt_apply_info& I, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
+                        cudaStream_t st) {
+    GemmKernel kern;
+    const cudaError_t e = gemm_kernel_for(g, I.smem_bytes, &kern);
+    if (e != cudaSuccess) return e;
     CUtensorMap ta, tb, tx;
     memcpy(&ta, tmap_a, sizeof ta);
     memcpy(&tb, tmap_b, sizeof tb);
@@ -2858,29 +3163,25 @@ cudaError_t launch_gemm(const tt_apply_info& I, const GemmArgs& g, const void* t
         ++n_attr;
     }
     cfg.attrs = attr; cfg.numAttrs = (unsigned)n_attr;
-    // which build runs is the record's choice (ctas_per_sm), resolved by the legaliser
-    if (g.two_per_sm && gemm_two_per_sm(I.smem_bytes, g.tmem_cols)) return cudaLaunchKernelEx(&cfg, tt_gemm_tc_kernel<2>, ta, tb, tx, g);
-    return cudaLaunchKernelEx(&cfg, tt_gemm_tc_kernel<1>, ta, tb, tx, g);
+    return cudaLaunchKernelEx(&cfg, kern, ta, tb, tx, g);
 }
 
 // The persistent form: one CTA (or one pair of CTAs, as a cluster of two) per SM.
-cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
-                           cudaStream_t st) {
+cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const TmapPair& maps, cudaStream_t st) {
     static int attr_set_for = -1, sm_count = 148;
     int dev = 0;
     cudaGetDevice(&dev);
     if (attr_set_for != dev) {
         cudaError_t e = cudaFuncSetAttribute(tt_gemm_ps_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(tt_gemm_ps_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tt_gemm_ps_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tt_gemm_ps_tap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
         if (e != cudaSuccess) return e;
         cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
         attr_set_for = dev;
     }
-    CUtensorMap ta, tb, tx;
-    memcpy(&ta, tmap_a, sizeof ta);
-    memcpy(&tb, tmap_b, sizeof tb);
-    memcpy(&tx, tmap_x, sizeof tx);
+    CUtensorMap ta, tb, tx, ty, tr;
+    memcpy(&ta, maps.a, sizeof ta);
+    memcpy(&tb, maps.b, sizeof tb);
     const int cg = g.cta_group == 2 ? 2 : 1;
     const long long units = std::min<long long>(g.total_tiles, sm_count / cg);
     cudaLaunchConfig_t cfg{};
@@ -2897,22 +3198,29 @@ cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const void
         ++n_attr;
     }
     cfg.attrs = attr; cfg.numAttrs = (unsigned)n_attr;
-    if (cg == 2) return cudaLaunchKernelEx(&cfg, tt_gemm_ps_kernel<2>, ta, tb, tx, g);
-    return cudaLaunchKernelEx(&cfg, tt_gemm_ps_kernel<1>, ta, tb, tx, g);
+    if (g.tap_major) {
+        memcpy(&tx, maps.x, sizeof tx);
+        return cudaLaunchKernelEx(&cfg, tt_gemm_ps_tap_kernel, ta, tx, g);
+    }
+    memcpy(&ty, maps.y, sizeof ty);
+    memcpy(&tr, maps.r, sizeof tr);
+    if (cg == 2) return cudaLaunchKernelEx(&cfg, tt_gemm_ps_kernel<2>, ta, tb, ty, tr, g);
+    return cudaLaunchKernelEx(&cfg, tt_gemm_ps_kernel<1>, ta, tb, ty, tr, g);
 }
 
-// Can a cluster of `cluster` CTAs with this much shared memory each be resident at all?
-cudaError_t gemm_cluster_fits(int smem_bytes, int cluster, int* fits) {
-    cudaError_t e = cudaFuncSetAttribute(tt_gemm_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+// Can a cluster of a plan's CTAs be resident at all?
+cudaError_t gemm_cluster_fits(const GemmArgs& g, int smem_bytes, int* fits) {
+    GemmKernel kern;
+    cudaError_t e = gemm_kernel_for(g, smem_bytes, &kern);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(1, (unsigned)cluster, 1); cfg.blockDim = dim3(kGemmThreads, 1, 1); cfg.dynamicSmemBytes = (size_t)smem_bytes;
+    cfg.gridDim = dim3(1, (unsigned)g.cluster, 1); cfg.blockDim = dim3(kGemmThreads, 1, 1); cfg.dynamicSmemBytes = (size_t)smem_bytes;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = (unsigned)cluster; attr[0].val.clusterDim.z = 1;
+    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = (unsigned)g.cluster; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, tt_gemm_tc_kernel<1>, &cfg);   // the other build needs no more of anything
+    e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
     if (e != cudaSuccess) return e;
     *fits = n > 0;
     return cudaSuccess;

@@ -962,3 +962,28 @@ def test_softmax_ragged_rows(cols):
     ref = util.oracle_ref(spec, a)
     for bx in (1, 4, 16, 32):
         run_spec(spec, B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=bx, block_y=8, vec_width=4), a, ref, ref_elem=ref)
+
+
+@pytest.mark.parametrize("spec", [
+    W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(40, 20, 14, 14, 200, 1, 1, 1, 0, True, B.TT_ACT_RELU, True), 1, "mn_conv1x1_res_n40", "uniform"),
+    W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(3, 33, 6, 6, 17, 1, 1, 1, 0, True, B.TT_ACT_RELU6, True), 1, "mn_conv1x1_c33", "uniform"),
+    W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(5, 70, 132, 36, False), 1, "mn_bmm_nn_ragged", "bert"),
+    W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(3, 130, 44, 35, False), 1, "mn_bmm_nn_gathered_a", "bert"),
+], ids=lambda s: s.name)
+def test_mn_major_operands_and_tma_read_out(spec):
+    """Operands whose row index is the contiguous one, multiplied as they lie: boxes of 32 rows with tails in rows and in
+    K, tiles of less than a box, split-K through a cluster and through the workspace, several accumulators, the residual
+    read ahead through the read-out's ring (several tiles per CTA, both output orders, tiles that are no whole blocks)."""
+    a = W.make_inputs(spec, 93)
+    ref = util.oracle_ref(spec, a)
+    re = elem_ref(spec, a, ref)
+    probe = spec.workload()
+    recs = [tc(tile_n=tn, tile_k=tk, stages=st, mma_m_axis=ax, persistent=ps, split_k=sk, acc_split=acc, slab_tiles=sl)
+            for tn, tk, st, ax, ps, sk, acc, sl in (
+                (16, 8, 2, 1, 0, 1, 1, 0), (48, 16, 3, 1, 0, 3, 1, 0), (64, 32, 2, 2, 0, 2, 2, 0), (256, 64, 1, 1, 0, 1, 1, 0),
+                (32, 8, 2, 2, 0, 12, 1, 0), (32, 32, 2, 1, 1, 1, 1, 0), (64, 16, 8, 1, 1, 1, 1, 2), (256, 32, 2, 1, 1, 1, 1, 0),
+                (48, 32, 2, 1, 1, 1, 1, 3), (32, 64, 2, 2, 1, 1, 1, 0), (160, 32, 1, 2, 1, 1, 1, 1))]
+    for rec in recs:
+        assert probe.check(rec)[0] == B.TT_OK
+        run_spec(spec, rec, a, ref, ref_elem=re)
+    probe.close()
