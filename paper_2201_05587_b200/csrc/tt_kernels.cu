@@ -810,7 +810,7 @@ enum GemmForm {
     kFormMn = 1,        // both by TMA, one of them (or both) MN-major
     kFormIm2col = 2,    // one operand expanded from a slab of input rows, the other by TMA or gathered
     kFormTap = 3,       // tap-major convolution
-    kFormGather = 4     // an operand gathered from global memory
+    kFormGather = 4     // an operand gathered from global memory (the other one any way but by expansion)
 };
 
 template <int MIN_CTAS, int FORM>
@@ -855,9 +855,10 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     const uint32_t stage_bytes = FORM == kFormTma && g.x3 ? 2u * lo_off : lo_off;
     // what the instantiation is made for (GemmForm); within it only the modes that its form leaves open are looked at
     constexpr bool im2col = FORM == kFormIm2col, tapm = FORM == kFormTap;     // tapm: reduction walked by channel block and tap
-    const bool a_mn = FORM == kFormMn && g.a_mode == OPM_TMA_MN, b_mn = FORM == kFormMn && g.b_mode == OPM_TMA_MN;
-    const bool a_tma = FORM == kFormTma || FORM == kFormMn || FORM == kFormTap || g.a_mode == OPM_TMA;
-    const bool b_tma = FORM == kFormTma || FORM == kFormMn || (FORM != kFormTap && g.b_mode == OPM_TMA);
+    constexpr bool may_mn = FORM == kFormMn || FORM == kFormGather;
+    const bool a_mn = may_mn && g.a_mode == OPM_TMA_MN, b_mn = may_mn && g.b_mode == OPM_TMA_MN;
+    const bool a_tma = FORM == kFormTma || FORM == kFormMn || FORM == kFormTap || g.a_mode == OPM_TMA || a_mn;
+    const bool b_tma = FORM == kFormTma || FORM == kFormMn || (FORM != kFormTap && (g.b_mode == OPM_TMA || b_mn));
     const bool any_tma = a_tma || b_tma, any_gather = !a_tma || !b_tma;
     const bool slab_tma = (im2col || tapm) && g.slab_tma != 0;
     const bool x3 = FORM == kFormTma && g.x3 != 0;       // error-compensated products
