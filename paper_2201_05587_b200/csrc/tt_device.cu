@@ -17,7 +17,9 @@ cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st)
 cudaError_t launch_dw_tma(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st);
 cudaError_t launch_row(const tt_apply_info& I, const RowArgs& row, cudaStream_t st);
 cudaError_t gemm_cluster_fits(const GemmArgs& g, int smem_bytes, int* fits);
-cudaError_t launch_repack(const float* w, float* out, int kout, int C, int RS, int CB, cudaStream_t st);
+cudaError_t launch_repack(const float* w, float* out, const ConvPmArgs& g, cudaStream_t st);
+cudaError_t launch_conv_pm(const tt_apply_info& I, const ConvPmArgs& g, const void* tmap_w, cudaStream_t st);
+cudaError_t conv_pm_cluster_fits(const tt_apply_info& I, const ConvPmArgs& g, int* fits);
 cudaError_t launch_floor(const tt_apply_info& I, int cluster, cudaStream_t st);
 cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const TmapPair& maps, cudaStream_t st);
 
@@ -193,6 +195,11 @@ tt_status bind_device(tt_workload* w) {
         if (gemm_cluster_fits(w->plan.g, w->plan.info.smem_bytes, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
         if (!fits) return TT_ERR_RESOURCE;
     }
+    if (w->family == TT_FAMILY_GEMM_TC && w->plan.repack && w->plan.pm.split > 1) {
+        int fits = 0;
+        if (conv_pm_cluster_fits(w->plan.info, w->plan.pm, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+        if (!fits) return TT_ERR_RESOURCE;
+    }
     const size_t need = (size_t)w->plan.info.workspace_bytes;
     if (need > w->workspace_bytes) {
         if (w->workspace) cudaFree(w->workspace);
@@ -288,6 +295,29 @@ static tt_status tensor_maps_for(tt_workload* w, const GemmArgs& g, const void* 
     return TT_OK;
 }
 
+// Tap-major convolution: the filters are brought into walk order first, once per weight pointer and applied record where
+// the caller has promised that they are constant.
+static tt_status launch_tap_major(tt_workload* w, const tt_tensors* t, cudaStream_t st) {
+    const Plan& p = w->plan;
+    bool repacked_now = false;
+    if (!(w->constant_weights && w->repacked_for == t->w)) {
+        if (launch_repack(static_cast<const float*>(t->w), static_cast<float*>(w->workspace), p.pm, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+        w->repacked_for = t->w;
+        repacked_now = true;
+    }
+    const TmapPair* maps = nullptr;
+    const tt_status s = tensor_maps_for(w, p.g, w->workspace, nullptr, &maps);
+    if (s != TT_OK) return s;
+    ConvPmArgs c = p.pm;
+    c.x = static_cast<const float*>(t->x); c.y = static_cast<float*>(t->y);
+    c.bias = w->sh.has_bias ? static_cast<const float*>(t->bias) : nullptr;
+    c.residual = w->sh.has_residual ? static_cast<const float*>(t->residual) : nullptr;
+    c.status = w->status_word; c.wait_ns = w->wait_ns; c.extra_tx = w->extra_tx;
+    c.early_filters = w->constant_weights && !repacked_now;
+    if (launch_conv_pm(p.info, c, maps->a, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+    return TT_OK;
+}
+
 tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
     if (!w || !t) return TT_ERR_INVALID_ARG;
     if (!w->plan.applied) return TT_ERR_NOT_APPLIED;
@@ -299,21 +329,10 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
     cudaError_t e = cudaSuccess;
     const Plan& p = w->plan;
     if (w->family == TT_FAMILY_GEMM_TC) {
+        if (p.repack) return launch_tap_major(w, t, st);
         GemmArgs g = p.g;
         const void* a_ptr = pick(t, p.a_tensor);
         const void* b_ptr = pick(t, p.b_tensor);
-        bool repacked_now = false;
-        if (p.repack) {
-            // tap-major convolution: the filters are brought into [filter][32-channel block][tap][channel] order first.
-            // Constant weights (the caller's promise) are re-packed once per weight pointer and applied record.
-            if (!(w->constant_weights && w->repacked_for == t->w)) {
-                if (launch_repack(static_cast<const float*>(t->w), static_cast<float*>(w->workspace), g.M, g.C, g.R * g.S,
-                                  p.repack_cb, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
-                w->repacked_for = t->w;
-                repacked_now = true;
-            }
-            a_ptr = w->workspace;
-        }
         g.a = static_cast<const float*>(a_ptr);
         g.b = static_cast<const float*>(b_ptr);
         g.y = static_cast<float*>(t->y);
@@ -330,7 +349,7 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
         g.wait_ns = w->wait_ns;
         g.extra_tx = w->extra_tx;
         g.w_operand = 0;
-        if (w->constant_weights && !repacked_now && !g.persistent && (w->op == TT_OP_DENSE || w->op == TT_OP_CONV2D)) {
+        if (w->constant_weights && !g.persistent && (w->op == TT_OP_DENSE || w->op == TT_OP_CONV2D)) {
             if (p.a_tensor == 1 && g.a_mode == OPM_TMA) g.w_operand = 1;
             else if (p.b_tensor == 1 && g.b_mode == OPM_TMA) g.w_operand = 2;
         }
@@ -433,7 +452,7 @@ static tt_status time_applied(tt_workload* w, const tt_tensors* sets, size_t n_s
             if (o.floor) {
                 // the launch floor of the applied record: an empty kernel with the same launch shape
                 for (int l = 0; l < w->plan.info.launches; ++l)
-                    if (launch_floor(w->plan.info, w->family == TT_FAMILY_GEMM_TC ? w->plan.g.cluster : 0, s) != cudaSuccess) {
+                    if (launch_floor(w->plan.info, w->family != TT_FAMILY_GEMM_TC ? 0 : w->plan.repack ? (w->plan.pm.split > 1 ? w->plan.pm.split : 0) : w->plan.g.cluster, s) != cudaSuccess) {
                         cudaGetLastError();
                         return TT_ERR_CUDA;
                     }

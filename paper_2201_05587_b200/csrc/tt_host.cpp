@@ -82,18 +82,35 @@ size_t tensor_elems(const tt_workload* w, int which) {
 
 // ---- legalisation -------------------------------------------------------------------------------------------
 
-// conv2d with k_order = 1: the reduction walks blocks of 32 channels and, inside a block, tap by tap.  Filters are
-// re-packed into that order ([filter][block][tap][32 channels], zero-padded) before each run and arrive by TMA;
-// the output columns are padded-linear pixels n = p * (W + gap) + q', so that the operand tile of tap (r, s) is the
-// pixel-major slab read (r * (W + gap) + s) rows further down -- a view, no expansion.  Columns with q' >= Q are
-// computed and dropped.
+// conv2d with k_order = 1: the reduction walks blocks of 32 channels and, inside a block, tap by tap (tt_conv.cu).  Filters
+// are re-packed into that order by a kernel of its own, once per weight pointer, which single images of other layouts
+// would not earn back: the order exists for stride-1 convolutions with 16-byte image rows and, for any stride and row length,
+// from two images on.
 static bool tap_major_possible(const tt_workload* w) {
     const tt_shapes& s = w->sh;
-    const int gap = round_up(std::max(1, std::max(s.pad_w, s.s - 1 - s.pad_w)), 4);
-    // (an output row must fit a padded image row: the columns are numbered p * (W + gap) + q')
-    return w->op == TT_OP_CONV2D && s.stride_h == 1 && s.stride_w == 1 && (s.w % 4) == 0 && !s.has_residual &&
-           s.r * s.s <= 64 && (long long)w->P * w->Q > 1 && w->Q <= s.w + gap;
+    return w->op == TT_OP_CONV2D && s.r * s.s <= 64 && (long long)w->P * w->Q > 1 && s.stride_h * s.stride_w <= kPmMaxPlanes &&
+           s.r < 100 && s.s < 100 && s.pad_h < 100 && s.pad_w < 100 && ((s.stride_h == 1 && s.stride_w == 1 && (s.w % 4) == 0) || s.n >= 2);
 }
+
+namespace {
+int floor_div(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
+// One axis of the padded-linear numbering: per parity class the first tap, its shift, the number of taps; the positions that a
+// row (or an image) takes so that taps which reach past its end find zeros.
+struct TapAxis { int first[16], shift[16], count[16], lo, hi, pitch; };
+TapAxis tap_axis(int taps, int stride, int pad, int extent, int outputs) {
+    TapAxis t{};
+    t.lo = floor_div(-pad, stride); t.hi = floor_div(taps - 1 - pad, stride);
+    for (int a = 0; a < stride; ++a)
+        for (int r = 0; r < taps; ++r) {
+            if (r - pad - stride * floor_div(r - pad, stride) != a) continue;
+            if (t.count[a]++ == 0) { t.first[a] = r; t.shift[a] = floor_div(r - pad, stride); }
+        }
+    const int data = (extent + stride - 1) / stride;
+    t.pitch = std::max(data + std::max(0, -t.lo), outputs + std::max(0, t.hi));
+    return t;
+}
+unsigned magic_of(int d) { return d == 1 ? 0xffffffffu : (unsigned)(0x100000000ull / (unsigned)d); }
+}  // namespace
 
 static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_record* rec, int mode, Plan* plan) {
     tt_apply_info& I = plan->info;
@@ -102,13 +119,14 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     tt_schedule_record L = *rec;
     int changed = 0;
     const int RS = s.r * s.s, CB = (s.c + 31) / 32;
-    const int gap = round_up(std::max(1, std::max(s.pad_w, s.s - 1 - s.pad_w)), 4), wp = s.w + gap;
-    if (wp > 256) return TT_ERR_RESOURCE;
-    const int M = s.k, B = s.n;
-    const long long Nl = (long long)w->P * wp;            // padded-linear output pixels
-    if (Nl > 0x7fffffffLL) return TT_ERR_RESOURCE;
-    const int N = (int)Nl, K = CB * RS * 32;
-    // fixed by the mode: filters on the 128 rows, no split-K, one accumulator; a reduction tile is `tps` taps of one
+    const TapAxis ty = tap_axis(s.r, s.stride_h, s.pad_h, s.h, w->P), tx = tap_axis(s.s, s.stride_w, s.pad_w, s.w, w->Q);
+    const long long image = (long long)ty.pitch * tx.pitch;
+    const int M = s.k;
+    // padded-linear positions up to the last output
+    const long long Nl = (s.n - 1) * image + (long long)(w->P - 1) * tx.pitch + w->Q, Kl = (long long)CB * RS * 32;
+    if (Nl > 0x3fffffffLL || Kl > 0x3fffffffLL) return TT_ERR_RESOURCE;
+    const int N = (int)Nl, K = (int)Kl;
+    // fixed by the mode: filters on the 128 rows, no split-K, one accumulator per tile; a reduction tile is `tps` taps of one
     // 32-channel block (tile_k = 32 * tps, tps a divisor of the tap count, tile_k <= 128)
     int tps = 1;
     for (int d = 1; d <= 4; ++d) if (RS % d == 0 && 32 * d <= rec->tile_k) tps = d;
@@ -118,10 +136,10 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     if (rec->persistent < 0 || rec->persistent > 1 || rec->cta_group < 0 || rec->cta_group > 2 || rec->ctas_per_sm < 0 ||
         rec->ctas_per_sm > 2 || rec->warp_layout != 0 || rec->precision < 0 || rec->precision > 1)
         return TT_ERR_INVALID_SCHEDULE;
-    // both kernel forms walk this reduction order; CTA pairs do not
+    // (one kernel serves both forms: its CTAs always walk; CTA pairs do not exist here)
     const bool persistent = rec->persistent == 1;
-    L.persistent = persistent ? 1 : 0; L.cta_group = 1;
-    if (rec->cta_group == 2) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_FORM; }
+    L.persistent = persistent ? 1 : 0; L.cta_group = 1; L.ctas_per_sm = 1;
+    if (rec->cta_group == 2 || rec->ctas_per_sm == 2) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_FORM; }
     L.precision = 0;                                      // (no error-compensated products for convolutions)
     if (rec->precision != 0) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_FORM; }
     if (rec->tile_m != kHwTileM) changed |= TT_CHG_TILE_M;
@@ -132,99 +150,82 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     if (tn != rec->tile_n) changed |= TT_CHG_TILE_N;
     L.tile_n = tn;
     const int k_tiles = CB * RS / tps;
-    // (the persistent form's filter pipeline runs on across tiles: no point in clamping it to one tile's reduction)
+    // (the walking kernel's filter pipeline runs on across tiles: no point in clamping it to one tile's reduction)
     int st = persistent ? std::min(kMaxStages, rec->stages) : std::min(std::min(kMaxStages, rec->stages), k_tiles);
     if (st != rec->stages) changed |= TT_CHG_STAGES;
     if (strict && (changed & ~TT_CHG_TILE_M)) return TT_ERR_INVALID_SCHEDULE;
-    // shared memory: filter stages | NCHW staging of a block (TMA box [32][in_rows][wp], one buffer) | pixel-major slab
-    // (two buffers of (in_rows * wp + reach) rows of 128 bytes)
-    const int out_rows = std::min(w->P, (tn + wp - 2) / wp + 1);
-    const int in_rows = out_rows - 1 + s.r;
-    if (in_rows > 256) return TT_ERR_RESOURCE;
-    const unsigned a_stage = (unsigned)tps * kHwTileM * 128;
-    const long long s_buf = (((long long)32 * in_rows * wp) * 4 + 127) / 128 * 128;
-    // furthest row a tile's views can touch (all tile_n rows are read, also those of pixels past the image)
-    const long long pm_rows = (long long)((tn + wp - 2) / wp + s.r) * wp + s.s + gap + 8;
-    const long long pm_buf = pm_rows * 128;
-    const int nbuf = (CB > 1 || persistent) ? 2 : 1;
-    long long smem = 0;
-    const long long min_pipe = (long long)kGatherWarps * 32 * 36 * 4;
-    // persistent form: the read-out has its own staging area (the pipeline buffers are busy with the next tile), and
-    // the NCHW staging ring is two boxes deep when that fits
-    const long long epi = persistent ? 4ll * 32 * 36 * 4 : 0;
-    int sd = persistent ? 2 : 1;
-    for (;;) {
-        const long long pipe = persistent ? (long long)st * a_stage : std::max<long long>((long long)st * a_stage, min_pipe);
-        smem = pipe + sd * s_buf + nbuf * pm_buf + epi + 1024;
-        if (smem <= kDynSmemLimit) break;
-        if (sd > 1) { --sd; continue; }
-        if (strict || st <= 1) break;
-        --st; changed |= TT_CHG_STAGES;
-    }
-    L.stages = st;
-    const long long pipe = persistent ? (long long)st * a_stage : std::max<long long>((long long)st * a_stage, min_pipe);
-    const int tiles_m = (M + kHwTileM - 1) / kHwTileM, tiles_n = (N + tn - 1) / tn;
-    const int tmem_cols_t = std::max(32, pow2_ceil(persistent ? 2 * tn : tn));
-    if (persistent) {
-        L.ctas_per_sm = 1;
-        if (rec->ctas_per_sm == 2) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_FORM; }
+    const int tiles_m = (M + kHwTileM - 1) / kHwTileM;
+    // How the record's tiles are laid over the SMs (148; the launch is right on any number).  Where they fill more than half of
+    // them, columns are dealt evenly over the rounds that the record's tile needs: 121 tiles of 224 columns become 141 of 192,
+    // a seventh less time for the one round (conv 3x3 128 -> 128 at 28 x 28, batch 32).  Where they fill less, CTAs share
+    // a tile's channel blocks as a cluster.
+    constexpr int kSms = 148;
+    long long tiles = (long long)tiles_m * ((N + tn - 1) / tn);
+    int split = 1;
+    if (tiles * 2 > kSms) {
+        const long long rounds = (tiles + kSms - 1) / kSms, columns = rounds * kSms / tiles_m;
+        if (columns >= 1) tn = std::min<long long>(tn, round_up64((N + columns - 1) / columns, 16));
     } else {
-        // which build: two CTAs per SM need half the shared memory and half the tensor memory each
-        const bool fits2 = smem <= 112 * 1024 && tmem_cols_t <= 256;
-        const long long ctas = (long long)tiles_m * tiles_n * B;
-        int cps = rec->ctas_per_sm == 0 ? ((ctas > 2 * 148 && fits2) ? 2 : 1) : rec->ctas_per_sm;
-        if (cps == 2 && !fits2) { if (strict) return TT_ERR_INVALID_SCHEDULE; cps = 1; changed |= TT_CHG_FORM; }
-        L.ctas_per_sm = cps;
+        split = (int)std::min<long long>(std::min<long long>(8, CB), kSms / tiles);
     }
+    const int tiles_n = (N + tn - 1) / tn;
+    tiles = (long long)tiles_m * tiles_n;
+    if (tiles > 0x7fffffffLL) return TT_ERR_RESOURCE;
+    // shared memory: filter stages (one tap each: `stages` reduction tiles, at most eight taps) | one or two slabs | staging
+    // blocks of the read-out (twelve warps' where all tiles are resident, a cluster's whole tile, each over the idle pipeline)
+    const int shift_min = ty.lo * tx.pitch + tx.lo, shift_max = std::max(0, ty.hi) * tx.pitch + std::max(0, tx.hi);
+    const int lines = tn + shift_max - std::min(shift_min, 0);
+    const long long slab = (long long)lines * 128;
+    const long long epi = 4ll * kPmEpiBlockBytes;
+    const long long tail = split > 1 ? (long long)((tn + 31) / 32) * 4 * kPmEpiBlockBytes : 12ll * kPmEpiBlockBytes;
+    int taps = std::min(kMaxStages, st * tps), bufs = (CB > 1 || ty.count[0] * tx.count[0] < RS || tiles > kSms) ? 2 : 1;
+    auto total = [&] { return std::max(round_up64(taps * (long long)kPmStageBytes + bufs * slab, 1024) + epi, round_up64(tail, 1024)) + 1024; };
+    while (total() > kDynSmemLimit) {
+        if (taps > 2) --taps;
+        else if (bufs > 1) --bufs;
+        else if (taps > 1) --taps;
+        else break;
+    }
+    // (a stage of the record is tps taps: fewer taps than the record's stages ask for is a shallower pipeline)
+    if ((taps + tps - 1) / tps < std::min(st, (kMaxStages + tps - 1) / tps)) { st = std::max(1, taps / tps); changed |= TT_CHG_STAGES; if (strict) return TT_ERR_RESOURCE; }
+    L.stages = st;
+    const long long smem = total();
+    const int tmem_cols = std::max(32, pow2_ceil(tiles * split > kSms ? tn + round_up(tn, 32) : round_up(tn, 32)));
     I = tt_apply_info{};
     I.legal = L; I.changed = changed;
-    I.grid_x = tiles_m * tiles_n; I.grid_y = 1; I.grid_z = B;
-    const long long units = (long long)tiles_m * tiles_n * B;
-    if (persistent) {
-        if (units > 0x7fffffffLL) return TT_ERR_RESOURCE;
-        I.grid_x = (int)std::min<long long>(units, 148); I.grid_z = 1;      // the launcher clamps to the device's SM count
-    }
-    I.threads = kGemmThreads;
-    I.smem_bytes = (int)std::min<long long>(persistent ? std::max<long long>(smem, 116 * 1024) : smem, 0x7fffffff);
-    I.tmem_cols = tmem_cols_t;
+    I.grid_x = (int)std::min<long long>(tiles, kSms / split); I.grid_y = split; I.grid_z = 1;
+    I.threads = 448;
+    I.smem_bytes = (int)std::min<long long>(std::max<long long>(smem, 116 * 1024), 0x7fffffff);     // one CTA per SM
+    I.tmem_cols = tmem_cols;
     I.workspace_bytes = (int64_t)M * K * 4;              // the re-packed filters
     I.launches = 2;
-    if (smem > kDynSmemLimit || (long long)tiles_m * tiles_n > 0x7fffffffLL || B > 65535) return TT_ERR_RESOURCE;
+    if (smem > kDynSmemLimit) return TT_ERR_RESOURCE;
     plan->swap_ab = false;
-    plan->gm = M; plan->gn = N; plan->gk = K; plan->gbatch = B;
+    plan->gm = M; plan->gn = N; plan->gk = K; plan->gbatch = 1;
     plan->partial_bytes = 0;
-    plan->repack = true; plan->repack_cb = CB;
-    plan->a_tensor = 1; plan->b_tensor = 0;               // A: filters (re-packed), B: the image
-    GemmArgs& g = plan->g;
-    g = GemmArgs{};
-    g.M = M; g.N = N; g.K = K; g.batch = B;
-    g.tile_n = tn; g.tile_k = tk; g.stages = st;
-    g.k_tiles = k_tiles; g.k_tiles_per_split = k_tiles; g.split_k = 1;
-    g.tiles_m = tiles_m; g.tiles_n = tiles_n; g.raster = L.raster;
-    g.atom_k = 32; g.n_atoms = tps; g.row_bytes = 128; g.swz_mask = 7;
-    g.a_stage_bytes = a_stage; g.b_stage_bytes = 0; g.tx_bytes = a_stage;
-    g.tmem_cols = (unsigned)I.tmem_cols; g.n_acc = 1; g.cluster = 0;
-    g.idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(tn >> 3) << 17) | ((unsigned)(kHwTileM >> 4) << 24);
-    g.a_mode = OPM_TMA; g.a_rs = K; g.a_ks = 1; g.a_bs = 0; g.a_tma_batched = 0;
-    g.b_mode = OPM_IM2COL_T; g.b_rs = 0; g.b_ks = 0; g.b_bs = (long long)s.c * s.h * s.w; g.b_tma_batched = 1;
-    g.y_ms = (long long)w->P * w->Q; g.y_ns = 1; g.y_bs = (long long)s.k * w->P * w->Q;
-    g.bias_mode = s.has_bias ? 1 : 0;
-    g.act = s.act;
-    g.C = s.c; g.H = s.h; g.W = s.w; g.R = s.r; g.S = s.s; g.Q = w->Q; g.Pout = w->P;
-    g.sh = 1; g.sw = 1; g.ph = s.pad_h; g.pw = s.pad_w;
-    g.vec_store = (w->Q % 4 == 0 && ((long long)w->P * w->Q) % 4 == 0) ? 1 : 0;   // a lane's four columns: one aligned 16-byte store
-    g.tap_major = 1;
-    g.two_per_sm = L.ctas_per_sm == 2;
-    g.b_rows_cta = tn; g.cta_group = 1;
-    g.persistent = persistent ? 1 : 0; g.total_tiles = (int)units; g.stg_depth = sd;
-    g.epi_off = (unsigned)(pipe + (long long)sd * s_buf + (long long)nbuf * pm_buf);
-    g.slab_tma = 1; g.slab_tiles = RS / tps; g.slab_nbuf = 1; g.pm_nbuf = nbuf;
-    g.slab_off = (unsigned)pipe; g.slab_buf_bytes = (unsigned)s_buf;
-    g.slab_wp = wp; g.slab_gap = gap; g.slab_chpitch = in_rows * wp; g.slab_in_rows = in_rows; g.slab_rstep = 1;
-    g.slab_box_ch = std::min(32, s.c);                   // (fewer than 32 channels: the rest of the staging buffer stays zero)
-    g.slab_box_bytes = (unsigned)((long long)g.slab_box_ch * in_rows * wp * 4);
-    g.slab_vec16 = 1;
-    g.pm_off = (unsigned)(pipe + (long long)sd * s_buf); g.pm_buf_bytes = (unsigned)pm_buf;
+    plan->repack = true;
+    plan->a_tensor = 1; plan->b_tensor = 0;
+    plan->g = GemmArgs{};
+    GemmArgs& g = plan->g;                               // what the filters' tensor map is made from
+    g.M = M; g.N = N; g.K = K; g.batch = 1; g.atom_k = 32; g.a_mode = OPM_TMA; g.b_mode = -1; g.a_rs = K; g.a_ks = 1;
+    ConvPmArgs& c = plan->pm;
+    c = ConvPmArgs{};
+    c.M = M; c.C = s.c; c.H = s.h; c.W = s.w; c.R = s.r; c.S = s.s; c.P = w->P; c.Q = w->Q; c.images = s.n;
+    c.sh = s.stride_h; c.sw = s.stride_w; c.act = s.act;
+    c.blocks = CB;
+    c.wp = tx.pitch; c.image_pitch = (int)image;
+    c.magic_wp = magic_of(c.wp); c.magic_image = magic_of(c.image_pitch);
+    c.shift_min = std::min(shift_min, 0); c.slab_lines = lines;
+    for (int a = 0; a < s.stride_h; ++a) for (int b = 0; b < s.stride_w; ++b)
+        if (ty.count[a] > 0 && tx.count[b] > 0)
+            c.planes[c.n_planes++] = ConvPlane{(signed char)a, (signed char)b, (signed char)ty.shift[a], (signed char)tx.shift[b],
+                                               (unsigned char)ty.count[a], (unsigned char)tx.count[b], (unsigned char)ty.first[a], (unsigned char)tx.first[b]};
+    c.tile_n = tn; c.tiles_m = tiles_m; c.tiles_n = tiles_n; c.total_tiles = (int)tiles; c.raster = L.raster; c.split = split;
+    c.stages = taps; c.slab_bufs = bufs;
+    c.slab_off = (unsigned)(taps * kPmStageBytes); c.slab_bytes = (unsigned)slab;
+    c.epi_off = (unsigned)round_up64(taps * (long long)kPmStageBytes + bufs * slab, 1024);
+    c.idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(tn >> 3) << 17) | ((unsigned)(kHwTileM >> 4) << 24);
+    c.tmem_cols = (unsigned)tmem_cols;
     return TT_OK;
 }
 

@@ -21,8 +21,6 @@ enum OperandMode : int {
     OPM_GATHER_ROWS = 1,  // strided view, lanes walk rows (row stride 1): 16-byte swizzled stores
     OPM_GATHER_K = 2,     // strided view, lanes walk k (k stride 1): 4-byte swizzled stores
     OPM_IM2COL = 3,       // rows are output pixels, k = (c, r, s): expanded from a slab of NCHW input rows
-    OPM_IM2COL_T = 4,     // rows are padded-linear output pixels, k = (32-channel block, tap, channel): every tap's tile
-                          // is a shifted view of a pixel-major slab in shared memory (nothing is staged per tile)
     OPM_TMA_MN = 5        // the row index is the contiguous one in memory: [tile_k][32 rows] boxes by TMA, multiplied as
                           // they lie (an MN-major tile)
 };
@@ -67,9 +65,6 @@ struct GemmArgs {
     int slab_tma;                               // 1: chunks arrive by TMA; 0: by cp.async from the gather warps
     int slab_box_ch;                            // channels per box
     unsigned slab_box_bytes;
-    unsigned pm_off, pm_buf_bytes; int pm_nbuf; // tap-major convolutions: the pixel-major slab buffers (one or two)
-    int tap_major;                              // 1: OPM_IM2COL_T on operand B
-    int Pout;                                   // output rows (padded-linear pixel -> (p, q'))
     const int* ktab_dev;                        // per reduction index: byte offset of (c, r, s) inside the slab (absolute channel)
     unsigned long long wait_ns;                 // limit of every bounded wait inside the kernel
     unsigned extra_tx;                          // test facility: bytes added to what the first stage's barrier expects
@@ -82,7 +77,6 @@ struct GemmArgs {
     int total_tiles;                            // tiles_m * tiles_n * batch; tiles_m counts 128 * cta_group rows
     int a_mn, b_mn;                             // the operand's tiles are MN-major
     int b_rows_cta;                             // rows of operand B one CTA loads: tile_n / cta_group
-    int stg_depth;                              // tap-major: boxes per staging ring
     unsigned epi_off;                           // read-out staging area: byte offset from the aligned tile base
     int epi_warps;                              // read-out warps: 4 or 8
     int epi_bufs;                               // 32 x 32 blocks in each read-out warp's ring
@@ -90,6 +84,28 @@ struct GemmArgs {
     int epi_tma;                                // outputs leave by TMA stores (contiguous along the tile's columns)
     int res_tma;                                // the residual comes in by TMA, one block ahead
     int y_tma_batched;                          // the output's tensor map has the batch as its third dimension
+};
+
+// conv2d by channel blocks and taps over a pixel-major slab (tt_conv_pm_kernel).
+constexpr int kPmMaxPlanes = 16;
+constexpr unsigned kPmStageBytes = kHwTileM * 32 * 4;       // one tap's filters: 128 x 32 channels
+constexpr unsigned kPmEpiBlockBytes = 32 * 36 * 4;          // a staged 32 x 32 block of the read-out
+// The taps of one parity class of (row, column) and the sub-image they read: padded input coordinates stride * i + a,
+// stride * j + b.  Its first tap is (r0, s0) and reads position (row + f0, column + e0) of the sub-image; the next ones of
+// the class follow at (+1, +1).
+struct ConvPlane { signed char a, b, f0, e0; unsigned char nr, ns, r0, s0; };
+struct ConvPmArgs {
+    const float* x; float* y; const float* bias; const float* residual;
+    unsigned* status; unsigned long long wait_ns;
+    unsigned extra_tx; int early_filters;
+    int M, C, H, W, R, S, P, Q, images, sh, sw, act;
+    int blocks;                                 // channel blocks of 32
+    int wp, image_pitch;                        // positions per row and per image of the padded-linear numbering
+    unsigned magic_wp, magic_image;             // floor(2^32 / divisor)
+    int shift_min, slab_lines;                  // the slab of a tile: positions n0 + shift_min .. + slab_lines - 1
+    int n_planes; ConvPlane planes[kPmMaxPlanes];
+    int tile_n, tiles_m, tiles_n, total_tiles, raster, split, stages, slab_bufs;
+    unsigned slab_off, slab_bytes, epi_off, idesc, tmem_cols;
 };
 
 struct DwArgs {
@@ -125,8 +141,8 @@ struct Plan {
     int a_tensor = 0, b_tensor = 1;   // which caller tensor feeds operand A / B: 0 = x, 1 = w
     GemmArgs g{};
     long long partial_bytes = 0;      // counters start here inside the workspace
-    bool repack = false;              // tap-major convolution: filters are re-packed into the workspace before each run
-    int repack_cb = 0;                // 32-channel blocks
+    bool repack = false;              // tap-major convolution: pm applies, filters are re-packed into the workspace
+    ConvPmArgs pm{};
     DwArgs dw{};
     RowArgs row{};
 };

@@ -23,249 +23,9 @@
 #include <algorithm>
 #include <atomic>
 #include <utility>
-#include "tt_internal.h"
+#include "tt_ptx.cuh"
 
 namespace tt {
-
-// ------------------------------------------------------------------------------------------------------------
-// PTX wrappers
-// ------------------------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// Raise the byte count the barrier's current phase expects, without arriving on it.
-__device__ __forceinline__ void mbar_expect_tx_only(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok;
-}
-// Non-blocking test of a barrier phase.
-__device__ __forceinline__ uint32_t mbar_test_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok;
-}
-__device__ __forceinline__ unsigned long long global_timer_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
-
-
-
-// Bounded wait.  Returns false when the CTA is aborting (this wait or another one expired).
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned* status,
-                                            unsigned where, unsigned long long limit_ns) {
-    const unsigned long long t0 = global_timer_ns();
-    unsigned spins = 0;
-    for (;;) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((++spins & 31u) == 0u) {
-            if (*abort_flag) return false;
-            if (global_timer_ns() - t0 > limit_ns) {
-                *abort_flag = 1;
-                atomicCAS(status, 0u, (unsigned)TT_ERR_TIMEOUT | (where << 8));
-                return false;
-            }
-        }
-    }
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned* status,
-                                          unsigned where, unsigned long long limit_ns) {
-    if (mbar_try_wait(bar, parity)) return true;         // the common case costs one instruction
-    return mbar_wait_slow(bar, parity, abort_flag, status, where, limit_ns);
-}
-
-// Programmatic dependent launch.  A kernel launched with programmatic stream serialization may become resident while
-// its predecessor in the stream is still running; it must wait here before its first access to global memory.  The
-// kernel after it is allowed to do the same from this kernel's entry on.  (Without the launch attribute both
-// instructions do nothing.)
-__device__ __forceinline__ void pdl_allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// One lane of a converged warp (the same lane every time): it issues the warp's asynchronous instructions.
-__device__ __forceinline__ bool elect_one() {
-    uint32_t pred;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "elect.sync _|p, 0xffffffff;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(pred));
-    return pred != 0u;
-}
-
-__device__ __forceinline__ void fence_proxy_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(tmap), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
-}
-
-// An MN-major operand tile: one box [tile_k][32 rows] after the other.
-__device__ __forceinline__ void load_mn_boxes(uint32_t dst, const void* tmap, uint32_t bar, int row0, int rows, int k0, int tile_k, int bz) {
-#pragma unroll 1
-    for (int r = 0; r < rows; r += 32, dst += (uint32_t)tile_k * 128u) tma_load_3d(dst, tmap, bar, row0 + r, k0, bz);
-}
-
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2, int c3) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-        ::"r"(dst), "l"(tmap), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
-}
-
-__device__ __forceinline__ void tmem_alloc(uint32_t slot_smem, uint32_t cols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_smem), "r"(cols) : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() {
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-}
-// D[tmem] (+)= A[smem] * B[smem]^T, one 128 x N x 8 TF32 step.
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// All 8-wide reduction steps of one pipeline stage into one accumulator: ATOMS swizzle atoms of K8 steps each.
-// Inside an atom a step advances both descriptors by 2 (32 bytes); the next atom starts a_atom / b_atom later.
-template <int ATOMS, int K8>
-__device__ __forceinline__ void issue_steps(uint32_t d_tmem, uint32_t d_hi, uint32_t a_lo, uint32_t b_lo, uint32_t a_atom,
-                                            uint32_t b_atom, uint32_t idesc, uint32_t accumulate) {
-#pragma unroll
-    for (int at = 0; at < ATOMS; ++at) {
-#pragma unroll
-        for (int k8 = 0; k8 < K8; ++k8) {
-            mma_tf32(d_tmem, ((uint64_t)d_hi << 32) | (uint64_t)(a_lo + (uint32_t)at * a_atom + 2u * (uint32_t)k8),
-                     ((uint64_t)d_hi << 32) | (uint64_t)(b_lo + (uint32_t)at * b_atom + 2u * (uint32_t)k8), idesc,
-                     (at == 0 && k8 == 0) ? accumulate : 1u);
-        }
-    }
-}
-// The same when an operand is MN-major: any number of steps, each operand with its own stride (k8_a, k8_b) per step inside
-// an atom of k8_n steps.
-__device__ __forceinline__ void issue_steps_any(uint32_t d_tmem, uint32_t a_hi, uint32_t b_hi, uint32_t a_lo, uint32_t b_lo, uint32_t k8_a,
-                                                uint32_t k8_b, uint32_t a_atom, uint32_t b_atom, int atoms, int k8_n, uint32_t idesc,
-                                                uint32_t accumulate) {
-#pragma unroll 1
-    for (int at = 0; at < atoms; ++at, a_lo += a_atom, b_lo += b_atom) {
-        uint32_t a = a_lo, b = b_lo;
-#pragma unroll 4
-        for (int k8 = 0; k8 < k8_n; ++k8, a += k8_a, b += k8_b) {
-            mma_tf32(d_tmem, ((uint64_t)a_hi << 32) | (uint64_t)a, ((uint64_t)b_hi << 32) | (uint64_t)b, idesc, accumulate);
-            accumulate = 1u;
-        }
-    }
-}
-
-// Arrive on an mbarrier once every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// 32 lanes x 16 consecutive 32-bit columns: thread i of the warp receives lane (base + i).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// Shared-memory matrix descriptor of a K-major tile whose rows are `row_bytes` long and hardware-swizzled with
-// the span of one row: start address >> 4 in bits 0-13, leading byte offset >> 4 in bits 16-29 (not used by
-// swizzled K-major tiles; set to 1), stride byte offset (distance between 8-row groups) >> 4 in bits 32-45,
-// constant 0b001 in bits 46-48, swizzle mode in bits 61-63 (2 = 128 B, 4 = 64 B, 6 = 32 B).
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, int row_bytes) {
-    const uint64_t swz = row_bytes == 128 ? 2ull : (row_bytes == 64 ? 4ull : 6ull);
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= 1ull << 16;
-    d |= (uint64_t)((8u * (uint32_t)row_bytes) >> 4) << 32;
-    d |= 1ull << 46;
-    d |= swz << 61;
-    return d;
-}
-
-// The same for an MN-major tile: the row index of the operand is the contiguous one in memory (the pixels of a 1x1
-// convolution, the columns of an NN batch_matmul's second operand), so a TMA box of 32 rows x tile_k is [k][32 rows] lines of
-// 128 bytes.  kind::tf32 reads that form with the 128-byte swizzle of 32-byte atoms (mode 1: the 32-byte chunk index is XORed
-// with the line index modulo 4; read out of the tensor core with an indexed tile): four lines make an atom of 512 bytes
-// (stride byte offset), and the next 32 rows begin a box further on (leading byte offset).
-__device__ __forceinline__ uint64_t make_desc_mn(uint32_t saddr, uint32_t box_bytes) {
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(box_bytes >> 4) << 16;
-    d |= (uint64_t)(512u >> 4) << 32;
-    d |= 1ull << 46;
-    d |= 1ull << 61;
-    return d;
-}
-// How far a descriptor's start address (in 16-byte units) moves per 8-wide reduction step and per swizzle atom of K.
-struct DescSteps { uint32_t lo, hi, k8, atom; };
-__device__ __forceinline__ DescSteps desc_steps(bool mn, int row_bytes, int rows, int tile_k, int atom_k) {
-    DescSteps s;
-    const uint64_t d = mn ? make_desc_mn(0u, (uint32_t)tile_k * 128u) : make_desc(0u, row_bytes);
-    s.lo = (uint32_t)d; s.hi = (uint32_t)(d >> 32);
-    s.k8 = mn ? 64u : 2u;                                // eight lines of 128 bytes; 32 bytes along a line
-    s.atom = mn ? 64u * (uint32_t)(atom_k >> 3) : (uint32_t)(rows * row_bytes) >> 4;
-    return s;
-}
-
-// GELU in its erf form, 0.5 x (1 + erf(x / sqrt 2)).  erf through the rational approximation 7.1.26 of Abramowitz and
-// Stegun (absolute error below 1.5e-7, far inside what a TF32 product carries): a dozen instructions instead of
-// the library routine's, which matters in a read-out that is a long serial instruction stream per thread.
-__device__ __forceinline__ float gelu_erf(float x) {
-    const float z = fabsf(x) * 0.70710678118654752440f;
-    const float t = __fdividef(1.f, fmaf(0.3275911f, z, 1.f));
-    float poly = fmaf(1.061405429f, t, -1.453152027f);
-    poly = fmaf(poly, t, 1.421413741f);
-    poly = fmaf(poly, t, -0.284496736f);
-    poly = fmaf(poly, t, 0.254829592f);
-    const float erf_abs = 1.f - poly * t * __expf(-z * z);
-    return 0.5f * x * (1.f + copysignf(erf_abs, x));
-}
-
-__device__ __forceinline__ float apply_act(float v, int act) {
-    switch (act) {
-        case TT_ACT_RELU: return fmaxf(v, 0.f);
-        case TT_ACT_RELU6: return fminf(fmaxf(v, 0.f), 6.f);
-        case TT_ACT_GELU_ERF: return gelu_erf(v);
-        default: return v;
-    }
-}
-
-// Byte offset of element (row, kk) inside one swizzle atom block of a K-major tile: rows are row_bytes apart
-// and the 16-byte chunk index is XORed with bits 7.. of the linear offset (the TMA swizzle patterns).
-__device__ __forceinline__ uint32_t swz_off(uint32_t row, uint32_t kbyte, uint32_t row_bytes, uint32_t mask) {
-    const uint32_t off = row * row_bytes + kbyte;
-    return off ^ (((off >> 7) & mask) << 4);
-}
 
 // ------------------------------------------------------------------------------------------------------------
 // Operand producers that do not go through TMA.
@@ -281,68 +41,6 @@ __device__ __forceinline__ uint32_t swz_off(uint32_t row, uint32_t kbyte, uint32
 // Strided views (the NN operand of batch_matmul) and K-contiguous operands with K % 4 != 0 are gathered from
 // global memory directly: the 8 gather warps form 1, 2 or 4 groups, group g fills stages g, g + groups, ...
 // ------------------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, float a, float b, float c, float d) {
-    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
-}
-__device__ __forceinline__ void st_shared_f32(uint32_t addr, float a) {
-    asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(a) : "memory");
-}
-__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t a) {
-    asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(a) : "memory");
-}
-__device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ uint32_t ld_shared_u32(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ uint4 ld_shared_v4u(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_4(uint32_t dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// Thread-block cluster primitives (split-K over a cluster: the splits of one output tile are the CTAs of a cluster
-// and exchange their partial tiles through distributed shared memory).
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t map_to_peer(uint32_t saddr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ float ld_peer_f32(uint32_t caddr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(caddr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_peer_v4(uint32_t caddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(caddr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ void st_peer_u32(uint32_t caddr, uint32_t a) {
-    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(caddr), "r"(a) : "memory");
-}
-__device__ __forceinline__ float4 ld_shared_v4f(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
 // Split-K over a cluster.  The output tile is cut into one band per CTA, along the direction in which the output is
 // NOT contiguous (bands of rows when outputs are contiguous along columns, bands of columns otherwise).  Every CTA
 // first writes its partial tile into its own shared memory (the pipeline buffers, idle by then) in the layout of the
@@ -354,28 +52,6 @@ __device__ __forceinline__ float4 ld_shared_v4f(uint32_t addr) {
 // CTA's own split has no slot):
 //   bands of rows:    [row in band][col], pitch tile_n + 4 floats;   bands of columns: [col in band][row], pitch 128.
 constexpr int kRedColPitch = kHwTileM;
-// One band of this CTA's staged partial tile -> the same band's slot in a peer's reduction area; the bytes are counted
-// on the peer's barrier (both destination addresses are shared::cluster addresses of the same peer).
-__device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_caddr, uint32_t src_saddr, uint32_t bytes, uint32_t bar_caddr) {
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst_caddr), "r"(src_saddr), "r"(bytes), "r"(bar_caddr) : "memory");
-}
-// Wait until every bulk copy this thread issued has been written at its destination.
-__device__ __forceinline__ void bulk_copies_done() {
-    asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group 0;" ::: "memory");
-}
-
-// Untiled copies between global and shared memory (16-byte aligned, whole multiples of 16 bytes).
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t bytes) {
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\tcp.async.bulk.commit_group;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
-}
-// Wait until the stores this thread issued have read their shared memory.
-__device__ __forceinline__ void bulk_stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-
 // All gather threads meet and learn whether every one of them is still healthy (named barrier 1).
 __device__ __forceinline__ bool gather_vote(bool ok) {
     uint32_t all;
@@ -644,24 +320,12 @@ __device__ __forceinline__ void gather_stage(int mode, uint32_t tile_smem, int r
 // ------------------------------------------------------------------------------------------------------------
 // Epilogue helpers
 // ------------------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(taddr) : "memory");
-}
-
 constexpr int kStagePitch = 36;                          // floats per staged row: 16-byte accesses stay conflict-free
 constexpr int kStageBytesPerWarp = 32 * kStagePitch * 4;
 
 // ReLU, ReLU6 and "none" are one clamp with per-kernel bounds (no branch per element); GELU is a separate path.
 struct EpiArgs {
     float* ybase; const float* rbase; long long y_ms, y_ns; int M; float lo, hi; bool gelu, vec;
-    int lin_wp, lin_q, lin_p;   // lin_wp > 0: column n is the padded-linear pixel p * lin_wp + q', stored at p * lin_q + q' if q' < lin_q
 };
 
 __device__ __forceinline__ float finish_one(float v, const EpiArgs& e) {
@@ -682,41 +346,6 @@ __device__ __forceinline__ void epilogue_block(float (&v)[32], const EpiArgs& e,
         for (int j = 0; j < 32; j += 4) st_shared_v4(stg + (uint32_t)(lane * kStagePitch + j) * 4u, v[j], v[j + 1], v[j + 2], v[j + 3]);
         __syncwarp();
         const int cc = (lane & 7) * 4;
-        if (e.lin_wp > 0) {
-            // tap-major convolution: column n is the padded-linear pixel p * wp + q'.  A lane's four columns lie in one
-            // padded row (wp is a multiple of 4); when Q is one too, all four are outputs or all four fall into the gap.
-            const int n = nb + cc;
-            const int p = n / e.lin_wp, q = n - p * e.lin_wp;
-            const bool col_ok = cc < cnt && q < e.lin_q && p < e.lin_p;
-            const int nq = min(4, e.lin_q - q);          // outputs among the four (4 whenever Q is a multiple of 4)
-            const long long coff = (long long)p * e.lin_q + q;
-#pragma unroll
-            for (int itr = 0; itr < 8; ++itr) {
-                const int rr = itr * 4 + (lane >> 3);
-                const int m = m_first + rr;
-                float4 t;
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w)
-                             : "r"(stg + (uint32_t)(rr * kStagePitch + cc) * 4u));
-                if (col_ok && m < e.M) {
-                    const long long o = (long long)m * e.y_ms + coff;
-                    if (POST) {
-                        t.x = finish_one(t.x + __ldg(e.rbase + o), e);
-                        if (nq > 1) t.y = finish_one(t.y + __ldg(e.rbase + o + 1), e);
-                        if (nq > 2) t.z = finish_one(t.z + __ldg(e.rbase + o + 2), e);
-                        if (nq > 3) t.w = finish_one(t.w + __ldg(e.rbase + o + 3), e);
-                    }
-                    if (e.vec) *reinterpret_cast<float4*>(e.ybase + o) = t;      // (vec implies Q % 4 == 0)
-                    else {
-                        e.ybase[o] = t.x;
-                        if (nq > 1) e.ybase[o + 1] = t.y;
-                        if (nq > 2) e.ybase[o + 2] = t.z;
-                        if (nq > 3) e.ybase[o + 3] = t.w;
-                    }
-                }
-            }
-            __syncwarp();
-            return;
-        }
 #pragma unroll
         for (int itr = 0; itr < 8; ++itr) {
             const int rr = itr * 4 + (lane >> 3);
@@ -767,34 +396,6 @@ __device__ __forceinline__ void epilogue_block(float (&v)[32], const EpiArgs& e,
 // Two builds of each: MIN_CTAS = 1 (all registers), and MIN_CTAS = 2 (registers capped so that two CTAs share an SM when a
 // record's shared memory and tensor memory allow it: one CTA's set-up and read-out then overlap the other's main loop).
 // ------------------------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok;
-}
-// Bounded wait on a barrier that CTAs of the cluster arrive on (acquire at cluster scope).
-__device__ __noinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned* status,
-                                               unsigned where, unsigned long long limit_ns) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    const unsigned long long t0 = global_timer_ns();
-    unsigned spins = 0;
-    for (;;) {
-        if (mbar_try_wait_cluster(bar, parity)) return true;
-        if ((++spins & 31u) == 0u) {
-            if (*abort_flag) return false;
-            if (global_timer_ns() - t0 > limit_ns) {
-                *abort_flag = 1;
-                atomicCAS(status, 0u, (unsigned)TT_ERR_TIMEOUT | (where << 8));
-                return false;
-            }
-        }
-    }
-}
-
 // Split-K over a cluster: extent (rows or columns) and bytes of the band of the output tile that split `owner` finishes.
 __device__ __forceinline__ int red_band_extent(const GemmArgs& g, int owner) {
     const int whole = g.y_ns == 1 ? kHwTileM : g.tile_n;
@@ -809,8 +410,7 @@ enum GemmForm {
     kFormTma = 0,       // both operands K-major by TMA
     kFormMn = 1,        // both by TMA, one of them (or both) MN-major
     kFormIm2col = 2,    // one operand expanded from a slab of input rows, the other by TMA or gathered
-    kFormTap = 3,       // tap-major convolution
-    kFormGather = 4     // an operand gathered from global memory (the other one any way but by expansion)
+    kFormGather = 3     // an operand gathered from global memory (the other one any way but by expansion)
 };
 
 template <int MIN_CTAS, int FORM>
@@ -823,8 +423,6 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     __shared__ uint64_t accum_bar;
     __shared__ uint64_t slab_full[2];     // a slab chunk has landed (TMA)
     __shared__ uint64_t slab_empty[2];    // all gather warps are done with a slab buffer
-    __shared__ uint64_t pm_full[2];       // tap-major convolution: a pixel-major slab buffer has been written
-    __shared__ uint64_t pm_empty[2];      // ... and every multiply-accumulate that reads it has completed
     __shared__ uint64_t red_bar;          // split-K over a cluster: the other splits' bands of this CTA's output have landed
     __shared__ uint64_t lo_bar[kMaxStages];   // error-compensated products: the remainders of a stage's operand tiles are written
     __shared__ uint32_t tmem_slot;
@@ -854,13 +452,13 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     const uint32_t lo_off = g.a_stage_bytes + g.b_stage_bytes;
     const uint32_t stage_bytes = FORM == kFormTma && g.x3 ? 2u * lo_off : lo_off;
     // what the instantiation is made for (GemmForm); within it only the modes that its form leaves open are looked at
-    constexpr bool im2col = FORM == kFormIm2col, tapm = FORM == kFormTap;     // tapm: reduction walked by channel block and tap
+    constexpr bool im2col = FORM == kFormIm2col;
     constexpr bool may_mn = FORM == kFormMn || FORM == kFormGather;
     const bool a_mn = may_mn && g.a_mode == OPM_TMA_MN, b_mn = may_mn && g.b_mode == OPM_TMA_MN;
-    const bool a_tma = FORM == kFormTma || FORM == kFormMn || FORM == kFormTap || g.a_mode == OPM_TMA || a_mn;
-    const bool b_tma = FORM == kFormTma || FORM == kFormMn || (FORM != kFormTap && (g.b_mode == OPM_TMA || b_mn));
+    const bool a_tma = FORM == kFormTma || FORM == kFormMn || g.a_mode == OPM_TMA || a_mn;
+    const bool b_tma = FORM == kFormTma || FORM == kFormMn || g.b_mode == OPM_TMA || b_mn;
     const bool any_tma = a_tma || b_tma, any_gather = !a_tma || !b_tma;
-    const bool slab_tma = (im2col || tapm) && g.slab_tma != 0;
+    const bool slab_tma = im2col && g.slab_tma != 0;
     const bool x3 = FORM == kFormTma && g.x3 != 0;       // error-compensated products
     // im2col geometry of this CTA: first output row of its pixels, the image row its slab starts at, slab chunks
     int ic_p_first = 0, ic_ih_lo = 0, ic_chunks = 0;
@@ -868,12 +466,6 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         const int row0 = g.a_mode == OPM_IM2COL ? m0 : n0;
         ic_p_first = row0 / g.Q;
         ic_ih_lo = ic_p_first * g.sh - g.ph;
-        ic_chunks = (iters + g.slab_tiles - 1) / g.slab_tiles;
-    }
-    if (tapm) {
-        // the tile's columns are padded-linear pixels n = p * wp + q'
-        ic_p_first = n0 / g.slab_wp;
-        ic_ih_lo = ic_p_first - g.ph;
         ic_chunks = (iters + g.slab_tiles - 1) / g.slab_tiles;
     }
     // gather groups (global gathers only): 4 groups of 2 warps from 4 stages up, 2 groups of 4 warps for 2-3 stages,
@@ -889,7 +481,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         if (slab_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
     }
     if (threadIdx.x == 0) {
-        const uint32_t full_count = tapm ? 1u : (any_tma ? 1u : 0u) + (any_gather ? (uint32_t)wpg : 0u);
+        const uint32_t full_count = (any_tma ? 1u : 0u) + (any_gather ? (uint32_t)wpg : 0u);
         for (int s = 0; s < g.stages; ++s) {
             mbar_init(smem_u32(&full_bar[s]), full_count);
             mbar_init(smem_u32(&empty_bar[s]), 1u);
@@ -899,8 +491,6 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&slab_full[b]), 1u);
             mbar_init(smem_u32(&slab_empty[b]), (uint32_t)kGatherWarps);
-            mbar_init(smem_u32(&pm_full[b]), (uint32_t)kGatherWarps);
-            mbar_init(smem_u32(&pm_empty[b]), 1u);
         }
         if (g.cluster) {
             // the bands this CTA finishes arrive from the other splits: rows x (tile_n + 4) or columns x 128 floats each
@@ -972,18 +562,16 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             const int RS = g.R * g.S, T = g.slab_tiles;
             const uint32_t slab0 = tiles_base + g.slab_off;
             int slab_issued = 0;
-            // (the tap-major path has one staging buffer -- it is transposed away at once --, the other two)
-            const int sbufs = tapm ? 1 : 2;
             auto issue_chunk = [&](int j) {
-                const int b = tapm ? 0 : (j & 1);
+                const int b = j & 1;
                 const uint32_t bar = smem_u32(&slab_full[b]);
                 mbar_expect_tx(bar, g.slab_box_bytes);
                 tma_load_4d(slab0 + (uint32_t)b * g.slab_buf_bytes, &tmap_x, bar, -g.slab_gap, ic_ih_lo,
                             (kt_begin * g.tile_k + j * T * g.tile_k) / RS, bz);
             };
             if (slab_tma) {
-                if (leader) { issue_chunk(0); if (sbufs > 1 && ic_chunks > 1) issue_chunk(1); }
-                slab_issued = min(ic_chunks, sbufs);
+                if (leader) { issue_chunk(0); if (ic_chunks > 1) issue_chunk(1); }
+                slab_issued = min(ic_chunks, 2);
             }
             int next_slab_it = slab_tma ? (slab_issued - 1) * T : 0x7fffffff;   // chunk `slab_issued` is requested when chunk slab_issued-1 starts
             bool ok = true;
@@ -993,8 +581,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                     if (slab_issued < ic_chunks) {
                         // its buffer is free once the gather warps have left chunk slab_issued - 2
                         const int j = slab_issued;
-                        const bool freed = tapm ? mbar_wait(smem_u32(&slab_empty[0]), (uint32_t)(j - 1) & 1u, abortp, g.status, 5u, g.wait_ns)
-                                                : mbar_wait(smem_u32(&slab_empty[j & 1]), (uint32_t)((j - 2) >> 1) & 1u, abortp, g.status, 5u, g.wait_ns);
+                        const bool freed = mbar_wait(smem_u32(&slab_empty[j & 1]), (uint32_t)((j - 2) >> 1) & 1u, abortp, g.status, 5u, g.wait_ns);
                         if (!__all_sync(0xffffffffu, freed)) { ok = false; break; }
                         if (leader) issue_chunk(j);
                         ++slab_issued;
@@ -1039,9 +626,9 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                         if (global_timer_ns() - t0 > 2000000ull) break;
                     }
                 }
-                for (int j = max(0, slab_issued - sbufs); j < slab_issued; ++j) {
+                for (int j = max(0, slab_issued - 2); j < slab_issued; ++j) {
                     const unsigned long long t0 = global_timer_ns();
-                    while (!mbar_try_wait(smem_u32(&slab_full[tapm ? 0 : (j & 1)]), (uint32_t)(tapm ? j : (j >> 1)) & 1u)) {
+                    while (!mbar_try_wait(smem_u32(&slab_full[j & 1]), (uint32_t)(j >> 1) & 1u)) {
                         if (global_timer_ns() - t0 > 2000000ull) break;
                     }
                 }
@@ -1073,41 +660,6 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             const uint32_t d_end = tmem_base + (uint32_t)(g.n_acc * g.tile_n);
             int fresh = g.n_acc;                         // accumulators not written yet
             uint32_t a_stage = a_lo0, b_stage = b_lo0, full_addr = full0, empty_addr = empty0;
-            if (tapm) {
-                // Tap-major convolution: the B tile of reduction tile `it` = (channel block, tap (r, s)) is the
-                // pixel-major slab of that block read from row lin0 + r * wp + s on (128-byte rows, one per
-                // padded-linear pixel; the hardware swizzles on absolute addresses, so any start row works).
-                const uint32_t pm0 = tiles_base + g.pm_off;
-                const int RS = g.R * g.S;
-                const int lin0 = (n0 - ic_p_first * g.slab_wp) + g.slab_gap - g.pw;
-                int chunk = 0, tap = 0, fr = 0, fs = 0;
-                for (int it = 0; it < iters; ++it) {
-                    bool got = mbar_wait(full_addr, ph, abortp, g.status, 2u, g.wait_ns);                       // the filter tile
-                    if (tap == 0) got = mbar_wait(smem_u32(&pm_full[chunk & 1]), (uint32_t)(chunk >> 1) & 1u, abortp, g.status, 7u, g.wait_ns) && got;
-                    if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-                    tc_fence_after();
-                    if (leader) {
-                        // the stage holds n_atoms taps of this channel block, one 128 x 32 filter atom each
-                        uint32_t a_lo = a_stage;
-                        int r2 = fr, s2 = fs;
-#pragma unroll 1
-                        for (int t = 0; t < g.n_atoms; ++t, a_lo += a_atom) {
-                            const uint32_t row = (uint32_t)(lin0 + r2 * g.slab_wp + s2);
-                            const uint32_t b_lo = d_lo + (((pm0 + (uint32_t)(chunk & 1) * g.pm_buf_bytes + row * 128u) & 0x3FFFFu) >> 4);
-                            issue_steps<1, 4>(tmem_base, d_hi, a_lo, b_lo, a_atom, b_atom, g.idesc, (it > 0 || t > 0) ? 1u : 0u);
-                            if (++s2 == g.S) { s2 = 0; ++r2; }
-                        }
-                        mma_commit(empty_addr);                                                  // filter stage reusable
-                        if (tap + g.n_atoms == RS) mma_commit(smem_u32(&pm_empty[chunk & 1]));      // slab buffer reusable
-                    }
-                    __syncwarp();
-                    for (int t = 0; t < g.n_atoms; ++t) if (++fs == g.S) { fs = 0; ++fr; }
-                    tap += g.n_atoms;
-                    if (tap == RS) { tap = 0; fr = 0; fs = 0; ++chunk; }
-                    a_stage += stage_step; full_addr += 8u; empty_addr += 8u;
-                    if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; a_stage = a_lo0; full_addr = full0; empty_addr = empty0; }
-                }
-            } else
             for (int it = 0; it < iters; ++it) {
                 bool got = mbar_wait(full_addr, ph, abortp, g.status, 2u, g.wait_ns);
                 if (x3) got = mbar_wait(smem_u32(&lo_bar[st]), ph, abortp, g.status, 16u, g.wait_ns) && got;   // the remainders too
@@ -1278,56 +830,6 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 }
             }
             cp_async_wait<0>();
-        } else if (tapm) {
-            // ---- conv2d, tap-major: transpose every 32-channel block of input rows, once, into a pixel-major slab ----
-            // staging buffer (TMA): [32 channels][in_rows][wp] floats; pixel-major slab: one 128-byte row per staged
-            // position (32 channels), 16-byte chunks swizzled by the row's absolute address like a TMA 128-byte tile.
-            const uint32_t st0 = tiles_base + g.slab_off, pm0 = tiles_base + g.pm_off;
-            const int npix = g.slab_in_rows * g.slab_wp;
-            // rows a view can touch beyond the transposed range must hold finite numbers: clear both buffers once
-            for (uint32_t o = (uint32_t)gt * 16u; o < (uint32_t)g.pm_nbuf * g.pm_buf_bytes; o += (uint32_t)kGatherThreads * 16u)
-                st_shared_v4(pm0 + o, 0.f, 0.f, 0.f, 0.f);
-            if (g.slab_box_ch < 32)                      // channels beyond the TMA box (which may already be landing) read as zero
-                for (uint32_t o = g.slab_box_bytes + (uint32_t)gt * 16u; o < g.slab_buf_bytes; o += (uint32_t)kGatherThreads * 16u)
-                    st_shared_v4(st0 + o, 0.f, 0.f, 0.f, 0.f);
-            bool ok = gather_vote(true);
-            const uint32_t ch_bytes = 4u * (uint32_t)g.slab_chpitch;
-            for (int j = 0; j < ic_chunks; ++j) {
-                const int b = j & 1;                     // pixel-major buffer; the staging buffer is always the same one
-                if (ok && !mbar_wait(smem_u32(&slab_full[0]), (uint32_t)j & 1u, abortp, g.status, 6u, g.wait_ns)) ok = false;
-                if (ok && j >= 2 && !mbar_wait(smem_u32(&pm_empty[b]), (uint32_t)((j - 2) >> 1) & 1u, abortp, g.status, 8u, g.wait_ns)) ok = false;
-                if (ok) {
-                    // warp gw moves channels 4 gw .. 4 gw + 3 of every staged position; lanes walk positions
-                    const uint32_t src = st0 + (uint32_t)(4 * gw) * ch_bytes;
-                    const uint32_t dst = pm0 + (uint32_t)b * g.pm_buf_bytes;
-                    for (int p0 = lane; p0 < npix; p0 += 128) {
-                        float v[4][4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int pix = min(p0 + 32 * u, npix - 1);
-                            const uint32_t a = src + 4u * (uint32_t)pix;
-                            v[u][0] = ld_shared_f32(a);
-                            v[u][1] = ld_shared_f32(a + ch_bytes);
-                            v[u][2] = ld_shared_f32(a + 2u * ch_bytes);
-                            v[u][3] = ld_shared_f32(a + 3u * ch_bytes);
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int pix = p0 + 32 * u;
-                            if (pix < npix) {
-                                const uint32_t rowa = dst + 128u * (uint32_t)pix;
-                                st_shared_v4(rowa + ((((uint32_t)gw) ^ ((rowa >> 7) & 7u)) << 4), v[u][0], v[u][1], v[u][2], v[u][3]);
-                            }
-                        }
-                    }
-                    fence_proxy_async_shared();          // generic-proxy stores -> visible to the tensor core's reads
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(smem_u32(&pm_full[b]));
-                        if (j + 1 < ic_chunks) mbar_arrive(smem_u32(&slab_empty[0]));   // the staging buffer may be refilled
-                    }
-                }
-            }
         } else if (any_gather) {
             const float* a_src = g.a + (long long)bz * g.a_bs;
             const float* b_src = g.b + (long long)bz * g.b_bs;
@@ -1506,7 +1008,6 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 e.hi = g.act == TT_ACT_RELU6 ? 6.f : INFINITY;
                 e.gelu = g.act == TT_ACT_GELU_ERF;
                 e.vec = (g.vec_store & 1) != 0;
-                e.lin_wp = tapm ? g.slab_wp : 0; e.lin_q = g.Q; e.lin_p = g.Pout;
                 const bool transposed = g.y_ns == 1 && g.y_ms != 1;
                 const uint32_t stg = tiles_base + (uint32_t)gw * (uint32_t)kStageBytesPerWarp;   // pipeline buffers are idle now
                 const int m_first = m0 + quad * 32;
@@ -1557,7 +1058,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                         }
                     }
                     // full blocks take the unguarded path (16-byte accesses need the aligned layout when transposed)
-                    const bool full = !tapm && cnt >= 32 && m_first + 32 <= g.M && (e.vec || !transposed);
+                    const bool full = cnt >= 32 && m_first + 32 <= g.M && (e.vec || !transposed);
                     if (e.rbase == nullptr) {
                         // no residual: activate here, once, outside the store loops
                         if (e.gelu) {
@@ -1732,11 +1233,6 @@ __device__ __forceinline__ void mma_commit_cg(uint32_t bar) {
         asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                      ::"r"(bar), "h"(mask) : "memory");
     }
-}
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
 }
 // Arrive on the barrier at the same offset in the CTA of rank `rank` of this cluster.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar, uint32_t rank) {
@@ -1966,7 +1462,6 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         e.hi = g.act == TT_ACT_RELU6 ? 6.f : INFINITY;
         e.gelu = g.act == TT_ACT_GELU_ERF;
         e.vec = (g.vec_store & 1) != 0;
-        e.lin_wp = 0; e.lin_q = 0; e.lin_p = 0;
         const bool transposed = g.y_ns == 1 && g.y_ms != 1;
         const bool tma_out = g.epi_tma != 0, res_in = g.res_tma != 0;
         const uint32_t ring = tiles_base + g.epi_off + (uint32_t)ew * g.epi_warp_bytes;
@@ -2128,384 +1623,6 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         tc_fence_after();
         if constexpr (CG == 1) tmem_dealloc(tmem_base, g.tmem_cols);
         else asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(g.tmem_cols) : "memory");
-    }
-}
-
-// ------------------------------------------------------------------------------------------------------------
-// GEMM_TC, persistent form of the tap-major convolution (records with k_order = 1 and persistent = 1): the same walk over
-// output tiles with two accumulators; operand A = re-packed filters by TMA, operand B = views of a pixel-major slab that
-// four transposer warps write once per 32-channel block from a staged NCHW box.
-// Warps: 0 TMA producer, 1 MMA issuer + tensor-memory owner, 2-5 transposers, 6-9 read-out.
-// ------------------------------------------------------------------------------------------------------------
-constexpr int kPsTransposeWarps = 4;
-constexpr int kPsEpilogueWarps = 4;
-
-__global__ void __launch_bounds__(kGemmThreads, 1)
-tt_gemm_ps_tap_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_x, const GemmArgs g) {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[kMaxStages];     // a stage's operands are in place (TMA bytes and/or the transposer warps)
-    __shared__ uint64_t empty_bar[kMaxStages];    // every multiply-accumulate that reads the stage has completed
-    __shared__ uint64_t stg_full[kMaxStages];     // a staging box has landed
-    __shared__ uint64_t stg_empty[kMaxStages];    // the transposer warps are done with it
-    __shared__ uint64_t pm_full[2];               // tap-major convolution: a pixel-major slab buffer has been written
-    __shared__ uint64_t pm_empty[2];              // ... and every multiply-accumulate that reads it has completed
-    __shared__ uint64_t acc_full[2];              // an accumulator holds a finished tile
-    __shared__ uint64_t acc_empty[2];             // the read-out warps (of both CTAs) have drained it
-    __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
-    __shared__ __align__(16) float s_bias[2][256];
-
-    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    volatile int* abortp = &abort_flag;
-    pdl_allow_next();
-    const int unit = (int)blockIdx.x, n_units = (int)gridDim.x;
-    const int my_tiles = g.total_tiles > unit ? (g.total_tiles - unit + n_units - 1) / n_units : 0;
-    const int tiles_per_batch = g.tiles_m * g.tiles_n;
-    const int kt_n = g.k_tiles;
-
-    const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t stage_bytes = g.a_stage_bytes + g.b_stage_bytes;
-    // Tap-major convolution (see the one-tile kernel): operand A = re-packed filters by TMA; operand B = views of a
-    // pixel-major slab that the transposer warps write once per 32-channel block from a staged NCHW box.  Here the
-    // staging ring, the two slab buffers and the filter stages all run on across tile boundaries.
-    const int RS = g.R * g.S;
-    const int blocks_per_tile = kt_n * g.n_atoms / RS;     // 32-channel blocks
-
-    if (threadIdx.x == 32) {
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
-    }
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < g.stages; ++s) {
-            mbar_init(smem_u32(&full_bar[s]), 1u);
-            mbar_init(smem_u32(&empty_bar[s]), 1u);
-        }
-        for (int s = 0; s < g.stg_depth; ++s) {
-            mbar_init(smem_u32(&stg_full[s]), 1u);
-            mbar_init(smem_u32(&stg_empty[s]), (uint32_t)kPsTransposeWarps);
-        }
-        for (int a = 0; a < 2; ++a) {
-            mbar_init(smem_u32(&pm_full[a]), (uint32_t)kPsTransposeWarps);
-            mbar_init(smem_u32(&pm_empty[a]), 1u);
-            mbar_init(smem_u32(&acc_full[a]), 1u);
-            mbar_init(smem_u32(&acc_empty[a]), (uint32_t)kPsEpilogueWarps);
-        }
-        abort_flag = 0;
-        fence_mbar_init();
-        fence_proxy_async_shared();
-    }
-    if (warp == 1) {
-        tmem_alloc(smem_u32(&tmem_slot), g.tmem_cols);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *(volatile uint32_t*)&tmem_slot;
-    pdl_wait_prev();                                      // the set-up above touched no global memory
-
-    auto decode = [&](int i, int& m0, int& n0, int& bz) {
-        const int t = unit + i * n_units;
-        bz = t / tiles_per_batch;
-        const int r = t - bz * tiles_per_batch;
-        int tm, tn;
-        if (g.raster == 0) { tm = r % g.tiles_m; tn = r / g.tiles_m; }
-        else               { tn = r % g.tiles_n; tm = r / g.tiles_n; }
-        m0 = tm * kHwTileM;
-        n0 = tn * g.tile_n;
-    };
-
-    if (warp == 0) {
-        // ---------------- TMA producer ----------------
-        // Two independent streams of requests, each with its own ring and cursor: NCHW boxes of input rows go to the staging
-        // ring, filter tiles to the pipeline stages.  The warp polls both rings and serves whichever has a free slot.
-        const bool leader = elect_one();
-        const uint32_t a_atom = (uint32_t)(kHwTileM * g.row_bytes);
-        struct Cursor { int i, kt, m0, n0, bz, slot; uint32_t ph; long long it; };
-        const long long total_it = (long long)my_tiles * kt_n;
-        const long long total_s = (long long)my_tiles * blocks_per_tile;    // a staging box per 32-channel block
-        auto cur_init = [&](Cursor& c) {
-            c.i = 0; c.kt = 0; c.slot = 0; c.ph = 0; c.it = 0; c.m0 = c.n0 = c.bz = 0;
-            if (my_tiles > 0) decode(0, c.m0, c.n0, c.bz);
-        };
-        auto cur_next = [&](Cursor& c, int depth, int inner) {
-            ++c.it;
-            if (++c.slot == depth) { c.slot = 0; c.ph ^= 1u; }
-            if (++c.kt == inner) {
-                c.kt = 0;
-                if (++c.i < my_tiles) decode(c.i, c.m0, c.n0, c.bz);
-            }
-        };
-        Cursor cs, ck;
-        cur_init(cs); cur_init(ck);
-        bool ok = true;
-        unsigned long long t_last = global_timer_ns();
-        unsigned idle = 0;
-        while (cs.it < total_s || ck.it < total_it) {
-            bool progressed = false;
-            if (cs.it < total_s && mbar_test_wait(smem_u32(&stg_empty[cs.slot]), cs.ph ^ 1u)) {
-                if (leader) {
-                    // the input rows of 32-channel block cs.kt behind this tile's pixels: one box that starts `gap` columns
-                    // left of the image and at the tile's first input row (zero fill supplies padding and gaps)
-                    const uint32_t bar = smem_u32(&stg_full[cs.slot]);
-                    mbar_expect_tx(bar, g.slab_box_bytes);
-                    tma_load_4d(tiles_base + g.slab_off + (uint32_t)cs.slot * g.slab_buf_bytes, &tmap_x, bar, -g.slab_gap,
-                                cs.n0 / g.slab_wp - g.ph, cs.kt * 32, cs.bz);
-                }
-                __syncwarp();
-                cur_next(cs, g.stg_depth, blocks_per_tile);
-                progressed = true;
-            }
-            if (ck.it < total_it && mbar_test_wait(smem_u32(&empty_bar[ck.slot]), ck.ph ^ 1u)) {
-                if (leader) {
-                    const uint32_t bar = smem_u32(&full_bar[ck.slot]);
-                    // (test facility: the first stage may be told to expect more than arrives, see tt_workload_test_stall)
-                    mbar_expect_tx(bar, g.a_stage_bytes + (ck.it == 0 ? g.extra_tx : 0u));
-                    uint32_t dst = tiles_base + (uint32_t)ck.slot * stage_bytes;
-                    int kc = ck.kt * g.tile_k;
-#pragma unroll 1
-                    for (int at = 0; at < g.n_atoms; ++at, dst += a_atom, kc += g.atom_k) tma_load_3d(dst, &tmap_a, bar, kc, ck.m0, 0);
-                }
-                __syncwarp();
-                cur_next(ck, g.stages, kt_n);
-                progressed = true;
-            }
-            if (progressed) { idle = 0; continue; }
-            if ((++idle & 63u) == 0u) {
-                // nothing to do for a while: the same bounded patience as every other wait of the kernel
-                if (idle == 64u) t_last = global_timer_ns();
-                bool give_up = *abortp != 0;
-                if (!give_up && global_timer_ns() - t_last > g.wait_ns) {
-                    *abortp = 1;
-                    atomicCAS(g.status, 0u, (unsigned)TT_ERR_TIMEOUT | (1u << 8));
-                    give_up = true;
-                }
-                if (__any_sync(0xffffffffu, give_up)) { ok = false; break; }
-            }
-        }
-        if ((!ok || *abortp) && lane == 0) {
-            // let copies in flight land before shared memory is given back (bounded)
-            for (int pass = 0; pass < 2; ++pass) {
-                const long long issued = pass == 0 ? ck.it : cs.it;
-                const int depth = pass == 0 ? g.stages : g.stg_depth;
-                const long long first = issued > depth ? issued - depth : 0;
-                for (long long it = first; it < issued; ++it) {
-                    const uint32_t bar = pass == 0 ? smem_u32(&full_bar[it % depth]) : smem_u32(&stg_full[it % depth]);
-                    const uint32_t par = (uint32_t)(it / depth) & 1u;
-                    const unsigned long long t0 = global_timer_ns();
-                    while (!mbar_try_wait(bar, par)) { if (global_timer_ns() - t0 > 2000000ull) break; }
-                }
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
-        const bool leader = elect_one();
-        uint32_t st = 0, ph = 0;
-        bool ok = true;
-        {
-            const uint64_t d0 = make_desc(0u, g.row_bytes);
-            const uint32_t d_hi = (uint32_t)(d0 >> 32), d_lo = (uint32_t)d0;
-            const uint32_t a_lo0 = d_lo + ((tiles_base & 0x3FFFFu) >> 4);
-            const uint32_t stage_step = stage_bytes >> 4;
-            const uint32_t a_atom = (uint32_t)(kHwTileM * g.row_bytes) >> 4;
-            uint32_t gblock = 0;                         // tap-major: 32-channel blocks consumed so far, over all tiles
-            for (int i = 0; i < my_tiles && ok; ++i) {
-                const uint32_t acc = (uint32_t)i & 1u, aph = ((uint32_t)i >> 1) & 1u;
-                // the read-out of the tile that used this accumulator two tiles ago has finished
-                const bool freed = mbar_wait(smem_u32(&acc_empty[acc]), aph ^ 1u, abortp, g.status, 12u, g.wait_ns);
-                if (!__all_sync(0xffffffffu, freed)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + acc * (uint32_t)g.tile_n;
-                {
-                    // the B tile of reduction tile kt = (channel block, taps) is the block's pixel-major slab read from row
-                    // lin0 + r * wp + s on: only the descriptor's start address changes from tap to tap
-                    int m0t, n0t, bzt;
-                    decode(i, m0t, n0t, bzt);
-                    const uint32_t pm0 = tiles_base + g.pm_off;
-                    const int lin0 = (n0t - (n0t / g.slab_wp) * g.slab_wp) + g.slab_gap - g.pw;
-                    int tap = 0, fr = 0, fs = 0;
-                    for (int kt = 0; kt < kt_n; ++kt) {
-                        bool got = mbar_wait(smem_u32(&full_bar[st]), ph, abortp, g.status, 2u, g.wait_ns);        // the filter tile
-                        if (tap == 0 && got) got = mbar_wait(smem_u32(&pm_full[gblock & 1u]), (gblock >> 1) & 1u, abortp, g.status, 7u, g.wait_ns);
-                        if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-                        tc_fence_after();
-                        if (leader) {
-                            uint32_t a_lo = a_lo0 + st * stage_step;
-                            int r2 = fr, s2 = fs;
-#pragma unroll 1
-                            for (int t = 0; t < g.n_atoms; ++t, a_lo += a_atom) {
-                                const uint32_t row = (uint32_t)(lin0 + r2 * g.slab_wp + s2);
-                                const uint32_t b_lo = d_lo + (((pm0 + (gblock & 1u) * g.pm_buf_bytes + row * 128u) & 0x3FFFFu) >> 4);
-#pragma unroll
-                                for (int k8 = 0; k8 < 4; ++k8)
-                                    mma_tf32(d_tmem, ((uint64_t)d_hi << 32) | (uint64_t)(a_lo + 2u * (uint32_t)k8),
-                                                    ((uint64_t)d_hi << 32) | (uint64_t)(b_lo + 2u * (uint32_t)k8), g.idesc,
-                                                    (kt > 0 || t > 0 || k8 > 0) ? 1u : 0u);
-                                if (++s2 == g.S) { s2 = 0; ++r2; }
-                            }
-                            mma_commit(smem_u32(&empty_bar[st]));                           // filter stage reusable
-                            if (tap + g.n_atoms == RS) mma_commit(smem_u32(&pm_empty[gblock & 1u]));   // slab buffer reusable
-                        }
-                        __syncwarp();
-                        for (int t = 0; t < g.n_atoms; ++t) if (++fs == g.S) { fs = 0; ++fr; }
-                        tap += g.n_atoms;
-                        if (tap == RS) { tap = 0; fr = 0; fs = 0; ++gblock; }
-                        if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
-                    }
-                }
-                if (ok && leader) mma_commit(smem_u32(&acc_full[acc]));   // the tile's accumulator is complete
-                __syncwarp();
-            }
-        }
-    } else if (warp < 2 + kPsTransposeWarps) {
-        // ---------------- transposers ----------------
-        {
-            // staging box [32 channels][in_rows][wp] -> pixel-major slab: one 128-byte row per staged position (32
-            // channels), 16-byte chunks swizzled by the row's absolute address like a TMA 128-byte tile.  Warp tw moves
-            // the channel groups tw and tw + 4 of every position; lanes walk positions.
-            const int tw = warp - 2;
-            const int tt = (int)threadIdx.x - 64;
-            const uint32_t st0 = tiles_base + g.slab_off, pm0 = tiles_base + g.pm_off;
-            const int npix = g.slab_in_rows * g.slab_wp;
-            // rows a view can touch beyond the transposed range must hold finite numbers: clear both buffers once
-            for (uint32_t o = (uint32_t)tt * 16u; o < 2u * g.pm_buf_bytes; o += 32u * kPsTransposeWarps * 16u)
-                st_shared_v4(pm0 + o, 0.f, 0.f, 0.f, 0.f);
-            if (g.slab_box_ch < 32)                      // channels beyond the TMA box (which may already be landing) read as zero
-                for (int sl = 0; sl < g.stg_depth; ++sl)
-                    for (uint32_t o = g.slab_box_bytes + (uint32_t)tt * 16u; o < g.slab_buf_bytes; o += 32u * kPsTransposeWarps * 16u)
-                        st_shared_v4(st0 + (uint32_t)sl * g.slab_buf_bytes + o, 0.f, 0.f, 0.f, 0.f);
-            asm volatile("bar.sync 3, %0;" ::"n"(32 * kPsTransposeWarps) : "memory");
-            const uint32_t ch_bytes = 4u * (uint32_t)g.slab_chpitch;
-            uint32_t sst = 0, sph = 0, gb = 0;
-            bool ok = true;
-            const long long total_blocks = (long long)my_tiles * blocks_per_tile;
-            for (long long j = 0; j < total_blocks && ok; ++j, ++gb) {
-                const uint32_t b = gb & 1u;
-                if (!mbar_wait(smem_u32(&stg_full[sst]), sph, abortp, g.status, 6u, g.wait_ns) ||
-                    !mbar_wait(smem_u32(&pm_empty[b]), ((gb >> 1) & 1u) ^ 1u, abortp, g.status, 8u, g.wait_ns)) { ok = false; break; }
-                const uint32_t dst = pm0 + b * g.pm_buf_bytes;
-#pragma unroll 1
-                for (int grp = tw; grp < 8; grp += kPsTransposeWarps) {
-                    const uint32_t src = st0 + sst * g.slab_buf_bytes + (uint32_t)(4 * grp) * ch_bytes;
-                    for (int p0 = lane; p0 < npix; p0 += 128) {
-                        float v[4][4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int pix = min(p0 + 32 * u, npix - 1);
-                            const uint32_t a = src + 4u * (uint32_t)pix;
-                            v[u][0] = ld_shared_f32(a);
-                            v[u][1] = ld_shared_f32(a + ch_bytes);
-                            v[u][2] = ld_shared_f32(a + 2u * ch_bytes);
-                            v[u][3] = ld_shared_f32(a + 3u * ch_bytes);
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int pix = p0 + 32 * u;
-                            if (pix < npix) {
-                                const uint32_t rowa = dst + 128u * (uint32_t)pix;
-                                st_shared_v4(rowa + ((((uint32_t)grp) ^ ((rowa >> 7) & 7u)) << 4), v[u][0], v[u][1], v[u][2], v[u][3]);
-                            }
-                        }
-                    }
-                }
-                fence_proxy_async_shared();              // generic-proxy stores -> visible to the tensor core's reads
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(smem_u32(&pm_full[b]));
-                    mbar_arrive(smem_u32(&stg_empty[sst]));
-                }
-                if (++sst == (uint32_t)g.stg_depth) { sst = 0; sph ^= 1u; }
-            }
-        }
-    } else {
-        // ---------------- read-out: tensor memory -> bias, residual, activation -> global memory ----------------
-        const int ew = warp - (2 + kPsTransposeWarps);
-        const int et = (int)threadIdx.x - 32 * (2 + kPsTransposeWarps);
-        const int quad = warp & 3;                       // tensor-memory lane quadrant this warp may read
-        EpiArgs e;
-        e.y_ms = g.y_ms; e.y_ns = g.y_ns; e.M = g.M;
-        e.lo = g.act == TT_ACT_NONE || g.act == TT_ACT_GELU_ERF ? -INFINITY : 0.f;
-        e.hi = g.act == TT_ACT_RELU6 ? 6.f : INFINITY;
-        e.gelu = g.act == TT_ACT_GELU_ERF;
-        e.vec = (g.vec_store & 1) != 0;
-        e.lin_wp = g.slab_wp; e.lin_q = g.Q; e.lin_p = g.Pout;
-        const bool transposed = g.y_ns == 1 && g.y_ms != 1;
-        const uint32_t stg = tiles_base + g.epi_off + (uint32_t)ew * (uint32_t)kStageBytesPerWarp;
-        bool ok = true;
-        for (int i = 0; i < my_tiles && ok; ++i) {
-            int m0, n0, bz;
-            decode(i, m0, n0, bz);
-            const uint32_t acc = (uint32_t)i & 1u, aph = ((uint32_t)i >> 1) & 1u;
-            const int m_first = m0 + quad * 32, m = m_first + lane;
-            // this tile's bias values, staged while the tile is still being accumulated (the buffer's previous readers
-            // finished two tiles ago: they passed the barrier below for tile i - 1 since)
-            if (g.bias_mode == 2) for (int c = et; c < g.tile_n; c += 32 * kPsEpilogueWarps) s_bias[acc][c] = (n0 + c < g.N) ? __ldg(g.bias + n0 + c) : 0.f;
-            const float bias_row = (g.bias_mode == 1 && m < g.M) ? __ldg(g.bias + m) : 0.f;
-            const bool have = mbar_wait(smem_u32(&acc_full[acc]), aph, abortp, g.status, 4u, g.wait_ns);
-            uint32_t all_acc;
-            asm volatile(
-                "{\n\t.reg .pred p, q;\n\t"
-                "setp.ne.u32 q, %1, 0;\n\t"
-                "bar.red.and.pred p, 2, %2, q;\n\t"
-                "selp.u32 %0, 1, 0, p;\n\t}"
-                : "=r"(all_acc) : "r"((uint32_t)have), "n"(32 * kPsEpilogueWarps) : "memory");
-            if (!all_acc) { ok = false; break; }
-            tc_fence_after();
-            e.ybase = g.y + (long long)bz * g.y_bs;
-            e.rbase = g.residual ? g.residual + (long long)bz * g.y_bs : nullptr;
-            const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * (uint32_t)g.tile_n;
-            uint32_t r[32];
-            tmem_ld32(t_row, r);
-#pragma unroll 1
-            for (int c0 = 0; c0 < g.tile_n; c0 += 32) {
-                float v[32];
-                const int nb = n0 + c0;
-                const int cnt = min(g.N - nb, g.tile_n - c0);
-                tmem_wait_ld();
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-                if (c0 + 32 < g.tile_n) tmem_ld32(t_row + (uint32_t)(c0 + 32), r);
-                else {
-                    // every value of this accumulator is in registers: hand it back to the MMA warp
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(smem_u32(&acc_empty[acc]));
-                    }
-                }
-                if (cnt <= 0) continue;                  // warp-uniform
-                if (g.bias_mode == 1) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] += bias_row;
-                } else if (g.bias_mode == 2) {
-#pragma unroll
-                    for (int j = 0; j < 32; j += 4) {
-                        const float4 b = *reinterpret_cast<const float4*>(&s_bias[acc][c0 + j]);
-                        v[j] += b.x; v[j + 1] += b.y; v[j + 2] += b.z; v[j + 3] += b.w;
-                    }
-                }
-                if (e.rbase == nullptr) {
-                    if (e.gelu) {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) v[j] = gelu_erf(v[j]);
-                    } else if (g.act != TT_ACT_NONE) {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) v[j] = fminf(fmaxf(v[j], e.lo), e.hi);
-                    }
-                    epilogue_block<false, false>(v, e, m_first, nb, cnt, stg, lane, transposed);
-                } else {
-                    epilogue_block<false, true>(v, e, m_first, nb, cnt, stg, lane, transposed);
-                }
-            }
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        __syncwarp();
-        tc_fence_after();
-        tmem_dealloc(tmem_base, g.tmem_cols);
     }
 }
 
@@ -3078,22 +2195,6 @@ __global__ void tt_softmax_ragged_kernel(const RowArgs a, int chunk) {
     }
 }
 
-// Filters [kout][C][RS] -> [kout][block of 32 channels][tap][channel in block], zero beyond C: the reduction order of the
-// tap-major convolution.  One thread per output element; reads walk the channels of a tap (stride RS), writes are
-// contiguous.
-__global__ void tt_repack_filters_kernel(const float* __restrict__ w, float* __restrict__ out, int kout, int C, int RS, int CB) {
-    const long long per_filter = (long long)CB * RS * 32;
-    const long long total = (long long)kout * per_filter;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const long long f = i / per_filter;
-        const int rem = (int)(i - f * per_filter);
-        const int ci = rem & 31, t2 = rem >> 5;
-        const int cb = t2 / RS, tap = t2 - cb * RS;
-        const int c = cb * 32 + ci;
-        out[i] = c < C ? __ldg(w + (f * C + c) * RS + tap) : 0.f;
-    }
-}
-
 // A kernel that does nothing, for the launch floor: launched with a record's grid, block size, shared memory,
 // cluster shape and dependent-launch attribute, its time is what a launch of that record costs before any work.
 __global__ void tt_floor_kernel() {
@@ -3109,12 +2210,11 @@ __global__ void tt_floor_kernel() {
 static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <= 112 * 1024 && tmem_cols <= 256; }
 
 typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
-static const GemmKernel kGemmKernels[2][5] = {
-    {tt_gemm_tc_kernel<1, kFormTma>, tt_gemm_tc_kernel<1, kFormMn>, tt_gemm_tc_kernel<1, kFormIm2col>, tt_gemm_tc_kernel<1, kFormTap>, tt_gemm_tc_kernel<1, kFormGather>},
-    {tt_gemm_tc_kernel<2, kFormTma>, tt_gemm_tc_kernel<2, kFormMn>, tt_gemm_tc_kernel<2, kFormIm2col>, tt_gemm_tc_kernel<2, kFormTap>, tt_gemm_tc_kernel<2, kFormGather>}};
+static const GemmKernel kGemmKernels[2][4] = {
+    {tt_gemm_tc_kernel<1, kFormTma>, tt_gemm_tc_kernel<1, kFormMn>, tt_gemm_tc_kernel<1, kFormIm2col>, tt_gemm_tc_kernel<1, kFormGather>},
+    {tt_gemm_tc_kernel<2, kFormTma>, tt_gemm_tc_kernel<2, kFormMn>, tt_gemm_tc_kernel<2, kFormIm2col>, tt_gemm_tc_kernel<2, kFormGather>}};
 
 static int gemm_form(const GemmArgs& g) {
-    if (g.tap_major) return kFormTap;
     if (g.a_mode == OPM_IM2COL || g.b_mode == OPM_IM2COL) return kFormIm2col;
     const bool a = g.a_mode == OPM_TMA || g.a_mode == OPM_TMA_MN, b = g.b_mode == OPM_TMA || g.b_mode == OPM_TMA_MN;
     if (!a || !b) return kFormGather;
@@ -3124,7 +2224,7 @@ static int gemm_form(const GemmArgs& g) {
 // Which instantiation a plan runs; its shared-memory limit is raised once per device.  Which build (two CTAs per SM) is the
 // record's choice (ctas_per_sm), resolved by the legaliser.
 static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel* out) {
-    static std::atomic<uint64_t> raised[2][5];           // a bit per device
+    static std::atomic<uint64_t> raised[2][4];           // a bit per device
     const int two = g.two_per_sm && gemm_two_per_sm(smem_bytes, g.tmem_cols), form = gemm_form(g);
     int dev = 0;
     cudaGetDevice(&dev);
@@ -3175,12 +2275,11 @@ cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const Tmap
     if (attr_set_for != dev) {
         cudaError_t e = cudaFuncSetAttribute(tt_gemm_ps_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(tt_gemm_ps_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tt_gemm_ps_tap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
         if (e != cudaSuccess) return e;
         cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
         attr_set_for = dev;
     }
-    CUtensorMap ta, tb, tx, ty, tr;
+    CUtensorMap ta, tb, ty, tr;
     memcpy(&ta, maps.a, sizeof ta);
     memcpy(&tb, maps.b, sizeof tb);
     const int cg = g.cta_group == 2 ? 2 : 1;
@@ -3199,10 +2298,6 @@ cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const Tmap
         ++n_attr;
     }
     cfg.attrs = attr; cfg.numAttrs = (unsigned)n_attr;
-    if (g.tap_major) {
-        memcpy(&tx, maps.x, sizeof tx);
-        return cudaLaunchKernelEx(&cfg, tt_gemm_ps_tap_kernel, ta, tx, g);
-    }
     memcpy(&ty, maps.y, sizeof ty);
     memcpy(&tr, maps.r, sizeof tr);
     if (cg == 2) return cudaLaunchKernelEx(&cfg, tt_gemm_ps_kernel<2>, ta, tb, ty, tr, g);
@@ -3251,13 +2346,6 @@ cudaError_t launch_floor(const tt_apply_info& I, int cluster, cudaStream_t st) {
     }
     cfg.attrs = attr; cfg.numAttrs = (unsigned)n_attr;
     return cudaLaunchKernelEx(&cfg, tt_floor_kernel);
-}
-
-cudaError_t launch_repack(const float* w, float* out, int kout, int C, int RS, int CB, cudaStream_t st) {
-    const long long total = (long long)kout * CB * RS * 32;
-    const int blocks = (int)std::min<long long>((total + 255) / 256, 148 * 8);
-    tt_repack_filters_kernel<<<blocks, 256, 0, st>>>(w, out, kout, C, RS, CB);
-    return cudaGetLastError();
 }
 
 // Launch with programmatic stream serialization (the kernels wait before their first global access): in a stream or

@@ -987,3 +987,28 @@ def test_mn_major_operands_and_tma_read_out(spec):
         assert probe.check(rec)[0] == B.TT_OK
         run_spec(spec, rec, a, ref, ref_elem=re)
     probe.close()
+
+
+@pytest.mark.parametrize("shape", [
+    # n, c, h, w, k, r, s, stride_h, stride_w, pad_h, pad_w, residual
+    (3, 33, 7, 7, 40, 3, 3, 1, 1, 1, 1, True), (5, 8, 9, 5, 130, 3, 3, 2, 2, 1, 1, False), (2, 64, 14, 14, 16, 1, 1, 2, 2, 0, 0, True),
+    (2, 40, 11, 13, 24, 5, 3, 2, 1, 2, 0, False), (4, 16, 6, 6, 20, 2, 4, 3, 2, 0, 3, True), (2, 70, 23, 8, 150, 7, 7, 1, 1, 3, 3, False),
+    (160, 32, 8, 8, 136, 3, 3, 1, 1, 1, 1, True), (70, 40, 9, 9, 40, 3, 3, 2, 2, 1, 1, True), (1, 96, 12, 12, 48, 3, 3, 1, 1, 1, 1, True),
+], ids=lambda s: "x".join(map(str, s)))
+def test_tap_major_convolutions_of_every_layout(shape):
+    """The tap-major order over padded-linear positions of a whole batch: rows that are no 16-byte multiples, tiles that
+    cross rows and images, strides (one sub-image per parity class), unequal padding, partial channel blocks, the skip
+    tensor, channel blocks shared by a cluster, and tiles that CTAs walk with two accumulators."""
+    n, c, h, w, k, r, s, sh, sw, ph, pw, res = shape
+    sp = W.Spec(B.TT_OP_CONV2D, B.make_shapes(n=n, c=c, h=h, w=w, k=k, r=r, s=s, stride_h=sh, stride_w=sw, pad_h=ph, pad_w=pw, has_bias=1,
+                                              has_residual=int(res), act=B.TT_ACT_RELU), 1, "tap", "uniform")
+    a = W.make_inputs(sp, 94)
+    ref = util.oracle_ref(sp, a)
+    re = elem_ref(sp, a, ref)
+    probe = sp.workload()
+    for tn, tk, st, ps in ((16, 32, 4, 0), (224, 96, 2, 0), (128, 32, 2, 1), (64, 128, 8, 0)):
+        rec = tc(tile_n=tn, tile_k=tk, stages=st, k_order=1, persistent=ps, mma_m_axis=1)
+        stat, info = probe.check(rec)
+        assert stat == B.TT_OK and info.legal.k_order == 1
+        run_spec(sp, rec, a, ref, ref_elem=re)
+    probe.close()
