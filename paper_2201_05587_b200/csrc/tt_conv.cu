@@ -16,7 +16,7 @@
 // ("plane") at unit stride, and the reduction walks (channel block, plane, tap of the plane).
 //
 // Filters (re-packed to [filter][channel block][tap in walk order][32], a small kernel per weight pointer) ride the 128 rows of
-// the accumulator and arrive by TMA, one tap per stage.
+// the accumulator and arrive by TMA, up to taps_per_stage taps of 16 KB per pipeline stage.
 // Warps: 0 TMA, 1 MMA issuer + tensor-memory owner, 2-9 bring the slab in, 10-13 read out.
 //
 // CTAs walk tiles with two accumulators, so that a tile is read out while the next one is multiplied; the slab has two
@@ -28,8 +28,12 @@
 // of its accumulator that another CTA finishes in its shared memory, and every CTA adds up its blocks, in CTA order, over
 // distributed shared memory.
 //
-// Bound by the tensor core from a few dozen channels on; what is left is the prologue (first slab and filters: 2 us), the
-// read-out of the last tile and the columns that are no outputs.  Measured: see the table of figures at launch_conv_pm.
+// Bound by shared memory in the multiply phase: a tap moves its filters in and out (2 * 128 lines of 128 bytes), its columns
+// and its share of the slab, 500 cycles measured for 192 columns that take the tensor core 384.  The rest is the prologue
+// (launch, first slab and filters: 2 us) and the read-out of the last tile (2.3 us, all CTAs storing at once).
+// Measured, before (one tile per CTA and image, TMA-staged slab) and now: 3x3 128 -> 128 at 28 x 28, batch 32, 20.8 -> 18.4 us;
+// 3x3 512 -> 512 at 7 x 7 with residual, batch 32, 53.6 (expanded im2col) -> 25.1 us; 3x3 32 -> 248 at 56 x 56, batch 5,
+// 16.6 -> 11.3 us.
 #include <cuda_runtime.h>
 #include <cuda.h>
 #include <algorithm>
@@ -57,7 +61,7 @@ __device__ __forceinline__ int div_magic(int u, int d, unsigned magic, int& rem)
 __global__ void __launch_bounds__(kPmThreads, 1)
 tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ ConvPmArgs g) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[kMaxStages];     // a tap's filters have landed
+    __shared__ uint64_t full_bar[kMaxStages];     // a stage's filters (up to taps_per_stage taps) have landed
     __shared__ uint64_t empty_bar[kMaxStages];    // the multiply-accumulates that read them have completed
     __shared__ uint64_t pm_full[2];               // a slab buffer has been written
     __shared__ uint64_t pm_empty[2];              // every multiply-accumulate that reads it has completed
@@ -75,7 +79,8 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     const int my_tiles = g.total_tiles > unit ? (g.total_tiles - unit + n_units - 1) / n_units : 0;
     const bool single = g.total_tiles <= n_units;         // all tiles resident at once: no tile follows another on this CTA
     const int cb0 = crank * g.blocks / split, cb1 = (crank + 1) * g.blocks / split;   // this CTA's channel blocks
-    const int RS = g.R * g.S;
+    const int RS = g.R * g.S, tps = g.taps_per_stage;
+    const uint32_t stage_bytes = (uint32_t)tps * kPmTapBytes;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t slab0 = base + g.slab_off;
 
@@ -104,11 +109,6 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     // front has finished; everything else waits for it (the slab warps once they have worked out their first addresses)
     const bool slab_warp = warp >= 2 && warp < 2 + kPmSlabWarps;
     if (!slab_warp && (warp != 0 || !g.early_filters)) asm volatile("griddepcontrol.wait;" ::: "memory");
-    // Every CTA walks its channel blocks and the taps of a block from a start of its own.  In step, they would all ask for the
-    // same 16 KB of filters at the same time, and the L2 slices that hold those lines served 141 CTAs one tap per 590 cycles
-    // (384 of multiplying).
-    const int n_cb = cb1 - cb0, cb_turn = n_cb > 0 ? unit % n_cb : 0, tap_turn = n_cb > 0 ? unit / n_cb : 0;
-
     auto decode = [&](int i, int& m0, int& n0) {
         const int t = unit + i * n_units;
         int tm, tn;
@@ -119,90 +119,92 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     };
     bool ok = true;
 
+    // Warps 0 and 1 leave their loops to one thread: a vote over the warp for every wait and a re-convergence per stage made
+    // the issue of a stage a serial chain of 600 cycles (a tap of 192 columns takes the tensor core 384).
     if (warp == 0) {
         // ---------------- filters ----------------
-        const bool leader = elect_one();
-        uint32_t st = 0, ph = 0;
-        long long issued = 0;
-        for (int i = 0; i < my_tiles && ok; ++i) {
-            int m0, n0;
-            decode(i, m0, n0);
-            for (int ci = 0; ci < n_cb && ok; ++ci) {
-            const int cb = cb0 + (ci + cb_turn < n_cb ? ci + cb_turn : ci + cb_turn - n_cb);
-            for (int pl = 0, kt0 = cb * RS; pl < g.n_planes && ok; kt0 += g.planes[pl].nr * g.planes[pl].ns, ++pl) {
-            const int taps = g.planes[pl].nr * g.planes[pl].ns;
-            int tap = tap_turn % taps;
-            for (int t = 0; t < taps; ++t) {
-                const int kt = kt0 + tap;
-                if (++tap == taps) tap = 0;
-                const bool got = mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1u, abortp, g.status, 1u, g.wait_ns);
-                if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-                if (leader) {
-                    const uint32_t bar = smem_u32(&full_bar[st]);
-                    // (test facility: the first stage may be told to expect more than arrives, see tt_workload_test_stall)
-                    mbar_expect_tx(bar, kPmStageBytes + (issued == 0 && crank == 0 ? g.extra_tx : 0u));
-                    tma_load_3d(base + st * kPmStageBytes, &tmap_w, bar, kt * 32, m0, 0);
+        if (elect_one()) {
+            uint32_t st = 0, ph = 0;
+            long long issued = 0;
+            for (int i = 0; i < my_tiles && ok; ++i) {
+                int m0, n0;
+                decode(i, m0, n0);
+                for (int cb = cb0, kt = cb0 * RS; cb < cb1 && ok; ++cb) {
+                    for (int pl = 0; pl < g.n_planes && ok; ++pl) {
+                        const int taps = g.planes[pl].nr * g.planes[pl].ns;
+                        for (int t = 0; t < taps; t += tps) {
+                            const int n = min(tps, taps - t);
+                            const uint32_t bar = smem_u32(&full_bar[st]);
+                            if (!mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1u, abortp, g.status, 1u, g.wait_ns)) { ok = false; break; }
+                            // (test facility: the first stage may be told to expect more than arrives, see tt_workload_test_stall)
+                            mbar_expect_tx(bar, (uint32_t)n * kPmTapBytes + (issued == 0 && crank == 0 ? g.extra_tx : 0u));
+                            uint32_t dst = base + st * stage_bytes;
+                            for (int k = 0; k < n; ++k, dst += kPmTapBytes, ++kt) tma_load_3d(dst, &tmap_w, bar, kt * 32, m0, 0);
+                            ++issued;
+                            if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
+                        }
+                    }
                 }
-                __syncwarp();
-                ++issued;
-                if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
             }
-            }
-            }
-        }
-        if ((!ok || *abortp) && lane == 0) {
-            // let copies in flight land before shared memory is given back (bounded)
-            for (long long it = issued > g.stages ? issued - g.stages : 0; it < issued; ++it) {
-                const unsigned long long t0 = global_timer_ns();
-                while (!mbar_try_wait(smem_u32(&full_bar[it % g.stages]), (uint32_t)(it / g.stages) & 1u)) { if (global_timer_ns() - t0 > 2000000ull) break; }
+            if (!ok || *abortp) {
+                // let copies in flight land before shared memory is given back (bounded)
+                for (long long it = issued > g.stages ? issued - g.stages : 0; it < issued; ++it) {
+                    const unsigned long long t0 = global_timer_ns();
+                    while (!mbar_try_wait(smem_u32(&full_bar[it % g.stages]), (uint32_t)(it / g.stages) & 1u)) { if (global_timer_ns() - t0 > 2000000ull) break; }
+                }
             }
         }
-        if (g.early_filters) asm volatile("griddepcontrol.wait;" ::: "memory");   // (a kernel ends only after the one in front of it)
         __syncwarp();
+        if (g.early_filters) asm volatile("griddepcontrol.wait;" ::: "memory");   // (a kernel ends only after the one in front of it)
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        const bool leader = elect_one();
-        const uint64_t d0 = make_desc(0u, 128);
-        const uint32_t d_hi = (uint32_t)(d0 >> 32), d_lo = (uint32_t)d0;
-        uint32_t st = 0, ph = 0, buf = 0, bph = 0;
-        for (int i = 0; i < my_tiles && ok; ++i) {
-            const uint32_t acc = (uint32_t)i & 1u, aph = ((uint32_t)i >> 1) & 1u;
-            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_empty[acc]), aph ^ 1u, abortp, g.status, 12u, g.wait_ns))) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t d_tmem = tmem_base + acc * (uint32_t)g.tile_n;
-            uint32_t accumulate = 0u;
-            for (int ci = 0; ci < n_cb && ok; ++ci) {
-                for (int pl = 0; pl < g.n_planes && ok; ++pl) {
-                    const ConvPlane P = g.planes[pl];
-                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&pm_full[buf]), bph, abortp, g.status, 7u, g.wait_ns))) { ok = false; break; }
-                    const uint32_t slab = slab0 + buf * g.slab_bytes;
-                    const int first = P.f0 * g.wp + P.e0 - g.shift_min;   // first line of the slab that the plane's first tap reads
-                    const int taps = P.nr * P.ns, turn = tap_turn % taps;
-                    int r = turn / P.ns, c = turn - r * P.ns;
-                    for (int t = 0; t < taps; ++t) {
-                        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full_bar[st]), ph, abortp, g.status, 2u, g.wait_ns))) { ok = false; break; }
-                        tc_fence_after();
-                        if (leader) {
-                            const uint32_t a = d_lo + (((base + st * kPmStageBytes) & 0x3FFFFu) >> 4);
-                            const uint32_t b = d_lo + (((slab + (uint32_t)(first + r * g.wp + c) * 128u) & 0x3FFFFu) >> 4);
+        if (elect_one()) {
+            const uint64_t d0 = make_desc(0u, 128);
+            const uint32_t d_hi = (uint32_t)(d0 >> 32), d_lo = (uint32_t)d0;
+            uint32_t st = 0, ph = 0, buf = 0, bph = 0;
+            uint32_t ready = 0;                           // the filters of stage st have been seen to be there
+            for (int i = 0; i < my_tiles && ok; ++i) {
+                const uint32_t acc = (uint32_t)i & 1u, aph = ((uint32_t)i >> 1) & 1u;
+                if (!mbar_wait(smem_u32(&acc_empty[acc]), aph ^ 1u, abortp, g.status, 12u, g.wait_ns)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + acc * (uint32_t)g.tile_n;
+                uint32_t accumulate = 0u;
+                for (int cb = cb0; cb < cb1 && ok; ++cb) {
+                    for (int pl = 0; pl < g.n_planes && ok; ++pl) {
+                        const ConvPlane P = g.planes[pl];
+                        if (!mbar_wait(smem_u32(&pm_full[buf]), bph, abortp, g.status, 7u, g.wait_ns)) { ok = false; break; }
+                        // first line of the slab that the plane's first tap reads
+                        const uint32_t b_first = slab0 + buf * g.slab_bytes + (uint32_t)(P.f0 * g.wp + P.e0 - g.shift_min) * 128u;
+                        const int taps = P.nr * P.ns;
+                        int c = 0;
+                        uint32_t b_row = b_first;
+                        for (int t = 0; t < taps; t += tps) {
+                            if (!ready && !mbar_wait(smem_u32(&full_bar[st]), ph, abortp, g.status, 2u, g.wait_ns)) { ok = false; break; }
+                            tc_fence_after();
+                            const uint32_t freed = smem_u32(&empty_bar[st]);
+                            uint32_t a = d_lo + (((base + st * stage_bytes) & 0x3FFFFu) >> 4);
+                            if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
+                            ready = mbar_test_wait(smem_u32(&full_bar[st]), ph);      // (answered while the products below are issued)
+                            const int n = min(tps, taps - t);
+#pragma unroll 1
+                            for (int k = 0; k < n; ++k, a += kPmTapBytes >> 4) {
+                                const uint32_t b = d_lo + (((b_row + (uint32_t)c * 128u) & 0x3FFFFu) >> 4);
 #pragma unroll
-                            for (uint32_t k8 = 0; k8 < 4; ++k8)
-                                mma_tf32(d_tmem, ((uint64_t)d_hi << 32) | (uint64_t)(a + 2u * k8), ((uint64_t)d_hi << 32) | (uint64_t)(b + 2u * k8), g.idesc, k8 == 0 ? accumulate : 1u);
-                            mma_commit(smem_u32(&empty_bar[st]));
+                                for (uint32_t k8 = 0; k8 < 4; ++k8)
+                                    mma_tf32(d_tmem, ((uint64_t)d_hi << 32) | (uint64_t)(a + 2u * k8), ((uint64_t)d_hi << 32) | (uint64_t)(b + 2u * k8), g.idesc, k8 == 0 ? accumulate : 1u);
+                                accumulate = 1u;
+                                if (++c == P.ns) { c = 0; b_row += (uint32_t)g.wp * 128u; }
+                            }
+                            mma_commit(freed);
                         }
-                        accumulate = 1u;
-                        __syncwarp();
-                        if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
-                        if (++c == P.ns) { c = 0; if (++r == P.nr) r = 0; }
+                        if (ok) mma_commit(smem_u32(&pm_empty[buf]));
+                        if (++buf == (uint32_t)g.slab_bufs) { buf = 0; bph ^= 1u; }
                     }
-                    if (ok && leader) mma_commit(smem_u32(&pm_empty[buf]));
-                    __syncwarp();
-                    if (++buf == (uint32_t)g.slab_bufs) { buf = 0; bph ^= 1u; }
                 }
+                if (ok) mma_commit(smem_u32(&acc_full[acc]));
             }
-            if (ok && leader) mma_commit(smem_u32(&acc_full[acc]));
-            __syncwarp();
         }
+        __syncwarp();
     } else if (slab_warp) {
         // ---------------- slab: 32 positions x 32 channels at a time, lanes walk positions ----------------
         const int sw = warp - 2;
@@ -211,8 +213,7 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
         for (int i = 0; i < my_tiles && ok; ++i) {
             int m0, n0;
             decode(i, m0, n0);
-            for (int ci = 0; ci < n_cb && ok; ++ci) {
-                const int cb = cb0 + (ci + cb_turn < n_cb ? ci + cb_turn : ci + cb_turn - n_cb);
+            for (int cb = cb0; cb < cb1 && ok; ++cb) {
                 const int c_left = g.C - cb * 32;        // channels of the block that exist (the rest reads as zero)
                 for (int pl = 0; pl < g.n_planes && ok; ++pl) {
                     const int pa = g.planes[pl].a, pb = g.planes[pl].b;
@@ -312,11 +313,21 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
         float* y = g.y + off + (long long)m_first * PQ;
         const uint32_t from = stg + (uint32_t)lane * 4u;
         if (g.residual != nullptr) {
+            // (the activation's branch stays outside the unrolled loops: code that runs once per launch is read from the L2, and
+            // 32 inlined copies of GELU to jump over cost 5 us)
+            float t[32];
 #pragma unroll
-            for (int r = 0; r < 32; ++r, y += PQ) {
-                float o = ld_shared_f32(from + (uint32_t)(r * kPmPitch) * 4u) + w[r];
-                o = g.act == TT_ACT_GELU_ERF ? gelu_erf(o) : fminf(fmaxf(o, lo), hi);
-                if (out && r < rows) *y = o;
+            for (int r = 0; r < 32; ++r) t[r] = ld_shared_f32(from + (uint32_t)(r * kPmPitch) * 4u) + w[r];
+            if (g.act == TT_ACT_GELU_ERF) {
+#pragma unroll
+                for (int r = 0; r < 32; ++r) t[r] = gelu_erf(t[r]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 32; ++r) t[r] = fminf(fmaxf(t[r], lo), hi);
+            }
+            if (out) {
+#pragma unroll
+                for (int r = 0; r < 32; ++r, y += PQ) if (r < rows) *y = t[r];
             }
         } else if (rows >= 32) {
             if (out) {
@@ -386,7 +397,10 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                     tmem_wait_ld();
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-                    stage_block(base + (uint32_t)(b * 4 + quad) * kPmBlockBytes, v);
+                    // (as the registers lie, 512 contiguous bytes per four columns: lanes a row's pitch apart cost the reader 6000 cycles)
+                    const uint32_t at = base + (uint32_t)(b * 4 + quad) * kPmBlockBytes + (uint32_t)lane * 16u;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) st_shared_v4(at + (uint32_t)j * 512u, v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
                 }
             }
         }
@@ -396,7 +410,7 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
 #pragma unroll 1
             for (int b = own; b < blocks_n; b += own_step) {
                 const uint32_t stg = base + (uint32_t)(b * 4 + quad) * kPmBlockBytes;
-                const uint32_t at = stg + (uint32_t)(lane * kPmPitch) * 4u;
+                const uint32_t at = stg + (uint32_t)lane * 16u;
                 uint32_t r[32];
                 float v[32];
                 tmem_ld32(t_row + (uint32_t)(b * 32), r);
@@ -412,7 +426,7 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                         const uint32_t src = map_to_peer(at, (uint32_t)p);
                         float4 q[8];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) q[j] = ld_peer_v4(src + (uint32_t)j * 16u);
+                        for (int j = 0; j < 8; ++j) q[j] = ld_peer_v4(src + (uint32_t)j * 512u);
 #pragma unroll
                         for (int j = 0; j < 8; ++j) { v[4 * j] += q[j].x; v[4 * j + 1] += q[j].y; v[4 * j + 2] += q[j].z; v[4 * j + 3] += q[j].w; }
                     }

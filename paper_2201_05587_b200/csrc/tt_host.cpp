@@ -156,41 +156,59 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     if (strict && (changed & ~TT_CHG_TILE_M)) return TT_ERR_INVALID_SCHEDULE;
     const int tiles_m = (M + kHwTileM - 1) / kHwTileM;
     // How the record's tiles are laid over the SMs (148; the launch is right on any number).  Where they fill more than half of
-    // them, columns are dealt evenly over the rounds that the record's tile needs: 121 tiles of 224 columns become 141 of 192,
-    // a seventh less time for the one round (conv 3x3 128 -> 128 at 28 x 28, batch 32).  Where they fill less, CTAs share
-    // a tile's channel blocks as a cluster.
+    // them, columns are dealt evenly over the rounds that the record's tile needs: 121 tiles of 224 columns become 141 of 192.
+    // Where they fill less, CTAs share a tile's channel blocks as a cluster.  Fewer rounds, or the widest tile, take the place of
+    // the record's where they are a tenth cheaper: a tap costs what shared memory has to move in 128-byte lines -- its filters in
+    // and out, 2 * 128, its columns, about 32 for the slab -- and the filters' part is paid per tile (3x3 512 -> 512 at 7 x 7,
+    // batch 32: 31.4 us with 128 columns, 25.1 with 256).
     constexpr int kSms = 148;
-    long long tiles = (long long)tiles_m * ((N + tn - 1) / tn);
-    int split = 1;
-    if (tiles * 2 > kSms) {
-        const long long rounds = (tiles + kSms - 1) / kSms, columns = rounds * kSms / tiles_m;
-        if (columns >= 1) tn = std::min<long long>(tn, round_up64((N + columns - 1) / columns, 16));
-    } else {
-        split = (int)std::min<long long>(std::min<long long>(8, CB), kSms / tiles);
+    const auto tiles_of = [&](int n) { return (long long)tiles_m * ((N + n - 1) / n); };
+    const auto split_of = [&](int n) { return (int)std::max<long long>(1, std::min<long long>(std::min(8, CB), kSms / tiles_of(n))); };
+    const auto cost_of = [&](int n) {
+        const int k = split_of(n);
+        const long long rounds = (tiles_of(n) + kSms - 1) / kSms;
+        return rounds * ((CB + k - 1) / k) * RS * std::max(2 * n, n + 288) + 25ll * n / k;
+    };
+    const auto dealt = [&](long long rounds) {           // the columns of a tile when all of them take `rounds` rounds
+        const long long columns = rounds * kSms / tiles_m;
+        return columns >= 1 ? std::max<long long>(16, round_up64((N + columns - 1) / columns, 16)) : 0x7fffffffLL;
+    };
+    int wide = std::min(256, round_up(N, 16));
+    if (tiles_of(tn) * 2 > kSms) {
+        const long long rounds = (tiles_of(tn) + kSms - 1) / kSms;
+        tn = (int)std::min<long long>(tn, dealt(rounds));
+        wide = tn;
+        for (long long r = 1; r < rounds && r <= 4; ++r) if (dealt(r) <= 256) { wide = (int)dealt(r); break; }
     }
+    if (cost_of(wide) * 10 < cost_of(tn) * 9) tn = wide;
+    const int split = tiles_of(tn) * 2 > kSms ? 1 : split_of(tn);
     const int tiles_n = (N + tn - 1) / tn;
-    tiles = (long long)tiles_m * tiles_n;
+    const long long tiles = (long long)tiles_m * tiles_n;
     if (tiles > 0x7fffffffLL) return TT_ERR_RESOURCE;
-    // shared memory: filter stages (one tap each: `stages` reduction tiles, at most eight taps) | one or two slabs | staging
-    // blocks of the read-out (twelve warps' where all tiles are resident, a cluster's whole tile, each over the idle pipeline)
+    // shared memory: filter stages | one or two slabs | staging blocks of the read-out (twelve warps' where all tiles are
+    // resident, a cluster's whole tile, each over the idle pipeline).  A stage takes up to three taps, whose issue then hides
+    // the latency of the stage's barriers; the record's stages times its taps per reduction tile say how many are in flight.
     const int shift_min = ty.lo * tx.pitch + tx.lo, shift_max = std::max(0, ty.hi) * tx.pitch + std::max(0, tx.hi);
     const int lines = tn + shift_max - std::min(shift_min, 0);
     const long long slab = (long long)lines * 128;
     const long long epi = 4ll * kPmEpiBlockBytes;
     const long long tail = split > 1 ? (long long)((tn + 31) / 32) * 4 * kPmEpiBlockBytes : 12ll * kPmEpiBlockBytes;
-    int taps = std::min(kMaxStages, st * tps), bufs = (CB > 1 || ty.count[0] * tx.count[0] < RS || tiles > kSms) ? 2 : 1;
-    auto total = [&] { return std::max(round_up64(taps * (long long)kPmStageBytes + bufs * slab, 1024) + epi, round_up64(tail, 1024)) + 1024; };
+    const int plane_taps = *std::max_element(ty.count, ty.count + 16) * *std::max_element(tx.count, tx.count + 16);   // of the largest parity class
+    const int want = std::min(kMaxStages, st * tps);
+    int q = plane_taps == 4 ? 2 : std::min(3, plane_taps), depth = std::max(2, (want + q - 1) / q);
+    int bufs = (CB > 1 || plane_taps < RS || tiles > kSms) ? 2 : 1;
+    auto total = [&] { return std::max(round_up64((long long)depth * q * kPmTapBytes + bufs * slab, 1024) + epi, round_up64(tail, 1024)) + 1024; };
     while (total() > kDynSmemLimit) {
-        if (taps > 2) --taps;
+        if (depth > 2) --depth;
+        else if (q > 1) --q;
         else if (bufs > 1) --bufs;
-        else if (taps > 1) --taps;
+        else if (depth > 1) --depth;
         else break;
     }
-    // (a stage of the record is tps taps: fewer taps than the record's stages ask for is a shallower pipeline)
-    if ((taps + tps - 1) / tps < std::min(st, (kMaxStages + tps - 1) / tps)) { st = std::max(1, taps / tps); changed |= TT_CHG_STAGES; if (strict) return TT_ERR_RESOURCE; }
+    if (depth * q < want) { changed |= TT_CHG_STAGES; if (strict) return TT_ERR_RESOURCE; st = std::max(1, depth * q / tps); }
     L.stages = st;
     const long long smem = total();
-    const int tmem_cols = std::max(32, pow2_ceil(tiles * split > kSms ? tn + round_up(tn, 32) : round_up(tn, 32)));
+    const int tmem_cols = std::max(32, pow2_ceil(tiles > kSms ? tn + round_up(tn, 32) : round_up(tn, 32)));
     I = tt_apply_info{};
     I.legal = L; I.changed = changed;
     I.grid_x = (int)std::min<long long>(tiles, kSms / split); I.grid_y = split; I.grid_z = 1;
@@ -221,9 +239,9 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
             c.planes[c.n_planes++] = ConvPlane{(signed char)a, (signed char)b, (signed char)ty.shift[a], (signed char)tx.shift[b],
                                                (unsigned char)ty.count[a], (unsigned char)tx.count[b], (unsigned char)ty.first[a], (unsigned char)tx.first[b]};
     c.tile_n = tn; c.tiles_m = tiles_m; c.tiles_n = tiles_n; c.total_tiles = (int)tiles; c.raster = L.raster; c.split = split;
-    c.stages = taps; c.slab_bufs = bufs;
-    c.slab_off = (unsigned)(taps * kPmStageBytes); c.slab_bytes = (unsigned)slab;
-    c.epi_off = (unsigned)round_up64(taps * (long long)kPmStageBytes + bufs * slab, 1024);
+    c.stages = depth; c.taps_per_stage = q; c.slab_bufs = bufs;
+    c.slab_off = (unsigned)(depth * q * kPmTapBytes); c.slab_bytes = (unsigned)slab;
+    c.epi_off = (unsigned)round_up64((long long)depth * q * kPmTapBytes + bufs * slab, 1024);
     c.idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(tn >> 3) << 17) | ((unsigned)(kHwTileM >> 4) << 24);
     c.tmem_cols = (unsigned)tmem_cols;
     return TT_OK;

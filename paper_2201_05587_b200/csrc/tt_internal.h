@@ -88,7 +88,7 @@ struct GemmArgs {
 
 // conv2d by channel blocks and taps over a pixel-major slab (tt_conv_pm_kernel).
 constexpr int kPmMaxPlanes = 16;
-constexpr unsigned kPmStageBytes = kHwTileM * 32 * 4;       // one tap's filters: 128 x 32 channels
+constexpr unsigned kPmTapBytes = kHwTileM * 32 * 4;         // one tap's filters: 128 x 32 channels
 constexpr unsigned kPmEpiBlockBytes = 32 * 36 * 4;          // a staged 32 x 32 block of the read-out
 // The taps of one parity class of (row, column) and the sub-image they read: padded input coordinates stride * i + a,
 // stride * j + b.  Its first tap is (r0, s0) and reads position (row + f0, column + e0) of the sub-image; the next ones of
@@ -104,7 +104,7 @@ struct ConvPmArgs {
     unsigned magic_wp, magic_image;             // floor(2^32 / divisor)
     int shift_min, slab_lines;                  // the slab of a tile: positions n0 + shift_min .. + slab_lines - 1
     int n_planes; ConvPlane planes[kPmMaxPlanes];
-    int tile_n, tiles_m, tiles_n, total_tiles, raster, split, stages, slab_bufs;
+    int tile_n, tiles_m, tiles_n, total_tiles, raster, split, stages, taps_per_stage, slab_bufs;
     unsigned slab_off, slab_bytes, epi_off, idesc, tmem_cols;
 };
 
