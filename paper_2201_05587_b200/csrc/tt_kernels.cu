@@ -1259,7 +1259,10 @@ __device__ __forceinline__ void bulk_stores_commit() { asm volatile("cp.async.bu
 template <int N>
 __device__ __forceinline__ void bulk_stores_pending() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 
-template <int CG>
+// Instantiated for what a plan uses, so that a launch carries only the code it runs (a single-wave launch meets it cold: 3-6 %
+// on every record of this form, dense 2268 x 2256 -> 3944 76 -> 71 us).  MN: an operand is MN-major (otherwise the descriptors
+// step by constants).  OUT: outputs leave by TMA stores.
+template <int CG, bool MN, bool OUT>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                   const __grid_constant__ CUtensorMap tmap_y, const __grid_constant__ CUtensorMap tmap_r, const GemmArgs g) {
@@ -1271,7 +1274,7 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     __shared__ uint64_t res_full[8 * kMaxEpiBufs];   // per read-out warp and ring buffer: a residual block has landed
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ __align__(16) float s_bias[8][32];   // per read-out warp: the bias of its current block
+    __shared__ __align__(16) float s_bias[4][256];  // per tile under way: the bias of its columns
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     volatile int* abortp = &abort_flag;
@@ -1284,14 +1287,14 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
 
     const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t stage_bytes = g.a_stage_bytes + g.b_stage_bytes;
-    const bool a_mn = g.a_mn != 0, b_mn = g.b_mn != 0;
+    const bool a_mn = MN && g.a_mn != 0, b_mn = MN && g.b_mn != 0;
     const int b_rows = g.b_rows_cta;
     const int epi_warps = g.epi_warps;
 
     if (threadIdx.x == 32) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_b) : "memory");
-        if (g.epi_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_y) : "memory");
+        if (OUT) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_y) : "memory");
         if (g.res_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_r) : "memory");
     }
     if (threadIdx.x == 0) {
@@ -1427,12 +1430,13 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                         uint32_t accumulate = kt > 0 ? 1u : 0u;
 #pragma unroll 1
                         for (int at = 0; at < g.n_atoms; ++at, a_lo += da.atom, b_lo += db.atom) {
-                            if (k8n == 4 && !a_mn && !b_mn) {
+                            if (!MN && k8n == 4) {
 #pragma unroll
                                 for (uint32_t k8 = 0; k8 < 4; ++k8) {
-                                    mma_tf32_cg<CG>(d_tmem, ((uint64_t)da.hi << 32) | (uint64_t)(a_lo + 2u * k8), ((uint64_t)db.hi << 32) | (uint64_t)(b_lo + 2u * k8), g.idesc, accumulate);
-                                    accumulate = 1u;
+                                    mma_tf32_cg<CG>(d_tmem, ((uint64_t)da.hi << 32) | (uint64_t)(a_lo + 2u * k8), ((uint64_t)da.hi << 32) | (uint64_t)(b_lo + 2u * k8), g.idesc,
+                                                    k8 == 0 ? accumulate : 1u);
                                 }
+                                accumulate = 1u;
                             } else {
                                 uint32_t a = a_lo, b = b_lo;
 #pragma unroll 4
@@ -1463,7 +1467,8 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         e.gelu = g.act == TT_ACT_GELU_ERF;
         e.vec = (g.vec_store & 1) != 0;
         const bool transposed = g.y_ns == 1 && g.y_ms != 1;
-        const bool tma_out = g.epi_tma != 0, res_in = g.res_tma != 0;
+        constexpr bool tma_out = OUT;
+        const bool res_in = g.res_tma != 0;
         const uint32_t ring = tiles_base + g.epi_off + (uint32_t)ew * g.epi_warp_bytes;
         const int bufs = g.epi_bufs;
         const int per_tile = c_first < g.tile_n ? (g.tile_n - c_first + c_step - 1) / c_step : 0;    // blocks of a tile
@@ -1494,8 +1499,14 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             decode(i, m0, n0, bz);
             const uint32_t acc = (uint32_t)i & 1u, aph = ((uint32_t)i >> 1) & 1u;
             const int m_first = m0 + quad * 32, m = m_first + lane;
-            // bias of this warp's first block, fetched while the tile is still being accumulated; later ones a block ahead
-            float bias_col = (g.bias_mode == 2 && c_first < g.tile_n && n0 + c_first + lane < g.N) ? __ldg(g.bias + n0 + c_first + lane) : 0.f;
+            // the bias of this warp's blocks, staged while the tile is still being accumulated.  Warps that share columns write
+            // the same values; four buffers, because a warp can be up to three tiles ahead of the slowest (whose arrival on an
+            // accumulator the third needs)
+            float* tile_bias = s_bias[i & 3];
+            if (g.bias_mode == 2) {
+                for (int c = c_first; c < g.tile_n; c += c_step) tile_bias[c + lane] = (n0 + c + lane < g.N) ? __ldg(g.bias + n0 + c + lane) : 0.f;
+                __syncwarp();
+            }
             const float bias_row = (g.bias_mode == 1 && m < g.M) ? __ldg(g.bias + m) : 0.f;
             // (each read-out warp walks on its own: a barrier over the eight of them per tile cost batch_matmul NT
             // 3072 x 128 x 128 x 64 a tenth of its time, 73 us against 65 us)
@@ -1547,14 +1558,9 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] += bias_row;
                 } else if (g.bias_mode == 2) {
-                    __syncwarp();                        // (the previous block's values have been read)
-                    s_bias[ew][lane] = bias_col;
-                    const int nc = c0 + c_step;
-                    bias_col = (nc < g.tile_n && n0 + nc + lane < g.N) ? __ldg(g.bias + n0 + nc + lane) : 0.f;
-                    __syncwarp();
 #pragma unroll
                     for (int j = 0; j < 32; j += 4) {
-                        const float4 b = *reinterpret_cast<const float4*>(&s_bias[ew][j]);
+                        const float4 b = *reinterpret_cast<const float4*>(tile_bias + c0 + j);
                         v[j] += b.x; v[j + 1] += b.y; v[j + 2] += b.z; v[j + 3] += b.w;
                     }
                 }
@@ -2267,14 +2273,20 @@ cudaError_t launch_gemm(const tt_apply_info& I, const GemmArgs& g, const void* t
     return cudaLaunchKernelEx(&cfg, kern, ta, tb, tx, g);
 }
 
+typedef void (*PsKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
+static const PsKernel kPs[3][2] = {{tt_gemm_ps_kernel<1, false, false>, tt_gemm_ps_kernel<1, false, true>},
+                                   {tt_gemm_ps_kernel<1, true, false>, tt_gemm_ps_kernel<1, true, true>},
+                                   {tt_gemm_ps_kernel<2, false, false>, tt_gemm_ps_kernel<2, false, true>}};
+
 // The persistent form: one CTA (or one pair of CTAs, as a cluster of two) per SM.
 cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const TmapPair& maps, cudaStream_t st) {
     static int attr_set_for = -1, sm_count = 148;
     int dev = 0;
     cudaGetDevice(&dev);
     if (attr_set_for != dev) {
-        cudaError_t e = cudaFuncSetAttribute(tt_gemm_ps_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tt_gemm_ps_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+        cudaError_t e = cudaSuccess;
+        for (const PsKernel kern : {kPs[0][0], kPs[0][1], kPs[1][0], kPs[1][1], kPs[2][0], kPs[2][1]})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
         if (e != cudaSuccess) return e;
         cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
         attr_set_for = dev;
@@ -2300,8 +2312,7 @@ cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const Tmap
     cfg.attrs = attr; cfg.numAttrs = (unsigned)n_attr;
     memcpy(&ty, maps.y, sizeof ty);
     memcpy(&tr, maps.r, sizeof tr);
-    if (cg == 2) return cudaLaunchKernelEx(&cfg, tt_gemm_ps_kernel<2>, ta, tb, ty, tr, g);
-    return cudaLaunchKernelEx(&cfg, tt_gemm_ps_kernel<1>, ta, tb, ty, tr, g);
+    return cudaLaunchKernelEx(&cfg, kPs[cg == 2 ? 2 : (g.a_mn || g.b_mn ? 1 : 0)][g.epi_tma ? 1 : 0], ta, tb, ty, tr, g);
 }
 
 // Can a cluster of a plan's CTAs be resident at all?
