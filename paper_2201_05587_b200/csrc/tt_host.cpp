@@ -450,10 +450,10 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
         g.tx_bytes = a_stage + b_stage;
         g.vec_store = (g.y_ns == 1 && g.y_ms % 4 == 0 && g.y_bs % 4 == 0) ? 1 : 0;
         // TMA read-out: 16-byte rows, whole 32-column blocks (a narrower last block would write its neighbour's columns), and
-        // two ring blocks per warp, so that one fills while the other is sent (with one the last tile's read-out, which nothing
-        // hides, took twice as long: dense 1854 x 680 -> 1248 14.3 -> 16.0 us)
+        // two ring blocks per warp for the last tile, whose read-out nothing hides, so that one fills while the other is sent
+        g.epi_late = ew == 4 && !res && depth * stage >= 8ll * kLateRingBytes;
         g.y_tma_batched = y_bs != 0;
-        g.epi_tma = g.vec_store && tn % 32 == 0 && g.y_ms != 1 && eb >= 2;
+        g.epi_tma = g.vec_store && tn % 32 == 0 && g.y_ms != 1 && (eb >= 2 || g.epi_late);
         g.res_tma = res && eb >= 2 && (g.epi_tma || (g.y_ms == 1 && g.y_ns % 4 == 0 && g.y_bs % 4 == 0));
         return TT_OK;
     }

@@ -79,6 +79,7 @@ struct GemmArgs {
     int b_rows_cta;                             // rows of operand B one CTA loads: tile_n / cta_group
     unsigned epi_off;                           // read-out staging area: byte offset from the aligned tile base
     int epi_warps;                              // read-out warps: 4 or 8
+    int epi_late;                               // 4 of them: the other four help with the last tile, over the idle pipeline
     int epi_bufs;                               // 32 x 32 blocks in each read-out warp's ring
     unsigned epi_warp_bytes;                    // ... and its bytes
     int epi_tma;                                // outputs leave by TMA stores (contiguous along the tile's columns)
@@ -148,6 +149,7 @@ struct Plan {
 };
 
 constexpr int kMaxEpiBufs = 3;
+constexpr unsigned kLateRingBytes = 8192;   // two 32 x 32 blocks per warp
 
 // The tensor maps of a launch, cached by the pointers they were made for.
 struct TmapPair {

@@ -1271,6 +1271,7 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     __shared__ uint64_t empty_bar[kMaxStages];    // every multiply-accumulate that reads the stage has completed
     __shared__ uint64_t acc_full[2];              // an accumulator holds a finished tile
     __shared__ uint64_t acc_empty[2];             // the read-out warps (of both CTAs) have drained it
+    __shared__ uint64_t last_full;                // the CTA's last tile is complete, and with it the pipeline idle
     __shared__ uint64_t res_full[8 * kMaxEpiBufs];   // per read-out warp and ring buffer: a residual block has landed
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
@@ -1306,6 +1307,7 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             mbar_init(smem_u32(&acc_full[a]), 1u);
             mbar_init(smem_u32(&acc_empty[a]), (uint32_t)(epi_warps * CG));
         }
+        mbar_init(smem_u32(&last_full), 1u);
         if (g.res_tma) for (int b = 0; b < 8 * kMaxEpiBufs; ++b) mbar_init(smem_u32(&res_full[b]), 1u);
         abort_flag = 0;
         fence_mbar_init();
@@ -1452,14 +1454,19 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                     if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
                 }
                 if (ok && leader) mma_commit_cg<CG>(smem_u32(&acc_full[acc]));   // the tile's accumulator is complete
+                if (ok && leader && i + 1 == my_tiles) mma_commit_cg<CG>(smem_u32(&last_full));
                 __syncwarp();
             }
         }
-    } else if (warp >= 10 - epi_warps) {
+    } else if (warp >= 10 - epi_warps || g.epi_late) {
         // ---------------- read-out: tensor memory -> bias, residual, activation -> global memory ----------------
-        const int ew = warp - (10 - epi_warps);
+        // A plan whose stages leave room for four read-out warps only gets the other four for the last tile, whose read-out
+        // nothing hides: the pipeline's buffers are idle by then and take the staging blocks of all eight (dense 1854 x 680 ->
+        // 1248 by CTA pairs, one tile each: 15.6 -> 13.8 us).
+        const bool helper = warp < 10 - epi_warps;
+        const int ew = helper ? 0 : warp - (10 - epi_warps);
         const int quad = warp & 3;                       // tensor-memory lane quadrant this warp may read
-        const int c_first = (ew >> 2) * 32, c_step = epi_warps * 8;      // the 32-column blocks of a tile that this warp takes
+        int c_first = (ew >> 2) * 32, c_step = epi_warps * 8;            // the 32-column blocks of a tile that this warp takes
         EpiArgs e;
         e.y_ms = g.y_ms; e.y_ns = g.y_ns; e.M = g.M;
         e.lo = g.act == TT_ACT_NONE || g.act == TT_ACT_GELU_ERF ? -INFINITY : 0.f;
@@ -1469,8 +1476,8 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         const bool transposed = g.y_ns == 1 && g.y_ms != 1;
         constexpr bool tma_out = OUT;
         const bool res_in = g.res_tma != 0;
-        const uint32_t ring = tiles_base + g.epi_off + (uint32_t)ew * g.epi_warp_bytes;
-        const int bufs = g.epi_bufs;
+        uint32_t ring = tiles_base + g.epi_off + (uint32_t)ew * g.epi_warp_bytes;
+        int bufs = g.epi_bufs;
         const int per_tile = c_first < g.tile_n ? (g.tile_n - c_first + c_step - 1) / c_step : 0;    // blocks of a tile
         bool ok = true;
         // residual blocks are requested one ahead of their use: cursor of the next request
@@ -1494,30 +1501,35 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         }
         int buf = 0;                                     // ring position of the current block
         uint32_t rph = 0;                                // phase of the residual barriers at `buf`
-        for (int i = 0; i < my_tiles; ++i) {
+        for (int i = helper ? max(0, my_tiles - 1) : 0; i < my_tiles; ++i) {
             int m0, n0, bz;
             decode(i, m0, n0, bz);
             const uint32_t acc = (uint32_t)i & 1u, aph = ((uint32_t)i >> 1) & 1u;
+            const bool all_eight = g.epi_late && i + 1 == my_tiles;
+            if (all_eight) { c_first = ((warp - 2) >> 2) * 32; c_step = 64; ring = tiles_base + (uint32_t)(warp - 2) * kLateRingBytes; bufs = 2; buf = 0; }
             const int m_first = m0 + quad * 32, m = m_first + lane;
             // the bias of this warp's blocks, staged while the tile is still being accumulated.  Warps that share columns write
             // the same values; four buffers, because a warp can be up to three tiles ahead of the slowest (whose arrival on an
             // accumulator the third needs)
             float* tile_bias = s_bias[i & 3];
-            if (g.bias_mode == 2) {
+            auto stage_bias = [&]() {
                 for (int c = c_first; c < g.tile_n; c += c_step) tile_bias[c + lane] = (n0 + c + lane < g.N) ? __ldg(g.bias + n0 + c + lane) : 0.f;
                 __syncwarp();
-            }
+            };
+            if (g.bias_mode == 2 && !helper) stage_bias();
             const float bias_row = (g.bias_mode == 1 && m < g.M) ? __ldg(g.bias + m) : 0.f;
             // (each read-out warp walks on its own: a barrier over the eight of them per tile cost batch_matmul NT
             // 3072 x 128 x 128 x 64 a tenth of its time, 73 us against 65 us)
-            ok = ok && mbar_wait(smem_u32(&acc_full[acc]), aph, abortp, g.status, 4u, g.wait_ns);
+            // (a helper has not followed the accumulators' phases: the last tile has a barrier of its own)
+            ok = ok && mbar_wait(helper ? smem_u32(&last_full) : smem_u32(&acc_full[acc]), helper ? 0u : aph, abortp, g.status, 4u, g.wait_ns);
             if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
             tc_fence_after();
+            if (g.bias_mode == 2 && helper) stage_bias();       // (not earlier: its buffer may have been an older tile's)
             e.ybase = g.y + (long long)bz * g.y_bs;
             e.rbase = g.residual ? g.residual + (long long)bz * g.y_bs : nullptr;
             const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * (uint32_t)g.tile_n;
             uint32_t r[32];
-            if (per_tile > 0) tmem_ld32(t_row + (uint32_t)c_first, r);
+            if (c_first < g.tile_n) tmem_ld32(t_row + (uint32_t)c_first, r);
             else if (lane == 0) {
                 if (CG == 2) mbar_arrive_remote(smem_u32(&acc_empty[acc]), 0u);
                 else mbar_arrive(smem_u32(&acc_empty[acc]));
