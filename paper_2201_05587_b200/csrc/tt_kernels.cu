@@ -391,7 +391,7 @@ __device__ __forceinline__ void epilogue_block(float (&v)[32], const EpiArgs& e,
 // ------------------------------------------------------------------------------------------------------------
 // GEMM_TC kernel.  grid = (tiles_m * tiles_n, split_k, batch), block = 320 threads:
 // warp 0 TMA producer, warp 1 MMA issuer + tensor-memory owner, warps 2-9 gather producers, then epilogue.
-// Built for each way its operands reach shared memory (GemmForm), so that a kernel carries only the code it runs: the
+// Built for each way its operands reach shared memory (GemmForm), with and without the cluster reduction, so that a kernel carries only the code it runs: the
 // launches of a batch-1 model pass are a few microseconds long and meet a cold instruction cache.
 // Two builds of each: MIN_CTAS = 1 (all registers), and MIN_CTAS = 2 (registers capped so that two CTAs share an SM when a
 // record's shared memory and tensor memory allow it: one CTA's set-up and read-out then overlap the other's main loop).
@@ -413,7 +413,7 @@ enum GemmForm {
     kFormGather = 3     // an operand gathered from global memory (the other one any way but by expansion)
 };
 
-template <int MIN_CTAS, int FORM>
+template <int MIN_CTAS, int FORM, bool CLUSTER>
 __global__ void __launch_bounds__(kGemmThreads, MIN_CTAS)
 tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                   const __grid_constant__ CUtensorMap tmap_x, const GemmArgs g) {
@@ -492,7 +492,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             mbar_init(smem_u32(&slab_full[b]), 1u);
             mbar_init(smem_u32(&slab_empty[b]), (uint32_t)kGatherWarps);
         }
-        if (g.cluster) {
+        if (CLUSTER) {
             // the bands this CTA finishes arrive from the other splits: rows x (tile_n + 4) or columns x 128 floats each
             mbar_init(smem_u32(&red_bar), 1u);
             mbar_expect_tx(smem_u32(&red_bar), (uint32_t)(g.split_k - 1) * red_band_bytes(g, split));
@@ -513,7 +513,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     // A CTA's reduction area and its barrier may be used by a peer only once they exist: every thread announces
     // itself here (the barrier above is initialised) and checks, just before the first copy to a peer could be issued,
     // that all peers have done the same.
-    if (g.cluster) cluster_arrive();
+    if (CLUSTER) cluster_arrive();
     // Programmatic dependent launch: everything above (barriers, tensor memory) touched no global memory and may
     // run while the previous kernel of the stream is still draining; from here on its results are needed.  The
     // kernel that follows this one was allowed to start its own set-up at this kernel's entry.  (Without the launch
@@ -635,7 +635,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             }
             __syncwarp();
         }
-        if (g.cluster) cluster_wait();
+        if (CLUSTER) cluster_wait();
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
         {
@@ -704,7 +704,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                         }
                         a_lo += a_next_atom; b_lo += b_next_atom;
                     }
-                    mma_commit(empty_addr);              // stage reusable once these MMAs have read it
+                    if (it + g.stages < iters) mma_commit(empty_addr);   // stage reusable once these MMAs have read it (if anything follows)
                 }
                 __syncwarp();
                 a_stage += stage_step; b_stage += stage_step; full_addr += 8u; empty_addr += 8u;
@@ -713,7 +713,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             if (ok && leader) mma_commit(smem_u32(&accum_bar));    // accumulator complete
             __syncwarp();
         }
-        if (g.cluster) cluster_wait();
+        if (CLUSTER) cluster_wait();
     } else {
         // ---------------- gather producers, then epilogue ----------------
         const int gw = warp - 2;
@@ -722,7 +722,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         const int m = m0 + quad * 32 + lane;
         // bias is fetched now so that its latency hides behind the main loop
         if (g.bias_mode == 2 && gt < g.tile_n) s_bias[gt] = (n0 + gt < g.N) ? __ldg(g.bias + n0 + gt) : 0.f;
-        if (g.bias_mode == 1 && g.cluster && gt < kHwTileM) s_bias[gt] = (m0 + gt < g.M) ? __ldg(g.bias + m0 + gt) : 0.f;   // for the cluster reduction
+        if (CLUSTER && g.bias_mode == 1 && gt < kHwTileM) s_bias[gt] = (m0 + gt < g.M) ? __ldg(g.bias + m0 + gt) : 0.f;   // for the cluster reduction
         const float bias_row = (g.bias_mode == 1 && m < g.M) ? __ldg(g.bias + m) : 0.f;
         if (im2col) {
             // ---- conv2d: slab staging + expansion; all eight warps work on the same stage ----
@@ -880,7 +880,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             int sk, whole, per; uint32_t line, slot, red; bool along_cols, gelu, clamp, vec_ok; int bias_mode;
             float lo, hi; float* ybase; const float* rbase; long long y_ms, y_ns;
         } cr;
-        if (g.cluster) {
+        if (CLUSTER) {
             cr.sk = g.split_k;
             cr.along_cols = g.y_ns == 1;                                 // bands of rows
             cr.whole = cr.along_cols ? kHwTileM : g.tile_n;
@@ -915,19 +915,19 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             "bar.red.and.pred p, 1, %2, q;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(all_acc) : "r"((uint32_t)have_acc), "n"(kGatherThreads) : "memory");
-        if (g.cluster) cluster_wait();                   // every peer is set up: its reduction area and barrier may be used
+        if (CLUSTER) cluster_wait();                   // every peer is set up: its reduction area and barrier may be used
         if (all_acc) {
             tc_fence_after();
             const int half = gw >> 2;
             const bool m_ok = m < g.M;
             const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16);
-            const bool split_mode = g.split_k > 1 && g.cluster == 0;   // splits beyond a cluster go through the workspace
+            const bool split_mode = !CLUSTER && g.split_k > 1;   // splits beyond a cluster go through the workspace
             // a split with fewer reduction steps than accumulators leaves the last ones unwritten
             const int n_acc = min(g.n_acc, iters * (g.tile_k >> 3));
             // split-K workspace [split][batch][N][M]: a column of the tile is contiguous across lanes
             const long long per_split = (long long)g.batch * g.M * (long long)g.N;
             float* pcol = g.partial + (long long)bz * g.M * (long long)g.N + m;
-            if (g.cluster) {
+            if (CLUSTER) {
                 // split-K over a cluster, step 1: this split's partial tile goes to the pipeline buffers (idle: every
                 // multiply-accumulate has completed) in the layout of the reduction area, a band being one run of bytes
                 const int row = quad * 32 + lane;
@@ -997,7 +997,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 }
                 asm volatile("bar.sync 1, %0;" ::"n"(kGatherThreads) : "memory");
             }
-            const bool finish = g.cluster == 0 && (!split_mode || (*(volatile int*)&last_split_flag != 0));
+            const bool finish = !CLUSTER && (!split_mode || (*(volatile int*)&last_split_flag != 0));
             if (finish) {
                 if (split_mode) __threadfence();
                 EpiArgs e;
@@ -1077,7 +1077,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 }
             }
         }
-        if (g.cluster) {
+        if (CLUSTER) {
             // step 2: once every read-out warp has staged its part, one thread per peer sends that peer's band
             asm volatile("bar.sync 1, %0;" ::"n"(kGatherThreads) : "memory");
             if (all_acc && lane == 0 && gw < cr.sk && gw != split) {
@@ -1170,7 +1170,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             }
         }
     }
-    if (g.cluster) {
+    if (CLUSTER) {
         // Every thread of every CTA of the cluster takes part in both rounds of the cluster barrier, also after a
         // tripped wait: the second round completes when no CTA sends any more, so none leaves while a copy into its
         // shared memory could still be under way.
@@ -2228,9 +2228,9 @@ __global__ void tt_floor_kernel() {
 static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <= 112 * 1024 && tmem_cols <= 256; }
 
 typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
-static const GemmKernel kGemmKernels[2][4] = {
-    {tt_gemm_tc_kernel<1, kFormTma>, tt_gemm_tc_kernel<1, kFormMn>, tt_gemm_tc_kernel<1, kFormIm2col>, tt_gemm_tc_kernel<1, kFormGather>},
-    {tt_gemm_tc_kernel<2, kFormTma>, tt_gemm_tc_kernel<2, kFormMn>, tt_gemm_tc_kernel<2, kFormIm2col>, tt_gemm_tc_kernel<2, kFormGather>}};
+#define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>}
+static const GemmKernel kGemmKernels[2][2][4] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
+#undef TT_GEMM_FORMS
 
 static int gemm_form(const GemmArgs& g) {
     if (g.a_mode == OPM_IM2COL || g.b_mode == OPM_IM2COL) return kFormIm2col;
@@ -2242,16 +2242,17 @@ static int gemm_form(const GemmArgs& g) {
 // Which instantiation a plan runs; its shared-memory limit is raised once per device.  Which build (two CTAs per SM) is the
 // record's choice (ctas_per_sm), resolved by the legaliser.
 static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel* out) {
-    static std::atomic<uint64_t> raised[2][4];           // a bit per device
+    static std::atomic<uint64_t> raised[2][2][4];           // a bit per device
     const int two = g.two_per_sm && gemm_two_per_sm(smem_bytes, g.tmem_cols), form = gemm_form(g);
     int dev = 0;
     cudaGetDevice(&dev);
     const uint64_t bit = 1ull << (dev & 63);
-    *out = kGemmKernels[two][form];
-    if (!(raised[two][form].load(std::memory_order_relaxed) & bit)) {
+    const int cl = g.cluster > 0;
+    *out = kGemmKernels[two][cl][form];
+    if (!(raised[two][cl][form].load(std::memory_order_relaxed) & bit)) {
         cudaError_t e = cudaFuncSetAttribute(*out, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
         if (e != cudaSuccess) return e;
-        raised[two][form].fetch_or(bit, std::memory_order_relaxed);
+        raised[two][cl][form].fetch_or(bit, std::memory_order_relaxed);
     }
     return cudaSuccess;
 }
