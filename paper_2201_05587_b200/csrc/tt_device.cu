@@ -11,7 +11,7 @@
 
 namespace tt {
 
-cudaError_t launch_gemm(const tt_apply_info& I, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
+cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
                         cudaStream_t st);
 cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st);
 cudaError_t launch_dw_tma(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st);
@@ -192,7 +192,7 @@ tt_status bind_device(tt_workload* w) {
     if (w->family == TT_FAMILY_GEMM_TC && w->plan.g.cluster) {
         // a cluster whose CTAs cannot be resident together can never launch: an invalid pair, not a device error
         int fits = 0;
-        if (gemm_cluster_fits(w->plan.g, w->plan.info.smem_bytes, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+        if (gemm_cluster_fits(w->plan.g, w->plan.run_smem, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
         if (!fits) return TT_ERR_RESOURCE;
     }
     if (w->family == TT_FAMILY_GEMM_TC && w->plan.repack && w->plan.pm.split > 1) {
@@ -356,7 +356,7 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
         const TmapPair* maps = nullptr;
         const tt_status s = tensor_maps_for(w, g, a_ptr, b_ptr, &maps);
         if (s != TT_OK) return s;
-        e = g.persistent ? launch_gemm_ps(p.info, g, *maps, st) : launch_gemm(p.info, g, maps->a, maps->b, maps->x, st);
+        e = g.persistent ? launch_gemm_ps(p.info, g, *maps, st) : launch_gemm(p.info, p.run_smem, g, maps->a, maps->b, maps->x, st);
     } else if (w->family == TT_FAMILY_DW_SIMT) {
         DwArgs d = p.dw;
         d.x = static_cast<const float*>(t->x); d.w = static_cast<const float*>(t->w);
@@ -1012,7 +1012,7 @@ extern "C" tt_status tt_dense_static_scratch(const void* x, const void* w, const
     if (plan.g.cluster) {
         // as in tt_schedule_apply: a split-K cluster whose CTAs cannot be resident together is an invalid pair
         int fits = 0;
-        if (gemm_cluster_fits(plan.g, plan.info.smem_bytes, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+        if (gemm_cluster_fits(plan.g, plan.run_smem, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
         if (!fits) return TT_ERR_RESOURCE;
     }
     unsigned char* base = nullptr;
@@ -1044,7 +1044,7 @@ extern "C" tt_status tt_dense_static_scratch(const void* x, const void* w, const
     if (s == TT_OK && g.b_mode == OPM_TMA)
         s = encode_operand(maps.b, g.b, g.K, g.N, g.batch, g.b_rs, g.b_bs, g.b_tma_batched != 0, g.atom_k, g.tile_n);
     if (s != TT_OK) return s;
-    if (launch_gemm(plan.info, g, maps.a, maps.b, maps.x, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+    if (launch_gemm(plan.info, plan.run_smem, g, maps.a, maps.b, maps.x, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     if (cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     unsigned v = 0;
     if (cudaMemcpy(&v, base, 4, cudaMemcpyDeviceToHost) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }

@@ -575,18 +575,28 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
     I.launches = 1;
     if (smem > kDynSmemLimit) return TT_ERR_RESOURCE;
 
+    // The record's pipeline depth is what it needs at least: with one CTA per SM the shared memory that is left serves no one
+    // else, so the ring takes as many stages as fit, up to a CTA's whole reduction.  A batch-1 layer then requests all of its
+    // weights at once instead of a refill of two stages per trip to memory (the 84 kernels of the 12-layer encoder at batch 1
+    // and 128 tokens: 528 us with the record's depth, 501 with this one).
+    int depth = st;
+    if (L.ctas_per_sm != 2)
+        while (depth < std::min(kMaxStages, per_split) &&
+               std::max<long long>((depth + 1ll) * (a_stage + b_stage) * (x3 ? 2 : 1), min_pipe) + smem - pipe <= kDynSmemLimit) ++depth;
+    const long long run_pipe = std::max<long long>((long long)depth * (a_stage + b_stage) * (x3 ? 2 : 1), min_pipe);
+    plan->run_smem = (int)(smem - pipe + run_pipe);
     GemmArgs& g = plan->g;
     g = GemmArgs{};
     g.M = M; g.N = N; g.K = K; g.batch = B;
-    g.tile_n = tn; g.tile_k = tk; g.stages = st;
+    g.tile_n = tn; g.tile_k = tk; g.stages = depth;
     g.k_tiles = k_tiles; g.k_tiles_per_split = per_split; g.split_k = sk;
     g.tiles_m = tiles_m; g.tiles_n = tiles_n; g.raster = L.raster;
     g.atom_k = atom_k; g.n_atoms = n_atoms; g.row_bytes = row_bytes;
     g.swz_mask = row_bytes == 128 ? 7 : (row_bytes == 64 ? 3 : 1);
     g.a_stage_bytes = a_stage; g.b_stage_bytes = b_stage;
-    g.ktab_off = (unsigned)pipe;
-    g.slab_off = (unsigned)(pipe + ktab);
-    g.red_off = (unsigned)(pipe + ktab + (long long)sl_nbuf * sl_buf_bytes);
+    g.ktab_off = (unsigned)run_pipe;
+    g.slab_off = (unsigned)(run_pipe + ktab);
+    g.red_off = (unsigned)(run_pipe + ktab + (long long)sl_nbuf * sl_buf_bytes);
     g.slab_buf_bytes = (unsigned)sl_buf_bytes; g.slab_nbuf = sl_nbuf; g.slab_tiles = sl_tiles;
     g.slab_wp = sl_wp; g.slab_gap = sl_gap; g.slab_chpitch = sl_chpitch; g.slab_in_rows = sl_in_rows;
     g.slab_rstep = sl_rstep;

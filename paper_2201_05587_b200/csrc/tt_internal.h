@@ -142,6 +142,7 @@ struct Plan {
     int a_tensor = 0, b_tensor = 1;   // which caller tensor feeds operand A / B: 0 = x, 1 = w
     GemmArgs g{};
     long long partial_bytes = 0;      // counters start here inside the workspace
+    int run_smem = 0;                 // one-tile GEMM: shared memory of a launch (the ring may be deeper than the record's)
     bool repack = false;              // tap-major convolution: pm applies, filters are re-packed into the workspace
     ConvPmArgs pm{};
     DwArgs dw{};

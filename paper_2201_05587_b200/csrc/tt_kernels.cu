@@ -410,6 +410,7 @@ enum GemmForm {
     kFormTma = 0,       // both operands K-major by TMA
     kFormMn = 1,        // both by TMA, one of them (or both) MN-major
     kFormIm2col = 2,    // one operand expanded from a slab of input rows, the other by TMA or gathered
+    kFormX3 = 4,        // both K-major by TMA, error-compensated products
     kFormGather = 3     // an operand gathered from global memory (the other one any way but by expansion)
 };
 
@@ -450,16 +451,16 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     // (error-compensated products: a stage holds the two operand tiles and, behind them, their remainders)
     const uint32_t lo_off = g.a_stage_bytes + g.b_stage_bytes;
-    const uint32_t stage_bytes = FORM == kFormTma && g.x3 ? 2u * lo_off : lo_off;
+    const uint32_t stage_bytes = FORM == kFormX3 ? 2u * lo_off : lo_off;
     // what the instantiation is made for (GemmForm); within it only the modes that its form leaves open are looked at
     constexpr bool im2col = FORM == kFormIm2col;
     constexpr bool may_mn = FORM == kFormMn || FORM == kFormGather;
     const bool a_mn = may_mn && g.a_mode == OPM_TMA_MN, b_mn = may_mn && g.b_mode == OPM_TMA_MN;
-    const bool a_tma = FORM == kFormTma || FORM == kFormMn || g.a_mode == OPM_TMA || a_mn;
-    const bool b_tma = FORM == kFormTma || FORM == kFormMn || g.b_mode == OPM_TMA || b_mn;
+    const bool a_tma = FORM == kFormTma || FORM == kFormX3 || FORM == kFormMn || g.a_mode == OPM_TMA || a_mn;
+    const bool b_tma = FORM == kFormTma || FORM == kFormX3 || FORM == kFormMn || g.b_mode == OPM_TMA || b_mn;
     const bool any_tma = a_tma || b_tma, any_gather = !a_tma || !b_tma;
     const bool slab_tma = im2col && g.slab_tma != 0;
-    const bool x3 = FORM == kFormTma && g.x3 != 0;       // error-compensated products
+    constexpr bool x3 = FORM == kFormX3;                 // error-compensated products
     // im2col geometry of this CTA: first output row of its pixels, the image row its slab starts at, slab chunks
     int ic_p_first = 0, ic_ih_lo = 0, ic_chunks = 0;
     if (im2col) {
@@ -2228,11 +2229,12 @@ __global__ void tt_floor_kernel() {
 static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <= 112 * 1024 && tmem_cols <= 256; }
 
 typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
-#define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>}
-static const GemmKernel kGemmKernels[2][2][4] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
+#define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>}
+static const GemmKernel kGemmKernels[2][2][5] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
 #undef TT_GEMM_FORMS
 
 static int gemm_form(const GemmArgs& g) {
+    if (g.x3) return kFormX3;
     if (g.a_mode == OPM_IM2COL || g.b_mode == OPM_IM2COL) return kFormIm2col;
     const bool a = g.a_mode == OPM_TMA || g.a_mode == OPM_TMA_MN, b = g.b_mode == OPM_TMA || g.b_mode == OPM_TMA_MN;
     if (!a || !b) return kFormGather;
@@ -2242,7 +2244,7 @@ static int gemm_form(const GemmArgs& g) {
 // Which instantiation a plan runs; its shared-memory limit is raised once per device.  Which build (two CTAs per SM) is the
 // record's choice (ctas_per_sm), resolved by the legaliser.
 static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel* out) {
-    static std::atomic<uint64_t> raised[2][2][4];           // a bit per device
+    static std::atomic<uint64_t> raised[2][2][5];           // a bit per device
     const int two = g.two_per_sm && gemm_two_per_sm(smem_bytes, g.tmem_cols), form = gemm_form(g);
     int dev = 0;
     cudaGetDevice(&dev);
@@ -2257,10 +2259,10 @@ static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel
     return cudaSuccess;
 }
 
-cudaError_t launch_gemm(const tt_apply_info& I, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
+cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
                         cudaStream_t st) {
     GemmKernel kern;
-    const cudaError_t e = gemm_kernel_for(g, I.smem_bytes, &kern);
+    const cudaError_t e = gemm_kernel_for(g, smem_bytes, &kern);
     if (e != cudaSuccess) return e;
     CUtensorMap ta, tb, tx;
     memcpy(&ta, tmap_a, sizeof ta);
@@ -2268,7 +2270,7 @@ cudaError_t launch_gemm(const tt_apply_info& I, const GemmArgs& g, const void* t
     memcpy(&tx, tmap_x, sizeof tx);
     dim3 grid(I.grid_x, I.grid_y, I.grid_z);
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid; cfg.blockDim = dim3(kGemmThreads, 1, 1); cfg.dynamicSmemBytes = (size_t)I.smem_bytes; cfg.stream = st;
+    cfg.gridDim = grid; cfg.blockDim = dim3(kGemmThreads, 1, 1); cfg.dynamicSmemBytes = (size_t)smem_bytes; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     int n_attr = 0;
     // the kernel's set-up may overlap the tail of the kernel before it in the stream (it waits before its first

@@ -989,6 +989,18 @@ def test_mn_major_operands_and_tma_read_out(spec):
     probe.close()
 
 
+@pytest.mark.parametrize("k", [8, 22, 72, 136, 263, 1032])
+def test_ring_deeper_than_the_record(k):
+    """One CTA per SM: the ring takes as many stages as fit, from one up to the kernel's limit, a CTA's whole reduction or a
+    part of it, beside a gather table, a compensated operand pair and a cluster's reduction."""
+    sp = W.Spec(B.TT_OP_DENSE, B.dense_shapes(37, k, 50, True, B.TT_ACT_RELU), 1, "ring_k%d" % k, "bert")
+    a = W.make_inputs(sp, 95)
+    ref = util.oracle_ref(sp, a)
+    re = elem_ref(sp, a, ref)
+    for tn, tk, st, ax, sk, x3 in ((16, 8, 1, 1, 1, 0), (16, 32, 2, 2, 1, 1), (32, 8, 2, 1, 4, 0), (128, 64, 1, 2, 2, 0), (256, 32, 3, 1, 1, 0)):
+        run_spec(sp, tc(tile_n=tn, tile_k=tk, stages=st, mma_m_axis=ax, split_k=sk, precision=x3), a, ref, ref_elem=re)
+
+
 @pytest.mark.parametrize("shape", [
     # n, c, h, w, k, r, s, stride_h, stride_w, pad_h, pad_w, residual
     (3, 33, 7, 7, 40, 3, 3, 1, 1, 1, 1, True), (5, 8, 9, 5, 130, 3, 3, 2, 2, 1, 1, False), (2, 64, 14, 14, 16, 1, 1, 2, 2, 0, 0, True),
