@@ -14,7 +14,7 @@ namespace tt {
 cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
                         cudaStream_t st);
 cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st);
-cudaError_t launch_dw_tma(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st);
+cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st);
 cudaError_t launch_row(const tt_apply_info& I, const RowArgs& row, cudaStream_t st);
 cudaError_t gemm_cluster_fits(const GemmArgs& g, int smem_bytes, int* fits);
 cudaError_t launch_repack(const float* w, float* out, const ConvPmArgs& g, cudaStream_t st);
@@ -367,20 +367,22 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
         if (d.tma_stages > 0) {
             // the image's tensor map, cached per input pointer like the contraction's maps
             const TmapPair* maps = nullptr;
-            for (const TmapPair& m : w->tmaps) if (m.a_ptr == t->x) { maps = &m; break; }
-            if (!maps) {
-                TmapPair m;
-                std::memset(&m, 0, sizeof m);
-                m.a_ptr = t->x;
-                tt_status s = encode_planes(m.x, d.x, d.W, d.H, (long long)d.N * d.C, d.box_w, d.in_h, d.tile_c);
-                if (s != TT_OK) return s;
-                if (w->tmaps.size() >= 4096) w->tmaps.clear();
-                w->tmaps.push_back(m);
-                maps = &w->tmaps.back();
-            }
+            if (!d.runs) {
+                for (const TmapPair& m : w->tmaps) if (m.a_ptr == t->x) { maps = &m; break; }
+                if (!maps) {
+                    TmapPair m;
+                    std::memset(&m, 0, sizeof m);
+                    m.a_ptr = t->x;
+                    tt_status s = encode_planes(m.x, d.x, d.W, d.H, (long long)d.N * d.C, d.box_w, d.in_h, d.tile_c);
+                    if (s != TT_OK) return s;
+                    if (w->tmaps.size() >= 4096) w->tmaps.clear();
+                    w->tmaps.push_back(m);
+                    maps = &w->tmaps.back();
+                }
+            } else d.vec_in = (reinterpret_cast<uintptr_t>(t->x) & 15u) == 0;
             d.status = w->status_word;
             d.wait_ns = w->wait_ns;
-            e = launch_dw_tma(p.info, d, maps->x, st);
+            e = launch_dw_staged(p.info, d, maps ? maps->x : nullptr, st);
         } else
         e = launch_dw(p.info, d, st);
     } else {

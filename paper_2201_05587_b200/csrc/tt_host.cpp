@@ -660,6 +660,126 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
     return TT_OK;
 }
 
+// Wavefronts of one 16-byte read of a window row by the first warps of a staged depthwise tile (8 lanes a phase, the banks
+// repeat every 128 bytes), for strips `gw_step` 16-byte units apart, strip rows `gh_step` and planes `pl_step` apart.
+static int dw_read_wavefronts(int groups_w, int groups_h, int planes, bool plane_next, int gw_step, int gh_step, int pl_step) {
+    const int spp = groups_w * groups_h, lanes = std::min(128, planes * spp);
+    int total = 0;
+    for (int l0 = 0; l0 < lanes; l0 += 8) {
+        int count[8] = {};
+        for (int l = l0; l < std::min(lanes, l0 + 8); ++l) {
+            const int gw = l % groups_w, r = l / groups_w;
+            const int pl = plane_next ? r % planes : r / groups_h, gh = plane_next ? r / planes : r % groups_h;
+            ++count[(gw * gw_step + gh * gh_step + pl * pl_step) & 7];
+        }
+        total += *std::max_element(count, count + 8);
+    }
+    return total;
+}
+
+// Geometry of the staged persistent kernel for a tile of d.tile_c planes x d.tile_h x d.tile_w outputs in strips of `rows` x `items`:
+// box, buffers, the lanes' order.  Returns the bytes of one stage.
+static long long plan_dw_boxes(DwArgs& d, int rows, int items) {
+    const int ncol = (items - 1) * d.sw + d.S, nld = (4 - d.pw + ncol + 3) / 4;      // 16-byte loads per window row
+    // strips are `rows` tall: the box covers the rows of the last, possibly partial, strip too
+    d.in_h = (round_up(d.tile_h, rows) - 1) * d.sh + d.R;
+    d.box_w = (d.tile_w - items) * d.sw + 4 * nld;
+    d.plane_next = 0;
+    const int gw = d.tile_w / items, gh = (d.tile_h + rows - 1) / rows;
+    if (gw * gh <= 256) {
+        // one more 16-byte unit per row and the order of the lanes are free: take what the banks serve in the fewest turns, the wider row
+        // only for a fifth fewer
+        int best = 0, wide = 0;
+        for (int extra = 0; extra < 2; ++extra)
+            for (int order = 0; order < 2; ++order) {
+                const int bw4 = d.box_w / 4 + extra;
+                const int n = dw_read_wavefronts(gw, gh, d.tile_c, order != 0, items / 4 * d.sw, rows * d.sh * bw4, d.in_h * bw4);
+                if (best == 0 || (extra == wide ? n < best : 5 * n <= 4 * best)) { best = n; wide = extra; d.plane_next = order; }
+            }
+        d.box_w += 4 * wide;
+    }
+    d.stage_bytes = (int)std::min<long long>(0x7fffff80, (((long long)d.tile_c * d.in_h * d.box_w * 4) + 127) / 128 * 128);
+    d.wstage_bytes = (int)((((long long)d.tile_c * round_up(d.R * d.S + 1, 4) * 4) + 127) / 128 * 128);
+    return (long long)d.stage_bytes + d.wstage_bytes;
+}
+
+// Image rows that are no 16-byte multiples: no box can fetch them, and a register-window strip fetches each value of its rows
+// with a load of its own.  The run-staged persistent kernel runs instead; its tiles are this rule's, as the record has no fields
+// for them: strips of the height that takes the fewest instructions for the image's rows, channels for up to 256 threads in
+// buffers of 24 KB, but two tiles for every SM first.  From a quarter of a million outputs on: 480 x 14 x 14, 5x5, takes 4.5 us either
+// way for one image, 4.7 instead of 7.5 for 4 and 78 instead of 134 for 256; 960 x 7 x 7, 3x3, 3.6 instead of 2.9 for 4 (188 thousand
+// outputs), 5.0 instead of 5.2 for 16 and 30 instead of 44 for 256.
+static bool plan_dw_runs(const tt_workload* w, DwArgs& d, tt_apply_info& I) {
+    const tt_shapes& s = w->sh;
+    const long long planes = (long long)s.n * s.c, hw = (long long)s.h * s.w;
+    if (s.w % 4 == 0 || w->Q > 256 || planes > 0x7fffffffLL || hw > (1 << 24)) return false;
+    DwArgs t = d;
+    double best_cost = 0;
+    for (int rows : {7, 4, 2}) {
+        const int in_rows = (rows - 1) * s.stride_h + s.r;
+        const double cost = (double)((w->P + rows - 1) / rows) * (in_rows * (2.0 * s.r + 3) + rows * (s.r * s.r + 4.0) + 40);
+        if (best_cost == 0 || cost < best_cost) { best_cost = cost; t.window_rows = rows; }
+    }
+    const int rows = t.window_rows;
+    t.items = s.w % 2 == 0 ? 2 : 1;                        // even rows: a thread takes two columns, read in aligned pairs
+    t.runs = 1; t.tile_w = w->Q;
+    t.vec = w->Q % 2 == 0 ? t.items : 1;
+    const int lanes_q = (w->Q + t.items - 1) / t.items;    // threads of a strip row
+    const int upw = lanes_q <= 32 ? 32 / lanes_q : 0;      // strip rows a warp takes side by side
+    const int fit = upw ? 8 * upw : 256 / lanes_q;         // ... and 256 threads
+    t.tile_h = w->P; t.tile_c = 1;
+    if (hw * 4 > 24 * 1024) {
+        // bands of one plane, of whole strips
+        t.tile_h = rows;
+        while (t.tile_h + rows <= w->P && (long long)((t.tile_h + rows - 1) * s.stride_h + s.r) * s.w * 4 <= 24 * 1024) t.tile_h += rows;
+    }
+    t.tiles_h = (w->P + t.tile_h - 1) / t.tile_h; t.tiles_w = 1;
+    const int strips_h = (t.tile_h + rows - 1) / rows;
+    t.strip_rows = std::min(strips_h, fit);
+    if (t.tiles_h == 1) {
+        const long long share = std::max(1LL, planes / (2 * 148));
+        t.tile_c = (int)std::min<long long>({(long long)s.c, share, (long long)std::max(1, fit / t.strip_rows), std::max(1LL, 24 * 1024 / (hw * 4))});
+        // groups of channels as equal as they come
+        const int groups = (s.c + t.tile_c - 1) / t.tile_c;
+        t.tile_c = (s.c + groups - 1) / groups;
+    }
+    t.in_h = (round_up(t.tile_h, rows) - 1) * s.stride_h + s.r;
+    const int units = t.tile_c * t.strip_rows;
+    t.units_per_warp = upw; t.unit_far = 0;
+    if (upw > 1) {
+        // which units share a warp decides how its reads fall on the banks: neighbours, or ones a fixed distance apart
+        const int far = (units + upw - 1) / upw;
+        int turns[2] = {};
+        for (int pass = 0; pass < 2; ++pass)
+            for (int wp = 0; wp < far; ++wp) {
+                int count[2][32] = {};                     // a pair takes two banks: half a warp at a time
+                for (int j = 0; j < upw; ++j) {
+                    const int unit = pass ? wp + j * far : wp * upw + j;
+                    if (unit >= units) continue;
+                    const long long off = unit / t.strip_rows * hw + (long long)(unit % t.strip_rows) * rows * s.stride_h * s.w;
+                    for (int q = 0; q < lanes_q; ++q)
+                        ++count[t.items == 2 && j * lanes_q + q >= 16][(off + (long long)q * t.items * s.stride_w) & 31];
+                }
+                turns[pass] += *std::max_element(count[0], count[0] + 32) + *std::max_element(count[1], count[1] + 32);
+            }
+        if (turns[1] < turns[0]) t.unit_far = far;
+    }
+    const int threads = std::min(256, upw ? (units + upw - 1) / upw * 32 : round_up(units * lanes_q, 32));
+    const long long run = t.tiles_h == 1 ? t.tile_c * hw : (long long)std::min(t.in_h, s.h) * s.w;
+    t.stage_bytes = (int)((run * 4 + 32 + 127) / 128 * 128);
+    t.tma_stages = 2;
+    while (t.tma_stages < 4 && (t.tma_stages + 1ll) * t.stage_bytes <= 56 * 1024) ++t.tma_stages;
+    const long long smem = (long long)t.tma_stages * t.stage_bytes + round_up(s.w * 4, 128);
+    const long long total = (long long)((s.c + t.tile_c - 1) / t.tile_c) * s.n * t.tiles_h;
+    if (smem > kDynSmemLimit || total > 0x7fffffffLL || planes * w->P * w->Q < 1 << 18) return false;
+    t.total_tiles = (int)total;
+    const long long per_sm = std::max<long long>(1, std::min<long long>({16LL, (228 * 1024) / (smem + 1024), 2048LL / threads}));
+    d = t;
+    I.grid_x = (int)std::min<long long>(total, 148 * per_sm); I.grid_y = 1; I.grid_z = 1;
+    I.threads = threads; I.smem_bytes = (int)smem; I.launches = 1;
+    return true;
+}
+
 static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec, int mode, Plan* plan) {
     const tt_shapes& s = w->sh;
     const bool strict = mode == TT_MODE_STRICT;
@@ -729,22 +849,23 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     L.raster = 0;
     if (rec->raster < 0 || rec->raster > 1) return TT_ERR_INVALID_SCHEDULE;
     if (rec->raster == 1 && window_rows > 0 && (s.w % 4) == 0) {
-        const int st = d.sh, pad = d.pw;
-        const int ncol = (items - 1) * st + d.R, nld = (4 - pad + ncol + 3) / 4;      // 16-byte loads per window row
-        const int box_w = (d.tile_w - items) * st + 4 * nld;
-        // strips are window_rows tall: the box covers the rows of the last, possibly partial, strip too
-        const int in_h_box = (round_up(d.tile_h, window_rows) - 1) * d.sh + d.R;
         const long long planes = (long long)s.n * s.c;
-        const long long box = (((long long)d.tile_c * in_h_box * box_w * 4) + 127) / 128 * 128;
-        const long long wstage = (((long long)d.tile_c * round_up(d.R * d.S + 1, 4) * 4) + 127) / 128 * 128;
-        const long long stage = box + wstage;
+        // a 5x5 filter's tallest strip becomes one of seven rows where that covers the tile as well and the chip has tiles to spare: a
+        // strip then reads 11 rows for 7, not 8 for 4 (3x3: 9 for 7 against 6 for 4, and it was slower on 56-pixel rows, 157 -> 173 us)
+        int rows = window_rows;
+        if (rows == 4 && s.r == 5 && round_up(d.tile_h, 7) <= round_up(d.tile_h, 4) && (planes + d.tile_c - 1) / d.tile_c * d.tiles_h * d.tiles_w >= 148 * 4) rows = 7;
+        DwArgs t = d;
+        const long long stage = plan_dw_boxes(t, rows, items);
         int stg = std::min(4, std::max(2, rec->stages));
         while (stg > 2 && stg * stage + 128 > kDynSmemLimit) --stg;
-        if (box_w <= 256 && in_h_box <= 256 && d.tile_c <= 256 && stg * stage + 128 <= kDynSmemLimit && planes <= 0x7fffffffLL) {
-            d.in_h = in_h_box;
+        if (t.box_w <= 256 && t.in_h <= 256 && t.tile_c <= 256 && stg * stage + 128 <= kDynSmemLimit && planes <= 0x7fffffffLL) {
+            d = t;
+            d.window_rows = rows;
             if (stg != rec->stages) { if (strict) return TT_ERR_INVALID_SCHEDULE; I.changed |= TT_CHG_STAGES; }
             L.raster = 1; L.stages = stg;
-            d.tma_stages = stg; d.box_w = box_w; d.stage_bytes = (int)box; d.wstage_bytes = (int)wstage;
+            d.tma_stages = stg;
+            // no more threads than a tile has strips
+            th = std::min(th, round_up(d.tile_c * ((d.tile_h + rows - 1) / rows) * (d.tile_w / items), 32));
             d.tiles_p = (int)((planes + d.tile_c - 1) / d.tile_c);
             const long long total = (long long)d.tiles_p * d.tiles_h * d.tiles_w;
             if (total > 0x7fffffffLL) return TT_ERR_RESOURCE;
@@ -760,6 +881,7 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     }
     if (rec->raster != 0) { if (strict) return TT_ERR_INVALID_SCHEDULE; I.changed |= TT_CHG_FORM; }
     I.legal = L;
+    if (window_rows > 0 && plan_dw_runs(w, d, I)) return TT_OK;
     I.grid_x = (int)std::min<long long>(gx, 0x7fffffff); I.grid_y = s.n; I.grid_z = 1;
     I.threads = th; I.smem_bytes = (int)std::min<long long>(smem, 0x7fffffff);
     I.launches = 1;

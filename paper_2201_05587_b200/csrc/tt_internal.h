@@ -116,11 +116,15 @@ struct DwArgs {
     int tiles_c, tiles_h, tiles_w;
     int window_rows;   // > 0: register-window kernel with this many output rows per thread; 0: staged kernel
     int vec_in;        // input rows start on 16-byte boundaries (W % 4 == 0 and x aligned)
-    // TMA-staged persistent kernel (record raster = 1): tiles of tile_c planes x tile_h x tile_w outputs, their input
-    // boxes [tile_c][in_h][box_w] land in `stages` shared-memory buffers by TMA (zero fill = padding)
-    int tma_stages;    // > 0 selects it
+    // persistent kernels: tiles of tile_c planes x tile_h x tile_w outputs, whose input lands in `tma_stages` shared-memory buffers:
+    // as boxes [tile_c][in_h][box_w] by TMA (zero fill = padding), or (runs) as packed planes or rows of a plane
+    int tma_stages;    // > 0 selects them
     int box_w, stage_bytes, tiles_p, total_tiles;   // box width in floats (multiple of 4), bytes per buffer (multiple of 128)
-    int wstage_bytes;  // bytes per filter-and-bias buffer (one per box buffer, multiple of 128)
+    int wstage_bytes;  // boxes: bytes per filter-and-bias buffer (one per box buffer, multiple of 128)
+    int plane_next;    // boxes: lanes after a row of strips continue with the next plane's strips, not with the next strip row
+    int runs;
+    int strip_rows;    // runs: strip rows of a plane that are computed at a time
+    int units_per_warp, unit_far;   // runs: strip rows side by side in a warp (0: they run on through the warps), their distance (0: 1)
     unsigned* status;  // the workload's status word (bounded waits)
     unsigned long long wait_ns;   // limit of every bounded wait inside the kernel
 };

@@ -1845,7 +1845,10 @@ __global__ void __launch_bounds__(256, WIDTH == 4 ? 6 : 4) tt_dwconv_window_kern
 // The instruction stream per output is what bounds this kernel next to the memory system, so everything that does
 // not depend on the plane is hoisted: a thread keeps its strip position for the whole kernel, tile coordinates
 // advance by additions, and the filters and biases of a tile's planes are staged in shared memory (one buffer per
-// box buffer, [tile_c][WP] floats: filter, bias, padding) when the tile's box is requested.
+// box buffer, [tile_c][WP] floats: filter, bias, padding) when the tile's box is requested.  They travel by cp.async on the
+// box's barrier: no thread waits for them (fetched through registers, a tile's refill held every thread up for a trip to L2).
+// A CTA has no more threads than a tile has strips, so more CTAs fit; the order of the lanes and the row pitch keep a warp's reads
+// off the same banks.  240 x 28 x 28, 5x5, 256 images: 109 -> 88 us (HBM 59), bound by issue: three instructions in five are products.
 // ------------------------------------------------------------------------------------------------------------
 template <int R, int STRIDE, int ROWS, int WIDTH>
 __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constant__ CUtensorMap tmap_x, const DwArgs d) {
@@ -1863,7 +1866,7 @@ __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constan
     volatile int* abortp = &abort_flag;
     pdl_allow_next();
     if (threadIdx.x == 0) {
-        for (int s = 0; s < d.tma_stages; ++s) mbar_init(smem_u32(&full_bar[s]), 1u);
+        for (int s = 0; s < d.tma_stages; ++s) mbar_init(smem_u32(&full_bar[s]), blockDim.x + 1u);   // every thread's filter copies, and the box
         abort_flag = 0;
         fence_mbar_init();
         fence_proxy_async_shared();
@@ -1901,37 +1904,32 @@ __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constan
         if (t.th >= d.tiles_h) { t.th -= d.tiles_h; ++t.tp; t.c0 += tile_c_mod; }
         while (t.c0 >= d.C) t.c0 -= d.C;
     };
-    auto issue = [&](const TilePos& t, int s) {           // thread 0: request the input box of a tile into buffer s
+    auto fill = [&](const TilePos& t, int s) {            // all threads: request a tile's box, filters and biases into buffer s
         const uint32_t bar = smem_u32(&full_bar[s]);
-        mbar_expect_tx(bar, (uint32_t)(d.tile_c * d.in_h * d.box_w * 4));
-        tma_load_3d(base + (uint32_t)s * (uint32_t)d.stage_bytes, &tmap_x, bar, t.tw * d.tile_w * STRIDE - 4,
-                    t.th * d.tile_h * STRIDE - PAD, t.tp * d.tile_c);
-    };
-    auto stage_weights = [&](const TilePos& t, int s) {   // all threads: the filters and biases of the tile's planes
-        const uint32_t dst = wbase + (uint32_t)s * (uint32_t)d.wstage_bytes;
         const int pl0 = t.tp * d.tile_c;
+        if (threadIdx.x == 0) {
+            mbar_expect_tx(bar, (uint32_t)(d.tile_c * d.in_h * d.box_w * 4));
+            tma_load_3d(base + (uint32_t)s * (uint32_t)d.stage_bytes, &tmap_x, bar, t.tw * d.tile_w * STRIDE - 4,
+                        t.th * d.tile_h * STRIDE - PAD, pl0);
+        }
+        const uint32_t dst = wbase + (uint32_t)s * (uint32_t)d.wstage_bytes;
         for (int idx = (int)threadIdx.x; idx < d.tile_c * WP; idx += (int)blockDim.x) {
             const int cl = idx / WP, k = idx - cl * WP;
             int c = t.c0 + cl;                            // tile_c <= C: one subtraction wraps it
             if (c >= d.C) c -= d.C;
-            float v = 0.f;
-            if (pl0 + cl < planes) {
-                if (k < R * R) v = __ldg(d.w + c * (R * R) + k);
-                else if (k == R * R && d.bias) v = __ldg(d.bias + c);
-            }
-            st_shared_f32(dst + 4u * (uint32_t)idx, v);
+            const bool filter = k < R * R, have = pl0 + cl < planes && (filter || (k == R * R && d.bias));
+            cp_async_4_or_zero(dst + 4u * (uint32_t)idx, !have ? d.w : filter ? d.w + c * (R * R) + k : d.bias + c, have);
         }
+        cp_async_arrive(bar);
     };
     TilePos cur = first_pos(), nxt = cur;
     {
         const int pre = min(my_tiles, d.tma_stages);
         for (int i = 0; i < pre; ++i) {
-            if (threadIdx.x == 0) issue(nxt, i);
-            stage_weights(nxt, i);
+            fill(nxt, i);
             advance(nxt);
         }
     }
-    __syncthreads();                                      // the first weight buffers are in place
     // a thread's strip position inside a plane is fixed for the whole kernel when a plane has at most blockDim strips
     // (the thread then walks planes cl_f, cl_f + cpp, ...); otherwise it also walks strips
     const int groups_w = d.tile_w / WIDTH;
@@ -1939,10 +1937,19 @@ __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constan
     const int spp = groups_h * groups_w;                  // strips per plane
     const bool fixed_pos = spp <= (int)blockDim.x;
     const int cpp = fixed_pos ? (int)blockDim.x / spp : 1;                  // planes per pass
-    const int cl_f = fixed_pos ? (int)threadIdx.x / spp : 0;
-    const int s_f = (int)threadIdx.x - cl_f * spp;
+    // neighbouring lanes take the strips of a row, then the plane's next strip row or (plane_next) the next plane's strips:
+    // whichever spreads a warp's 16-byte reads over more of the banks
+    int cl_f = 0, s_f = (int)threadIdx.x;
+    if (fixed_pos && d.plane_next) {
+        const int r = (int)threadIdx.x / groups_w;
+        cl_f = r % cpp;
+        s_f = r / cpp * groups_w + ((int)threadIdx.x - r * groups_w);
+    } else if (fixed_pos) {
+        cl_f = (int)threadIdx.x / spp;
+        s_f = (int)threadIdx.x - cl_f * spp;
+    }
     const int s_step = fixed_pos ? spp : (int)blockDim.x;                    // fixed: the strip loop runs once
-    const bool active = cl_f < cpp;
+    const bool active = cl_f < cpp && s_f < spp;
     const int gh_f = s_f / groups_w, gwi_f = s_f - gh_f * groups_w;
     const uint32_t plane_bytes = 4u * (uint32_t)(d.in_h * d.box_w);
     const long long plane_out = (long long)d.P * d.Q;
@@ -2029,14 +2036,214 @@ __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constan
         }
         __syncthreads();                                  // everyone is done with this box and its weight buffer
         if (i + d.tma_stages < my_tiles) {
-            if (threadIdx.x == 0) issue(nxt, s);
-            stage_weights(nxt, s);                        // read again only after a later barrier (stages >= 2)
+            fill(nxt, s);
             advance(nxt);
         }
         advance(cur);
         if (++s == d.tma_stages) { s = 0; ph ^= 1u; }
     }
+    cp_async_wait_all();
     // after a tripped wait: let the boxes still in flight land before the shared memory is given back (bounded)
+    if (threadIdx.x == 0 && *abortp) {
+        for (int b = 0; b < d.tma_stages; ++b) {
+            const unsigned long long t0 = global_timer_ns();
+            while (!mbar_try_wait(smem_u32(&full_bar[b]), 0u) && !mbar_try_wait(smem_u32(&full_bar[b]), 1u)) {
+                if (global_timer_ns() - t0 > 2000000ull) break;
+            }
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------
+// DW_SIMT, run-staged persistent form (3x3 and 5x5 "same" filters, stride 1 or 2, image rows that are no 16-byte multiples, which
+// fit no TMA box).  Consecutive planes of an image, or consecutive rows of one plane, are one run of floats: a bulk copy brings it
+// in from the 16-byte boundary before it (up to three floats at the tensor's end by cp.async).  Its rows lie packed, so a thread
+// takes one output column x ROWS rows and neighbouring lanes neighbouring columns: 4-byte reads without bank conflicts inside a
+// row, coalesced stores.  A window column outside the image is a predicate that holds for the strip, a window row outside it is
+// read from a row of zeros.  Same products in the same order as the other forms.
+// Instruction issue bounds it next to the memory system, so a thread keeps its column, and its channel's filter in registers: the
+// tiles are counted channels first, a CTA takes a consecutive range of them and meets a new filter once or twice.
+// Even rows: a thread takes two columns, read as pairs; with stride 1 their products are paired too (half the issue slots).
+// 256 images, against the register-window form's best record: 480 x 14 x 14, 5x5: 134 -> 57 us (HBM 30); 384 x 14 x 14, 3x3: 61 -> 33
+// (24); 576 x 14 x 14, 3x3 stride 2: 53 -> 29 (22); 960 x 7 x 7, 3x3: 44 -> 30 (15); 64 images of 144 x 55 x 55, 3x3: 77 -> 54 (34).
+// ------------------------------------------------------------------------------------------------------------
+template <int R, int STRIDE, int ROWS, int WIDTH>
+__global__ void __launch_bounds__(256, R == 5 && STRIDE == 1 && WIDTH == 2 ? 2 : 3) tt_dwconv_run_kernel(const DwArgs d) {
+    constexpr int IN_ROWS = (ROWS - 1) * STRIDE + R;
+    constexpr int PAD = R / 2;
+    // two columns: window columns are read in pairs from an even one on, each of them inside the image or outside as a whole
+    constexpr int LEFT = WIDTH == 2 ? 2 : PAD, FIRST = LEFT - PAD;
+    constexpr int NLD = WIDTH == 2 ? (FIRST + STRIDE + R + 1) / 2 : R;
+    const int lanes_q = (d.Q + WIDTH - 1) / WIDTH;        // threads of one strip row
+    extern __shared__ __align__(128) float dw_floats[];
+    __shared__ uint64_t full_bar[4];
+    __shared__ int abort_flag;
+    const int stage_f = d.stage_bytes / 4, zero_f = d.tma_stages * stage_f;      // after the buffers: the row of zeros
+    const uint32_t base = smem_u32(dw_floats);
+    volatile int* abortp = &abort_flag;
+    pdl_allow_next();
+    if (threadIdx.x == 0) {
+        // the run's request and the copies of thread 0, or (x not on 16 bytes) of every thread
+        for (int s = 0; s < d.tma_stages; ++s) mbar_init(smem_u32(&full_bar[s]), d.vec_in ? 2u : blockDim.x + 1u);
+        abort_flag = 0;
+        fence_mbar_init();
+        fence_proxy_async_shared();
+    }
+    for (int i = (int)threadIdx.x; i < d.W; i += (int)blockDim.x) dw_floats[zero_f + i] = 0.f;
+    __syncthreads();
+    pdl_wait_prev();                                      // the set-up above touched no global memory
+    const int HW = d.H * d.W;
+    const long long all = (long long)d.N * d.C * HW;
+    const bool whole = d.tiles_h == 1;                    // tiles of whole planes; otherwise of a band of one plane
+    const int per_ct = d.N * d.tiles_h;                   // tiles of one group of tile_c channels
+    const int t0 = (int)((long long)d.total_tiles * blockIdx.x / gridDim.x), t1 = (int)((long long)d.total_tiles * (blockIdx.x + 1) / gridDim.x);
+    struct Tile { int ct, n, th; };
+    auto next = [&](Tile& t) {
+        if (++t.th < d.tiles_h) return;
+        t.th = 0;
+        if (++t.n < d.N) return;
+        t.n = 0; ++t.ct;
+    };
+    Tile cur;
+    cur.ct = t0 / per_ct; cur.th = t0 - cur.ct * per_ct; cur.n = cur.th / d.tiles_h; cur.th -= cur.n * d.tiles_h;
+    // the run's first float and first image row
+    auto start_of = [&](const Tile& t, int& row0) {
+        row0 = whole ? 0 : max(0, t.th * d.tile_h * STRIDE - PAD);
+        return ((long long)t.n * d.C + t.ct * d.tile_c) * HW + row0 * d.W;
+    };
+    auto fill = [&](const Tile& t, int s) {
+        if (d.vec_in && threadIdx.x != 0) return;
+        int row0;
+        const long long start = start_of(t, row0), first = start & ~3LL;
+        const long long end = start + (whole ? min(d.tile_c, d.C - t.ct * d.tile_c) * HW
+                                             : (min(d.H, t.th * d.tile_h * STRIDE - PAD + d.in_h) - row0) * d.W);
+        const uint32_t bar = smem_u32(&full_bar[s]), dst = base + (uint32_t)s * (uint32_t)d.stage_bytes;
+        if (threadIdx.x == 0) {
+            const long long split = d.vec_in ? min((end + 3) & ~3LL, all & ~3LL) : first;      // [first, split) in one copy
+            const uint32_t bytes = split > first ? (uint32_t)(split - first) * 4u : 0u;
+            mbar_expect_tx(bar, bytes);
+            if (bytes) bulk_load(dst, d.x + first, bytes, bar);
+            if (d.vec_in) for (long long e = max(split, first); e < end; ++e) cp_async_4(dst + 4u * (uint32_t)(e - first), d.x + e);
+        }
+        if (!d.vec_in) for (long long e = start + (int)threadIdx.x; e < end; e += (int)blockDim.x) cp_async_4(dst + 4u * (uint32_t)(e - first), d.x + e);
+        cp_async_arrive(bar);
+    };
+    Tile ahead = cur;
+    for (int i = 0; i < min(t1 - t0, d.tma_stages); ++i) { fill(ahead, i); next(ahead); }
+    // This thread's column q of strip row gh (and gh + strip_rows, ...) of plane pl.  A unit is one strip row of one plane: Q columns.
+    // Narrow images put `units_per_warp` of them side by side in a warp, either consecutive ones or ones `unit_far` apart,
+    // whichever spreads the reads over more banks; wide ones run on through the warps.
+    int pl, gh0, q;
+    bool active;
+    {
+        const int units = d.tile_c * d.strip_rows;
+        int u;
+        if (d.units_per_warp) {
+            const int lane = (int)threadIdx.x & 31, warp = (int)threadIdx.x >> 5, slot = lane / lanes_q;
+            q = lane - slot * lanes_q;
+            u = d.unit_far ? warp + slot * d.unit_far : warp * d.units_per_warp + slot;
+            active = slot < d.units_per_warp && u < units;
+        } else {
+            u = (int)threadIdx.x / lanes_q; q = (int)threadIdx.x - u * lanes_q;
+            active = u < units;
+        }
+        pl = u / d.strip_rows; gh0 = u - pl * d.strip_rows;
+    }
+    q *= WIDTH;
+    const int col0 = q * STRIDE - LEFT;
+    bool in_col[NLD];
+#pragma unroll
+    for (int k = 0; k < NLD; ++k) in_col[k] = (unsigned)(col0 + k * WIDTH) < (unsigned)d.W;
+    const bool pair_out = WIDTH == 2 && d.Q % 2 == 0 && d.vec >= 2;      // d.vec: what y's alignment allows
+    const bool clamp = d.act == TT_ACT_RELU || d.act == TT_ACT_RELU6, gelu = d.act == TT_ACT_GELU_ERF;
+    const float hi = d.act == TT_ACT_RELU6 ? 6.f : INFINITY;
+    float wv[R * R], bias = 0.f;
+    int s = 0, have_ct = -1;
+    uint32_t ph = 0;
+    for (int i = 0; i < t1 - t0; ++i) {
+        const int c = cur.ct * d.tile_c + pl;             // this thread's channel
+        const bool mine = active && c < d.C;
+        if (cur.ct != have_ct && mine) {
+#pragma unroll
+            for (int k = 0; k < R * R; ++k) wv[k] = __ldg(d.w + (long long)c * (R * R) + k);
+            if (d.bias) bias = __ldg(d.bias + c);
+        }
+        have_ct = cur.ct;
+        if (!mbar_wait(smem_u32(&full_bar[s]), ph, abortp, d.status, 9u, d.wait_ns)) break;
+        int row0;
+        const int shift = (int)(start_of(cur, row0) & 3LL);
+        const int p0 = cur.th * d.tile_h, p_end = min(d.P, p0 + d.tile_h);
+        const int x0 = s * stage_f + shift + pl * HW - row0 * d.W + col0;      // image row 0 of this thread's first window column
+        float* __restrict__ y0 = d.y + (((long long)cur.n * d.C + c) * d.P) * d.Q + q;
+        if (mine) {
+#pragma unroll 1
+            for (int p = p0 + gh0 * ROWS; p < p_end; p += d.strip_rows * ROWS) {
+                float2 acc[ROWS];                         // .y: the second column
+#pragma unroll
+                for (int ro = 0; ro < ROWS; ++ro) acc[ro] = make_float2(bias, bias);
+                const int ih0 = p * STRIDE - PAD;
+                int at = x0 + ih0 * d.W;
+#pragma unroll
+                for (int ri = 0; ri < IN_ROWS; ++ri) {
+                    const int r = (unsigned)(ih0 + ri) < (unsigned)d.H ? at : zero_f + col0;
+                    at += d.W;
+                    float v[NLD * WIDTH];
+#pragma unroll
+                    for (int k = 0; k < NLD; ++k) {
+                        if constexpr (WIDTH == 2) {
+                            const float2 f = in_col[k] ? *reinterpret_cast<const float2*>(dw_floats + r + 2 * k) : make_float2(0.f, 0.f);
+                            v[2 * k] = f.x; v[2 * k + 1] = f.y;
+                        } else v[k] = in_col[k] ? dw_floats[r + k] : 0.f;
+                    }
+#pragma unroll
+                    for (int ro = 0; ro < ROWS; ++ro) {
+                        const int fr = ri - ro * STRIDE;  // compile-time after unrolling
+                        if (fr >= 0 && fr < R) {
+#pragma unroll
+                            for (int fs = 0; fs < R; ++fs) {
+                                const float w = wv[fr * R + fs];
+                                if constexpr (WIDTH == 1) acc[ro].x = fmaf(v[fs], w, acc[ro].x);
+                                else if constexpr (STRIDE == 1) acc[ro] = fma_pair(make_float2(v[FIRST + fs], v[FIRST + fs + 1]), make_float2(w, w), acc[ro]);
+                                else {
+                                    acc[ro].x = fmaf(v[FIRST + fs], w, acc[ro].x);
+                                    acc[ro].y = fmaf(v[FIRST + fs + STRIDE], w, acc[ro].y);
+                                }
+                            }
+                        }
+                    }
+                }
+                if (clamp) {
+#pragma unroll
+                    for (int ro = 0; ro < ROWS; ++ro) {
+                        acc[ro].x = fminf(fmaxf(acc[ro].x, 0.f), hi);
+                        if (WIDTH == 2) acc[ro].y = fminf(fmaxf(acc[ro].y, 0.f), hi);
+                    }
+                } else if (gelu) {
+#pragma unroll
+                    for (int ro = 0; ro < ROWS; ++ro) {
+                        acc[ro].x = gelu_erf(acc[ro].x);
+                        if (WIDTH == 2) acc[ro].y = gelu_erf(acc[ro].y);
+                    }
+                }
+                float* __restrict__ yo = y0 + p * d.Q;
+#pragma unroll
+                for (int ro = 0; ro < ROWS; ++ro) {
+                    if (p + ro >= p_end) break;
+                    if (pair_out) *reinterpret_cast<float2*>(yo + ro * d.Q) = acc[ro];
+                    else {
+                        yo[ro * d.Q] = acc[ro].x;
+                        if (WIDTH == 2 && q + 1 < d.Q) yo[ro * d.Q + 1] = acc[ro].y;
+                    }
+                }
+            }
+        }
+        __syncthreads();                                  // everyone is done with this run
+        if (i + d.tma_stages < t1 - t0) { fill(ahead, s); next(ahead); }
+        next(cur);
+        if (++s == d.tma_stages) { s = 0; ph ^= 1u; }
+    }
+    cp_async_wait_all();
+    // after a tripped wait: let the runs still in flight land before the shared memory is given back (bounded)
     if (threadIdx.x == 0 && *abortp) {
         for (int b = 0; b < d.tma_stages; ++b) {
             const unsigned long long t0 = global_timer_ns();
@@ -2407,26 +2614,36 @@ struct ResidentCtas {
     }
 };
 
-cudaError_t launch_dw_tma(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st) {
+cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st) {
     CUtensorMap tx;
-    memcpy(&tx, tmap_x, sizeof tx);
+    if (tmap_x) memcpy(&tx, tmap_x, sizeof tx); else memset(&tx, 0, sizeof tx);
     dim3 grid(I.grid_x, 1, 1);
     int dev = 0;
     cudaGetDevice(&dev);
     // resident CTAs of this instantiation, looked up once per launch shape (the query costs more than the launch)
-#define TT_DWT_CASE(RR, SS, RO, WI) \
-    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == WI) { \
+#define TT_DWT_CASE(KERNEL, ...) \
+    { \
         static thread_local ResidentCtas known; \
         long long resident = 0; \
-        cudaError_t e = known.get(tt_dwconv_tma_kernel<RR, SS, RO, WI>, dev, I.threads, I.smem_bytes, &resident); \
+        cudaError_t e = known.get(KERNEL, dev, I.threads, I.smem_bytes, &resident); \
         if (e != cudaSuccess) return e; \
         /* persistent CTAs: never more than are resident at once (registers may allow fewer than shared memory does) */ \
         grid.x = (unsigned)std::min<long long>(grid.x, resident); \
-        return launch_serialized(tt_dwconv_tma_kernel<RR, SS, RO, WI>, grid, (unsigned)I.threads, (size_t)I.smem_bytes, st, tx, dw); }
-    TT_DWT_CASE(3, 1, 1, 4) TT_DWT_CASE(3, 1, 2, 4) TT_DWT_CASE(3, 1, 4, 4) TT_DWT_CASE(3, 1, 1, 8) TT_DWT_CASE(3, 1, 2, 8)
-    TT_DWT_CASE(3, 2, 1, 4) TT_DWT_CASE(3, 2, 2, 4) TT_DWT_CASE(3, 2, 4, 4) TT_DWT_CASE(3, 2, 1, 8) TT_DWT_CASE(3, 2, 2, 8)
-    TT_DWT_CASE(5, 1, 1, 4) TT_DWT_CASE(5, 1, 2, 4) TT_DWT_CASE(5, 1, 4, 4) TT_DWT_CASE(5, 1, 1, 8) TT_DWT_CASE(5, 1, 2, 8)
-    TT_DWT_CASE(5, 2, 1, 4) TT_DWT_CASE(5, 2, 2, 4) TT_DWT_CASE(5, 2, 4, 4) TT_DWT_CASE(5, 2, 1, 8) TT_DWT_CASE(5, 2, 2, 8)
+        return launch_serialized(KERNEL, grid, (unsigned)I.threads, (size_t)I.smem_bytes, st, __VA_ARGS__); }
+#define TT_DWT_BOX(RR, SS, RO, WI) \
+    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == WI) TT_DWT_CASE((tt_dwconv_tma_kernel<RR, SS, RO, WI>), tx, dw)
+#define TT_DWT_RUN(RR, SS, RO) \
+    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == 1) TT_DWT_CASE((tt_dwconv_run_kernel<RR, SS, RO, 1>), dw) \
+    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == 2) TT_DWT_CASE((tt_dwconv_run_kernel<RR, SS, RO, 2>), dw)
+#define TT_DWT_FILTER(RR, SS) \
+    if (!dw.runs) { \
+        TT_DWT_BOX(RR, SS, 1, 4) TT_DWT_BOX(RR, SS, 2, 4) TT_DWT_BOX(RR, SS, 4, 4) TT_DWT_BOX(RR, SS, 1, 8) TT_DWT_BOX(RR, SS, 2, 8) \
+    } else { TT_DWT_RUN(RR, SS, 2) TT_DWT_RUN(RR, SS, 4) TT_DWT_RUN(RR, SS, 7) }
+    TT_DWT_FILTER(3, 1) TT_DWT_FILTER(3, 2) TT_DWT_FILTER(5, 1) TT_DWT_FILTER(5, 2)
+    if (!dw.runs) { TT_DWT_BOX(5, 1, 7, 4) TT_DWT_BOX(5, 2, 7, 4) }
+#undef TT_DWT_FILTER
+#undef TT_DWT_RUN
+#undef TT_DWT_BOX
 #undef TT_DWT_CASE
     return cudaErrorInvalidValue;
 }

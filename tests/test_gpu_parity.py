@@ -989,6 +989,40 @@ def test_mn_major_operands_and_tma_read_out(spec):
     probe.close()
 
 
+@pytest.mark.parametrize("n, c, h, w, r, stride, act, bias, off", [
+    (5, 301, 14, 14, 5, 1, B.TT_ACT_RELU6, True, 0), (29, 190, 7, 7, 3, 1, B.TT_ACT_NONE, False, 0), (23, 47, 17, 18, 3, 2, B.TT_ACT_RELU, True, 0),
+    (33, 33, 31, 30, 5, 2, B.TT_ACT_GELU_ERF, True, 0), (3, 9, 111, 109, 3, 1, B.TT_ACT_RELU, True, 0), (2, 11, 130, 131, 5, 1, B.TT_ACT_NONE, True, 0),
+    (3, 53, 5, 342, 3, 1, B.TT_ACT_RELU, True, 0), (9, 65, 33, 45, 5, 1, B.TT_ACT_RELU6, True, 1), (4, 403, 13, 14, 3, 1, B.TT_ACT_RELU6, True, 3),
+    (1, 131200, 2, 1, 3, 1, B.TT_ACT_RELU, True, 0), (3, 70, 253, 37, 3, 2, B.TT_ACT_NONE, False, 2), (3, 5, 150, 150, 5, 2, B.TT_ACT_NONE, False, 0)])
+def test_depthwise_rows_staged_as_runs(n, c, h, w, r, stride, act, bias, off):
+    """A batch of images whose rows are no 16-byte multiples: odd and even rows, planes and bands of planes, groups of channels
+    with a remainder, a tensor that ends inside 16 bytes, an input that starts inside them.  Each output is bounded against the
+    oracle, and the first and the last image equal, bit for bit, what the register-window form makes of them alone."""
+    def spec_for(m):
+        return W.Spec(B.TT_OP_DWCONV2D, B.make_shapes(n=m, c=c, h=h, w=w, k=c, r=r, s=r, stride_h=stride, stride_w=stride, pad_h=r // 2,
+                                                      pad_w=r // 2, has_bias=int(bias), act=act), 1, "dw_runs", "uniform")
+    spec = spec_for(n)
+    a = W.make_inputs(spec, 96)
+    ref = util.oracle_ref(spec, a)
+    rec = B.make_record(B.TT_FAMILY_DW_SIMT, tile_m=4, block_y=8, block_x=32, items_per_thread=4, vec_width=4, threads=128, unroll=2)
+    y = run_spec(spec, rec, a, ref, ref_elem=ref)
+    if off:
+        t, _ = W.device_tensors(spec, a)
+        import torch
+        x = torch.empty(t["x"].numel() + 4, device="cuda")[off:off + t["x"].numel()].view(t["x"].shape).copy_(t["x"])
+        wl = spec.workload()
+        wl.apply(rec)
+        wl.run(B.tensors(x, t["w"], t["bias"], t["residual"], t["y"]))
+        assert wl.status() == B.TT_OK
+        np.testing.assert_array_equal(t["y"].cpu().numpy(), y)
+        wl.close()
+    one = spec_for(1)
+    for i in {0, n - 1}:
+        alone = dict(a, x=np.ascontiguousarray(a["x"][i:i + 1]))
+        if n > 1:
+            np.testing.assert_array_equal(run_spec(one, rec, alone)[0], y[i])
+
+
 @pytest.mark.parametrize("k", [8, 22, 72, 136, 263, 1032])
 def test_ring_deeper_than_the_record(k):
     """One CTA per SM: the ring takes as many stages as fit, from one up to the kernel's limit, a CTA's whole reduction or a
