@@ -862,12 +862,19 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             for (int it = 0; it < iters; ++it) {
                 if (!mbar_wait(full0 + st * 8u, ph, abortp, g.status, 15u, g.wait_ns)) break;
                 const uint32_t hi = tiles_base + st * stage_bytes;
-                for (uint32_t off = 16u * (uint32_t)gt; off < lo_off; off += 16u * (uint32_t)kGatherThreads) {
-                    const float4 v = ld_shared_v4f(hi + off);
-                    st_shared_v4(hi + lo_off + off, v.x - __uint_as_float(__float_as_uint(v.x) & 0xFFFFE000u),
-                                 v.y - __uint_as_float(__float_as_uint(v.y) & 0xFFFFE000u),
-                                 v.z - __uint_as_float(__float_as_uint(v.z) & 0xFFFFE000u),
-                                 v.w - __uint_as_float(__float_as_uint(v.w) & 0xFFFFE000u));
+                constexpr uint32_t step = 16u * (uint32_t)kGatherThreads;
+                for (uint32_t off = 16u * (uint32_t)gt; off < lo_off; off += 4u * step) {      // four reads in flight
+                    float4 v[4];
+#pragma unroll
+                    for (uint32_t j = 0; j < 4u; ++j)
+                        if (off + j * step < lo_off) v[j] = ld_shared_v4f(hi + off + j * step);
+#pragma unroll
+                    for (uint32_t j = 0; j < 4u; ++j)
+                        if (off + j * step < lo_off)
+                            st_shared_v4(hi + lo_off + off + j * step, v[j].x - __uint_as_float(__float_as_uint(v[j].x) & 0xFFFFE000u),
+                                         v[j].y - __uint_as_float(__float_as_uint(v[j].y) & 0xFFFFE000u),
+                                         v[j].z - __uint_as_float(__float_as_uint(v[j].z) & 0xFFFFE000u),
+                                         v[j].w - __uint_as_float(__float_as_uint(v[j].w) & 0xFFFFE000u));
                 }
                 fence_proxy_async_shared();              // generic-proxy stores -> visible to the tensor core's reads
                 __syncwarp();

@@ -989,6 +989,19 @@ def test_mn_major_operands_and_tma_read_out(spec):
     probe.close()
 
 
+@pytest.mark.parametrize("m, k, n, tn, tk, sk", [(512, 1000, 1100, 64, 64, 4), (300, 200, 2000, 32, 128, 2), (1030, 520, 700, 16, 32, 3),
+                                                   (129, 68, 513, 128, 64, 1), (515, 260, 1030, 128, 128, 2), (700, 2052, 300, 64, 64, 8)])
+def test_compensated_tiles_of_twice_the_columns(m, k, n, tn, tk, sk):
+    """Compensated products whose tile runs with twice the record's columns, or whose one stage runs as several: remainders of
+    rows, columns and of the reduction, split over a cluster, on either axis."""
+    sp = W.Spec(B.TT_OP_DENSE, B.dense_shapes(m, k, n, True, B.TT_ACT_RELU), 1, "x3_wide", "bert")
+    a = W.make_inputs(sp, 97)
+    ref = util.oracle_ref(sp, a)
+    re = elem_ref(sp, a, ref)
+    for ax in (1, 2):
+        run_spec(sp, tc(tile_n=tn, tile_k=tk, stages=2, mma_m_axis=ax, split_k=sk, precision=1), a, ref, ref_elem=re)
+
+
 @pytest.mark.parametrize("n, c, h, w, r, stride, act, bias, off", [
     (5, 301, 14, 14, 5, 1, B.TT_ACT_RELU6, True, 0), (29, 190, 7, 7, 3, 1, B.TT_ACT_NONE, False, 0), (23, 47, 17, 18, 3, 2, B.TT_ACT_RELU, True, 0),
     (33, 33, 31, 30, 5, 2, B.TT_ACT_GELU_ERF, True, 0), (3, 9, 111, 109, 3, 1, B.TT_ACT_RELU, True, 0), (2, 11, 130, 131, 5, 1, B.TT_ACT_NONE, True, 0),
