@@ -48,7 +48,7 @@ CLASS_OF_OP = {0: "conv2d", 1: "depthwise", 2: "dense", 3: "batch_matmul", 4: "s
 def kernel_source_hash():
     import hashlib
     h = hashlib.sha256()
-    for name in ("tt_kernels.cu", "tt_internal.h"):
+    for name in ("tt_kernels.cu", "tt_conv.cu", "tt_ptx.cuh", "tt_internal.h"):
         with open(os.path.join(ROOT, "paper_2201_05587_b200", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]

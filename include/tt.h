@@ -92,7 +92,7 @@ typedef struct tt_shapes {
  *                accumulator's row loop)
  *   Fuse+Parallel -> the (tile_m x tile_n x split_k x batch) grid
  *   cache buffer / ComputeAt -> the accumulator lives in tensor memory and the bias/activation run on read-out;
- *                               `stages` shared-memory buffers decouple loading from the multiply
+ *                               `stages` shared-memory buffers (at least; more where memory is left over) decouple loading from the multiply
  *   Vectorize -> vec_width;   Unroll -> unroll / items_per_thread
  * GEMM_TC uses tile_m, tile_n, tile_k, stages, split_k, raster, mma_m_axis, slab_tiles, acc_split, k_order, persistent,
  *         cta_group, ctas_per_sm, warp_layout, precision.
@@ -116,8 +116,8 @@ typedef struct tt_schedule_record {
                               1 output rows (conv filters, dense/bmm rows m), 2 output columns (conv pixels, nn) */
     int32_t slab_tiles;    /* GEMM_TC, conv2d: reduction tiles served by one staging of the input rows in shared
                               memory (the cache buffer of the im2col operand); 0 = as many as fit.  Persistent form with a
-                              row-contiguous operand: boxes in that operand's staging ring, i.e. how much is in flight
-                              from memory; 0 = as many as fit, at most 8 */
+                              row-contiguous operand: how many stages of it are in flight from memory; 0 = as many as
+                              fit, at most 8 */
     int32_t acc_split;     /* GEMM_TC: independent accumulators in tensor memory (1, 2, 4 or 8; 0 = 1) to which the
                               8-wide reduction steps are dealt round-robin; they are added in fixed order on read-out.
                               Consecutive multiply-accumulates into one accumulator wait for each other; into several,
@@ -125,17 +125,17 @@ typedef struct tt_schedule_record {
     int32_t k_order;       /* GEMM_TC, conv2d: order in which the reduction (c, r, s) is walked.  0 = as the filters are
                               stored (channel-major; the im2col operand is expanded stage by stage).  1 = blocks of 32
                               channels, tap by tap inside a block: the filters are re-packed into that order by a small
-                              kernel (once per weight pointer: again only when tt_run sees other weights), the input rows are transposed once per block into a pixel-major
+                              kernel (once per weight pointer: again only when tt_run sees other weights), the input is transposed once per block into a pixel-major
                               slab, and every tap's operand tile is a shifted view of that slab -- no expansion.
-                              Stride-1 convolutions with 16-byte image rows, filters on the 128 rows, split_k = 1;
+                              Filters on the 128 rows, split_k = 1;
                               tile_k = 32 * (taps per pipeline stage), the tap count a divisor of r*s, at most 128. */
     int32_t persistent;    /* GEMM_TC: 1 = the grid is one CTA (or CTA pair) per SM and every CTA walks output tiles; the
                               operand pipeline runs on across tiles and two accumulators in tensor memory alternate, so a
                               tile is read out (bias, activation, stores) while the next one is accumulated.  Needs
                               split_k = 1 and operands that TMA can fetch: dense and batch_matmul with 16-byte rows, 1x1
                               stride-1 unpadded convolutions with h*w and c multiples of 4 (an operand whose row index is
-                              the contiguous one -- the image, the second operand of an NN batch_matmul -- is staged as
-                              [tile_k][rows] boxes and transposed in shared memory).  Elsewhere legalised to 0. */
+                              the contiguous one -- the image, the second operand of an NN batch_matmul -- is read as it
+                              lies).  Elsewhere legalised to 0. */
     int32_t cta_group;     /* GEMM_TC, persistent: 2 = two CTAs of a cluster share a 256-row tile; each loads its own rows of
                               the first operand and HALF of the second operand's rows, the multiply-accumulate runs across
                               both SMs (tcgen05 cta_group::2).  K-major operands only, tile_n >= 32.  0 or 1 = one CTA. */
@@ -144,7 +144,7 @@ typedef struct tt_schedule_record {
                               CTA's set-up and read-out overlap the other's main loop); 1 = all registers, one CTA per SM;
                               0 = the library's choice by grid size (2 when the grid has more than two CTAs per SM). */
     int32_t warp_layout;   /* GEMM_TC: warps by role.  0 = the only layout of each kernel form: 1 TMA + 1 MMA + 8 operand
-                              producers that then read out (320 threads), or, persistent, 1 TMA + 1 MMA + 4 transposers + 4
+                              producers that then read out (320 threads), or, persistent, 1 TMA + 1 MMA + 8
                               read-out warps.  Reserved for further layouts; any other value is invalid. */
     int32_t precision;     /* GEMM_TC: 0 = operands are read by the tensor core as TF32 (their fp32 values truncated to 10
                               mantissa bits).  1 = error-compensated ("3xTF32"): each operand tile is split in shared memory
