@@ -722,10 +722,10 @@ static long long plan_dw_boxes(DwArgs& d, int rows, int items) {
     d.plane_next = 0;
     const int gw = d.tile_w / items, gh = (d.tile_h + rows - 1) / rows;
     if (gw * gh <= 256) {
-        // one more 16-byte unit per row and the order of the lanes are free: take what the banks serve in the fewest turns, the wider row
+        // the order of the lanes is free, and so is one more 16-byte unit per row where that lies outside the image: take what the banks serve in the fewest turns, the wider row
         // only for a fifth fewer
         int best = 0, wide = 0;
-        for (int extra = 0; extra < 2; ++extra)
+        for (int extra = 0; extra < (d.tiles_w == 1 ? 2 : 1); ++extra)
             for (int order = 0; order < 2; ++order) {
                 const int bw4 = d.box_w / 4 + extra;
                 const int n = dw_read_wavefronts(gw, gh, d.tile_c, order != 0, items / 4 * d.sw, rows * d.sh * bw4, d.in_h * bw4);
@@ -760,7 +760,8 @@ static bool plan_dw_runs(const tt_workload* w, DwArgs& d, tt_apply_info& I) {
     t.runs = 1; t.tile_w = w->Q;
     t.vec = w->Q % 2 == 0 ? t.items : 1;
     const int lanes_q = (w->Q + t.items - 1) / t.items;    // threads of a strip row
-    const int upw = lanes_q <= 32 ? 32 / lanes_q : 0;      // strip rows a warp takes side by side
+    int upw = lanes_q <= 32 ? 32 / lanes_q : 0;            // strip rows a warp takes side by side ...
+    if (upw * lanes_q < 28) upw = 0;                       // ... unless that leaves more than an eighth of its lanes idle
     const int fit = upw ? 8 * upw : 256 / lanes_q;         // ... and 256 threads
     t.tile_h = w->P; t.tile_c = 1;
     if (hw * 4 > 24 * 1024) {
@@ -894,6 +895,10 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
         int stg = std::min(4, std::max(2, rec->stages));
         while (stg > 2 && stg * stage + 128 > kDynSmemLimit) --stg;
         if (t.box_w <= 256 && t.in_h <= 256 && t.tile_c <= 256 && stg * stage + 128 <= kDynSmemLimit && planes <= 0x7fffffffLL) {
+            // tiles keep to one image, in groups of channels as equal as they come
+            const int groups = (s.c + t.tile_c - 1) / t.tile_c;
+            t.tile_c = (s.c + groups - 1) / groups;
+            plan_dw_boxes(t, rows, items);
             d = t;
             d.window_rows = rows;
             if (stg != rec->stages) { if (strict) return TT_ERR_INVALID_SCHEDULE; I.changed |= TT_CHG_STAGES; }
@@ -901,11 +906,10 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
             d.tma_stages = stg;
             // no more threads than a tile has strips
             th = std::min(th, round_up(d.tile_c * ((d.tile_h + rows - 1) / rows) * (d.tile_w / items), 32));
-            d.tiles_p = (int)((planes + d.tile_c - 1) / d.tile_c);
-            const long long total = (long long)d.tiles_p * d.tiles_h * d.tiles_w;
+            const long long total = (long long)groups * s.n * d.tiles_h * d.tiles_w;
             if (total > 0x7fffffffLL) return TT_ERR_RESOURCE;
             d.total_tiles = (int)total;
-            smem = stg * stage + 128;
+            smem = (long long)stg * d.stage_bytes + d.wstage_bytes + 128;
             const long long per_sm = std::max<long long>(1, std::min<long long>(8, (228 * 1024) / (smem + 1024)));   // the launcher lowers it to what registers allow
             gx = std::min<long long>(total, 148 * per_sm);
             I.legal = L;

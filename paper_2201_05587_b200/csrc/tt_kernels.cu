@@ -1842,6 +1842,41 @@ __global__ void __launch_bounds__(256, WIDTH == 4 ? 6 : 4) tt_dwconv_window_kern
     }
 }
 
+// The tiles of the persistent depthwise kernels: (channel group, image, row tile, column tile).  A CTA keeps its channel group, and
+// with it the filters.  step > 0: CTA b has group b % groups and every step-th of its other coordinates, so that the CTAs work
+// on neighbouring planes at any time; step = 0: consecutive ranges of all tiles, counted groups first (the launcher's choice).
+struct DwTile { int ct, n, th, tw; };
+struct DwWalk { DwTile first; int count, s_n, s_th, s_tw; };
+__device__ __forceinline__ DwWalk dw_walk(const DwArgs& d) {
+    DwWalk w;
+    const int per_image = d.tiles_h * d.tiles_w, per_ct = d.N * per_image;
+    int j;
+    if (d.step) {
+        const int groups = (d.C + d.tile_c - 1) / d.tile_c;
+        j = (int)blockIdx.x / groups;
+        w.first.ct = (int)blockIdx.x - j * groups;
+        w.count = j < per_ct ? (per_ct - j + d.step - 1) / d.step : 0;
+        w.s_n = d.step / per_image;
+        const int rem = d.step - w.s_n * per_image;
+        w.s_th = rem / d.tiles_w; w.s_tw = rem - w.s_th * d.tiles_w;
+    } else {
+        const int t0 = (int)((long long)d.total_tiles * blockIdx.x / gridDim.x);
+        w.count = (int)((long long)d.total_tiles * (blockIdx.x + 1) / gridDim.x) - t0;
+        w.first.ct = t0 / per_ct;
+        j = t0 - w.first.ct * per_ct;
+        w.s_n = per_image == 1 ? 1 : 0; w.s_th = per_image > 1 && d.tiles_w == 1 ? 1 : 0; w.s_tw = d.tiles_w > 1 ? 1 : 0;
+    }
+    w.first.n = j / per_image; j -= w.first.n * per_image;
+    w.first.th = j / d.tiles_w; w.first.tw = j - w.first.th * d.tiles_w;
+    return w;
+}
+__device__ __forceinline__ void dw_next(const DwArgs& d, const DwWalk& w, DwTile& t) {
+    t.tw += w.s_tw; t.th += w.s_th; t.n += w.s_n;
+    if (t.tw >= d.tiles_w) { t.tw -= d.tiles_w; ++t.th; }
+    if (t.th >= d.tiles_h) { t.th -= d.tiles_h; ++t.n; }
+    if (t.n >= d.N && d.step == 0) { t.n = 0; ++t.ct; }
+}
+
 // ------------------------------------------------------------------------------------------------------------
 // DW_SIMT, TMA-staged persistent form (3x3 and 5x5 "same" filters, stride 1 or 2, image rows of 16-byte multiples).
 // The image is one 3-D tensor (W, H, planes = N * C).  A tile is tile_c consecutive planes x tile_h x tile_w
@@ -1851,15 +1886,15 @@ __global__ void __launch_bounds__(256, WIDTH == 4 ? 6 : 4) tt_dwconv_window_kern
 // limits the register-window kernel.  Threads work on ROWS x WIDTH strips exactly as there, reading the window rows
 // with aligned 16-byte shared-memory loads.  Same FMAs in the same order: bit-identical outputs.
 // The instruction stream per output is what bounds this kernel next to the memory system, so everything that does
-// not depend on the plane is hoisted: a thread keeps its strip position for the whole kernel, tile coordinates
-// advance by additions, and the filters and biases of a tile's planes are staged in shared memory (one buffer per
-// box buffer, [tile_c][WP] floats: filter, bias, padding) when the tile's box is requested.  They travel by cp.async on the
-// box's barrier: no thread waits for them (fetched through registers, a tile's refill held every thread up for a trip to L2).
+// not depend on the plane is hoisted: a thread keeps its strip position for the whole kernel, and the tiles are counted channels
+// first, so that a CTA meets new filters once or twice, mostly once: they stay in registers where a thread has one plane, else in a shared-memory buffer ([tile_c][WP] floats: filter, bias, padding).
 // A CTA has no more threads than a tile has strips, so more CTAs fit; the order of the lanes and the row pitch keep a warp's reads
-// off the same banks.  240 x 28 x 28, 5x5, 256 images: 109 -> 88 us (HBM 59), bound by issue: three instructions in five are products.
+// off the same banks.  240 x 28 x 28, 5x5, 256 images: 109 -> 85 us (HBM 59), bound by issue; 200 x 56 x 56, 5x5
+// stride 2, 32 images: 31 -> 23 (15); 16 images of 240 x 28 x 28, 5x5: 10.5 -> 9.7.  Stride 2 is compiled for one CTA per SM: its
+// strips need 95 registers, held to 64 they spilled (144 x 56 x 56, 3x3: 98 -> 92).
 // ------------------------------------------------------------------------------------------------------------
 template <int R, int STRIDE, int ROWS, int WIDTH>
-__global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constant__ CUtensorMap tmap_x, const DwArgs d) {
+__global__ void __launch_bounds__(256, STRIDE == 2 ? 1 : 0) tt_dwconv_tma_kernel(const __grid_constant__ CUtensorMap tmap_x, const DwArgs d) {
     constexpr int NCOL = (WIDTH - 1) * STRIDE + R;
     constexpr int IN_ROWS = (ROWS - 1) * STRIDE + R;
     constexpr int PAD = R / 2;
@@ -1870,11 +1905,11 @@ __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constan
     __shared__ uint64_t full_bar[4];
     __shared__ int abort_flag;
     const uint32_t base = (smem_u32(dw_raw) + 127u) & ~127u;
-    const uint32_t wbase = base + (uint32_t)d.tma_stages * (uint32_t)d.stage_bytes;
+    const uint32_t wst = base + (uint32_t)d.tma_stages * (uint32_t)d.stage_bytes;
     volatile int* abortp = &abort_flag;
     pdl_allow_next();
     if (threadIdx.x == 0) {
-        for (int s = 0; s < d.tma_stages; ++s) mbar_init(smem_u32(&full_bar[s]), blockDim.x + 1u);   // every thread's filter copies, and the box
+        for (int s = 0; s < d.tma_stages; ++s) mbar_init(smem_u32(&full_bar[s]), 1u);
         abort_flag = 0;
         fence_mbar_init();
         fence_proxy_async_shared();
@@ -1882,62 +1917,17 @@ __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constan
     }
     __syncthreads();
     pdl_wait_prev();                                      // the set-up above touched no global memory
-    const int planes = d.N * d.C;
-    const int per_plane_tiles = d.tiles_h * d.tiles_w;
-    const int my_tiles = d.total_tiles > (int)blockIdx.x ? (d.total_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    // Tile t = blockIdx.x + i * gridDim.x as (plane tile, row tile, column tile, first channel): decomposed once, then
-    // advanced by the decomposition of gridDim.x with carries -- no division per tile.
-    struct TilePos { int tp, th, tw, c0; };
-    int step_tp, step_th, step_tw, step_c;
-    {
-        const int gsz = (int)gridDim.x;
-        step_tp = gsz / per_plane_tiles;
-        const int rem = gsz - step_tp * per_plane_tiles;
-        step_th = rem / d.tiles_w; step_tw = rem - step_th * d.tiles_w;
-        step_c = (int)(((long long)step_tp * d.tile_c) % d.C);
-    }
-    const int tile_c_mod = d.tile_c % d.C;
-    auto first_pos = [&]() {
-        TilePos t;
-        const int b = (int)blockIdx.x;
-        t.tp = b / per_plane_tiles;
-        const int rem = b - t.tp * per_plane_tiles;
-        t.th = rem / d.tiles_w; t.tw = rem - t.th * d.tiles_w;
-        t.c0 = (int)(((long long)t.tp * d.tile_c) % d.C);
-        return t;
-    };
-    auto advance = [&](TilePos& t) {
-        t.tw += step_tw; t.th += step_th; t.tp += step_tp; t.c0 += step_c;
-        if (t.tw >= d.tiles_w) { t.tw -= d.tiles_w; ++t.th; }
-        if (t.th >= d.tiles_h) { t.th -= d.tiles_h; ++t.tp; t.c0 += tile_c_mod; }
-        while (t.c0 >= d.C) t.c0 -= d.C;
-    };
-    auto fill = [&](const TilePos& t, int s) {            // all threads: request a tile's box, filters and biases into buffer s
+    const DwWalk walk = dw_walk(d);
+    DwTile cur = walk.first;
+    auto fill = [&](const DwTile& t, int s) {               // thread 0: request a tile's box into buffer s
+        if (threadIdx.x != 0) return;
         const uint32_t bar = smem_u32(&full_bar[s]);
-        const int pl0 = t.tp * d.tile_c;
-        if (threadIdx.x == 0) {
-            mbar_expect_tx(bar, (uint32_t)(d.tile_c * d.in_h * d.box_w * 4));
-            tma_load_3d(base + (uint32_t)s * (uint32_t)d.stage_bytes, &tmap_x, bar, t.tw * d.tile_w * STRIDE - 4,
-                        t.th * d.tile_h * STRIDE - PAD, pl0);
-        }
-        const uint32_t dst = wbase + (uint32_t)s * (uint32_t)d.wstage_bytes;
-        for (int idx = (int)threadIdx.x; idx < d.tile_c * WP; idx += (int)blockDim.x) {
-            const int cl = idx / WP, k = idx - cl * WP;
-            int c = t.c0 + cl;                            // tile_c <= C: one subtraction wraps it
-            if (c >= d.C) c -= d.C;
-            const bool filter = k < R * R, have = pl0 + cl < planes && (filter || (k == R * R && d.bias));
-            cp_async_4_or_zero(dst + 4u * (uint32_t)idx, !have ? d.w : filter ? d.w + c * (R * R) + k : d.bias + c, have);
-        }
-        cp_async_arrive(bar);
+        mbar_expect_tx(bar, (uint32_t)(d.tile_c * d.in_h * d.box_w * 4));
+        tma_load_3d(base + (uint32_t)s * (uint32_t)d.stage_bytes, &tmap_x, bar, t.tw * d.tile_w * STRIDE - 4,
+                    t.th * d.tile_h * STRIDE - PAD, t.n * d.C + t.ct * d.tile_c);
     };
-    TilePos cur = first_pos(), nxt = cur;
-    {
-        const int pre = min(my_tiles, d.tma_stages);
-        for (int i = 0; i < pre; ++i) {
-            fill(nxt, i);
-            advance(nxt);
-        }
-    }
+    DwTile ahead = cur;
+    for (int i = 0; i < min(walk.count, d.tma_stages); ++i) { fill(ahead, i); dw_next(d, walk, ahead); }
     // a thread's strip position inside a plane is fixed for the whole kernel when a plane has at most blockDim strips
     // (the thread then walks planes cl_f, cl_f + cpp, ...); otherwise it also walks strips
     const int groups_w = d.tile_w / WIDTH;
@@ -1963,15 +1953,36 @@ __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constan
     const long long plane_out = (long long)d.P * d.Q;
     const bool clamp = d.act == TT_ACT_RELU || d.act == TT_ACT_RELU6, gelu = d.act == TT_ACT_GELU_ERF;
     const float hi = d.act == TT_ACT_RELU6 ? 6.f : INFINITY;
-    int s = 0;
+    const bool keep = d.tile_c <= cpp;                    // one plane per thread: its filter stays in registers
+    float wv[WP];
+    int s = 0, have_ct = -1;
     uint32_t ph = 0;
-    for (int i = 0; i < my_tiles; ++i) {
+    for (int i = 0; i < walk.count; ++i) {
+        const int c0 = cur.ct * d.tile_c, ncl = min(d.tile_c, d.C - c0);
+        if (cur.ct != have_ct) {                          // the same for every thread
+            have_ct = cur.ct;
+            if (keep) {
+                if (cl_f < ncl) {
+                    const float* w = d.w + (long long)(c0 + cl_f) * (R * R);
+#pragma unroll
+                    for (int k = 0; k < R * R; ++k) wv[k] = __ldg(w + k);
+                    wv[R * R] = d.bias ? __ldg(d.bias + c0 + cl_f) : 0.f;
+                }
+            } else {                                      // (the barrier after the last tile has passed)
+                for (int idx = (int)threadIdx.x; idx < ncl * WP; idx += (int)blockDim.x) {
+                    const int cl = idx / WP, k = idx - cl * WP;
+                    float v = 0.f;
+                    if (k < R * R) v = __ldg(d.w + (long long)(c0 + cl) * (R * R) + k);
+                    else if (k == R * R && d.bias) v = __ldg(d.bias + c0 + cl);
+                    st_shared_f32(wst + 4u * (uint32_t)idx, v);
+                }
+                __syncthreads();
+            }
+        }
         // every thread waits for the box itself (all take the same decision: the same barrier and phase)
         if (!mbar_wait(smem_u32(&full_bar[s]), ph, abortp, d.status, 9u, d.wait_ns)) break;
-        const int pl0 = cur.tp * d.tile_c, p0 = cur.th * d.tile_h, q0 = cur.tw * d.tile_w;
-        const int ncl = min(d.tile_c, planes - pl0);
+        const int pl0 = cur.n * d.C + c0, p0 = cur.th * d.tile_h, q0 = cur.tw * d.tile_w;
         const uint32_t stage = base + (uint32_t)s * (uint32_t)d.stage_bytes;
-        const uint32_t wst = wbase + (uint32_t)s * (uint32_t)d.wstage_bytes;
         for (int sidx = s_f; active && sidx < spp; sidx += s_step) {
             int gh = gh_f, gwi = gwi_f;
             if (sidx != s_f) { gh = sidx / groups_w; gwi = sidx - gh * groups_w; }
@@ -1984,11 +1995,12 @@ __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constan
             float* __restrict__ y0 = d.y + ((long long)pl0 * d.P + p) * (long long)d.Q + q;
 #pragma unroll 1
             for (int cl = cl_f; cl < ncl; cl += cpp) {
-                float wv[WP];
+                if (!keep) {
 #pragma unroll
-                for (int k = 0; k < WP / 4; ++k) {
-                    const float4 f = ld_shared_v4f(wst + 4u * (uint32_t)(cl * WP + 4 * k));
-                    wv[4 * k] = f.x; wv[4 * k + 1] = f.y; wv[4 * k + 2] = f.z; wv[4 * k + 3] = f.w;
+                    for (int k = 0; k < WP / 4; ++k) {
+                        const float4 f = ld_shared_v4f(wst + 4u * (uint32_t)(cl * WP + 4 * k));
+                        wv[4 * k] = f.x; wv[4 * k + 1] = f.y; wv[4 * k + 2] = f.z; wv[4 * k + 3] = f.w;
+                    }
                 }
                 float acc[ROWS][WIDTH];
 #pragma unroll
@@ -2042,15 +2054,11 @@ __global__ void __launch_bounds__(256) tt_dwconv_tma_kernel(const __grid_constan
                 }
             }
         }
-        __syncthreads();                                  // everyone is done with this box and its weight buffer
-        if (i + d.tma_stages < my_tiles) {
-            fill(nxt, s);
-            advance(nxt);
-        }
-        advance(cur);
+        __syncthreads();                                  // everyone is done with this box
+        if (i + d.tma_stages < walk.count) { fill(ahead, s); dw_next(d, walk, ahead); }
+        dw_next(d, walk, cur);
         if (++s == d.tma_stages) { s = 0; ph ^= 1u; }
     }
-    cp_async_wait_all();
     // after a tripped wait: let the boxes still in flight land before the shared memory is given back (bounded)
     if (threadIdx.x == 0 && *abortp) {
         for (int b = 0; b < d.tma_stages; ++b) {
@@ -2103,23 +2111,14 @@ __global__ void __launch_bounds__(256, R == 5 && STRIDE == 1 && WIDTH == 2 ? 2 :
     const int HW = d.H * d.W;
     const long long all = (long long)d.N * d.C * HW;
     const bool whole = d.tiles_h == 1;                    // tiles of whole planes; otherwise of a band of one plane
-    const int per_ct = d.N * d.tiles_h;                   // tiles of one group of tile_c channels
-    const int t0 = (int)((long long)d.total_tiles * blockIdx.x / gridDim.x), t1 = (int)((long long)d.total_tiles * (blockIdx.x + 1) / gridDim.x);
-    struct Tile { int ct, n, th; };
-    auto next = [&](Tile& t) {
-        if (++t.th < d.tiles_h) return;
-        t.th = 0;
-        if (++t.n < d.N) return;
-        t.n = 0; ++t.ct;
-    };
-    Tile cur;
-    cur.ct = t0 / per_ct; cur.th = t0 - cur.ct * per_ct; cur.n = cur.th / d.tiles_h; cur.th -= cur.n * d.tiles_h;
+    const DwWalk walk = dw_walk(d);
+    DwTile cur = walk.first;
     // the run's first float and first image row
-    auto start_of = [&](const Tile& t, int& row0) {
+    auto start_of = [&](const DwTile& t, int& row0) {
         row0 = whole ? 0 : max(0, t.th * d.tile_h * STRIDE - PAD);
         return ((long long)t.n * d.C + t.ct * d.tile_c) * HW + row0 * d.W;
     };
-    auto fill = [&](const Tile& t, int s) {
+    auto fill = [&](const DwTile& t, int s) {
         if (d.vec_in && threadIdx.x != 0) return;
         int row0;
         const long long start = start_of(t, row0), first = start & ~3LL;
@@ -2136,8 +2135,8 @@ __global__ void __launch_bounds__(256, R == 5 && STRIDE == 1 && WIDTH == 2 ? 2 :
         if (!d.vec_in) for (long long e = start + (int)threadIdx.x; e < end; e += (int)blockDim.x) cp_async_4(dst + 4u * (uint32_t)(e - first), d.x + e);
         cp_async_arrive(bar);
     };
-    Tile ahead = cur;
-    for (int i = 0; i < min(t1 - t0, d.tma_stages); ++i) { fill(ahead, i); next(ahead); }
+    DwTile ahead = cur;
+    for (int i = 0; i < min(walk.count, d.tma_stages); ++i) { fill(ahead, i); dw_next(d, walk, ahead); }
     // This thread's column q of strip row gh (and gh + strip_rows, ...) of plane pl.  A unit is one strip row of one plane: Q columns.
     // Narrow images put `units_per_warp` of them side by side in a warp, either consecutive ones or ones `unit_far` apart,
     // whichever spreads the reads over more banks; wide ones run on through the warps.
@@ -2168,7 +2167,7 @@ __global__ void __launch_bounds__(256, R == 5 && STRIDE == 1 && WIDTH == 2 ? 2 :
     float wv[R * R], bias = 0.f;
     int s = 0, have_ct = -1;
     uint32_t ph = 0;
-    for (int i = 0; i < t1 - t0; ++i) {
+    for (int i = 0; i < walk.count; ++i) {
         const int c = cur.ct * d.tile_c + pl;             // this thread's channel
         const bool mine = active && c < d.C;
         if (cur.ct != have_ct && mine) {
@@ -2246,8 +2245,8 @@ __global__ void __launch_bounds__(256, R == 5 && STRIDE == 1 && WIDTH == 2 ? 2 :
             }
         }
         __syncthreads();                                  // everyone is done with this run
-        if (i + d.tma_stages < t1 - t0) { fill(ahead, s); next(ahead); }
-        next(cur);
+        if (i + d.tma_stages < walk.count) { fill(ahead, s); dw_next(d, walk, ahead); }
+        dw_next(d, walk, cur);
         if (++s == d.tma_stages) { s = 0; ph ^= 1u; }
     }
     cp_async_wait_all();
@@ -2622,7 +2621,20 @@ struct ResidentCtas {
     }
 };
 
-cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st) {
+// CTAs per channel group; 0: consecutive ranges.  Whole planes are runs of memory of their own and go by ranges, which use every CTA.
+// Bands of planes (two tiles and more a plane) lose the memory's locality that way (256 images of 144 x 56 x 56, 3x3: 173 us
+// against 154), so there the CTAs keep to neighbouring planes, unless whole groups leave more than an eighth of them idle.
+static int dw_step(int ctas, int groups, long long per_group) {
+    const long long m = std::min<long long>(ctas / groups, per_group);
+    if (m < 1) return 0;
+    const long long rounds = (per_group + m - 1) / m;
+    return 8 * groups * per_group >= 7 * rounds * ctas ? (int)m : 0;
+}
+
+cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& args, const void* tmap_x, cudaStream_t st) {
+    DwArgs dw = args;
+    const int groups = (dw.C + dw.tile_c - 1) / dw.tile_c;
+    const long long per_group = (long long)dw.N * dw.tiles_h * dw.tiles_w;
     CUtensorMap tx;
     if (tmap_x) memcpy(&tx, tmap_x, sizeof tx); else memset(&tx, 0, sizeof tx);
     dim3 grid(I.grid_x, 1, 1);
@@ -2637,6 +2649,8 @@ cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& dw, const voi
         if (e != cudaSuccess) return e; \
         /* persistent CTAs: never more than are resident at once (registers may allow fewer than shared memory does) */ \
         grid.x = (unsigned)std::min<long long>(grid.x, resident); \
+        dw.step = dw.tiles_h * dw.tiles_w > 1 ? dw_step((int)grid.x, groups, per_group) : 0; \
+        if (dw.step) grid.x = (unsigned)(dw.step * groups); \
         return launch_serialized(KERNEL, grid, (unsigned)I.threads, (size_t)I.smem_bytes, st, __VA_ARGS__); }
 #define TT_DWT_BOX(RR, SS, RO, WI) \
     if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == WI) TT_DWT_CASE((tt_dwconv_tma_kernel<RR, SS, RO, WI>), tx, dw)
