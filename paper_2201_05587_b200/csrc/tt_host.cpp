@@ -713,8 +713,8 @@ static int dw_read_wavefronts(int groups_w, int groups_h, int planes, bool plane
 }
 
 // Geometry of the staged persistent kernel for a tile of d.tile_c planes x d.tile_h x d.tile_w outputs in strips of `rows` x `items`:
-// box, buffers, the lanes' order.  Returns the bytes of one stage.
-static long long plan_dw_boxes(DwArgs& d, int rows, int items) {
+// box, buffers, the lanes' order.  may_widen: a row may take one more 16-byte unit than it needs.
+static void plan_dw_boxes(DwArgs& d, int rows, int items, bool may_widen) {
     const int ncol = (items - 1) * d.sw + d.S, nld = (4 - d.pw + ncol + 3) / 4;      // 16-byte loads per window row
     // strips are `rows` tall: the box covers the rows of the last, possibly partial, strip too
     d.in_h = (round_up(d.tile_h, rows) - 1) * d.sh + d.R;
@@ -725,7 +725,7 @@ static long long plan_dw_boxes(DwArgs& d, int rows, int items) {
         // the order of the lanes is free, and so is one more 16-byte unit per row where that lies outside the image: take what the banks serve in the fewest turns, the wider row
         // only for a fifth fewer
         int best = 0, wide = 0;
-        for (int extra = 0; extra < (d.tiles_w == 1 ? 2 : 1); ++extra)
+        for (int extra = 0; extra < (may_widen && d.tiles_w == 1 ? 2 : 1); ++extra)
             for (int order = 0; order < 2; ++order) {
                 const int bw4 = d.box_w / 4 + extra;
                 const int n = dw_read_wavefronts(gw, gh, d.tile_c, order != 0, items / 4 * d.sw, rows * d.sh * bw4, d.in_h * bw4);
@@ -735,7 +735,6 @@ static long long plan_dw_boxes(DwArgs& d, int rows, int items) {
     }
     d.stage_bytes = (int)std::min<long long>(0x7fffff80, (((long long)d.tile_c * d.in_h * d.box_w * 4) + 127) / 128 * 128);
     d.wstage_bytes = (int)((((long long)d.tile_c * round_up(d.R * d.S + 1, 4) * 4) + 127) / 128 * 128);
-    return (long long)d.stage_bytes + d.wstage_bytes;
 }
 
 // Image rows that are no 16-byte multiples: no box can fetch them, and a register-window strip fetches each value of its rows
@@ -890,15 +889,19 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
         // strip then reads 11 rows for 7, not 8 for 4 (3x3: 9 for 7 against 6 for 4, and it was slower on 56-pixel rows, 157 -> 173 us)
         int rows = window_rows;
         if (rows == 4 && s.r == 5 && round_up(d.tile_h, 7) <= round_up(d.tile_h, 4) && (planes + d.tile_c - 1) / d.tile_c * d.tiles_h * d.tiles_w >= 148 * 4) rows = 7;
+        // tiles keep to one image, in groups of channels as equal as they come; everything below is about the tile that runs
         DwArgs t = d;
-        const long long stage = plan_dw_boxes(t, rows, items);
-        int stg = std::min(4, std::max(2, rec->stages));
-        while (stg > 2 && stg * stage + 128 > kDynSmemLimit) --stg;
-        if (t.box_w <= 256 && t.in_h <= 256 && t.tile_c <= 256 && stg * stage + 128 <= kDynSmemLimit && planes <= 0x7fffffffLL) {
-            // tiles keep to one image, in groups of channels as equal as they come
-            const int groups = (s.c + t.tile_c - 1) / t.tile_c;
-            t.tile_c = (s.c + groups - 1) / groups;
-            plan_dw_boxes(t, rows, items);
+        const int groups = (s.c + t.tile_c - 1) / t.tile_c;
+        t.tile_c = (s.c + groups - 1) / groups;
+        int stg = 0;
+        auto smem_of = [&](int n) { return (long long)n * t.stage_bytes + t.wstage_bytes + 128; };
+        for (const bool may_widen : {true, false}) {       // (a wider row that does not fit is no reason to leave this form)
+            plan_dw_boxes(t, rows, items, may_widen);
+            stg = std::min(4, std::max(2, rec->stages));
+            while (stg > 2 && smem_of(stg) > kDynSmemLimit) --stg;
+            if (smem_of(stg) <= kDynSmemLimit && t.box_w <= 256) break;
+        }
+        if (t.box_w <= 256 && t.in_h <= 256 && t.tile_c <= 256 && smem_of(stg) <= kDynSmemLimit && planes <= 0x7fffffffLL) {
             d = t;
             d.window_rows = rows;
             if (stg != rec->stages) { if (strict) return TT_ERR_INVALID_SCHEDULE; I.changed |= TT_CHG_STAGES; }
@@ -909,7 +912,7 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
             const long long total = (long long)groups * s.n * d.tiles_h * d.tiles_w;
             if (total > 0x7fffffffLL) return TT_ERR_RESOURCE;
             d.total_tiles = (int)total;
-            smem = (long long)stg * d.stage_bytes + d.wstage_bytes + 128;
+            smem = smem_of(stg);
             const long long per_sm = std::max<long long>(1, std::min<long long>(8, (228 * 1024) / (smem + 1024)));   // the launcher lowers it to what registers allow
             gx = std::min<long long>(total, 148 * per_sm);
             I.legal = L;

@@ -589,3 +589,31 @@ def test_run_chain_checks_its_arguments(lanes, waits, want):
     at = ctypes.c_size_t(99)
     assert B.lib().tt_run_chain(steps, 2, (ctypes.c_void_p * 2)(), 2, ctypes.byref(at)) == want
     assert at.value == (0 if want == B.TT_ERR_NOT_APPLIED else 1)
+
+
+DYN_SMEM_LIMIT = 227 * 1024 - 6144      # dynamic shared memory a CTA may ask for beside its barriers
+
+
+def test_depthwise_plans_fit_shared_memory():
+    """A record that is accepted never asks for more shared memory than a launch can have: boxes whose channel groups are
+    evened out (38 for 40 of 301 channels, 46 for 48 of 504) and whose rows are then widened, and a sweep of the like."""
+    import random
+    rng = random.Random(5)
+    cases = [((16, 301, 114, 16, 5, 2), (40, 12, 256, 2, 2)), ((47, 504, 11, 16, 5, 1), (48, 16, 16, 2, 2))]
+    for _ in range(3000):
+        r = rng.choice((3, 5))
+        cases.append(((rng.randint(1, 48), rng.randint(1, 520), rng.randint(r, 120), 4 * rng.randint(2, 30), r, rng.choice((1, 2))),
+                      (rng.randint(1, 64), rng.randint(1, 56), rng.choice((8, 16, 28, 32, 56, 112, 256)), rng.choice((1, 2, 4)), rng.randint(2, 4))))
+    boxes = 0
+    for (n, c, h, w, r, st), (tc_, by, bx, un, sg) in cases:
+        wl = B.Workload(B.TT_OP_DWCONV2D, B.make_shapes(n=n, c=c, h=h, w=w, k=c, r=r, s=r, stride_h=st, stride_w=st, pad_h=r // 2, pad_w=r // 2,
+                                                        has_bias=1, act=B.TT_ACT_RELU), "dw")
+        rec = B.make_record(B.TT_FAMILY_DW_SIMT, tile_m=tc_, block_y=by, block_x=bx, items_per_thread=4, vec_width=1, threads=256, unroll=un,
+                            raster=1, stages=sg)
+        status, info = wl.check(rec)
+        assert status in (B.TT_OK, B.TT_ERR_RESOURCE)
+        if status == B.TT_OK:
+            assert info.smem_bytes <= DYN_SMEM_LIMIT, ((n, c, h, w, r, st), rec.short(), info.smem_bytes)
+            boxes += info.legal.raster
+        wl.close()
+    assert boxes > 1000
