@@ -250,7 +250,11 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
 static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, Plan* plan) {
     if (rec->k_order < 0 || rec->k_order > 1) return TT_ERR_INVALID_SCHEDULE;
     if (rec->k_order == 1) {
-        if (tap_major_possible(w)) return legalise_conv_tapmajor(w, rec, mode, plan);
+        if (tap_major_possible(w)) {
+            // (rows so wide that the taps' slab of positions exceeds shared memory are walked in the stored order)
+            const tt_status st = legalise_conv_tapmajor(w, rec, mode, plan);
+            if (st != TT_ERR_RESOURCE || mode == TT_MODE_STRICT) return st;
+        }
         if (mode == TT_MODE_STRICT) return TT_ERR_INVALID_SCHEDULE;       // no such reduction order on this kernel
     }
     tt_apply_info& I = plan->info;

@@ -617,3 +617,27 @@ def test_depthwise_plans_fit_shared_memory():
             boxes += info.legal.raster
         wl.close()
     assert boxes > 1000
+
+
+@pytest.mark.parametrize("shape", [
+    # n, c, h, w, k, r, stride, residual: rows beyond what the taps' slab can hold
+    (2, 8, 5, 1025, 16, 3, 1, 0), (3, 2, 40, 2000, 8, 5, 2, 0), (2, 32, 64, 1028, 64, 3, 1, 1), (4, 8, 9, 701, 24, 5, 1, 0), (1, 8, 9, 1200, 24, 3, 1, 0),
+])
+def test_tap_major_records_on_wide_images_run_in_the_stored_order(shape):
+    """A record that names the tap-major order applies wherever the same record in the stored order does."""
+    n, c, h, w, k, r, stride, res = shape
+    wl = B.Workload(B.TT_OP_CONV2D, B.make_shapes(n=n, c=c, h=h, w=w, k=k, r=r, s=r, stride_h=stride, stride_w=stride, pad_h=r // 2, pad_w=r // 2,
+                                                  has_bias=1, has_residual=res, act=B.TT_ACT_RELU), "wide")
+    for tn, tk, stages in ((16, 32, 1), (64, 32, 2), (128, 96, 2)):
+        stored = B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tn, tile_k=tk, stages=stages, mma_m_axis=1)
+        tap = B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tn, tile_k=tk, stages=stages, k_order=1, mma_m_axis=1)
+        st0, i0 = wl.check(stored)
+        st1, i1 = wl.check(tap)
+        assert st1 == st0
+        if st0 != B.TT_OK:                               # the stored order's own rows do not fit either
+            assert tn > 16
+            continue
+        assert i1.legal.k_order == 0 and i1.changed & B.TT_CHG_KORDER and i1.launches == 1
+        assert bytes(i1.legal) == bytes(i0.legal) and (i1.grid_x, i1.grid_z, i1.smem_bytes) == (i0.grid_x, i0.grid_z, i0.smem_bytes)
+        assert wl.check(tap, mode=B.TT_MODE_STRICT)[0] != B.TT_OK
+    wl.close()
