@@ -133,9 +133,6 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     const int tk = 32 * tps;
     if (strict && (rec->mma_m_axis == 2 || rec->tile_k != tk || rec->split_k != 1)) return TT_ERR_INVALID_SCHEDULE;
     L.mma_m_axis = 1; L.tile_m = kHwTileM; L.tile_k = tk; L.split_k = 1; L.acc_split = 1; L.slab_tiles = 0; L.k_order = 1;
-    if (rec->persistent < 0 || rec->persistent > 1 || rec->cta_group < 0 || rec->cta_group > 2 || rec->ctas_per_sm < 0 ||
-        rec->ctas_per_sm > 2 || rec->warp_layout != 0 || rec->precision < 0 || rec->precision > 1)
-        return TT_ERR_INVALID_SCHEDULE;
     // (one kernel serves both forms: its CTAs always walk; CTA pairs do not exist here)
     const bool persistent = rec->persistent == 1;
     L.persistent = persistent ? 1 : 0; L.cta_group = 1; L.ctas_per_sm = 1;
@@ -248,7 +245,13 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
 }
 
 static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, Plan* plan) {
-    if (rec->k_order < 0 || rec->k_order > 1) return TT_ERR_INVALID_SCHEDULE;
+    // nonsense is refused whatever the kernel and the reduction order
+    if (rec->tile_m <= 0 || rec->tile_n <= 0 || rec->tile_k <= 0 || rec->stages <= 0 || rec->split_k <= 0 ||
+        rec->raster < 0 || rec->raster > 1 || rec->mma_m_axis < 0 || rec->mma_m_axis > 2 || rec->persistent < 0 ||
+        rec->persistent > 1 || rec->cta_group < 0 || rec->cta_group > 2 || rec->ctas_per_sm < 0 || rec->ctas_per_sm > 2 ||
+        rec->acc_split < 0 || rec->k_order < 0 || rec->k_order > 1 || rec->warp_layout != 0 || rec->precision < 0 || rec->precision > 1 ||
+        (w->op == TT_OP_CONV2D && rec->slab_tiles < 0))
+        return TT_ERR_INVALID_SCHEDULE;
     if (rec->k_order == 1) {
         if (tap_major_possible(w)) {
             // (rows so wide that the taps' slab of positions exceeds shared memory are walked in the stored order)
@@ -261,11 +264,6 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     tt_schedule_record L = *rec;
     int changed = 0;
     const bool strict = mode == TT_MODE_STRICT;
-    if (rec->tile_m <= 0 || rec->tile_n <= 0 || rec->tile_k <= 0 || rec->stages <= 0 || rec->split_k <= 0 ||
-        rec->raster < 0 || rec->raster > 1 || rec->mma_m_axis < 0 || rec->mma_m_axis > 2 || rec->persistent < 0 ||
-        rec->persistent > 1 || rec->cta_group < 0 || rec->cta_group > 2 || rec->ctas_per_sm < 0 || rec->ctas_per_sm > 2 ||
-        rec->warp_layout != 0 || rec->precision < 0 || rec->precision > 1)
-        return TT_ERR_INVALID_SCHEDULE;
     // Which output axis becomes the accumulator's 128 rows.  Left to the library (0), the shorter-than-a-tile
     // axis goes to the MMA's N side, where 16..256 columns are legal.
     tt_shapes s = w->sh;                                  // a copy: a pointwise convolution is re-viewed below
@@ -340,7 +338,6 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     if (sk != rec->split_k) changed |= TT_CHG_SPLIT_K;
     L.split_k = sk;
     // accumulators: a power of two, all of them inside the 512 columns of tensor memory, none left without a step
-    if (rec->acc_split < 0) return TT_ERR_INVALID_SCHEDULE;
     int nacc = (persistent || x3) ? 1 : std::min(8, pow2_floor(std::max(1, rec->acc_split)));
     while (nacc > 1 && (nacc * tn > 512 || (long long)nacc > (long long)per_split * (tk / 8))) nacc >>= 1;
     if (nacc != std::max(1, rec->acc_split)) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_ACC; }
@@ -363,8 +360,8 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         const bool a_mn = swap ? v_mn : u_mn, b_mn = swap ? u_mn : v_mn;
         // How many stages: the record's, or, with a row-contiguous operand (whose boxes come from memory one after the other),
         // what the record field slab_tiles asks for; 0 = as many as fit, at most 8.
-        if (rec->slab_tiles < 0) return TT_ERR_INVALID_SCHEDULE;
         const bool mn = a_mn || b_mn;
+        if (mn && rec->slab_tiles < 0) return TT_ERR_INVALID_SCHEDULE;
         const long long stage = (long long)a_stage + b_stage;
         // Read-out staging: eight warps with three (a residual passes through them) or two 32 x 32 blocks each, fewer where
         // the record's stages need the room; never less than four warps with one block (5 KB, the width the unaligned
@@ -480,14 +477,13 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     const long long red_bytes = cluster ? (4 * std::max<long long>((long long)(sk - 1) * ((kHwTileM + sk - 1) / sk) * (tn + 4),
                                                                     (long long)(sk - 1) * ((tn + sk - 1) / sk) * kHwTileM) + 127) / 128 * 128 : 0;
     // A pointwise convolution on images of 16-byte multiples needs no slab: its pixels are an MN-major operand.
+    if (strict && w->op == TT_OP_CONV2D && rec->slab_tiles > per_split) return TT_ERR_INVALID_SCHEDULE;
     const bool conv = w->op == TT_OP_CONV2D && !mn_operand;
     const long long ktab = conv ? (((long long)per_split * tk * 4 + 127) / 128) * 128 : 0;
     int sl_tiles = 0, sl_nbuf = 0, sl_wp = 0, sl_gap = 0, sl_chpitch = 0, sl_in_rows = 0, sl_rstep = 1;
     long long sl_buf_bytes = 0, chp = 0;
     const int RS = conv ? s.r * s.s : 1;
     if (conv) {
-        if (rec->slab_tiles < 0) return TT_ERR_INVALID_SCHEDULE;
-        if (strict && rec->slab_tiles > per_split) return TT_ERR_INVALID_SCHEDULE;
         const int pix_rows = swap ? kHwTileM : tn;       // output pixels per tile of the im2col operand
         // A pointwise convolution (1x1, stride 1, no padding) sees no neighbourhood: its H x W pixels are one run of
         // H*W values per channel, and any H' x W' with the same product is the same kernel.  Rows of W' pixels with

@@ -641,3 +641,24 @@ def test_tap_major_records_on_wide_images_run_in_the_stored_order(shape):
         assert bytes(i1.legal) == bytes(i0.legal) and (i1.grid_x, i1.grid_z, i1.smem_bytes) == (i0.grid_x, i0.grid_z, i0.smem_bytes)
         assert wl.check(tap, mode=B.TT_MODE_STRICT)[0] != B.TT_OK
     wl.close()
+
+
+def test_nonsense_fields_are_refused_in_every_reduction_order():
+    tap, pointwise, dense = W._conv(64, 28, 64, 3, 1, 1).workload(), W._conv(64, 28, 64, 1, 1, 0).workload(), W._dense(64, 128, 96).workload()
+    base = dict(tile_n=64, tile_k=32, stages=2, mma_m_axis=1)
+    nonsense = [dict(tile_m=0), dict(tile_n=-16), dict(tile_k=0), dict(stages=-3), dict(stages=0), dict(split_k=0), dict(raster=7), dict(raster=-1),
+                dict(mma_m_axis=3), dict(acc_split=-1), dict(persistent=2), dict(ctas_per_sm=3), dict(warp_layout=1), dict(precision=2)]
+    for wl in (tap, pointwise, dense):
+        for order in (0, 1):
+            assert wl.check(B.make_record(B.TT_FAMILY_GEMM_TC, **dict(base, k_order=order)))[0] == B.TT_OK
+            for bad in nonsense:
+                for mode in (B.TT_MODE_LEGALISE, B.TT_MODE_STRICT):
+                    rec = B.make_record(B.TT_FAMILY_GEMM_TC, **dict(base, k_order=order, **{k: v for k, v in bad.items() if k not in base}))
+                    for k, v in bad.items():
+                        setattr(rec, k, v)
+                    assert wl.check(rec, mode=mode)[0] == B.TT_ERR_INVALID_SCHEDULE, (order, bad, mode)
+    # a convolution's slab of input rows, whether or not this layer stages one; a dense layer has none
+    rec = B.make_record(B.TT_FAMILY_GEMM_TC, slab_tiles=-1, **base)
+    assert [wl.check(rec)[0] for wl in (tap, pointwise, dense)] == [B.TT_ERR_INVALID_SCHEDULE, B.TT_ERR_INVALID_SCHEDULE, B.TT_OK]
+    rec = B.make_record(B.TT_FAMILY_GEMM_TC, slab_tiles=3, **base)           # (64 channels are two reduction tiles)
+    assert pointwise.check(rec, mode=B.TT_MODE_STRICT)[0] == B.TT_ERR_INVALID_SCHEDULE
