@@ -400,7 +400,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         I.threads = kGemmThreads;
         // one CTA per SM: ask for more than half of an SM's shared memory
         I.smem_bytes = (int)std::max<long long>(smem_p, 116 * 1024);
-        I.tmem_cols = std::max(32, pow2_ceil(2 * tn));
+        I.tmem_cols = std::max(32, pow2_ceil(tn + round_up(tn, 32)));     // (the read-out takes whole blocks of 32 columns)
         I.workspace_bytes = 0; I.launches = 1;
         plan->partial_bytes = 0;
         if (smem_p > kDynSmemLimit) return TT_ERR_RESOURCE;
@@ -549,7 +549,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     } else {
         L.slab_tiles = 0;
     }
-    int tmem_cols = std::max(32, pow2_ceil(nacc * tn));
+    int tmem_cols = std::max(32, pow2_ceil((nacc - 1) * tn + round_up(tn, 32)));     // (the read-out takes whole blocks of 32 columns)
     const int tiles_m = (M + kHwTileM - 1) / kHwTileM, tiles_n = (N + tn - 1) / tn;
     if ((long long)tiles_m * tiles_n > 0x7fffffffLL || sk > 65535 || B > 65535) return TT_ERR_RESOURCE;
 

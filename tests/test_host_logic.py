@@ -662,3 +662,16 @@ def test_nonsense_fields_are_refused_in_every_reduction_order():
     assert [wl.check(rec)[0] for wl in (tap, pointwise, dense)] == [B.TT_ERR_INVALID_SCHEDULE, B.TT_ERR_INVALID_SCHEDULE, B.TT_OK]
     rec = B.make_record(B.TT_FAMILY_GEMM_TC, slab_tiles=3, **base)           # (64 channels are two reduction tiles)
     assert pointwise.check(rec, mode=B.TT_MODE_STRICT)[0] == B.TT_ERR_INVALID_SCHEDULE
+
+
+@pytest.mark.parametrize("tn", range(16, 257, 16))
+def test_tensor_memory_covers_what_the_read_out_reads(tn):
+    """The read-out takes 32 columns at a time, also from the last accumulator: the last block of a tile whose columns are no
+    multiple of 32 has to lie inside the allocation."""
+    wl = W._dense(300, 256, 1030).workload()
+    for acc in (1, 2, 4, 8):
+        for kw in (dict(), dict(persistent=1), dict(split_k=3), dict(persistent=1, cta_group=2)):
+            st, info = wl.check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tn, tile_k=32, stages=2, mma_m_axis=1, acc_split=acc, **kw))
+            assert st == B.TT_OK and info.legal.tile_n == tn
+            n_acc = 2 if info.legal.persistent else info.legal.acc_split
+            assert (n_acc - 1) * tn + (tn + 31) // 32 * 32 <= info.tmem_cols <= 512 and info.tmem_cols & (info.tmem_cols - 1) == 0
