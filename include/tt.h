@@ -127,8 +127,11 @@ typedef struct tt_schedule_record {
                               channels, tap by tap inside a block: the filters are re-packed into that order by a small
                               kernel (once per weight pointer: again only when tt_run sees other weights), the input is transposed once per block into a pixel-major
                               slab, and every tap's operand tile is a shifted view of that slab -- no expansion.
-                              Filters on the 128 rows, split_k = 1;
-                              tile_k = 32 * (taps per pipeline stage), the tap count a divisor of r*s, at most 128. */
+                              Filters on the 128 rows, split_k = 1, CTAs that walk tiles (persistent: always 1 in the
+                              legal record); stages * tile_k / 32 taps' filters are in flight, at most 8 (legal records:
+                              tile_k = 32, stages = that number); cta_group CTAs of a cluster share a tile's channel blocks.
+                              In legalise mode tile_n and cta_group are laid over the SMs for the kernel's size and the
+                              legal record says how; in strict mode they run as written. */
     int32_t persistent;    /* GEMM_TC: 1 = the grid is one CTA (or CTA pair) per SM and every CTA walks output tiles; the
                               operand pipeline runs on across tiles and two accumulators in tensor memory alternate, so a
                               tile is read out (bias, activation, stores) while the next one is accumulated.  Needs
@@ -138,7 +141,9 @@ typedef struct tt_schedule_record {
                               lies).  Elsewhere legalised to 0. */
     int32_t cta_group;     /* GEMM_TC, persistent: 2 = two CTAs of a cluster share a 256-row tile; each loads its own rows of
                               the first operand and HALF of the second operand's rows, the multiply-accumulate runs across
-                              both SMs (tcgen05 cta_group::2).  K-major operands only, tile_n >= 32.  0 or 1 = one CTA. */
+                              both SMs (tcgen05 cta_group::2).  K-major operands only, tile_n >= 32.  0 or 1 = one CTA.
+                              k_order = 1: 1..8, the CTAs of a cluster that share a tile's channel blocks, each adding up
+                              some of them; their parts of the tile are added in CTA order. */
     int32_t ctas_per_sm;   /* GEMM_TC, not persistent: 2 = the register-capped build of the kernel, so that two CTAs share an
                               SM when the record needs at most 112 KB of shared memory and 256 tensor-memory columns (one
                               CTA's set-up and read-out overlap the other's main loop); 1 = all registers, one CTA per SM;
@@ -182,7 +187,8 @@ typedef struct tt_apply_info {
 
 enum { TT_CHG_TILE_M = 1, TT_CHG_TILE_N = 2, TT_CHG_TILE_K = 4, TT_CHG_STAGES = 8, TT_CHG_SPLIT_K = 16,
        TT_CHG_VEC = 32, TT_CHG_BLOCK = 64, TT_CHG_ITEMS = 128, TT_CHG_SLAB = 256, TT_CHG_ACC = 512, TT_CHG_KORDER = 1024,
-       TT_CHG_FORM = 2048   /* the record named a kernel form this shape does not have (DW_SIMT unroll / raster) */ };
+       TT_CHG_FORM = 2048,  /* the record named a kernel form this shape does not have (DW_SIMT unroll / raster) */
+       TT_CHG_CLUSTER = 4096   /* GEMM_TC, k_order = 1: how many CTAs share a tile (cta_group) */ };
 
 /* Validity modes for mapping a record onto another shape (Section 4.1).
  *   TT_MODE_LEGALISE  reformulate: clamp/round tile sizes to the new extents and the hardware's legal set,

@@ -24,8 +24,8 @@ TT_ACT_NONE, TT_ACT_RELU, TT_ACT_RELU6, TT_ACT_GELU_ERF = range(4)
 TT_FAMILY_GEMM_TC, TT_FAMILY_DW_SIMT, TT_FAMILY_ROW_SIMT = range(3)
 TT_MODE_LEGALISE, TT_MODE_STRICT = 0, 1
 TT_RECORD_VERSION = 3
-TT_CHG_TILE_M, TT_CHG_TILE_N, TT_CHG_TILE_K, TT_CHG_STAGES, TT_CHG_SPLIT_K, TT_CHG_VEC, TT_CHG_BLOCK, TT_CHG_ITEMS, TT_CHG_SLAB, TT_CHG_ACC, TT_CHG_KORDER, TT_CHG_FORM = \
-    1, 2, 4, 8, 16, 32, 64, 128, 256, 512, 1024, 2048
+TT_CHG_TILE_M, TT_CHG_TILE_N, TT_CHG_TILE_K, TT_CHG_STAGES, TT_CHG_SPLIT_K, TT_CHG_VEC, TT_CHG_BLOCK, TT_CHG_ITEMS, TT_CHG_SLAB, TT_CHG_ACC, TT_CHG_KORDER, TT_CHG_FORM, \
+    TT_CHG_CLUSTER = 1, 2, 4, 8, 16, 32, 64, 128, 256, 512, 1024, 2048, 4096
 
 i32, u32, f32 = C.c_int32, C.c_uint32, C.c_float
 
@@ -56,7 +56,7 @@ class tt_schedule_record(C.Structure):
             return (f"tc[{self.tile_m}x{self.tile_n}x{self.tile_k} st{self.stages} sk{self.split_k} "
                     f"r{self.raster} ax{self.mma_m_axis}" + (f" sl{self.slab_tiles}" if self.slab_tiles else "") +
                     (f" acc{self.acc_split}" if self.acc_split > 1 else "") + (" tap" if self.k_order else "") +
-                    (" ps" if self.persistent else "") + (" cg2" if self.cta_group == 2 else "") +
+                    (" ps" if self.persistent else "") + (f" cg{self.cta_group}" if self.cta_group > 1 else "") +
                     (" 2/sm" if self.ctas_per_sm == 2 else "") + (" x3" if self.precision else "") + "]")
         if self.family == TT_FAMILY_DW_SIMT:
             return (f"dw[c{self.tile_m} {self.block_y}x{self.block_x} it{self.items_per_thread} "

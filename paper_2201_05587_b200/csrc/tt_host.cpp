@@ -133,31 +133,28 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     const int tk = 32 * tps;
     if (strict && (rec->mma_m_axis == 2 || rec->tile_k != tk || rec->split_k != 1)) return TT_ERR_INVALID_SCHEDULE;
     L.mma_m_axis = 1; L.tile_m = kHwTileM; L.tile_k = tk; L.split_k = 1; L.acc_split = 1; L.slab_tiles = 0; L.k_order = 1;
-    // (one kernel serves both forms: its CTAs always walk; CTA pairs do not exist here)
+    // (one kernel serves both forms: its CTAs always walk)
     const bool persistent = rec->persistent == 1;
-    L.persistent = persistent ? 1 : 0; L.cta_group = 1; L.ctas_per_sm = 1;
-    if (rec->cta_group == 2 || rec->ctas_per_sm == 2) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_FORM; }
+    L.persistent = 1; L.ctas_per_sm = 1;
+    if (rec->ctas_per_sm == 2) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_FORM; }
     L.precision = 0;                                      // (no error-compensated products for convolutions)
     if (rec->precision != 0) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_FORM; }
     if (rec->tile_m != kHwTileM) changed |= TT_CHG_TILE_M;
-    if (rec->tile_k != tk) changed |= TT_CHG_TILE_K;
     if (rec->split_k != 1) changed |= TT_CHG_SPLIT_K;
     int tn = std::min(256, std::max(16, round_up(rec->tile_n, 16)));
     tn = std::min(tn, round_up(N, 16));
-    if (tn != rec->tile_n) changed |= TT_CHG_TILE_N;
-    L.tile_n = tn;
     const int k_tiles = CB * RS / tps;
     // (the walking kernel's filter pipeline runs on across tiles: no point in clamping it to one tile's reduction)
-    int st = persistent ? std::min(kMaxStages, rec->stages) : std::min(std::min(kMaxStages, rec->stages), k_tiles);
-    if (st != rec->stages) changed |= TT_CHG_STAGES;
-    if (strict && (changed & ~TT_CHG_TILE_M)) return TT_ERR_INVALID_SCHEDULE;
+    const int st = persistent ? std::min(kMaxStages, rec->stages) : std::min(std::min(kMaxStages, rec->stages), k_tiles);
+    if (strict && (tn != rec->tile_n || st != rec->stages || (changed & ~TT_CHG_TILE_M))) return TT_ERR_INVALID_SCHEDULE;
     const int tiles_m = (M + kHwTileM - 1) / kHwTileM;
-    // How the record's tiles are laid over the SMs (148; the launch is right on any number).  Where they fill more than half of
-    // them, columns are dealt evenly over the rounds that the record's tile needs: 121 tiles of 224 columns become 141 of 192.
-    // Where they fill less, CTAs share a tile's channel blocks as a cluster.  Fewer rounds, or the widest tile, take the place of
-    // the record's where they are a tenth cheaper: a tap costs what shared memory has to move in 128-byte lines -- its filters in
-    // and out, 2 * 128, its columns, about 32 for the slab -- and the filters' part is paid per tile (3x3 512 -> 512 at 7 x 7,
-    // batch 32: 31.4 us with 128 columns, 25.1 with 256).
+    // How the tiles are laid over the SMs (148; the launch is right on any number) is this rule's choice unless the record is to
+    // run as written (strict mode); the legal record says what it chose (tile_n, cta_group).
+    // Where the record's tiles fill more than half of the SMs, columns are dealt evenly over the rounds that its tile needs: 121
+    // tiles of 224 columns become 141 of 192.  Where they fill less, CTAs share a tile's channel blocks as a cluster.  Fewer
+    // rounds, or the widest tile, take the place of the record's where they are a tenth cheaper: a tap costs what shared memory has to move in
+    // 128-byte lines -- its filters in and out, 2 * 128, its columns, about 32 for the slab -- and the filters' part is paid per
+    // tile (3x3 512 -> 512 at 7 x 7, batch 32: 31.4 us with 128 columns, 25.1 with 256).
     constexpr int kSms = 148;
     const auto tiles_of = [&](int n) { return (long long)tiles_m * ((N + n - 1) / n); };
     const auto split_of = [&](int n) { return (int)std::max<long long>(1, std::min<long long>(std::min(8, CB), kSms / tiles_of(n))); };
@@ -170,21 +167,31 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
         const long long columns = rounds * kSms / tiles_m;
         return columns >= 1 ? std::max<long long>(16, round_up64((N + columns - 1) / columns, 16)) : 0x7fffffffLL;
     };
-    int wide = std::min(256, round_up(N, 16));
-    if (tiles_of(tn) * 2 > kSms) {
-        const long long rounds = (tiles_of(tn) + kSms - 1) / kSms;
-        tn = (int)std::min<long long>(tn, dealt(rounds));
-        wide = tn;
-        for (long long r = 1; r < rounds && r <= 4; ++r) if (dealt(r) <= 256) { wide = (int)dealt(r); break; }
+    int split = std::max(1, rec->cta_group);
+    if (strict) {
+        // (the CTAs of a cluster take one tile: all tiles have to be resident at once)
+        if (split > std::min(8, CB) || (split > 1 && tiles_of(tn) * split > kSms)) return TT_ERR_INVALID_SCHEDULE;
+    } else {
+        int wide = std::min(256, round_up(N, 16));
+        if (tiles_of(tn) * 2 > kSms) {
+            const long long rounds = (tiles_of(tn) + kSms - 1) / kSms;
+            tn = (int)std::min<long long>(tn, dealt(rounds));
+            wide = tn;
+            for (long long r = 1; r < rounds && r <= 4; ++r) if (dealt(r) <= 256) { wide = (int)dealt(r); break; }
+        }
+        if (cost_of(wide) * 10 < cost_of(tn) * 9) tn = wide;
+        split = tiles_of(tn) * 2 > kSms ? 1 : split_of(tn);
     }
-    if (cost_of(wide) * 10 < cost_of(tn) * 9) tn = wide;
-    const int split = tiles_of(tn) * 2 > kSms ? 1 : split_of(tn);
+    L.tile_n = tn; L.cta_group = split;
+    if (tn != rec->tile_n) changed |= TT_CHG_TILE_N;
+    if (split != std::max(1, rec->cta_group)) changed |= TT_CHG_CLUSTER;
     const int tiles_n = (N + tn - 1) / tn;
     const long long tiles = (long long)tiles_m * tiles_n;
     if (tiles > 0x7fffffffLL) return TT_ERR_RESOURCE;
     // shared memory: filter stages | one or two slabs | staging blocks of the read-out (twelve warps' where all tiles are
-    // resident, a cluster's whole tile, each over the idle pipeline).  A stage takes up to three taps, whose issue then hides
-    // the latency of the stage's barriers; the record's stages times its taps per reduction tile say how many are in flight.
+    // resident, a cluster's whole tile, each over the idle pipeline).  A barrier is passed for up to three taps, whose issue then
+    // hides its latency; the record's stages times its taps per reduction tile say how many taps' filters are in flight.  Records
+    // that ask for the same run the same, so the legal one names them in one way: reduction tiles of one tap.
     const int shift_min = ty.lo * tx.pitch + tx.lo, shift_max = std::max(0, ty.hi) * tx.pitch + std::max(0, tx.hi);
     const int lines = tn + shift_max - std::min(shift_min, 0);
     const long long slab = (long long)lines * 128;
@@ -202,8 +209,13 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
         else if (depth > 1) --depth;
         else break;
     }
-    if (depth * q < want) { changed |= TT_CHG_STAGES; if (strict) return TT_ERR_RESOURCE; st = std::max(1, depth * q / tps); }
-    L.stages = st;
+    if (strict) {
+        if (depth * q < want) return TT_ERR_RESOURCE;
+    } else {
+        L.tile_k = 32; L.stages = std::min(kMaxStages, depth * q);
+        if (rec->tile_k != L.tile_k) changed |= TT_CHG_TILE_K;
+        if (rec->stages != L.stages) changed |= TT_CHG_STAGES;
+    }
     const long long smem = total();
     const int tmem_cols = std::max(32, pow2_ceil(tiles > kSms ? tn + round_up(tn, 32) : round_up(tn, 32)));
     I = tt_apply_info{};
@@ -248,7 +260,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     // nonsense is refused whatever the kernel and the reduction order
     if (rec->tile_m <= 0 || rec->tile_n <= 0 || rec->tile_k <= 0 || rec->stages <= 0 || rec->split_k <= 0 ||
         rec->raster < 0 || rec->raster > 1 || rec->mma_m_axis < 0 || rec->mma_m_axis > 2 || rec->persistent < 0 ||
-        rec->persistent > 1 || rec->cta_group < 0 || rec->cta_group > 2 || rec->ctas_per_sm < 0 || rec->ctas_per_sm > 2 ||
+        rec->persistent > 1 || rec->cta_group < 0 || rec->cta_group > (rec->k_order == 1 ? 8 : 2) || rec->ctas_per_sm < 0 || rec->ctas_per_sm > 2 ||
         rec->acc_split < 0 || rec->k_order < 0 || rec->k_order > 1 || rec->warp_layout != 0 || rec->precision < 0 || rec->precision > 1 ||
         (w->op == TT_OP_CONV2D && rec->slab_tiles < 0))
         return TT_ERR_INVALID_SCHEDULE;
@@ -326,6 +338,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         : w->op == TT_OP_BATCH_MATMUL && !w->sh.trans_b && w->sh.nn % 4 == 0;
     int cg = rec->cta_group == 2 ? 2 : 1;
     if (cg == 2 && (!persistent || mn_operand || tn < 32)) { if (strict) return TT_ERR_INVALID_SCHEDULE; cg = 1; changed |= TT_CHG_FORM; }
+    if (rec->cta_group > 2) changed |= TT_CHG_FORM;       // (a cluster of the tap-major order, which is not this kernel's)
     L.persistent = persistent ? 1 : 0;
     L.cta_group = cg;
     int sk = persistent ? 1 : rec->split_k;

@@ -1071,3 +1071,20 @@ def test_tap_major_convolutions_of_every_layout(shape):
         assert stat == B.TT_OK and info.legal.k_order == 1
         run_spec(sp, rec, a, ref, ref_elem=re)
     probe.close()
+
+
+@pytest.mark.parametrize("cg", [1, 2, 3, 5])
+def test_tap_major_records_run_as_written_in_strict_mode(cg):
+    """Columns, taps in flight and the CTAs that share a tile's channel blocks (5 blocks, the last one partial) as the record has
+    them, where legalise mode would lay them out for the kernel's size."""
+    sp = W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(3, 140, 9, 9, 150, 3, 3, 1, 1, True, B.TT_ACT_RELU, True), 1, "tap_strict", "uniform")
+    a = W.make_inputs(sp, 98)
+    ref = util.oracle_ref(sp, a)
+    re = elem_ref(sp, a, ref)
+    for tn, tk, st in ((32, 32, 1), (112, 96, 2)):
+        rec = tc(tile_n=tn, tile_k=tk, stages=st, k_order=1, mma_m_axis=1, cta_group=cg)
+        probe = sp.workload()
+        status, info = probe.check(rec, mode=B.TT_MODE_STRICT)
+        assert status == B.TT_OK and (info.legal.tile_n, info.legal.stages, info.grid_y) == (tn, st, cg)
+        probe.close()
+        run_spec(sp, rec, a, ref, mode=B.TT_MODE_STRICT, ref_elem=re)

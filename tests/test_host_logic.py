@@ -675,3 +675,80 @@ def test_tensor_memory_covers_what_the_read_out_reads(tn):
             assert st == B.TT_OK and info.legal.tile_n == tn
             n_acc = 2 if info.legal.persistent else info.legal.acc_split
             assert (n_acc - 1) * tn + (tn + 31) // 32 * 32 <= info.tmem_cols <= 512 and info.tmem_cols & (info.tmem_cols - 1) == 0
+
+
+def _launch_of(info):
+    """What a launch is made from, as far as the apply info says it."""
+    return (info.grid_x, info.grid_y, info.grid_z, info.threads, info.smem_bytes, info.tmem_cols, info.workspace_bytes)
+
+
+def _check_legal_says_what_runs(wl, recs):
+    """The legal record is what runs: legalising it again changes nothing and gives the same launch; every field that was
+    replaced is reported; a record taken in strict mode runs as written.  Returns {legal record: launch}."""
+    seen = {}
+    for rec in recs:
+        st, info = wl.check(rec)
+        if st != B.TT_OK:
+            continue
+        st2, again = wl.check(info.legal)
+        assert st2 == B.TT_OK and _rec_key(again.legal) == _rec_key(info.legal), (rec.short(), info.legal.short(), again.legal.short())
+        assert not again.changed and _launch_of(again) == _launch_of(info), (rec.short(), info.legal.short(), again.changed)
+        bits = {"tile_n": B.TT_CHG_TILE_N, "tile_k": B.TT_CHG_TILE_K, "stages": B.TT_CHG_STAGES, "split_k": B.TT_CHG_SPLIT_K,
+                "k_order": B.TT_CHG_KORDER, "block_x": B.TT_CHG_BLOCK, "block_y": B.TT_CHG_BLOCK, "threads": B.TT_CHG_BLOCK,
+                "items_per_thread": B.TT_CHG_ITEMS, "vec_width": B.TT_CHG_VEC, "unroll": B.TT_CHG_FORM}
+        used = ("tile_n", "tile_k", "stages", "split_k", "k_order") if rec.family == B.TT_FAMILY_GEMM_TC else \
+            ("block_x", "block_y", "threads", "items_per_thread", "vec_width", "unroll") + (("stages",) if info.legal.raster else ())
+        for f in used:
+            assert getattr(info.legal, f) == getattr(rec, f) or info.changed & bits[f], (rec.short(), info.legal.short(), f, info.changed)
+        if info.legal.k_order and info.legal.cta_group != max(1, rec.cta_group):
+            assert info.changed & B.TT_CHG_CLUSTER
+        if rec.family == B.TT_FAMILY_DW_SIMT and info.legal.tile_m != rec.tile_m:
+            assert info.changed & B.TT_CHG_TILE_M
+        st3, strict = wl.check(rec, mode=B.TT_MODE_STRICT)
+        if st3 == B.TT_OK:
+            for f in used:
+                assert getattr(strict.legal, f) == getattr(rec, f) and not strict.changed & ~B.TT_CHG_TILE_M
+        seen.setdefault(_rec_key(info.legal), set()).add(_launch_of(info))
+    assert all(len(v) == 1 for v in seen.values())
+    return seen
+
+
+def test_tap_major_legal_records_say_what_runs():
+    """Columns and clusters that are laid over the SMs, taps in flight: named by the legal record, as written in strict mode."""
+    import random
+    rng = random.Random(3)
+    def conv(n, c, h, w, k, r, st, pad):
+        return B.Workload(B.TT_OP_CONV2D, B.make_shapes(n=n, c=c, h=h, w=w, k=k, r=r, s=r, stride_h=st, stride_w=st, pad_h=pad, pad_w=pad,
+                                                        has_bias=1, act=B.TT_ACT_RELU), "tap")
+    shapes = [(32, 128, 28, 28, 128, 3, 1, 1), (32, 512, 7, 7, 512, 3, 1, 1), (1, 64, 28, 28, 64, 3, 1, 1), (2, 16, 9, 9, 24, 1, 1, 0)]
+    for _ in range(150):
+        r = rng.choice((1, 2, 3, 3, 5, 7))
+        shapes.append((rng.choice((2, 3, 8, 32, 70)), 8 * rng.randint(1, 64), rng.randint(7, 64), rng.randint(7, 64), 8 * rng.randint(1, 64), r,
+                       rng.choice((1, 1, 2, 3)), rng.randint(0, r - 1)))
+    recs = [B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tn, tile_k=tk, stages=sg, mma_m_axis=1, k_order=1, persistent=ps, cta_group=cg)
+            for tn in (16, 48, 64, 112, 128, 192, 224, 256) for tk in (32, 64, 96, 128) for sg, ps, cg in ((1, 0, 1), (2, 0, 1), (4, 1, 2), (8, 0, 8))]
+    for shape in shapes:
+        wl = conv(*shape)
+        _check_legal_says_what_runs(wl, recs)
+        wl.close()
+    # the two records that used to be one launch under two names
+    wl = conv(32, 128, 28, 28, 128, 3, 1, 1)
+    a, b = (wl.check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tn, tile_k=tk, stages=sg, mma_m_axis=1, k_order=1))[1] for tn, tk, sg in ((224, 96, 2), (128, 32, 4)))
+    assert _rec_key(a.legal) == _rec_key(b.legal) and (a.legal.tile_n, a.legal.stages, a.grid_x) == (192, 6, 141) and a.changed & B.TT_CHG_TILE_N
+    st, s = wl.check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=224, tile_k=96, stages=2, mma_m_axis=1, k_order=1), mode=B.TT_MODE_STRICT)
+    assert st == B.TT_OK and s.legal.tile_n == 224 and s.grid_x == 121 and s.grid_y == 1
+    wl.close()
+    wl = conv(32, 512, 7, 7, 512, 3, 1, 1)
+    info = wl.check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=128, tile_k=32, stages=4, mma_m_axis=1, k_order=1))[1]
+    assert (info.legal.tile_n, info.legal.cta_group, info.grid_x, info.grid_y) == (256, 4, 32, 4) and info.changed & B.TT_CHG_CLUSTER
+    rec = B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=256, tile_k=32, stages=4, mma_m_axis=1, k_order=1, cta_group=3)
+    st, s = wl.check(rec, mode=B.TT_MODE_STRICT)
+    assert st == B.TT_OK and (s.legal.cta_group, s.grid_x, s.grid_y) == (3, 32, 3)
+    rec.cta_group = 8                                    # 32 tiles of 8 CTAs are not resident at once
+    assert wl.check(rec, mode=B.TT_MODE_STRICT)[0] == B.TT_ERR_INVALID_SCHEDULE
+    # a cluster of that order on a kernel without it
+    st, info = W._dense(128, 256, 128).workload().check(rec)
+    assert st == B.TT_OK and info.legal.cta_group == 1 and info.changed & B.TT_CHG_FORM
+    rec.k_order = 0
+    assert wl.check(rec)[0] == B.TT_ERR_INVALID_SCHEDULE
+    wl.close()
