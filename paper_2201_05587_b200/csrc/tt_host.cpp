@@ -592,33 +592,22 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     // else, so the ring takes as many stages as fit, up to a CTA's whole reduction.  A batch-1 layer then requests all of its
     // weights at once instead of a refill of two stages per trip to memory (the 84 kernels of the 12-layer encoder at batch 1
     // and 128 tokens: 528 us with the record's depth, 501 with this one).
-    // A compensated stage is twice the size and passes through the warps' hands between its arrival and its products.  Where only
-    // one of the record's fits, it runs as several of 32, so that the three steps overlap (512 x 1024 over 4096, stages of 64 with
-    // 128 columns: 182 us; as three of 32: 99).  Two of 64 are 3 % faster than four of 32.
-    int depth = st, run_tk = tk, run_tiles = k_tiles, run_split = per_split;
-    unsigned run_a = a_stage, run_b = b_stage;
-    if (L.ctas_per_sm != 2 && x3)
-        while (depth < std::min(kMaxStages, per_split) && (depth + 1ll) * (a_stage + b_stage) * 2 + smem - pipe <= kDynSmemLimit) ++depth;
-    if (x3 && tk > 32 && depth == 1 && per_split > 1) {
-        const int f = tk / 32;
-        run_tk = 32; run_tiles = (K + 31) / 32; run_split = per_split * f;
-        run_a /= f; run_b /= f; depth = std::min({kMaxStages, st * f, run_split});
-    }
-    const long long run_stage = (long long)(run_a + run_b) * (x3 ? 2 : 1);
+    int depth = st;
+    const long long run_stage = (long long)(a_stage + b_stage) * (x3 ? 2 : 1);
     auto run_bytes = [&](int d) { return std::max<long long>(d * run_stage, min_pipe) + smem - pipe; };
     if (L.ctas_per_sm != 2)
-        while (depth < std::min(kMaxStages, run_split) && run_bytes(depth + 1) <= kDynSmemLimit) ++depth;
+        while (depth < std::min(kMaxStages, per_split) && run_bytes(depth + 1) <= kDynSmemLimit) ++depth;
     const long long run_pipe = std::max<long long>(depth * run_stage, min_pipe);
     plan->run_smem = (int)run_bytes(depth);
     GemmArgs& g = plan->g;
     g = GemmArgs{};
     g.M = M; g.N = N; g.K = K; g.batch = B;
-    g.tile_n = tn; g.tile_k = run_tk; g.stages = depth;
-    g.k_tiles = run_tiles; g.k_tiles_per_split = run_split; g.split_k = sk;
+    g.tile_n = tn; g.tile_k = tk; g.stages = depth;
+    g.k_tiles = k_tiles; g.k_tiles_per_split = per_split; g.split_k = sk;
     g.tiles_m = tiles_m; g.tiles_n = tiles_n; g.raster = L.raster;
-    g.atom_k = atom_k; g.n_atoms = run_tk / atom_k; g.row_bytes = row_bytes;
+    g.atom_k = atom_k; g.n_atoms = n_atoms; g.row_bytes = row_bytes;
     g.swz_mask = row_bytes == 128 ? 7 : (row_bytes == 64 ? 3 : 1);
-    g.a_stage_bytes = run_a; g.b_stage_bytes = run_b;
+    g.a_stage_bytes = a_stage; g.b_stage_bytes = b_stage;
     g.ktab_off = (unsigned)run_pipe;
     g.slab_off = (unsigned)(run_pipe + ktab);
     g.red_off = (unsigned)(run_pipe + ktab + (long long)sl_nbuf * sl_buf_bytes);
@@ -680,31 +669,53 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     g.C = s.c; g.H = s.h; g.W = s.w; g.R = s.r; g.S = s.s; g.Q = Q;
     g.sh = s.stride_h; g.sw = s.stride_w; g.ph = s.pad_h; g.pw = s.pad_w;
     g.idesc |= (A.mode == OPM_TMA_MN ? 1u << 15 : 0u) | (Bo.mode == OPM_TMA_MN ? 1u << 16 : 0u);
-    g.tx_bytes = (A.mode == OPM_TMA || A.mode == OPM_TMA_MN ? run_a : 0) + (Bo.mode == OPM_TMA || Bo.mode == OPM_TMA_MN ? run_b : 0);
+    g.tx_bytes = (A.mode == OPM_TMA || A.mode == OPM_TMA_MN ? a_stage : 0) + (Bo.mode == OPM_TMA || Bo.mode == OPM_TMA_MN ? b_stage : 0);
     g.vec_store = (g.y_ns == 1 && g.y_ms % 4 == 0 && g.y_bs % 4 == 0) ? 1 : 0;
     return TT_OK;
 }
 
 // Compensated products are bound by shared memory: every operand byte is written by TMA, read and written again for its
 // remainder and read by three products, 1.5 cycles per row of both tiles for each 8 of the reduction, and that is more than the
-// products take up to 256 columns.  Where a tile of twice the record's columns does a round of the SMs for less, it runs instead
-// (512 x 1024 over 4096 in quarters: 256 tiles of 64 columns are two rounds of 288 cycles a step, 128 of 128 one of 384).
+// products take up to 256 columns.  A compensated stage is twice the size and passes through the warps' hands between its arrival
+// and its products.  Unless the record is to run as written (strict mode), two rules lay its tile out for that; the legal record
+// says what they chose.
+// Where only one of the record's stages fits, it becomes several of 32, so that the three steps overlap (512 x 1024 over 4096,
+// stages of 64 with 128 columns: 182 us; as three of 32: 99).  Two of 64 are 3 % faster than four of 32.
+// Where a tile of twice the record's columns does a round of the SMs for less, it takes its place (512 x 1024 over 4096 in
+// quarters: 256 tiles of 64 columns are two rounds of 288 cycles a step, 128 of 128 one of 384).
 static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, Plan* plan) {
-    Plan p = *plan;
+    const Plan fresh = *plan;
     const tt_status s = plan_gemm(w, rec, mode, plan);
+    if (s != TT_OK || !plan->g.x3 || mode == TT_MODE_STRICT) return s;
+    const int changed = plan->info.changed;
+    auto replan = [&](const tt_schedule_record& r, bool same_splits) {
+        Plan p = fresh;
+        if (plan_gemm(w, &r, TT_MODE_LEGALISE, &p) != TT_OK || p.info.legal.stages < std::min(2, p.g.k_tiles_per_split) ||
+            (same_splits && p.info.legal.split_k != plan->info.legal.split_k)) return;
+        const tt_schedule_record& L = p.info.legal;
+        p.info.changed = changed & ~(TT_CHG_TILE_N | TT_CHG_TILE_K | TT_CHG_STAGES | TT_CHG_SPLIT_K);
+        if (L.tile_n != rec->tile_n) p.info.changed |= TT_CHG_TILE_N;
+        if (L.tile_k != rec->tile_k) p.info.changed |= TT_CHG_TILE_K;
+        if (L.stages != rec->stages) p.info.changed |= TT_CHG_STAGES;
+        if (L.split_k != rec->split_k) p.info.changed |= TT_CHG_SPLIT_K;
+        *plan = p;
+    };
+    if (plan->info.legal.tile_k > 32 && plan->g.stages == 1 && plan->g.k_tiles_per_split > 1) {
+        tt_schedule_record thin = plan->info.legal;
+        thin.stages = thin.tile_k / 32; thin.tile_k = 32;
+        replan(thin, false);
+    }
     const tt_schedule_record L = plan->info.legal;
-    if (s != TT_OK || !plan->g.x3 || L.tile_n > 128 || rec->ctas_per_sm != 0) return s;
     auto cost = [&](int tn) {
         const long long ctas = (long long)((plan->gm + kHwTileM - 1) / kHwTileM) * ((plan->gn + tn - 1) / tn) * L.split_k * plan->gbatch;
         return (double)((ctas + 147) / 148) * std::max(1.5 * (kHwTileM + tn), 2.13 * tn);
     };
-    if (cost(2 * L.tile_n) > 0.85 * cost(L.tile_n)) return s;
-    tt_schedule_record wide = L;
-    wide.tile_n = 2 * L.tile_n; wide.tile_k = std::min(32, L.tile_k); wide.stages = 2;
-    wide.ctas_per_sm = 0;
-    if (plan_gemm(w, &wide, TT_MODE_LEGALISE, &p) != TT_OK || p.info.legal.split_k != L.split_k || p.info.legal.stages < std::min(2, p.g.k_tiles_per_split)) return s;
-    p.info.legal = L; p.info.changed = plan->info.changed;
-    *plan = p;
+    if (L.tile_n <= 128 && rec->ctas_per_sm == 0 && cost(2 * L.tile_n) <= 0.85 * cost(L.tile_n)) {
+        tt_schedule_record wide = L;
+        wide.tile_n = 2 * L.tile_n; wide.tile_k = std::min(32, L.tile_k); wide.stages = 2;
+        wide.ctas_per_sm = 0;
+        replan(wide, true);
+    }
     return s;
 }
 

@@ -752,3 +752,25 @@ def test_tap_major_legal_records_say_what_runs():
     rec.k_order = 0
     assert wl.check(rec)[0] == B.TT_ERR_INVALID_SCHEDULE
     wl.close()
+
+
+def test_compensated_legal_records_say_what_runs():
+    """Tiles of twice the columns and stages of 32 are named by the legal record; strict mode runs the record as written."""
+    import random
+    rng = random.Random(9)
+    recs = [B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tn, tile_k=tk, stages=sg, split_k=sk, mma_m_axis=ax, precision=1, ctas_per_sm=cps)
+            for tn in (16, 32, 64, 128, 256) for tk in (8, 32, 64, 128) for sg, sk in ((1, 1), (2, 4), (3, 3), (4, 12)) for ax in (1, 2) for cps in (0, 2)]
+    for m, k, n in [(512, 4096, 1024), (1030, 520, 700), (64, 64, 64)] + [(rng.randint(1, 2000), 4 * rng.randint(1, 500), rng.randint(1, 2000)) for _ in range(20)]:
+        wl = W._dense(m, k, n).workload()
+        _check_legal_says_what_runs(wl, recs)
+        wl.close()
+    wl = W._dense(512, 4096, 1024).workload()
+    rec = B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=64, tile_k=64, stages=2, split_k=4, mma_m_axis=1, precision=1)
+    st, info = wl.check(rec)
+    assert st == B.TT_OK and (info.legal.tile_n, info.legal.tile_k, info.grid_x) == (128, 32, 32) and info.changed & B.TT_CHG_TILE_N
+    st, info = wl.check(rec, mode=B.TT_MODE_STRICT)
+    assert st == B.TT_OK and (info.legal.tile_n, info.legal.tile_k, info.grid_x) == (64, 64, 64) and not info.changed & B.TT_CHG_TILE_N
+    rec = B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=256, tile_k=64, stages=1, mma_m_axis=1, precision=1)
+    st, info = wl.check(rec)
+    assert st == B.TT_OK and info.legal.tile_k == 32 and info.legal.stages == 2 and info.changed & B.TT_CHG_TILE_K
+    wl.close()
