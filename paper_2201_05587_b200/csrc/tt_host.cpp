@@ -383,12 +383,13 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         auto warp_bytes = [](int bufs) { return bufs == 1 ? 5120ll : bufs * 4096ll; };
         const bool res = w->sh.has_residual != 0;
         int ew = 4, eb = 1;
-        const int want = !mn ? st : (rec->slab_tiles == 0 ? kMaxStages : std::min(kMaxStages, std::max(st, rec->slab_tiles)));
         auto total = [&](int stages, int warps, int bufs) { return round_up64(stages * stage, 1024) + warps * warp_bytes(bufs) + 1024; };
         while (!strict && st > 1 && total(st, 4, 1) > kDynSmemLimit) { --st; changed |= TT_CHG_STAGES; }
-        if (mn && rec->slab_tiles != 0 && want > st && total(want, 4, 1) > kDynSmemLimit) {
+        // (from here on only what fits is asked for: a request for more must not cost the read-out its buffers)
+        int want = !mn ? st : (rec->slab_tiles == 0 ? kMaxStages : std::min(kMaxStages, std::max(st, rec->slab_tiles)));
+        while (rec->slab_tiles != 0 && want > st && total(want, 4, 1) > kDynSmemLimit) {
             if (strict) return TT_ERR_INVALID_SCHEDULE;
-            changed |= TT_CHG_SLAB;
+            --want;
         }
         // with a free depth the read-out's ring comes first, as long as three stages (or the record's) stay in flight
         const int keep = rec->slab_tiles == 0 && mn ? std::max(st, 3) : std::max(want, st);
@@ -401,6 +402,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         const long long smem_p = total(depth, ew, eb);
         if (!mn && rec->slab_tiles != 0) changed |= TT_CHG_SLAB;
         L.stages = st; L.split_k = 1; L.acc_split = 1; L.slab_tiles = (mn && rec->slab_tiles != 0) ? depth : 0; L.ctas_per_sm = 1;
+        if (!strict && L.slab_tiles != rec->slab_tiles) changed |= TT_CHG_SLAB;
         if (rec->ctas_per_sm == 2) { if (strict) return TT_ERR_INVALID_SCHEDULE; changed |= TT_CHG_FORM; }
         if (strict && (changed & ~TT_CHG_TILE_M)) return TT_ERR_INVALID_SCHEDULE;
         const int rows_m = kHwTileM * cg;

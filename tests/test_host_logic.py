@@ -774,3 +774,15 @@ def test_compensated_legal_records_say_what_runs():
     st, info = wl.check(rec)
     assert st == B.TT_OK and info.legal.tile_k == 32 and info.legal.stages == 2 and info.changed & B.TT_CHG_TILE_K
     wl.close()
+
+
+def test_persistent_legal_records_say_what_runs():
+    """More stages, or a deeper ring of a row-contiguous operand, than fit: the legal record's launch is the one that runs."""
+    recs = [B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tn, tile_k=tk, stages=sg, slab_tiles=sl, mma_m_axis=ax, persistent=1, cta_group=cg)
+            for tn in (16, 64, 112, 256) for tk in (16, 64, 128) for sg in (1, 2, 5, 8) for sl in (0, 1, 8) for ax in (1, 2) for cg in (1, 2)]
+    specs = [W._dense(478, 6 * 8, 484), W._dense(41, 120, 416), W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(105, 10, 88, 44, False), 1, "nn"),
+             W._conv(64, 28, 96, 1, 1, 0, residual=True)]
+    for sp in specs:
+        wl = sp.workload()
+        _check_legal_says_what_runs(wl, recs)
+        wl.close()
