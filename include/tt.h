@@ -102,6 +102,10 @@ typedef struct tt_shapes {
  *         (3x3 and 5x5 filters with "same" padding, stride 1 or 2; strips of 4 or 8 columns).  raster = 1 with
  *         unroll >= 1 and image rows of 16-byte multiples: the same strips, but CTAs walk the tiles persistently and
  *         a tile's input box and its planes' filters are staged in `stages` (2..4) shared-memory buffers by TMA.
+ *         raster = 1 on image rows that are no 16-byte multiples: whole planes, or bands of rows of one, staged as runs of
+ *         memory; unroll = 2, 4 or 7 rows x items_per_thread = 1 or 2 columns per thread, block_x the whole row.  From 2^18
+ *         outputs on every record with unroll >= 1 becomes the one of this form that is laid out for the kernel's size
+ *         (legalise mode; strict mode takes that one or a register-window record as written).
  * ROW_SIMT uses block_x (threads cooperating on one row: 1..32, power of two), block_y (rows per CTA), vec_width.
  * origin_* say which kernel the record was tuned on (its "native" kernel, Section 3). */
 typedef struct tt_schedule_record {

@@ -785,8 +785,11 @@ tt_status tt_grid_tune(tt_workload* w, const tt_tensors* t, void* cuda_stream, c
         tt_apply_info info;
         if (tt_schedule_check(w, &r, TT_MODE_LEGALISE, 0, &info) != TT_OK) return false;
         // (a pipeline made shallower to fit short reductions or shared memory is kept: exact duplicates are dropped below)
-        // (includes a reformulated reduction order; a tap-major tile is laid over the SMs for the kernel's size, and tried as that)
-        const int free_here = TT_CHG_TILE_M | TT_CHG_STAGES | (info.legal.k_order ? TT_CHG_TILE_N | TT_CHG_TILE_K | TT_CHG_CLUSTER : 0);
+        // (includes a reformulated reduction order; a tap-major tile and the staged depthwise forms are laid out for the kernel's
+        // size, and tried as that)
+        int free_here = TT_CHG_TILE_M | TT_CHG_STAGES;
+        if (info.legal.k_order) free_here |= TT_CHG_TILE_N | TT_CHG_TILE_K | TT_CHG_CLUSTER;
+        if (w->family == TT_FAMILY_DW_SIMT && r.raster == 1 && info.legal.raster == 1) free_here |= TT_CHG_BLOCK | TT_CHG_ITEMS | TT_CHG_VEC | TT_CHG_FORM;
         if (info.changed & ~free_here) return false;
         cand.push_back(info.legal);
         return true;

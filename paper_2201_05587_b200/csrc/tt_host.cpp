@@ -764,12 +764,13 @@ static void plan_dw_boxes(DwArgs& d, int rows, int items, bool may_widen) {
 }
 
 // Image rows that are no 16-byte multiples: no box can fetch them, and a register-window strip fetches each value of its rows
-// with a load of its own.  The run-staged persistent kernel runs instead; its tiles are this rule's, as the record has no fields
-// for them: strips of the height that takes the fewest instructions for the image's rows, channels for up to 256 threads in
-// buffers of 24 KB, but two tiles for every SM first.  From a quarter of a million outputs on: 480 x 14 x 14, 5x5, takes 4.5 us either
-// way for one image, 4.7 instead of 7.5 for 4 and 78 instead of 134 for 256; 960 x 7 x 7, 3x3, 3.6 instead of 2.9 for 4 (188 thousand
-// outputs), 5.0 instead of 5.2 for 16 and 30 instead of 44 for 256.
-static bool plan_dw_runs(const tt_workload* w, DwArgs& d, tt_apply_info& I) {
+// with a load of its own.  The run-staged persistent kernel runs instead, whatever the record's tile (except in strict mode); its
+// tiles are this rule's, and the legal record (raster = 1 on such rows) names them: strips of the height that takes the fewest
+// instructions for the image's rows, channels for up to 256 threads in buffers of 24 KB, but two tiles for every SM first.  From a
+// quarter of a million outputs on: 480 x 14 x 14, 5x5, takes 4.5 us either way for one image, 4.7 instead of 7.5 for 4 and 78
+// instead of 134 for 256; 960 x 7 x 7, 3x3, 3.6 instead of 2.9 for 4 (188 thousand outputs), 5.0 instead of 5.2 for 16 and 30
+// instead of 44 for 256.
+static bool plan_dw_runs(const tt_workload* w, DwArgs& d, tt_apply_info& I, tt_schedule_record& L) {
     const tt_shapes& s = w->sh;
     const long long planes = (long long)s.n * s.c, hw = (long long)s.h * s.w;
     if (s.w % 4 == 0 || w->Q > 256 || planes > 0x7fffffffLL || hw > (1 << 24)) return false;
@@ -838,6 +839,8 @@ static bool plan_dw_runs(const tt_workload* w, DwArgs& d, tt_apply_info& I) {
     d = t;
     I.grid_x = (int)std::min<long long>(total, 148 * per_sm); I.grid_y = 1; I.grid_z = 1;
     I.threads = threads; I.smem_bytes = (int)smem; I.launches = 1;
+    L.raster = 1; L.stages = d.tma_stages; L.unroll = rows; L.items_per_thread = d.items; L.vec_width = d.vec;
+    L.tile_m = d.tile_c; L.block_y = d.tile_h; L.block_x = d.tile_w; L.threads = threads;
     return true;
 }
 
@@ -847,8 +850,37 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     tt_schedule_record L = *rec;
     int changed = 0;
     if (rec->tile_m <= 0 || rec->block_x <= 0 || rec->block_y <= 0 || rec->items_per_thread <= 0 ||
-        rec->vec_width <= 0 || rec->threads <= 0)
+        rec->vec_width <= 0 || rec->threads <= 0 || rec->unroll < 0 || rec->raster < 0 || rec->raster > 1)
         return TT_ERR_INVALID_SCHEDULE;
+    // unroll >= 1 asks for the register-window kernel (that many output rows per thread: 1, 2 or 4), which exists
+    // for square 3x3 / 5x5 filters with "same" padding and stride 1 or 2 and works on strips of 4 columns;
+    // unroll == 0, or any other filter, takes the shared-memory staged kernel
+    const bool window_ok = s.r == s.s && (s.r == 3 || s.r == 5) && s.stride_h == s.stride_w &&
+                           (s.stride_h == 1 || s.stride_h == 2) && s.pad_h == s.r / 2 && s.pad_w == s.r / 2;
+    DwArgs& d = plan->dw;
+    d = DwArgs{};
+    d.N = s.n; d.C = s.c; d.H = s.h; d.W = s.w; d.R = s.r; d.S = s.s; d.P = w->P; d.Q = w->Q;
+    d.sh = s.stride_h; d.sw = s.stride_w; d.ph = s.pad_h; d.pw = s.pad_w; d.act = s.act;
+    tt_apply_info& I = plan->info;
+    I = tt_apply_info{};
+    if (rec->unroll >= 1 && window_ok) {
+        DwArgs runs = d;
+        tt_schedule_record R = *rec;
+        if (plan_dw_runs(w, runs, I, R)) {
+            int replaced = 0;
+            if (R.tile_m != rec->tile_m) replaced |= TT_CHG_TILE_M;
+            if (R.block_x != rec->block_x || R.block_y != rec->block_y || R.threads != rec->threads) replaced |= TT_CHG_BLOCK;
+            if (R.items_per_thread != rec->items_per_thread) replaced |= TT_CHG_ITEMS;
+            if (R.vec_width != rec->vec_width) replaced |= TT_CHG_VEC;
+            if (R.stages != rec->stages) replaced |= TT_CHG_STAGES;
+            if (R.raster != rec->raster || R.unroll != rec->unroll) replaced |= TT_CHG_FORM;
+            if (!strict || replaced == 0) {
+                I.legal = R; I.changed = replaced;
+                d = runs;
+                return TT_OK;
+            }
+        }
+    }
     if (strict && (rec->tile_m > s.c || rec->block_y > w->P || rec->block_x > round_up(w->Q, 4)))
         return TT_ERR_INVALID_SCHEDULE;
     L.tile_m = std::min(rec->tile_m, s.c);
@@ -858,13 +890,7 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     while (vec > 1 && (w->Q % vec) != 0) vec >>= 1;        // rows of y must stay vector-aligned
     int items = std::min(8, pow2_floor(rec->items_per_thread));
     items = std::max(items, vec);
-    // unroll >= 1 asks for the register-window kernel (that many output rows per thread: 1, 2 or 4), which exists
-    // for square 3x3 / 5x5 filters with "same" padding and stride 1 or 2 and works on strips of 4 columns;
-    // unroll == 0, or any other filter, takes the shared-memory staged kernel
-    const bool window_ok = s.r == s.s && (s.r == 3 || s.r == 5) && s.stride_h == s.stride_w &&
-                           (s.stride_h == 1 || s.stride_h == 2) && s.pad_h == s.r / 2 && s.pad_w == s.r / 2;
     int window_rows = 0;
-    if (rec->unroll < 0) return TT_ERR_INVALID_SCHEDULE;
     if (rec->unroll >= 1 && window_ok) {
         window_rows = rec->unroll >= 4 ? 4 : (rec->unroll >= 2 ? 2 : 1);
         items = rec->items_per_thread >= 8 ? 8 : 4;      // strips of 4 or 8 columns; 8-wide strips are at most 2 rows tall
@@ -887,10 +913,6 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     L.threads = th;
     if (strict && changed) return TT_ERR_INVALID_SCHEDULE;
 
-    DwArgs& d = plan->dw;
-    d = DwArgs{};
-    d.N = s.n; d.C = s.c; d.H = s.h; d.W = s.w; d.R = s.r; d.S = s.s; d.P = w->P; d.Q = w->Q;
-    d.sh = s.stride_h; d.sw = s.stride_w; d.ph = s.pad_h; d.pw = s.pad_w; d.act = s.act;
     d.tile_c = L.tile_m; d.tile_h = L.block_y; d.tile_w = L.block_x;
     d.in_h = (d.tile_h - 1) * d.sh + d.R;
     d.in_w = (d.tile_w - 1) * d.sw + d.S;
@@ -901,14 +923,12 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     d.window_rows = window_rows;
     d.vec_in = (s.w % 4) == 0;
     long long smem = window_rows ? 0 : (long long)d.tile_c * ((long long)d.in_h * d.in_w + d.R * d.S + 1) * 4;
-    tt_apply_info& I = plan->info;
     I = tt_apply_info{};
     I.legal = L; I.changed = changed;
     long long gx = (long long)d.tiles_w * d.tiles_h * d.tiles_c;
     // raster = 1 (with a window-kernel filter and 16-byte image rows): the tiles' input boxes are staged by TMA in
     // `stages` buffers, next to the filters and biases of their planes, and CTAs walk the tiles persistently
     L.raster = 0;
-    if (rec->raster < 0 || rec->raster > 1) return TT_ERR_INVALID_SCHEDULE;
     if (rec->raster == 1 && window_rows > 0 && (s.w % 4) == 0) {
         const long long planes = (long long)s.n * s.c;
         // a 5x5 filter's tallest strip becomes one of seven rows where that covers the tile as well and the chip has tiles to spare: a
@@ -949,7 +969,6 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     }
     if (rec->raster != 0) { if (strict) return TT_ERR_INVALID_SCHEDULE; I.changed |= TT_CHG_FORM; }
     I.legal = L;
-    if (window_rows > 0 && plan_dw_runs(w, d, I)) return TT_OK;
     I.grid_x = (int)std::min<long long>(gx, 0x7fffffff); I.grid_y = s.n; I.grid_z = 1;
     I.threads = th; I.smem_bytes = (int)std::min<long long>(smem, 0x7fffffff);
     I.launches = 1;

@@ -786,3 +786,37 @@ def test_persistent_legal_records_say_what_runs():
         wl = sp.workload()
         _check_legal_says_what_runs(wl, recs)
         wl.close()
+
+
+DW_RECORDS = [B.make_record(B.TT_FAMILY_DW_SIMT, tile_m=tm, block_y=by, block_x=bx, items_per_thread=it, vec_width=vw, threads=th, unroll=un, raster=ra, stages=sg)
+              for tm, by, bx in ((1, 8, 32), (4, 14, 28), (4, 28, 56), (5, 7, 16), (16, 14, 28), (48, 56, 112)) for it, vw, th in ((4, 4, 64), (4, 1, 256), (8, 2, 256))
+              for un in (0, 1, 2, 4, 7) for ra, sg in ((0, 1), (1, 2), (1, 4))]
+
+
+def _dw_batch(n, c, h, w, r, st):
+    return B.Workload(B.TT_OP_DWCONV2D, B.make_shapes(n=n, c=c, h=h, w=w, k=c, r=r, s=r, stride_h=st, stride_w=st, pad_h=r // 2, pad_w=r // 2,
+                                                      has_bias=1, act=B.TT_ACT_RELU6), "dw")
+
+
+def test_run_staged_depthwise_is_a_record_form():
+    """Batches of ragged rows: every register-window record becomes the one record of the run-staged form, which says what runs;
+    strict mode takes that record, or a register-window one as written."""
+    for shape in ((256, 480, 14, 14, 5, 1), (64, 480, 14, 14, 5, 1), (64, 144, 55, 55, 3, 1), (40, 96, 33, 31, 3, 2), (3, 9, 253, 253, 5, 1)):
+        wl = _dw_batch(*shape)
+        window = [r for r in DW_RECORDS if r.unroll >= 1]
+        seen = _check_legal_says_what_runs(wl, window)
+        assert len(seen) == 1
+        legal = wl.check(window[0])[1].legal
+        assert legal.raster == 1 and legal.unroll in (2, 4, 7) and legal.items_per_thread in (1, 2) and legal.block_x == wl.check(legal)[1].legal.block_x
+        assert wl.check(legal, mode=B.TT_MODE_STRICT)[0] == B.TT_OK
+        rec = B.make_record(B.TT_FAMILY_DW_SIMT, tile_m=4, block_y=7, block_x=12, items_per_thread=4, vec_width=1, threads=64, unroll=2)
+        st, info = wl.check(rec, mode=B.TT_MODE_STRICT)
+        assert st == B.TT_OK and info.legal.raster == 0 and info.legal.unroll == 2 and info.threads == 64 and info.smem_bytes == 0
+        rec.raster = 1
+        assert wl.check(rec, mode=B.TT_MODE_STRICT)[0] == B.TT_ERR_INVALID_SCHEDULE
+        _check_legal_says_what_runs(wl, [r for r in DW_RECORDS if r.unroll == 0])
+        # and away from there it is a record like any other
+        other = _dw_batch(4, 32, 28, 28, 3, 1)
+        assert other.check(legal)[0] == B.TT_OK
+        other.close()
+        wl.close()
