@@ -102,6 +102,8 @@ typedef struct tt_shapes {
  *         (3x3 and 5x5 filters with "same" padding, stride 1 or 2; strips of 4 or 8 columns).  raster = 1 with
  *         unroll >= 1 and image rows of 16-byte multiples: the same strips, but CTAs walk the tiles persistently and
  *         a tile's input box and its planes' filters are staged in `stages` (2..4) shared-memory buffers by TMA.
+ *         Legalise mode evens out the channels of its tiles, drops threads without a strip and makes 5x5 strips of 4 rows ones
+ *         of 7 (unroll = 7) where that is cheaper; the legal record says so, strict mode does not.
  *         raster = 1 on image rows that are no 16-byte multiples: whole planes, or bands of rows of one, staged as runs of
  *         memory; unroll = 2, 4 or 7 rows x items_per_thread = 1 or 2 columns per thread, block_x the whole row.  From 2^18
  *         outputs on every record with unroll >= 1 becomes the one of this form that is laid out for the kernel's size

@@ -896,10 +896,12 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
         items = rec->items_per_thread >= 8 ? 8 : 4;      // strips of 4 or 8 columns; 8-wide strips are at most 2 rows tall
         if (items == 8 && window_rows > 2) window_rows = 2;
     }
-    L.unroll = window_rows;
+    // (strips of 7 rows exist in the box-staged form of 5x5 filters)
+    const bool seven = rec->unroll == 7 && rec->raster == 1 && window_rows == 4 && s.r == 5 && s.w % 4 == 0;
+    L.unroll = seven ? 7 : window_rows;
     // a record that names the register-window form (or a strip height it does not have) on a filter without one runs
     // another kernel form than it was written for: a reformulation, invalid when nothing may be reformulated
-    if (window_rows != rec->unroll) changed |= TT_CHG_FORM;
+    if (L.unroll != rec->unroll) changed |= TT_CHG_FORM;
     int bx = std::min(rec->block_x, round_up(w->Q, items));
     bx = round_up(bx, items);
     if (bx != rec->block_x || L.block_y != rec->block_y) changed |= TT_CHG_BLOCK;
@@ -920,7 +922,7 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     d.tiles_c = (s.c + d.tile_c - 1) / d.tile_c;
     d.tiles_h = (w->P + d.tile_h - 1) / d.tile_h;
     d.tiles_w = (w->Q + d.tile_w - 1) / d.tile_w;
-    d.window_rows = window_rows;
+    d.window_rows = window_rows;                           // (a box-staged plan may change it below)
     d.vec_in = (s.w % 4) == 0;
     long long smem = window_rows ? 0 : (long long)d.tile_c * ((long long)d.in_h * d.in_w + d.R * d.S + 1) * 4;
     I = tt_apply_info{};
@@ -931,14 +933,18 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     L.raster = 0;
     if (rec->raster == 1 && window_rows > 0 && (s.w % 4) == 0) {
         const long long planes = (long long)s.n * s.c;
-        // a 5x5 filter's tallest strip becomes one of seven rows where that covers the tile as well and the chip has tiles to spare: a
-        // strip then reads 11 rows for 7, not 8 for 4 (3x3: 9 for 7 against 6 for 4, and it was slower on 56-pixel rows, 157 -> 173 us)
-        int rows = window_rows;
-        if (rows == 4 && s.r == 5 && round_up(d.tile_h, 7) <= round_up(d.tile_h, 4) && (planes + d.tile_c - 1) / d.tile_c * d.tiles_h * d.tiles_w >= 148 * 4) rows = 7;
-        // tiles keep to one image, in groups of channels as equal as they come; everything below is about the tile that runs
+        // Unless the record is to run as written (strict mode): tiles keep to one image, in groups of channels as equal as they
+        // come, and a 5x5 filter's tallest strip becomes one of seven rows where that covers the tile as well and the chip has tiles to spare: a
+        // strip then reads 11 rows for 7, not 8 for 4 (3x3: 9 for 7 against 6 for 4, and it was slower on 56-pixel rows, 157 -> 173 us).
+        // Everything below is about the tile that runs, and so is the legal record.
+        int rows = L.unroll;
         DwArgs t = d;
         const int groups = (s.c + t.tile_c - 1) / t.tile_c;
-        t.tile_c = (s.c + groups - 1) / groups;
+        if (!strict) {
+            rows = window_rows;
+            if (rows == 4 && s.r == 5 && round_up(d.tile_h, 7) <= round_up(d.tile_h, 4) && (planes + d.tile_c - 1) / d.tile_c * d.tiles_h * d.tiles_w >= 148 * 4) rows = 7;
+            t.tile_c = (s.c + groups - 1) / groups;
+        }
         int stg = 0;
         auto smem_of = [&](int n) { return (long long)n * t.stage_bytes + t.wstage_bytes + 128; };
         for (const bool may_widen : {true, false}) {       // (a wider row that does not fit is no reason to leave this form)
@@ -954,7 +960,11 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
             L.raster = 1; L.stages = stg;
             d.tma_stages = stg;
             // no more threads than a tile has strips
-            th = std::min(th, round_up(d.tile_c * ((d.tile_h + rows - 1) / rows) * (d.tile_w / items), 32));
+            if (!strict) th = std::min(th, round_up(d.tile_c * ((d.tile_h + rows - 1) / rows) * (d.tile_w / items), 32));
+            L.unroll = rows; L.tile_m = d.tile_c; L.threads = th;
+            if (L.unroll != rec->unroll) I.changed |= TT_CHG_FORM;
+            if (L.tile_m != rec->tile_m) I.changed |= TT_CHG_TILE_M;
+            if (L.threads != rec->threads) I.changed |= TT_CHG_BLOCK;
             const long long total = (long long)groups * s.n * d.tiles_h * d.tiles_w;
             if (total > 0x7fffffffLL) return TT_ERR_RESOURCE;
             d.total_tiles = (int)total;
@@ -968,6 +978,7 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
         }
     }
     if (rec->raster != 0) { if (strict) return TT_ERR_INVALID_SCHEDULE; I.changed |= TT_CHG_FORM; }
+    L.unroll = window_rows;
     I.legal = L;
     I.grid_x = (int)std::min<long long>(gx, 0x7fffffff); I.grid_y = s.n; I.grid_z = 1;
     I.threads = th; I.smem_bytes = (int)std::min<long long>(smem, 0x7fffffff);

@@ -1088,3 +1088,20 @@ def test_tap_major_records_run_as_written_in_strict_mode(cg):
         assert status == B.TT_OK and (info.legal.tile_n, info.legal.stages, info.grid_y) == (tn, st, cg)
         probe.close()
         run_spec(sp, rec, a, ref, mode=B.TT_MODE_STRICT, ref_elem=re)
+
+
+@pytest.mark.parametrize("shape, kw", [
+    ((9, 50, 20, 28, 5, 1), dict(tile_m=7, block_y=20, block_x=28, threads=256, unroll=7, stages=3)),      # 8 groups, the last of one channel
+    ((9, 50, 20, 28, 5, 2), dict(tile_m=12, block_y=5, block_x=8, threads=256, unroll=7, stages=2)),       # more threads than strips
+    ((5, 33, 17, 36, 3, 1), dict(tile_m=16, block_y=17, block_x=36, threads=64, unroll=4, stages=2)),      # two groups of 16 and one of 1
+], ids=str)
+def test_box_staged_depthwise_records_run_as_written_in_strict_mode(shape, kw):
+    n, c, h, w, r, st = shape
+    sp = W.Spec(B.TT_OP_DWCONV2D, B.make_shapes(n=n, c=c, h=h, w=w, k=c, r=r, s=r, stride_h=st, stride_w=st, pad_h=r // 2, pad_w=r // 2, has_bias=1,
+                                                act=B.TT_ACT_RELU6), 1, "dw_strict", "uniform")
+    a = W.make_inputs(sp, 99)
+    ref = util.oracle_ref(sp, a)
+    q = (w - 1) // st + 1
+    rec = B.make_record(B.TT_FAMILY_DW_SIMT, items_per_thread=4, vec_width=4 if q % 4 == 0 else 2 if q % 2 == 0 else 1, raster=1, **kw)
+    y = run_spec(sp, rec, a, ref, mode=B.TT_MODE_STRICT, ref_elem=ref)
+    np.testing.assert_array_equal(run_spec(sp, rec, a), y)

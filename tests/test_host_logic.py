@@ -820,3 +820,31 @@ def test_run_staged_depthwise_is_a_record_form():
         assert other.check(legal)[0] == B.TT_OK
         other.close()
         wl.close()
+
+
+def test_box_staged_depthwise_legal_records_say_what_runs():
+    """Evened channel groups, strips of 7 rows and threads without a strip are named by the legal record; strict mode runs the
+    record as written."""
+    for shape in ((256, 240, 28, 28, 5, 1), (2, 35, 121, 92, 5, 2), (16, 301, 114, 16, 5, 2), (64, 144, 56, 56, 3, 1), (1, 10, 9, 12, 3, 1)):
+        wl = _dw_batch(*shape)
+        _check_legal_says_what_runs(wl, DW_RECORDS)
+        wl.close()
+    wl = _dw_batch(256, 240, 28, 28, 5, 1)
+    rec = B.make_record(B.TT_FAMILY_DW_SIMT, tile_m=7, block_y=28, block_x=28, items_per_thread=4, vec_width=4, threads=256, unroll=4, raster=1, stages=2)
+    st, info = wl.check(rec)                             # 35 groups of 7 channels: 240 = 34 * 7 + 2
+    assert st == B.TT_OK and (info.legal.tile_m, info.legal.unroll, info.legal.threads) == (7, 7, 224)
+    assert info.changed & B.TT_CHG_FORM and info.changed & B.TT_CHG_BLOCK
+    rec.tile_m = 50
+    rec.block_y = 4
+    st, info = wl.check(rec)                             # 5 groups of 48, not of 50
+    assert st == B.TT_OK and (info.legal.tile_m, info.legal.unroll) == (48, 4) and info.changed & B.TT_CHG_TILE_M
+    rec.tile_m, rec.block_y = 7, 28
+    for unroll in (4, 7):
+        rec.unroll = unroll
+        st, info = wl.check(rec, mode=B.TT_MODE_STRICT)
+        assert st == B.TT_OK and (info.legal.tile_m, info.legal.unroll, info.threads) == (7, unroll, 256) and not info.changed
+    wl.close()
+    wl = _dw_batch(64, 144, 56, 56, 3, 1)                # (3x3: no such strips)
+    assert wl.check(rec, mode=B.TT_MODE_STRICT)[0] == B.TT_ERR_INVALID_SCHEDULE
+    assert wl.check(rec)[1].legal.unroll == 4
+    wl.close()
