@@ -108,7 +108,7 @@ typedef struct tt_shapes {
  *         memory; unroll = 2, 4 or 7 rows x items_per_thread = 1 or 2 columns per thread, block_x the whole row.  From 2^18
  *         outputs on every record with unroll >= 1 becomes the one of this form that is laid out for the kernel's size
  *         (legalise mode; strict mode takes that one or a register-window record as written).
- * ROW_SIMT uses block_x (threads cooperating on one row: 1..32, power of two), block_y (rows per CTA), vec_width.
+ * ROW_SIMT uses block_x (threads cooperating on one row: 1..32, power of two), block_y (rows a CTA works on at a time), vec_width.
  * origin_* say which kernel the record was tuned on (its "native" kernel, Section 3). */
 typedef struct tt_schedule_record {
     uint32_t version;      /* TT_RECORD_VERSION */
@@ -186,9 +186,11 @@ typedef struct tt_apply_info {
     tt_schedule_record legal;   /* the record after legalisation: what will actually run */
     int32_t changed;            /* bit mask of fields legalisation had to change (TT_CHG_*) */
     int32_t grid_x, grid_y, grid_z, threads;
-    int32_t smem_bytes, tmem_cols;
+    int32_t smem_bytes;         /* dynamic shared memory per CTA that the legal record needs; a launch of the one-tile GEMM
+                                   form takes what is left over as well, for more stages */
+    int32_t tmem_cols;
     int64_t workspace_bytes;
-    int32_t launches;           /* kernels per tt_run (2 with split-K) */
+    int32_t launches;           /* kernels per tt_run (2 with the filter re-pack of k_order = 1) */
 } tt_apply_info;
 
 enum { TT_CHG_TILE_M = 1, TT_CHG_TILE_N = 2, TT_CHG_TILE_K = 4, TT_CHG_STAGES = 8, TT_CHG_SPLIT_K = 16,

@@ -20,7 +20,7 @@ cudaError_t gemm_cluster_fits(const GemmArgs& g, int smem_bytes, int* fits);
 cudaError_t launch_repack(const float* w, float* out, const ConvPmArgs& g, cudaStream_t st);
 cudaError_t launch_conv_pm(const tt_apply_info& I, const ConvPmArgs& g, const void* tmap_w, cudaStream_t st);
 cudaError_t conv_pm_cluster_fits(const tt_apply_info& I, const ConvPmArgs& g, int* fits);
-cudaError_t launch_floor(const tt_apply_info& I, int cluster, cudaStream_t st);
+cudaError_t launch_floor(const tt_apply_info& I, int smem_bytes, int cluster, cudaStream_t st);
 cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const TmapPair& maps, cudaStream_t st);
 
 namespace {
@@ -388,8 +388,7 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
     } else {
         RowArgs r = p.row;
         r.x = static_cast<const float*>(t->x); r.y = static_cast<float*>(t->y);
-        r.aligned = ((reinterpret_cast<uintptr_t>(t->y) | reinterpret_cast<uintptr_t>(t->x)) & 15u) == 0;
-        if (!r.aligned) r.vec = 1;
+        if (((reinterpret_cast<uintptr_t>(t->y) | reinterpret_cast<uintptr_t>(t->x)) & 15u) != 0) { r.vec = 1; r.chunk = r.warps = 0; }
         r.status = w->status_word; r.wait_ns = w->wait_ns;
         e = launch_row(p.info, r, st);
     }
@@ -453,8 +452,11 @@ static tt_status time_applied(tt_workload* w, const tt_tensors* sets, size_t n_s
         for (int i = 0; i < n; ++i) {
             if (o.floor) {
                 // the launch floor of the applied record: an empty kernel with the same launch shape
-                for (int l = 0; l < w->plan.info.launches; ++l)
-                    if (launch_floor(w->plan.info, w->family != TT_FAMILY_GEMM_TC ? 0 : w->plan.repack ? (w->plan.pm.split > 1 ? w->plan.pm.split : 0) : w->plan.g.cluster, s) != cudaSuccess) {
+                const Plan& p = w->plan;
+                const bool gemm = w->family == TT_FAMILY_GEMM_TC;
+                const int cluster = !gemm ? 0 : p.repack ? (p.pm.split > 1 ? p.pm.split : 0) : p.g.cluster;
+                for (int l = 0; l < p.info.launches; ++l)
+                    if (launch_floor(p.info, p.run_smem ? p.run_smem : p.info.smem_bytes, cluster, s) != cudaSuccess) {
                         cudaGetLastError();
                         return TT_ERR_CUDA;
                     }

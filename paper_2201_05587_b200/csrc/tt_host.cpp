@@ -1010,11 +1010,27 @@ static tt_status legalise_row(const tt_workload* w, const tt_schedule_record* re
     r.rows = rows; r.cols = s.nn; r.scale = s.scale; r.lanes_per_row = lanes; r.rows_per_cta = rpc; r.vec = vec;
     tt_apply_info& I = plan->info;
     I = tt_apply_info{};
-    I.legal = L; I.changed = changed;
-    const long long gx = (rows + rpc - 1) / rpc;
-    I.grid_x = (int)std::min<long long>(gx, 0x7fffffff); I.grid_y = 1; I.grid_z = 1;
+    long long gx = (rows + rpc - 1) / rpc;
+    const bool too_many = gx > 0x7fffffffLL;
     I.threads = rpc * lanes; I.launches = 1;
-    if (gx > 0x7fffffffLL) return TT_ERR_RESOURCE;
+    if ((s.nn & 3) != 0) {
+        // Ragged rows pass through shared memory as long as a lane's values stay in registers and a warp's rows fit.  A chunk is the
+        // least number of rows that is a multiple of four (whole 16-byte groups) and keeps all lanes busy; warps per CTA follow the
+        // record, fewer where their rows would not fit.  The lanes' accesses are single values.
+        const int per_lane = (s.nn + lanes - 1) / lanes, chunk = std::max(4, 32 / lanes);
+        const int warps = (int)std::min<long long>(rpc * lanes / 32, kRowSmem / ((long long)chunk * s.nn * 4));
+        if (warps >= 1 && per_lane <= kRaggedMost && !(strict && (vec != 1 || warps * 32 != rpc * lanes))) {
+            r.warps = warps; r.chunk = chunk;
+            L.vec_width = 1; L.block_y = warps * 32 / lanes;
+            if (L.vec_width != rec->vec_width) changed |= TT_CHG_VEC;
+            if (L.block_y != rec->block_y) changed |= TT_CHG_BLOCK;
+            gx = (rows + (long long)warps * chunk - 1) / ((long long)warps * chunk);
+            I.threads = 32 * warps; I.smem_bytes = warps * chunk * s.nn * 4;
+        }
+    }
+    I.legal = L; I.changed = changed;
+    I.grid_x = (int)std::min<long long>(gx, 0x7fffffff); I.grid_y = 1; I.grid_z = 1;
+    if (too_many) return TT_ERR_RESOURCE;
     return TT_OK;
 }
 

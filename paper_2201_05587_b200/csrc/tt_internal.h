@@ -11,6 +11,8 @@ constexpr int kHwTileM = 128;           // tcgen05 accumulator rows per CTA (cta
 constexpr int kMaxStages = 8;
 constexpr int kSmemLimit = 232448;      // 227 KB opt-in shared memory per CTA on sm_100
 constexpr int kDynSmemLimit = kSmemLimit - 6144;  // what is left for dynamic shared memory beside barriers
+constexpr int kRowSmem = 100 * 1024;    // shared memory of a CTA of the ragged softmax, so that two fit an SM
+constexpr int kRaggedMost = 65;         // ... and the values a lane of it keeps in registers at most
 constexpr int kGatherWarps = 8;
 constexpr int kGatherThreads = kGatherWarps * 32;
 constexpr int kGemmThreads = 64 + kGatherThreads;   // warp 0 TMA, warp 1 MMA + TMEM, warps 2-9 gather + epilogue
@@ -133,7 +135,7 @@ struct DwArgs {
 struct RowArgs {
     const float* x; float* y; long long rows; int cols; float scale;
     int lanes_per_row, rows_per_cta, vec;
-    int aligned;       // x and y start on 16-byte boundaries
+    int warps, chunk;  // > 0: ragged rows through shared memory, `chunk` rows a warp (x and y on 16-byte boundaries)
     unsigned* status; unsigned long long wait_ns;   // the workload's status word and wait limit
 };
 

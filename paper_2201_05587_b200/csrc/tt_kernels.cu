@@ -2351,7 +2351,6 @@ __global__ void tt_softmax_cached_kernel(const RowArgs a) {
 // 151296 rows of 197 columns: 136 us in three passes of 4-byte accesses from memory, 57 us with guards on every value,
 // 38 us this way (6.3 TB/s; floor 36 us).
 constexpr int kRaggedExact = 32;                         // values per lane up to which there is an instantiation for each count
-constexpr int kRowSmem = 100 * 1024;                     // shared memory of a CTA of this kernel, so that two fit an SM
 template <int NV>
 __global__ void tt_softmax_ragged_kernel(const RowArgs a, int chunk) {
     extern __shared__ __align__(16) float sm_rows[];
@@ -2562,7 +2561,7 @@ cudaError_t gemm_cluster_fits(const GemmArgs& g, int smem_bytes, int* fits) {
     return cudaSuccess;
 }
 
-cudaError_t launch_floor(const tt_apply_info& I, int cluster, cudaStream_t st) {
+cudaError_t launch_floor(const tt_apply_info& I, int smem_bytes, int cluster, cudaStream_t st) {
     static int attr_set_for = -1;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -2573,7 +2572,7 @@ cudaError_t launch_floor(const tt_apply_info& I, int cluster, cudaStream_t st) {
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(I.grid_x, I.grid_y, I.grid_z); cfg.blockDim = dim3(I.threads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)I.smem_bytes; cfg.stream = st;
+    cfg.dynamicSmemBytes = (size_t)smem_bytes; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     int n_attr = 0;
     attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -2697,20 +2696,19 @@ cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st)
 }
 
 template <int NV>
-static cudaError_t launch_row_ragged(const RowArgs& row, int warps, int chunk, cudaStream_t st) {
-    const size_t smem = (size_t)warps * chunk * row.cols * 4;
-    static thread_local int limit_set_for = -1;
+static cudaError_t launch_row_ragged(const tt_apply_info& I, const RowArgs& row, cudaStream_t st) {
+    static std::atomic<uint64_t> raised;                 // a bit per device
     int dev = 0;
     cudaGetDevice(&dev);
-    if (limit_set_for != dev) {
+    const uint64_t bit = 1ull << (dev & 63);
+    if (!(raised.load(std::memory_order_relaxed) & bit)) {
         cudaError_t e = cudaFuncSetAttribute(tt_softmax_ragged_kernel<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem);
         if (e != cudaSuccess) return e;
-        limit_set_for = dev;
+        raised.fetch_or(bit, std::memory_order_relaxed);
     }
-    const long long per_cta = (long long)warps * chunk;
-    return launch_serialized(tt_softmax_ragged_kernel<NV>, dim3((unsigned)((row.rows + per_cta - 1) / per_cta), 1, 1), 32u * (unsigned)warps, smem, st, row, chunk);
+    return launch_serialized(tt_softmax_ragged_kernel<NV>, dim3((unsigned)I.grid_x, 1, 1), (unsigned)I.threads, (size_t)I.smem_bytes, st, row, row.chunk);
 }
-typedef cudaError_t (*RaggedLauncher)(const RowArgs&, int, int, cudaStream_t);
+typedef cudaError_t (*RaggedLauncher)(const tt_apply_info&, const RowArgs&, cudaStream_t);
 template <int... I>
 static RaggedLauncher ragged_launcher(int per_lane, std::integer_sequence<int, I...>) {
     static const RaggedLauncher exact[] = {launch_row_ragged<I + 1>...};
@@ -2727,21 +2725,14 @@ cudaError_t launch_row(const tt_apply_info& I, const RowArgs& row, cudaStream_t 
         if (per_lane <= 4) return launch_serialized(tt_softmax_cached_kernel<4>, grid, (unsigned)I.threads, 0, st, row);
         if (per_lane <= 8) return launch_serialized(tt_softmax_cached_kernel<8>, grid, (unsigned)I.threads, 0, st, row);
         if (per_lane <= 16) return launch_serialized(tt_softmax_cached_kernel<16>, grid, (unsigned)I.threads, 0, st, row);
-    } else if ((row.cols & 3) != 0 && row.aligned) {
-        // Ragged rows, whatever width the record asked for (it was lowered to what divides the row): through shared memory,
-        // as long as a lane's values stay in registers and a warp's rows fit.  A chunk is the least number of rows that is
-        // a multiple of four and keeps all lanes busy; warps per CTA follow the record, fewer where their rows would not fit.
+    } else if (row.chunk > 0) {
         const int per_lane = (row.cols + row.lanes_per_row - 1) / row.lanes_per_row;
-        const int chunk = std::max(4, 32 / row.lanes_per_row);
-        const long long per_warp = (long long)chunk * row.cols * 4;
-        const int warps = (int)std::min<long long>(std::max(1, I.threads / 32), kRowSmem / per_warp);
-        if (warps >= 1) {
-            if (per_lane <= kRaggedExact) return ragged_launcher(per_lane, std::make_integer_sequence<int, kRaggedExact>{})(row, warps, chunk, st);
-            if (per_lane <= 48) return launch_row_ragged<48>(row, warps, chunk, st);
-            if (per_lane <= 65) return launch_row_ragged<65>(row, warps, chunk, st);
-        }
+        if (per_lane <= kRaggedExact) return ragged_launcher(per_lane, std::make_integer_sequence<int, kRaggedExact>{})(I, row, st);
+        if (per_lane <= 48) return launch_row_ragged<48>(I, row, st);
+        return launch_row_ragged<kRaggedMost>(I, row, st);
     }
-    return launch_serialized(tt_softmax_kernel, dim3(I.grid_x, 1, 1), (unsigned)I.threads, 0, st, row);
+    const unsigned grid = (unsigned)((row.rows + row.rows_per_cta - 1) / row.rows_per_cta);
+    return launch_serialized(tt_softmax_kernel, dim3(grid, 1, 1), (unsigned)(row.rows_per_cta * row.lanes_per_row), 0, st, row);
 }
 
 }  // namespace tt

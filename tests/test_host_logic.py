@@ -848,3 +848,24 @@ def test_box_staged_depthwise_legal_records_say_what_runs():
     assert wl.check(rec, mode=B.TT_MODE_STRICT)[0] == B.TT_ERR_INVALID_SCHEDULE
     assert wl.check(rec)[1].legal.unroll == 4
     wl.close()
+
+
+def test_softmax_legal_records_say_what_runs():
+    """Ragged rows: warps that fit, single-value accesses and the launch that the rows are staged in; strict mode as written."""
+    recs = [B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=bx, block_y=by, vec_width=vw) for bx in (1, 2, 4, 8, 16, 32) for by in (1, 4, 16, 32) for vw in (1, 2, 4)]
+    for rows, cols in ((151296, 197), (35, 1), (1000, 2), (4097, 1023), (17, 2046), (17, 2081), (300, 64), (300, 66), (5, 4097)):
+        wl = W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(1, rows, cols, 1.0), 1, "rows").workload()
+        _check_legal_says_what_runs(wl, recs)
+        for rec in recs:
+            st, info = wl.check(rec)
+            assert st == B.TT_OK and info.smem_bytes <= 100 * 1024 and info.threads <= 1024
+            assert info.legal.block_x * info.legal.block_y == info.threads
+            if info.smem_bytes:
+                assert cols % 4 and info.legal.vec_width == 1 and info.smem_bytes % (16 * info.threads // 32) == 0
+        wl.close()
+    wl = W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(1, 300, 66, 1.0), 1, "rows").workload()
+    rec = B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=8, block_y=4, vec_width=2)
+    assert wl.check(rec)[1].legal.vec_width == 1 and wl.check(rec)[1].changed & B.TT_CHG_VEC
+    st, info = wl.check(rec, mode=B.TT_MODE_STRICT)
+    assert st == B.TT_OK and info.legal.vec_width == 2 and info.smem_bytes == 0
+    wl.close()
