@@ -388,7 +388,7 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
     } else {
         RowArgs r = p.row;
         r.x = static_cast<const float*>(t->x); r.y = static_cast<float*>(t->y);
-        if (((reinterpret_cast<uintptr_t>(t->y) | reinterpret_cast<uintptr_t>(t->x)) & 15u) != 0) { r.vec = 1; r.chunk = r.warps = 0; }
+        if (((reinterpret_cast<uintptr_t>(t->y) | reinterpret_cast<uintptr_t>(t->x)) & 15u) != 0) { r.vec = 1; r.cached = r.chunk = r.warps = 0; }
         r.status = w->status_word; r.wait_ns = w->wait_ns;
         e = launch_row(p.info, r, st);
     }

@@ -1016,9 +1016,9 @@ static tt_status legalise_row(const tt_workload* w, const tt_schedule_record* re
     if ((s.nn & 3) != 0) {
         // Ragged rows pass through shared memory as long as a lane's values stay in registers and a warp's rows fit.  A chunk is the
         // least number of rows that is a multiple of four (whole 16-byte groups) and keeps all lanes busy; warps per CTA follow the
-        // record, fewer where their rows would not fit.  The lanes' accesses are single values.
+        // record, fewer where their rows or registers would not fit.  The lanes' accesses are single values.
         const int per_lane = (s.nn + lanes - 1) / lanes, chunk = std::max(4, 32 / lanes);
-        const int warps = (int)std::min<long long>(rpc * lanes / 32, kRowSmem / ((long long)chunk * s.nn * 4));
+        const int warps = (int)std::min<long long>(std::min(rpc * lanes, ragged_threads(per_lane)) / 32, kRowSmem / ((long long)chunk * s.nn * 4));
         if (warps >= 1 && per_lane <= kRaggedMost && !(strict && (vec != 1 || warps * 32 != rpc * lanes))) {
             r.warps = warps; r.chunk = chunk;
             L.vec_width = 1; L.block_y = warps * 32 / lanes;
@@ -1026,6 +1026,16 @@ static tt_status legalise_row(const tt_workload* w, const tt_schedule_record* re
             if (L.block_y != rec->block_y) changed |= TT_CHG_BLOCK;
             gx = (rows + (long long)warps * chunk - 1) / ((long long)warps * chunk);
             I.threads = 32 * warps; I.smem_bytes = warps * chunk * s.nn * 4;
+        }
+    }
+    const int groups = ((s.nn >> 2) + lanes - 1) / lanes;      // 16-byte groups per lane
+    if (vec == 4 && groups <= kCachedMost && !(strict && rpc * lanes > cached_threads(groups))) {
+        // rows that fit the lanes' registers are read once, by as many threads as have that many registers
+        r.cached = groups;
+        if (rpc * lanes > cached_threads(groups)) {
+            rpc = r.rows_per_cta = cached_threads(groups) / lanes;
+            L.block_y = rpc; changed |= TT_CHG_BLOCK;
+            gx = (rows + rpc - 1) / rpc; I.threads = rpc * lanes;
         }
     }
     I.legal = L; I.changed = changed;

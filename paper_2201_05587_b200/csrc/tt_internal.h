@@ -13,6 +13,10 @@ constexpr int kSmemLimit = 232448;      // 227 KB opt-in shared memory per CTA o
 constexpr int kDynSmemLimit = kSmemLimit - 6144;  // what is left for dynamic shared memory beside barriers
 constexpr int kRowSmem = 100 * 1024;    // shared memory of a CTA of the ragged softmax, so that two fit an SM
 constexpr int kRaggedMost = 65;         // ... and the values a lane of it keeps in registers at most
+constexpr int kCachedMost = 16;         // 16-byte groups a lane of the register-resident softmax keeps at most
+// Threads that their registers (both kernels are compiled for it) leave room for: values, or groups, per lane.
+constexpr int ragged_threads(int values) { return values <= 17 ? 1024 : values <= 27 ? 768 : values <= 32 ? 640 : 256; }
+constexpr int cached_threads(int groups) { return groups <= 8 ? 1024 : 512; }
 constexpr int kGatherWarps = 8;
 constexpr int kGatherThreads = kGatherWarps * 32;
 constexpr int kGemmThreads = 64 + kGatherThreads;   // warp 0 TMA, warp 1 MMA + TMEM, warps 2-9 gather + epilogue
@@ -135,6 +139,7 @@ struct DwArgs {
 struct RowArgs {
     const float* x; float* y; long long rows; int cols; float scale;
     int lanes_per_row, rows_per_cta, vec;
+    int cached;        // > 0: 16-byte groups per lane, kept in registers (x and y on 16-byte boundaries)
     int warps, chunk;  // > 0: ragged rows through shared memory, `chunk` rows a warp (x and y on 16-byte boundaries)
     unsigned* status; unsigned long long wait_ns;   // the workload's status word and wait limit
 };

@@ -2302,7 +2302,7 @@ __global__ void tt_softmax_kernel(const RowArgs a) {
 // so x is read from memory once and each exponential is computed once.  Rows of up to lanes_per_row * 4 * NV columns
 // whose length is a multiple of 4 and whose pointers are 16-byte aligned; other rows take the two kernels around it.
 template <int NV>
-__global__ void tt_softmax_cached_kernel(const RowArgs a) {
+__global__ void __launch_bounds__(cached_threads(NV)) tt_softmax_cached_kernel(const RowArgs a) {
     pdl_allow_next();
     pdl_wait_prev();
     const int lpr = a.lanes_per_row;
@@ -2352,7 +2352,7 @@ __global__ void tt_softmax_cached_kernel(const RowArgs a) {
 // 38 us this way (6.3 TB/s; floor 36 us).
 constexpr int kRaggedExact = 32;                         // values per lane up to which there is an instantiation for each count
 template <int NV>
-__global__ void tt_softmax_ragged_kernel(const RowArgs a, int chunk) {
+__global__ void __launch_bounds__(ragged_threads(NV)) tt_softmax_ragged_kernel(const RowArgs a, int chunk) {
     extern __shared__ __align__(16) float sm_rows[];
     __shared__ uint64_t landed[32];
     pdl_allow_next();
@@ -2716,15 +2716,13 @@ static RaggedLauncher ragged_launcher(int per_lane, std::integer_sequence<int, I
 }
 
 cudaError_t launch_row(const tt_apply_info& I, const RowArgs& row, cudaStream_t st) {
-    if ((row.cols & 3) == 0 && row.vec == 4) {
-        // rows that fit the lanes' registers (and allow 16-byte accesses) are read once: at most 16 groups per lane
-        const int per_lane = ((row.cols >> 2) + row.lanes_per_row - 1) / row.lanes_per_row;
+    if (row.cached > 0) {
         const dim3 grid(I.grid_x, 1, 1);
-        if (per_lane == 1) return launch_serialized(tt_softmax_cached_kernel<1>, grid, (unsigned)I.threads, 0, st, row);
-        if (per_lane == 2) return launch_serialized(tt_softmax_cached_kernel<2>, grid, (unsigned)I.threads, 0, st, row);
-        if (per_lane <= 4) return launch_serialized(tt_softmax_cached_kernel<4>, grid, (unsigned)I.threads, 0, st, row);
-        if (per_lane <= 8) return launch_serialized(tt_softmax_cached_kernel<8>, grid, (unsigned)I.threads, 0, st, row);
-        if (per_lane <= 16) return launch_serialized(tt_softmax_cached_kernel<16>, grid, (unsigned)I.threads, 0, st, row);
+        if (row.cached == 1) return launch_serialized(tt_softmax_cached_kernel<1>, grid, (unsigned)I.threads, 0, st, row);
+        if (row.cached == 2) return launch_serialized(tt_softmax_cached_kernel<2>, grid, (unsigned)I.threads, 0, st, row);
+        if (row.cached <= 4) return launch_serialized(tt_softmax_cached_kernel<4>, grid, (unsigned)I.threads, 0, st, row);
+        if (row.cached <= 8) return launch_serialized(tt_softmax_cached_kernel<8>, grid, (unsigned)I.threads, 0, st, row);
+        return launch_serialized(tt_softmax_cached_kernel<kCachedMost>, grid, (unsigned)I.threads, 0, st, row);
     } else if (row.chunk > 0) {
         const int per_lane = (row.cols + row.lanes_per_row - 1) / row.lanes_per_row;
         if (per_lane <= kRaggedExact) return ragged_launcher(per_lane, std::make_integer_sequence<int, kRaggedExact>{})(I, row, st);

@@ -1105,3 +1105,15 @@ def test_box_staged_depthwise_records_run_as_written_in_strict_mode(shape, kw):
     rec = B.make_record(B.TT_FAMILY_DW_SIMT, items_per_thread=4, vec_width=4 if q % 4 == 0 else 2 if q % 2 == 0 else 1, raster=1, **kw)
     y = run_spec(sp, rec, a, ref, mode=B.TT_MODE_STRICT, ref_elem=ref)
     np.testing.assert_array_equal(run_spec(sp, rec, a), y)
+
+
+@pytest.mark.parametrize("cols", [577, 637, 865, 1023, 1025, 1028, 1535, 2047, 2048, 2081])
+def test_softmax_rows_under_the_largest_blocks(cols):
+    """1024 threads of lanes that keep up to 16 groups or 65 values of a row each: more registers than an SM has."""
+    spec = W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(3, 23, cols, scale=0.125), 1, f"softmax_69x{cols}", "bert")
+    a = W.make_inputs(spec, 12)
+    ref = util.oracle_ref(spec, a)
+    for bx in (8, 32):
+        rec = B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=bx, block_y=1024 // bx, vec_width=4 if cols % 4 == 0 else 1)
+        for mode in (B.TT_MODE_LEGALISE, B.TT_MODE_STRICT):
+            run_spec(spec, rec, a, ref, mode=mode, ref_elem=ref)

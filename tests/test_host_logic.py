@@ -869,3 +869,17 @@ def test_softmax_legal_records_say_what_runs():
     st, info = wl.check(rec, mode=B.TT_MODE_STRICT)
     assert st == B.TT_OK and info.legal.vec_width == 2 and info.smem_bytes == 0
     wl.close()
+
+
+def test_softmax_threads_leave_their_registers_room():
+    """A lane that keeps many values takes many registers: fewer threads per CTA, said by the legal record."""
+    for cols, lanes, most in ((2048, 32, 512), (1028, 32, 512), (1024, 32, 1024), (576, 16, 512), (637, 32, 768), (1023, 32, 640), (1537, 32, 256), (47, 1, 256), (577, 32, 1024)):
+        wl = W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(1, 5000, cols, 1.0), 1, "rows").workload()
+        rec = B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=lanes, block_y=1024 // lanes, vec_width=4 if cols % 4 == 0 else 1)
+        st, info = wl.check(rec)
+        assert st == B.TT_OK and info.threads <= most, (cols, lanes, info.threads)
+        assert (info.threads == 1024) == (info.legal.block_y == rec.block_y) and (info.threads == 1024 or info.changed & B.TT_CHG_BLOCK)
+        _check_legal_says_what_runs(wl, [rec])
+        st, info = wl.check(rec, mode=B.TT_MODE_STRICT)       # as written, in passes over memory
+        assert st == B.TT_OK and info.threads == 1024
+        wl.close()
