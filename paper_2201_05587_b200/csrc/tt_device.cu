@@ -353,6 +353,12 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
             if (p.a_tensor == 1 && g.a_mode == OPM_TMA) g.w_operand = 1;
             else if (p.b_tensor == 1 && g.b_mode == OPM_TMA) g.w_operand = 2;
         }
+        // A row-contiguous operand that does not start on 16 bytes cannot come by TMA: it is gathered into a K-major tile (which
+        // takes no more room than the MN-major one).  Images with rows of 16-byte multiples are asked for that in every form.
+        if (!g.persistent && (w->op != TT_OP_CONV2D || w->sh.w % 4 != 0)) {
+            if (g.a_mode == OPM_TMA_MN && (reinterpret_cast<uintptr_t>(a_ptr) & 15u) != 0) { g.a_mode = OPM_GATHER_ROWS; g.idesc &= ~(1u << 15); }
+            if (g.b_mode == OPM_TMA_MN && (reinterpret_cast<uintptr_t>(b_ptr) & 15u) != 0) { g.b_mode = OPM_GATHER_ROWS; g.idesc &= ~(1u << 16); }
+        }
         const TmapPair* maps = nullptr;
         const tt_status s = tensor_maps_for(w, g, a_ptr, b_ptr, &maps);
         if (s != TT_OK) return s;

@@ -1117,3 +1117,33 @@ def test_softmax_rows_under_the_largest_blocks(cols):
         rec = B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=bx, block_y=1024 // bx, vec_width=4 if cols % 4 == 0 else 1)
         for mode in (B.TT_MODE_LEGALISE, B.TT_MODE_STRICT):
             run_spec(spec, rec, a, ref, mode=mode, ref_elem=ref)
+
+
+@pytest.mark.parametrize("spec, operand", [
+    (W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(3, 37, 14, 14, 70, 1, 1, 1, 0, True, B.TT_ACT_RELU, True), 1, "off_conv1x1_14", "uniform"), "x"),
+    (W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(2, 64, 6, 6, 40, 1, 1, 1, 0, True, B.TT_ACT_RELU6), 1, "off_conv1x1_6", "uniform"), "x"),
+    (W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(4, 70, 132, 36, False), 1, "off_bmm_nn", "bert"), "w"),
+    (W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(3, 130, 44, 35, False), 1, "off_bmm_nn_odd_k", "bert"), "w"),
+], ids=lambda v: v.name if isinstance(v, W.Spec) else v)
+def test_row_contiguous_operands_that_start_anywhere(spec, operand):
+    """A pointwise convolution's image, or an NN product's second operand, that starts inside a 16-byte group: no TMA box can fetch
+    it, the one-tile form gathers it."""
+    import torch
+    a = W.make_inputs(spec, 92)
+    ref = util.oracle_ref(spec, a)
+    re = elem_ref(spec, a, ref)
+    for off, rec in ((1, tc(tile_n=16, tile_k=8, stages=2, mma_m_axis=1)), (2, tc(tile_n=64, tile_k=32, stages=3, mma_m_axis=2)),
+                     (3, tc(tile_n=48, tile_k=32, stages=2, split_k=2, mma_m_axis=1, acc_split=2)), (1, tc(tile_n=32, tile_k=8, stages=4, split_k=4, mma_m_axis=2))):
+        wl = spec.workload()
+        wl.apply(rec)
+        wl.set_constant_weights(True)
+        t, _ = W.device_tensors(spec, a)
+        t["y"], buf = guarded_output(spec)
+        n = t[operand].numel()
+        t[operand] = torch.empty(n + 4, device="cuda")[off:off + n].view(t[operand].shape).copy_(t[operand])
+        wl.run(B.tensors(t["x"], t["w"], t["bias"], t["residual"], t["y"]))
+        assert wl.status() == B.TT_OK and guards_intact(buf)
+        y = t["y"].cpu().numpy()
+        assert util.rel_l2(y, ref) <= util.TOL_TF32, (spec.name, rec.short())
+        assert float(np.abs(y.astype(np.float64) - re).max()) <= ELEM_TF32 * float(np.abs(re).max())
+        wl.close()
