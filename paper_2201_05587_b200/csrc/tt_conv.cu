@@ -37,7 +37,6 @@
 #include <cuda_runtime.h>
 #include <cuda.h>
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 #include "tt_ptx.cuh"
 
@@ -478,14 +477,8 @@ cudaError_t launch_repack(const float* w, float* out, const ConvPmArgs& g, cudaS
 }
 
 static cudaError_t raise_smem_limit() {
-    static std::atomic<uint64_t> raised;                 // a bit per device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = 1ull << (dev & 63);
-    if (raised.load(std::memory_order_relaxed) & bit) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(tt_conv_pm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-    if (e == cudaSuccess) raised.fetch_or(bit, std::memory_order_relaxed);
-    return e;
+    static OncePerDevice once;
+    return once([] { return cudaFuncSetAttribute(tt_conv_pm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
 }
 
 static void launch_config(const tt_apply_info& I, const ConvPmArgs& g, cudaLaunchConfig_t* cfg, cudaLaunchAttribute (&attr)[2]) {

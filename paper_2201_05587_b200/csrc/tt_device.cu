@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <cuda.h>
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cstring>
 #include <mutex>
@@ -32,18 +33,15 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 // The driver entry point is looked up through the runtime, so the library links against cudart only and loads
 // on machines without a driver.
 EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const EncodeTiledFn fn = [] {                 // (looked up by one thread, the others wait for it)
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-        else
-            cudaGetLastError();
-    }
+            return reinterpret_cast<EncodeTiledFn>(p);
+        cudaGetLastError();
+        return EncodeTiledFn(nullptr);
+    }();
     return fn;
 }
 
@@ -981,7 +979,7 @@ namespace tt {
 namespace {
 constexpr int kMaxDevices = 64;
 constexpr int64_t kStaticStatusBytes = 512;   // the status area, sized like the one tt_schedule_apply allocates
-unsigned char* g_scratch_addr[kMaxDevices] = {};
+std::atomic<unsigned char*> g_scratch_addr[kMaxDevices] = {};
 
 // In host code the array's name only stands for the symbol; the device address is asked for once per device,
 // with that device current.

@@ -22,7 +22,6 @@
 #include <cstdint>
 #include <cstring>
 #include <algorithm>
-#include <atomic>
 #include <utility>
 #include "tt_ptx.cuh"
 
@@ -2457,19 +2456,10 @@ static int gemm_form(const GemmArgs& g) {
 // Which instantiation a plan runs; its shared-memory limit is raised once per device.  Which build (two CTAs per SM) is the
 // record's choice (ctas_per_sm), resolved by the legaliser.
 static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel* out) {
-    static std::atomic<uint64_t> raised[2][2][5];           // a bit per device
-    const int two = g.two_per_sm && gemm_two_per_sm(smem_bytes, g.tmem_cols), form = gemm_form(g);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = 1ull << (dev & 63);
-    const int cl = g.cluster > 0;
+    static OncePerDevice raised[2][2][5];
+    const int two = g.two_per_sm && gemm_two_per_sm(smem_bytes, g.tmem_cols), form = gemm_form(g), cl = g.cluster > 0;
     *out = kGemmKernels[two][cl][form];
-    if (!(raised[two][cl][form].load(std::memory_order_relaxed) & bit)) {
-        cudaError_t e = cudaFuncSetAttribute(*out, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-        if (e != cudaSuccess) return e;
-        raised[two][cl][form].fetch_or(bit, std::memory_order_relaxed);
-    }
-    return cudaSuccess;
+    return raised[two][cl][form]([&] { return cudaFuncSetAttribute(*out, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
 }
 
 cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
@@ -2508,17 +2498,18 @@ static const PsKernel kPs[3][2] = {{tt_gemm_ps_kernel<1, false, false>, tt_gemm_
 
 // The persistent form: one CTA (or one pair of CTAs, as a cluster of two) per SM.
 cudaError_t launch_gemm_ps(const tt_apply_info& I, const GemmArgs& g, const TmapPair& maps, cudaStream_t st) {
-    static int attr_set_for = -1, sm_count = 148;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (attr_set_for != dev) {
+    static OncePerDevice raised;
+    const cudaError_t ready = raised([] {
         cudaError_t e = cudaSuccess;
         for (const PsKernel kern : {kPs[0][0], kPs[0][1], kPs[1][0], kPs[1][1], kPs[2][0], kPs[2][1]})
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-        if (e != cudaSuccess) return e;
-        cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
-        attr_set_for = dev;
-    }
+        return e;
+    });
+    if (ready != cudaSuccess) return ready;
+    int dev = 0, sm_count = 0;
+    cudaGetDevice(&dev);
+    const cudaError_t counted = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
+    if (counted != cudaSuccess) return counted;
     CUtensorMap ta, tb, ty, tr;
     memcpy(&ta, maps.a, sizeof ta);
     memcpy(&tb, maps.b, sizeof tb);
@@ -2562,14 +2553,9 @@ cudaError_t gemm_cluster_fits(const GemmArgs& g, int smem_bytes, int* fits) {
 }
 
 cudaError_t launch_floor(const tt_apply_info& I, int smem_bytes, int cluster, cudaStream_t st) {
-    static int attr_set_for = -1;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (attr_set_for != dev) {
-        cudaError_t e = cudaFuncSetAttribute(tt_floor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-        if (e != cudaSuccess) return e;
-        attr_set_for = dev;
-    }
+    static OncePerDevice raised;
+    const cudaError_t ready = raised([] { return cudaFuncSetAttribute(tt_floor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
+    if (ready != cudaSuccess) return ready;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(I.grid_x, I.grid_y, I.grid_z); cfg.blockDim = dim3(I.threads, 1, 1);
     cfg.dynamicSmemBytes = (size_t)smem_bytes; cfg.stream = st;
@@ -2670,14 +2656,9 @@ cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& args, const v
 }
 
 cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st) {
-    static int attr_set_for = -1;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (attr_set_for != dev) {
-        cudaError_t e = cudaFuncSetAttribute(tt_dwconv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-        if (e != cudaSuccess) return e;
-        attr_set_for = dev;
-    }
+    static OncePerDevice raised;
+    const cudaError_t ready = raised([] { return cudaFuncSetAttribute(tt_dwconv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
+    if (ready != cudaSuccess) return ready;
     dim3 grid(I.grid_x, I.grid_y, 1);
     if (dw.window_rows > 0) {
         // register-window kernels: one instantiation per (filter size, stride, output rows per thread)
@@ -2697,15 +2678,9 @@ cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st)
 
 template <int NV>
 static cudaError_t launch_row_ragged(const tt_apply_info& I, const RowArgs& row, cudaStream_t st) {
-    static std::atomic<uint64_t> raised;                 // a bit per device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = 1ull << (dev & 63);
-    if (!(raised.load(std::memory_order_relaxed) & bit)) {
-        cudaError_t e = cudaFuncSetAttribute(tt_softmax_ragged_kernel<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem);
-        if (e != cudaSuccess) return e;
-        raised.fetch_or(bit, std::memory_order_relaxed);
-    }
+    static OncePerDevice raised;
+    const cudaError_t ready = raised([] { return cudaFuncSetAttribute(tt_softmax_ragged_kernel<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem); });
+    if (ready != cudaSuccess) return ready;
     return launch_serialized(tt_softmax_ragged_kernel<NV>, dim3((unsigned)I.grid_x, 1, 1), (unsigned)I.threads, (size_t)I.smem_bytes, st, row, row.chunk);
 }
 typedef cudaError_t (*RaggedLauncher)(const tt_apply_info&, const RowArgs&, cudaStream_t);

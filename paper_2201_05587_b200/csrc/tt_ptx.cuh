@@ -2,10 +2,29 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda.h>
+#include <atomic>
 #include <cstdint>
 #include "tt_internal.h"
 
 namespace tt {
+
+// Host side: what a launcher sets up on a device before its first launch there (a kernel's shared-memory limit).  Threads may make
+// their first calls at once; two that do both set up, which is harmless, and neither launches before it has.
+class OncePerDevice {
+public:
+    template <typename F>
+    cudaError_t operator()(F&& set_up) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        const uint64_t bit = 1ull << (dev & 63);
+        if (done_.load(std::memory_order_acquire) & bit) return cudaSuccess;
+        const cudaError_t e = set_up();
+        if (e == cudaSuccess) done_.fetch_or(bit, std::memory_order_release);
+        return e;
+    }
+private:
+    std::atomic<uint64_t> done_{0};
+};
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 

@@ -1,6 +1,9 @@
 """GPU parity: the CUDA path, called through the C ABI, against the CPU oracle on the same seeded inputs."""
 import ctypes
 import itertools
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -1147,3 +1150,51 @@ def test_row_contiguous_operands_that_start_anywhere(spec, operand):
         assert util.rel_l2(y, ref) <= util.TOL_TF32, (spec.name, rec.short())
         assert float(np.abs(y.astype(np.float64) - re).max()) <= ELEM_TF32 * float(np.abs(re).max())
         wl.close()
+
+
+FIRST_CALLS = """
+import threading
+import torch
+from paper_2201_05587_b200 import binding as B
+from paper_2201_05587_b200 import workloads as W
+tc = lambda **kw: B.make_record(B.TT_FAMILY_GEMM_TC, **kw)
+dw = lambda **kw: B.make_record(B.TT_FAMILY_DW_SIMT, items_per_thread=4, vec_width=4, **kw)
+def dwc(n, hw): return W.Spec(B.TT_OP_DWCONV2D, B.make_shapes(n=n, c=32, h=hw, w=hw, k=32, r=3, s=3, stride_h=1, stride_w=1, pad_h=1, pad_w=1, has_bias=1), 1, "dw")
+kinds = [(W._dense(300, 256, 400), tc(tile_n=128, tile_k=32, stages=3, mma_m_axis=1, persistent=1)), (W._dense(300, 256, 400), tc(tile_n=64, tile_k=32, stages=2, mma_m_axis=1)),
+         (W._dense(64, 512, 200), tc(tile_n=64, tile_k=32, stages=2, split_k=4, mma_m_axis=1)), (W._conv(32, 28, 64, 3, 1, 1), tc(tile_n=64, tile_k=32, stages=2, k_order=1, mma_m_axis=1)),
+         (dwc(4, 28), dw(tile_m=4, block_y=28, block_x=28, threads=128, unroll=2, raster=1, stages=2)), (dwc(2, 20), dw(tile_m=8, block_y=20, block_x=20, threads=128, unroll=0)),
+         (W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(4, 100, 197, 0.1), 1, "rows"), B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=16, block_y=4, vec_width=1))]
+torch.zeros(1, device="cuda")
+gate, out = threading.Barrier(2 * len(kinds)), [None] * (2 * len(kinds))
+def work(i):
+    try:
+        sp, rec = kinds[i % len(kinds)]
+        wl = sp.workload()
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            t, tt = W.device_tensors(sp, W.make_inputs(sp, 7))
+            t["y"].fill_(float("nan"))
+            gate.wait()
+            wl.apply(rec)
+            wl.run(tt)
+            assert wl.status() == B.TT_OK
+            out[i] = t["y"].cpu()
+    except BaseException as e:
+        out[i] = e
+        gate.abort()
+threads = [threading.Thread(target=work, args=(i,)) for i in range(2 * len(kinds))]
+[t.start() for t in threads]
+[t.join() for t in threads]
+for i in range(len(kinds)):
+    for o in (out[i], out[i + len(kinds)]):
+        assert torch.is_tensor(o), (kinds[i][0].name, o)
+        assert not torch.isnan(o).any() and torch.equal(o, out[i]), kinds[i][0].name
+print("first calls ok")
+"""
+
+
+def test_first_calls_of_several_threads_at_once():
+    """Kernels of every form, each set up for the device by whichever thread comes first: a fresh process, all threads at once."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "first calls ok" in r.stdout, r.stdout + r.stderr
