@@ -281,7 +281,8 @@ tt_status tt_schedule_apply_ex(tt_workload* w, const tt_schedule_record* rec, in
  * factors traverse it exactly?  reformulate != 0 tests Split(N, N/f, f) for the single factor f instead. */
 tt_status tt_split_check(int64_t extent, const int64_t* factors, size_t n_factors, int32_t reformulate, int32_t* valid);
 
-/* Run the workload once under the applied record (device pointers). */
+/* Run the workload once under the applied record (device pointers).  Where that has scratch (workspace_bytes > 0) runs of one
+ * handle share it: the caller orders them when they go to different streams. */
 tt_status tt_run(tt_workload* w, const tt_tensors* t, void* cuda_stream);
 
 /* One layer of a chained pass: a workload on its tensors, enqueued on stream number `lane`, after the layers whose
@@ -296,7 +297,8 @@ typedef struct tt_chain_step {
 /* Enqueue a whole pass of a model in one call: streams[0] is the caller's stream (a capturing one, too), the others are
  * side streams that fork from it where they are first used and join it again at the end.  Nothing is synchronised.  On an
  * error the layers in front of the failing one have been enqueued and the side streams joined; failed_at (may be NULL)
- * receives its position.  Layers may share a workload; calls for the same workloads do not overlap in time (one handle,
+ * receives its position.  Layers may share a workload; those on different lanes run side by side, or one after the other
+ * where the workload has scratch (workspace_bytes > 0).  Calls for the same workloads do not overlap in time (one handle,
  * one thread), calls for different ones may run on different threads. */
 tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* streams, size_t n_streams, size_t* failed_at);
 /* tt_run with HOST pointers: copies x, w, bias, residual to library-owned device buffers, runs, copies y back,

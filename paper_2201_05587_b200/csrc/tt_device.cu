@@ -7,6 +7,7 @@
 #include <chrono>
 #include <cstring>
 #include <mutex>
+#include <unordered_map>
 #include <vector>
 #include "tt_internal.h"
 
@@ -576,6 +577,22 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
         }
         side = side || s.lane != 0;
     }
+    // Layers of one workload share its scratch (re-packed filters, partial sums and arrival counters): on different lanes they
+    // run one after the other, in chain order
+    std::vector<int64_t> after(n_steps, -1);
+    if (side) {
+        std::unordered_map<const tt_workload*, size_t> last;
+        for (size_t i = 0; i < n_steps; ++i) {
+            const tt_workload* w = steps[i].workload;
+            if (!w || w->plan.info.workspace_bytes == 0) continue;
+            const auto seen = last.find(w);
+            if (seen != last.end() && steps[seen->second].lane != steps[i].lane) {
+                after[i] = (int64_t)seen->second;
+                needed[seen->second] = 1;
+            }
+            last[w] = i;
+        }
+    }
     EventLoan events;
     tt_status rc = TT_OK;
     cudaEvent_t start = nullptr;
@@ -592,6 +609,7 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
         if (s.lane != 0 && !used[(size_t)s.lane]) e = cudaStreamWaitEvent(st, start, 0);      // the side stream forks (a capture, or the caller's ordering)
         used[(size_t)s.lane] = 1;
         for (int32_t j = 0; j < s.n_waits && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(st, done[(size_t)s.waits[j]], 0);
+        if (after[i] >= 0 && e == cudaSuccess) e = cudaStreamWaitEvent(st, done[(size_t)after[i]], 0);
         if (e == cudaSuccess) rc = launch(s.workload, s.tensors, st);
         if (e == cudaSuccess && rc == TT_OK && needed[i]) {
             done[i] = events.get();

@@ -1198,3 +1198,31 @@ def test_first_calls_of_several_threads_at_once():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "first calls ok" in r.stdout, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("spec, rec", [
+    (W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(2, 512, 14, 14, 512, 3, 3, 1, 1, True, B.TT_ACT_RELU), 1, "lanes_tap", "uniform"),
+     tc(tile_n=64, tile_k=32, stages=4, k_order=1, mma_m_axis=1)),
+    (W._dense(64, 4096, 512, name="lanes_split12"), tc(tile_n=64, tile_k=32, stages=2, split_k=12, mma_m_axis=1)),
+], ids=lambda v: v.name if isinstance(v, W.Spec) else "")
+def test_chain_layers_that_share_scratch_on_different_lanes(spec, rec):
+    """Layers of one workload with different weights on three lanes of a chain, no wait between them: its scratch (re-packed
+    filters; partial sums and counters) serves one layer at a time."""
+    import torch
+    arrays = [W.make_inputs(spec, 60 + i) for i in range(3)]
+    refs = [util.oracle_ref(spec, a) for a in arrays]
+    for constant in (False, True):
+        wl = spec.workload()
+        assert wl.apply(rec).workspace_bytes > 0
+        wl.set_constant_weights(constant)
+        ts, tts = zip(*[W.device_tensors(spec, a) for a in arrays])
+        steps = [type("Node", (), {"kernel": 0})() for _ in arrays]
+        streams = [torch.cuda.current_stream()] + [torch.cuda.Stream() for _ in range(2)]
+        for _ in range(5):
+            for t in ts:
+                t["y"].fill_(float("nan"))
+            W.run_chain([wl], steps, list(tts), [(0, ()), (1, ()), (2, ())], streams)
+            assert wl.status() == B.TT_OK
+            for t, ref in zip(ts, refs):
+                assert util.rel_l2(t["y"].cpu().numpy(), ref) <= util.TOL_TF32
+        wl.close()
