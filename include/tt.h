@@ -295,7 +295,8 @@ typedef struct tt_chain_step {
     int32_t lane;
 } tt_chain_step;
 /* Enqueue a whole pass of a model in one call: streams[0] is the caller's stream (a capturing one, too), the others are
- * side streams that fork from it where they are first used and join it again at the end.  Nothing is synchronised.  On an
+ * side streams that fork from it where they are first used and join it again at the end.  All are streams of the current
+ * device.  Nothing is synchronised.  On an
  * error the layers in front of the failing one have been enqueued and the side streams joined; failed_at (may be NULL)
  * receives its position.  Layers may share a workload; those on different lanes run side by side, or one after the other
  * where the workload has scratch (workspace_bytes > 0).  Calls for the same workloads do not overlap in time (one handle,

@@ -309,13 +309,18 @@ def tensors(x, w=None, bias=None, residual=None, y=None) -> tt_tensors:
 _torch = None
 
 
-def _raw_stream() -> int:
-    """The current stream of the current device as an integer (torch's own stream object costs a microsecond to make)."""
+def _import_torch():
     global _torch
     if _torch is None:
         import torch
         _torch = torch
-    return _torch._C._cuda_getCurrentRawStream(_torch.cuda.current_device())
+    return _torch
+
+
+def _raw_stream() -> int:
+    """The current stream of the current device as an integer (torch's own stream object costs a microsecond to make)."""
+    torch = _torch or _import_torch()
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _stream():
@@ -323,10 +328,40 @@ def _stream():
 
 
 def run_chain(wls, steps, tts, plan, streams):
-    """tt_run_chain over the nodes of a chain (workloads.run_chain): streams are torch streams."""
-    st, at = _call.run_chain(wls, steps, tts, plan, [s.cuda_stream for s in streams])
+    """tt_run_chain over the nodes of a chain (workloads.run_chain): streams are torch streams, whose device is made current."""
+    torch = _torch or _import_torch()
+    devices = {s.device_index for s in streams}
+    if len(devices) > 1:
+        return _run_chain_over_devices(wls, steps, tts, plan, streams)
+    if devices == {torch.cuda.current_device()}:
+        st, at = _call.run_chain(wls, steps, tts, plan, [s.cuda_stream for s in streams])
+    else:
+        with torch.cuda.device(streams[0].device):
+            st, at = _call.run_chain(wls, steps, tts, plan, [s.cuda_stream for s in streams])
     if st != TT_OK:
         raise TTError(st, f"tt_run({wls[steps[at].kernel].name})" if at >= 0 else "tt_run_chain")
+
+
+def _run_chain_over_devices(wls, steps, tts, plan, streams):
+    """The same pass layer by layer, for lanes on several devices: a native call enqueues on one."""
+    needed = {p for pl in plan if pl is not None for p in pl[1]}
+    start, events, used = streams[0].record_event(), {}, set()
+    for i, (st, tt, pl) in enumerate(zip(steps, tts, plan)):
+        if pl is None:
+            continue
+        lane, waits = pl
+        s = streams[lane]
+        if lane != 0 and lane not in used:
+            s.wait_event(start)
+        used.add(lane)
+        for p in waits:
+            s.wait_event(events[p])
+        with _torch.cuda.stream(s):
+            wls[st.kernel].run(tt)
+        if i in needed:
+            events[i] = s.record_event()
+    for lane in sorted(used - {0}):
+        streams[0].wait_event(streams[lane].record_event())
 
 
 class Workload:

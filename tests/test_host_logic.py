@@ -883,3 +883,51 @@ def test_softmax_threads_leave_their_registers_room():
         st, info = wl.check(rec, mode=B.TT_MODE_STRICT)       # as written, in passes over memory
         assert st == B.TT_OK and info.threads == 1024
         wl.close()
+
+
+def test_chain_is_enqueued_with_its_streams_device_current(monkeypatch):
+    """Streams of a device that is not the current one: that device is current while the pass is enqueued, and only then; lanes
+    on several devices are enqueued layer by layer, each with its own device current and with the plan's waits."""
+    import contextlib
+    import torch
+    now, log = [0], []
+
+    @contextlib.contextmanager
+    def device(d):
+        back, now[0] = now[0], torch.device(d).index
+        yield
+        now[0] = back
+
+    class Stream:
+        def __init__(self, index, name):
+            self.device_index, self.device, self.cuda_stream, self.name = index, torch.device("cuda", index), 0, name
+
+        def record_event(self):
+            log.append(("record", self.name))
+            return len(log)
+
+        def wait_event(self, e):
+            log.append(("wait", self.name, e))
+
+    class Call:
+        @staticmethod
+        def run_chain(*args):
+            log.append(("native", now[0]))
+            return B.TT_OK, -1
+
+    class Kernel:
+        def run(self, tt):
+            log.append(("run", now[0], tt))
+
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: now[0])
+    monkeypatch.setattr(torch.cuda, "device", device)
+    monkeypatch.setattr(torch.cuda, "stream", lambda s: device(s.device))
+    monkeypatch.setattr(B, "_call", Call)
+    node = type("Node", (), {"kernel": 0})()
+    plan = [None, (0, ()), (1, ()), (0, (2,))]
+    for index in (0, 1):
+        B.run_chain([Kernel()], [node] * 4, list("abcd"), plan, [Stream(index, "m"), Stream(index, "s")])
+        assert log.pop() == ("native", index) and now == [0] and not log
+    B.run_chain([Kernel()], [node] * 4, list("abcd"), plan, [Stream(0, "m"), Stream(1, "s")])
+    assert log == [("record", "m"), ("run", 0, "b"), ("wait", "s", 1), ("run", 1, "c"), ("record", "s"), ("wait", "m", 5), ("run", 0, "d"),
+                   ("record", "s"), ("wait", "m", 8)] and now == [0]
