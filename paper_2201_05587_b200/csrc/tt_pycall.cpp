@@ -7,6 +7,7 @@
 // links against nothing.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
+#include <algorithm>
 #include <vector>
 #include "tt.h"
 
@@ -73,17 +74,18 @@ PyObject* run_chain(PyObject*, PyObject* const* args, Py_ssize_t n) {
     std::vector<tt_tensors> tens;
     std::vector<int32_t> waits, index;
     std::vector<void*> streams;
-    const Py_ssize_t n_nodes = ok ? PySequence_Fast_GET_SIZE(seq[3]) : 0;
-    if (ok && (PySequence_Fast_GET_SIZE(seq[1]) < n_nodes || PySequence_Fast_GET_SIZE(seq[2]) < n_nodes)) {
-        PyErr_SetString(PyExc_ValueError, "run_chain: steps, tensors and plan differ in length");
-        ok = false;
-    }
+    std::vector<PyObject*> entries;
+    // (as many nodes as the shortest of the three has)
+    const Py_ssize_t n_nodes = !ok ? 0 : std::min({PySequence_Fast_GET_SIZE(seq[1]), PySequence_Fast_GET_SIZE(seq[2]), PySequence_Fast_GET_SIZE(seq[3])});
     std::vector<int32_t> position((size_t)n_nodes, -1), first_wait;      // node -> its place among the layers
     tens.reserve((size_t)n_nodes); chain.reserve((size_t)n_nodes); index.reserve((size_t)n_nodes); first_wait.reserve((size_t)n_nodes);
     for (Py_ssize_t i = 0; ok && i < n_nodes; ++i) {
         PyObject* pl = PySequence_Fast_GET_ITEM(seq[3], i);
         if (pl == Py_None) continue;                      // an external tensor
-        if (!PyTuple_Check(pl) || PyTuple_GET_SIZE(pl) != 2) { PyErr_SetString(PyExc_TypeError, "run_chain: a plan entry is (lane, waits)"); ok = false; break; }
+        PyObject* pair = PySequence_Fast(pl, "run_chain: a plan entry is (lane, waits)");
+        if (pair && PySequence_Fast_GET_SIZE(pair) != 2) { PyErr_SetString(PyExc_ValueError, "run_chain: a plan entry is (lane, waits)"); Py_CLEAR(pair); }
+        if (!pair) { ok = false; break; }
+        entries.push_back(pair);
         tt_chain_step st{};
         long k = 0;
         void* h = nullptr;
@@ -91,10 +93,10 @@ PyObject* run_chain(PyObject*, PyObject* const* args, Py_ssize_t n) {
         if (k < 0 || k >= PySequence_Fast_GET_SIZE(seq[0])) { PyErr_SetString(PyExc_IndexError, "run_chain: no such workload"); ok = false; break; }
         if (!long_attr(PySequence_Fast_GET_ITEM(seq[0], k), g_handle_attr, &h, nullptr)) { ok = false; break; }
         st.workload = static_cast<tt_workload*>(h);
-        st.lane = (int32_t)PyLong_AsLong(PyTuple_GET_ITEM(pl, 0));
+        st.lane = (int32_t)PyLong_AsLong(PySequence_Fast_GET_ITEM(pair, 0));
         tt_tensors t;
         if (PyErr_Occurred() || !tensors_of(PySequence_Fast_GET_ITEM(seq[2], i), &t)) { ok = false; break; }
-        PyObject* ws = PySequence_Fast(PyTuple_GET_ITEM(pl, 1), "run_chain: waits is a sequence");
+        PyObject* ws = PySequence_Fast(PySequence_Fast_GET_ITEM(pair, 1), "run_chain: waits is a sequence");
         if (!ws) { ok = false; break; }
         first_wait.push_back((int32_t)waits.size());
         for (Py_ssize_t j = 0; ok && j < PySequence_Fast_GET_SIZE(ws); ++j) {
@@ -120,6 +122,7 @@ PyObject* run_chain(PyObject*, PyObject* const* args, Py_ssize_t n) {
         s = g_run_chain(chain.data(), chain.size(), streams.data(), streams.size(), &at);
         Py_END_ALLOW_THREADS
     }
+    for (PyObject* o : entries) Py_DECREF(o);
     for (PyObject* o : seq) Py_XDECREF(o);
     if (!ok) return nullptr;
     return Py_BuildValue("(ii)", (int)s, at < index.size() ? (int)index[at] : -1);

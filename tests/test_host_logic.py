@@ -931,3 +931,23 @@ def test_chain_is_enqueued_with_its_streams_device_current(monkeypatch):
     B.run_chain([Kernel()], [node] * 4, list("abcd"), plan, [Stream(0, "m"), Stream(1, "s")])
     assert log == [("record", "m"), ("run", 0, "b"), ("wait", "s", 1), ("run", 1, "c"), ("record", "s"), ("wait", "m", 5), ("run", 0, "d"),
                    ("record", "s"), ("wait", "m", 8)] and now == [0]
+
+
+def test_run_chain_takes_plans_of_any_sequence(monkeypatch):
+    """A plan entry is a pair of any kind, the waits any iterable, and the chain as long as the shortest of its lists; a layer
+    without an applied record is what the pass then fails on."""
+    import torch
+    wls = [W._dense(8, 16, 8, name="first").workload(), W._dense(8, 16, 8, name="second").workload()]
+    node = lambda k: type("Node", (), {"kernel": k})()
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    stream = type("Stream", (), {"cuda_stream": 0, "device_index": 0})()
+    t = B.tt_tensors()
+    for plan in ([(0, ()), (0, (0,))], [[0, []], [0, [0]]], ((0, set()), (0, {0})), [None, [0, ()]], [(0, ()), (0, (0,)), (0, (1,))]):
+        at = 0 if plan[0] is not None else 1
+        with pytest.raises(B.TTError) as err:
+            B.run_chain(wls, [node(0), node(1)], [t, t], plan, [stream])
+        assert err.value.status == B.TT_ERR_NOT_APPLIED and wls[at].name in str(err.value)
+    B.run_chain(wls, [node(0), node(1)], [t, t], [], [stream])
+    for bad, kind in (([(0,)], ValueError), ([5], TypeError), ([(0, (0,))], ValueError), ([(0, ()), ("x", ())], TypeError)):
+        with pytest.raises(kind):
+            B.run_chain(wls, [node(0), node(1)], [t, t], bad, [stream])
