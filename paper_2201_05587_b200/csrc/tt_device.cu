@@ -142,23 +142,26 @@ const void* pick(const tt_tensors* t, int which) { return which == 0 ? t->x : t-
 // each device, the rest are destroyed; any thread may borrow.
 class EventLoan {
 public:
-    EventLoan() { if (cudaGetDevice(&dev_) != cudaSuccess || dev_ >= kDevices) dev_ = -1; }
+    explicit EventLoan(size_t most) {
+        taken_.reserve(most);
+        if (cudaGetDevice(&dev_) != cudaSuccess || dev_ >= kDevices) dev_ = -1;
+    }
     ~EventLoan() {
         if (taken_.empty()) return;
         std::lock_guard<std::mutex> hold(lock());
         for (cudaEvent_t e : taken_) {
-            if (kept()[dev_].size() < kKept) kept()[dev_].push_back(e);
+            if (n_kept()[dev_] < kKept) kept()[dev_][n_kept()[dev_]++] = e;
             else cudaEventDestroy(e);
         }
     }
     EventLoan(const EventLoan&) = delete;
     EventLoan& operator=(const EventLoan&) = delete;
     cudaEvent_t get() {
-        if (dev_ < 0) return nullptr;
+        if (dev_ < 0 || taken_.size() == taken_.capacity()) return nullptr;
         cudaEvent_t e = nullptr;
         {
             std::lock_guard<std::mutex> hold(lock());
-            if (!kept()[dev_].empty()) { e = kept()[dev_].back(); kept()[dev_].pop_back(); }
+            if (n_kept()[dev_] > 0) e = kept()[dev_][--n_kept()[dev_]];
         }
         if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); return nullptr; }
         taken_.push_back(e);
@@ -167,8 +170,10 @@ public:
 private:
     static constexpr int kDevices = 64;
     static constexpr size_t kKept = 128;
+    typedef cudaEvent_t Kept[kKept];
     static std::mutex& lock() { static std::mutex m; return m; }
-    static std::vector<cudaEvent_t>* kept() { static std::vector<cudaEvent_t> k[kDevices]; return k; }
+    static Kept* kept() { static Kept k[kDevices]; return k; }
+    static size_t* n_kept() { static size_t n[kDevices]; return n; }
     int dev_ = -1;
     std::vector<cudaEvent_t> taken_;
 };
@@ -186,7 +191,7 @@ void release_device(tt_workload* w) {
     cudaGetLastError();
 }
 
-tt_status bind_device(tt_workload* w) {
+tt_status bind_device(tt_workload* w) try {
     if (!device_present()) return TT_ERR_CUDA;
     if (w->family == TT_FAMILY_GEMM_TC && w->plan.g.cluster) {
         // a cluster whose CTAs cannot be resident together can never launch: an invalid pair, not a device error
@@ -242,7 +247,7 @@ tt_status bind_device(tt_workload* w) {
     w->tmaps.clear();
     w->repacked_for = nullptr;
     return TT_OK;
-}
+} TT_NO_THROW
 
 static tt_status tensor_maps_for(tt_workload* w, const GemmArgs& g, const void* a_ptr, const void* b_ptr, const TmapPair** out) {
     const void* y_ptr = g.epi_tma ? g.y : nullptr;
@@ -317,7 +322,7 @@ static tt_status launch_tap_major(tt_workload* w, const tt_tensors* t, cudaStrea
     return TT_OK;
 }
 
-tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
+tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) try {
     if (!w || !t) return TT_ERR_INVALID_ARG;
     if (!w->plan.applied) return TT_ERR_NOT_APPLIED;
     if (!t->x || !t->y) return TT_ERR_INVALID_ARG;
@@ -399,7 +404,7 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) {
     }
     if (e != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     return TT_OK;
-}
+} TT_NO_THROW
 
 static tt_status read_status(tt_workload* w, cudaStream_t st) {
     if (!w->status_word) return TT_ERR_NOT_APPLIED;
@@ -441,11 +446,13 @@ static float median_of(std::vector<float>& v, float* q1, float* q3) {
 }
 
 static tt_status time_applied(tt_workload* w, const tt_tensors* sets, size_t n_sets, cudaStream_t st,
-                              const tt_timing_opts* oin, tt_timing* out) {
+                              const tt_timing_opts* oin, tt_timing* out) try {
     tt_timing_opts o{};
     if (oin) o = *oin;
     default_timing(&o);
     if (n_sets == 0) return TT_ERR_INVALID_ARG;
+    std::vector<float> per;                              // (before anything that would have to be given back)
+    per.reserve((size_t)o.batches);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
@@ -500,8 +507,6 @@ static tt_status time_applied(tt_workload* w, const tt_tensors* sets, size_t n_s
             if (ce != cudaSuccess || !graph) { fail(TT_ERR_CUDA); break; }
             if (cudaGraphInstantiate(&gexec, graph, 0) != cudaSuccess) { fail(TT_ERR_CUDA); break; }
         }
-        std::vector<float> per;
-        per.reserve(o.batches);
         for (int b = 0; b < o.warmup_batches + o.batches; ++b) {
             cudaEventRecord(e0, st);
             if (gexec) {
@@ -527,7 +532,7 @@ static tt_status time_applied(tt_workload* w, const tt_tensors* sets, size_t n_s
     if (e1) cudaEventDestroy(e1);
     if (rc == TT_ERR_CUDA) cudaGetLastError();
     return rc;
-}
+} TT_NO_THROW
 
 static tt_status apply_impl(tt_workload* w, const tt_schedule_record* rec, int mode, int strict_class, tt_apply_info* info) {
     if (!w || !rec) return TT_ERR_INVALID_ARG;
@@ -561,7 +566,7 @@ tt_status tt_schedule_apply_ex(tt_workload* w, const tt_schedule_record* rec, in
 
 tt_status tt_run(tt_workload* w, const tt_tensors* t, void* cuda_stream) { return launch(w, t, cuda_stream); }
 
-tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* streams, size_t n_streams, size_t* failed_at) {
+tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* streams, size_t n_streams, size_t* failed_at) try {
     if (!steps || n_steps == 0 || !streams || n_streams == 0) return TT_ERR_INVALID_ARG;
     // which layers some layer on another stream waits for
     std::vector<cudaEvent_t> done(n_steps, nullptr);
@@ -593,7 +598,7 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
             last[w] = i;
         }
     }
-    EventLoan events;
+    EventLoan events(n_steps + n_streams + 1);           // (nothing below allocates once the pass is being enqueued)
     tt_status rc = TT_OK;
     cudaEvent_t start = nullptr;
     cudaStream_t main_stream = static_cast<cudaStream_t>(streams[0]);
@@ -624,7 +629,7 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
             cudaStreamWaitEvent(main_stream, end, 0) != cudaSuccess) { cudaGetLastError(); if (rc == TT_OK) rc = TT_ERR_CUDA; }
     }
     return rc;
-}
+} TT_NO_THROW
 
 tt_status tt_workload_set_constant_weights(tt_workload* w, int32_t on) {
     if (!w) return TT_ERR_INVALID_ARG;
@@ -717,7 +722,7 @@ tt_status tt_transfer_tune_sets(tt_workload* const* wls, const tt_tensors* tenso
 
 static tt_status transfer_tune_impl(tt_workload* const* wls, const tt_tensors* tensors, const size_t* set_counts, size_t n_wl,
                                     const tt_schedule_record* pool, size_t n_pool, const tt_tune_opts* oin, void* cuda_stream,
-                                    tt_tune_result* out) {
+                                    tt_tune_result* out) try {
     if (!wls || !tensors || !out || (n_pool && !pool) || !out->chosen || !out->best_us || !out->times_us || !out->status)
         return TT_ERR_INVALID_ARG;
     tt_tune_opts o{};
@@ -794,10 +799,10 @@ static tt_status transfer_tune_impl(tt_workload* const* wls, const tt_tensors* t
     out->pairs_timed = timed; out->pairs_invalid = invalid; out->pairs_skipped = skipped;
     out->search_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t_begin).count();
     return TT_OK;
-}
+} TT_NO_THROW
 
 tt_status tt_grid_tune(tt_workload* w, const tt_tensors* t, void* cuda_stream, const tt_timing_opts* o, int32_t level,
-                       size_t top_k, tt_schedule_record* out_records, float* out_us, size_t* n_out, int32_t* n_tried) {
+                       size_t top_k, tt_schedule_record* out_records, float* out_us, size_t* n_out, int32_t* n_tried) try {
     if (!w || !t || !out_records || !out_us || !n_out || top_k == 0) return TT_ERR_INVALID_ARG;
     if (!device_present()) return TT_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
@@ -951,7 +956,7 @@ tt_status tt_grid_tune(tt_workload* w, const tt_tensors* t, void* cuda_stream, c
     *n_out = n;
     if (n > 0) return apply_impl(w, &out_records[0], TT_MODE_LEGALISE, 0, nullptr);
     return TT_ERR_INVALID_SCHEDULE;
-}
+} TT_NO_THROW
 
 namespace {
 struct RefineCtx { tt_workload* w; const tt_tensors* t; cudaStream_t st; const tt_timing_opts* o; tt_status fatal; };

@@ -5,7 +5,6 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <string>
 #include <vector>
 #include <new>
 #include "tt_internal.h"
@@ -1247,7 +1246,7 @@ const std::vector<FieldLadder>& ladders_of(uint32_t family) {
 }  // namespace
 
 tt_status tt_record_neighbours(const tt_workload* w, const tt_schedule_record* rec, tt_schedule_record* out, size_t cap,
-                               size_t* n_out) {
+                               size_t* n_out) try {
     if (!w || !rec || !n_out || (cap > 0 && !out)) return TT_ERR_INVALID_ARG;
     if (rec->version != TT_RECORD_VERSION || (int)rec->family != (int)w->family) return TT_ERR_INVALID_SCHEDULE;
     // the start in its legalised form: a neighbour that legalises back to it is no neighbour
@@ -1280,11 +1279,11 @@ tt_status tt_record_neighbours(const tt_workload* w, const tt_schedule_record* r
     if (found.size() > cap) return cap == 0 ? TT_OK : TT_ERR_RESOURCE;     // cap == 0: count only
     for (size_t i = 0; i < found.size(); ++i) out[i] = found[i];
     return TT_OK;
-}
+} TT_NO_THROW
 
 tt_status tt_refine_with(const tt_workload* w, const tt_schedule_record* start, tt_time_fn time_us, void* user,
                          int32_t max_rounds, float min_gain, tt_schedule_record* best, float* best_us, float* start_us,
-                         int32_t* n_timed) {
+                         int32_t* n_timed) try {
     if (!w || !start || !time_us || !best || !best_us || max_rounds < 0 || !(min_gain >= 0.f)) return TT_ERR_INVALID_ARG;
     tt_apply_info info;
     const tt_status s0 = tt_schedule_check(w, start, TT_MODE_LEGALISE, 0, &info);
@@ -1319,7 +1318,7 @@ tt_status tt_refine_with(const tt_workload* w, const tt_schedule_record* start, 
     *best = cur; *best_us = cur_us;
     if (n_timed) *n_timed = timed;
     return TT_OK;
-}
+} TT_NO_THROW
 
 // ---- pool files ---------------------------------------------------------------------------------------------------
 namespace {
@@ -1380,14 +1379,14 @@ tt_status tt_pool_load(const char* path, tt_schedule_record* out, float* us, siz
             char* eq = std::strchr(tok, '=');
             if (!eq) { rc = TT_ERR_INVALID_ARG; break; }
             *eq = 0;
-            const std::string key(tok);
+            auto is = [&](const char* name) { return std::strcmp(tok, name) == 0; };
             const char* val = eq + 1;
             char* end = nullptr;
-            if (key == "version") { r.version = (uint32_t)std::strtoul(val, &end, 10); have_version = true; }
-            else if (key == "family") r.family = (uint32_t)std::strtoul(val, &end, 10);
-            else if (key == "origin_op") r.origin_op = (int32_t)std::strtol(val, &end, 10);
-            else if (key == "us") t = std::strtof(val, &end);
-            else if (key == "origin") {
+            if (is("version")) { r.version = (uint32_t)std::strtoul(val, &end, 10); have_version = true; }
+            else if (is("family")) r.family = (uint32_t)std::strtoul(val, &end, 10);
+            else if (is("origin_op")) r.origin_op = (int32_t)std::strtol(val, &end, 10);
+            else if (is("us")) t = std::strtof(val, &end);
+            else if (is("origin")) {
                 const char* q = val;
                 for (int j = 0; j < kShapeInts && rc == TT_OK; ++j) {
                     *shape_ints(r.origin, j) = (int32_t)std::strtol(q, &end, 10);
@@ -1398,7 +1397,7 @@ tt_status tt_pool_load(const char* path, tt_schedule_record* out, float* us, siz
             } else {
                 bool found = false;
                 for (const RecField& rf : kRecFields)
-                    if (key == rf.name) { r.*(rf.field) = (int32_t)std::strtol(val, &end, 10); found = true; break; }
+                    if (is(rf.name)) { r.*(rf.field) = (int32_t)std::strtol(val, &end, 10); found = true; break; }
                 if (!found) rc = TT_ERR_INVALID_ARG;
             }
             if (rc == TT_OK && (end == val || (end && *end != 0))) rc = TT_ERR_INVALID_ARG;
@@ -1414,7 +1413,7 @@ tt_status tt_pool_load(const char* path, tt_schedule_record* out, float* us, siz
     return (cap && n > cap) ? TT_ERR_RESOURCE : TT_OK;
 }
 
-tt_status tt_pool_subsample(size_t n_pool, size_t count, uint64_t seed, int32_t* idx_out) {
+tt_status tt_pool_subsample(size_t n_pool, size_t count, uint64_t seed, int32_t* idx_out) try {
     if (count > n_pool || (count && !idx_out) || n_pool > 0x7fffffffu) return TT_ERR_INVALID_ARG;
     std::vector<int32_t> perm(n_pool);
     for (size_t i = 0; i < n_pool; ++i) perm[i] = (int32_t)i;
@@ -1431,7 +1430,7 @@ tt_status tt_pool_subsample(size_t n_pool, size_t count, uint64_t seed, int32_t*
         idx_out[i] = perm[i];
     }
     return TT_OK;
-}
+} TT_NO_THROW
 
 tt_status tt_split_check(int64_t extent, const int64_t* factors, size_t n, int32_t reformulate, int32_t* valid) {
     if (!factors || !valid || n == 0 || extent <= 0) return TT_ERR_INVALID_ARG;
@@ -1467,7 +1466,7 @@ tt_status tt_select(const float* times_us, size_t n_wl, size_t n_cols, int32_t* 
 }
 
 tt_status tt_rank_pools(const double* class_share, size_t n_classes, const int32_t* class_kernels, size_t n_models,
-                        double* scores, int32_t* order) {
+                        double* scores, int32_t* order) try {
     if (!class_share || !class_kernels || !order || n_classes == 0) return TT_ERR_INVALID_ARG;
     std::vector<double> sc(n_models, 0.0);
     for (size_t t = 0; t < n_models; ++t) {
@@ -1483,7 +1482,7 @@ tt_status tt_rank_pools(const double* class_share, size_t n_classes, const int32
     std::stable_sort(order, order + n_models, [&](int32_t a, int32_t b) { return sc[a] > sc[b]; });
     if (scores) for (size_t t = 0; t < n_models; ++t) scores[t] = sc[t];
     return TT_OK;
-}
+} TT_NO_THROW
 
 tt_status tt_model_latency(const float* times_us, size_t n_wl, size_t n_cols, const int32_t* chosen,
                            const int32_t* use_count, double* latency_us) {

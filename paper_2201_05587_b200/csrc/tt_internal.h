@@ -177,6 +177,9 @@ struct TmapPair {
 
 }  // namespace tt
 
+// Nothing throws across the C ABI: a function whose containers may run out of memory is a try block that ends in this.
+#define TT_NO_THROW catch (...) { return TT_ERR_OOM; }
+
 struct tt_workload {
     tt_op op;
     tt_shapes sh;

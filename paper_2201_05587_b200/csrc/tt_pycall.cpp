@@ -63,69 +63,78 @@ bool long_attr(PyObject* o, PyObject* name, void** as_ptr, long* as_long) {
     return !PyErr_Occurred();
 }
 
-// run_chain(workloads, steps, tensors, plan, streams) -> (status, index of the step it belongs to)
-// The arguments of workloads.run_chain, streams as integers.
-PyObject* run_chain(PyObject*, PyObject* const* args, Py_ssize_t n) {
-    if (n != 5 || !g_run_chain) { PyErr_SetString(PyExc_TypeError, "run_chain(workloads, steps, tensors, plan, streams)"); return nullptr; }
-    PyObject* seq[5] = {};
-    bool ok = true;
-    for (int i = 0; i < 5 && ok; ++i) ok = (seq[i] = PySequence_Fast(args[i], "run_chain takes sequences")) != nullptr;
+// The body of run_chain.  `held` takes over the references made on the way, so that an exception (a container that cannot grow)
+// loses none of them.
+PyObject* enqueue_chain(PyObject* const* args, std::vector<PyObject*>& held) {
+    PyObject* seq[5];
+    held.reserve(5);
+    for (int i = 0; i < 5; ++i) {
+        if (!(seq[i] = PySequence_Fast(args[i], "run_chain takes sequences"))) return nullptr;
+        held.push_back(seq[i]);
+    }
+    // (as many nodes as the shortest of the three has)
+    const Py_ssize_t n_nodes = std::min({PySequence_Fast_GET_SIZE(seq[1]), PySequence_Fast_GET_SIZE(seq[2]), PySequence_Fast_GET_SIZE(seq[3])});
     std::vector<tt_chain_step> chain;
     std::vector<tt_tensors> tens;
-    std::vector<int32_t> waits, index;
+    std::vector<int32_t> waits, index, first_wait, position((size_t)n_nodes, -1);      // position: node -> its place among the layers
     std::vector<void*> streams;
-    std::vector<PyObject*> entries;
-    // (as many nodes as the shortest of the three has)
-    const Py_ssize_t n_nodes = !ok ? 0 : std::min({PySequence_Fast_GET_SIZE(seq[1]), PySequence_Fast_GET_SIZE(seq[2]), PySequence_Fast_GET_SIZE(seq[3])});
-    std::vector<int32_t> position((size_t)n_nodes, -1), first_wait;      // node -> its place among the layers
+    held.reserve(5 + 2 * (size_t)n_nodes);
     tens.reserve((size_t)n_nodes); chain.reserve((size_t)n_nodes); index.reserve((size_t)n_nodes); first_wait.reserve((size_t)n_nodes);
-    for (Py_ssize_t i = 0; ok && i < n_nodes; ++i) {
+    for (Py_ssize_t i = 0; i < n_nodes; ++i) {
         PyObject* pl = PySequence_Fast_GET_ITEM(seq[3], i);
         if (pl == Py_None) continue;                      // an external tensor
         PyObject* pair = PySequence_Fast(pl, "run_chain: a plan entry is (lane, waits)");
-        if (pair && PySequence_Fast_GET_SIZE(pair) != 2) { PyErr_SetString(PyExc_ValueError, "run_chain: a plan entry is (lane, waits)"); Py_CLEAR(pair); }
-        if (!pair) { ok = false; break; }
-        entries.push_back(pair);
+        if (!pair) return nullptr;
+        held.push_back(pair);
+        if (PySequence_Fast_GET_SIZE(pair) != 2) { PyErr_SetString(PyExc_ValueError, "run_chain: a plan entry is (lane, waits)"); return nullptr; }
         tt_chain_step st{};
         long k = 0;
         void* h = nullptr;
-        if (!long_attr(PySequence_Fast_GET_ITEM(seq[1], i), g_kernel_attr, nullptr, &k)) { ok = false; break; }
-        if (k < 0 || k >= PySequence_Fast_GET_SIZE(seq[0])) { PyErr_SetString(PyExc_IndexError, "run_chain: no such workload"); ok = false; break; }
-        if (!long_attr(PySequence_Fast_GET_ITEM(seq[0], k), g_handle_attr, &h, nullptr)) { ok = false; break; }
+        if (!long_attr(PySequence_Fast_GET_ITEM(seq[1], i), g_kernel_attr, nullptr, &k)) return nullptr;
+        if (k < 0 || k >= PySequence_Fast_GET_SIZE(seq[0])) { PyErr_SetString(PyExc_IndexError, "run_chain: no such workload"); return nullptr; }
+        if (!long_attr(PySequence_Fast_GET_ITEM(seq[0], k), g_handle_attr, &h, nullptr)) return nullptr;
         st.workload = static_cast<tt_workload*>(h);
         st.lane = (int32_t)PyLong_AsLong(PySequence_Fast_GET_ITEM(pair, 0));
         tt_tensors t;
-        if (PyErr_Occurred() || !tensors_of(PySequence_Fast_GET_ITEM(seq[2], i), &t)) { ok = false; break; }
+        if (PyErr_Occurred() || !tensors_of(PySequence_Fast_GET_ITEM(seq[2], i), &t)) return nullptr;
         PyObject* ws = PySequence_Fast(PySequence_Fast_GET_ITEM(pair, 1), "run_chain: waits is a sequence");
-        if (!ws) { ok = false; break; }
+        if (!ws) return nullptr;
+        held.push_back(ws);
         first_wait.push_back((int32_t)waits.size());
-        for (Py_ssize_t j = 0; ok && j < PySequence_Fast_GET_SIZE(ws); ++j) {
+        for (Py_ssize_t j = 0; j < PySequence_Fast_GET_SIZE(ws); ++j) {
             const long p = PyLong_AsLong(PySequence_Fast_GET_ITEM(ws, j));
-            if (PyErr_Occurred()) ok = false;
-            else if (p < 0 || p >= i || position[(size_t)p] < 0) { PyErr_SetString(PyExc_ValueError, "run_chain: a layer waits for a layer in front of it"); ok = false; }
-            else waits.push_back(position[(size_t)p]);
+            if (PyErr_Occurred()) return nullptr;
+            if (p < 0 || p >= i || position[(size_t)p] < 0) { PyErr_SetString(PyExc_ValueError, "run_chain: a layer waits for a layer in front of it"); return nullptr; }
+            waits.push_back(position[(size_t)p]);
         }
         st.n_waits = (int32_t)PySequence_Fast_GET_SIZE(ws);
-        Py_DECREF(ws);
         position[(size_t)i] = (int32_t)chain.size();
         tens.push_back(t); chain.push_back(st); index.push_back((int32_t)i);
     }
-    for (Py_ssize_t i = 0; ok && i < PySequence_Fast_GET_SIZE(seq[4]); ++i) {
+    for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(seq[4]); ++i) {
         streams.push_back(PyLong_AsVoidPtr(PySequence_Fast_GET_ITEM(seq[4], i)));
-        if (PyErr_Occurred()) ok = false;
+        if (PyErr_Occurred()) return nullptr;
     }
     tt_status s = TT_OK;
     size_t at = 0;
-    if (ok && !chain.empty()) {
+    if (!chain.empty()) {
         for (size_t i = 0; i < chain.size(); ++i) { chain[i].tensors = &tens[i]; chain[i].waits = waits.data() + first_wait[i]; }
         Py_BEGIN_ALLOW_THREADS
         s = g_run_chain(chain.data(), chain.size(), streams.data(), streams.size(), &at);
         Py_END_ALLOW_THREADS
     }
-    for (PyObject* o : entries) Py_DECREF(o);
-    for (PyObject* o : seq) Py_XDECREF(o);
-    if (!ok) return nullptr;
     return Py_BuildValue("(ii)", (int)s, at < index.size() ? (int)index[at] : -1);
+}
+
+// run_chain(workloads, steps, tensors, plan, streams) -> (status, index of the step it belongs to)
+// The arguments of workloads.run_chain, streams as integers.
+PyObject* run_chain(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    if (n != 5 || !g_run_chain) { PyErr_SetString(PyExc_TypeError, "run_chain(workloads, steps, tensors, plan, streams)"); return nullptr; }
+    std::vector<PyObject*> held;
+    PyObject* result = nullptr;
+    try { result = enqueue_chain(args, held); } catch (...) { PyErr_NoMemory(); }
+    for (PyObject* o : held) Py_DECREF(o);
+    return result;
 }
 
 PyMethodDef kMethods[] = {

@@ -951,3 +951,22 @@ def test_run_chain_takes_plans_of_any_sequence(monkeypatch):
     for bad, kind in (([(0,)], ValueError), ([5], TypeError), ([(0, (0,))], ValueError), ([(0, ()), ("x", ())], TypeError)):
         with pytest.raises(kind):
             B.run_chain(wls, [node(0), node(1)], [t, t], bad, [stream])
+
+
+def test_nothing_throws_across_the_c_abi():
+    """Containers that cannot be made are a status, not an exception through C frames (which ends the process: run in a child)."""
+    import subprocess
+    import sys
+    code = """
+import ctypes as C
+from paper_2201_05587_b200 import binding as B
+lib, huge = B.lib(), 1 << 61
+share, counts, order = (C.c_double * 1)(1.0), (C.c_int32 * 1)(1), (C.c_int32 * 1)()
+assert lib.tt_rank_pools(share, 1, counts, huge, None, order) == B.TT_ERR_OOM
+steps, streams, at = (B.tt_chain_step * 1)(), (C.c_void_p * 1)(), C.c_size_t()
+assert lib.tt_run_chain(steps, huge, streams, 1, C.byref(at)) == B.TT_ERR_OOM
+assert lib.tt_run_chain(steps, 1, streams, huge, C.byref(at)) == B.TT_ERR_OOM
+print("statuses")
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and "statuses" in r.stdout, r.stderr
