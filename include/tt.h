@@ -316,7 +316,10 @@ tt_status tt_run_host_async(tt_workload* w, const tt_tensors* host, void* cuda_s
  * (the parameters of an inference pass) -- no kernel enqueued directly in front of the run on the same stream writes
  * them.  A dense or conv2d kernel then requests the first tiles of w BEFORE it waits for the kernel in front of it
  * (kernels are launched with programmatic stream serialization), so the weights stream in while that kernel is still
- * running.  Results are unchanged as long as the promise holds.  batch_matmul operands are never treated this way. */
+ * running.  Results are unchanged as long as the promise holds.  batch_matmul operands are never treated this way.
+ * A k_order = 1 convolution re-packs its filters once per weight pointer then; switching the promise off forgets the copy.  A
+ * captured pass keeps the copy that it was captured with: calls for other weights get a workspace of their own, all of them
+ * released by the next apply or by destroy. */
 tt_status tt_workload_set_constant_weights(tt_workload* w, int32_t on);
 /* Read and clear the device status word of the last runs (TT_OK or TT_ERR_TIMEOUT); synchronises the stream.
  * After a TT_ERR_TIMEOUT the split-K arrival counters of the applied record are cleared too, so the next run starts

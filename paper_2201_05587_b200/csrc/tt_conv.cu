@@ -459,6 +459,10 @@ __global__ void tt_repack_filters_kernel(const float* __restrict__ w, float* __r
         const int c = cb * 32 + ci;
         out[i] = c < C ? __ldg(w + (f * C + c) * RS + tap) : 0.f;
     }
+    // The convolution behind this kernel waits for it; the one behind that may fetch its filters as soon as the first has started,
+    // which is when the blocks here have left: what they wrote has to be in place by then, for copy engines too.
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    __threadfence();
 }
 
 cudaError_t launch_repack(const float* w, float* out, const ConvPmArgs& g, cudaStream_t st) {

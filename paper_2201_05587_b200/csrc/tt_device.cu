@@ -180,7 +180,15 @@ private:
 
 }  // namespace
 
+// Forget what the workspace holds of re-packed filters, and the workspaces that passes captured under the record in force read.
+static void forget_filters(tt_workload* w) {
+    for (void* p : w->kept) cudaFree(p);
+    w->kept.clear();
+    w->repacked_for = nullptr; w->repacked_in = 0; w->captured_read = w->captured_fill = false;
+}
+
 void release_device(tt_workload* w) {
+    forget_filters(w);
     if (w->workspace) cudaFree(w->workspace);
     if (w->status_word) cudaFree(w->status_word);
     if (w->ktab_dev) cudaFree(w->ktab_dev);
@@ -204,6 +212,7 @@ tt_status bind_device(tt_workload* w) try {
         if (conv_pm_cluster_fits(w->plan.info, w->plan.pm, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
         if (!fits) return TT_ERR_RESOURCE;
     }
+    forget_filters(w);
     const size_t need = (size_t)w->plan.info.workspace_bytes;
     if (need > w->workspace_bytes) {
         if (w->workspace) cudaFree(w->workspace);
@@ -245,7 +254,6 @@ tt_status bind_device(tt_workload* w) try {
         if (cudaMemcpy(w->ktab_dev, tab.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     }
     w->tmaps.clear();
-    w->repacked_for = nullptr;
     return TT_OK;
 } TT_NO_THROW
 
@@ -300,17 +308,48 @@ static tt_status tensor_maps_for(tt_workload* w, const GemmArgs& g, const void* 
 }
 
 // Tap-major convolution: the filters are brought into walk order first, once per weight pointer and applied record where
-// the caller has promised that they are constant.
+// the caller has promised that they are constant.  A capture only records the re-pack, and what it records runs whenever the
+// pass is replayed.  So a copy made inside a capture serves that capture alone; a copy that a captured pass was told to read is
+// kept for it, and a call for other weights goes to a workspace of its own; and calls under the promise leave a workspace that a
+// captured pass fills.
+static tt_status filters_for(tt_workload* w, const void* weights, cudaStream_t st, bool* repacked_now) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long capture = 0;
+    if (cudaStreamGetCaptureInfo(st, &status, &capture) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+    if (status != cudaStreamCaptureStatusActive) capture = 0;
+    *repacked_now = false;
+    if (w->constant_weights && w->repacked_for == weights && (w->repacked_in == 0 || w->repacked_in == capture)) {
+        if (capture != 0 && w->repacked_in == 0) w->captured_read = true;
+        return TT_OK;
+    }
+    if (w->captured_read || (w->constant_weights && capture == 0 && w->captured_fill)) {
+        void* fresh = nullptr;
+        w->kept.reserve(w->kept.size() + 1);
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;       // (an allocation belongs to no capture)
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        const cudaError_t e = cudaMalloc(&fresh, w->workspace_bytes);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) { cudaGetLastError(); return TT_ERR_OOM; }
+        w->kept.push_back(w->workspace);
+        w->workspace = fresh;
+        w->captured_read = w->captured_fill = false;
+    }
+    w->repacked_for = nullptr;
+    if (launch_repack(static_cast<const float*>(weights), static_cast<float*>(w->workspace), w->plan.pm, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+    if (w->constant_weights) w->repacked_for = weights;
+    w->repacked_in = capture;
+    if (capture != 0) w->captured_fill = true;
+    *repacked_now = true;
+    return TT_OK;
+}
+
 static tt_status launch_tap_major(tt_workload* w, const tt_tensors* t, cudaStream_t st) {
     const Plan& p = w->plan;
     bool repacked_now = false;
-    if (!(w->constant_weights && w->repacked_for == t->w)) {
-        if (launch_repack(static_cast<const float*>(t->w), static_cast<float*>(w->workspace), p.pm, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
-        w->repacked_for = t->w;
-        repacked_now = true;
-    }
+    tt_status s = filters_for(w, t->w, st, &repacked_now);
+    if (s != TT_OK) return s;
     const TmapPair* maps = nullptr;
-    const tt_status s = tensor_maps_for(w, p.g, w->workspace, nullptr, &maps);
+    s = tensor_maps_for(w, p.g, w->workspace, nullptr, &maps);
     if (s != TT_OK) return s;
     ConvPmArgs c = p.pm;
     c.x = static_cast<const float*>(t->x); c.y = static_cast<float*>(t->y);
@@ -453,6 +492,8 @@ static tt_status time_applied(tt_workload* w, const tt_tensors* sets, size_t n_s
     if (n_sets == 0) return TT_ERR_INVALID_ARG;
     std::vector<float> per;                              // (before anything that would have to be given back)
     per.reserve((size_t)o.batches);
+    const void* filters_in = w->workspace;
+    const bool captured_read = w->captured_read, captured_fill = w->captured_fill;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
@@ -527,6 +568,12 @@ static tt_status time_applied(tt_workload* w, const tt_tensors* sets, size_t n_s
     } while (false);
     if (gexec) cudaGraphExecDestroy(gexec);
     if (graph) cudaGraphDestroy(graph);
+    if (w->plan.repack) {
+        // the batch's graph is gone: nobody reads or fills the filters' workspace on its account any more
+        const bool same = w->workspace == filters_in;
+        w->captured_read = same && captured_read; w->captured_fill = same && captured_fill;
+        if (w->repacked_in != 0) w->repacked_for = nullptr;
+    }
     if (cap) cudaStreamDestroy(cap);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
@@ -634,6 +681,7 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
 tt_status tt_workload_set_constant_weights(tt_workload* w, int32_t on) {
     if (!w) return TT_ERR_INVALID_ARG;
     w->constant_weights = on != 0;
+    if (!on) w->repacked_for = nullptr;                  // (what is promised from here on is about the weights as they are then)
     return TT_OK;
 }
 

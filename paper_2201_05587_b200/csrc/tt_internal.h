@@ -195,7 +195,12 @@ struct tt_workload {
     unsigned long long wait_ns = 1000000000ull;   // one second per wait inside a kernel, then the kernel gives up
     unsigned extra_tx = 0;            // test facility (tt_workload_test_stall)
     bool constant_weights = false;    // the caller's promise of tt_workload_set_constant_weights
-    const void* repacked_for = nullptr;   // tap-major convolution: the weight pointer whose re-packed copy the workspace holds
+    // tap-major convolution: the workspace holds the re-packed filters of ...
+    const void* repacked_for = nullptr;   // ... these weights (null: of none that the next call may take for its own),
+    unsigned long long repacked_in = 0;   // put there by a call that ran (0) or only inside this capture
+    bool captured_read = false;           // a captured pass reads them as they are now: they are not to be overwritten
+    bool captured_fill = false;           // a captured pass fills the workspace itself: what else is put there does not last
+    std::vector<void*> kept;              // workspaces that captured passes still read, until the next apply
     // device staging buffers of tt_run_host
     void* hbuf[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     size_t hbytes[5] = {0, 0, 0, 0, 0};

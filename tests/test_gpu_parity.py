@@ -1226,3 +1226,98 @@ def test_chain_layers_that_share_scratch_on_different_lanes(spec, rec):
             for t, ref in zip(ts, refs):
                 assert util.rel_l2(t["y"].cpu().numpy(), ref) <= util.TOL_TF32
         wl.close()
+
+
+def test_repacked_filters_follow_the_promise_and_captured_passes():
+    """The re-packed filters of a tap-major convolution: forgotten when the promise of constant weights is switched off, kept for
+    the captured pass that reads them while other weights run, and not taken from a capture that has never run."""
+    import torch
+    sp = W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(2, 96, 14, 14, 200, 3, 3, 1, 1, True, B.TT_ACT_RELU), 1, "filters", "uniform")
+    rec = tc(tile_n=64, tile_k=32, stages=4, k_order=1, mma_m_axis=1)
+    arrays = [W.make_inputs(sp, 70 + i) for i in range(2)]
+    refs = [util.oracle_ref(sp, a) for a in arrays]
+    (t0, tt0), (t1, tt1) = [W.device_tensors(sp, a) for a in arrays]
+
+    def right(t, ref):
+        torch.cuda.synchronize()
+        assert wl.status() == B.TT_OK
+        ok = util.rel_l2(t["y"].cpu().numpy(), ref) <= util.TOL_TF32
+        t["y"].fill_(float("nan"))
+        return ok
+
+    def capture(*tts):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            for tt in tts:
+                wl.run(tt)
+        return g
+
+    # weights written between a run without the promise and one with it
+    wl = sp.workload()
+    assert wl.apply(rec).legal.k_order == 1
+    w0 = t0["w"].clone()
+    t0["w"].mul_(3.0)
+    wl.run(tt0)
+    t0["w"].copy_(w0)
+    torch.cuda.synchronize()
+    wl.set_constant_weights(True)
+    wl.run(tt0)
+    assert right(t0, refs[0])
+    # ... and while it is switched off
+    wl.set_constant_weights(False)
+    t0["w"].mul_(3.0)
+    torch.cuda.synchronize()
+    wl.set_constant_weights(True)
+    wl.run(tt0)
+    wl.set_constant_weights(False)
+    t0["w"].copy_(w0)
+    torch.cuda.synchronize()
+    wl.set_constant_weights(True)
+    wl.run(tt0)
+    assert right(t0, refs[0])
+    # a captured pass reads the copy in place; other weights in between, run and captured
+    g0 = capture(tt0)
+    wl.run(tt1)
+    assert right(t1, refs[1])
+    g0.replay()
+    assert right(t0, refs[0])
+    both = capture(tt0, tt1, tt0)
+    for _ in range(2):
+        both.replay()
+        assert right(t0, refs[0]) and right(t1, refs[1])
+        g0.replay()
+        assert right(t0, refs[0])
+        wl.run(tt1)
+        assert right(t1, refs[1])
+        wl.run(tt0)
+        assert right(t0, refs[0])
+    wl.close()
+    # captured before anything has run
+    for constant in (True, False):
+        wl = sp.workload()
+        wl.apply(rec)
+        wl.set_constant_weights(constant)
+        g0 = capture(tt0)
+        wl.run(tt0)
+        assert right(t0, refs[0])
+        wl.run(tt1)
+        g0.replay()
+        assert right(t0, refs[0]) and right(t1, refs[1])
+        wl.run(tt1)
+        assert right(t1, refs[1])
+        g0.replay()
+        assert right(t0, refs[0])
+        # timing captures too, and keeps nothing for its own captures
+        opts = B.tt_timing_opts()
+        opts.use_graph, opts.batches, opts.min_batch_us = 1, 2, 50
+        wl.time([tt0, tt1], opts)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        for _ in range(40):
+            wl.time([tt0, tt1], opts)
+        assert free - torch.cuda.mem_get_info()[0] < 16 << 20
+        wl.run(tt1)
+        assert right(t1, refs[1])
+        g0.replay()
+        assert right(t0, refs[0])
+        wl.close()
