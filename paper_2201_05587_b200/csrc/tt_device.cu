@@ -16,6 +16,7 @@ namespace tt {
 cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
                         cudaStream_t st);
 cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st);
+cudaError_t plan_dw_staged(tt_apply_info& I, DwArgs& dw);
 cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st);
 cudaError_t launch_row(const tt_apply_info& I, const RowArgs& row, cudaStream_t st);
 cudaError_t gemm_cluster_fits(const GemmArgs& g, int smem_bytes, int* fits);
@@ -211,6 +212,10 @@ tt_status bind_device(tt_workload* w) try {
         int fits = 0;
         if (conv_pm_cluster_fits(w->plan.info, w->plan.pm, &fits) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
         if (!fits) return TT_ERR_RESOURCE;
+    }
+    if (w->family == TT_FAMILY_DW_SIMT && w->plan.dw.tma_stages > 0) {
+        const cudaError_t e = plan_dw_staged(w->plan.info, w->plan.dw);
+        if (e != cudaSuccess) { cudaGetLastError(); return e == cudaErrorLaunchOutOfResources ? TT_ERR_RESOURCE : TT_ERR_CUDA; }
     }
     forget_filters(w);
     const size_t need = (size_t)w->plan.info.workspace_bytes;
@@ -592,6 +597,7 @@ static tt_status apply_impl(tt_workload* w, const tt_schedule_record* rec, int m
     s = bind_device(w);
     if (s != TT_OK) { w->plan = old; w->plan.applied = false; return s; }
     w->plan.applied = true;
+    if (info) *info = w->plan.info;               // (the grid that the device holds)
     return TT_OK;
 }
 

@@ -968,7 +968,7 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
             if (total > 0x7fffffffLL) return TT_ERR_RESOURCE;
             d.total_tiles = (int)total;
             smem = smem_of(stg);
-            const long long per_sm = std::max<long long>(1, std::min<long long>(8, (228 * 1024) / (smem + 1024)));   // the launcher lowers it to what registers allow
+            const long long per_sm = std::max<long long>(1, std::min<long long>(8, (228 * 1024) / (smem + 1024)));   // (applying the record lowers it to what registers allow)
             gx = std::min<long long>(total, 148 * per_sm);
             I.legal = L;
             I.grid_x = (int)gx; I.grid_y = 1; I.grid_z = 1;

@@ -128,7 +128,7 @@ struct DwArgs {
     int box_w, stage_bytes, total_tiles;   // box width in floats (multiple of 4), bytes per buffer (multiple of 128)
     int wstage_bytes;  // boxes: bytes of the filter-and-bias buffer (multiple of 128)
     int plane_next;    // boxes: lanes after a row of strips continue with the next plane's strips, not with the next strip row
-    int step;          // how a CTA's tiles follow each other (dw_walk); set by the launcher
+    int step;          // how a CTA's tiles follow each other (dw_walk); set when the record is applied
     int runs;
     int strip_rows;    // runs: strip rows of a plane that are computed at a time
     int units_per_warp, unit_far;   // runs: strip rows side by side in a warp (0: they run on through the warps), their distance (0: 1)

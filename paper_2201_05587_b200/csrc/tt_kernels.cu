@@ -22,6 +22,7 @@
 #include <cstdint>
 #include <cstring>
 #include <algorithm>
+#include <type_traits>
 #include <utility>
 #include "tt_ptx.cuh"
 
@@ -2586,26 +2587,6 @@ static cudaError_t launch_serialized(void (*kern)(KArgs...), dim3 grid, unsigned
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// How many CTAs of a kernel a device holds at once, remembered for the launch shape asked for last.
-struct ResidentCtas {
-    int dev = -1, threads = 0, smem = -1;
-    long long ctas = 0;
-    template <typename K>
-    cudaError_t get(K kern, int d, int t, int sm, long long* out) {
-        if (d != dev || t != threads || sm != smem) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
-            if (e != cudaSuccess) return e;
-            int occ = 0, sm_count = 0;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, t, (size_t)sm)) != cudaSuccess) return e;
-            if ((e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, d)) != cudaSuccess) return e;
-            if (occ < 1) return cudaErrorLaunchOutOfResources;
-            dev = d; threads = t; smem = sm; ctas = (long long)sm_count * occ;
-        }
-        *out = ctas;
-        return cudaSuccess;
-    }
-};
-
 // CTAs per channel group; 0: consecutive ranges.  Whole planes are runs of memory of their own and go by ranges, which use every CTA.
 // Bands of planes (two tiles and more a plane) lose the memory's locality that way (256 images of 144 x 56 x 56, 3x3: 173 us
 // against 154), so there the CTAs keep to neighbouring planes, unless whole groups leave more than an eighth of them idle.
@@ -2616,32 +2597,14 @@ static int dw_step(int ctas, int groups, long long per_group) {
     return 8 * groups * per_group >= 7 * rounds * ctas ? (int)m : 0;
 }
 
-cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& args, const void* tmap_x, cudaStream_t st) {
-    DwArgs dw = args;
-    const int groups = (dw.C + dw.tile_c - 1) / dw.tile_c;
-    const long long per_group = (long long)dw.N * dw.tiles_h * dw.tiles_w;
-    CUtensorMap tx;
-    if (tmap_x) memcpy(&tx, tmap_x, sizeof tx); else memset(&tx, 0, sizeof tx);
-    dim3 grid(I.grid_x, 1, 1);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    // resident CTAs of this instantiation, looked up once per launch shape (the query costs more than the launch)
-#define TT_DWT_CASE(KERNEL, ...) \
-    { \
-        static thread_local ResidentCtas known; \
-        long long resident = 0; \
-        cudaError_t e = known.get(KERNEL, dev, I.threads, I.smem_bytes, &resident); \
-        if (e != cudaSuccess) return e; \
-        /* persistent CTAs: never more than are resident at once (registers may allow fewer than shared memory does) */ \
-        grid.x = (unsigned)std::min<long long>(grid.x, resident); \
-        dw.step = dw.tiles_h * dw.tiles_w > 1 ? dw_step((int)grid.x, groups, per_group) : 0; \
-        if (dw.step) grid.x = (unsigned)(dw.step * groups); \
-        return launch_serialized(KERNEL, grid, (unsigned)I.threads, (size_t)I.smem_bytes, st, __VA_ARGS__); }
+// Calls f with the instantiation that a staged plan runs.
+template <typename F>
+static cudaError_t with_dw_staged(const DwArgs& dw, F&& f) {
 #define TT_DWT_BOX(RR, SS, RO, WI) \
-    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == WI) TT_DWT_CASE((tt_dwconv_tma_kernel<RR, SS, RO, WI>), tx, dw)
+    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == WI) return f(tt_dwconv_tma_kernel<RR, SS, RO, WI>);
 #define TT_DWT_RUN(RR, SS, RO) \
-    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == 1) TT_DWT_CASE((tt_dwconv_run_kernel<RR, SS, RO, 1>), dw) \
-    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == 2) TT_DWT_CASE((tt_dwconv_run_kernel<RR, SS, RO, 2>), dw)
+    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == 1) return f(tt_dwconv_run_kernel<RR, SS, RO, 1>); \
+    if (dw.R == RR && dw.sh == SS && dw.window_rows == RO && dw.items == 2) return f(tt_dwconv_run_kernel<RR, SS, RO, 2>);
 #define TT_DWT_FILTER(RR, SS) \
     if (!dw.runs) { \
         TT_DWT_BOX(RR, SS, 1, 4) TT_DWT_BOX(RR, SS, 2, 4) TT_DWT_BOX(RR, SS, 4, 4) TT_DWT_BOX(RR, SS, 1, 8) TT_DWT_BOX(RR, SS, 2, 8) \
@@ -2651,8 +2614,40 @@ cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& args, const v
 #undef TT_DWT_FILTER
 #undef TT_DWT_RUN
 #undef TT_DWT_BOX
-#undef TT_DWT_CASE
     return cudaErrorInvalidValue;
+}
+
+// When a record is applied: the grid of persistent CTAs, never more than the device holds at once (registers may allow fewer than
+// shared memory does; asking costs more than a launch), and the tiles' order.
+cudaError_t plan_dw_staged(tt_apply_info& I, DwArgs& dw) {
+    int dev = 0, per_sm = 0, sm_count = 0;
+    cudaGetDevice(&dev);
+    cudaError_t e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = with_dw_staged(dw, [&](auto* kern) {
+            const cudaError_t raised = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+            return raised != cudaSuccess ? raised : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, I.threads, (size_t)I.smem_bytes);
+        });
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorLaunchOutOfResources;
+    const int groups = (dw.C + dw.tile_c - 1) / dw.tile_c;
+    I.grid_x = (int)std::min<long long>(I.grid_x, (long long)sm_count * per_sm);
+    dw.step = dw.tiles_h * dw.tiles_w > 1 ? dw_step(I.grid_x, groups, (long long)dw.N * dw.tiles_h * dw.tiles_w) : 0;
+    if (dw.step) I.grid_x = dw.step * groups;
+    return cudaSuccess;
+}
+
+cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st) {
+    const dim3 grid(I.grid_x, 1, 1);
+    return with_dw_staged(dw, [&](auto* kern) {
+        if constexpr (std::is_invocable_v<decltype(kern), const CUtensorMap, const DwArgs>) {
+            CUtensorMap tx;
+            memcpy(&tx, tmap_x, sizeof tx);
+            return launch_serialized(kern, grid, (unsigned)I.threads, (size_t)I.smem_bytes, st, tx, dw);
+        } else {
+            return launch_serialized(kern, grid, (unsigned)I.threads, (size_t)I.smem_bytes, st, dw);
+        }
+    });
 }
 
 cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st) {

@@ -1321,3 +1321,30 @@ def test_repacked_filters_follow_the_promise_and_captured_passes():
         g0.replay()
         assert right(t0, refs[0])
         wl.close()
+
+
+def test_staged_depthwise_grid_is_settled_when_the_record_is_applied():
+    """Two layers that share a kernel instantiation and differ in their launch, run in turn: the apply info has the grid that the
+    device holds, and a launch asks the driver nothing."""
+    import torch
+    sp = [W.Spec(B.TT_OP_DWCONV2D, B.make_shapes(n=n, c=96, h=28, w=28, k=96, r=3, s=3, stride_h=1, stride_w=1, pad_h=1, pad_w=1, has_bias=1,
+                                                 act=B.TT_ACT_RELU6), 1, f"dw_turns_{n}", "uniform") for n in (40, 33)]
+    recs = [B.make_record(B.TT_FAMILY_DW_SIMT, tile_m=tm, block_y=by, block_x=28, items_per_thread=4, vec_width=4, threads=256, unroll=2, raster=1, stages=sg)
+            for tm, by, sg in ((4, 28, 2), (2, 14, 4))]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    wls = [s.workload() for s in sp]
+    infos = [wl.apply(r) for wl, r in zip(wls, recs)]
+    for wl, rec, info in zip(wls, recs, infos):
+        checked = wl.check(rec)[1]
+        assert 0 < info.grid_x <= checked.grid_x and info.grid_x <= 32 * sms and (info.threads, info.smem_bytes) == (checked.threads, checked.smem_bytes)
+    arrays = [W.make_inputs(s, 80 + i) for i, s in enumerate(sp)]
+    bufs = [W.device_tensors(s, a) for s, a in zip(sp, arrays)]
+    for _ in range(3):
+        for wl, (t, tt) in zip(wls, bufs):
+            t["y"].fill_(float("nan"))
+            wl.run(tt)
+            assert wl.status() == B.TT_OK
+    for s, a, (t, _) in zip(sp, arrays, bufs):
+        assert util.rel_l2(t["y"].cpu().numpy(), util.oracle_ref(s, a)) <= util.TOL_FP32
+    for wl in wls:
+        wl.close()
