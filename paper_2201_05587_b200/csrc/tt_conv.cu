@@ -475,7 +475,7 @@ cudaError_t launch_repack(const float* w, float* out, const ConvPmArgs& g, cudaS
         for (int r = 0; r < p.nr; ++r) for (int s = 0; s < p.ns; ++s) order.tap[t++] = (unsigned char)((p.r0 + r * g.sh) * g.S + p.s0 + s * g.sw);
     }
     const long long total = (long long)g.M * g.blocks * g.R * g.S * 32;
-    const int grid = (int)std::min<long long>((total + 255) / 256, 148 * 8);
+    const int grid = (int)std::min<long long>((total + 255) / 256, kSms * 8);
     tt_repack_filters_kernel<<<grid, 256, 0, st>>>(w, out, g.M, g.C, g.R * g.S, g.blocks, order);
     return cudaGetLastError();
 }

@@ -147,14 +147,13 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     const int st = persistent ? std::min(kMaxStages, rec->stages) : std::min(std::min(kMaxStages, rec->stages), k_tiles);
     if (strict && (tn != rec->tile_n || st != rec->stages || (changed & ~TT_CHG_TILE_M))) return TT_ERR_INVALID_SCHEDULE;
     const int tiles_m = (M + kHwTileM - 1) / kHwTileM;
-    // How the tiles are laid over the SMs (148; the launch is right on any number) is this rule's choice unless the record is to
+    // How the tiles are laid over the SMs is this rule's choice unless the record is to
     // run as written (strict mode); the legal record says what it chose (tile_n, cta_group).
     // Where the record's tiles fill more than half of the SMs, columns are dealt evenly over the rounds that its tile needs: 121
     // tiles of 224 columns become 141 of 192.  Where they fill less, CTAs share a tile's channel blocks as a cluster.  Fewer
     // rounds, or the widest tile, take the place of the record's where they are a tenth cheaper: a tap costs what shared memory has to move in
     // 128-byte lines -- its filters in and out, 2 * 128, its columns, about 32 for the slab -- and the filters' part is paid per
     // tile (3x3 512 -> 512 at 7 x 7, batch 32: 31.4 us with 128 columns, 25.1 with 256).
-    constexpr int kSms = 148;
     const auto tiles_of = [&](int n) { return (long long)tiles_m * ((N + n - 1) / n); };
     const auto split_of = [&](int n) { return (int)std::max<long long>(1, std::min<long long>(std::min(8, CB), kSms / tiles_of(n))); };
     const auto cost_of = [&](int n) {
@@ -410,7 +409,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         if (units > 0x7fffffffLL) return TT_ERR_RESOURCE;
         I = tt_apply_info{};
         I.legal = L; I.changed = changed;
-        I.grid_x = (int)std::min<long long>(units, 148 / cg) * cg; I.grid_y = 1; I.grid_z = 1;   // the launcher clamps to the device's SM count
+        I.grid_x = (int)std::min<long long>(units, kSms / cg) * cg; I.grid_y = 1; I.grid_z = 1;   // the launcher clamps to the device's SM count
         I.threads = kGemmThreads;
         // one CTA per SM: ask for more than half of an SM's shared memory
         I.smem_bytes = (int)std::max<long long>(smem_p, 116 * 1024);
@@ -571,7 +570,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         // which build: two CTAs per SM need half the shared memory and half the tensor memory each
         const bool fits2 = smem <= 112 * 1024 && tmem_cols <= 256;
         const long long ctas = (long long)tiles_m * tiles_n * sk * B;
-        int cps = rec->ctas_per_sm == 0 ? ((ctas > 2 * 148 && fits2) ? 2 : 1) : rec->ctas_per_sm;
+        int cps = rec->ctas_per_sm == 0 ? ((ctas > 2 * kSms && fits2) ? 2 : 1) : rec->ctas_per_sm;
         if (cps == 2 && !fits2) { if (strict) return TT_ERR_INVALID_SCHEDULE; cps = 1; changed |= TT_CHG_FORM; }
         L.ctas_per_sm = cps;
     }
@@ -709,7 +708,7 @@ static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* r
     const tt_schedule_record L = plan->info.legal;
     auto cost = [&](int tn) {
         const long long ctas = (long long)((plan->gm + kHwTileM - 1) / kHwTileM) * ((plan->gn + tn - 1) / tn) * L.split_k * plan->gbatch;
-        return (double)((ctas + 147) / 148) * std::max(1.5 * (kHwTileM + tn), 2.13 * tn);
+        return (double)((ctas + kSms - 1) / kSms) * std::max(1.5 * (kHwTileM + tn), 2.13 * tn);
     };
     if (L.tile_n <= 128 && rec->ctas_per_sm == 0 && cost(2 * L.tile_n) <= 0.85 * cost(L.tile_n)) {
         tt_schedule_record wide = L;
@@ -798,7 +797,7 @@ static bool plan_dw_runs(const tt_workload* w, DwArgs& d, tt_apply_info& I, tt_s
     const int strips_h = (t.tile_h + rows - 1) / rows;
     t.strip_rows = std::min(strips_h, fit);
     if (t.tiles_h == 1) {
-        const long long share = std::max(1LL, planes / (2 * 148));
+        const long long share = std::max(1LL, planes / (2 * kSms));
         t.tile_c = (int)std::min<long long>({(long long)s.c, share, (long long)std::max(1, fit / t.strip_rows), std::max(1LL, 24 * 1024 / (hw * 4))});
         // groups of channels as equal as they come
         const int groups = (s.c + t.tile_c - 1) / t.tile_c;
@@ -836,7 +835,7 @@ static bool plan_dw_runs(const tt_workload* w, DwArgs& d, tt_apply_info& I, tt_s
     t.total_tiles = (int)total;
     const long long per_sm = std::max<long long>(1, std::min<long long>({16LL, (228 * 1024) / (smem + 1024), 2048LL / threads}));
     d = t;
-    I.grid_x = (int)std::min<long long>(total, 148 * per_sm); I.grid_y = 1; I.grid_z = 1;
+    I.grid_x = (int)std::min<long long>(total, kSms * per_sm); I.grid_y = 1; I.grid_z = 1;
     I.threads = threads; I.smem_bytes = (int)smem; I.launches = 1;
     L.raster = 1; L.stages = d.tma_stages; L.unroll = rows; L.items_per_thread = d.items; L.vec_width = d.vec;
     L.tile_m = d.tile_c; L.block_y = d.tile_h; L.block_x = d.tile_w; L.threads = threads;
@@ -941,7 +940,7 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
         const int groups = (s.c + t.tile_c - 1) / t.tile_c;
         if (!strict) {
             rows = window_rows;
-            if (rows == 4 && s.r == 5 && round_up(d.tile_h, 7) <= round_up(d.tile_h, 4) && (planes + d.tile_c - 1) / d.tile_c * d.tiles_h * d.tiles_w >= 148 * 4) rows = 7;
+            if (rows == 4 && s.r == 5 && round_up(d.tile_h, 7) <= round_up(d.tile_h, 4) && (planes + d.tile_c - 1) / d.tile_c * d.tiles_h * d.tiles_w >= kSms * 4) rows = 7;
             t.tile_c = (s.c + groups - 1) / groups;
         }
         int stg = 0;
@@ -969,7 +968,7 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
             d.total_tiles = (int)total;
             smem = smem_of(stg);
             const long long per_sm = std::max<long long>(1, std::min<long long>(8, (228 * 1024) / (smem + 1024)));   // (applying the record lowers it to what registers allow)
-            gx = std::min<long long>(total, 148 * per_sm);
+            gx = std::min<long long>(total, kSms * per_sm);
             I.legal = L;
             I.grid_x = (int)gx; I.grid_y = 1; I.grid_z = 1;
             I.threads = th; I.smem_bytes = (int)smem; I.launches = 1;

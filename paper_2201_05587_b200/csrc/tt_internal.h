@@ -9,6 +9,7 @@ namespace tt {
 
 constexpr int kHwTileM = 128;           // tcgen05 accumulator rows per CTA (cta_group::1, M = 128)
 constexpr int kMaxStages = 8;
+constexpr int kSms = 148;               // SMs that the layout rules deal tiles over (a launch is right on any number)
 constexpr int kSmemLimit = 232448;      // 227 KB opt-in shared memory per CTA on sm_100
 constexpr int kDynSmemLimit = kSmemLimit - 6144;  // what is left for dynamic shared memory beside barriers
 constexpr int kRowSmem = 100 * 1024;    // shared memory of a CTA of the ragged softmax, so that two fit an SM

@@ -66,8 +66,6 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
     return t;
 }
 
-
-
 // Bounded wait.  Returns false when the CTA is aborting (this wait or another one expired).
 static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned* status,
                                             unsigned where, unsigned long long limit_ns) {
@@ -185,14 +183,6 @@ __device__ __forceinline__ void issue_steps_any(uint32_t d_tmem, uint32_t a_hi, 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-// 32 lanes x 16 consecutive 32-bit columns: thread i of the warp receives lane (base + i).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr) : "memory");
-}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor of a K-major tile whose rows are `row_bytes` long and hardware-swizzled with
@@ -254,13 +244,6 @@ __device__ __forceinline__ float apply_act(float v, int act) {
         case TT_ACT_GELU_ERF: return gelu_erf(v);
         default: return v;
     }
-}
-
-// Byte offset of element (row, kk) inside one swizzle atom block of a K-major tile: rows are row_bytes apart
-// and the 16-byte chunk index is XORed with bits 7.. of the linear offset (the TMA swizzle patterns).
-__device__ __forceinline__ uint32_t swz_off(uint32_t row, uint32_t kbyte, uint32_t row_bytes, uint32_t mask) {
-    const uint32_t off = row * row_bytes + kbyte;
-    return off ^ (((off >> 7) & mask) << 4);
 }
 
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, float a, float b, float c, float d) {
@@ -354,6 +337,7 @@ __device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t byt
 // Wait until the stores this thread issued have read their shared memory.
 __device__ __forceinline__ void bulk_stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
+// 32 lanes x 32 consecutive 32-bit columns: thread i of the warp receives lane (base + i).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
