@@ -1006,10 +1006,10 @@ def test_compensated_tiles_of_twice_the_columns(m, k, n, tn, tk, sk):
 
 
 @pytest.mark.parametrize("n, c, h, w, r, stride, act, bias, off", [
-    (5, 301, 14, 14, 5, 1, B.TT_ACT_RELU6, True, 0), (29, 190, 7, 7, 3, 1, B.TT_ACT_NONE, False, 0), (23, 47, 17, 18, 3, 2, B.TT_ACT_RELU, True, 0),
-    (33, 33, 31, 30, 5, 2, B.TT_ACT_GELU_ERF, True, 0), (3, 9, 111, 109, 3, 1, B.TT_ACT_RELU, True, 0), (2, 11, 130, 131, 5, 1, B.TT_ACT_NONE, True, 0),
+    (5, 301, 14, 14, 5, 1, B.TT_ACT_RELU6, True, 0), (29, 190, 7, 7, 3, 1, B.TT_ACT_NONE, False, 0), (80, 47, 17, 18, 3, 2, B.TT_ACT_RELU, True, 0),
+    (37, 33, 31, 30, 5, 2, B.TT_ACT_GELU_ERF, True, 0), (3, 9, 111, 109, 3, 1, B.TT_ACT_RELU, True, 0), (2, 11, 130, 131, 5, 1, B.TT_ACT_NONE, True, 0),
     (3, 53, 5, 342, 3, 1, B.TT_ACT_RELU, True, 0), (9, 65, 33, 45, 5, 1, B.TT_ACT_RELU6, True, 1), (4, 403, 13, 14, 3, 1, B.TT_ACT_RELU6, True, 3),
-    (1, 131200, 2, 1, 3, 1, B.TT_ACT_RELU, True, 0), (3, 70, 253, 37, 3, 2, B.TT_ACT_NONE, False, 2), (3, 5, 150, 150, 5, 2, B.TT_ACT_NONE, False, 0)])
+    (1, 131200, 2, 1, 3, 1, B.TT_ACT_RELU, True, 0), (3, 70, 253, 37, 3, 2, B.TT_ACT_NONE, False, 2), (3, 17, 150, 150, 5, 2, B.TT_ACT_NONE, False, 0)])
 def test_depthwise_rows_staged_as_runs(n, c, h, w, r, stride, act, bias, off):
     """A batch of images whose rows are no 16-byte multiples: odd and even rows, planes and bands of planes, groups of channels
     with a remainder, a tensor that ends inside 16 bytes, an input that starts inside them.  Each output is bounded against the
@@ -1021,6 +1021,10 @@ def test_depthwise_rows_staged_as_runs(n, c, h, w, r, stride, act, bias, off):
     a = W.make_inputs(spec, 96)
     ref = util.oracle_ref(spec, a)
     rec = B.make_record(B.TT_FAMILY_DW_SIMT, tile_m=4, block_y=8, block_x=32, items_per_thread=4, vec_width=4, threads=128, unroll=2)
+    probe = spec.workload()
+    legal = probe.check(rec)[1].legal                    # (rows of more than 256 outputs have no such form)
+    assert legal.raster == ((w - 1) // stride + 1 <= 256), legal.short()
+    probe.close()
     y = run_spec(spec, rec, a, ref, ref_elem=ref)
     if off:
         t, _ = W.device_tensors(spec, a)
@@ -1347,4 +1351,41 @@ def test_staged_depthwise_grid_is_settled_when_the_record_is_applied():
     for s, a, (t, _) in zip(sp, arrays, bufs):
         assert util.rel_l2(t["y"].cpu().numpy(), util.oracle_ref(s, a)) <= util.TOL_FP32
     for wl in wls:
+        wl.close()
+
+
+@pytest.mark.parametrize("items", [1, 2])
+@pytest.mark.parametrize("rows", [2, 4, 7])
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("r", [3, 5])
+def test_every_run_staged_instantiation(r, stride, rows, items):
+    """Filter, stride, strip height and columns per thread of the run-staged form, each reached by its own batch: planes with a
+    partial last strip, rows that end inside a strip's columns, bands of a plane, an input that starts inside 16 bytes.  Bounded against the oracle and
+    bit-identical to the register-window form, which strict mode runs as written."""
+    import torch
+    p = {2: 2, 4: 8, 7: 13}[rows]
+    shapes = [(p, 21 if items == 1 else 22)] + ([(131, 77 if items == 1 else 50)] if rows == 7 else [])
+    for k, (out_h, w) in enumerate(shapes):
+        h = out_h if k or stride == 1 else 2 * out_h - (items - 1)
+        ph, q = (h - 1) // stride + 1, (w - 1) // stride + 1
+        c = 37
+        n = -(-(1 << 18) // (c * ph * q))
+        spec = W.Spec(B.TT_OP_DWCONV2D, B.make_shapes(n=n, c=c, h=h, w=w, k=c, r=r, s=r, stride_h=stride, stride_w=stride, pad_h=r // 2, pad_w=r // 2,
+                                                      has_bias=1, act=(B.TT_ACT_RELU6, B.TT_ACT_GELU_ERF)[k]), 1, f"runs_{r}{stride}{rows}{items}", "uniform")
+        a = W.make_inputs(spec, 100 + k)
+        ref = util.oracle_ref(spec, a)
+        rec = B.make_record(B.TT_FAMILY_DW_SIMT, tile_m=4, block_y=min(8, ph), block_x=8, items_per_thread=4, vec_width=1, threads=64, unroll=2)
+        wl = spec.workload()
+        legal = wl.apply(rec).legal
+        assert (legal.raster, legal.unroll, legal.items_per_thread) == (1, rows, items), legal.short()
+        assert (legal.block_y < ph) == (k == 1)
+        y = run_spec(spec, rec, a, ref, ref_elem=ref)
+        np.testing.assert_array_equal(run_spec(spec, rec, a, mode=B.TT_MODE_STRICT), y)
+        t, _ = W.device_tensors(spec, a)
+        size = t["x"].numel()
+        x = torch.empty(size + 4, device="cuda")[3:3 + size].view(t["x"].shape).copy_(t["x"])
+        t["y"].fill_(float("nan"))
+        wl.run(B.tensors(x, t["w"], t["bias"], t["residual"], t["y"]))
+        assert wl.status() == B.TT_OK
+        np.testing.assert_array_equal(t["y"].cpu().numpy(), y)
         wl.close()
