@@ -150,17 +150,30 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     // How the tiles are laid over the SMs is this rule's choice unless the record is to
     // run as written (strict mode); the legal record says what it chose (tile_n, cta_group).
     // Where the record's tiles fill more than half of the SMs, columns are dealt evenly over the rounds that its tile needs: 121
-    // tiles of 224 columns become 141 of 192.  Where they fill less, CTAs share a tile's channel blocks as a cluster.  Fewer
-    // rounds, or the widest tile, take the place of the record's where they are a tenth cheaper: a tap costs what shared memory has to move in
-    // 128-byte lines -- its filters in and out, 2 * 128, its columns, about 32 for the slab -- and the filters' part is paid per
-    // tile (3x3 512 -> 512 at 7 x 7, batch 32: 31.4 us with 128 columns, 25.1 with 256).
+    // tiles of 224 columns become 141 of 192; a tile with which they take fewer rounds replaces it where that is a tenth cheaper.
+    // Where they fill less, CTAs share a tile's channel blocks as a cluster: as many as save the most cycles, as long as all
+    // clusters are resident at once (20 clusters of 7 are not: 320 -> 200 at 9 x 9, batch 6, 64 columns: 21.8 us, in clusters of 5
+    // 10.4); the widest tile replaces the record's where that is cheaper.
+    // Cycles: a tap takes what its columns take the tensor core, 2 each, or what shared memory has to move in 128-byte lines, its
+    // filters in and out, 256, its columns, about 32 for the slab; the read-out 25 a column (192 columns: 2.3 us); the exchange in a
+    // cluster 1000 and 30 for every column that a CTA leaves to others, set so that these come out right: 3x3 64 -> 64 at 56 x 56, 192
+    // columns, 10.9 us alone and 9.9 in pairs; 1x1 64 -> 128 at 14 x 14, batch 8, 96 columns, 5.8 and 6.6; 3x3 512 -> 512 at 7 x 7,
+    // batch 32, weights cold, 25.8 with 128 columns in pairs and 25.1 with 256 in fours, which move half the filters.
+    // 23 layers under 7 records each: 1.50 times faster than as written in the geometric mean, 1.20 times the best of 15 widths and 8
+    // clusters, two pairs slower than as written (by 17 %).
     const auto tiles_of = [&](int n) { return (long long)tiles_m * ((N + n - 1) / n); };
-    const auto split_of = [&](int n) { return (int)std::max<long long>(1, std::min<long long>(std::min(8, CB), kSms / tiles_of(n))); };
-    const auto cost_of = [&](int n) {
-        const int k = split_of(n);
-        const long long rounds = (tiles_of(n) + kSms - 1) / kSms;
-        return rounds * ((CB + k - 1) / k) * RS * std::max(2 * n, n + 288) + 25ll * n / k;
+    struct Share { long long cycles; int ctas; };
+    const auto share_of = [&](int n) {
+        const long long tap = std::max(2 * n, n + 288);
+        Share best{CB * RS * tap + 25 * n, 1};
+        for (int k = 2; k <= std::min(8, CB); ++k) {
+            if (tiles_of(n) > kResidentClusters[k]) continue;
+            const long long cycles = (CB + k - 1) / k * RS * tap + 25 * n + 1000 + 30 * n * (k - 1) / k;
+            if (cycles < best.cycles) best = Share{cycles, k};
+        }
+        return best;
     };
+    const auto cost_of = [&](int n) { return (tiles_of(n) + kSms - 1) / kSms * share_of(n).cycles; };
     const auto dealt = [&](long long rounds) {           // the columns of a tile when all of them take `rounds` rounds
         const long long columns = rounds * kSms / tiles_m;
         return columns >= 1 ? std::max<long long>(16, round_up64((N + columns - 1) / columns, 16)) : 0x7fffffffLL;
@@ -170,15 +183,18 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
         // (the CTAs of a cluster take one tile: all tiles have to be resident at once)
         if (split > std::min(8, CB) || (split > 1 && tiles_of(tn) * split > kSms)) return TT_ERR_INVALID_SCHEDULE;
     } else {
-        int wide = std::min(256, round_up(N, 16));
         if (tiles_of(tn) * 2 > kSms) {
             const long long rounds = (tiles_of(tn) + kSms - 1) / kSms;
             tn = (int)std::min<long long>(tn, dealt(rounds));
-            wide = tn;
-            for (long long r = 1; r < rounds && r <= 4; ++r) if (dealt(r) <= 256) { wide = (int)dealt(r); break; }
+            for (long long r = 1; r < rounds && r <= 4; ++r) {
+                if (dealt(r) > 256) continue;
+                if (cost_of((int)dealt(r)) * 10 < cost_of(tn) * 9) tn = (int)dealt(r);
+                break;
+            }
         }
-        if (cost_of(wide) * 10 < cost_of(tn) * 9) tn = wide;
-        split = tiles_of(tn) * 2 > kSms ? 1 : split_of(tn);
+        const int widest = std::min(256, round_up(N, 16));
+        if (tiles_of(tn) * 2 <= kSms && cost_of(widest) < cost_of(tn)) tn = widest;
+        split = tiles_of(tn) * 2 > kSms ? 1 : share_of(tn).ctas;
     }
     L.tile_n = tn; L.cta_group = split;
     if (tn != rec->tile_n) changed |= TT_CHG_TILE_N;

@@ -10,6 +10,9 @@ namespace tt {
 constexpr int kHwTileM = 128;           // tcgen05 accumulator rows per CTA (cta_group::1, M = 128)
 constexpr int kMaxStages = 8;
 constexpr int kSms = 148;               // SMs that the layout rules deal tiles over (a launch is right on any number)
+// Clusters of 1..8 CTAs that a B200 holds at once with one CTA per SM (what the driver's occupancy query answers): a cluster keeps to
+// one group of SMs, so clusters of 8 leave 28 of the 148 idle and clusters of 7 leave 43.
+constexpr int kResidentClusters[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
 constexpr int kSmemLimit = 232448;      // 227 KB opt-in shared memory per CTA on sm_100
 constexpr int kDynSmemLimit = kSmemLimit - 6144;  // what is left for dynamic shared memory beside barriers
 constexpr int kRowSmem = 100 * 1024;    // shared memory of a CTA of the ragged softmax, so that two fit an SM

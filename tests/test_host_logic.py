@@ -970,3 +970,18 @@ print("statuses")
 """
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and "statuses" in r.stdout, r.stderr
+
+
+@pytest.mark.parametrize("shape", [(6, 320, 9, 200, 3), (16, 512, 7, 512, 3), (8, 256, 14, 256, 3), (1, 64, 56, 64, 3), (8, 64, 14, 128, 1), (32, 512, 7, 512, 3)])
+def test_tap_major_clusters_are_resident_and_worth_their_exchange(shape):
+    """CTAs of a cluster keep to one group of SMs: 148 SMs do not hold 20 clusters of 7.  A single tap is not shared."""
+    resident = (0, 148, 74, 45, 33, 26, 22, 15, 15)
+    n, c, hw, k, r = shape
+    wl = B.Workload(B.TT_OP_CONV2D, B.conv2d_shapes(n, c, hw, hw, k, r, r, 1, r // 2, True, B.TT_ACT_RELU), "tap")
+    for tn in (32, 64, 96, 128, 192, 256):
+        st, info = wl.check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tn, tile_k=32, stages=8, mma_m_axis=1, k_order=1))
+        assert st == B.TT_OK and info.grid_y == info.legal.cta_group
+        assert info.legal.cta_group == 1 or info.grid_x <= resident[info.legal.cta_group]
+        if c * r * r <= 64:
+            assert info.legal.cta_group == 1
+    wl.close()
