@@ -23,8 +23,8 @@
 // buffers and the loads of a block run while the block before it is multiplied.  The slab warps load from global memory
 // straight into registers (32 channels of 32 positions in flight per warp) and store 16 bytes per lane without conflicts: no
 // staging buffer, no alignment asked of the image rows.
-// Where all tiles are resident at once there is nothing to overlap with: then the slab warps help to read out, and if the
-// tiles would leave more than half of the SMs idle, a cluster of CTAs shares a tile's channel blocks: each leaves the blocks
+// Where all tiles are resident at once there is nothing to overlap with: then the slab warps help to read out, and a cluster of
+// CTAs (the record's cta_group) may share a tile's channel blocks: each leaves the blocks
 // of its accumulator that another CTA finishes in its shared memory, and every CTA adds up its blocks, in CTA order, over
 // distributed shared memory.
 //

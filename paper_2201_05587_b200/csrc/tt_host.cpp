@@ -698,7 +698,10 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
 // Where only one of the record's stages fits, it becomes several of 32, so that the three steps overlap (512 x 1024 over 4096,
 // stages of 64 with 128 columns: 182 us; as three of 32: 99).  Two of 64 are 3 % faster than four of 32.
 // Where a tile of twice the record's columns does a round of the SMs for less, it takes its place (512 x 1024 over 4096 in
-// quarters: 256 tiles of 64 columns are two rounds of 288 cycles a step, 128 of 128 one of 384).
+// quarters: 256 tiles of 64 columns are two rounds of 288 cycles a step, 128 of 128 one of 384).  The line lies at 0.85 of the
+// record's cycles: at 0.60-0.67 the wide tile took 51.9 -> 39.4 us there, 97.1 -> 48.4 (32 columns), 31.7 -> 23.5 (256 x 4096 over
+// 1024), 29.0 -> 17.3 (4096 x 512 over 512) and once 41.4 -> 42.5 (600 x 600 over 3000, 48 columns); at 0.89 46.0 -> 43.7 to
+// 27.5 -> 24.1, which the wider grid's share of idle SMs makes a gamble on other sizes; at 1.4-1.5 30.5 -> 50.7 and 23.4 -> 38.1.
 static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, Plan* plan) {
     const Plan fresh = *plan;
     const tt_status s = plan_gemm(w, rec, mode, plan);
@@ -790,6 +793,10 @@ static bool plan_dw_runs(const tt_workload* w, DwArgs& d, tt_apply_info& I, tt_s
     if (s.w % 4 == 0 || w->Q > 256 || planes > 0x7fffffffLL || hw > (1 << 24)) return false;
     DwArgs t = d;
     double best_cost = 0;
+    // Instructions of a strip: per window row its reads, their predicates and its address, per output row its products, clamp and
+    // store, 40 to set it up.  On 12 shapes of both filters and strides the choice is the fastest of the three or within 5 % of it
+    // (480 x 14 x 14, 5x5, 256 images: 7 rows 58.9 us, 4 84.4, 2 113; 200 x 15 x 15, 5x5, 64 images: 4 rows 15.9, 7 16.3; 120 x 31 x 33, 3x3
+    // stride 2, 32 images: 4 rows 6.9, 7 7.5; the 5 %: 576 x 14 x 14, 3x3 stride 2, 256 images: 7 rows 28.1, 4 26.7).
     for (int rows : {7, 4, 2}) {
         const int in_rows = (rows - 1) * s.stride_h + s.r;
         const double cost = (double)((w->P + rows - 1) / rows) * (in_rows * (2.0 * s.r + 3) + rows * (s.r * s.r + 4.0) + 40);
@@ -948,8 +955,11 @@ static tt_status legalise_dw(const tt_workload* w, const tt_schedule_record* rec
     if (rec->raster == 1 && window_rows > 0 && (s.w % 4) == 0) {
         const long long planes = (long long)s.n * s.c;
         // Unless the record is to run as written (strict mode): tiles keep to one image, in groups of channels as equal as they
-        // come, and a 5x5 filter's tallest strip becomes one of seven rows where that covers the tile as well and the chip has tiles to spare: a
-        // strip then reads 11 rows for 7, not 8 for 4 (3x3: 9 for 7 against 6 for 4, and it was slower on 56-pixel rows, 157 -> 173 us).
+        // come, and a 5x5 filter's strips of 4 rows become strips of 7 where those cover the tile as well and the chip has tiles to
+        // spare: a strip then reads 11 rows for 7, not 8 for 4.  256 images of 240 x 28 x 28: 98 -> 81 us; 32 of 200 x 56 x 56: 43 -> 37; 16 of
+        // 240 x 28 x 28: 10.9 -> 10.2; stride 2, 64 of 96 x 112 x 112: 76 -> 66, but 32 of 200 x 56 x 56: 22.5 -> 23.6.  Elsewhere: 4 of 240 x 28 x 28
+        // (240 tiles) 5.3 -> 6.3, 20-row tiles 38 -> 40, 12-row tiles 16 -> 20.  A 3x3 filter reads 9 rows for 7 against 6 for 4: 56-pixel rows 44 -> 45
+        // and 40 -> 45, 28-pixel 61 -> 62, 20-pixel 36 -> 38, stride 2 at 112 32.9 -> 32.7.
         // Everything below is about the tile that runs, and so is the legal record.
         int rows = L.unroll;
         DwArgs t = d;

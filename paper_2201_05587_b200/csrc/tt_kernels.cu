@@ -2347,7 +2347,8 @@ __global__ void __launch_bounds__(cached_threads(NV)) tt_softmax_cached_kernel(c
 // One bulk copy brings them to shared memory, the lanes read them value by value (NV per lane, kept in registers), write
 // the results over them, and one bulk copy takes them back: memory sees whole lines only.  Warps do not meet.
 // Next to memory the instructions per value bind (4-byte accesses; the exponential alone is half a dozen), so NV is the
-// exact number of values per lane up to 32 and only the last of them is guarded.
+// exact number of values per lane up to 32 and only the last of them is guarded.  (Even counts only, the last two guarded: 5 to
+// 13 % slower up to 8 values, 45.8 -> 49.3 us for rows of 197 with 7; 5 % at 13 and 25; the same at 16 and 32.)
 // 151296 rows of 197 columns: 136 us in three passes of 4-byte accesses from memory, 57 us with guards on every value,
 // 38 us this way (6.3 TB/s; floor 36 us).
 constexpr int kRaggedExact = 32;                         // values per lane up to which there is an instantiation for each count
