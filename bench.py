@@ -443,6 +443,8 @@ class Bench:
                 for _ in range(u):
                     w.run(t)
 
+        if plan is not None:
+            launches_pass = B.chain_launches(wls, steps_, ch_tts, plan)      # (layers that go to the device together are one)
         n_side = max(5, min(steps, 30))
         graph = self.capture(chained_pass)
         self.timed_steps(warmup, graph.replay)

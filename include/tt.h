@@ -299,9 +299,15 @@ typedef struct tt_chain_step {
  * device.  Nothing is synchronised.  On an
  * error the layers in front of the failing one have been enqueued and the side streams joined; failed_at (may be NULL)
  * receives its position.  Layers may share a workload; those on different lanes run side by side, or one after the other
- * where the workload has scratch (workspace_bytes > 0).  Calls for the same workloads do not overlap in time (one handle,
+ * where the workload has scratch (workspace_bytes > 0).  Layers may share a launch, where the results are the same: up to three
+ * dense layers of one workload on the same x that do not touch one another's tensors (on the lane of the first, under the record
+ * applied), and a batch_matmul NT, the softmax of its result and the batch_matmul NN of that (up to 256 columns, as many rows as
+ * are resident at once, not under strict records; all three outputs are written).  Calls for the same workloads do not overlap in time (one handle,
  * one thread), calls for different ones may run on different threads. */
 tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* streams, size_t n_streams, size_t* failed_at);
+/* How many kernels that pass launches: layers may go to the device together (see above), a layer under a record with a filter
+ * re-pack takes two. */
+tt_status tt_chain_launches(const tt_chain_step* steps, size_t n_steps, size_t* launches);
 /* tt_run with HOST pointers: copies x, w, bias, residual to library-owned device buffers, runs, copies y back,
  * synchronises.  bytes_h2d/bytes_d2h (may be NULL) receive the bytes copied. */
 tt_status tt_run_host(tt_workload* w, const tt_tensors* host, void* cuda_stream, int64_t* bytes_h2d, int64_t* bytes_d2h);

@@ -118,6 +118,7 @@ EXPORTS = {
     "tt_split_check": (i32, [C.c_int64, C.POINTER(C.c_int64), C.c_size_t, i32, C.POINTER(i32)]),
     "tt_run": (i32, [C.c_void_p, C.POINTER(tt_tensors), C.c_void_p]),
     "tt_run_chain": (i32, [C.POINTER(tt_chain_step), C.c_size_t, C.POINTER(C.c_void_p), C.c_size_t, C.POINTER(C.c_size_t)]),
+    "tt_chain_launches": (i32, [C.POINTER(tt_chain_step), C.c_size_t, C.POINTER(C.c_size_t)]),
     "tt_run_host": (i32, [C.c_void_p, C.POINTER(tt_tensors), C.c_void_p, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]),
     "tt_run_host_async": (i32, [C.c_void_p, C.POINTER(tt_tensors), C.c_void_p, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]),
     "tt_workload_status": (i32, [C.c_void_p, C.c_void_p]),
@@ -340,6 +341,22 @@ def run_chain(wls, steps, tts, plan, streams):
             st, at = _call.run_chain(wls, steps, tts, plan, [s.cuda_stream for s in streams])
     if st != TT_OK:
         raise TTError(st, f"tt_run({wls[steps[at].kernel].name})" if at >= 0 else "tt_run_chain")
+
+
+def chain_launches(wls, steps, tts, plan):
+    """How many kernels run_chain launches for these arguments (tt_chain_launches)."""
+    chain, position, keep = [], {}, []
+    for i, (st, tt, pl) in enumerate(zip(steps, tts, plan)):
+        if pl is None:
+            continue
+        lane, waits = pl
+        waits = (i32 * max(len(waits), 1))(*[position[p] for p in waits])
+        keep.append(waits)
+        position[i] = len(chain)
+        chain.append(tt_chain_step(wls[st.kernel].handle, C.pointer(tt), waits, len(pl[1]), lane))
+    n = C.c_size_t()
+    _check(lib().tt_chain_launches((tt_chain_step * len(chain))(*chain), len(chain), C.byref(n)), "tt_chain_launches")
+    return n.value
 
 
 def _run_chain_over_devices(wls, steps, tts, plan, streams):

@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libtt.so")
-SOURCES = ["tt_host.cpp", "tt_kernels.cu", "tt_conv.cu", "tt_device.cu"]
+SOURCES = ["tt_host.cpp", "tt_kernels.cu", "tt_conv.cu", "tt_attention.cu", "tt_device.cu"]
 HEADERS = [os.path.join(CSRC, "tt_internal.h"), os.path.join(CSRC, "tt_ptx.cuh"), os.path.join(ROOT, "include", "tt.h")]
 CALL_LIB = os.path.join(HERE, "_ttcall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 CALL_SOURCE = os.path.join(CSRC, "tt_pycall.cpp")

@@ -14,7 +14,8 @@
 namespace tt {
 
 cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
-                        cudaStream_t st);
+                        const void* tmap_z, cudaStream_t st);
+cudaError_t launch_attention(const AttnArgs& g, int heads, const void* tmap_q, const void* tmap_k, const void* tmap_v, cudaStream_t st);
 cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st);
 cudaError_t plan_dw_staged(tt_apply_info& I, DwArgs& dw);
 cudaError_t launch_dw_staged(const tt_apply_info& I, const DwArgs& dw, const void* tmap_x, cudaStream_t st);
@@ -366,7 +367,19 @@ static tt_status launch_tap_major(tt_workload* w, const tt_tensors* t, cudaStrea
     return TT_OK;
 }
 
-tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) try {
+// What a launch of a chained pass does beside its own layer: further layers of the same plan on the same x (their tensors), and
+// the weights it brings into the L2 for the launches behind it.
+struct Beside {
+    const tt_tensors* more[2] = {nullptr, nullptr};
+    int n_more = 0;
+    Ahead ahead{};
+};
+
+static tt_status launch_with(tt_workload* w, const tt_tensors* t, void* stream, const Beside& beside);
+
+tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) { return launch_with(w, t, stream, Beside{}); }
+
+static tt_status launch_with(tt_workload* w, const tt_tensors* t, void* stream, const Beside& beside) try {
     if (!w || !t) return TT_ERR_INVALID_ARG;
     if (!w->plan.applied) return TT_ERR_NOT_APPLIED;
     if (!t->x || !t->y) return TT_ERR_INVALID_ARG;
@@ -375,7 +388,7 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) try {
     if (w->sh.has_residual && !t->residual) return TT_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaSuccess;
-    const Plan& p = w->plan;
+    const Plan& p = beside.n_more > 0 ? w->group[beside.n_more - 1] : w->plan;
     if (w->family == TT_FAMILY_GEMM_TC) {
         if (p.repack) return launch_tap_major(w, t, st);
         GemmArgs g = p.g;
@@ -407,10 +420,24 @@ tt_status launch(tt_workload* w, const tt_tensors* t, void* stream) try {
             if (g.a_mode == OPM_TMA_MN && (reinterpret_cast<uintptr_t>(a_ptr) & 15u) != 0) { g.a_mode = OPM_GATHER_ROWS; g.idesc &= ~(1u << 15); }
             if (g.b_mode == OPM_TMA_MN && (reinterpret_cast<uintptr_t>(b_ptr) & 15u) != 0) { g.b_mode = OPM_GATHER_ROWS; g.idesc &= ~(1u << 16); }
         }
+        // (copies: what a further member's maps add to the cache may move the first's)
         const TmapPair* maps = nullptr;
+        unsigned char more[2][128];
+        g.group = 1 + beside.n_more;
+        g.w_member = p.a_tensor == 1 ? 1 : 2;
+        for (int i = 0; i < beside.n_more; ++i) {
+            const tt_tensors* o = beside.more[i];
+            const tt_status s = tensor_maps_for(w, g, pick(o, p.a_tensor), pick(o, p.b_tensor), &maps);
+            if (s != TT_OK) return s;
+            std::memcpy(more[i], p.a_tensor == 1 ? maps->a : maps->b, 128);
+            g.bias_more[i] = w->sh.has_bias ? static_cast<const float*>(o->bias) : nullptr;
+            g.y_more[i] = static_cast<float*>(o->y);
+        }
         const tt_status s = tensor_maps_for(w, g, a_ptr, b_ptr, &maps);
         if (s != TT_OK) return s;
-        e = g.persistent ? launch_gemm_ps(p.info, g, *maps, st) : launch_gemm(p.info, p.run_smem, g, maps->a, maps->b, maps->x, st);
+        g.ahead = beside.ahead;
+        e = g.persistent ? launch_gemm_ps(p.info, g, *maps, st)
+                         : launch_gemm(p.info, p.run_smem, g, maps->a, maps->b, beside.n_more > 0 ? more[0] : maps->x, beside.n_more > 1 ? more[1] : maps->x, st);
     } else if (w->family == TT_FAMILY_DW_SIMT) {
         DwArgs d = p.dw;
         d.x = static_cast<const float*>(t->x); d.w = static_cast<const float*>(t->w);
@@ -597,6 +624,8 @@ static tt_status apply_impl(tt_workload* w, const tt_schedule_record* rec, int m
     s = bind_device(w);
     if (s != TT_OK) { w->plan = old; w->plan.applied = false; return s; }
     w->plan.applied = true;
+    w->plan.strict = mode == TT_MODE_STRICT;
+    plan_groups(w);
     if (info) *info = w->plan.info;               // (the grid that the device holds)
     return TT_OK;
 }
@@ -619,39 +648,238 @@ tt_status tt_schedule_apply_ex(tt_workload* w, const tt_schedule_record* rec, in
 
 tt_status tt_run(tt_workload* w, const tt_tensors* t, void* cuda_stream) { return launch(w, t, cuda_stream); }
 
+// ---- chained passes -----------------------------------------------------------------------------------------
+
+// Layers that go to the device together, and where.
+struct ChainLaunch {
+    size_t first; int count; bool attention;
+    int32_t lane;
+    bool needed, moved;                                  // somebody on another lane waits for it; a member's plan lane is another one
+    Ahead ahead;
+};
+
+struct Range { const char* p; size_t bytes; };
+static bool overlap(const Range& a, const Range& b) { return a.p && b.p && a.p < b.p + b.bytes && b.p < a.p + a.bytes; }
+// x, w, bias, residual, y of a layer
+static Range range_of(const tt_chain_step& s, int which) {
+    const tt_tensors& t = *s.tensors;
+    const void* p[5] = {t.x, t.w, t.bias, t.residual, t.y};
+    return Range{static_cast<const char*>(p[which]), tensor_elems(s.workload, which) * 4};
+}
+// May layer b run beside layer a (neither writes what the other one touches)?
+static bool independent(const tt_chain_step& a, const tt_chain_step& b) {
+    const Range ya = range_of(a, 4), yb = range_of(b, 4);
+    for (int i = 0; i < 5; ++i)
+        if (overlap(ya, range_of(b, i)) || overlap(yb, range_of(a, i))) return false;
+    return true;
+}
+static bool usable(const tt_chain_step& s) {
+    return s.workload && s.tensors && s.workload->plan.applied && s.tensors->x && s.tensors->y && (s.workload->op == TT_OP_SOFTMAX || s.tensors->w) &&
+           (!s.workload->sh.has_bias || s.tensors->bias) && (!s.workload->sh.has_residual || s.tensors->residual);
+}
+static bool waits_in_front(const tt_chain_step& s, size_t first) {
+    for (int32_t j = 0; j < s.n_waits; ++j) if ((size_t)s.waits[j] >= first) return false;
+    return true;
+}
+
+// How many layers from `first` on are one plan on the same activations: the projections of an attention block.  One launch of
+// three fills the SMs that a launch of one leaves idle (768 -> 768 on 128 rows: 48 CTAs), without streams to fork and join.
+static int group_at(const tt_chain_step* steps, size_t n_steps, size_t first) {
+    const tt_chain_step& a = steps[first];
+    if (!usable(a)) return 1;
+    const tt_workload* w = a.workload;
+    if (w->extra_tx || !(w->group[0].applied || w->group[1].applied)) return 1;
+    int count = 1;
+    while (count < 3 && first + count < n_steps) {
+        const tt_chain_step& b = steps[first + count];
+        if (b.workload != w || !usable(b) || b.tensors->x != a.tensors->x || !waits_in_front(b, first)) break;
+        // (a layer that cannot run is left to fail by itself)
+        if (((reinterpret_cast<uintptr_t>(a.tensors->w) | reinterpret_cast<uintptr_t>(b.tensors->w)) & 15u) != 0) break;
+        // one launch stores all members the same way
+        if (((reinterpret_cast<uintptr_t>(b.tensors->y) ^ reinterpret_cast<uintptr_t>(a.tensors->y)) & 15u) != 0) break;
+        bool apart = true;
+        for (int i = 0; i < count; ++i) apart = apart && independent(steps[first + i], b);
+        if (!apart) break;
+        ++count;
+    }
+    while (count > 1 && !w->group[count - 2].applied) --count;
+    return count;
+}
+
+// Scores, softmax, context from `first` on, as one launch: 12 heads of 128 rows and 64 columns took three launches of 3.6, 1.6
+// and 5.4 us, the 12-layer encoder 511 us with them and 430 with this one.  Only where the heads' blocks of query rows are resident at once (batch 1); from there on the layers fill the chip
+// one by one and each has a kernel made for that.
+static bool attention_at(const tt_chain_step* steps, size_t n_steps, size_t first, AttnArgs* g) {
+    if (first + 3 > n_steps) return false;
+    const tt_chain_step *s = steps + first;
+    for (int i = 0; i < 3; ++i)
+        if (!usable(s[i]) || s[i].workload->plan.strict || s[i].workload->extra_tx) return false;
+    const tt_workload *qk = s[0].workload, *sm = s[1].workload, *pv = s[2].workload;
+    if (qk->op != TT_OP_BATCH_MATMUL || !qk->sh.trans_b || sm->op != TT_OP_SOFTMAX || pv->op != TT_OP_BATCH_MATMUL || pv->sh.trans_b) return false;
+    for (const tt_workload* w : {qk, pv})
+        if (w->sh.has_bias || w->sh.has_residual || w->sh.act != TT_ACT_NONE || w->plan.g.x3) return false;
+    const int heads = qk->sh.batch, m = qk->sh.m, n = qk->sh.nn, d = qk->sh.kk, dv = pv->sh.nn;
+    if (sm->sh.batch != heads || sm->sh.m != m || sm->sh.nn != n || pv->sh.batch != heads || pv->sh.m != m || pv->sh.kk != n) return false;
+    if (n > 256 || d > 128 || dv > 128 || d % 4 || dv % 4 || (long long)heads * ((m + kAttnRows - 1) / kAttnRows) > kSms) return false;
+    const tt_tensors &tq = *s[0].tensors, &ts = *s[1].tensors, &tv = *s[2].tensors;
+    if (ts.x != tq.y || tv.x != ts.y || ((reinterpret_cast<uintptr_t>(tq.x) | reinterpret_cast<uintptr_t>(tq.w) | reinterpret_cast<uintptr_t>(tv.w)) & 15u)) return false;
+    // the three outputs lie apart from each other and from everything that is read
+    const Range in[3] = {range_of(s[0], 0), range_of(s[0], 1), range_of(s[2], 1)}, out[3] = {range_of(s[0], 4), range_of(s[1], 4), range_of(s[2], 4)};
+    for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j)
+            if (overlap(out[i], in[j]) || (i != j && overlap(out[i], out[j]))) return false;
+    // waits and streams: a layer behind the first may only wait for layers in front of it or inside
+    for (int i = 0; i < 3; ++i)
+        for (int32_t j = 0; j < s[i].n_waits; ++j) if ((size_t)s[i].waits[j] >= first + i) return false;
+    AttnArgs a{};
+    a.scores = static_cast<float*>(tq.y); a.probs = static_cast<float*>(ts.y); a.ctx = static_cast<float*>(tv.y);
+    a.status = qk->status_word; a.wait_ns = qk->wait_ns;
+    a.m = m; a.n = n; a.dv = dv; a.tiles_m = (m + kAttnRows - 1) / kAttnRows;
+    a.n16 = (n + 15) / 16 * 16; a.n8 = (n + 7) / 8 * 8; a.n_blocks = (n + 31) / 32;
+    a.d_atoms = (d + 31) / 32; a.d_steps = (d + 7) / 8; a.v_boxes = (dv + 31) / 32;
+    const auto vec = [](const void* p, int cols) { return cols % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
+    a.scores_vec = vec(a.scores, n); a.probs_vec = vec(a.probs, n); a.ctx_vec = vec(a.ctx, dv);
+    a.scale = sm->sh.scale;
+    const int block = kAttnRows * 128;                   // 32 columns of a tile of query rows
+    a.p_off = (unsigned)(a.d_atoms * block);
+    a.k_off = a.p_off + (unsigned)(a.n_blocks * block);
+    a.v_off = a.k_off + (unsigned)std::max(a.d_atoms * a.n16 * 128, a.n_blocks * block);
+    // (the tensor core reads 128 rows of a tile that has 32: all of that lies inside)
+    const int over = 128 * 128 - block;
+    const int bytes = std::max((int)a.v_off + a.v_boxes * a.n8 * 128, (int)a.k_off + over) + 1024;
+    if (bytes > kDynSmemLimit) return false;
+    a.smem_bytes = bytes;
+    a.o_col = a.n_blocks * 32;
+    a.tmem_cols = 32;
+    while (a.tmem_cols < (unsigned)(a.o_col + a.v_boxes * 32)) a.tmem_cols *= 2;
+    const unsigned tf32 = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(kHwTileM >> 4) << 24);
+    a.idesc_s = tf32 | ((unsigned)(a.n16 >> 3) << 17);
+    a.idesc_o = tf32 | ((unsigned)((dv + 15) / 16 * 2) << 17) | (1u << 16);
+    if (g) *g = a;
+    return true;
+}
+
+// How many layers from `first` on go to the device together.
+static int together_at(const tt_chain_step* steps, size_t n_steps, size_t first, bool* attention) {
+    *attention = attention_at(steps, n_steps, first, nullptr);
+    return *attention ? 3 : group_at(steps, n_steps, first);
+}
+
+static tt_status launch_chain_attention(const tt_chain_step* s, const AttnArgs& g, cudaStream_t st) {
+    tt_workload *qk = s[0].workload, *pv = s[2].workload;
+    const tt_shapes& sh = qk->sh;
+    // the maps of the queries and keys are kept with the scores' workload, the values' with the context's
+    const auto cached = [](tt_workload* w, const void* a, const void* b) -> const TmapPair* {
+        for (const TmapPair& m : w->tmaps) if (m.a_ptr == a && m.b_ptr == b && m.y_ptr == w && !m.r_ptr) return &m;
+        return nullptr;
+    };
+    const auto keep = [](tt_workload* w, TmapPair& m, const void* a, const void* b) {
+        m.a_ptr = a; m.b_ptr = b; m.y_ptr = w; m.r_ptr = nullptr;
+        if (w->tmaps.size() >= 4096) w->tmaps.clear();
+        w->tmaps.push_back(m);
+        return &w->tmaps.back();
+    };
+    const void *q = s[0].tensors->x, *k = s[0].tensors->w, *v = s[2].tensors->w;
+    const TmapPair* m = cached(qk, q, k);
+    if (!m) {
+        TmapPair e;
+        std::memset(&e, 0, sizeof e);
+        tt_status r = encode_operand(e.a, static_cast<const float*>(q), sh.kk, sh.m, sh.batch, sh.kk, (long long)sh.m * sh.kk, true, 32, kAttnRows);
+        if (r == TT_OK) r = encode_operand(e.b, static_cast<const float*>(k), sh.kk, sh.nn, sh.batch, sh.kk, (long long)sh.nn * sh.kk, true, 32, g.n16);
+        if (r != TT_OK) return r;
+        m = keep(qk, e, q, k);
+    }
+    unsigned char maps[2][128];
+    std::memcpy(maps[0], m->a, 128); std::memcpy(maps[1], m->b, 128);
+    m = cached(pv, v, v);
+    if (!m) {
+        TmapPair e;
+        std::memset(&e, 0, sizeof e);
+        const tt_status r = encode_operand_mn(e.a, static_cast<const float*>(v), g.dv, g.n, sh.batch, g.dv, (long long)g.n * g.dv, true, g.n8);
+        if (r != TT_OK) return r;
+        m = keep(pv, e, v, v);
+    }
+    if (launch_attention(g, sh.batch, maps[0], maps[1], m->a, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+    return TT_OK;
+}
+
 tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* streams, size_t n_streams, size_t* failed_at) try {
     if (!steps || n_steps == 0 || !streams || n_streams == 0) return TT_ERR_INVALID_ARG;
-    // which layers some layer on another stream waits for
-    std::vector<cudaEvent_t> done(n_steps, nullptr);
-    std::vector<char> needed(n_steps, 0), used(n_streams, 0);
-    bool side = false;
+    constexpr size_t kNone = ~(size_t)0;
+    std::vector<ChainLaunch> plan;
+    std::vector<size_t> launch_of(n_steps), waits, first_wait, tail(n_streams, kNone);
+    std::vector<char> used(n_streams, 0);
+    plan.reserve(n_steps); waits.reserve(n_steps); first_wait.reserve(n_steps + 1);
     for (size_t i = 0; i < n_steps; ++i) {
         const tt_chain_step& s = steps[i];
         if (failed_at) *failed_at = i;
         if (s.lane < 0 || (size_t)s.lane >= n_streams || s.n_waits < 0 || (s.n_waits && !s.waits)) return TT_ERR_INVALID_ARG;
-        for (int32_t j = 0; j < s.n_waits; ++j) {
+        for (int32_t j = 0; j < s.n_waits; ++j)
             if (s.waits[j] < 0 || (size_t)s.waits[j] >= i) return TT_ERR_INVALID_ARG;
-            needed[(size_t)s.waits[j]] = 1;
-        }
-        side = side || s.lane != 0;
     }
-    // Layers of one workload share its scratch (re-packed filters, partial sums and arrival counters): on different lanes they
-    // run one after the other, in chain order
-    std::vector<int64_t> after(n_steps, -1);
-    if (side) {
+    // which layers go to the device together: the launches, on the lanes of their first layers
+    for (size_t i = 0; i < n_steps;) {
+        bool attention = false;
+        const int count = together_at(steps, n_steps, i, &attention);
+        ChainLaunch l{i, count, attention, steps[i].lane, false, false, Ahead{}};
+        for (int m = 0; m < l.count; ++m) { launch_of[i + (size_t)m] = plan.size(); l.moved = l.moved || steps[i + (size_t)m].lane != l.lane; }
+        plan.push_back(l);
+        i += (size_t)l.count;
+    }
+    // What a launch waits for: the launches of the layers its layers name, the last launch of each of its layers' lanes where that
+    // went to another one, and, where it shares scratch (re-packed filters, partial sums and arrival counters) with an earlier
+    // launch of the same workload, that one.
+    bool side = false;
+    {
         std::unordered_map<const tt_workload*, size_t> last;
-        for (size_t i = 0; i < n_steps; ++i) {
-            const tt_workload* w = steps[i].workload;
-            if (!w || w->plan.info.workspace_bytes == 0) continue;
-            const auto seen = last.find(w);
-            if (seen != last.end() && steps[seen->second].lane != steps[i].lane) {
-                after[i] = (int64_t)seen->second;
-                needed[seen->second] = 1;
+        bool lanes = false;
+        for (size_t i = 0; i < n_steps; ++i) lanes = lanes || steps[i].lane != 0;
+        for (size_t l = 0; l < plan.size(); ++l) {
+            first_wait.push_back(waits.size());
+            const auto after = [&](size_t dep) {
+                if (dep == kNone || dep == l || plan[dep].lane == plan[l].lane) return;
+                if (std::find(waits.begin() + (long)first_wait[l], waits.end(), dep) != waits.end()) return;
+                waits.push_back(dep);
+                plan[dep].needed = true;
+            };
+            for (int m = 0; m < plan[l].count && lanes; ++m) {
+                const tt_chain_step& s = steps[plan[l].first + (size_t)m];
+                for (int32_t j = 0; j < s.n_waits; ++j) after(launch_of[(size_t)s.waits[j]]);
+                after(tail[(size_t)s.lane]);
+                if (s.workload && s.workload->plan.info.workspace_bytes != 0 && !plan[l].attention) {
+                    const auto seen = last.find(s.workload);
+                    if (seen != last.end()) after(seen->second);
+                    last[s.workload] = l;
+                }
             }
-            last[w] = i;
+            for (int m = 0; m < plan[l].count; ++m) tail[(size_t)steps[plan[l].first + (size_t)m].lane] = l;
+            side = side || plan[l].lane != 0 || plan[l].moved;
+        }
+        first_wait.push_back(waits.size());
+        for (size_t k = 1; k < n_streams; ++k) if (tail[k] != kNone && plan[tail[k]].lane != (int32_t)k) plan[tail[k]].needed = true;
+    }
+    // A launch brings the weights of the launches up to three behind it into the L2 while it runs: at batch 1 a layer is over before
+    // its weights could have come from memory at anything like the memory's rate (the 12-layer encoder on 128 tokens 436 -> 430 us, two
+    // of its layers with a cold L2 82 -> 80).
+    for (size_t l = 0, next = 0; l < plan.size(); ++l) {
+        next = std::max(next, l + 1);
+        int n = 0;
+        for (unsigned bytes = 0; n < 3 && next < plan.size() && next <= l + 3; ++next) {
+            const ChainLaunch& c = plan[next];
+            const tt_chain_step& s = steps[c.first];
+            if (c.attention || !usable(s) || (s.workload->op != TT_OP_DENSE && s.workload->op != TT_OP_CONV2D) || s.workload->plan.repack) continue;
+            if (n + c.count > 3 || bytes > (24u << 20)) break;
+            for (int m = 0; m < c.count; ++m) {
+                const Range w = range_of(steps[c.first + (size_t)m], 1);
+                const size_t skip = (16 - reinterpret_cast<uintptr_t>(w.p)) & 15u;
+                if (w.bytes < skip + 16 || w.bytes > (1u << 30)) continue;
+                plan[l].ahead.p[n] = w.p + skip; plan[l].ahead.bytes[n++] = (unsigned)(w.bytes - skip) & ~15u;
+                bytes += (unsigned)w.bytes;
+            }
         }
     }
-    EventLoan events(n_steps + n_streams + 1);           // (nothing below allocates once the pass is being enqueued)
+    EventLoan events(plan.size() + 2 * n_streams + 2);   // (nothing below allocates once the pass is being enqueued)
+    std::vector<cudaEvent_t> done(plan.size(), nullptr);
     tt_status rc = TT_OK;
     cudaEvent_t start = nullptr;
     cudaStream_t main_stream = static_cast<cudaStream_t>(streams[0]);
@@ -659,30 +887,73 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
         start = events.get();
         if (!start || cudaEventRecord(start, main_stream) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     }
-    for (size_t i = 0; i < n_steps && rc == TT_OK; ++i) {
-        const tt_chain_step& s = steps[i];
-        if (failed_at) *failed_at = i;
-        cudaStream_t st = static_cast<cudaStream_t>(streams[s.lane]);
+    for (size_t l = 0; l < plan.size() && rc == TT_OK; ++l) {
+        const ChainLaunch& c = plan[l];
+        const tt_chain_step& s = steps[c.first];
+        if (failed_at) *failed_at = c.first;
+        cudaStream_t st = static_cast<cudaStream_t>(streams[c.lane]);
         cudaError_t e = cudaSuccess;
-        if (s.lane != 0 && !used[(size_t)s.lane]) e = cudaStreamWaitEvent(st, start, 0);      // the side stream forks (a capture, or the caller's ordering)
-        used[(size_t)s.lane] = 1;
-        for (int32_t j = 0; j < s.n_waits && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(st, done[(size_t)s.waits[j]], 0);
-        if (after[i] >= 0 && e == cudaSuccess) e = cudaStreamWaitEvent(st, done[(size_t)after[i]], 0);
-        if (e == cudaSuccess) rc = launch(s.workload, s.tensors, st);
-        if (e == cudaSuccess && rc == TT_OK && needed[i]) {
-            done[i] = events.get();
-            e = done[i] ? cudaEventRecord(done[i], st) : cudaErrorUnknown;
+        // a side stream forks (a capture, or the caller's ordering) where a layer of its lane is first used
+        for (int m = 0; m < c.count && e == cudaSuccess; ++m) {
+            const size_t lane = (size_t)steps[c.first + (size_t)m].lane;
+            if (lane != 0 && !used[lane]) {
+                e = cudaStreamWaitEvent(static_cast<cudaStream_t>(streams[lane]), start, 0);
+                if (e == cudaSuccess && lane != (size_t)c.lane) {
+                    // (the layer runs on another lane: behind what the caller had put on its own)
+                    cudaEvent_t in = events.get();
+                    e = in ? cudaEventRecord(in, static_cast<cudaStream_t>(streams[lane])) : cudaErrorUnknown;
+                    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, in, 0);
+                }
+            }
+            used[lane] = 1;
+        }
+        for (size_t j = first_wait[l]; j < first_wait[l + 1] && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(st, done[waits[j]], 0);
+        if (e == cudaSuccess) {
+            AttnArgs g;
+            if (c.attention && attention_at(steps, n_steps, c.first, &g)) {
+                g.ahead = c.ahead;
+                rc = launch_chain_attention(&s, g, st);
+            } else {
+                Beside b;
+                b.ahead = c.ahead;
+                for (int m = 1; m < c.count; ++m) b.more[b.n_more++] = steps[c.first + (size_t)m].tensors;
+                rc = launch_with(s.workload, s.tensors, st, b);
+            }
+        }
+        if (e == cudaSuccess && rc == TT_OK && c.needed) {
+            done[l] = events.get();
+            e = done[l] ? cudaEventRecord(done[l], st) : cudaErrorUnknown;
         }
         if (e != cudaSuccess) { cudaGetLastError(); rc = TT_ERR_CUDA; }
     }
     for (size_t l = 1; l < n_streams; ++l) {
         if (!used[l]) continue;
+        // (a layer of this lane that ran on another one: what the caller puts on the lane's stream comes behind it)
+        if (rc == TT_OK && tail[l] != kNone && plan[tail[l]].lane != (int32_t)l && cudaStreamWaitEvent(static_cast<cudaStream_t>(streams[l]), done[tail[l]], 0) != cudaSuccess) {
+            cudaGetLastError();
+            rc = TT_ERR_CUDA;
+        }
         cudaEvent_t end = events.get();
         if (!end || cudaEventRecord(end, static_cast<cudaStream_t>(streams[l])) != cudaSuccess ||
             cudaStreamWaitEvent(main_stream, end, 0) != cudaSuccess) { cudaGetLastError(); if (rc == TT_OK) rc = TT_ERR_CUDA; }
     }
     return rc;
 } TT_NO_THROW
+
+tt_status tt_chain_launches(const tt_chain_step* steps, size_t n_steps, size_t* launches) {
+    if (!steps || n_steps == 0 || !launches) return TT_ERR_INVALID_ARG;
+    *launches = 0;
+    for (size_t i = 0; i < n_steps;) {
+        const tt_chain_step& s = steps[i];
+        if (!s.workload || !s.workload->plan.applied) return TT_ERR_NOT_APPLIED;
+        for (int32_t j = 0; j < s.n_waits; ++j) if (!s.waits || s.waits[j] < 0 || (size_t)s.waits[j] >= i) return TT_ERR_INVALID_ARG;
+        bool attention = false;
+        const int count = together_at(steps, n_steps, i, &attention);
+        *launches += attention ? 1 : (size_t)s.workload->plan.info.launches;
+        i += (size_t)count;
+    }
+    return TT_OK;
+}
 
 tt_status tt_workload_set_constant_weights(tt_workload* w, int32_t on) {
     if (!w) return TT_ERR_INVALID_ARG;
@@ -1134,7 +1405,7 @@ extern "C" tt_status tt_dense_static_scratch(const void* x, const void* w, const
     if (s == TT_OK && g.b_mode == OPM_TMA)
         s = encode_operand(maps.b, g.b, g.K, g.N, g.batch, g.b_rs, g.b_bs, g.b_tma_batched != 0, g.atom_k, g.tile_n);
     if (s != TT_OK) return s;
-    if (launch_gemm(plan.info, plan.run_smem, g, maps.a, maps.b, maps.x, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+    if (launch_gemm(plan.info, plan.run_smem, g, maps.a, maps.b, maps.x, maps.x, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     if (cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     unsigned v = 0;
     if (cudaMemcpy(&v, base, 4, cudaMemcpyDeviceToHost) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }

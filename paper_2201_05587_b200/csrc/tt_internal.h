@@ -35,6 +35,10 @@ enum OperandMode : int {
                           // they lie (an MN-major tile)
 };
 
+// What a launch of a chained pass brings into the L2 for the launches behind it: weights, which nothing in front of them writes
+// (and if something did: the L2 is where memory is coherent).
+struct Ahead { const void* p[3]; unsigned bytes[3]; };      // 16-byte aligned, multiples of 16 bytes, the first ones used
+
 // Device-side arguments of the GEMM_TC kernel (plain data, passed by value).
 struct GemmArgs {
     int M, N, K, batch;
@@ -82,6 +86,11 @@ struct GemmArgs {
                                                 // writing): its first stages are requested before the wait on the kernel in front
     int two_per_sm;                             // the register-capped build, so that two CTAs share an SM
     int x3;                                     // error-compensated products: a stage holds [A][B][A lo][B lo]
+    // layers of one plan on the same activations in one launch (both operands K-major by TMA, no batch): gridDim.z = group, the
+    // further members' bias and output here, their weights' tensor maps beside the first member's
+    int group, w_member;                        // ... and which operand (1 A, 2 B) the weights are
+    const float* bias_more[2]; float* y_more[2];
+    Ahead ahead;
     // persistent kernel (record field persistent = 1)
     int persistent, cta_group;
     int total_tiles;                            // tiles_m * tiles_n * batch; tiles_m counts 128 * cta_group rows
@@ -119,6 +128,22 @@ struct ConvPmArgs {
     unsigned slab_off, slab_bytes, epi_off, idesc, tmem_cols;
 };
 
+// The attention of a chained pass in one launch (tt_attention_kernel).
+constexpr int kAttnRows = 32;                               // query rows of a CTA
+struct AttnArgs {
+    float* scores; float* probs; float* ctx;
+    unsigned* status; unsigned long long wait_ns;
+    int m, n, dv, tiles_m;                      // query rows and keys of a head, columns of its values, CTAs per head
+    int n16, n8, n_blocks;                      // keys in 16s, in 8s, in blocks of 32
+    int d_atoms, d_steps, v_boxes;              // head size in 32s and 8s, value columns in 32s
+    int scores_vec, probs_vec, ctx_vec;         // rows allow 16-byte stores
+    float scale;
+    int o_col;                                  // the context's accumulator behind the scores'
+    unsigned p_off, k_off, v_off, idesc_s, idesc_o, tmem_cols;
+    int smem_bytes;
+    Ahead ahead;
+};
+
 struct DwArgs {
     const float* x; const float* w; const float* bias; float* y;
     int N, C, H, W, R, S, P, Q, sh, sw, ph, pw, act;
@@ -151,6 +176,7 @@ struct RowArgs {
 // Host-side plan of an applied record.
 struct Plan {
     bool applied = false;
+    bool strict = false;              // the record is to run as written
     tt_apply_info info{};
     // GEMM lowering
     int gm = 0, gn = 0, gk = 0, gbatch = 1;
@@ -191,6 +217,7 @@ struct tt_workload {
     int P, Q;                    // conv output size
     tt_gemm_view view;
     tt::Plan plan;
+    tt::Plan group[2];           // the plan of two and of three layers in one launch of a chained pass (applied: there is one)
     void* workspace = nullptr;   // device: split-K partials
     int* ktab_dev = nullptr;     // device: conv2d reduction-index table of the applied record
     size_t ktab_bytes = 0;
@@ -215,6 +242,7 @@ struct tt_workload {
 namespace tt {
 // host logic (tt_host.cpp)
 tt_status legalise(const tt_workload* w, const tt_schedule_record* rec, int mode, int strict_class, Plan* plan);
+void plan_groups(tt_workload* w);                               // from the applied plan
 uint64_t class_hash(int op, const tt_shapes& s);
 size_t tensor_elems(const tt_workload* w, int which);   // 0 x, 1 w, 2 bias, 3 residual, 4 y
 // device side (launch.cu)

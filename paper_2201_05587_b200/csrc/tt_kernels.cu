@@ -417,8 +417,9 @@ enum GemmForm {
 
 template <int MIN_CTAS, int FORM, bool CLUSTER>
 __global__ void __launch_bounds__(kGemmThreads, MIN_CTAS)
-tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
-                  const __grid_constant__ CUtensorMap tmap_x, const GemmArgs g) {
+tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_constant__ CUtensorMap tmap_b0,
+                  const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_z,
+                  const __grid_constant__ GemmArgs g) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_bar[kMaxStages];
     __shared__ uint64_t empty_bar[kMaxStages];
@@ -444,7 +445,14 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     if (g.raster == 0) { tm = blockIdx.x % g.tiles_m; tn = blockIdx.x / g.tiles_m; }
     else               { tn = blockIdx.x % g.tiles_n; tm = blockIdx.x / g.tiles_n; }
     const int m0 = tm * kHwTileM, n0 = tn * g.tile_n;
-    const int split = blockIdx.y, bz = blockIdx.z;
+    // which layer of a group: the first one's weights are in their operand's slot, the others' in the image's and the last
+    const int member = FORM == kFormTma && g.group > 1 ? (int)blockIdx.z : 0;
+    const int split = blockIdx.y, bz = FORM == kFormTma && g.group > 1 ? 0 : (int)blockIdx.z;
+    const CUtensorMap* w_map = member == 1 ? &tmap_x : &tmap_z;
+    const CUtensorMap& tmap_a = FORM == kFormTma && member != 0 && g.w_member == 1 ? *w_map : tmap_a0;
+    const CUtensorMap& tmap_b = FORM == kFormTma && member != 0 && g.w_member == 2 ? *w_map : tmap_b0;
+    const float* g_bias = member == 0 ? g.bias : member == 1 ? g.bias_more[0] : g.bias_more[1];
+    float* g_y = member == 0 ? g.y : member == 1 ? g.y_more[0] : g.y_more[1];
     const int kt_begin = split * g.k_tiles_per_split;
     const int kt_end = min(g.k_tiles, kt_begin + g.k_tiles_per_split);
     const int iters = kt_end - kt_begin;
@@ -521,6 +529,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     // kernel that follows this one was allowed to start its own set-up at this kernel's entry.  (Without the launch
     // attribute both instructions do nothing.)
     // (The TMA warp waits a little later: it first requests the constant operand's first stages, see below.)
+    if (g.ahead.bytes[0] != 0u && threadIdx.x == 64) prefetch_ahead(g.ahead, blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z), gridDim.x * gridDim.y * gridDim.z);
     if (warp != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     // Warps 0 and 1 run their loops with all 32 lanes: waits, counters and descriptor arithmetic stay
@@ -723,9 +732,9 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         const int quad = warp & 3;                       // tensor-memory lane quadrant this warp may read
         const int m = m0 + quad * 32 + lane;
         // bias is fetched now so that its latency hides behind the main loop
-        if (g.bias_mode == 2 && gt < g.tile_n) s_bias[gt] = (n0 + gt < g.N) ? __ldg(g.bias + n0 + gt) : 0.f;
-        if (CLUSTER && g.bias_mode == 1 && gt < kHwTileM) s_bias[gt] = (m0 + gt < g.M) ? __ldg(g.bias + m0 + gt) : 0.f;   // for the cluster reduction
-        const float bias_row = (g.bias_mode == 1 && m < g.M) ? __ldg(g.bias + m) : 0.f;
+        if (g.bias_mode == 2 && gt < g.tile_n) s_bias[gt] = (n0 + gt < g.N) ? __ldg(g_bias + n0 + gt) : 0.f;
+        if (CLUSTER && g.bias_mode == 1 && gt < kHwTileM) s_bias[gt] = (m0 + gt < g.M) ? __ldg(g_bias + m0 + gt) : 0.f;   // for the cluster reduction
+        const float bias_row = (g.bias_mode == 1 && m < g.M) ? __ldg(g_bias + m) : 0.f;
         if (im2col) {
             // ---- conv2d: slab staging + expansion; all eight warps work on the same stage ----
             const bool on_a = g.a_mode == OPM_IM2COL;
@@ -897,7 +906,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             cr.line = 4u * (uint32_t)(cr.along_cols ? g.tile_n + 4 : kRedColPitch);   // bytes per line
             cr.slot = (uint32_t)cr.per * cr.line;                        // bytes between the bands of two consecutive splits
             cr.red = tiles_base + g.red_off;
-            cr.ybase = g.y + (long long)bz * g.y_bs;
+            cr.ybase = g_y + (long long)bz * g.y_bs;
             cr.rbase = g.residual ? g.residual + (long long)bz * g.y_bs : nullptr;
             cr.lo = g.act == TT_ACT_NONE || g.act == TT_ACT_GELU_ERF ? -INFINITY : 0.f;
             cr.hi = g.act == TT_ACT_RELU6 ? 6.f : INFINITY;
@@ -1010,7 +1019,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             if (finish) {
                 if (split_mode) __threadfence();
                 EpiArgs e;
-                e.ybase = g.y + (long long)bz * g.y_bs;
+                e.ybase = g_y + (long long)bz * g.y_bs;
                 e.rbase = g.residual ? g.residual + (long long)bz * g.y_bs : nullptr;
                 e.y_ms = g.y_ms; e.y_ns = g.y_ns; e.M = g.M;
                 e.lo = g.act == TT_ACT_NONE || g.act == TT_ACT_GELU_ERF ? -INFINITY : 0.f;
@@ -1337,6 +1346,7 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     if constexpr (CG == 2) cluster_sync_all();           // the peer's barriers exist before anything arrives on them
     tc_fence_after();
     const uint32_t tmem_base = *(volatile uint32_t*)&tmem_slot;
+    if (g.ahead.bytes[0] != 0u && threadIdx.x == 64) prefetch_ahead(g.ahead, blockIdx.x, gridDim.x);
     pdl_wait_prev();                                      // the set-up above touched no global memory
 
     auto decode = [&](int i, int& m0, int& n0, int& bz) {
@@ -2442,7 +2452,7 @@ __global__ void tt_floor_kernel() {
 // system's, plus the kernel's static part) and half of its 512 tensor-memory columns.
 static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <= 112 * 1024 && tmem_cols <= 256; }
 
-typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
+typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
 #define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>}
 static const GemmKernel kGemmKernels[2][2][5] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
 #undef TT_GEMM_FORMS
@@ -2465,15 +2475,16 @@ static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel
 }
 
 cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
-                        cudaStream_t st) {
+                        const void* tmap_z, cudaStream_t st) {
     GemmKernel kern;
     const cudaError_t e = gemm_kernel_for(g, smem_bytes, &kern);
     if (e != cudaSuccess) return e;
-    CUtensorMap ta, tb, tx;
+    CUtensorMap ta, tb, tx, tz;
     memcpy(&ta, tmap_a, sizeof ta);
     memcpy(&tb, tmap_b, sizeof tb);
     memcpy(&tx, tmap_x, sizeof tx);
-    dim3 grid(I.grid_x, I.grid_y, I.grid_z);
+    memcpy(&tz, tmap_z, sizeof tz);
+    dim3 grid(I.grid_x, I.grid_y, g.group > 1 ? g.group : I.grid_z);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = dim3(kGemmThreads, 1, 1); cfg.dynamicSmemBytes = (size_t)smem_bytes; cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -2490,7 +2501,7 @@ cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& 
         ++n_attr;
     }
     cfg.attrs = attr; cfg.numAttrs = (unsigned)n_attr;
-    return cudaLaunchKernelEx(&cfg, kern, ta, tb, tx, g);
+    return cudaLaunchKernelEx(&cfg, kern, ta, tb, tx, tz, g);
 }
 
 typedef void (*PsKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);

@@ -97,6 +97,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ void pdl_allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// CTA `cta` of `ctas` asks for its share of what the launches behind this one will read (one thread; nothing waits for it).
+__device__ __forceinline__ void prefetch_ahead(const Ahead& a, unsigned cta, unsigned ctas) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const unsigned share = ((a.bytes[i] + ctas - 1u) / ctas + 127u) & ~127u;
+        const unsigned first = cta * share;
+        if (first >= a.bytes[i]) continue;
+        const unsigned end = min(first + share, a.bytes[i]);
+#pragma unroll 1
+        for (unsigned o = first; o < end; o += 16384u)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const char*>(a.p[i]) + o), "r"(min(16384u, end - o)) : "memory");
+    }
+}
+
 // One lane of a converged warp (the same lane every time): it issues the warp's asynchronous instructions.
 __device__ __forceinline__ bool elect_one() {
     uint32_t pred;

@@ -1389,3 +1389,47 @@ def test_every_run_staged_instantiation(r, stride, rows, items):
         assert wl.status() == B.TT_OK
         np.testing.assert_array_equal(t["y"].cpu().numpy(), y)
         wl.close()
+
+
+@pytest.mark.parametrize("seq,heads,d", [(1, 2, 64), (31, 3, 64), (32, 12, 64), (33, 2, 32), (64, 1, 128), (97, 12, 64), (130, 12, 64), (192, 3, 36), (255, 12, 64), (256, 12, 64), (257, 2, 64), (129, 48, 16)])
+def test_attention_and_projections_of_a_chain(seq, heads, d):
+    """One encoder layer as a chained pass, on lanes and on one stream: the three projections run as one launch, scores, softmax and
+    context as another (up to 256 keys and 148 CTAs of 32 rows).  Every layer's output against the oracle chain, between guard bands
+    and starting as NaN; blocks of 32 rows and keys with remainders of every kind."""
+    import torch
+    specs, steps = W.bert_base_net(seq=seq, hidden=heads * d, heads=heads, ffn=2 * heads * d, layers=1)
+    arrays = W.make_chain_inputs(steps, 9, init="bert")
+    refs, depth = util.oracle_chain(steps, arrays), _tf32_depth(steps)
+    wls = [sp.workload() for sp in specs]
+    for wl in wls:
+        wl.apply(tc(tile_n=64, tile_k=64, stages=2, split_k=4, mma_m_axis=2) if wl.family() == B.TT_FAMILY_GEMM_TC else wl.default_schedule())
+        wl.set_constant_weights(True)
+    bufs, _ = W.chain_device_tensors(steps, arrays)
+    tts, guards = [], []
+    for st, b in zip(steps, bufs):
+        if st.spec is None:
+            tts.append(None)
+            continue
+        b["y"], buf = guarded_output(st.spec)
+        guards.append(buf)
+        xs, ws, _, _, _ = W.tensor_shapes(st.spec)
+        w = b["w"] if st.w_from is None else bufs[st.w_from]["y"].view(ws)
+        tts.append(B.tensors(bufs[st.x]["y"].view(xs), w, b["bias"], None, b["y"]))
+    fused = seq <= 256 and heads * ((seq + 31) // 32) <= 148
+    streams = [torch.cuda.current_stream()] + [torch.cuda.Stream() for _ in range(3)]
+    lanes = W.chain_lanes(steps, max_lanes=4)
+    for plan in (lanes, [None if pl is None else (0, ()) for pl in lanes]):
+        assert B.chain_launches(wls, steps, tts, plan) == (5 if fused else 7)
+        for st, b in zip(steps, bufs):
+            if st.spec is not None:
+                b["y"].fill_(float("nan"))
+        torch.cuda.synchronize()
+        W.run_chain(wls, steps, tts, plan, streams)
+        torch.cuda.synchronize()
+        assert all(wl.status() == B.TT_OK for wl in wls) and all(guards_intact(g) for g in guards)
+        for i, (st, b, ref, k) in enumerate(zip(steps, bufs, refs, depth)):
+            if st.spec is not None:
+                y = b["y"].cpu().numpy()
+                assert not np.isnan(y).any() and util.rel_l2(y, ref) <= max(k, 1) * util.TOL_TF32, (i, st.spec.name, util.rel_l2(y, ref))
+    for wl in wls:
+        wl.close()
