@@ -24,15 +24,14 @@
 // straight into registers (32 channels of 32 positions in flight per warp) and store 16 bytes per lane without conflicts: no
 // staging buffer, no alignment asked of the image rows.
 // Where all tiles are resident at once there is nothing to overlap with: then the slab warps help to read out, and a cluster of
-// CTAs (the record's cta_group) may share a tile's channel blocks: each leaves the blocks
-// of its accumulator that another CTA finishes in its shared memory, and every CTA adds up its blocks, in CTA order, over
-// distributed shared memory.
+// CTAs (the record's cta_group) may share a tile's channel blocks: each leaves the blocks of its accumulator that another CTA
+// finishes in scratch memory, and every CTA adds up its blocks, in CTA order, after the cluster's barrier.
 //
 // Bound by shared memory in the multiply phase: a tap moves its filters in and out (2 * 128 lines of 128 bytes), its columns
 // and its share of the slab, 500 cycles measured for 192 columns that take the tensor core 384.  The rest is the prologue
 // (launch, first slab and filters: 2 us) and the read-out of the last tile (2.3 us, all CTAs storing at once).
-// Measured, before (one tile per CTA and image, TMA-staged slab) and now: 3x3 128 -> 128 at 28 x 28, batch 32, 20.8 -> 18.4 us;
-// 3x3 512 -> 512 at 7 x 7 with residual, batch 32, 53.6 (expanded im2col) -> 25.1 us; 3x3 32 -> 248 at 56 x 56, batch 5,
+// Measured, before (one tile per CTA and image, TMA-staged slab) and now: 3x3 128 -> 128 at 28 x 28, batch 32, 20.8 -> 17.4 us;
+// 3x3 512 -> 512 at 7 x 7 with residual, batch 32, 53.6 (expanded im2col) -> 23.7 us; 3x3 32 -> 248 at 56 x 56, batch 5,
 // 16.6 -> 11.3 us.
 #include <cuda_runtime.h>
 #include <cuda.h>
@@ -373,12 +372,16 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
             }
         }
     } else {
-        // every CTA of the cluster reads out the blocks b with b % split == its rank, and leaves the others to their CTAs
+        // Every CTA of the cluster reads out the blocks b with b % split == its rank, and leaves the others to their CTAs: in scratch
+        // memory, as the registers lie, 512 contiguous bytes per four columns.  That goes through the L2.  Loads from the other CTAs' shared
+        // memory came to 10 bytes a cycle and SM (a tile of 256 columns in fours: 12300 cycles for 96 KB and the stores); this way
+        // 512 -> 512 at 7 x 7, batch 32, takes 23.7 us instead of 25.2, 208 -> 120 at 56 x 56, stride 2, 4 images, 15.4 instead of 17.6.
         int m0 = 0, n0 = 0;
         if (my_tiles > 0) decode(0, m0, n0);
         const int m_first = m0 + quad * 32;
         const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16);
         const int own = crank + mine * split, own_step = per_quad * split;       // the own blocks, dealt to the warps of a quadrant
+        const auto part_of = [&](int cta, int b) { return reinterpret_cast<float4*>(g.partial) + (((long long)(unit * split + cta) * blocks_n + b) * 4 + quad) * 256 + lane; };
         float w[32];
         float bias = 0.f;
         if (reader && my_tiles > 0) {
@@ -391,25 +394,21 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                 for (int b = mine; b < blocks_n; b += per_quad) {
                     if (b % split == crank) continue;
                     uint32_t r[32];
-                    float v[32];
                     tmem_ld32(t_row + (uint32_t)(b * 32), r);
                     tmem_wait_ld();
+                    float4* to = part_of(crank, b);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-                    // (as the registers lie, 512 contiguous bytes per four columns: lanes a row's pitch apart cost the reader 6000 cycles)
-                    const uint32_t at = base + (uint32_t)(b * 4 + quad) * kPmBlockBytes + (uint32_t)lane * 16u;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) st_shared_v4(at + (uint32_t)j * 512u, v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    for (int j = 0; j < 8; ++j)
+                        __stcg(to + j * 32, make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]), __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3])));
                 }
             }
         }
         if (!ok) *abortp = 1;
         cluster_sync_all();                              // (executed by every thread, also after a tripped wait)
         if (reader && my_tiles > 0 && ok) {
+            const uint32_t stg = base + (uint32_t)(warp - 2) * kPmBlockBytes;       // (the pipeline's shared memory is idle)
 #pragma unroll 1
             for (int b = own; b < blocks_n; b += own_step) {
-                const uint32_t stg = base + (uint32_t)(b * 4 + quad) * kPmBlockBytes;
-                const uint32_t at = stg + (uint32_t)lane * 16u;
                 uint32_t r[32];
                 float v[32];
                 tmem_ld32(t_row + (uint32_t)(b * 32), r);
@@ -422,10 +421,10 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
 #pragma unroll
                         for (int j = 0; j < 32; ++j) v[j] += __uint_as_float(r[j]);
                     } else {
-                        const uint32_t src = map_to_peer(at, (uint32_t)p);
+                        const float4* from = part_of(p, b);
                         float4 q[8];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) q[j] = ld_peer_v4(src + (uint32_t)j * 512u);
+                        for (int j = 0; j < 8; ++j) q[j] = __ldcg(from + j * 32);
 #pragma unroll
                         for (int j = 0; j < 8; ++j) { v[4 * j] += q[j].x; v[4 * j + 1] += q[j].y; v[4 * j + 2] += q[j].z; v[4 * j + 3] += q[j].w; }
                     }
@@ -434,7 +433,6 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                 if (g.residual && b + own_step < blocks_n) load_residual(w, m_first, n0, b + own_step);
             }
         }
-        cluster_sync_all();                              // nobody's shared memory is read any more
     }
     tc_fence_before();
     __syncthreads();

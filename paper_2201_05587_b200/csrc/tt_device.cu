@@ -192,6 +192,8 @@ static void forget_filters(tt_workload* w) {
 void release_device(tt_workload* w) {
     forget_filters(w);
     if (w->workspace) cudaFree(w->workspace);
+    if (w->exchange) cudaFree(w->exchange);
+    w->exchange = nullptr; w->exchange_bytes = 0;
     if (w->status_word) cudaFree(w->status_word);
     if (w->ktab_dev) cudaFree(w->ktab_dev);
     w->ktab_dev = nullptr; w->ktab_bytes = 0;
@@ -225,6 +227,12 @@ tt_status bind_device(tt_workload* w) try {
         w->workspace = nullptr; w->workspace_bytes = 0;
         if (cudaMalloc(&w->workspace, need) != cudaSuccess) { cudaGetLastError(); return TT_ERR_OOM; }
         w->workspace_bytes = need;
+    }
+    if ((size_t)w->plan.exchange_bytes > w->exchange_bytes) {
+        if (w->exchange) cudaFree(w->exchange);
+        w->exchange = nullptr; w->exchange_bytes = 0;
+        if (cudaMalloc(&w->exchange, (size_t)w->plan.exchange_bytes) != cudaSuccess) { cudaGetLastError(); return TT_ERR_OOM; }
+        w->exchange_bytes = (size_t)w->plan.exchange_bytes;
     }
     if (need > 0 && !w->plan.repack) {
         // arrival counters start at zero; each launch leaves them at zero again
@@ -361,6 +369,7 @@ static tt_status launch_tap_major(tt_workload* w, const tt_tensors* t, cudaStrea
     c.x = static_cast<const float*>(t->x); c.y = static_cast<float*>(t->y);
     c.bias = w->sh.has_bias ? static_cast<const float*>(t->bias) : nullptr;
     c.residual = w->sh.has_residual ? static_cast<const float*>(t->residual) : nullptr;
+    c.partial = static_cast<float*>(w->exchange);
     c.status = w->status_word; c.wait_ns = w->wait_ns; c.extra_tx = w->extra_tx;
     c.early_filters = w->constant_weights && !repacked_now;
     if (launch_conv_pm(p.info, c, maps->a, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }

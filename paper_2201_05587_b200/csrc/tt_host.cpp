@@ -203,14 +203,14 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     const long long tiles = (long long)tiles_m * tiles_n;
     if (tiles > 0x7fffffffLL) return TT_ERR_RESOURCE;
     // shared memory: filter stages | one or two slabs | staging blocks of the read-out (twelve warps' where all tiles are
-    // resident, a cluster's whole tile, each over the idle pipeline).  A barrier is passed for up to three taps, whose issue then
+    // resident, over the idle pipeline).  A barrier is passed for up to three taps, whose issue then
     // hides its latency; the record's stages times its taps per reduction tile say how many taps' filters are in flight.  Records
     // that ask for the same run the same, so the legal one names them in one way: reduction tiles of one tap.
     const int shift_min = ty.lo * tx.pitch + tx.lo, shift_max = std::max(0, ty.hi) * tx.pitch + std::max(0, tx.hi);
     const int lines = tn + shift_max - std::min(shift_min, 0);
     const long long slab = (long long)lines * 128;
     const long long epi = 4ll * kPmEpiBlockBytes;
-    const long long tail = split > 1 ? (long long)((tn + 31) / 32) * 4 * kPmEpiBlockBytes : 12ll * kPmEpiBlockBytes;
+    const long long tail = 12ll * kPmEpiBlockBytes;
     const int plane_taps = *std::max_element(ty.count, ty.count + 16) * *std::max_element(tx.count, tx.count + 16);   // of the largest parity class
     const int want = std::min(kMaxStages, st * tps);
     int q = plane_taps == 4 ? 2 : std::min(3, plane_taps), depth = std::max(2, (want + q - 1) / q);
@@ -239,6 +239,7 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     I.smem_bytes = (int)std::min<long long>(std::max<long long>(smem, 116 * 1024), 0x7fffffff);     // one CTA per SM
     I.tmem_cols = tmem_cols;
     I.workspace_bytes = (int64_t)M * K * 4;              // the re-packed filters
+    plan->exchange_bytes = split > 1 ? tiles * split * ((tn + 31) / 32) * 4 * 4096 : 0;      // a block per CTA, 32 columns and lane quadrant
     I.launches = 2;
     if (smem > kDynSmemLimit) return TT_ERR_RESOURCE;
     plan->swap_ab = false;

@@ -116,6 +116,7 @@ constexpr unsigned kPmEpiBlockBytes = 32 * 36 * 4;          // a staged 32 x 32 
 struct ConvPlane { signed char a, b, f0, e0; unsigned char nr, ns, r0, s0; };
 struct ConvPmArgs {
     const float* x; float* y; const float* bias; const float* residual;
+    float* partial;                             // clusters: what the CTAs leave to one another
     unsigned* status; unsigned long long wait_ns;
     unsigned extra_tx; int early_filters;
     int M, C, H, W, R, S, P, Q, images, sh, sw, act;
@@ -185,6 +186,7 @@ struct Plan {
     GemmArgs g{};
     long long partial_bytes = 0;      // counters start here inside the workspace
     int run_smem = 0;                 // one-tile GEMM: shared memory of a launch (the ring may be deeper than the record's)
+    long long exchange_bytes = 0;     // tap-major convolution by clusters: what their CTAs leave to one another (scratch beside the filters)
     bool repack = false;              // tap-major convolution: pm applies, filters are re-packed into the workspace
     ConvPmArgs pm{};
     DwArgs dw{};
@@ -222,6 +224,8 @@ struct tt_workload {
     int* ktab_dev = nullptr;     // device: conv2d reduction-index table of the applied record
     size_t ktab_bytes = 0;
     size_t workspace_bytes = 0;
+    void* exchange = nullptr;    // device: what the CTAs of a tap-major convolution's clusters leave to one another
+    size_t exchange_bytes = 0;
     unsigned* status_word = nullptr;  // device
     unsigned long long wait_ns = 1000000000ull;   // one second per wait inside a kernel, then the kernel gives up
     unsigned extra_tx = 0;            // test facility (tt_workload_test_stall)
