@@ -956,6 +956,16 @@ def test_compensated_products_come_within_fp32_accumulation_of_the_exact_result(
         assert e3 <= 2e-5 and e3 * 20 <= e0, (spec.name, kw, e0, e3)
 
 
+@pytest.mark.parametrize("rows,cols", [(60001, 33), (150003, 5), (40001, 61), (19002, 198), (20003, 1174)])
+def test_softmax_of_many_short_ragged_rows(rows, cols):
+    """Rows that come several passes at a time, and even ones in chunks of two rows; the last rows fill no whole chunk."""
+    spec = W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(1, rows, cols, scale=0.125), 1, f"softmax_{rows}x{cols}", "bert")
+    a = W.make_inputs(spec, 12)
+    ref = util.oracle_ref(spec, a)
+    for bx in (8, 32):
+        run_spec(spec, B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=bx, block_y=8, vec_width=1), a, ref, ref_elem=ref)
+
+
 @pytest.mark.parametrize("cols", [1, 2, 3, 5, 31, 33, 63, 127, 129, 197, 255, 257, 1023, 1025, 2045, 2047, 2049, 2051])
 def test_softmax_ragged_rows(cols):
     """Rows that start at every offset inside a 16-byte group, up to the longest row that stays in registers and just
