@@ -356,10 +356,38 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     if (rec->cta_group > 2) changed |= TT_CHG_FORM;       // (a cluster of the tap-major order, which is not this kernel's)
     L.persistent = persistent ? 1 : 0;
     L.cta_group = cg;
+    if (persistent && !strict) {
+        // Columns are dealt evenly over the rounds of the SMs that the record's tile needs, as long as those are few: 152 tiles of 256
+        // columns are one full round and four tiles more, 240 of 160 are two rounds of little more than half the work (2419 x 1976 over 888:
+        // 36.0 -> 30.8 us, by pairs of CTAs 24.9 -> 22.3; 2000 x 1600 over 2000 from 128 columns 41.8 -> 39.4).
+        const int per = kHwTileM * cg, step = cg == 2 || tn % 32 == 0 ? 32 : 16;
+        const long long rows = (long long)((M + per - 1) / per) * B, units = kSms / cg;
+        const long long rounds = (rows * ((N + tn - 1) / tn) + units - 1) / units, columns = rounds * units / rows;
+        if (rounds >= 2 && rounds <= 4) {
+            const int even = round_up((int)((N + columns - 1) / columns), step);
+            if (even < tn) { tn = even; changed |= TT_CHG_TILE_N; L.tile_n = tn; }
+        }
+    }
     int sk = persistent ? 1 : rec->split_k;
     if (sk > k_tiles) {
         if (strict) return TT_ERR_INVALID_SCHEDULE;
         sk = k_tiles;
+    }
+    if (!strict && !persistent && !x3 && sk >= 2 && sk <= 8 && rec->ctas_per_sm != 2) {
+        // The splits of a tile are a cluster, and a cluster keeps to one group of SMs: where the record's splits of all tiles are not
+        // resident at once, fewer of them may take fewer rounds.  36 tiles of 64 columns in fours, of which 33 are resident, take two
+        // rounds of a quarter of the reduction, in threes one round of a third (533 x 464 over 4096: 28.7 -> 20.5 us; as written in eighths 32.8;
+        // 494 tiles in fours 119 -> 53, 608 in sevens 256 -> 52).  Cycles: 8 of the reduction take 64 to
+        // issue or what the columns take, a round 3000 for its ends and 1000 for the exchange; the line is drawn at 0.85.
+        const long long tiles = (long long)((M + kHwTileM - 1) / kHwTileM) * ((N + tn - 1) / tn) * B;
+        const auto cost = [&](int n) {
+            const long long rounds = (tiles + kResidentClusters[n] - 1) / kResidentClusters[n];
+            return rounds * ((long long)((k_tiles + n - 1) / n) * (tk / 8) * std::max(64, tn) + (n > 1 ? 4000 : 3000));
+        };
+        int best = sk;
+        if (tiles > kResidentClusters[sk])
+            for (int n = sk - 1; n >= 1; --n) if (cost(n) * 20 < cost(sk) * 17 && cost(n) < cost(best)) best = n;
+        sk = best;
     }
     const int per_split = (k_tiles + sk - 1) / sk;
     sk = (k_tiles + per_split - 1) / per_split;          // every split owns at least one reduction tile

@@ -985,3 +985,27 @@ def test_tap_major_clusters_are_resident_and_worth_their_exchange(shape):
         if c * r * r <= 64:
             assert info.legal.cta_group == 1
     wl.close()
+
+
+@pytest.mark.parametrize("m,k,n,rec,tile_n,split", [
+    (2419, 888, 1976, dict(tile_n=256, tile_k=32, stages=2, persistent=1), 160, 1),                  # 152 tiles: two rounds of less
+    (2419, 888, 1976, dict(tile_n=256, tile_k=32, stages=6, persistent=1, cta_group=2), 160, 1),     # 80 pairs of CTAs
+    (1500, 512, 2000, dict(tile_n=256, tile_k=32, stages=2, persistent=1), 256, 1),                  # one round: as the record says
+    (4096, 64, 4096, dict(tile_n=64, tile_k=32, stages=2, persistent=1), 64, 1),                     # many rounds: likewise
+    (533, 4096, 464, dict(tile_n=64, tile_k=64, stages=3, split_k=4), 64, 3),                        # 40 clusters of 4, of which 33 are resident
+    (533, 4096, 464, dict(tile_n=64, tile_k=64, stages=2, split_k=8), 64, 3),
+    (128, 768, 768, dict(tile_n=64, tile_k=64, stages=3, split_k=4), 64, 4),                         # all resident
+    (128, 256, 768, dict(tile_n=16, tile_k=128, stages=1, split_k=2), 16, 2),
+])
+def test_tiles_and_splits_follow_the_rounds_of_the_sms(m, k, n, rec, tile_n, split):
+    """Columns of a persistent record are dealt evenly over its rounds, splits are as many as pay for their rounds; the legal record
+    says so, legalising it again changes nothing, and strict mode runs the record as written."""
+    wl = W._dense(m, k, n).workload()
+    r = B.make_record(B.TT_FAMILY_GEMM_TC, mma_m_axis=1, **rec)
+    st, info = wl.check(r)
+    assert st == B.TT_OK and (info.legal.tile_n, info.legal.split_k) == (tile_n, split)
+    assert bool(info.changed & B.TT_CHG_TILE_N) == (tile_n != r.tile_n) and bool(info.changed & B.TT_CHG_SPLIT_K) == (split != r.split_k)
+    _check_legal_says_what_runs(wl, [r])
+    st, info = wl.check(r, mode=B.TT_MODE_STRICT)
+    assert st == B.TT_OK and (info.legal.tile_n, info.legal.split_k) == (r.tile_n, r.split_k)
+    wl.close()
