@@ -309,7 +309,7 @@ static tt_status tensor_maps_for(tt_workload* w, const GemmArgs& g, const void* 
         st = g.epi_tma ? encode_blocks(e.r, static_cast<const float*>(r_ptr), g.N, g.M, g.batch, g.y_ms, g.y_bs, g.y_tma_batched != 0, true)
                        : encode_blocks(e.r, static_cast<const float*>(r_ptr), g.M, g.N, g.batch, g.y_ns, g.y_bs, g.y_tma_batched != 0, false);
     if (st != TT_OK) return st;
-    if (g.slab_tma) {
+    if (g.slab_tma == 1) {
         const float* img = static_cast<const float*>(g.a_mode == OPM_IM2COL ? a_ptr : b_ptr);
         if ((reinterpret_cast<uintptr_t>(img) & 15u) != 0) return TT_ERR_INVALID_ARG;   // images must be 16-byte aligned
         st = encode_image(e.x, img, g.W, g.H, g.C, g.batch, g.slab_wp, g.slab_in_rows, g.slab_box_ch);
@@ -429,6 +429,7 @@ static tt_status launch_with(tt_workload* w, const tt_tensors* t, void* stream, 
             if (g.a_mode == OPM_TMA_MN && (reinterpret_cast<uintptr_t>(a_ptr) & 15u) != 0) { g.a_mode = OPM_GATHER_ROWS; g.idesc &= ~(1u << 15); }
             if (g.b_mode == OPM_TMA_MN && (reinterpret_cast<uintptr_t>(b_ptr) & 15u) != 0) { g.b_mode = OPM_GATHER_ROWS; g.idesc &= ~(1u << 16); }
         }
+        if (g.slab_tma == 2 && (reinterpret_cast<uintptr_t>(t->x) & 15u) != 0) g.slab_tma = 0;
         // (copies: what a further member's maps add to the cache may move the first's)
         const TmapPair* maps = nullptr;
         unsigned char more[2][128];

@@ -77,7 +77,8 @@ struct GemmArgs {
     unsigned magic_wpieces, magic_in_rows, magic_rstep;
     // slab by TMA (rows 16-byte aligned, stride <= filter height): a chunk is one box [box_ch channels][in_rows][W + gap]
     // starting `gap` columns left of the image, so the hardware's zero fill writes the gaps and the rows outside
-    int slab_tma;                               // 1: chunks arrive by TMA; 0: by cp.async from the gather warps
+    int slab_tma;                               // 1: chunks arrive by TMA; 2: as one run of whole channels (images of one tile, pointwise;
+                                                // x on 16 bytes); 0: by cp.async from the gather warps
     int slab_box_ch;                            // channels per box
     unsigned slab_box_bytes;
     const int* ktab_dev;                        // per reduction index: byte offset of (c, r, s) inside the slab (absolute channel)

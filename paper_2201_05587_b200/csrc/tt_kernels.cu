@@ -488,7 +488,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
         // kernel of the stream could still be writing)
         if (a_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
         if (b_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_b) : "memory");
-        if (slab_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
+        if (slab_tma && g.slab_tma == 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
     }
     if (threadIdx.x == 0) {
         const uint32_t full_count = (any_tma ? 1u : 0u) + (any_gather ? (uint32_t)wpg : 0u);
@@ -575,10 +575,19 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
             int slab_issued = 0;
             auto issue_chunk = [&](int j) {
                 const int b = j & 1;
-                const uint32_t bar = smem_u32(&slab_full[b]);
-                mbar_expect_tx(bar, g.slab_box_bytes);
-                tma_load_4d(slab0 + (uint32_t)b * g.slab_buf_bytes, &tmap_x, bar, -g.slab_gap, ic_ih_lo,
-                            (kt_begin * g.tile_k + j * T * g.tile_k) / RS, bz);
+                const uint32_t bar = smem_u32(&slab_full[b]), dst = slab0 + (uint32_t)b * g.slab_buf_bytes;
+                const int c_first = (kt_begin * g.tile_k + j * T * g.tile_k) / RS;
+                if (g.slab_tma == 1) {
+                    mbar_expect_tx(bar, g.slab_box_bytes);
+                    tma_load_4d(dst, &tmap_x, bar, -g.slab_gap, ic_ih_lo, c_first, bz);
+                } else {
+                    // (c_first, the channels and a chunk's length are multiples of four)
+                    const bool on_a = g.a_mode == OPM_IM2COL;
+                    const float* img = (on_a ? g.a : g.b) + (long long)bz * (on_a ? g.a_bs : g.b_bs);
+                    const uint32_t bytes = 4u * (uint32_t)(min(g.slab_box_ch, g.C - c_first) * g.slab_chpitch);
+                    mbar_expect_tx(bar, bytes);
+                    bulk_load(dst, img + (long long)c_first * g.slab_chpitch, bytes, bar);
+                }
             };
             if (slab_tma) {
                 if (leader) { issue_chunk(0); if (ic_chunks > 1) issue_chunk(1); }

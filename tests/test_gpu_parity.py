@@ -1443,3 +1443,29 @@ def test_attention_and_projections_of_a_chain(seq, heads, d):
                 assert not np.isnan(y).any() and util.rel_l2(y, ref) <= max(k, 1) * util.TOL_TF32, (i, st.spec.name, util.rel_l2(y, ref))
     for wl in wls:
         wl.close()
+
+
+@pytest.mark.parametrize("spec", [
+    W._conv(64, 7, 48, 1, 1, 0, name="run_64x7x7"),
+    W._conv(132, 11, 40, 1, 1, 0, residual=True, name="run_132x11x11_res"),
+    W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(3, 20, 5, 3, 70, 1, 1, 1, 0, True, B.TT_ACT_RELU6), 1, "run_n3_5x3", "uniform"),
+    W._conv(30, 7, 16, 1, 1, 0, name="no_run_30_channels"),
+], ids=lambda s: s.name)
+def test_pointwise_images_of_one_tile(spec):
+    """A 1x1 convolution whose image is no multiple of 16 bytes and fits a tile: its channels arrive as runs of memory, in one chunk or
+    several, the last one shorter; images that do not start on 16 bytes by smaller copies."""
+    import torch
+    a = W.make_inputs(spec, 23)
+    ref = util.oracle_ref(spec, a)
+    re = elem_ref(spec, a, ref)
+    for kw in (dict(tile_n=128, tile_k=32, stages=2, mma_m_axis=1), dict(tile_n=16, tile_k=16, stages=3, mma_m_axis=2, slab_tiles=1),
+               dict(tile_n=64, tile_k=8, stages=2, split_k=3, mma_m_axis=2), dict(tile_n=32, tile_k=32, stages=2, mma_m_axis=1)):
+        run_spec(spec, tc(**kw), a, ref, ref_elem=re)
+    wl = spec.workload()
+    wl.apply(tc(tile_n=128, tile_k=32, stages=2, mma_m_axis=1))
+    t, _ = W.device_tensors(spec, a)
+    x2 = torch.empty(t["x"].numel() + 1, device="cuda")[1:].view(t["x"].shape)
+    x2.copy_(t["x"])
+    wl.run(B.tensors(x2, t["w"], t["bias"], t["residual"], t["y"]))
+    assert wl.status() == B.TT_OK and util.rel_l2(t["y"].cpu().numpy(), ref) <= util.TOL_TF32
+    wl.close()
