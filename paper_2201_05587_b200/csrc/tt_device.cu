@@ -91,6 +91,20 @@ tt_status encode_operand_mn(void* out, const float* base, int rows, int K, int b
     return r == CUDA_SUCCESS ? TT_OK : TT_ERR_CUDA;
 }
 
+// Ragged rows [rows][K] in groups of four, which are multiples of 16 bytes: box = [box_k + 4, box_rows] of the groups' lines, no swizzle.
+tt_status encode_operand_raw(void* out, const float* base, int K, int rows, int box_k, int box_rows) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return TT_ERR_CUDA;
+    cuuint64_t dims[3] = {4 * (cuuint64_t)K, (cuuint64_t)(rows / 4), 1};
+    cuuint64_t strides[2] = {16 * (cuuint64_t)K, 16 * (cuuint64_t)K * (cuuint64_t)(rows / 4)};
+    cuuint32_t box[3] = {(cuuint32_t)box_k + 4, (cuuint32_t)box_rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(reinterpret_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims,
+                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? TT_OK : TT_ERR_CUDA;
+}
+
 // A matrix [batch][rows][cols] (rows `pitch` elements apart) in 32 x 32 blocks: the read-out's stores and residual loads.
 tt_status encode_blocks(void* out, const float* base, int cols, int rows, int batch, long long pitch, long long bs, bool batched, bool swizzled) {
     EncodeTiledFn fn = encode_fn();
@@ -294,6 +308,9 @@ static tt_status tensor_maps_for(tt_workload* w, const GemmArgs& g, const void* 
         st = encode_operand(e.b, static_cast<const float*>(b_ptr), g.K, g.N, g.batch, g.b_rs, g.b_bs, g.b_tma_batched != 0,
                             g.atom_k, g.b_rows_cta);
     if (st != TT_OK) return st;
+    if (g.a_mode == OPM_RAW) st = encode_operand_raw(e.a, static_cast<const float*>(a_ptr), g.K, g.a_rows_all, g.tile_k, kHwTileM / 4);
+    if (st == TT_OK && g.b_mode == OPM_RAW) st = encode_operand_raw(e.b, static_cast<const float*>(b_ptr), g.K, g.b_rows_all, g.tile_k, g.tile_n / 4);
+    if (st != TT_OK) return st;
     if (g.a_mode == OPM_TMA_MN)
         st = encode_operand_mn(e.a, static_cast<const float*>(a_ptr), g.M, g.K, g.batch, g.a_ks, g.a_bs, g.a_tma_batched != 0,
                                g.tile_k);
@@ -429,6 +446,8 @@ static tt_status launch_with(tt_workload* w, const tt_tensors* t, void* stream, 
             if (g.a_mode == OPM_TMA_MN && (reinterpret_cast<uintptr_t>(a_ptr) & 15u) != 0) { g.a_mode = OPM_GATHER_ROWS; g.idesc &= ~(1u << 15); }
             if (g.b_mode == OPM_TMA_MN && (reinterpret_cast<uintptr_t>(b_ptr) & 15u) != 0) { g.b_mode = OPM_GATHER_ROWS; g.idesc &= ~(1u << 16); }
         }
+        if (g.a_mode == OPM_RAW && (reinterpret_cast<uintptr_t>(a_ptr) & 15u) != 0) g.a_mode = OPM_GATHER_K;
+        if (g.b_mode == OPM_RAW && (reinterpret_cast<uintptr_t>(b_ptr) & 15u) != 0) g.b_mode = OPM_GATHER_K;
         if (g.slab_tma == 2 && (reinterpret_cast<uintptr_t>(t->x) & 15u) != 0) g.slab_tma = 0;
         // (copies: what a further member's maps add to the cache may move the first's)
         const TmapPair* maps = nullptr;
@@ -1414,6 +1433,10 @@ extern "C" tt_status tt_dense_static_scratch(const void* x, const void* w, const
         s = encode_operand(maps.a, g.a, g.K, g.M, g.batch, g.a_rs, g.a_bs, g.a_tma_batched != 0, g.atom_k, kHwTileM);
     if (s == TT_OK && g.b_mode == OPM_TMA)
         s = encode_operand(maps.b, g.b, g.K, g.N, g.batch, g.b_rs, g.b_bs, g.b_tma_batched != 0, g.atom_k, g.tile_n);
+    if (g.a_mode == OPM_RAW && (reinterpret_cast<uintptr_t>(g.a) & 15u) != 0) g.a_mode = OPM_GATHER_K;
+    if (g.b_mode == OPM_RAW && (reinterpret_cast<uintptr_t>(g.b) & 15u) != 0) g.b_mode = OPM_GATHER_K;
+    if (s == TT_OK && g.a_mode == OPM_RAW) s = encode_operand_raw(maps.a, g.a, g.K, g.a_rows_all, g.tile_k, kHwTileM / 4);
+    if (s == TT_OK && g.b_mode == OPM_RAW) s = encode_operand_raw(maps.b, g.b, g.K, g.b_rows_all, g.tile_k, g.tile_n / 4);
     if (s != TT_OK) return s;
     if (launch_gemm(plan.info, plan.run_smem, g, maps.a, maps.b, maps.x, maps.x, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     if (cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }

@@ -271,7 +271,7 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     return TT_OK;
 }
 
-static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, Plan* plan) {
+static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, bool boxes, Plan* plan) {
     // nonsense is refused whatever the kernel and the reduction order
     if (rec->tile_m <= 0 || rec->tile_n <= 0 || rec->tile_k <= 0 || rec->stages <= 0 || rec->split_k <= 0 ||
         rec->raster < 0 || rec->raster > 1 || rec->mma_m_axis < 0 || rec->mma_m_axis > 2 || rec->persistent < 0 ||
@@ -578,9 +578,17 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         // a tail of gap + 4 zeros follows the last row of the last channel
         return ((chunk_channels(tiles) * chp + sl_gap + 4) * 4 + 127) / 128 * 128;
     };
+    // Operands whose rows are no 16-byte multiples: boxes of groups of four rows, beside the stages that they are realigned into
+    // (`boxes`: unless the plan has no room for them; fewer than four rows make no group).
+    const int x_rows = w->op == TT_OP_DENSE ? s.m : B * s.m, w_rows = w->op == TT_OP_DENSE ? s.nn : B * s.nn;
+    const bool ragged = boxes && w->op != TT_OP_CONV2D && (K % 4) != 0;
+    const bool x_raw = ragged && x_rows >= 4, w_raw = ragged && w_rows >= 4 && (w->op == TT_OP_DENSE || w->sh.trans_b);
+    const unsigned a_box = (swap ? w_raw : x_raw) ? (unsigned)round_up((tk + 4) * 4 * (kHwTileM / 4), 128) : 0u;
+    const unsigned b_box = (swap ? x_raw : w_raw) ? (unsigned)round_up((tk + 4) * 4 * (tn / 4), 128) : 0u;
+    const long long raw_stage = 4ll * (a_box + b_box);
     long long smem = 0;
     for (;;) {
-        const long long pipe_try = std::max<long long>((long long)st * (a_stage + b_stage) * (x3 ? 2 : 1), min_pipe);
+        const long long pipe_try = std::max<long long>((long long)st * (a_stage + b_stage) * (x3 ? 2 : 1), min_pipe) + st * raw_stage;
         long long slab_total = 0;
         bool fits = true;
         if (conv) {
@@ -602,7 +610,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         changed |= TT_CHG_STAGES;
     }
     L.stages = st;
-    const long long pipe = std::max<long long>((long long)st * (a_stage + b_stage) * (x3 ? 2 : 1), min_pipe);
+    const long long pipe = std::max<long long>((long long)st * (a_stage + b_stage) * (x3 ? 2 : 1), min_pipe) + st * raw_stage;
     if (conv) {
         if (rec->slab_tiles != 0 && sl_tiles != rec->slab_tiles) {
             if (strict) return TT_ERR_INVALID_SCHEDULE;
@@ -644,7 +652,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     // and 128 tokens: 528 us with the record's depth, 501 with this one).
     int depth = st;
     const long long run_stage = (long long)(a_stage + b_stage) * (x3 ? 2 : 1);
-    auto run_bytes = [&](int d) { return std::max<long long>(d * run_stage, min_pipe) + smem - pipe; };
+    auto run_bytes = [&](int d) { return std::max<long long>(d * run_stage, min_pipe) + d * raw_stage + smem - pipe; };
     if (L.ctas_per_sm != 2)
         while (depth < std::min(kMaxStages, per_split) && run_bytes(depth + 1) <= kDynSmemLimit) ++depth;
     const long long run_pipe = std::max<long long>(depth * run_stage, min_pipe);
@@ -661,6 +669,8 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     g.ktab_off = (unsigned)run_pipe;
     g.slab_off = (unsigned)(run_pipe + ktab);
     g.red_off = (unsigned)(run_pipe + ktab + (long long)sl_nbuf * sl_buf_bytes);
+    g.raw_off = (unsigned)(g.red_off + red_bytes); g.raw_stage_bytes = (unsigned)raw_stage; g.a_raw_box = a_box; g.b_raw_box = b_box;
+    g.a_rows_all = swap ? w_rows : x_rows; g.b_rows_all = swap ? x_rows : w_rows;
     g.slab_buf_bytes = (unsigned)sl_buf_bytes; g.slab_nbuf = sl_nbuf; g.slab_tiles = sl_tiles;
     g.slab_wp = sl_wp; g.slab_gap = sl_gap; g.slab_chpitch = sl_chpitch; g.slab_in_rows = sl_in_rows;
     g.slab_rstep = sl_rstep;
@@ -697,12 +707,12 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         else V = {OPM_IM2COL, 0, 0, (long long)s.c * hw, 1};                   // pixels x (c,r,s) gathered from NCHW
         y_is = (long long)P * Q; y_js = 1; y_bs = (long long)s.k * P * Q; bias_on = 1;
     } else if (w->op == TT_OP_DENSE) {
-        U = {k4 ? OPM_TMA : OPM_GATHER_K, K, 1, 0, 0};
-        V = {k4 ? OPM_TMA : OPM_GATHER_K, K, 1, 0, 0};
+        U = {k4 ? OPM_TMA : x_raw ? OPM_RAW : OPM_GATHER_K, K, 1, 0, 0};
+        V = {k4 ? OPM_TMA : w_raw ? OPM_RAW : OPM_GATHER_K, K, 1, 0, 0};
         y_is = s.nn; y_js = 1; y_bs = 0; bias_on = 2;
     } else {
-        U = {k4 ? OPM_TMA : OPM_GATHER_K, K, 1, (long long)s.m * K, 1};
-        if (s.trans_b) V = {k4 ? OPM_TMA : OPM_GATHER_K, K, 1, (long long)s.nn * K, 1};
+        U = {k4 ? OPM_TMA : x_raw ? OPM_RAW : OPM_GATHER_K, K, 1, (long long)s.m * K, 1};
+        if (s.trans_b) V = {k4 ? OPM_TMA : w_raw ? OPM_RAW : OPM_GATHER_K, K, 1, (long long)s.nn * K, 1};
         else V = {mn_operand ? OPM_TMA_MN : OPM_GATHER_ROWS, 1, s.nn, (long long)s.nn * K, 1};   // w[b][k][j]: rows j are contiguous
         y_is = s.nn; y_js = 1; y_bs = (long long)s.m * s.nn; bias_on = 2;
     }
@@ -738,12 +748,17 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
 // 27.5 -> 24.1, which the wider grid's share of idle SMs makes a gamble on other sizes; at 1.4-1.5 30.5 -> 50.7 and 23.4 -> 38.1.
 static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, Plan* plan) {
     const Plan fresh = *plan;
-    const tt_status s = plan_gemm(w, rec, mode, plan);
+    tt_status s = plan_gemm(w, rec, mode, true, plan);
+    if (s != TT_OK && w->op != TT_OP_CONV2D && w->sh.kk % 4 != 0) {
+        // (ragged rows and no room for their boxes: gathered value by value)
+        *plan = fresh;
+        s = plan_gemm(w, rec, mode, false, plan);
+    }
     if (s != TT_OK || !plan->g.x3 || mode == TT_MODE_STRICT) return s;
     const int changed = plan->info.changed;
     auto replan = [&](const tt_schedule_record& r, bool same_splits) {
         Plan p = fresh;
-        if (plan_gemm(w, &r, TT_MODE_LEGALISE, &p) != TT_OK || p.info.legal.stages < std::min(2, p.g.k_tiles_per_split) ||
+        if (plan_gemm(w, &r, TT_MODE_LEGALISE, true, &p) != TT_OK || p.info.legal.stages < std::min(2, p.g.k_tiles_per_split) ||
             (same_splits && p.info.legal.split_k != plan->info.legal.split_k)) return;
         const tt_schedule_record& L = p.info.legal;
         p.info.changed = changed & ~(TT_CHG_TILE_N | TT_CHG_TILE_K | TT_CHG_STAGES | TT_CHG_SPLIT_K);

@@ -32,6 +32,7 @@ enum OperandMode : int {
     OPM_GATHER_ROWS = 1,  // strided view, lanes walk rows (row stride 1): 16-byte swizzled stores
     OPM_GATHER_K = 2,     // strided view, lanes walk k (k stride 1): 4-byte swizzled stores
     OPM_IM2COL = 3,       // rows are output pixels, k = (c, r, s): expanded from a slab of NCHW input rows
+    OPM_RAW = 4,          // k contiguous, rows of any length: groups of four rows by TMA, turned into K-major rows by the warps
     OPM_TMA_MN = 5        // the row index is the contiguous one in memory: [tile_k][32 rows] boxes by TMA, multiplied as
                           // they lie (an MN-major tile)
 };
@@ -87,6 +88,9 @@ struct GemmArgs {
     int w_operand;                              // 1 / 2: operand A / B is constant (weights the caller promised nobody is
                                                 // writing): its first stages are requested before the wait on the kernel in front
     int two_per_sm;                             // the register-capped build, so that two CTAs share an SM
+    // operands of ragged rows (OPM_RAW): raw stages behind the pipeline's, A's part in front of B's, four boxes each
+    unsigned raw_off, raw_stage_bytes, a_raw_box, b_raw_box;     // (0: the operand has none)
+    int a_rows_all, b_rows_all;                 // rows of the whole tensor
     int x3;                                     // error-compensated products: a stage holds [A][B][A lo][B lo]
     // layers of one plan on the same activations in one launch (both operands K-major by TMA, no batch): gridDim.z = group, the
     // further members' bias and output here, their weights' tensor maps beside the first member's

@@ -308,6 +308,72 @@ __device__ __forceinline__ void gather_k_stage(uint32_t tile_smem, int rows, con
     }
 }
 
+// One stage of an operand of ragged rows (OPM_RAW).  Four rows of K floats are a multiple of 16 bytes, so the tensor in groups of
+// four rows is a matrix that TMA can read: row 4 l + c lies in line l from column c K on.  Its box starts at the 16-byte boundary in
+// front of that, the same distance s for every fourth row, and is one 16-byte group wider than the tile.
+// Eight lanes (fewer where the tile has fewer columns) take a row, each four neighbouring values of it: they read them one by one,
+// s floats further on than the box begins, and write them as one 16-byte group of the swizzled K-major row.  The lanes of a quarter
+// warp fill a whole 128-byte line, and rows side by side differ in s where K is odd: neither side meets a bank twice.  What a whole
+// tile does not need (the end of the rows; rows behind the last group of four, which come from memory directly) is an instantiation
+// of its own.  Bound by the instructions of eight warps beside the products: 2048 x 2048 over 1023 takes 62 us, 41 without this step,
+// 25 over 1024.  Gathered value by value from memory before, with whole tunings of a pool: 1001 x 777 over 1003 143 -> 43 us, 4000 x 3001 over
+// 2047 928 -> 384, 300 heads of 506 x 64 over 506 281 -> 133, 36 of 297 x 64 over 297 41 -> 19.
+struct RealignArgs {
+    uint32_t tile, raw, box_bytes;
+    int rows, row_first, rows_all, k0, K, tile_k, atom_k, row_bytes, swz_mask, wig, wpg;
+};
+template <bool EDGE>
+__device__ __forceinline__ void realign_rows(const RealignArgs& r, const float* __restrict__ src, int lane) {
+    const int per_row = r.atom_k >> 2, shift = r.atom_k == 32 ? 3 : (r.atom_k == 16 ? 2 : 1);          // lanes of a row
+    const int chunk = lane & (per_row - 1), ri = lane >> shift, step = 32 >> shift;       // rows at a time: 4, 8 or 16
+    const int swz_shift = r.row_bytes == 128 ? 0 : (r.row_bytes == 64 ? 1 : 2), j = ri & 3;
+    const int s = (((r.row_first + j) & 3) * r.K) & 3;
+    const uint32_t pitch = 4u * (uint32_t)(r.tile_k + 4), atom_bytes = (uint32_t)(r.rows * r.row_bytes);
+    uint32_t from0 = r.raw + (uint32_t)j * r.box_bytes + (uint32_t)(ri >> 2) * pitch + 16u * (uint32_t)chunk + 4u * (uint32_t)s, to0 = r.tile;
+#pragma unroll 1
+    for (int k = 0; k < r.tile_k; k += r.atom_k, from0 += (uint32_t)r.row_bytes, to0 += atom_bytes) {
+        constexpr int kBatch = 4;
+#pragma unroll 1
+        for (int r0 = r.wig * step; r0 < r.rows; r0 += r.wpg * step * kBatch) {
+            float v[kBatch][4];
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b) {
+                const int row0 = r0 + b * r.wpg * step;
+                if (row0 >= r.rows) break;               // (warp-uniform)
+                const uint32_t from = from0 + (uint32_t)(row0 >> 2) * pitch;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[b][e] = ld_shared_f32(from + 4u * (uint32_t)e);
+                if (EDGE) {
+                    const int row = r.row_first + row0 + ri, k_here = r.k0 + k + 4 * chunk;
+                    const bool direct = row >= (r.rows_all & ~3) && row < r.rows_all;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        // (what lies behind a row's end in its box is the next row)
+                        if (k_here + e >= r.K) v[b][e] = 0.f;
+                        else if (direct) v[b][e] = __ldg(src + (long long)row * r.K + k_here + e);
+                    }
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b) {
+                const int row = r0 + b * r.wpg * step + ri;
+                if (row >= r.rows) break;
+                st_shared_v4(to0 + (uint32_t)(row * r.row_bytes) + ((uint32_t)(chunk ^ ((row >> swz_shift) & r.swz_mask)) << 4), v[b][0], v[b][1], v[b][2], v[b][3]);
+            }
+        }
+    }
+}
+__device__ __forceinline__ void realign_stage(const RealignArgs& r, const float* __restrict__ src, int lane) {
+    if (r.k0 + r.tile_k > r.K || r.row_first + r.rows > (r.rows_all & ~3)) realign_rows<true>(r, src, lane);
+    else realign_rows<false>(r, src, lane);
+}
+// ... and the request of its four boxes (one thread).
+__device__ __forceinline__ void load_raw_boxes(uint32_t dst, const void* tmap, uint32_t bar, uint32_t box_bytes, int row_first, int K, int k0) {
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j, dst += box_bytes)
+        tma_load_3d(dst, tmap, bar, ((((row_first + j) & 3) * K) & ~3) + k0, (row_first + j) >> 2, 0);
+}
+
 __device__ __forceinline__ void gather_stage(int mode, uint32_t tile_smem, int rows, const float* __restrict__ src,
                                              long long rs, long long ks, int row0, int row_extent, int k0, int K,
                                              int tile_k, int atom_k, int row_bytes, int swz_mask, int wig, int wpg,
@@ -427,7 +493,8 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
     __shared__ uint64_t slab_full[2];     // a slab chunk has landed (TMA)
     __shared__ uint64_t slab_empty[2];    // all gather warps are done with a slab buffer
     __shared__ uint64_t red_bar;          // split-K over a cluster: the other splits' bands of this CTA's output have landed
-    __shared__ uint64_t lo_bar[kMaxStages];   // error-compensated products: the remainders of a stage's operand tiles are written
+    __shared__ uint64_t lo_bar[kMaxStages];   // error-compensated products: the remainders of a stage's operand tiles are written;
+                                              // operands of ragged rows: a stage's boxes have landed
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ int last_split_flag;
@@ -468,6 +535,9 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
     const bool a_tma = FORM == kFormTma || FORM == kFormX3 || FORM == kFormMn || g.a_mode == OPM_TMA || a_mn;
     const bool b_tma = FORM == kFormTma || FORM == kFormX3 || FORM == kFormMn || g.b_mode == OPM_TMA || b_mn;
     const bool any_tma = a_tma || b_tma, any_gather = !a_tma || !b_tma;
+    const bool a_raw = FORM == kFormGather && g.a_mode == OPM_RAW, b_raw = FORM == kFormGather && g.b_mode == OPM_RAW;
+    const bool any_raw = a_raw || b_raw;
+    const int a_row0 = bz * g.M + m0, b_row0 = (g.b_tma_batched ? bz * g.N : 0) + n0;      // OPM_RAW: the tile's first row in the whole tensor
     const bool slab_tma = im2col && g.slab_tma != 0;
     constexpr bool x3 = FORM == kFormX3;                 // error-compensated products
     // im2col geometry of this CTA: first output row of its pixels, the image row its slab starts at, slab chunks
@@ -486,8 +556,8 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
     if (threadIdx.x == 32) {
         // the tensor maps are fetched ahead of their first use (they are kernel parameters: nothing the previous
         // kernel of the stream could still be writing)
-        if (a_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
-        if (b_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_b) : "memory");
+        if (a_tma || a_raw) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
+        if (b_tma || b_raw) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_b) : "memory");
         if (slab_tma && g.slab_tma == 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
     }
     if (threadIdx.x == 0) {
@@ -498,6 +568,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
         }
         mbar_init(smem_u32(&accum_bar), 1u);
         if (x3) for (int s = 0; s < g.stages; ++s) mbar_init(smem_u32(&lo_bar[s]), (uint32_t)kGatherWarps);
+        if (any_raw) for (int s = 0; s < g.stages; ++s) mbar_init(smem_u32(&lo_bar[s]), 1u);
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&slab_full[b]), 1u);
             mbar_init(smem_u32(&slab_empty[b]), (uint32_t)kGatherWarps);
@@ -562,7 +633,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
             __syncwarp();
         }
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        if (any_tma || slab_tma) {
+        if (any_tma || slab_tma || any_raw) {
             int armed = n_pref;   // stages whose loads were issued
             uint32_t st = 0, ph = 0;
             const uint32_t full0 = smem_u32(&full_bar[0]), empty0 = smem_u32(&empty_bar[0]);
@@ -607,10 +678,18 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                         ++slab_issued;
                     }
                 }
-                if (!any_tma) continue;
+                if (!any_tma && !any_raw) continue;
                 const bool got = mbar_wait(empty_addr, ph ^ 1u, abortp, g.status, 1u, g.wait_ns);
                 if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-                if (leader) {
+                if (leader && any_raw) {
+                    // (a stage whose products are done has been realigned, too: its boxes' buffer is free)
+                    const uint32_t bar = smem_u32(&lo_bar[st]), dst = tiles_base + g.raw_off + st * g.raw_stage_bytes;
+                    const uint32_t boxes = 4u * (uint32_t)(g.tile_k + 4);
+                    mbar_expect_tx(bar, (a_raw ? boxes * (uint32_t)kHwTileM : 0u) + (b_raw ? boxes * (uint32_t)g.tile_n : 0u));
+                    if (a_raw) load_raw_boxes(dst, &tmap_a, bar, g.a_raw_box, a_row0, g.K, k0);
+                    if (b_raw) load_raw_boxes(dst + 4u * g.a_raw_box, &tmap_b, bar, g.b_raw_box, b_row0, g.K, k0);
+                }
+                if (leader && any_tma) {
                     // (test facility: split 0 may be told to expect more than arrives, see tt_workload_test_stall)
                     const bool a_here = a_tma && !(it < n_pref && g.w_operand == 1), b_here = b_tma && !(it < n_pref && g.w_operand == 2);
                     mbar_expect_tx(full_addr, (a_here ? g.a_stage_bytes : 0u) + (b_here ? g.b_stage_bytes : 0u) +
@@ -644,6 +723,9 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                     const unsigned long long t0 = global_timer_ns();
                     while (!mbar_try_wait(smem_u32(&full_bar[it % g.stages]), (uint32_t)(it / g.stages) & 1u)) {
                         if (global_timer_ns() - t0 > 2000000ull) break;
+                    }
+                    while (any_raw && !mbar_try_wait(smem_u32(&lo_bar[it % g.stages]), (uint32_t)(it / g.stages) & 1u)) {
+                        if (global_timer_ns() - t0 > 4000000ull) break;
                     }
                 }
                 for (int j = max(0, slab_issued - 2); j < slab_issued; ++j) {
@@ -861,9 +943,20 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                 if (!mbar_wait(empty0 + (uint32_t)st * 8u, ph ^ 1u, abortp, g.status, 3u, g.wait_ns)) break;
                 const uint32_t a_s = tiles_base + (uint32_t)st * stage_bytes, b_s = a_s + g.a_stage_bytes;
                 const int k0 = (kt_begin + it) * g.tile_k;
-                if (!a_tma) gather_stage(g.a_mode, a_s, kHwTileM, a_src, g.a_rs, g.a_ks, m0, g.M, k0, g.K, g.tile_k,
+                if (any_raw) {
+                    if (!mbar_wait(smem_u32(&lo_bar[st]), ph, abortp, g.status, 18u, g.wait_ns)) break;
+                    const uint32_t raw = tiles_base + g.raw_off + (uint32_t)st * g.raw_stage_bytes;
+#pragma unroll 1
+                    for (int o = 0; o < 2; ++o) {        // (one copy of the code for both operands)
+                        if (!(o == 0 ? a_raw : b_raw)) continue;
+                        const RealignArgs r{o == 0 ? a_s : b_s, o == 0 ? raw : raw + 4u * g.a_raw_box, o == 0 ? g.a_raw_box : g.b_raw_box, o == 0 ? kHwTileM : g.tile_n,
+                                            o == 0 ? a_row0 : b_row0, o == 0 ? g.a_rows_all : g.b_rows_all, k0, g.K, g.tile_k, g.atom_k, g.row_bytes, g.swz_mask, wig, wpg};
+                        realign_stage(r, o == 0 ? g.a : g.b, lane);
+                    }
+                }
+                if (!a_tma && !a_raw) gather_stage(g.a_mode, a_s, kHwTileM, a_src, g.a_rs, g.a_ks, m0, g.M, k0, g.K, g.tile_k,
                                          g.atom_k, g.row_bytes, g.swz_mask, wig, wpg, lane);
-                if (!b_tma) gather_stage(g.b_mode, b_s, g.tile_n, b_src, g.b_rs, g.b_ks, n0, g.N, k0, g.K, g.tile_k,
+                if (!b_tma && !b_raw) gather_stage(g.b_mode, b_s, g.tile_n, b_src, g.b_rs, g.b_ks, n0, g.N, k0, g.K, g.tile_k,
                                          g.atom_k, g.row_bytes, g.swz_mask, wig, wpg, lane);
                 fence_proxy_async_shared();              // generic-proxy stores -> visible to the tensor core's reads
                 __syncwarp();

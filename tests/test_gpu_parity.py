@@ -1446,6 +1446,41 @@ def test_attention_and_projections_of_a_chain(seq, heads, d):
 
 
 @pytest.mark.parametrize("spec", [
+    W._dense(130, 421, 295, act=B.TT_ACT_RELU, name="raw_dense_421"),
+    W._dense(3, 7, 6, name="raw_dense_too_few_rows"),
+    W._dense(258, 1030, 66, name="raw_dense_1030"),
+    W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(5, 131, 64, 161, False), 1, "raw_nn_161", "bert"),
+    W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(3, 37, 50, 33, True), 1, "raw_nt_33", "bert"),
+    W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(3, 70, 61, 35, False), 1, "raw_nn_61", "bert"),
+], ids=lambda s: s.name)
+def test_operands_of_ragged_rows(spec):
+    """Rows that are no 16-byte multiples, by boxes of four rows' lines: every tile depth, both accumulator axes, splits, the rows
+    behind the last whole group of four, and a NaN in one row, which stays in that row's results."""
+    import torch
+    a = W.make_inputs(spec, 17)
+    ref = util.oracle_ref(spec, a)
+    re = elem_ref(spec, a, ref)
+    for tk in (8, 16, 32, 64, 128):
+        for kw in (dict(tile_n=64, stages=2, mma_m_axis=1), dict(tile_n=16, stages=3, split_k=3, mma_m_axis=2), dict(tile_n=128, stages=1, mma_m_axis=1, ctas_per_sm=2)):
+            run_spec(spec, tc(tile_k=tk, **kw), a, ref, ref_elem=re)
+    wl = spec.workload()
+    wl.apply(tc(tile_n=64, tile_k=32, stages=2, mma_m_axis=1))
+    t, tt = W.device_tensors(spec, a)
+    bad = a["x"].shape[-2] - 2
+    t["x"][..., bad, :] = float("nan")
+    wl.run(tt)
+    y = t["y"].cpu().numpy()
+    keep = np.arange(y.shape[-2]) != bad
+    assert util.rel_l2(y[..., keep, :], ref.reshape(y.shape)[..., keep, :]) <= util.TOL_TF32
+    # an operand that does not start on 16 bytes is gathered value by value
+    x2 = torch.empty(t["x"].numel() + 1, device="cuda")[1:].view(t["x"].shape)
+    x2.copy_(torch.from_numpy(a["x"]))
+    wl.run(B.tensors(x2, t["w"], t["bias"], None, t["y"]))
+    assert wl.status() == B.TT_OK and util.rel_l2(t["y"].cpu().numpy(), ref) <= util.TOL_TF32
+    wl.close()
+
+
+@pytest.mark.parametrize("spec", [
     W._conv(64, 7, 48, 1, 1, 0, name="run_64x7x7"),
     W._conv(132, 11, 40, 1, 1, 0, residual=True, name="run_132x11x11_res"),
     W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(3, 20, 5, 3, 70, 1, 1, 1, 0, True, B.TT_ACT_RELU6), 1, "run_n3_5x3", "uniform"),
