@@ -651,10 +651,14 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     // weights at once instead of a refill of two stages per trip to memory (the 84 kernels of the 12-layer encoder at batch 1
     // and 128 tokens: 528 us with the record's depth, 501 with this one).
     int depth = st;
-    const long long run_stage = (long long)(a_stage + b_stage) * (x3 ? 2 : 1);
+    // A compensated CTA with a long reduction multiplies A and its remainders from tensor memory (the record is accounted for as if it
+    // did not, so its ring may be deeper): 512 x 4096 -> 1024 in quarters 37.2 -> 29.9 us, 2000 x 1000 -> 3000 78.4 -> 73.3, 1024 x 1024 ->
+    // 1024 22.5 -> 20.6.  The way there takes longer, which short ones do not earn back: 36 x 520 -> 280 6.7 -> 7.4, 3 x 288 -> 1648 4.8 -> 6.4.
+    const bool x3_tmem = x3 && per_split * tk >= 512 && L.ctas_per_sm != 2;
+    const long long run_stage = a_stage + b_stage + (x3_tmem ? b_stage : x3 ? (long long)a_stage + b_stage : 0);
     auto run_bytes = [&](int d) { return std::max<long long>(d * run_stage, min_pipe) + d * raw_stage + smem - pipe; };
-    if (L.ctas_per_sm != 2)
-        while (depth < std::min(kMaxStages, per_split) && run_bytes(depth + 1) <= kDynSmemLimit) ++depth;
+    const long long ring_limit = L.ctas_per_sm == 2 ? smem : kDynSmemLimit;
+    while (depth < std::min(kMaxStages, per_split) && run_bytes(depth + 1) <= ring_limit) ++depth;
     const long long run_pipe = std::max<long long>(depth * run_stage, min_pipe);
     plan->run_smem = (int)run_bytes(depth);
     GemmArgs& g = plan->g;
@@ -691,6 +695,14 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     g.cluster = cluster;
     g.two_per_sm = L.ctas_per_sm == 2;
     g.x3 = x3 ? 1 : 0;
+    if (x3_tmem) {
+        // A's buffers in tensor memory, behind the accumulator: one per stage as far as the columns go
+        const int acc = round_up(tn, 32);
+        g.x3_col = (unsigned)acc;
+        g.x3_bufs = std::min(depth, (512 - acc) / (2 * tk));
+        I.tmem_cols = std::max(32, pow2_ceil(acc + g.x3_bufs * 2 * tk));
+        g.tmem_cols = (unsigned)I.tmem_cols;
+    }
     g.b_rows_cta = tn; g.cta_group = 1;
     // Instruction descriptor, kind::tf32: D = F32 (bits 4-5 = 1), A and B = TF32 (bits 7-9, 10-12 = 2), K-major or
     // (bits 15, 16 = 1) MN-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28.

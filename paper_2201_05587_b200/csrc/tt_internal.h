@@ -91,7 +91,9 @@ struct GemmArgs {
     // operands of ragged rows (OPM_RAW): raw stages behind the pipeline's, A's part in front of B's, four boxes each
     unsigned raw_off, raw_stage_bytes, a_raw_box, b_raw_box;     // (0: the operand has none)
     int a_rows_all, b_rows_all;                 // rows of the whole tensor
-    int x3;                                     // error-compensated products: a stage holds [A][B][A lo][B lo]
+    int x3;                                     // error-compensated products: a stage holds [A][B][A lo][B lo], or
+    int x3_bufs; unsigned x3_col;               // (> 0) [A][B][B lo], A and its remainders multiplied from this many buffers of 2 * tile_k
+                                                // columns of tensor memory, from this one on
     // layers of one plan on the same activations in one launch (both operands K-major by TMA, no batch): gridDim.z = group, the
     // further members' bias and output here, their weights' tensor maps beside the first member's
     int group, w_member;                        // ... and which operand (1 A, 2 B) the weights are

@@ -477,7 +477,8 @@ enum GemmForm {
     kFormTma = 0,       // both operands K-major by TMA
     kFormMn = 1,        // both by TMA, one of them (or both) MN-major
     kFormIm2col = 2,    // one operand expanded from a slab of input rows, the other by TMA or gathered
-    kFormX3 = 4,        // both K-major by TMA, error-compensated products
+    kFormX3 = 4,        // both K-major by TMA, error-compensated products, A and its remainders multiplied from shared memory ...
+    kFormX3Tmem = 5,    // ... or from tensor memory
     kFormGather = 3     // an operand gathered from global memory (the other one any way but by expansion)
 };
 
@@ -525,21 +526,21 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
     const int iters = kt_end - kt_begin;
 
     const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    // (error-compensated products: a stage holds the two operand tiles and, behind them, their remainders)
-    const uint32_t lo_off = g.a_stage_bytes + g.b_stage_bytes;
-    const uint32_t stage_bytes = FORM == kFormX3 ? 2u * lo_off : lo_off;
+    // (error-compensated products: a stage holds the two operand tiles and, behind them, their remainders, or B's alone)
+    constexpr bool x3_tmem = FORM == kFormX3Tmem, x3 = FORM == kFormX3 || x3_tmem;
+    const uint32_t lo_off = FORM == kFormX3Tmem ? g.b_stage_bytes : g.a_stage_bytes + g.b_stage_bytes;      // from an operand to its remainders
+    const uint32_t stage_bytes = g.a_stage_bytes + g.b_stage_bytes + (x3 ? lo_off : 0u);
     // what the instantiation is made for (GemmForm); within it only the modes that its form leaves open are looked at
     constexpr bool im2col = FORM == kFormIm2col;
     constexpr bool may_mn = FORM == kFormMn || FORM == kFormGather;
     const bool a_mn = may_mn && g.a_mode == OPM_TMA_MN, b_mn = may_mn && g.b_mode == OPM_TMA_MN;
-    const bool a_tma = FORM == kFormTma || FORM == kFormX3 || FORM == kFormMn || g.a_mode == OPM_TMA || a_mn;
-    const bool b_tma = FORM == kFormTma || FORM == kFormX3 || FORM == kFormMn || g.b_mode == OPM_TMA || b_mn;
+    const bool a_tma = FORM == kFormTma || x3 || FORM == kFormMn || g.a_mode == OPM_TMA || a_mn;
+    const bool b_tma = FORM == kFormTma || x3 || FORM == kFormMn || g.b_mode == OPM_TMA || b_mn;
     const bool any_tma = a_tma || b_tma, any_gather = !a_tma || !b_tma;
     const bool a_raw = FORM == kFormGather && g.a_mode == OPM_RAW, b_raw = FORM == kFormGather && g.b_mode == OPM_RAW;
     const bool any_raw = a_raw || b_raw;
     const int a_row0 = bz * g.M + m0, b_row0 = (g.b_tma_batched ? bz * g.N : 0) + n0;      // OPM_RAW: the tile's first row in the whole tensor
     const bool slab_tma = im2col && g.slab_tma != 0;
-    constexpr bool x3 = FORM == kFormX3;                 // error-compensated products
     // im2col geometry of this CTA: first output row of its pixels, the image row its slab starts at, slab chunks
     int ic_p_first = 0, ic_ih_lo = 0, ic_chunks = 0;
     if (im2col) {
@@ -567,7 +568,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
             mbar_init(smem_u32(&empty_bar[s]), 1u);
         }
         mbar_init(smem_u32(&accum_bar), 1u);
-        if (x3) for (int s = 0; s < g.stages; ++s) mbar_init(smem_u32(&lo_bar[s]), (uint32_t)kGatherWarps);
+        if (x3) for (int s = 0; s < g.stages; ++s) mbar_init(smem_u32(&lo_bar[s]), (uint32_t)(x3_tmem ? kGatherWarps / 2 : kGatherWarps));
         if (any_raw) for (int s = 0; s < g.stages; ++s) mbar_init(smem_u32(&lo_bar[s]), 1u);
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&slab_full[b]), 1u);
@@ -761,6 +762,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
             uint32_t d_tmem = tmem_base;
             const uint32_t d_end = tmem_base + (uint32_t)(g.n_acc * g.tile_n);
             int fresh = g.n_acc;                         // accumulators not written yet
+            uint32_t x3_buf = 0;
             uint32_t a_stage = a_lo0, b_stage = b_lo0, full_addr = full0, empty_addr = empty0;
             for (int it = 0; it < iters; ++it) {
                 bool got = mbar_wait(full_addr, ph, abortp, g.status, 2u, g.wait_ns);
@@ -783,8 +785,22 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                             else issue_steps<1, 1>(tmem_base, d_hi, a0, b0, a_atom, b_atom, g.idesc, accumulate);
                         };
                         const uint32_t accumulate = it > 0 ? 1u : 0u;
-                        if (x3) {
+                        if (x3_tmem) {
                             // the two cross terms first (small), then the product of what the tensor core sees of a and b
+                            const uint32_t lo = lo_off >> 4, ta = tmem_base + g.x3_col + x3_buf * 2u * (uint32_t)g.tile_k;
+                            auto issue = [&](uint32_t a, uint32_t b, uint32_t acc) {
+#pragma unroll 1
+                                for (int at = 0; at < g.n_atoms; ++at, b += b_atom) {
+#pragma unroll 4
+                                    for (uint32_t k8 = 0; k8 < (uint32_t)k8_per_atom; ++k8, a += 8u, acc = 1u)
+                                        mma_tf32_ta(tmem_base, a, ((uint64_t)d_hi << 32) | (uint64_t)(b + 2u * k8), g.idesc, acc);
+                                }
+                            };
+                            issue(ta + (uint32_t)g.tile_k, b_lo, accumulate);
+                            issue(ta, b_lo + lo, 1u);
+                            issue(ta, b_lo, 1u);
+                            if (++x3_buf == (uint32_t)g.x3_bufs) x3_buf = 0u;
+                        } else if (x3) {
                             const uint32_t lo = lo_off >> 4;
                             issue_stage(a_lo + lo, b_lo, accumulate);
                             issue_stage(a_lo, b_lo + lo, 1u);
@@ -806,7 +822,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                         }
                         a_lo += a_next_atom; b_lo += b_next_atom;
                     }
-                    if (it + g.stages < iters) mma_commit(empty_addr);   // stage reusable once these MMAs have read it (if anything follows)
+                    if (it + (x3_tmem ? g.x3_bufs : g.stages) < iters) mma_commit(empty_addr);   // stage reusable once these MMAs have read it (if anything follows)
                 }
                 __syncwarp();
                 a_stage += stage_step; b_stage += stage_step; full_addr += 8u; empty_addr += 8u;
@@ -965,7 +981,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                 while (st >= g.stages) { st -= g.stages; ph ^= 1u; }
             }
         }
-        if (x3) {
+        if (x3 && !x3_tmem) {
             // ---- error-compensated products: once a stage's operand tiles have landed, the eight warps write, 16 bytes
             // per thread and step, what the tensor core will NOT see of every value (x minus x truncated to TF32's ten
             // mantissa bits: exact in fp32) into the second half of the stage, in the same swizzled layout ----
@@ -992,6 +1008,57 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&lo_bar[st]));
                 if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1u; }
+            }
+        }
+        if (x3_tmem) {
+            // ---- the same where a CTA's reduction is long.  B's remainders go behind the stage, A and its remainders to tensor
+            // memory, where all three products read A: that takes two thirds of A's traffic off shared memory, which bounds this form
+            // (a step of 8 with 128 columns: 384 cycles with A in shared memory, 256 this way, the products 192). ----
+            const uint32_t full0 = smem_u32(&full_bar[0]), empty0 = smem_u32(&empty_bar[0]);
+            const int row = quad * 32 + lane, half = gw >> 2, atom_shift = g.atom_k == 32 ? 5 : (g.atom_k == 16 ? 4 : 3);
+            const uint32_t swz = (uint32_t)((row >> (g.row_bytes == 128 ? 0 : (g.row_bytes == 64 ? 1 : 2))) & g.swz_mask) << 4;
+            const uint32_t line = (uint32_t)(row * g.row_bytes), atom_bytes = (uint32_t)(kHwTileM * g.row_bytes);
+            const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + g.x3_col;
+            auto lo_of = [](float x) { return x - __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); };
+            // two groups of four warps (one per lane quadrant) take alternate stages, so that one stage's way through their hands, of which
+            // most is waiting (arrival, reads, stores, fence), hides behind the other's
+            for (int it = half; it < iters; it += 2) {
+                const uint32_t st = (uint32_t)(it % g.stages), buf = (uint32_t)(it % g.x3_bufs);
+                bool ok = mbar_wait(full0 + st * 8u, (uint32_t)(it / g.stages) & 1u, abortp, g.status, 15u, g.wait_ns);
+                if (it >= g.x3_bufs) {                   // the products that read this buffer of tensor memory are done
+                    const int before = it - g.x3_bufs;
+                    ok = ok && mbar_wait(empty0 + (uint32_t)(before % g.stages) * 8u, (uint32_t)(before / g.stages) & 1u, abortp, g.status, 19u, g.wait_ns);
+                }
+                if (!__all_sync(0xffffffffu, ok)) break;
+                tc_fence_after();
+                const uint32_t hi = tiles_base + st * stage_bytes;
+                // A: a lane has one row, 8 columns at a time
+                const uint32_t t_buf = t_row + buf * 2u * (uint32_t)g.tile_k;
+#pragma unroll 2
+                for (int u = 0; u < g.tile_k >> 3; ++u) {
+                    const uint32_t at = hi + (uint32_t)((u * 8) >> atom_shift) * atom_bytes + line, in = (uint32_t)((u * 8) & (g.atom_k - 1)) * 4u;
+                    const float4 p = ld_shared_v4f(at + (in ^ swz)), q = ld_shared_v4f(at + ((in + 16u) ^ swz));
+                    const float a[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+                    const float r[8] = {lo_of(p.x), lo_of(p.y), lo_of(p.z), lo_of(p.w), lo_of(q.x), lo_of(q.y), lo_of(q.z), lo_of(q.w)};
+                    tmem_st8(t_buf + (uint32_t)u * 8u, a);
+                    tmem_st8(t_buf + (uint32_t)g.tile_k + (uint32_t)u * 8u, r);
+                }
+                constexpr uint32_t step = 16u * (uint32_t)(kGatherThreads / 2);
+                const uint32_t b = hi + g.a_stage_bytes;
+                for (uint32_t off = 16u * (uint32_t)(gt & (kGatherThreads / 2 - 1)); off < g.b_stage_bytes; off += 4u * step) {      // four reads in flight
+                    float4 v[4];
+#pragma unroll
+                    for (uint32_t j = 0; j < 4u; ++j)
+                        if (off + j * step < g.b_stage_bytes) v[j] = ld_shared_v4f(b + off + j * step);
+#pragma unroll
+                    for (uint32_t j = 0; j < 4u; ++j)
+                        if (off + j * step < g.b_stage_bytes) st_shared_v4(b + lo_off + off + j * step, lo_of(v[j].x), lo_of(v[j].y), lo_of(v[j].z), lo_of(v[j].w));
+                }
+                fence_proxy_async_shared();              // generic-proxy stores -> visible to the tensor core's reads
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&lo_bar[st]));
             }
         }
         // split-K over a cluster: everything the reduction needs that does not depend on the accumulator is worked out
@@ -2555,12 +2622,12 @@ __global__ void tt_floor_kernel() {
 static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <= 112 * 1024 && tmem_cols <= 256; }
 
 typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
-#define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>}
-static const GemmKernel kGemmKernels[2][2][5] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
+#define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>, tt_gemm_tc_kernel<CTAS, kFormX3Tmem, CL>}
+static const GemmKernel kGemmKernels[2][2][6] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
 #undef TT_GEMM_FORMS
 
 static int gemm_form(const GemmArgs& g) {
-    if (g.x3) return kFormX3;
+    if (g.x3) return g.x3_bufs > 0 ? kFormX3Tmem : kFormX3;
     if (g.a_mode == OPM_IM2COL || g.b_mode == OPM_IM2COL) return kFormIm2col;
     const bool a = g.a_mode == OPM_TMA || g.a_mode == OPM_TMA_MN, b = g.b_mode == OPM_TMA || g.b_mode == OPM_TMA_MN;
     if (!a || !b) return kFormGather;
@@ -2570,7 +2637,7 @@ static int gemm_form(const GemmArgs& g) {
 // Which instantiation a plan runs; its shared-memory limit is raised once per device.  Which build (two CTAs per SM) is the
 // record's choice (ctas_per_sm), resolved by the legaliser.
 static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel* out) {
-    static OncePerDevice raised[2][2][5];
+    static OncePerDevice raised[2][2][6];
     const int two = g.two_per_sm && gemm_two_per_sm(smem_bytes, g.tmem_cols), form = gemm_form(g), cl = g.cluster > 0;
     *out = kGemmKernels[two][cl][form];
     return raised[two][cl][form]([&] { return cudaFuncSetAttribute(*out, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
