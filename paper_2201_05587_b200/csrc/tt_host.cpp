@@ -1148,14 +1148,14 @@ tt_status legalise(const tt_workload* w, const tt_schedule_record* rec, int mode
     return TT_ERR_INVALID_ARG;
 }
 
-// Layers of one plan on the same activations may share a launch (dense, both operands K-major by TMA, reduction by a cluster or in
-// one piece).  Together they have that many times the tiles, and all of their clusters should be resident at once, which the splits
+// Layers of one plan on the same activations may share a launch (dense without skip tensor, both operands K-major by TMA,
+// reduction by a cluster or in one piece).  Together they have that many times the tiles, and all of their clusters should be resident at once, which the splits
 // of one layer may be too many for: three of 768 -> 768 on 128 rows are 36 clusters of 4 where 33 fit, and the three that are left
 // made the launch take 11 us instead of 5 (the 12-layer encoder 430 -> 380); so the splits are as many as the SMs hold clusters for.  No group where not even whole tiles fit.
 void plan_groups(tt_workload* w) {
     const Plan& p = w->plan;
     for (int i = 0; i < 2; ++i) w->group[i].applied = false;
-    if (w->op != TT_OP_DENSE || p.strict || p.g.persistent || p.g.x3 || p.info.workspace_bytes != 0 || p.g.a_mode != OPM_TMA || p.g.b_mode != OPM_TMA) return;
+    if (w->op != TT_OP_DENSE || w->sh.has_residual || p.strict || p.g.persistent || p.g.x3 || p.info.workspace_bytes != 0 || p.g.a_mode != OPM_TMA || p.g.b_mode != OPM_TMA) return;
     for (int i = 0; i < 2; ++i) {
         const int clusters = p.info.grid_x * (i + 2);
         int split = p.g.split_k;

@@ -1445,6 +1445,39 @@ def test_attention_and_projections_of_a_chain(seq, heads, d):
         wl.close()
 
 
+@pytest.mark.parametrize("residual", [False, True], ids=["plain", "skip_tensor"])
+def test_dense_layers_of_one_input_in_a_chain(residual):
+    """Three layers of one plan on one input, each with its own weights, bias and skip tensor: one launch where the kernel has that
+    form, else three; between them a layer that reads the first one's output.  Each against the layer run by itself."""
+    import types
+    import torch
+    spec = W.Spec(B.TT_OP_DENSE, B.dense_shapes(70, 192, 192, True, B.TT_ACT_RELU), 1, "chain_dense", "he")
+    spec.shapes.has_residual = residual
+    wl = spec.workload()
+    wl.apply(tc(tile_n=64, tile_k=32, stages=2, split_k=2))
+    wl.set_constant_weights(True)
+    rng = torch.Generator().manual_seed(3)
+    draw = lambda *s: torch.randn(*s, generator=rng).cuda()
+    x, out, tts = draw(70, 192), [], []
+    ops = [(draw(192, 192), draw(192), draw(70, 192) if residual else None) for _ in range(4)]
+    for i, (w, b, r) in enumerate(ops):
+        out.append(torch.full((70, 192), float("nan"), device="cuda"))
+        tts.append(B.tensors(x if i < 3 else out[0], w, b, r, out[i]))
+    node = types.SimpleNamespace(kernel=0)
+    args = ([wl], [node] * 4, tts, [(0, ())] * 4)
+    assert B.chain_launches(*args) == (4 if residual else 2)
+    B.run_chain(*args, [torch.cuda.current_stream()])
+    torch.cuda.synchronize()
+    assert wl.status() == B.TT_OK
+    got = [y.cpu().numpy() for y in out]
+    for i, (y, tt) in enumerate(zip(out, tts)):
+        y.fill_(float("nan"))
+        wl.run(tt)
+        # (a group may take other splits, whose sums round differently)
+        assert util.rel_l2(got[i], y.cpu().numpy()) <= (2e-6 if i < 3 else 4e-4), i
+    wl.close()
+
+
 @pytest.mark.parametrize("spec", [
     W._dense(130, 421, 295, act=B.TT_ACT_RELU, name="raw_dense_421"),
     W._dense(3, 7, 6, name="raw_dense_too_few_rows"),
