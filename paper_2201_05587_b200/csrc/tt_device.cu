@@ -14,7 +14,9 @@
 namespace tt {
 
 cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
-                        const void* tmap_z, cudaStream_t st);
+                        cudaStream_t st);
+cudaError_t launch_gemm_chain(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const ChainArgs& c, const void* tmap_a, const void* tmap_b,
+                              const void* tmap_x, const void* tmap_z, cudaStream_t st);
 cudaError_t launch_attention(const AttnArgs& g, int heads, const void* tmap_q, const void* tmap_k, const void* tmap_v, cudaStream_t st);
 cudaError_t launch_dw(const tt_apply_info& I, const DwArgs& dw, cudaStream_t st);
 cudaError_t plan_dw_staged(tt_apply_info& I, DwArgs& dw);
@@ -394,12 +396,20 @@ static tt_status launch_tap_major(tt_workload* w, const tt_tensors* t, cudaStrea
 }
 
 // What a launch of a chained pass does beside its own layer: further layers of the same plan on the same x (their tensors), and
-// the weights it brings into the L2 for the launches behind it.
+// the weights it brings into the L2 for the launches behind it.  chained: a launch of the pass does, and then all its dense layers
+// take the kernel that can: two builds in turn meet a cold instruction cache (12-layer encoder 380 us with one, 391 with both).
 struct Beside {
+    bool chained = false;
     const tt_tensors* more[2] = {nullptr, nullptr};
     int n_more = 0;
     Ahead ahead{};
 };
+
+// The form of the one-tile kernel that does more than its layer.
+static bool chain_form(const tt_workload* w, const Plan& p) {
+    return w->op == TT_OP_DENSE && !w->sh.has_residual && !p.g.persistent && !p.g.x3 && p.g.a_mode == OPM_TMA && p.g.b_mode == OPM_TMA && !p.g.two_per_sm &&
+           p.info.workspace_bytes == 0;
+}
 
 static tt_status launch_with(tt_workload* w, const tt_tensors* t, void* stream, const Beside& beside);
 
@@ -449,24 +459,29 @@ static tt_status launch_with(tt_workload* w, const tt_tensors* t, void* stream, 
         if (g.a_mode == OPM_RAW && (reinterpret_cast<uintptr_t>(a_ptr) & 15u) != 0) g.a_mode = OPM_GATHER_K;
         if (g.b_mode == OPM_RAW && (reinterpret_cast<uintptr_t>(b_ptr) & 15u) != 0) g.b_mode = OPM_GATHER_K;
         if (g.slab_tma == 2 && (reinterpret_cast<uintptr_t>(t->x) & 15u) != 0) g.slab_tma = 0;
-        // (copies: what a further member's maps add to the cache may move the first's)
         const TmapPair* maps = nullptr;
-        unsigned char more[2][128];
-        g.group = 1 + beside.n_more;
-        g.w_member = p.a_tensor == 1 ? 1 : 2;
-        for (int i = 0; i < beside.n_more; ++i) {
-            const tt_tensors* o = beside.more[i];
-            const tt_status s = tensor_maps_for(w, g, pick(o, p.a_tensor), pick(o, p.b_tensor), &maps);
+        if (beside.chained && chain_form(w, p)) {
+            ChainArgs c{};
+            c.group = 1 + beside.n_more;
+            c.w_member = p.a_tensor == 1 ? 1 : 2;
+            c.ahead = beside.ahead;
+            unsigned char more[2][128] = {};             // (copies: what a further member's maps add to the cache may move the others)
+            for (int i = 0; i < beside.n_more; ++i) {
+                const tt_tensors* o = beside.more[i];
+                const tt_status s = tensor_maps_for(w, g, pick(o, p.a_tensor), pick(o, p.b_tensor), &maps);
+                if (s != TT_OK) return s;
+                std::memcpy(more[i], p.a_tensor == 1 ? maps->a : maps->b, 128);
+                c.bias_more[i] = w->sh.has_bias ? static_cast<const float*>(o->bias) : nullptr;
+                c.y_more[i] = static_cast<float*>(o->y);
+            }
+            const tt_status s = tensor_maps_for(w, g, a_ptr, b_ptr, &maps);
             if (s != TT_OK) return s;
-            std::memcpy(more[i], p.a_tensor == 1 ? maps->a : maps->b, 128);
-            g.bias_more[i] = w->sh.has_bias ? static_cast<const float*>(o->bias) : nullptr;
-            g.y_more[i] = static_cast<float*>(o->y);
+            e = launch_gemm_chain(p.info, p.run_smem, g, c, maps->a, maps->b, more[0], more[1], st);
+        } else {
+            const tt_status s = tensor_maps_for(w, g, a_ptr, b_ptr, &maps);
+            if (s != TT_OK) return s;
+            e = g.persistent ? launch_gemm_ps(p.info, g, *maps, st) : launch_gemm(p.info, p.run_smem, g, maps->a, maps->b, maps->x, st);
         }
-        const tt_status s = tensor_maps_for(w, g, a_ptr, b_ptr, &maps);
-        if (s != TT_OK) return s;
-        g.ahead = beside.ahead;
-        e = g.persistent ? launch_gemm_ps(p.info, g, *maps, st)
-                         : launch_gemm(p.info, p.run_smem, g, maps->a, maps->b, beside.n_more > 0 ? more[0] : maps->x, beside.n_more > 1 ? more[1] : maps->x, st);
     } else if (w->family == TT_FAMILY_DW_SIMT) {
         DwArgs d = p.dw;
         d.x = static_cast<const float*>(t->x); d.w = static_cast<const float*>(t->w);
@@ -887,11 +902,14 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
         first_wait.push_back(waits.size());
         for (size_t k = 1; k < n_streams; ++k) if (tail[k] != kNone && plan[tail[k]].lane != (int32_t)k) plan[tail[k]].needed = true;
     }
-    // A launch brings the weights of the launches up to three behind it into the L2 while it runs: at batch 1 a layer is over before
+    // A dense or attention launch brings the weights of the launches up to three behind it into the L2 while it runs: at batch 1 a layer is over before
     // its weights could have come from memory at anything like the memory's rate (the 12-layer encoder on 128 tokens 436 -> 430 us, two
     // of its layers with a cold L2 82 -> 80).
+    bool chained = false;
     for (size_t l = 0, next = 0; l < plan.size(); ++l) {
         next = std::max(next, l + 1);
+        const tt_chain_step& from = steps[plan[l].first];
+        if (!plan[l].attention && (!usable(from) || !chain_form(from.workload, from.workload->plan))) continue;
         int n = 0;
         for (unsigned bytes = 0; n < 3 && next < plan.size() && next <= l + 3; ++next) {
             const ChainLaunch& c = plan[next];
@@ -906,6 +924,7 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
                 bytes += (unsigned)w.bytes;
             }
         }
+        chained = chained || n > 0 || plan[l].count > 1;
     }
     EventLoan events(plan.size() + 2 * n_streams + 2);   // (nothing below allocates once the pass is being enqueued)
     std::vector<cudaEvent_t> done(plan.size(), nullptr);
@@ -944,6 +963,7 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
                 rc = launch_chain_attention(&s, g, st);
             } else {
                 Beside b;
+                b.chained = chained;
                 b.ahead = c.ahead;
                 for (int m = 1; m < c.count; ++m) b.more[b.n_more++] = steps[c.first + (size_t)m].tensors;
                 rc = launch_with(s.workload, s.tensors, st, b);
@@ -1438,7 +1458,7 @@ extern "C" tt_status tt_dense_static_scratch(const void* x, const void* w, const
     if (s == TT_OK && g.a_mode == OPM_RAW) s = encode_operand_raw(maps.a, g.a, g.K, g.a_rows_all, g.tile_k, kHwTileM / 4);
     if (s == TT_OK && g.b_mode == OPM_RAW) s = encode_operand_raw(maps.b, g.b, g.K, g.b_rows_all, g.tile_k, g.tile_n / 4);
     if (s != TT_OK) return s;
-    if (launch_gemm(plan.info, plan.run_smem, g, maps.a, maps.b, maps.x, maps.x, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
+    if (launch_gemm(plan.info, plan.run_smem, g, maps.a, maps.b, maps.x, st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     if (cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }
     unsigned v = 0;
     if (cudaMemcpy(&v, base, 4, cudaMemcpyDeviceToHost) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; }

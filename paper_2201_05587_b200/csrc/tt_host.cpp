@@ -1155,7 +1155,7 @@ tt_status legalise(const tt_workload* w, const tt_schedule_record* rec, int mode
 void plan_groups(tt_workload* w) {
     const Plan& p = w->plan;
     for (int i = 0; i < 2; ++i) w->group[i].applied = false;
-    if (w->op != TT_OP_DENSE || w->sh.has_residual || p.strict || p.g.persistent || p.g.x3 || p.info.workspace_bytes != 0 || p.g.a_mode != OPM_TMA || p.g.b_mode != OPM_TMA) return;
+    if (w->op != TT_OP_DENSE || w->sh.has_residual || p.strict || p.g.persistent || p.g.x3 || p.g.two_per_sm || p.info.workspace_bytes != 0 || p.g.a_mode != OPM_TMA || p.g.b_mode != OPM_TMA) return;
     for (int i = 0; i < 2; ++i) {
         const int clusters = p.info.grid_x * (i + 2);
         int split = p.g.split_k;
@@ -1167,7 +1167,7 @@ void plan_groups(tt_workload* w) {
             tt_schedule_record rec = p.info.legal;
             rec.split_k = split;
             Plan r;
-            if (legalise(w, &rec, TT_MODE_LEGALISE, 0, &r) != TT_OK || r.info.grid_x != p.info.grid_x || r.g.atom_k != p.g.atom_k || r.info.workspace_bytes != 0) {
+            if (legalise(w, &rec, TT_MODE_LEGALISE, 0, &r) != TT_OK || r.info.grid_x != p.info.grid_x || r.g.atom_k != p.g.atom_k || r.info.workspace_bytes != 0 || r.g.two_per_sm) {
                 q.applied = false;
                 continue;
             }

@@ -94,11 +94,6 @@ struct GemmArgs {
     int x3;                                     // error-compensated products: a stage holds [A][B][A lo][B lo], or
     int x3_bufs; unsigned x3_col;               // (> 0) [A][B][B lo], A and its remainders multiplied from this many buffers of 2 * tile_k
                                                 // columns of tensor memory, from this one on
-    // layers of one plan on the same activations in one launch (both operands K-major by TMA, no batch): gridDim.z = group, the
-    // further members' bias and output here, their weights' tensor maps beside the first member's
-    int group, w_member;                        // ... and which operand (1 A, 2 B) the weights are
-    const float* bias_more[2]; float* y_more[2];
-    Ahead ahead;
     // persistent kernel (record field persistent = 1)
     int persistent, cta_group;
     int total_tiles;                            // tiles_m * tiles_n * batch; tiles_m counts 128 * cta_group rows
@@ -112,6 +107,16 @@ struct GemmArgs {
     int epi_tma;                                // outputs leave by TMA stores (contiguous along the tile's columns)
     int res_tma;                                // the residual comes in by TMA, one block ahead
     int y_tma_batched;                          // the output's tensor map has the batch as its third dimension
+};
+
+// What the one-tile kernel does beside its layer in a chained pass: layers of one plan on the same activations share a launch (both
+// operands K-major by TMA, no batch; gridDim.z = group, the further members' bias and output here, their weights' tensor maps
+// beside the first member's).  An argument of an instantiation of its own: in the one that every call takes it cost 0.1 us a launch
+// (7 x 1960 -> 104 3.77 -> 3.85 us between graph nodes, the MobileNetV2-shaped pass of 53 launches 254 -> 258).
+struct ChainArgs {
+    int group, w_member;                        // layers of the launch; which operand (1 A, 2 B) the weights are
+    const float* bias_more[2]; float* y_more[2];
+    Ahead ahead;
 };
 
 // conv2d by channel blocks and taps over a pixel-major slab (tt_conv_pm_kernel).

@@ -482,11 +482,14 @@ enum GemmForm {
     kFormGather = 3     // an operand gathered from global memory (the other one any way but by expansion)
 };
 
-template <int MIN_CTAS, int FORM, bool CLUSTER>
+// CHAIN: a launch of a chained pass that does more than its layer (ChainArgs).
+template <bool CHAIN> struct ChainParam {};
+template <> struct ChainParam<true> { CUtensorMap tmap_z; ChainArgs a; };
+
+template <int MIN_CTAS, int FORM, bool CLUSTER, bool CHAIN = false>
 __global__ void __launch_bounds__(kGemmThreads, MIN_CTAS)
 tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_constant__ CUtensorMap tmap_b0,
-                  const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_z,
-                  const __grid_constant__ GemmArgs g) {
+                  const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ GemmArgs g, const __grid_constant__ ChainParam<CHAIN> chain) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_bar[kMaxStages];
     __shared__ uint64_t empty_bar[kMaxStages];
@@ -513,14 +516,21 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
     if (g.raster == 0) { tm = blockIdx.x % g.tiles_m; tn = blockIdx.x / g.tiles_m; }
     else               { tn = blockIdx.x % g.tiles_n; tm = blockIdx.x / g.tiles_n; }
     const int m0 = tm * kHwTileM, n0 = tn * g.tile_n;
-    // which layer of a group: the first one's weights are in their operand's slot, the others' in the image's and the last
-    const int member = FORM == kFormTma && g.group > 1 ? (int)blockIdx.z : 0;
-    const int split = blockIdx.y, bz = FORM == kFormTma && g.group > 1 ? 0 : (int)blockIdx.z;
-    const CUtensorMap* w_map = member == 1 ? &tmap_x : &tmap_z;
-    const CUtensorMap& tmap_a = FORM == kFormTma && member != 0 && g.w_member == 1 ? *w_map : tmap_a0;
-    const CUtensorMap& tmap_b = FORM == kFormTma && member != 0 && g.w_member == 2 ? *w_map : tmap_b0;
-    const float* g_bias = member == 0 ? g.bias : member == 1 ? g.bias_more[0] : g.bias_more[1];
-    float* g_y = member == 0 ? g.y : member == 1 ? g.y_more[0] : g.y_more[1];
+    const int split = blockIdx.y, bz = CHAIN ? 0 : (int)blockIdx.z;
+    // CHAIN: which layer of a group (a dense layer has no batch).  The first one's weights are in their operand's slot, the others' in
+    // the image's and the last; what only they need is only read by them.
+    const CUtensorMap *map_a = &tmap_a0, *map_b = &tmap_b0;
+    const float* g_bias = g.bias;
+    float* g_y = g.y;
+    if constexpr (CHAIN) {
+        if (blockIdx.z != 0u) {
+            const CUtensorMap* w_map = blockIdx.z == 1u ? &tmap_x : &chain.tmap_z;
+            if (chain.a.w_member == 1) map_a = w_map; else map_b = w_map;
+            g_bias = blockIdx.z == 1u ? chain.a.bias_more[0] : chain.a.bias_more[1];
+            g_y = blockIdx.z == 1u ? chain.a.y_more[0] : chain.a.y_more[1];
+        }
+    }
+    const CUtensorMap &tmap_a = *map_a, &tmap_b = *map_b;
     const int kt_begin = split * g.k_tiles_per_split;
     const int kt_end = min(g.k_tiles, kt_begin + g.k_tiles_per_split);
     const int iters = kt_end - kt_begin;
@@ -601,7 +611,9 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
     // kernel that follows this one was allowed to start its own set-up at this kernel's entry.  (Without the launch
     // attribute both instructions do nothing.)
     // (The TMA warp waits a little later: it first requests the constant operand's first stages, see below.)
-    if (g.ahead.bytes[0] != 0u && threadIdx.x == 64) prefetch_ahead(g.ahead, blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z), gridDim.x * gridDim.y * gridDim.z);
+    if constexpr (CHAIN) {
+        if (threadIdx.x == 64) prefetch_ahead(chain.a.ahead, blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z), gridDim.x * gridDim.y * gridDim.z);
+    }
     if (warp != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     // Warps 0 and 1 run their loops with all 32 lanes: waits, counters and descriptor arithmetic stay
@@ -1076,7 +1088,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
             cr.slot = (uint32_t)cr.per * cr.line;                        // bytes between the bands of two consecutive splits
             cr.red = tiles_base + g.red_off;
             cr.ybase = g_y + (long long)bz * g.y_bs;
-            cr.rbase = g.residual ? g.residual + (long long)bz * g.y_bs : nullptr;
+            cr.rbase = !CHAIN && g.residual ? g.residual + (long long)bz * g.y_bs : nullptr;      // (chained dense layers with a skip tensor take the other kernel)
             cr.lo = g.act == TT_ACT_NONE || g.act == TT_ACT_GELU_ERF ? -INFINITY : 0.f;
             cr.hi = g.act == TT_ACT_RELU6 ? 6.f : INFINITY;
             cr.gelu = g.act == TT_ACT_GELU_ERF; cr.clamp = g.act == TT_ACT_RELU || g.act == TT_ACT_RELU6;
@@ -1086,7 +1098,8 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                         (cr.rbase == nullptr || (reinterpret_cast<uintptr_t>(cr.rbase) & 15u) == 0);
             if constexpr (MIN_CTAS == 1) {               // (kept in registers; the register-capped build works them out again)
                 int pin = cr.per;
-                asm volatile("" : "+r"(pin), "+r"(cr.slot), "+r"(cr.red), "+l"(cr.ybase), "+l"(cr.rbase), "+l"(cr.y_ms), "+l"(cr.y_ns));
+                asm volatile("" : "+r"(pin), "+r"(cr.slot), "+r"(cr.red), "+l"(cr.ybase), "+l"(cr.y_ms), "+l"(cr.y_ns));
+                if constexpr (!CHAIN) asm volatile("" : "+l"(cr.rbase));
                 cr.per = pin;
             }
         }
@@ -1189,7 +1202,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                 if (split_mode) __threadfence();
                 EpiArgs e;
                 e.ybase = g_y + (long long)bz * g.y_bs;
-                e.rbase = g.residual ? g.residual + (long long)bz * g.y_bs : nullptr;
+                e.rbase = !CHAIN && g.residual ? g.residual + (long long)bz * g.y_bs : nullptr;
                 e.y_ms = g.y_ms; e.y_ns = g.y_ns; e.M = g.M;
                 e.lo = g.act == TT_ACT_NONE || g.act == TT_ACT_GELU_ERF ? -INFINITY : 0.f;
                 e.hi = g.act == TT_ACT_RELU6 ? 6.f : INFINITY;
@@ -1515,7 +1528,6 @@ tt_gemm_ps_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     if constexpr (CG == 2) cluster_sync_all();           // the peer's barriers exist before anything arrives on them
     tc_fence_after();
     const uint32_t tmem_base = *(volatile uint32_t*)&tmem_slot;
-    if (g.ahead.bytes[0] != 0u && threadIdx.x == 64) prefetch_ahead(g.ahead, blockIdx.x, gridDim.x);
     pdl_wait_prev();                                      // the set-up above touched no global memory
 
     auto decode = [&](int i, int& m0, int& n0, int& bz) {
@@ -2621,7 +2633,7 @@ __global__ void tt_floor_kernel() {
 // system's, plus the kernel's static part) and half of its 512 tensor-memory columns.
 static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <= 112 * 1024 && tmem_cols <= 256; }
 
-typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
+typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs, const ChainParam<false>);
 #define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>, tt_gemm_tc_kernel<CTAS, kFormX3Tmem, CL>}
 static const GemmKernel kGemmKernels[2][2][6] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
 #undef TT_GEMM_FORMS
@@ -2643,17 +2655,16 @@ static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel
     return raised[two][cl][form]([&] { return cudaFuncSetAttribute(*out, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
 }
 
-cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
-                        const void* tmap_z, cudaStream_t st) {
-    GemmKernel kern;
-    const cudaError_t e = gemm_kernel_for(g, smem_bytes, &kern);
-    if (e != cudaSuccess) return e;
-    CUtensorMap ta, tb, tx, tz;
+// A launch of the one-tile form, `layers` of them along grid.z where that is more than the plan's batch.
+template <bool CHAIN>
+static cudaError_t launch_one_tile(void (*kern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs, const ChainParam<CHAIN>),
+                                   const tt_apply_info& I, int smem_bytes, int layers, const GemmArgs& g, const ChainParam<CHAIN>& chain,
+                                   const void* tmap_a, const void* tmap_b, const void* tmap_x, cudaStream_t st) {
+    CUtensorMap ta, tb, tx;
     memcpy(&ta, tmap_a, sizeof ta);
     memcpy(&tb, tmap_b, sizeof tb);
     memcpy(&tx, tmap_x, sizeof tx);
-    memcpy(&tz, tmap_z, sizeof tz);
-    dim3 grid(I.grid_x, I.grid_y, g.group > 1 ? g.group : I.grid_z);
+    dim3 grid(I.grid_x, I.grid_y, layers > 1 ? layers : I.grid_z);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = dim3(kGemmThreads, 1, 1); cfg.dynamicSmemBytes = (size_t)smem_bytes; cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -2670,7 +2681,32 @@ cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& 
         ++n_attr;
     }
     cfg.attrs = attr; cfg.numAttrs = (unsigned)n_attr;
-    return cudaLaunchKernelEx(&cfg, kern, ta, tb, tx, tz, g);
+    return cudaLaunchKernelEx(&cfg, kern, ta, tb, tx, g, chain);
+}
+
+cudaError_t launch_gemm(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const void* tmap_a, const void* tmap_b, const void* tmap_x,
+                        cudaStream_t st) {
+    GemmKernel kern;
+    const cudaError_t e = gemm_kernel_for(g, smem_bytes, &kern);
+    if (e != cudaSuccess) return e;
+    return launch_one_tile<false>(kern, I, smem_bytes, 1, g, ChainParam<false>{}, tmap_a, tmap_b, tmap_x, st);
+}
+
+// The same with what a chained pass adds (both operands K-major by TMA, one CTA per SM).  tmap_x, tmap_z: the weights of a group's
+// second and third layer.
+cudaError_t launch_gemm_chain(const tt_apply_info& I, int smem_bytes, const GemmArgs& g, const ChainArgs& c, const void* tmap_a, const void* tmap_b,
+                              const void* tmap_x, const void* tmap_z, cudaStream_t st) {
+    static OncePerDevice raised;
+    const auto alone = tt_gemm_tc_kernel<1, kFormTma, false, true>, cluster = tt_gemm_tc_kernel<1, kFormTma, true, true>;
+    const cudaError_t ready = raised([&] {
+        const cudaError_t e = cudaFuncSetAttribute(alone, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+    });
+    if (ready != cudaSuccess) return ready;
+    ChainParam<true> p;
+    memcpy(&p.tmap_z, tmap_z, sizeof p.tmap_z);
+    p.a = c;
+    return launch_one_tile<true>(g.cluster ? cluster : alone, I, smem_bytes, c.group, g, p, tmap_a, tmap_b, tmap_x, st);
 }
 
 typedef void (*PsKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);

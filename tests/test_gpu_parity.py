@@ -1445,8 +1445,8 @@ def test_attention_and_projections_of_a_chain(seq, heads, d):
         wl.close()
 
 
-@pytest.mark.parametrize("residual", [False, True], ids=["plain", "skip_tensor"])
-def test_dense_layers_of_one_input_in_a_chain(residual):
+@pytest.mark.parametrize("residual,per_sm", [(False, 1), (True, 1), (False, 2)], ids=["plain", "skip_tensor", "two_per_sm"])
+def test_dense_layers_of_one_input_in_a_chain(residual, per_sm):
     """Three layers of one plan on one input, each with its own weights, bias and skip tensor: one launch where the kernel has that
     form, else three; between them a layer that reads the first one's output.  Each against the layer run by itself."""
     import types
@@ -1454,7 +1454,7 @@ def test_dense_layers_of_one_input_in_a_chain(residual):
     spec = W.Spec(B.TT_OP_DENSE, B.dense_shapes(70, 192, 192, True, B.TT_ACT_RELU), 1, "chain_dense", "he")
     spec.shapes.has_residual = residual
     wl = spec.workload()
-    wl.apply(tc(tile_n=64, tile_k=32, stages=2, split_k=2))
+    wl.apply(tc(tile_n=64, tile_k=32, stages=2, split_k=2, ctas_per_sm=per_sm))
     wl.set_constant_weights(True)
     rng = torch.Generator().manual_seed(3)
     draw = lambda *s: torch.randn(*s, generator=rng).cuda()
@@ -1465,7 +1465,7 @@ def test_dense_layers_of_one_input_in_a_chain(residual):
         tts.append(B.tensors(x if i < 3 else out[0], w, b, r, out[i]))
     node = types.SimpleNamespace(kernel=0)
     args = ([wl], [node] * 4, tts, [(0, ())] * 4)
-    assert B.chain_launches(*args) == (4 if residual else 2)
+    assert B.chain_launches(*args) == (4 if residual or per_sm == 2 else 2)
     B.run_chain(*args, [torch.cuda.current_stream()])
     torch.cuda.synchronize()
     assert wl.status() == B.TT_OK
