@@ -382,14 +382,17 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
         const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16);
         const int own = crank + mine * split, own_step = per_quad * split;       // the own blocks, dealt to the warps of a quadrant
         const auto part_of = [&](int cta, int b) { return reinterpret_cast<float4*>(g.partial) + (((long long)(unit * split + cta) * blocks_n + b) * 4 + quad) * 256 + lane; };
+        // A quadrant whose 32 filters are all beyond the layer's has nothing to pass on, and no traffic to slow the others with: 480 -> 24 at
+        // 7 x 7, 12 images, 12.0 -> 11.1 us, 256 -> 40 at 14 x 14, 16 images, 11.4 -> 10.9.
+        const bool sums = reader && my_tiles > 0 && m_first < g.M;
         float w[32];
         float bias = 0.f;
         if (reader && my_tiles > 0) {
             bias = g.bias && m_first + lane < g.M ? __ldg(g.bias + m_first + lane) : 0.f;
-            if (g.residual && own < blocks_n) load_residual(w, m_first, n0, own);
+            if (g.residual && sums && own < blocks_n) load_residual(w, m_first, n0, own);
             ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full[0]), 0u, abortp, g.status, 4u, g.wait_ns));
-            if (ok) {
-                tc_fence_after();
+            if (ok) tc_fence_after();
+            if (ok && sums) {
 #pragma unroll 1
                 for (int b = mine; b < blocks_n; b += per_quad) {
                     if (b % split == crank) continue;
@@ -405,7 +408,7 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
         }
         if (!ok) *abortp = 1;
         cluster_sync_all();                              // (executed by every thread, also after a tripped wait)
-        if (reader && my_tiles > 0 && ok) {
+        if (sums && ok) {
             const uint32_t stg = base + (uint32_t)(warp - 2) * kPmBlockBytes;       // (the pipeline's shared memory is idle)
 #pragma unroll 1
             for (int b = own; b < blocks_n; b += own_step) {
@@ -429,7 +432,7 @@ tt_conv_pm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                         for (int j = 0; j < 8; ++j) { v[4 * j] += q[j].x; v[4 * j + 1] += q[j].y; v[4 * j + 2] += q[j].z; v[4 * j + 3] += q[j].w; }
                     }
                 }
-                if (m_first < g.M) finish_block(v, w, m_first, n0, b, bias, stg);
+                finish_block(v, w, m_first, n0, b, bias, stg);
                 if (g.residual && b + own_step < blocks_n) load_residual(w, m_first, n0, b + own_step);
             }
         }
