@@ -477,6 +477,9 @@ enum GemmForm {
     kFormTma = 0,       // both operands K-major by TMA
     kFormMn = 1,        // both by TMA, one of them (or both) MN-major
     kFormIm2col = 2,    // one operand expanded from a slab of input rows, the other by TMA or gathered
+    kFormIm2colRun = 6, // the same where the slab's channels are one run of memory: in the form above that copy cost every convolution 0.3 us
+                        // (3x3 over 344 x 7 x 7 -> 32 9.02 us between graph nodes, 9.37 with it), more than two builds in turn do (the 53 layers of the
+                        // MobileNetV2-shaped pass 256.5 us, 254.9 with one build)
     kFormX3 = 4,        // both K-major by TMA, error-compensated products, A and its remainders multiplied from shared memory ...
     kFormX3Tmem = 5,    // ... or from tensor memory
     kFormGather = 3     // an operand gathered from global memory (the other one any way but by expansion)
@@ -541,7 +544,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
     const uint32_t lo_off = FORM == kFormX3Tmem ? g.b_stage_bytes : g.a_stage_bytes + g.b_stage_bytes;      // from an operand to its remainders
     const uint32_t stage_bytes = g.a_stage_bytes + g.b_stage_bytes + (x3 ? lo_off : 0u);
     // what the instantiation is made for (GemmForm); within it only the modes that its form leaves open are looked at
-    constexpr bool im2col = FORM == kFormIm2col;
+    constexpr bool slab_run = FORM == kFormIm2colRun, im2col = FORM == kFormIm2col || slab_run;
     constexpr bool may_mn = FORM == kFormMn || FORM == kFormGather;
     const bool a_mn = may_mn && g.a_mode == OPM_TMA_MN, b_mn = may_mn && g.b_mode == OPM_TMA_MN;
     const bool a_tma = FORM == kFormTma || x3 || FORM == kFormMn || g.a_mode == OPM_TMA || a_mn;
@@ -550,7 +553,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
     const bool a_raw = FORM == kFormGather && g.a_mode == OPM_RAW, b_raw = FORM == kFormGather && g.b_mode == OPM_RAW;
     const bool any_raw = a_raw || b_raw;
     const int a_row0 = bz * g.M + m0, b_row0 = (g.b_tma_batched ? bz * g.N : 0) + n0;      // OPM_RAW: the tile's first row in the whole tensor
-    const bool slab_tma = im2col && g.slab_tma != 0;
+    const bool slab_tma = slab_run || (im2col && g.slab_tma != 0);
     // im2col geometry of this CTA: first output row of its pixels, the image row its slab starts at, slab chunks
     int ic_p_first = 0, ic_ih_lo = 0, ic_chunks = 0;
     if (im2col) {
@@ -569,7 +572,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
         // kernel of the stream could still be writing)
         if (a_tma || a_raw) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_a) : "memory");
         if (b_tma || b_raw) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_b) : "memory");
-        if (slab_tma && g.slab_tma == 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
+        if (slab_tma && !slab_run) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
     }
     if (threadIdx.x == 0) {
         const uint32_t full_count = (any_tma ? 1u : 0u) + (any_gather ? (uint32_t)wpg : 0u);
@@ -661,7 +664,7 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
                 const int b = j & 1;
                 const uint32_t bar = smem_u32(&slab_full[b]), dst = slab0 + (uint32_t)b * g.slab_buf_bytes;
                 const int c_first = (kt_begin * g.tile_k + j * T * g.tile_k) / RS;
-                if (g.slab_tma == 1) {
+                if (!slab_run) {
                     mbar_expect_tx(bar, g.slab_box_bytes);
                     tma_load_4d(dst, &tmap_x, bar, -g.slab_gap, ic_ih_lo, c_first, bz);
                 } else {
@@ -2634,13 +2637,14 @@ __global__ void tt_floor_kernel() {
 static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <= 112 * 1024 && tmem_cols <= 256; }
 
 typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs, const ChainParam<false>);
-#define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>, tt_gemm_tc_kernel<CTAS, kFormX3Tmem, CL>}
-static const GemmKernel kGemmKernels[2][2][6] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
+#define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>, tt_gemm_tc_kernel<CTAS, kFormX3Tmem, CL>, \
+    tt_gemm_tc_kernel<CTAS, kFormIm2colRun, CL>}
+static const GemmKernel kGemmKernels[2][2][7] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
 #undef TT_GEMM_FORMS
 
 static int gemm_form(const GemmArgs& g) {
     if (g.x3) return g.x3_bufs > 0 ? kFormX3Tmem : kFormX3;
-    if (g.a_mode == OPM_IM2COL || g.b_mode == OPM_IM2COL) return kFormIm2col;
+    if (g.a_mode == OPM_IM2COL || g.b_mode == OPM_IM2COL) return g.slab_tma == 2 ? kFormIm2colRun : kFormIm2col;
     const bool a = g.a_mode == OPM_TMA || g.a_mode == OPM_TMA_MN, b = g.b_mode == OPM_TMA || g.b_mode == OPM_TMA_MN;
     if (!a || !b) return kFormGather;
     return g.a_mode == OPM_TMA && g.b_mode == OPM_TMA ? kFormTma : kFormMn;
@@ -2649,7 +2653,7 @@ static int gemm_form(const GemmArgs& g) {
 // Which instantiation a plan runs; its shared-memory limit is raised once per device.  Which build (two CTAs per SM) is the
 // record's choice (ctas_per_sm), resolved by the legaliser.
 static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel* out) {
-    static OncePerDevice raised[2][2][6];
+    static OncePerDevice raised[2][2][7];
     const int two = g.two_per_sm && gemm_two_per_sm(smem_bytes, g.tmem_cols), form = gemm_form(g), cl = g.cluster > 0;
     *out = kGemmKernels[two][cl][form];
     return raised[two][cl][form]([&] { return cudaFuncSetAttribute(*out, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
