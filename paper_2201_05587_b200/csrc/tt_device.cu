@@ -287,7 +287,7 @@ tt_status bind_device(tt_workload* w) try {
     return TT_OK;
 } TT_NO_THROW
 
-static tt_status tensor_maps_for(tt_workload* w, const GemmArgs& g, const void* a_ptr, const void* b_ptr, const TmapPair** out) {
+static tt_status tensor_maps_for(tt_workload* w, const GemmArgs& g, const void* a_ptr, const void* b_ptr, const TmapPair** out, int plan = 0) {
     const void* y_ptr = g.epi_tma ? g.y : nullptr;
     const void* r_ptr = g.res_tma ? g.residual : nullptr;
     // a pass calls a kernel's layers in the same order every time: the search begins behind the last hit
@@ -295,11 +295,11 @@ static tt_status tensor_maps_for(tt_workload* w, const GemmArgs& g, const void* 
     for (size_t i = 0, at = w->tmap_next; i < n_maps; ++i, ++at) {
         if (at >= n_maps) at = 0;
         const TmapPair& e = w->tmaps[at];
-        if (e.a_ptr == a_ptr && e.b_ptr == b_ptr && e.y_ptr == y_ptr && e.r_ptr == r_ptr) { w->tmap_next = at + 1; *out = &e; return TT_OK; }
+        if (e.plan == plan && e.a_ptr == a_ptr && e.b_ptr == b_ptr && e.y_ptr == y_ptr && e.r_ptr == r_ptr) { w->tmap_next = at + 1; *out = &e; return TT_OK; }
     }
     TmapPair e;
     std::memset(&e, 0, sizeof e);
-    e.a_ptr = a_ptr; e.b_ptr = b_ptr; e.y_ptr = y_ptr; e.r_ptr = r_ptr;
+    e.plan = plan; e.a_ptr = a_ptr; e.b_ptr = b_ptr; e.y_ptr = y_ptr; e.r_ptr = r_ptr;
     // A gathered operand keeps an all-zero map in its parameter slot; the kernel never issues a TMA load on it.
     tt_status st = TT_OK;
     if (g.a_mode == OPM_TMA)
@@ -468,13 +468,13 @@ static tt_status launch_with(tt_workload* w, const tt_tensors* t, void* stream, 
             unsigned char more[2][128] = {};             // (copies: what a further member's maps add to the cache may move the others)
             for (int i = 0; i < beside.n_more; ++i) {
                 const tt_tensors* o = beside.more[i];
-                const tt_status s = tensor_maps_for(w, g, pick(o, p.a_tensor), pick(o, p.b_tensor), &maps);
+                const tt_status s = tensor_maps_for(w, g, pick(o, p.a_tensor), pick(o, p.b_tensor), &maps, beside.n_more);
                 if (s != TT_OK) return s;
                 std::memcpy(more[i], p.a_tensor == 1 ? maps->a : maps->b, 128);
                 c.bias_more[i] = w->sh.has_bias ? static_cast<const float*>(o->bias) : nullptr;
                 c.y_more[i] = static_cast<float*>(o->y);
             }
-            const tt_status s = tensor_maps_for(w, g, a_ptr, b_ptr, &maps);
+            const tt_status s = tensor_maps_for(w, g, a_ptr, b_ptr, &maps, beside.n_more);
             if (s != TT_OK) return s;
             e = launch_gemm_chain(p.info, p.run_smem, g, c, maps->a, maps->b, more[0], more[1], st);
         } else {
@@ -814,11 +814,11 @@ static tt_status launch_chain_attention(const tt_chain_step* s, const AttnArgs& 
     const tt_shapes& sh = qk->sh;
     // the maps of the queries and keys are kept with the scores' workload, the values' with the context's
     const auto cached = [](tt_workload* w, const void* a, const void* b) -> const TmapPair* {
-        for (const TmapPair& m : w->tmaps) if (m.a_ptr == a && m.b_ptr == b && m.y_ptr == w && !m.r_ptr) return &m;
+        for (const TmapPair& m : w->tmaps) if (m.plan == kAttnMaps && m.a_ptr == a && m.b_ptr == b) return &m;
         return nullptr;
     };
     const auto keep = [](tt_workload* w, TmapPair& m, const void* a, const void* b) {
-        m.a_ptr = a; m.b_ptr = b; m.y_ptr = w; m.r_ptr = nullptr;
+        m.plan = kAttnMaps; m.a_ptr = a; m.b_ptr = b;
         if (w->tmaps.size() >= 4096) w->tmaps.clear();
         w->tmaps.push_back(m);
         return &w->tmaps.back();

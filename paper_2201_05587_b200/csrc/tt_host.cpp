@@ -1149,31 +1149,40 @@ tt_status legalise(const tt_workload* w, const tt_schedule_record* rec, int mode
 }
 
 // Layers of one plan on the same activations may share a launch (dense without skip tensor, both operands K-major by TMA,
-// reduction by a cluster or in one piece).  Together they have that many times the tiles, and all of their clusters should be resident at once, which the splits
-// of one layer may be too many for: three of 768 -> 768 on 128 rows are 36 clusters of 4 where 33 fit, and the three that are left
-// made the launch take 11 us instead of 5 (the 12-layer encoder 430 -> 380); so the splits are as many as the SMs hold clusters for.  No group where not even whole tiles fit.
+// reduction by a cluster or in one piece).  Together they have that many times the tiles, and all of their clusters should be
+// resident at once: three of 768 -> 768 on 128 rows in tiles of 64 columns are 36 clusters of 4 where 33 fit, and the three that
+// are left made the launch take 11 us instead of 5.  A result's sums depend on the splits, their steps and the accumulators, and
+// those stay the record's, so that a layer gives the same bits in a group as by itself; which operand is on the 128 rows and how
+// many columns a tile has is free.  Where the record's tiles are too many, the narrowest ones of either axis that are resident
+// take their place: they move the fewest operand bytes per CTA and are read out fastest.  The 12-layer encoder, 128 tokens: 384 us
+// with tiles of 80 columns, 386 with 96, 391 with 128, 470 with each layer by itself, 377 with three splits instead of four, whose
+// sums are others; 256 tokens: 523 with 160 columns, 584 with 256 and without a group, 497 with two splits.  No group where no tiles are resident.
 void plan_groups(tt_workload* w) {
     const Plan& p = w->plan;
     for (int i = 0; i < 2; ++i) w->group[i].applied = false;
     if (w->op != TT_OP_DENSE || w->sh.has_residual || p.strict || p.g.persistent || p.g.x3 || p.g.two_per_sm || p.info.workspace_bytes != 0 || p.g.a_mode != OPM_TMA || p.g.b_mode != OPM_TMA) return;
+    const int resident = kResidentClusters[p.g.split_k], own = p.info.legal.mma_m_axis;
     for (int i = 0; i < 2; ++i) {
-        const int clusters = p.info.grid_x * (i + 2);
-        int split = p.g.split_k;
-        while (split > 1 && clusters > kResidentClusters[split]) --split;
-        if (clusters > kSms) continue;
         Plan& q = w->group[i];
-        q = p;
-        if (split != p.g.split_k) {
-            tt_schedule_record rec = p.info.legal;
-            rec.split_k = split;
-            Plan r;
-            if (legalise(w, &rec, TT_MODE_LEGALISE, 0, &r) != TT_OK || r.info.grid_x != p.info.grid_x || r.g.atom_k != p.g.atom_k || r.info.workspace_bytes != 0 || r.g.two_per_sm) {
-                q.applied = false;
-                continue;
-            }
-            q = r;
+        if (p.info.grid_x * (i + 2) <= resident) {
+            q = p;
+            q.applied = true;
+            continue;
         }
-        q.applied = true;
+        for (const int axis : {own, 3 - own}) {
+            const int rows = axis == 2 ? w->sh.nn : w->sh.m, cols = axis == 2 ? w->sh.m : w->sh.nn;
+            const int columns = resident / ((rows + kHwTileM - 1) / kHwTileM * (i + 2));         // tiles along the columns
+            if (columns < 1) continue;
+            tt_schedule_record rec = p.info.legal;
+            rec.mma_m_axis = axis;
+            rec.tile_n = round_up((cols + columns - 1) / columns, 16);
+            if (rec.tile_n > 256 || (q.applied && rec.tile_n >= q.g.tile_n)) continue;
+            Plan r;
+            if (legalise(w, &rec, TT_MODE_LEGALISE, 0, &r) != TT_OK || r.info.grid_x * (i + 2) > resident || r.g.split_k != p.g.split_k ||
+                r.g.k_tiles_per_split != p.g.k_tiles_per_split || r.g.tile_k != p.g.tile_k || r.g.n_acc != p.g.n_acc || r.g.two_per_sm || r.info.workspace_bytes != 0) continue;
+            q = r;
+            q.applied = true;
+        }
     }
 }
 

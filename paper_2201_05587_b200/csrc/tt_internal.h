@@ -144,6 +144,7 @@ struct ConvPmArgs {
 
 // The attention of a chained pass in one launch (tt_attention_kernel).
 constexpr int kAttnRows = 32;                               // query rows of a CTA
+constexpr int kAttnMaps = 3;                                // its tensor maps, beside those of the plans (TmapPair)
 struct AttnArgs {
     float* scores; float* probs; float* ctx;
     unsigned* status; unsigned long long wait_ns;
@@ -209,8 +210,9 @@ struct Plan {
 constexpr int kMaxEpiBufs = 3;
 constexpr unsigned kLateRingBytes = 8192;   // two 32 x 32 blocks per warp
 
-// The tensor maps of a launch, cached by the pointers they were made for.
+// The tensor maps of a launch, cached by the plan and the pointers they were made for.
 struct TmapPair {
+    int plan;                               // 0: the applied one, 1 and 2: of a group of two and three layers, kAttnMaps
     const void* a_ptr; const void* b_ptr;
     const void* y_ptr; const void* r_ptr;   // persistent form with TMA read-out; null elsewhere
     alignas(64) unsigned char y[128];

@@ -1473,8 +1473,46 @@ def test_dense_layers_of_one_input_in_a_chain(residual, per_sm):
     for i, (y, tt) in enumerate(zip(out, tts)):
         y.fill_(float("nan"))
         wl.run(tt)
-        # (a group may take other splits, whose sums round differently)
-        assert util.rel_l2(got[i], y.cpu().numpy()) <= (2e-6 if i < 3 else 4e-4), i
+        np.testing.assert_array_equal(got[i], y.cpu().numpy(), err_msg=str(i))
+    wl.close()
+
+
+@pytest.mark.parametrize("m,k,n,rec", [
+    (128, 768, 768, dict(tile_n=64, tile_k=64, stages=3, split_k=4, mma_m_axis=2)),                 # 36 clusters of 4 as the record has them: other tiles
+    (128, 768, 768, dict(tile_n=64, tile_k=64, stages=3, split_k=4, mma_m_axis=1)),
+    (256, 768, 768, dict(tile_n=64, tile_k=64, stages=2, split_k=4, mma_m_axis=2)),
+    (33, 1000, 500, dict(tile_n=16, tile_k=32, stages=4, split_k=7, mma_m_axis=1, acc_split=2)),    # ragged, two accumulators
+    (200, 264, 900, dict(tile_n=32, tile_k=32, stages=2, split_k=1, mma_m_axis=2)),                 # no split: 148 tiles
+    (64, 2048, 96, dict(tile_n=32, tile_k=128, stages=1, split_k=8, mma_m_axis=2)),                 # the record's tiles fit
+])
+def test_layers_in_one_launch_give_the_bits_they_give_alone(m, k, n, rec):
+    """Two and three dense layers of one input in a chained pass: the tiles of the group may be others than the record's, its sums are
+    the record's.  Then each layer alone, and the group again: neither takes the other's tensor maps."""
+    import types
+    import torch
+    wl = W._dense(m, k, n, act=B.TT_ACT_RELU).workload()
+    wl.apply(tc(**rec))
+    rng = torch.Generator().manual_seed(4)
+    draw = lambda *s: torch.randn(*s, generator=rng).cuda()
+    x, ops = draw(m, k), [(draw(n, k), draw(n)) for _ in range(3)]
+    for layers in (2, 3):
+        out = [torch.empty(m, n, device="cuda") for _ in range(layers)]
+        tts = [B.tensors(x, w, b, None, y) for (w, b), y in zip(ops, out)]
+        args = ([wl], [types.SimpleNamespace(kernel=0)] * layers, tts, [(0, ())] * layers)
+        assert B.chain_launches(*args) == 1
+        runs = []
+        for chained in (True, False, True):
+            for y in out:
+                y.fill_(float("nan"))
+            if chained:
+                B.run_chain(*args, [torch.cuda.current_stream()])
+            else:
+                for tt in tts:
+                    wl.run(tt)
+            runs.append(torch.stack(out).cpu().numpy())
+        assert wl.status() == B.TT_OK and not np.isnan(runs[1]).any()
+        np.testing.assert_array_equal(runs[0], runs[1])
+        np.testing.assert_array_equal(runs[2], runs[1])
     wl.close()
 
 
