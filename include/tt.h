@@ -299,10 +299,11 @@ typedef struct tt_chain_step {
  * device.  Nothing is synchronised.  On an
  * error the layers in front of the failing one have been enqueued and the side streams joined; failed_at (may be NULL)
  * receives its position.  Layers may share a workload; those on different lanes run side by side, or one after the other
- * where the workload has scratch (workspace_bytes > 0).  Layers may share a launch, where the results are the same: up to three
- * dense layers of one workload on the same x that do not touch one another's tensors (on the lane of the first, under the record
- * applied), and a batch_matmul NT, the softmax of its result and the batch_matmul NN of that (up to 256 columns, as many rows as
- * are resident at once, not under strict records; all three outputs are written).  Calls for the same workloads do not overlap in time (one handle,
+ * where the workload has scratch (workspace_bytes > 0).  Layers may share a launch, where the results are the same to the bit:
+ * up to three dense layers of one workload on the same x that do not touch one another's tensors (on the lane of the first, with the
+ * splits and accumulators of the record applied), and a batch_matmul NT, the softmax of its result and the batch_matmul NN of that
+ * (up to 256 columns, as many rows as are resident at once, not under strict records, softmax rows of four lanes or more on 16 bytes,
+ * no splits of several accumulators each; all three outputs are written).  Calls for the same workloads do not overlap in time (one handle,
  * one thread), calls for different ones may run on different threads. */
 tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* streams, size_t n_streams, size_t* failed_at);
 /* How many kernels that pass launches: layers may go to the device together (see above), a layer under a record with a filter

@@ -3,7 +3,8 @@
 // At batch 1 the three launches are latency and nothing else (12 heads of 128 x 128 x 64: 12 or 24 CTAs, 3.6 + 1.6 + 5.4 us of
 // which the products take a tenth).  Here a CTA takes kAttnRows query rows of one head through all three: the scores stay in
 // tensor memory and registers between the products, and all three outputs are written as the separate layers write them.  The
-// arithmetic is theirs too: TF32 products with fp32 accumulation, fp32 softmax over the unrounded scores.
+// arithmetic is that of their records to the bit: as many accumulators as a record has splits or accumulators, added up in its
+// order, and row sums in the order of the softmax record's lanes.
 //
 // The accumulators have 128 rows, of which kAttnRows are used: with 32, 12 heads of 128 rows spread over 48 SMs, and the rows' work
 // (exponentials, 2 x 4 bytes written per score) is what is serial here, not the products.  The A tiles (queries, probabilities) hold
@@ -28,10 +29,83 @@ constexpr int kAttnThreads = 512;
 constexpr int kAttnSoftmaxWarps = 4, kAttnStoreWarps = 10;
 constexpr uint32_t kAttnAtom = kAttnRows * 128u;         // bytes of a 32-column block of a tile of kAttnRows rows
 
+// Builds: FAR, more than 128 keys (two blocks of 32 a softmax warp); ANY, records of several accumulators, single values a lane or rows
+// of fewer than 16 lanes.  A launch meets a cold instruction cache, and what ANY adds costs it 0.5 us where nothing of it is run (the
+// 12-layer encoder on 128 tokens 385 -> 391 us, on 256 525 -> 531; without FAR 381).  80 or 128 registers and 512 threads: no CTA that
+// needs tensor memory, too, fits beside one that has not got its columns yet.
+
+// One product: its steps of 8 of the reduction go into the accumulators of its record, `pitch` columns apart: `per` steps to each in
+// turn (a record with splits), or dealt one by one (per = 0).
+template <bool ANY, typename Issue>
+__device__ __forceinline__ void attn_steps(uint32_t col, uint32_t pitch, int accs, int per, int steps, Issue issue) {
+    if (ANY && accs > 1) {
+#pragma unroll 1
+        for (int a = 0; a < accs; ++a, col += pitch) {
+            const int first = per > 0 ? a * per : a, end = per > 0 ? min(steps, first + per) : steps;
+#pragma unroll 1
+            for (int k8 = first; k8 < end; k8 += per > 0 ? 1 : accs) issue(col, k8, k8 != first ? 1u : 0u);
+        }
+        return;
+    }
+    for (int k8 = 0; k8 < steps; ++k8) issue(col, k8, k8 > 0 ? 1u : 0u);
+}
+// ... and 32 of its columns, read out in accumulator order.
+template <bool ANY>
+__device__ __forceinline__ void attn_read(uint32_t col, uint32_t pitch, int accs, float (&v)[32]) {
+    uint32_t r[32];
+    tmem_ld32(col, r);
+    tmem_wait_ld();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+    if (!ANY) return;
+#pragma unroll 1
+    for (int a = 1; a < accs; ++a) {
+        tmem_ld32(col + (uint32_t)a * pitch, r);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] += __uint_as_float(r[j]);
+    }
+}
+
+// The sum of a row as 4 * m lanes come to it (m = 1, 2, 4, 8): lane l's share is the sum of values l, l + 4 m, ... of the line, the
+// shares are added in halves, l and l + 2 m first.  The line holds 8 groups of four values, or 16 (`far`).
+template <bool FAR, bool ANY>
+__device__ __forceinline__ float attn_row_sum(uint32_t line, bool far, int m) {
+    const auto add = [](float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; };
+    const auto at = [&](int q) { return ld_shared_v4f(line + 16u * (uint32_t)q); };
+    float4 x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = at(q);
+    if (ANY && m < 4) {
+        // (m = 2: two shares of every second group; m = 1: one of all)
+        const auto odd = [&](const float4& v) { if (m == 1) add(x[0], v); else add(x[1], v); };
+        if (m == 1) add(x[0], x[1]);
+#pragma unroll
+        for (int q = 2; q < 8; q += 2) { add(x[0], x[q]); odd(x[q + 1]); }
+#pragma unroll 1
+        for (int q = 8; q < (far ? 16 : 8); q += 2) { add(x[0], at(q)); odd(at(q + 1)); }
+        if (m == 2) add(x[0], x[1]);
+    } else {
+        if (FAR && far && m == 8) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) add(x[q], at(q + 8));
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) add(x[q], x[q + 4]);           // m = 8: the first halves; m = 4: a share's second group
+        if (FAR && far && m == 4) {
+#pragma unroll
+            for (int q = 8; q < 16; ++q) add(x[q & 3], at(q));
+        }
+        add(x[0], x[2]); add(x[1], x[3]); add(x[0], x[1]);
+    }
+    return (x[0].x + x[0].z) + (x[0].y + x[0].w);
+}
+
 // Named barriers: 1 the softmax warps, 2 and 3 the softmax and the storing warps (a tile is in shared memory).
 __device__ __forceinline__ void attn_meet(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 __device__ __forceinline__ void attn_report(int id, int threads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
+template <bool FAR, bool ANY>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                     const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ AttnArgs g) {
@@ -41,7 +115,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
     __shared__ uint64_t p_bar;                            // the probabilities' tile is written
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ float s_max[kAttnSoftmaxWarps][32], s_sum[kAttnSoftmaxWarps][32];
+    __shared__ float s_max[kAttnSoftmaxWarps][32];
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     volatile int* abortp = &abort_flag;
@@ -102,11 +176,10 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
             if (ok) {
                 tc_fence_after();
                 const uint32_t a0 = lo + ((q_s & 0x3FFFFu) >> 4), b0 = lo + ((k_s & 0x3FFFFu) >> 4), b_atom = (uint32_t)g.n16 * 8u;
-                for (int k8 = 0; k8 < g.d_steps; ++k8) {
+                attn_steps<ANY>(tmem_base, (uint32_t)g.n_blocks * 32u, g.s_accs, g.s_per, g.d_steps, [&](uint32_t d, int k8, uint32_t accumulate) {
                     const uint32_t at = (uint32_t)k8 >> 2, in = 2u * ((uint32_t)k8 & 3u);
-                    mma_tf32(tmem_base, ((uint64_t)hi << 32) | (uint64_t)(a0 + at * (kAttnAtom >> 4) + in), ((uint64_t)hi << 32) | (uint64_t)(b0 + at * b_atom + in),
-                             g.idesc_s, k8 > 0 ? 1u : 0u);
-                }
+                    mma_tf32(d, ((uint64_t)hi << 32) | (uint64_t)(a0 + at * (kAttnAtom >> 4) + in), ((uint64_t)hi << 32) | (uint64_t)(b0 + at * b_atom + in), g.idesc_s, accumulate);
+                });
                 mma_commit(smem_u32(&s_bar));
                 ok = mbar_wait(smem_u32(&v_bar), 0u, abortp, g.status, 2u, g.wait_ns) && mbar_wait(smem_u32(&p_bar), 0u, abortp, g.status, 3u, g.wait_ns);
             }
@@ -115,11 +188,11 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
                 const uint64_t v0 = make_desc_mn(0u, (uint32_t)g.n8 * 128u);
                 const uint32_t v_hi = (uint32_t)(v0 >> 32);
                 const uint32_t a0 = lo + ((p_s & 0x3FFFFu) >> 4);
-                uint32_t b = (uint32_t)v0 + ((v_s & 0x3FFFFu) >> 4);
-                for (int k8 = 0; k8 < g.n8 >> 3; ++k8, b += 64u) {
+                const uint32_t b0 = (uint32_t)v0 + ((v_s & 0x3FFFFu) >> 4);
+                attn_steps<ANY>(tmem_base + (uint32_t)g.o_col, (uint32_t)g.v_boxes * 32u, g.o_accs, g.o_per, g.n8 >> 3, [&](uint32_t d, int k8, uint32_t accumulate) {
                     const uint32_t a = a0 + ((uint32_t)k8 >> 2) * (kAttnAtom >> 4) + 2u * ((uint32_t)k8 & 3u);
-                    mma_tf32(tmem_base + (uint32_t)g.o_col, ((uint64_t)hi << 32) | (uint64_t)a, ((uint64_t)v_hi << 32) | (uint64_t)b, g.idesc_o, k8 > 0 ? 1u : 0u);
-                }
+                    mma_tf32(d, ((uint64_t)hi << 32) | (uint64_t)a, ((uint64_t)v_hi << 32) | (uint64_t)(b0 + 64u * (uint32_t)k8), g.idesc_o, accumulate);
+                });
                 mma_commit(smem_u32(&o_bar));
             }
         }
@@ -127,7 +200,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
     } else if (softmax_warp) {
         // ---------------- softmax: a lane has one query row, a warp every fourth block of 32 keys ----------------
         const int sw = warp >> 2, row = m0 + lane;
-        constexpr int kBlocks = 256 / 32 / kAttnSoftmaxWarps;     // blocks a warp can have
+        constexpr int kBlocks = FAR ? 2 : 1;             // blocks a warp can have
         const uint32_t line = (uint32_t)lane * 128u, swz = (uint32_t)(lane & 7);
         float v[kBlocks][32];
         float mx = -INFINITY;
@@ -138,17 +211,14 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
             for (int i = 0; i < kBlocks; ++i) {
                 const int blk = sw + i * kAttnSoftmaxWarps;
                 if (blk >= g.n_blocks) break;            // (warp-uniform)
-                uint32_t r[32];
-                tmem_ld32(tmem_base + (uint32_t)(blk * 32), r);
-                tmem_wait_ld();
+                attn_read<ANY>(tmem_base + (uint32_t)(blk * 32), (uint32_t)g.n_blocks * 32u, g.s_accs, v[i]);
 #pragma unroll
                 for (int j = 0; j < 32; j += 4)
-                    st_shared_v4(sc_s + (uint32_t)blk * kAttnAtom + line + ((((uint32_t)j >> 2) ^ swz) << 4), __uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                                 __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+                    st_shared_v4(sc_s + (uint32_t)blk * kAttnAtom + line + ((((uint32_t)j >> 2) ^ swz) << 4), v[i][j], v[i][j + 1], v[i][j + 2], v[i][j + 3]);
                 const int left = g.n - blk * 32;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
-                    v[i][j] = j < left ? __uint_as_float(r[j]) * g.scale : -INFINITY;
+                    v[i][j] = j < left ? __fmul_rn(v[i][j], g.scale) : -INFINITY;
                     mx = fmaxf(mx, v[i][j]);
                 }
             }
@@ -157,18 +227,45 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
         s_max[sw][lane] = mx;
         attn_meet(1, 32 * kAttnSoftmaxWarps);
         mx = fmaxf(fmaxf(s_max[0][lane], s_max[1][lane]), fmaxf(s_max[2][lane], s_max[3][lane]));
-        float sum = 0.f;
+        // The row's sum in the order of the softmax record's lanes: theirs are groups of four values, whose sums go to the row's line (zeros
+        // where the row has no more of them), ...
+        const uint32_t sums = base + g.x_off + (uint32_t)lane * kAttnSumLine;
+        const bool far = FAR && g.n_blocks > kAttnSoftmaxWarps;
 #pragma unroll
         for (int i = 0; i < kBlocks; ++i) {
-            if (sw + i * kAttnSoftmaxWarps >= g.n_blocks) break;
-            float part = 0.f;
+            const int blk = sw + i * kAttnSoftmaxWarps;
+            if (i > 0 && !far) break;
+            float t[8] = {};
+            if (blk < g.n_blocks) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) { v[i][j] = expf(v[i][j] - mx); part += v[i][j]; }
-            sum += part;
+                for (int j = 0; j < 32; ++j) v[i][j] = expf(v[i][j] - mx);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) t[j] = (v[i][4 * j] + v[i][4 * j + 1]) + (v[i][4 * j + 2] + v[i][4 * j + 3]);
+                if (ANY && !g.lane_groups) {
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4)
+                        st_shared_v4(p_s + (uint32_t)blk * kAttnAtom + line + ((((uint32_t)j >> 2) ^ swz) << 4), v[i][j], v[i][j + 1], v[i][j + 2], v[i][j + 3]);
+                }
+            }
+            st_shared_v4(sums + (uint32_t)blk * 32u, t[0], t[1], t[2], t[3]);
+            st_shared_v4(sums + (uint32_t)blk * 32u + 16u, t[4], t[5], t[6], t[7]);
         }
-        s_sum[sw][lane] = sum;
         attn_meet(1, 32 * kAttnSoftmaxWarps);
-        const float inv = 1.f / ((s_sum[0][lane] + s_sum[1][lane]) + (s_sum[2][lane] + s_sum[3][lane]));
+        if (ANY && !g.lane_groups) {
+            // ... or single values, every lane's 4 m apart: the warps add them up, four lanes' at a time
+#pragma unroll 1
+            for (int q = sw; q < 8; q += kAttnSoftmaxWarps) {
+                float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+                for (int u = q < g.lanes4 ? q : g.n_blocks * 8; u < g.n_blocks * 8; u += g.lanes4) {
+                    const float4 e = ld_shared_v4f(p_s + (uint32_t)(u >> 3) * kAttnAtom + line + ((((uint32_t)u & 7u) ^ swz) << 4));
+                    t.x += e.x; t.y += e.y; t.z += e.z; t.w += e.w;
+                }
+                st_shared_v4(sums + (uint32_t)q * 16u, t.x, t.y, t.z, t.w);
+            }
+            attn_meet(1, 32 * kAttnSoftmaxWarps);
+        }
+        const float inv = 1.f / attn_row_sum<FAR, ANY>(sums, far && g.lane_groups, g.lanes4);
 #pragma unroll
         for (int i = 0; i < kBlocks; ++i) {
             const int blk = sw + i * kAttnSoftmaxWarps;
@@ -185,17 +282,16 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
         ok = __all_sync(0xffffffffu, ok && mbar_wait(smem_u32(&o_bar), 0u, abortp, g.status, 4u, g.wait_ns));
         tc_fence_after();
         if (ok && sw * 32 < g.dv) {
-            uint32_t r[32];
-            tmem_ld32(tmem_base + (uint32_t)(g.o_col + sw * 32), r);
-            tmem_wait_ld();
+            float r[32];
+            attn_read<ANY>(tmem_base + (uint32_t)(g.o_col + sw * 32), (uint32_t)g.v_boxes * 32u, g.o_accs, r);
             if (row < g.m) {
                 float* y = g.ctx + ((long long)head * g.m + row) * g.dv + sw * 32;
                 const int left = g.dv - sw * 32;         // (a multiple of 4)
 #pragma unroll
                 for (int j = 0; j < 32; j += 4) {
                     if (j >= left) break;
-                    if (g.ctx_vec) *reinterpret_cast<float4*>(y + j) = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
-                    else for (int e = 0; e < 4; ++e) y[j + e] = __uint_as_float(r[j + e]);
+                    if (g.ctx_vec) *reinterpret_cast<float4*>(y + j) = make_float4(r[j], r[j + 1], r[j + 2], r[j + 3]);
+                    else for (int e = 0; e < 4; ++e) y[j + e] = r[j + e];
                 }
             }
         }
@@ -232,8 +328,11 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
 }
 
 cudaError_t launch_attention(const AttnArgs& g, int heads, const void* tmap_q, const void* tmap_k, const void* tmap_v, cudaStream_t st) {
-    static OncePerDevice raised;
-    const cudaError_t ready = raised([] { return cudaFuncSetAttribute(tt_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
+    static OncePerDevice raised[3];
+    const bool any = g.s_accs > 1 || g.o_accs > 1 || !g.lane_groups || g.lanes4 < 4;
+    const int build = any ? 2 : g.n > 128 ? 1 : 0;
+    const auto kern = any ? tt_attention_kernel<true, true> : g.n > 128 ? tt_attention_kernel<true, false> : tt_attention_kernel<false, false>;
+    const cudaError_t ready = raised[build]([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
     if (ready != cudaSuccess) return ready;
     CUtensorMap tq, tk, tv;
     memcpy(&tq, tmap_q, sizeof tq);
@@ -246,7 +345,7 @@ cudaError_t launch_attention(const AttnArgs& g, int heads, const void* tmap_q, c
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tt_attention_kernel, tq, tk, tv, g);
+    return cudaLaunchKernelEx(&cfg, kern, tq, tk, tv, g);
 }
 
 }  // namespace tt

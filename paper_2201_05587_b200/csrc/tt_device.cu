@@ -783,19 +783,35 @@ static bool attention_at(const tt_chain_step* steps, size_t n_steps, size_t firs
     a.d_atoms = (d + 31) / 32; a.d_steps = (d + 7) / 8; a.v_boxes = (dv + 31) / 32;
     const auto vec = [](const void* p, int cols) { return cols % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
     a.scores_vec = vec(a.scores, n); a.probs_vec = vec(a.probs, n); a.ctx_vec = vec(a.ctx, dv);
+    // The order in which the layers' records add up.  What the kernel has no order for takes three launches: splits of several
+    // accumulators each, the softmax from memory (other alignments, rows of few lanes).
+    const auto products = [](const GemmArgs& p, int steps, int* accs, int* per) {
+        *per = p.split_k > 1 ? p.k_tiles_per_split * (p.tile_k / 8) : 0;
+        *accs = p.split_k > 1 ? p.split_k : std::min(p.n_acc, steps);
+        return p.split_k == 1 || p.n_acc == 1;
+    };
+    if (!products(qk->plan.g, a.d_steps, &a.s_accs, &a.s_per) || !products(pv->plan.g, a.n8 / 8, &a.o_accs, &a.o_per)) return false;
+    const RowArgs& rows = sm->plan.row;
+    if (rows.cached == 0 && rows.chunk == 0) return false;
+    if (((reinterpret_cast<uintptr_t>(ts.x) | reinterpret_cast<uintptr_t>(ts.y)) & 15u) != 0 || rows.lanes_per_row < 4) return false;
+    a.lanes4 = rows.lanes_per_row / 4; a.lane_groups = rows.cached > 0;
     a.scale = sm->sh.scale;
     const int block = kAttnRows * 128;                   // 32 columns of a tile of query rows
     a.p_off = (unsigned)(a.d_atoms * block);
     a.k_off = a.p_off + (unsigned)(a.n_blocks * block);
-    a.v_off = a.k_off + (unsigned)std::max(a.d_atoms * a.n16 * 128, a.n_blocks * block);
+    // (the scores' tile and the partial sums behind it take the keys' place)
+    a.x_off = a.k_off + (unsigned)(a.n_blocks * block);
+    a.v_off = a.k_off + (unsigned)((std::max(a.d_atoms * a.n16 * 128, a.n_blocks * block + kAttnRows * (int)kAttnSumLine) + 1023) / 1024 * 1024);
     // (the tensor core reads 128 rows of a tile that has 32: all of that lies inside)
     const int over = 128 * 128 - block;
     const int bytes = std::max((int)a.v_off + a.v_boxes * a.n8 * 128, (int)a.k_off + over) + 1024;
     if (bytes > kDynSmemLimit) return false;
     a.smem_bytes = bytes;
-    a.o_col = a.n_blocks * 32;
+    a.o_col = a.s_accs * a.n_blocks * 32;
+    const int columns = a.o_col + a.o_accs * a.v_boxes * 32;
+    if (columns > 512) return false;
     a.tmem_cols = 32;
-    while (a.tmem_cols < (unsigned)(a.o_col + a.v_boxes * 32)) a.tmem_cols *= 2;
+    while ((int)a.tmem_cols < columns) a.tmem_cols *= 2;
     const unsigned tf32 = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(kHwTileM >> 4) << 24);
     a.idesc_s = tf32 | ((unsigned)(a.n16 >> 3) << 17);
     a.idesc_o = tf32 | ((unsigned)((dv + 15) / 16 * 2) << 17) | (1u << 16);

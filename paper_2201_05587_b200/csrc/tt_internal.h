@@ -144,6 +144,7 @@ struct ConvPmArgs {
 
 // The attention of a chained pass in one launch (tt_attention_kernel).
 constexpr int kAttnRows = 32;                               // query rows of a CTA
+constexpr unsigned kAttnSumLine = 17 * 16;                  // bytes of a row's partial sums, a lane's 16 away from every bank of the next one's
 constexpr int kAttnMaps = 3;                                // its tensor maps, beside those of the plans (TmapPair)
 struct AttnArgs {
     float* scores; float* probs; float* ctx;
@@ -153,8 +154,11 @@ struct AttnArgs {
     int d_atoms, d_steps, v_boxes;              // head size in 32s and 8s, value columns in 32s
     int scores_vec, probs_vec, ctx_vec;         // rows allow 16-byte stores
     float scale;
-    int o_col;                                  // the context's accumulator behind the scores'
-    unsigned p_off, k_off, v_off, idesc_s, idesc_o, tmem_cols;
+    int o_col;                                  // the context's accumulators behind the scores'
+    // the layers' records: accumulators of a product, and steps of the reduction to each (0: dealt one by one); lanes of a softmax
+    // row / 4, whose shares are groups of four values or single ones
+    int s_accs, s_per, o_accs, o_per, lanes4, lane_groups;
+    unsigned p_off, k_off, v_off, x_off, idesc_s, idesc_o, tmem_cols;
     int smem_bytes;
     Ahead ahead;
 };

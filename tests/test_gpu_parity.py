@@ -1,6 +1,7 @@
 """GPU parity: the CUDA path, called through the C ABI, against the CPU oracle on the same seeded inputs."""
 import ctypes
 import itertools
+import math
 import os
 import subprocess
 import sys
@@ -1514,6 +1515,61 @@ def test_layers_in_one_launch_give_the_bits_they_give_alone(m, k, n, rec):
         np.testing.assert_array_equal(runs[0], runs[1])
         np.testing.assert_array_equal(runs[2], runs[1])
     wl.close()
+
+
+_PLAIN = dict(tile_n=64, tile_k=64, stages=2, mma_m_axis=1)
+
+
+@pytest.mark.parametrize("n,d,qk,lanes,pv,launches", [
+    (1, 8, _PLAIN, 32, _PLAIN, 1),
+    (31, 64, _PLAIN, 8, _PLAIN, 1),
+    (64, 64, dict(tile_n=64, tile_k=64, stages=4, mma_m_axis=2, persistent=1), 16, dict(tile_n=64, tile_k=64, stages=3, mma_m_axis=1, persistent=1), 1),
+    (97, 36, dict(_PLAIN, tile_k=16, split_k=2), 16, dict(_PLAIN, tile_k=32, split_k=3), 1),
+    (128, 64, dict(_PLAIN, tile_k=16, split_k=3), 4, dict(_PLAIN, tile_k=64, split_k=2), 1),
+    (128, 64, dict(_PLAIN, acc_split=2), 32, dict(_PLAIN, acc_split=4, mma_m_axis=2), 1),
+    (130, 64, _PLAIN, 4, dict(_PLAIN, tile_n=32, tile_k=8, split_k=8, mma_m_axis=2), 3),                     # 160 + 8 x 64 columns
+    (130, 100, _PLAIN, 8, dict(_PLAIN, tile_n=128, tile_k=64, split_k=2), 1),
+    (200, 64, _PLAIN, 8, dict(_PLAIN, tile_k=128, split_k=2, mma_m_axis=2), 1),
+    (255, 32, dict(_PLAIN, tile_k=8), 32, dict(_PLAIN, tile_k=32, split_k=4), 1),
+    (256, 64, _PLAIN, 16, dict(_PLAIN, split_k=4), 1),
+    (256, 64, _PLAIN, 32, dict(_PLAIN, acc_split=2), 1),
+    (129, 64, _PLAIN, 2, _PLAIN, 3),                                                                       # rows of two lanes
+    (96, 64, _PLAIN, 16, dict(_PLAIN, tile_k=32, split_k=2, acc_split=2), 3),                               # splits of two accumulators
+])
+def test_attention_in_one_launch_gives_the_bits_of_its_layers(n, d, qk, lanes, pv, launches):
+    """Scores, softmax and context under records of every order of their sums: the one launch of a chained pass against the three
+    layers by themselves; orders that it does not know go to the device one by one."""
+    import types
+    import torch
+    heads = 3
+    specs = [W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(heads, n, n, d, True), 1, "qk", "bert"),
+             W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(heads, n, n, 2.0 / math.sqrt(d)), 1, "softmax", "bert"),
+             W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(heads, n, d, n, False), 1, "pv", "bert")]
+    wls = [sp.workload() for sp in specs]
+    wls[0].apply(tc(**qk))
+    wls[1].apply(B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=lanes, block_y=4, vec_width=4))
+    wls[2].apply(tc(**pv))
+    rng = torch.Generator().manual_seed(6)
+    q, k, v = (torch.randn(heads, n, d, generator=rng).cuda() for _ in range(3))
+    out = [torch.empty(heads, n, n, device="cuda"), torch.empty(heads, n, n, device="cuda"), torch.empty(heads, n, d, device="cuda")]
+    tts = [B.tensors(q, k, None, None, out[0]), B.tensors(out[0], None, None, None, out[1]), B.tensors(out[1], v, None, None, out[2])]
+    args = (wls, [types.SimpleNamespace(kernel=i) for i in range(3)], tts, [(0, ())] * 3)
+    assert B.chain_launches(*args) == launches
+    runs = []
+    for chained in (True, False):
+        for y in out:
+            y.fill_(float("nan"))
+        if chained:
+            B.run_chain(*args, [torch.cuda.current_stream()])
+        else:
+            for wl, tt in zip(wls, tts):
+                wl.run(tt)
+        runs.append([y.cpu().numpy() for y in out])
+    assert all(wl.status() == B.TT_OK for wl in wls) and not any(np.isnan(y).any() for y in runs[1])
+    for name, a, b in zip(("scores", "probabilities", "context"), *runs):
+        np.testing.assert_array_equal(a, b, err_msg=name)
+    for wl in wls:
+        wl.close()
 
 
 @pytest.mark.parametrize("spec", [
