@@ -334,7 +334,8 @@ tt_status tt_workload_set_constant_weights(tt_workload* w, int32_t on);
 tt_status tt_workload_status(tt_workload* w, void* cuda_stream);
 /* Every wait inside a kernel (on a copy, on a pipeline buffer, on the accumulator) gives up after this many
  * nanoseconds: the kernel then records TT_ERR_TIMEOUT in the status word, lets its copies land, releases its tensor
- * memory and returns, and the context stays usable.  Default: one second.  Takes effect with the next run. */
+ * memory and returns, and the context stays usable.  Default: one second.  Takes effect with the next run.  A launch that is the
+ * run of several workloads (tt_run_chain) has the shortest of their limits and records a wait that gave up with all of them. */
 tt_status tt_workload_set_wait_limit(tt_workload* w, uint64_t nanoseconds);
 /* Test facility for that path.  With extra_bytes > 0 (a multiple of 16) the barrier of the first pipeline stage of a
  * GEMM_TC kernel whose operands arrive by TMA is told to expect extra_bytes more than its copies deliver (in the CTAs

@@ -153,7 +153,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
         if (elect_one()) {
             const uint32_t qb = smem_u32(&qk_bar), vb = smem_u32(&v_bar);
             const uint32_t k_atom = (uint32_t)g.n16 * 128u, v_box = (uint32_t)g.n8 * 128u;
-            mbar_expect_tx(qb, (uint32_t)g.d_atoms * (kAttnAtom + k_atom));
+            mbar_expect_tx(qb, (uint32_t)g.d_atoms * (kAttnAtom + k_atom) + g.extra_tx);      // (test facility: tt_workload_test_stall)
             for (int at = 0; at < g.d_atoms; ++at) {
                 tma_load_3d(q_s + (uint32_t)at * kAttnAtom, &tmap_q, qb, at * 32, m0, head);
                 tma_load_3d(k_s + (uint32_t)at * k_atom, &tmap_k, qb, at * 32, 0, head);
@@ -281,7 +281,10 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
         // context: 32 columns a warp
         ok = __all_sync(0xffffffffu, ok && mbar_wait(smem_u32(&o_bar), 0u, abortp, g.status, 4u, g.wait_ns));
         tc_fence_after();
-        if (ok && sw * 32 < g.dv) {
+        if (!ok) {
+            // wherever a wait gave up, this one has too: the run of all three layers (the first one's status word has it from the wait)
+            if (lane == 0) for (unsigned* word : g.status_more) atomicCAS(word, 0u, (unsigned)TT_ERR_TIMEOUT | (20u << 8));
+        } else if (sw * 32 < g.dv) {
             float r[32];
             attn_read<ANY>(tmem_base + (uint32_t)(g.o_col + sw * 32), (uint32_t)g.v_boxes * 32u, g.o_accs, r);
             if (row < g.m) {

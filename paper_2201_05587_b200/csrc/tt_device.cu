@@ -732,7 +732,7 @@ static int group_at(const tt_chain_step* steps, size_t n_steps, size_t first) {
     const tt_chain_step& a = steps[first];
     if (!usable(a)) return 1;
     const tt_workload* w = a.workload;
-    if (w->extra_tx || !(w->group[0].applied || w->group[1].applied)) return 1;
+    if (!(w->group[0].applied || w->group[1].applied)) return 1;
     int count = 1;
     while (count < 3 && first + count < n_steps) {
         const tt_chain_step& b = steps[first + count];
@@ -757,7 +757,7 @@ static bool attention_at(const tt_chain_step* steps, size_t n_steps, size_t firs
     if (first + 3 > n_steps) return false;
     const tt_chain_step *s = steps + first;
     for (int i = 0; i < 3; ++i)
-        if (!usable(s[i]) || s[i].workload->plan.strict || s[i].workload->extra_tx) return false;
+        if (!usable(s[i]) || s[i].workload->plan.strict) return false;
     const tt_workload *qk = s[0].workload, *sm = s[1].workload, *pv = s[2].workload;
     if (qk->op != TT_OP_BATCH_MATMUL || !qk->sh.trans_b || sm->op != TT_OP_SOFTMAX || pv->op != TT_OP_BATCH_MATMUL || pv->sh.trans_b) return false;
     for (const tt_workload* w : {qk, pv})
@@ -777,7 +777,9 @@ static bool attention_at(const tt_chain_step* steps, size_t n_steps, size_t firs
         for (int32_t j = 0; j < s[i].n_waits; ++j) if ((size_t)s[i].waits[j] >= first + i) return false;
     AttnArgs a{};
     a.scores = static_cast<float*>(tq.y); a.probs = static_cast<float*>(ts.y); a.ctx = static_cast<float*>(tv.y);
-    a.status = qk->status_word; a.wait_ns = qk->wait_ns;
+    a.status = qk->status_word; a.status_more[0] = sm->status_word; a.status_more[1] = pv->status_word;
+    a.wait_ns = std::min({qk->wait_ns, sm->wait_ns, pv->wait_ns});
+    a.extra_tx = std::max({qk->extra_tx, sm->extra_tx, pv->extra_tx});
     a.m = m; a.n = n; a.dv = dv; a.tiles_m = (m + kAttnRows - 1) / kAttnRows;
     a.n16 = (n + 15) / 16 * 16; a.n8 = (n + 7) / 8 * 8; a.n_blocks = (n + 31) / 32;
     a.d_atoms = (d + 31) / 32; a.d_steps = (d + 7) / 8; a.v_boxes = (dv + 31) / 32;

@@ -147,20 +147,21 @@ constexpr int kAttnRows = 32;                               // query rows of a C
 constexpr unsigned kAttnSumLine = 17 * 16;                  // bytes of a row's partial sums, a lane's 16 away from every bank of the next one's
 constexpr int kAttnMaps = 3;                                // its tensor maps, beside those of the plans (TmapPair)
 struct AttnArgs {
-    float* scores; float* probs; float* ctx;
-    unsigned* status; unsigned long long wait_ns;
-    int m, n, dv, tiles_m;                      // query rows and keys of a head, columns of its values, CTAs per head
+    // (what every launch reads comes first: a launch meets a cold constant cache, line by line)
+    int tiles_m, m, n, dv;                      // CTAs per head; query rows and keys of a head, columns of its values
     int n16, n8, n_blocks;                      // keys in 16s, in 8s, in blocks of 32
     int d_atoms, d_steps, v_boxes;              // head size in 32s and 8s, value columns in 32s
-    int scores_vec, probs_vec, ctx_vec;         // rows allow 16-byte stores
-    float scale;
+    unsigned p_off, k_off, v_off, x_off, idesc_s, idesc_o, tmem_cols, extra_tx;
     int o_col;                                  // the context's accumulators behind the scores'
-    // the layers' records: accumulators of a product, and steps of the reduction to each (0: dealt one by one); lanes of a softmax
-    // row / 4, whose shares are groups of four values or single ones
-    int s_accs, s_per, o_accs, o_per, lanes4, lane_groups;
-    unsigned p_off, k_off, v_off, x_off, idesc_s, idesc_o, tmem_cols;
-    int smem_bytes;
+    float scale;
+    int lanes4, lane_groups;                    // the softmax record's lanes of a row / 4; their shares are groups of four values or single ones
+    int scores_vec, probs_vec, ctx_vec;         // rows allow 16-byte stores
+    float* scores; float* probs; float* ctx;
     Ahead ahead;
+    int s_accs, s_per, o_accs, o_per;           // accumulators of the products' records, steps of the reduction to each (0: dealt one by one)
+    int smem_bytes;
+    unsigned* status; unsigned* status_more[2]; // of the three layers
+    unsigned long long wait_ns;
 };
 
 struct DwArgs {

@@ -1572,6 +1572,52 @@ def test_attention_in_one_launch_gives_the_bits_of_its_layers(n, d, qk, lanes, p
         wl.close()
 
 
+def test_a_wait_that_gives_up_in_a_shared_launch_is_reported_by_every_layer():
+    """Attention as one launch, told to expect more than arrives on behalf of each of its workloads in turn: all three report the
+    time-out after the shortest of their wait limits, and the next pass is right.  Then a group of dense layers."""
+    import time
+    import types
+    import torch
+    heads, n, d = 2, 96, 32
+    specs = [W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(heads, n, n, d, True), 1, "qk", "bert"), W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(heads, n, n, 0.2), 1, "softmax", "bert"),
+             W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(heads, n, d, n, False), 1, "pv", "bert"), W._dense(n, 64, 48, name="dense")]
+    wls = [sp.workload() for sp in specs]
+    for wl in wls:
+        wl.apply(tc(tile_n=64, tile_k=32, stages=2) if wl.family() == B.TT_FAMILY_GEMM_TC else wl.default_schedule())
+    rng = torch.Generator().manual_seed(7)
+    draw = lambda *s: torch.randn(*s, generator=rng).cuda()
+    q, k, v, x = draw(heads, n, d), draw(heads, n, d), draw(heads, n, d), draw(n, 64)
+    out = [torch.empty(s, device="cuda") for s in ((heads, n, n), (heads, n, n), (heads, n, d), (n, 48), (n, 48))]
+    tts = [B.tensors(q, k, None, None, out[0]), B.tensors(out[0], None, None, None, out[1]), B.tensors(out[1], v, None, None, out[2])]
+    tts += [B.tensors(x, draw(48, 64), draw(48), None, y) for y in out[3:]]
+    stream = [torch.cuda.current_stream()]
+    node = lambda kernel: types.SimpleNamespace(kernel=kernel)
+    attention, group = (wls, [node(i) for i in range(3)], tts[:3], [(0, ())] * 3), (wls, [node(3)] * 2, tts[3:], [(0, ())] * 2)
+    for args, members, outs in ((attention, wls[:3], out[:3]), (group, wls[3:], out[3:])):
+        assert B.chain_launches(*args) == 1
+        B.run_chain(*args, stream)
+        right = [y.clone() for y in outs]
+        for i, wl in enumerate(members):
+            wl.test_stall(64)
+            members[(i + 1) % len(members)].set_wait_limit(2_000_000)
+            assert B.chain_launches(*args) == 1
+            torch.cuda.synchronize()
+            t0 = time.monotonic()
+            B.run_chain(*args, stream)
+            torch.cuda.synchronize()
+            assert time.monotonic() - t0 < 0.5                         # (not the others' second)
+            assert [w.status() for w in members] == [B.TT_ERR_TIMEOUT] * len(members)
+            wl.test_stall(0)
+            members[(i + 1) % len(members)].set_wait_limit(1_000_000_000)
+            for y in outs:
+                y.fill_(float("nan"))
+            B.run_chain(*args, stream)
+            assert [w.status() for w in members] == [B.TT_OK] * len(members)
+            assert all(torch.equal(y, r) for y, r in zip(outs, right))
+    for wl in wls:
+        wl.close()
+
+
 @pytest.mark.parametrize("spec", [
     W._dense(130, 421, 295, act=B.TT_ACT_RELU, name="raw_dense_421"),
     W._dense(3, 7, 6, name="raw_dense_too_few_rows"),
