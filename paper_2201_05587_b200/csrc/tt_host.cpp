@@ -271,7 +271,13 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     return TT_OK;
 }
 
-static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, bool boxes, Plan* plan) {
+// What a plan may do beside what its record says, as long as there is room for it.
+struct PlanOptions {
+    bool boxes;                                          // ragged rows come by TMA, in boxes of groups of four
+    bool fewer_splits;                                   // splits that are not resident at once are fewer
+};
+
+static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, PlanOptions may, Plan* plan) {
     // nonsense is refused whatever the kernel and the reduction order
     if (rec->tile_m <= 0 || rec->tile_n <= 0 || rec->tile_k <= 0 || rec->stages <= 0 || rec->split_k <= 0 ||
         rec->raster < 0 || rec->raster > 1 || rec->mma_m_axis < 0 || rec->mma_m_axis > 2 || rec->persistent < 0 ||
@@ -373,7 +379,7 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         if (strict) return TT_ERR_INVALID_SCHEDULE;
         sk = k_tiles;
     }
-    if (!strict && !persistent && !x3 && sk >= 2 && sk <= 8 && rec->ctas_per_sm != 2) {
+    if (may.fewer_splits && !strict && !persistent && !x3 && sk >= 2 && sk <= 8 && rec->ctas_per_sm != 2) {
         // The splits of a tile are a cluster, and a cluster keeps to one group of SMs: where the record's splits of all tiles are not
         // resident at once, fewer of them may take fewer rounds.  36 tiles of 64 columns in fours, of which 33 are resident, take two
         // rounds of a quarter of the reduction, in threes one round of a third (533 x 464 over 4096: 28.7 -> 20.5 us; as written in eighths 32.8;
@@ -579,9 +585,9 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
         return ((chunk_channels(tiles) * chp + sl_gap + 4) * 4 + 127) / 128 * 128;
     };
     // Operands whose rows are no 16-byte multiples: boxes of groups of four rows, beside the stages that they are realigned into
-    // (`boxes`: unless the plan has no room for them; fewer than four rows make no group).
+    // (unless the plan has no room for them; fewer than four rows make no group).
     const int x_rows = w->op == TT_OP_DENSE ? s.m : B * s.m, w_rows = w->op == TT_OP_DENSE ? s.nn : B * s.nn;
-    const bool ragged = boxes && w->op != TT_OP_CONV2D && (K % 4) != 0;
+    const bool ragged = may.boxes && w->op != TT_OP_CONV2D && (K % 4) != 0;
     const bool x_raw = ragged && x_rows >= 4, w_raw = ragged && w_rows >= 4 && (w->op == TT_OP_DENSE || w->sh.trans_b);
     const unsigned a_box = (swap ? w_raw : x_raw) ? (unsigned)round_up((tk + 4) * 4 * (kHwTileM / 4), 128) : 0u;
     const unsigned b_box = (swap ? x_raw : w_raw) ? (unsigned)round_up((tk + 4) * 4 * (tn / 4), 128) : 0u;
@@ -760,17 +766,25 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
 // 27.5 -> 24.1, which the wider grid's share of idle SMs makes a gamble on other sizes; at 1.4-1.5 30.5 -> 50.7 and 23.4 -> 38.1.
 static tt_status legalise_gemm(const tt_workload* w, const tt_schedule_record* rec, int mode, Plan* plan) {
     const Plan fresh = *plan;
-    tt_status s = plan_gemm(w, rec, mode, true, plan);
+    // Whether a record is valid is decided with its own splits; ragged rows are gathered value by value where there is no room for their boxes.
+    PlanOptions may{true, false};
+    tt_status s = plan_gemm(w, rec, mode, may, plan);
     if (s != TT_OK && w->op != TT_OP_CONV2D && w->sh.kk % 4 != 0) {
-        // (ragged rows and no room for their boxes: gathered value by value)
+        may.boxes = false;
         *plan = fresh;
-        s = plan_gemm(w, rec, mode, false, plan);
+        s = plan_gemm(w, rec, mode, may, plan);
+    }
+    if (s == TT_OK && plan->g.cluster && (long long)plan->info.grid_x * plan->gbatch > kResidentClusters[plan->g.cluster]) {
+        // fewer splits have a longer reduction each, whose table of a convolution may not fit: then the record's own stay
+        may.fewer_splits = true;
+        Plan fewer = fresh;
+        if (plan_gemm(w, rec, mode, may, &fewer) == TT_OK) *plan = fewer;
     }
     if (s != TT_OK || !plan->g.x3 || mode == TT_MODE_STRICT) return s;
     const int changed = plan->info.changed;
     auto replan = [&](const tt_schedule_record& r, bool same_splits) {
         Plan p = fresh;
-        if (plan_gemm(w, &r, TT_MODE_LEGALISE, true, &p) != TT_OK || p.info.legal.stages < std::min(2, p.g.k_tiles_per_split) ||
+        if (plan_gemm(w, &r, TT_MODE_LEGALISE, {true, true}, &p) != TT_OK || p.info.legal.stages < std::min(2, p.g.k_tiles_per_split) ||
             (same_splits && p.info.legal.split_k != plan->info.legal.split_k)) return;
         const tt_schedule_record& L = p.info.legal;
         p.info.changed = changed & ~(TT_CHG_TILE_N | TT_CHG_TILE_K | TT_CHG_STAGES | TT_CHG_SPLIT_K);

@@ -1,5 +1,6 @@
 """Host logic of the library (no GPU): ABI exports, workloads, classes, legaliser/validator, selector."""
 import ctypes
+import itertools
 import os
 import re
 
@@ -1009,3 +1010,25 @@ def test_tiles_and_splits_follow_the_rounds_of_the_sms(m, k, n, rec, tile_n, spl
     st, info = wl.check(r, mode=B.TT_MODE_STRICT)
     assert st == B.TT_OK and (info.legal.tile_n, info.legal.split_k) == (r.tile_n, r.split_k)
     wl.close()
+
+
+def test_what_runs_as_written_is_not_refused_when_it_may_be_laid_out():
+    """A rule that lays a record out otherwise gives way where its plan does not fit: whatever strict mode accepts, legalising accepts,
+    and the record's own splits then stay.  Wide 5x5 and 7x7 convolutions, whose table of the reduction is the longest."""
+    wide = W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(16, 2048, 13, 13, 256, 5, 5, 1, 2, True, B.TT_ACT_RELU), 1, "wide", "he").workload()
+    st, info = wide.check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=64, tile_k=64, stages=2, split_k=8, mma_m_axis=2))
+    assert st == B.TT_OK and info.legal.split_k == 8 and not info.changed & B.TT_CHG_SPLIT_K
+    wide.close()
+    accepted = 0
+    shapes = [W._conv(2048, 13, 256, 5, 1, 2), W._conv(1228, 29, 908, 7, 1, 3), W._conv(185, 31, 190, 1, 1, 0), W._dense(533, 4096, 464), W._dense(70, 8190, 1001)]
+    for spec, n in itertools.product(shapes, (1, 16, 28)):
+        if spec.op == B.TT_OP_CONV2D:
+            spec.shapes.n = n
+        wl = spec.workload()
+        for tn, tk, st_, sk, axis, sl in itertools.product((16, 64, 96, 128, 256), (16, 64, 128), (1, 2, 6), (3, 6, 8), (1, 2), (0, 2)):
+            rec = B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tn, tile_k=tk, stages=st_, split_k=sk, mma_m_axis=axis, slab_tiles=sl if spec.op == B.TT_OP_CONV2D else 0)
+            if wl.check(rec, mode=B.TT_MODE_STRICT)[0] == B.TT_OK:
+                accepted += 1
+                assert wl.check(rec)[0] == B.TT_OK, (spec.name, n, rec.short())
+        wl.close()
+    assert accepted > 1000
