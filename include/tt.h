@@ -309,6 +309,9 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
 /* How many kernels that pass launches: layers may go to the device together (see above), a layer under a record with a filter
  * re-pack takes two. */
 tt_status tt_chain_launches(const tt_chain_step* steps, size_t n_steps, size_t* launches);
+/* How many bytes of the weights of the layers behind it the launch that begins with each layer brings into the L2 (0 for the others):
+ * in passes whose layers share launches, whole layers of up to three launches, 10 MB at most.  bytes has n_steps entries. */
+tt_status tt_chain_ahead(const tt_chain_step* steps, size_t n_steps, size_t* bytes);
 /* tt_run with HOST pointers: copies x, w, bias, residual to library-owned device buffers, runs, copies y back,
  * synchronises.  bytes_h2d/bytes_d2h (may be NULL) receive the bytes copied. */
 tt_status tt_run_host(tt_workload* w, const tt_tensors* host, void* cuda_stream, int64_t* bytes_h2d, int64_t* bytes_d2h);

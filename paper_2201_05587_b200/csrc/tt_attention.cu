@@ -57,13 +57,14 @@ __device__ __forceinline__ void attn_read(uint32_t col, uint32_t pitch, int accs
     tmem_wait_ld();
 #pragma unroll
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-    if (!ANY) return;
+    if constexpr (ANY) {
 #pragma unroll 1
-    for (int a = 1; a < accs; ++a) {
-        tmem_ld32(col + (uint32_t)a * pitch, r);
-        tmem_wait_ld();
+        for (int a = 1; a < accs; ++a) {
+            tmem_ld32(col + (uint32_t)a * pitch, r);
+            tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] += __uint_as_float(r[j]);
+            for (int j = 0; j < 32; ++j) v[j] += __uint_as_float(r[j]);
+        }
     }
 }
 

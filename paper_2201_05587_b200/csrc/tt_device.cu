@@ -702,6 +702,8 @@ struct ChainLaunch {
     Ahead ahead;
 };
 
+constexpr size_t kAheadBytes = 10u << 20;                // weights that a launch asks for ahead, at most
+
 struct Range { const char* p; size_t bytes; };
 static bool overlap(const Range& a, const Range& b) { return a.p && b.p && a.p < b.p + b.bytes && b.p < a.p + a.bytes; }
 // x, w, bias, residual, y of a layer
@@ -865,13 +867,58 @@ static tt_status launch_chain_attention(const tt_chain_step* s, const AttnArgs& 
     return TT_OK;
 }
 
+// The launches of a pass, on the lanes of their first layers, and what they bring into the L2.  Whether layers share any: then all
+// dense layers take the chain build.
+static bool plan_launches(const tt_chain_step* steps, size_t n_steps, std::vector<ChainLaunch>& plan) {
+    bool shared = false;
+    plan.reserve(n_steps);
+    for (size_t i = 0; i < n_steps;) {
+        bool attention = false;
+        const int count = together_at(steps, n_steps, i, &attention);
+        ChainLaunch l{i, count, attention, steps[i].lane, false, false, Ahead{}};
+        for (int m = 0; m < l.count; ++m) l.moved = l.moved || steps[i + (size_t)m].lane != l.lane;
+        shared = shared || count > 1;
+        plan.push_back(l);
+        i += (size_t)l.count;
+    }
+    // In a pass with shared launches, a dense or attention launch whose CTAs are resident at once brings the weights of the launches up to
+    // three behind it into the L2 while it runs: whole layers, kAheadBytes in all.  12-layer encoder, 64 tokens 332 -> 320 us, 128 tokens
+    // 386 -> 381, 256 tokens 535 -> 527, as much as with 24 MB.  Not more, because weights that the L2 does not keep are read twice (two
+    // times 768 -> 768 -> 4096 -> 16384 -> 768 on one row: 202 us with whatever came next, 142 with 24 MB, 136 without), and not in
+    // other passes, whose layers it slows by 1 to 6 % at every size (32 times 1024 -> 1024 on 32 rows: 137 us without, 143 with).
+    for (size_t l = 0, next = 0; shared && l < plan.size(); ++l) {
+        next = std::max(next, l + 1);
+        const tt_chain_step& from = steps[plan[l].first];
+        if (!plan[l].attention) {
+            if (!usable(from) || !chain_form(from.workload, from.workload->plan)) continue;
+            const tt_apply_info& I = (plan[l].count > 1 ? from.workload->group[plan[l].count - 2] : from.workload->plan).info;
+            if ((long long)I.grid_x * I.grid_y * plan[l].count > kSms) continue;
+        }
+        int n = 0;
+        for (size_t bytes = 0; n < 3 && next < plan.size() && next <= l + 3; ++next) {
+            const ChainLaunch& c = plan[next];
+            const tt_chain_step& s = steps[c.first];
+            if (c.attention || !usable(s) || (s.workload->op != TT_OP_DENSE && s.workload->op != TT_OP_CONV2D) || s.workload->plan.repack) continue;
+            if (n + c.count > 3) break;
+            for (int m = 0; m < c.count; ++m) {
+                const Range w = range_of(steps[c.first + (size_t)m], 1);
+                const size_t skip = (16 - reinterpret_cast<uintptr_t>(w.p)) & 15u;
+                if (w.bytes < skip + 16 || bytes + w.bytes > kAheadBytes) continue;
+                plan[l].ahead.p[n] = w.p + skip; plan[l].ahead.bytes[n++] = (unsigned)(w.bytes - skip) & ~15u;
+                bytes += w.bytes;
+            }
+        }
+    }
+    return shared;
+}
+
 tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* streams, size_t n_streams, size_t* failed_at) try {
     if (!steps || n_steps == 0 || !streams || n_streams == 0) return TT_ERR_INVALID_ARG;
     constexpr size_t kNone = ~(size_t)0;
     std::vector<ChainLaunch> plan;
     std::vector<size_t> launch_of(n_steps), waits, first_wait, tail(n_streams, kNone);
     std::vector<char> used(n_streams, 0);
-    plan.reserve(n_steps); waits.reserve(n_steps); first_wait.reserve(n_steps + 1);
+    waits.reserve(n_steps); first_wait.reserve(n_steps + 1);
     for (size_t i = 0; i < n_steps; ++i) {
         const tt_chain_step& s = steps[i];
         if (failed_at) *failed_at = i;
@@ -879,15 +926,9 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
         for (int32_t j = 0; j < s.n_waits; ++j)
             if (s.waits[j] < 0 || (size_t)s.waits[j] >= i) return TT_ERR_INVALID_ARG;
     }
-    // which layers go to the device together: the launches, on the lanes of their first layers
-    for (size_t i = 0; i < n_steps;) {
-        bool attention = false;
-        const int count = together_at(steps, n_steps, i, &attention);
-        ChainLaunch l{i, count, attention, steps[i].lane, false, false, Ahead{}};
-        for (int m = 0; m < l.count; ++m) { launch_of[i + (size_t)m] = plan.size(); l.moved = l.moved || steps[i + (size_t)m].lane != l.lane; }
-        plan.push_back(l);
-        i += (size_t)l.count;
-    }
+    const bool chained = plan_launches(steps, n_steps, plan);
+    for (size_t l = 0; l < plan.size(); ++l)
+        for (int m = 0; m < plan[l].count; ++m) launch_of[plan[l].first + (size_t)m] = l;
     // What a launch waits for: the launches of the layers its layers name, the last launch of each of its layers' lanes where that
     // went to another one, and, where it shares scratch (re-packed filters, partial sums and arrival counters) with an earlier
     // launch of the same workload, that one.
@@ -919,30 +960,6 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
         }
         first_wait.push_back(waits.size());
         for (size_t k = 1; k < n_streams; ++k) if (tail[k] != kNone && plan[tail[k]].lane != (int32_t)k) plan[tail[k]].needed = true;
-    }
-    // A dense or attention launch brings the weights of the launches up to three behind it into the L2 while it runs: at batch 1 a layer is over before
-    // its weights could have come from memory at anything like the memory's rate (the 12-layer encoder on 128 tokens 436 -> 430 us, two
-    // of its layers with a cold L2 82 -> 80).
-    bool chained = false;
-    for (size_t l = 0, next = 0; l < plan.size(); ++l) {
-        next = std::max(next, l + 1);
-        const tt_chain_step& from = steps[plan[l].first];
-        if (!plan[l].attention && (!usable(from) || !chain_form(from.workload, from.workload->plan))) continue;
-        int n = 0;
-        for (unsigned bytes = 0; n < 3 && next < plan.size() && next <= l + 3; ++next) {
-            const ChainLaunch& c = plan[next];
-            const tt_chain_step& s = steps[c.first];
-            if (c.attention || !usable(s) || (s.workload->op != TT_OP_DENSE && s.workload->op != TT_OP_CONV2D) || s.workload->plan.repack) continue;
-            if (n + c.count > 3 || bytes > (24u << 20)) break;
-            for (int m = 0; m < c.count; ++m) {
-                const Range w = range_of(steps[c.first + (size_t)m], 1);
-                const size_t skip = (16 - reinterpret_cast<uintptr_t>(w.p)) & 15u;
-                if (w.bytes < skip + 16 || w.bytes > (1u << 30)) continue;
-                plan[l].ahead.p[n] = w.p + skip; plan[l].ahead.bytes[n++] = (unsigned)(w.bytes - skip) & ~15u;
-                bytes += (unsigned)w.bytes;
-            }
-        }
-        chained = chained || n > 0 || plan[l].count > 1;
     }
     EventLoan events(plan.size() + 2 * n_streams + 2);   // (nothing below allocates once the pass is being enqueued)
     std::vector<cudaEvent_t> done(plan.size(), nullptr);
@@ -1007,20 +1024,39 @@ tt_status tt_run_chain(const tt_chain_step* steps, size_t n_steps, void* const* 
     return rc;
 } TT_NO_THROW
 
-tt_status tt_chain_launches(const tt_chain_step* steps, size_t n_steps, size_t* launches) {
-    if (!steps || n_steps == 0 || !launches) return TT_ERR_INVALID_ARG;
-    *launches = 0;
-    for (size_t i = 0; i < n_steps;) {
+// (the arguments of the two functions below)
+static tt_status check_chain(const tt_chain_step* steps, size_t n_steps) {
+    if (!steps || n_steps == 0) return TT_ERR_INVALID_ARG;
+    for (size_t i = 0; i < n_steps; ++i) {
         const tt_chain_step& s = steps[i];
         if (!s.workload || !s.workload->plan.applied) return TT_ERR_NOT_APPLIED;
         for (int32_t j = 0; j < s.n_waits; ++j) if (!s.waits || s.waits[j] < 0 || (size_t)s.waits[j] >= i) return TT_ERR_INVALID_ARG;
+    }
+    return TT_OK;
+}
+
+tt_status tt_chain_launches(const tt_chain_step* steps, size_t n_steps, size_t* launches) {
+    const tt_status st = launches ? check_chain(steps, n_steps) : TT_ERR_INVALID_ARG;
+    if (st != TT_OK) return st;
+    *launches = 0;
+    for (size_t i = 0; i < n_steps;) {
         bool attention = false;
         const int count = together_at(steps, n_steps, i, &attention);
-        *launches += attention ? 1 : (size_t)s.workload->plan.info.launches;
+        *launches += attention ? 1 : (size_t)steps[i].workload->plan.info.launches;
         i += (size_t)count;
     }
     return TT_OK;
 }
+
+tt_status tt_chain_ahead(const tt_chain_step* steps, size_t n_steps, size_t* bytes) try {
+    const tt_status st = bytes ? check_chain(steps, n_steps) : TT_ERR_INVALID_ARG;
+    if (st != TT_OK) return st;
+    std::vector<ChainLaunch> plan;
+    plan_launches(steps, n_steps, plan);
+    std::fill(bytes, bytes + n_steps, (size_t)0);
+    for (const ChainLaunch& l : plan) for (const unsigned b : l.ahead.bytes) bytes[l.first] += b;
+    return TT_OK;
+} TT_NO_THROW
 
 tt_status tt_workload_set_constant_weights(tt_workload* w, int32_t on) {
     if (!w) return TT_ERR_INVALID_ARG;

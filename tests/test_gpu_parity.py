@@ -1618,6 +1618,41 @@ def test_a_wait_that_gives_up_in_a_shared_launch_is_reported_by_every_layer():
         wl.close()
 
 
+def test_what_a_pass_brings_into_the_l2_ahead_is_bounded():
+    """An encoder's launches ask for the weights behind them, whole layers of 10 MB in all at most, whatever the next layers' sizes; a
+    pass of single layers asks for nothing; results are those of the layers one by one."""
+    import types
+    import torch
+    stream = [torch.cuda.current_stream()]
+
+    def wired(specs, steps):
+        wls = [sp.workload() for sp in specs]
+        for wl in wls:
+            wl.apply(tc(tile_n=64, tile_k=64, stages=2, split_k=2) if wl.family() == B.TT_FAMILY_GEMM_TC else wl.default_schedule())
+        bufs, tts = W.chain_device_tensors(steps, W.make_chain_inputs(steps, 3, init="bert"))
+        plan = [None if st.spec is None else (0, ()) for st in steps]
+        ahead = B.chain_ahead(wls, steps, tts, plan)
+        W.run_chain(wls, steps, tts, plan, stream)
+        got = [b["y"].clone() for b in bufs]
+        for st, tt in zip(steps, tts):
+            if tt is not None:
+                wls[st.kernel].run(tt)
+        assert all(torch.equal(b["y"], y) for b, y in zip(bufs, got)) and all(wl.status() == B.TT_OK for wl in wls)
+        for wl in wls:
+            wl.close()
+        return ahead
+
+    limit = 10 << 20
+    for hidden, ffn in ((768, 3072), (256, 70000), (512, 2500)):          # projections and what comes behind: 2.4 + 9.4, 0.3 + 72, 1 + 5.1 MB
+        ahead = wired(*W.bert_base_net(seq=64, hidden=hidden, heads=hidden // 64, ffn=ffn, layers=2))
+        assert 0 < max(ahead) <= limit, (hidden, ffn, ahead)
+    net = W.Net()
+    cur = net.external((3, 256), "rows")
+    for a, b in ((256, 256), (256, 40000), (40000, 256)):
+        cur = net.add(W._dense(3, a, b, init="bert", name=f"d{a}_{b}"), x=cur)
+    assert not any(wired(*net.finish()))
+
+
 @pytest.mark.parametrize("spec", [
     W._dense(130, 421, 295, act=B.TT_ACT_RELU, name="raw_dense_421"),
     W._dense(3, 7, 6, name="raw_dense_too_few_rows"),
