@@ -19,9 +19,12 @@
  *   - Tensor pointers in tt_tensors are DEVICE pointers owned by the caller, fp32,
  *     dense row-major in the layouts stated at tt_op; they are borrowed for the
  *     call and never retained.  tt_run_host takes HOST pointers instead.
- *   - The only device memory the library owns is a per-workload workspace (split-K
- *     partial sums and a status word), allocated by tt_schedule_apply and released
- *     by tt_workload_destroy or the next apply.
+ *   - The only device memory the library owns is per workload: scratch (workspace_bytes,
+ *     exchange_kib: split-K partial sums, re-packed filters, what CTAs exchange), a
+ *     convolution's reduction-index table and a status word, allocated by
+ *     tt_schedule_apply and released by tt_workload_destroy or when a later apply needs
+ *     more; copies of the re-packed filters (tt_workload_set_constant_weights); and the
+ *     staging buffers of tt_run_host.
  *   - Launches are asynchronous on the given CUDA stream (a cudaStream_t passed as
  *     void*; NULL is the default stream).  tt_time, tt_transfer_tune, tt_grid_tune
  *     and tt_run_host synchronise that stream before returning.
@@ -189,8 +192,10 @@ typedef struct tt_apply_info {
     int32_t smem_bytes;         /* dynamic shared memory per CTA that the legal record needs; a launch of the one-tile GEMM
                                    form takes what is left over as well, for more stages */
     int32_t tmem_cols;
-    int64_t workspace_bytes;
+    int64_t workspace_bytes;    /* device scratch of a run: split-K partial sums and counters, or re-packed filters */
     int32_t launches;           /* kernels per tt_run (2 with the filter re-pack of k_order = 1) */
+    int32_t exchange_kib;       /* device scratch beside workspace_bytes, in KiB: what the CTAs of a k_order = 1 record's clusters leave
+                                   to one another */
 } tt_apply_info;
 
 enum { TT_CHG_TILE_M = 1, TT_CHG_TILE_N = 2, TT_CHG_TILE_K = 4, TT_CHG_STAGES = 8, TT_CHG_SPLIT_K = 16,

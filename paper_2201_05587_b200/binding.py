@@ -79,7 +79,7 @@ class tt_gemm_view(C.Structure):
 class tt_apply_info(C.Structure):
     _fields_ = [("legal", tt_schedule_record), ("changed", i32), ("grid_x", i32), ("grid_y", i32), ("grid_z", i32),
                 ("threads", i32), ("smem_bytes", i32), ("tmem_cols", i32), ("workspace_bytes", C.c_int64),
-                ("launches", i32)]
+                ("launches", i32), ("exchange_kib", i32)]
 
 
 class tt_timing_opts(C.Structure):

@@ -244,11 +244,12 @@ tt_status bind_device(tt_workload* w) try {
         if (cudaMalloc(&w->workspace, need) != cudaSuccess) { cudaGetLastError(); return TT_ERR_OOM; }
         w->workspace_bytes = need;
     }
-    if ((size_t)w->plan.exchange_bytes > w->exchange_bytes) {
+    const size_t exchange = (size_t)w->plan.info.exchange_kib * 1024;
+    if (exchange > w->exchange_bytes) {
         if (w->exchange) cudaFree(w->exchange);
         w->exchange = nullptr; w->exchange_bytes = 0;
-        if (cudaMalloc(&w->exchange, (size_t)w->plan.exchange_bytes) != cudaSuccess) { cudaGetLastError(); return TT_ERR_OOM; }
-        w->exchange_bytes = (size_t)w->plan.exchange_bytes;
+        if (cudaMalloc(&w->exchange, exchange) != cudaSuccess) { cudaGetLastError(); return TT_ERR_OOM; }
+        w->exchange_bytes = exchange;
     }
     if (need > 0 && !w->plan.repack) {
         // arrival counters start at zero; each launch leaves them at zero again

@@ -239,7 +239,7 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     I.smem_bytes = (int)std::min<long long>(std::max<long long>(smem, 116 * 1024), 0x7fffffff);     // one CTA per SM
     I.tmem_cols = tmem_cols;
     I.workspace_bytes = (int64_t)M * K * 4;              // the re-packed filters
-    plan->exchange_bytes = split > 1 ? tiles * split * ((tn + 31) / 32) * 4 * 4096 : 0;      // a block per CTA, 32 columns and lane quadrant
+    I.exchange_kib = (int32_t)(split > 1 ? tiles * split * ((tn + 31) / 32) * 16 : 0);   // 4 KiB per CTA, 32 columns and lane quadrant
     I.launches = 2;
     if (smem > kDynSmemLimit) return TT_ERR_RESOURCE;
     plan->swap_ab = false;

@@ -205,7 +205,6 @@ struct Plan {
     GemmArgs g{};
     long long partial_bytes = 0;      // counters start here inside the workspace
     int run_smem = 0;                 // one-tile GEMM: shared memory of a launch (the ring may be deeper than the record's)
-    long long exchange_bytes = 0;     // tap-major convolution by clusters: what their CTAs leave to one another (scratch beside the filters)
     bool repack = false;              // tap-major convolution: pm applies, filters are re-packed into the workspace
     ConvPmArgs pm{};
     DwArgs dw{};

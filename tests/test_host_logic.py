@@ -1032,3 +1032,18 @@ def test_what_runs_as_written_is_not_refused_when_it_may_be_laid_out():
                 assert wl.check(rec)[0] == B.TT_OK, (spec.name, n, rec.short())
         wl.close()
     assert accepted > 1000
+
+
+def test_the_scratch_that_clusters_exchange_through_is_reported():
+    """A tap-major record in clusters has, beside the re-packed filters, scratch for every CTA's accumulator in whole blocks of 32 columns;
+    one without clusters has the filters alone."""
+    wl = W.Spec(B.TT_OP_CONV2D, B.conv2d_shapes(32, 512, 7, 7, 512, 3, 3, 1, 1, True, B.TT_ACT_RELU, True), 1, "c", "he").workload()
+    for tile_n, cluster in ((224, 1), (224, 3), (256, 4), (144, 2)):
+        rec = B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tile_n, tile_k=32, stages=4, k_order=1, mma_m_axis=1, persistent=1, cta_group=cluster)
+        st, info = wl.check(rec, mode=B.TT_MODE_STRICT)
+        assert st == B.TT_OK and info.legal.cta_group == cluster and info.grid_y == cluster
+        assert info.workspace_bytes == 512 * 512 * 9 * 4
+        assert info.exchange_kib * 1024 == (info.grid_x * cluster * -(-tile_n // 32) * 128 * 32 * 4 if cluster > 1 else 0)
+    wl.close()
+    st, info = W._dense(128, 768, 768).workload().check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=64, tile_k=64, stages=2, split_k=4, mma_m_axis=2))
+    assert st == B.TT_OK and info.exchange_kib == 0
