@@ -2537,7 +2537,8 @@ __global__ void __launch_bounds__(cached_threads(NV)) tt_softmax_cached_kernel(c
 }
 
 // ROW_SIMT for ragged rows (the length is no multiple of 4, so rows begin anywhere inside a 16-byte group): a warp owns
-// `chunk` consecutive rows, a multiple of four, whose bytes therefore begin on a 16-byte boundary and fill whole groups.
+// `chunk` consecutive rows, whose values are a multiple of four (even rows in twos, others in fours), so that their bytes begin on a
+// 16-byte boundary and fill whole groups.
 // One bulk copy brings them to shared memory, the lanes read them value by value (NV per lane, kept in registers), write
 // the results over them, and one bulk copy takes them back: memory sees whole lines only.  Warps do not meet.
 // Next to memory the instructions per value bind (4-byte accesses; the exponential alone is half a dozen), so NV is the
@@ -2637,9 +2638,12 @@ __global__ void tt_floor_kernel() {
 static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <= 112 * 1024 && tmem_cols <= 256; }
 
 typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs, const ChainParam<false>);
-#define TT_GEMM_FORMS(CTAS, CL) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>, tt_gemm_tc_kernel<CTAS, kFormX3Tmem, CL>, \
-    tt_gemm_tc_kernel<CTAS, kFormIm2colRun, CL>}
-static const GemmKernel kGemmKernels[2][2][7] = {{TT_GEMM_FORMS(1, false), TT_GEMM_FORMS(1, true)}, {TT_GEMM_FORMS(2, false), TT_GEMM_FORMS(2, true)}};
+// (compensated products from tensor memory have one CTA per SM)
+#define TT_GEMM_FORMS(CTAS, CL, X3_TMEM) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, \
+    tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>, X3_TMEM, tt_gemm_tc_kernel<CTAS, kFormIm2colRun, CL>}
+static const GemmKernel kGemmKernels[2][2][7] = {
+    {TT_GEMM_FORMS(1, false, (tt_gemm_tc_kernel<1, kFormX3Tmem, false>)), TT_GEMM_FORMS(1, true, (tt_gemm_tc_kernel<1, kFormX3Tmem, true>))},
+    {TT_GEMM_FORMS(2, false, nullptr), TT_GEMM_FORMS(2, true, nullptr)}};
 #undef TT_GEMM_FORMS
 
 static int gemm_form(const GemmArgs& g) {
