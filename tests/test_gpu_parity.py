@@ -957,6 +957,31 @@ def test_compensated_products_come_within_fp32_accumulation_of_the_exact_result(
         assert e3 <= 2e-5 and e3 * 20 <= e0, (spec.name, kw, e0, e3)
 
 
+@pytest.mark.parametrize("tile_k,stages", [(8, 4), (16, 4), (32, 3), (64, 2), (128, 1)])
+def test_compensated_products_from_few_buffers_of_tensor_memory(tile_k, stages):
+    """Long reductions, whose A is multiplied from tensor memory, in an odd number of tiles of every depth and swizzle.  From 64 on there
+    are fewer buffers than stages (3 for 4 with tiles of 32 columns, 1 for 2), which then wrap at different places."""
+    spec = W._dense(150, 1060, 200, init="bert", name="x3_1060")
+    a = W.make_inputs(spec, 92)
+    ref = util.oracle_ref(spec, a)
+    for tile_n, axis in ((32, 1), (32, 2), (64, 1)):
+        if tile_k == 128 and tile_n == 64:
+            continue                                     # (no room for a stage)
+        y = run_spec(spec, tc(tile_n=tile_n, tile_k=tile_k, stages=stages, mma_m_axis=axis, precision=1), a, ref, mode=B.TT_MODE_STRICT)
+        assert util.rel_l2(y, ref) <= 2e-5, (tile_n, axis, util.rel_l2(y, ref))
+
+
+@pytest.mark.parametrize("tile_n", [96, 160, 224])
+def test_pairs_of_ctas_with_tiles_between_the_powers_of_two(tile_n):
+    """Widths that the columns of a persistent record are dealt in: a CTA of the pair loads 48, 80 or 112 rows of B.  Ragged rows and
+    columns, several tiles a pair."""
+    spec = W._dense(1301, 68, 2500, act=B.TT_ACT_RELU, name="pairs")
+    a = W.make_inputs(spec, 93)
+    ref = util.oracle_ref(spec, a)
+    for stages in (2, 4):
+        run_spec(spec, tc(tile_n=tile_n, tile_k=32, stages=stages, mma_m_axis=1, persistent=1, cta_group=2), a, ref, mode=B.TT_MODE_STRICT, ref_elem=elem_ref(spec, a, ref))
+
+
 @pytest.mark.parametrize("rows,cols", [(60001, 33), (150003, 5), (40001, 61), (19002, 198), (20003, 1174)])
 def test_softmax_of_many_short_ragged_rows(rows, cols):
     """Rows that come several passes at a time, and even ones in chunks of two rows; the last rows fill no whole chunk."""
