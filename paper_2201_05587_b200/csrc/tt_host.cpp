@@ -152,23 +152,24 @@ static tt_status legalise_conv_tapmajor(const tt_workload* w, const tt_schedule_
     // Where the record's tiles fill more than half of the SMs, columns are dealt evenly over the rounds that its tile needs: 121
     // tiles of 224 columns become 141 of 192; a tile with which they take fewer rounds replaces it where that is a tenth cheaper.
     // Where they fill less, CTAs share a tile's channel blocks as a cluster: as many as save the most cycles, as long as all
-    // clusters are resident at once (20 clusters of 7 are not: 320 -> 200 at 9 x 9, batch 6, 64 columns: 21.8 us, in clusters of 5
-    // 10.4); the widest tile replaces the record's where that is cheaper.
+    // clusters are resident at once (20 clusters of 7 are not: 320 -> 200 at 9 x 9, batch 6, 64 columns: 17.0 us, in clusters of 5
+    // 9.3); the widest tile replaces the record's where that is cheaper.
     // Cycles: a tap takes what its columns take the tensor core, 2 each, or what shared memory has to move in 128-byte lines, its
-    // filters in and out, 256, its columns, about 32 for the slab; the read-out 25 a column (192 columns: 2.3 us); the exchange in a
-    // cluster 1000 and 30 for every column that a CTA leaves to others, set so that these come out right: 3x3 64 -> 64 at 56 x 56, 192
-    // columns, 10.9 us alone and 9.9 in pairs; 1x1 64 -> 128 at 14 x 14, batch 8, 96 columns, 5.8 and 6.6; 3x3 512 -> 512 at 7 x 7,
-    // batch 32, weights cold, 25.8 with 128 columns in pairs and 25.1 with 256 in fours, which move half the filters.
-    // 23 layers under 7 records each: 1.50 times faster than as written in the geometric mean, 1.20 times the best of 15 widths and 8
-    // clusters, two pairs slower than as written (by 17 %).
+    // filters in and out, 256, its columns, about 32 for the slab; the read-out 30 a column; the exchange in a cluster 750 and 25 for every
+    // column that a CTA leaves to others.  Least squares over 27 layers under 15 widths and 8 clusters each give 29, 753 and 22 (and the
+    // taps' cycles a factor of 1.01).  3x3 64 -> 64 at 56 x 56, batch 4, 192 columns: 11.3 us alone, 10.1 in pairs; 1x1 64 -> 128 at
+    // 14 x 14, batch 8, 96 columns: 5.1 and 5.5; 1x1 512 -> 64 there, 256 columns: 29.9 and 11.6 in eights; 3x3 512 -> 512 at 7 x 7,
+    // batch 32: 22.7 with 128 columns in pairs, 22.2 with 256 in fours.
+    // Those layers under 7 records each: 1.81 times faster than as written without clusters in the geometric mean, 1.18 times the best of
+    // all widths and clusters; one pair slower than as written (by 4 %).
     const auto tiles_of = [&](int n) { return (long long)tiles_m * ((N + n - 1) / n); };
     struct Share { long long cycles; int ctas; };
     const auto share_of = [&](int n) {
         const long long tap = std::max(2 * n, n + 288);
-        Share best{CB * RS * tap + 25 * n, 1};
+        Share best{CB * RS * tap + 30 * n, 1};
         for (int k = 2; k <= std::min(8, CB); ++k) {
             if (tiles_of(n) > kResidentClusters[k]) continue;
-            const long long cycles = (CB + k - 1) / k * RS * tap + 25 * n + 1000 + 30 * n * (k - 1) / k;
+            const long long cycles = (CB + k - 1) / k * RS * tap + 30 * n + 750 + 25 * n * (k - 1) / k;
             if (cycles < best.cycles) best = Share{cycles, k};
         }
         return best;

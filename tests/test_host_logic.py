@@ -1047,3 +1047,14 @@ def test_the_scratch_that_clusters_exchange_through_is_reported():
     wl.close()
     st, info = W._dense(128, 768, 768).workload().check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=64, tile_k=64, stages=2, split_k=4, mma_m_axis=2))
     assert st == B.TT_OK and info.exchange_kib == 0
+
+
+def test_a_pointwise_layer_of_wide_tiles_is_shared_by_a_cluster():
+    """512 -> 64 channels, 1x1, 8 images of 14 x 14: seven tiles of 256 columns whose 16 channel blocks eight CTAs share (29.9 us by one
+    CTA each, 11.6 in eights); a tap of two blocks is not worth the exchange."""
+    rec = B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=256, tile_k=32, stages=8, mma_m_axis=1, k_order=1)
+    for c, k, cluster in ((512, 64, 8), (64, 128, 1)):
+        wl = B.Workload(B.TT_OP_CONV2D, B.conv2d_shapes(8, c, 14, 14, k, 1, 1, 1, 0, True, B.TT_ACT_RELU), "tap")
+        st, info = wl.check(rec)
+        assert st == B.TT_OK and info.legal.tile_n == 256 and info.legal.cta_group == cluster
+        wl.close()
