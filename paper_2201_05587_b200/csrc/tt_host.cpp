@@ -366,13 +366,18 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     if (persistent && !strict) {
         // Columns are dealt evenly over the rounds of the SMs that the record's tile needs, as long as those are few: 152 tiles of 256
         // columns are one full round and four tiles more, 240 of 160 are two rounds of little more than half the work (2419 x 1976 over 888:
-        // 36.0 -> 30.8 us, by pairs of CTAs 24.9 -> 22.3; 2000 x 1600 over 2000 from 128 columns 41.8 -> 39.4).
+        // 36.0 -> 30.8 us, by pairs of CTAs 24.9 -> 22.3; 2000 x 1600 over 2000 from 128 columns 41.8 -> 39.4).  Tiles narrower than 128
+        // columns move more operand bytes for each of their products, and a last round of few tiles is over soon: those records stay as
+        // they are below an eighth of a round (785 x 1160 over 384, 64 columns by pairs, 76 pairs' tiles: 14.3 us, 16.4 with 32; 3147 x 1352
+        // over 1592, 128 columns 54.6, 62.3 with 96).  150 records of other sizes: 1.043 times faster than as written in the geometric
+        // mean, six slower by more than 2 %; 1.041 and twenty without that line.
         const int per = kHwTileM * cg, step = cg == 2 || tn % 32 == 0 ? 32 : 16;
         const long long rows = (long long)((M + per - 1) / per) * B, units = kSms / cg;
-        const long long rounds = (rows * ((N + tn - 1) / tn) + units - 1) / units, columns = rounds * units / rows;
+        const long long tiles = rows * ((N + tn - 1) / tn), rounds = (tiles + units - 1) / units, columns = rounds * units / rows;
         if (rounds >= 2 && rounds <= 4) {
             const int even = round_up((int)((N + columns - 1) / columns), step);
-            if (even < tn) { tn = even; changed |= TT_CHG_TILE_N; L.tile_n = tn; }
+            const bool worth = even >= 128 || (tiles - (rounds - 1) * units) * 8 >= units;
+            if (even < tn && worth) { tn = even; changed |= TT_CHG_TILE_N; L.tile_n = tn; }
         }
     }
     int sk = persistent ? 1 : rec->split_k;

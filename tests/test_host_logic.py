@@ -1058,3 +1058,19 @@ def test_a_pointwise_layer_of_wide_tiles_is_shared_by_a_cluster():
         st, info = wl.check(rec)
         assert st == B.TT_OK and info.legal.tile_n == 256 and info.legal.cta_group == cluster
         wl.close()
+
+
+@pytest.mark.parametrize("m,k,n,rec,tile_n", [
+    (785, 384, 1160, dict(tile_n=64, tile_k=32, stages=2, mma_m_axis=1, cta_group=2), 64),           # 76 tiles for 74 pairs: 32 columns cost more
+    (3147, 1592, 1352, dict(tile_n=128, tile_k=32, stages=3, mma_m_axis=2, cta_group=2), 128),       # 150 for 74
+    (495, 1688, 3648, dict(tile_n=96, tile_k=32, stages=3, mma_m_axis=2, cta_group=2), 64),          # 90 for 74: the last round is a fifth full
+    (1160, 384, 4096, dict(tile_n=256, tile_k=32, stages=2, mma_m_axis=1), 160),                     # 160 for 148, wide tiles
+])
+def test_narrow_tiles_are_not_dealt_for_a_last_round_of_few(m, k, n, rec, tile_n):
+    """A record whose last round holds less than an eighth of the SMs keeps its columns, unless those that it would get are still 128."""
+    wl = W._dense(m, k, n).workload()
+    r = B.make_record(B.TT_FAMILY_GEMM_TC, persistent=1, **rec)
+    st, info = wl.check(r)
+    assert st == B.TT_OK and info.legal.tile_n == tile_n and bool(info.changed & B.TT_CHG_TILE_N) == (tile_n != r.tile_n)
+    _check_legal_says_what_runs(wl, [r])
+    wl.close()
