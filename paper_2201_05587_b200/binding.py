@@ -344,32 +344,20 @@ def run_chain(wls, steps, tts, plan, streams):
         raise TTError(st, f"tt_run({wls[steps[at].kernel].name})" if at >= 0 else "tt_run_chain")
 
 
-def _chain_steps(wls, steps, tts, plan):
-    """The layers of a chain as tt_chain_step, and the positions of their nodes."""
-    chain, position = [], {}
-    for i, (st, tt, pl) in enumerate(zip(steps, tts, plan)):
-        if pl is None:
-            continue
-        lane, waits = pl
-        position[i] = len(chain)
-        chain.append(tt_chain_step(wls[st.kernel].handle, C.pointer(tt), (i32 * max(len(waits), 1))(*[position[p] for p in waits]), len(waits), lane))
-    return (tt_chain_step * len(chain))(*chain), position
+def _query_chain(function, wls, steps, tts, plan):
+    st, values = _call.query_chain(wls, steps, tts, plan, C.cast(getattr(lib(), function), C.c_void_p).value)
+    _check(st, function)
+    return values
 
 
 def chain_launches(wls, steps, tts, plan):
     """How many kernels run_chain launches for these arguments (tt_chain_launches)."""
-    chain, _ = _chain_steps(wls, steps, tts, plan)
-    n = C.c_size_t()
-    _check(lib().tt_chain_launches(chain, len(chain), C.byref(n)), "tt_chain_launches")
-    return n.value
+    return sum(_query_chain("tt_chain_launches", wls, steps, tts, plan))
 
 
 def chain_ahead(wls, steps, tts, plan):
     """Per node, how many bytes of weights its launch brings into the L2 for the ones behind it (tt_chain_ahead)."""
-    chain, position = _chain_steps(wls, steps, tts, plan)
-    n = (C.c_size_t * len(chain))()
-    _check(lib().tt_chain_ahead(chain, len(chain), n), "tt_chain_ahead")
-    return [n[position[i]] if i in position else 0 for i in range(len(steps))]
+    return _query_chain("tt_chain_ahead", wls, steps, tts, plan)
 
 
 def _run_chain_over_devices(wls, steps, tts, plan, streams):
