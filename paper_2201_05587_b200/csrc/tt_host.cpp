@@ -665,8 +665,12 @@ static tt_status plan_gemm(const tt_workload* w, const tt_schedule_record* rec, 
     int depth = st;
     // A compensated CTA with a long reduction multiplies A and its remainders from tensor memory (the record is accounted for as if it
     // did not, so its ring may be deeper): 512 x 4096 -> 1024 in quarters 37.2 -> 29.9 us, 2000 x 1000 -> 3000 78.4 -> 73.3, 1024 x 1024 ->
-    // 1024 22.5 -> 20.6.  The way there takes longer, which short ones do not earn back: 36 x 520 -> 280 6.7 -> 7.4, 3 x 288 -> 1648 4.8 -> 6.4.
-    const bool x3_tmem = x3 && per_split * tk >= 512 && L.ctas_per_sm != 2;
+    // 1024 22.5 -> 20.6.  The way there takes longer, which short reductions do not earn back: 36 x 520 -> 280 6.7 -> 7.4, 3 x 288 -> 1648 4.8 ->
+    // 6.4.  Nor do stages with little in them: with 32 of the reduction it is 1.03 to 1.26 times faster for 128 to 176 columns, 0.97 to 1.01
+    // for 96 and 112, 0.77 to 0.87 up to 64 and 0.86 for 256; with 64 of the reduction 1.04 to 1.23 from 32 columns on and 0.83 for 16; with 16
+    // 0.64 to 0.88 for any.
+    const bool x3_stage = tk >= 64 ? tn >= 32 : tk == 32 && tn >= 128 && tn <= 176;
+    const bool x3_tmem = x3 && x3_stage && per_split * tk >= 512 && L.ctas_per_sm != 2;
     const long long run_stage = a_stage + b_stage + (x3_tmem ? b_stage : x3 ? (long long)a_stage + b_stage : 0);
     auto run_bytes = [&](int d) { return std::max<long long>(d * run_stage, min_pipe) + d * raw_stage + smem - pipe; };
     const long long ring_limit = L.ctas_per_sm == 2 ? smem : kDynSmemLimit;

@@ -1074,3 +1074,14 @@ def test_narrow_tiles_are_not_dealt_for_a_last_round_of_few(m, k, n, rec, tile_n
     assert st == B.TT_OK and info.legal.tile_n == tile_n and bool(info.changed & B.TT_CHG_TILE_N) == (tile_n != r.tile_n)
     _check_legal_says_what_runs(wl, [r])
     wl.close()
+
+
+@pytest.mark.parametrize("tile_n,tile_k,columns", [(64, 32, 64), (112, 32, 128), (128, 32, 512), (176, 32, 512), (192, 32, 256), (16, 64, 32), (32, 64, 512), (64, 64, 512), (128, 16, 128)])
+def test_compensated_products_take_tensor_memory_where_a_stage_is_worth_it(tile_n, tile_k, columns):
+    """Stages of 64 of the reduction from 32 columns on, of 32 between 128 and 176: the plan then asks for buffers behind the accumulator."""
+    wl = W._dense(300, 2048, 400).workload()
+    st, info = wl.check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=tile_n, tile_k=tile_k, stages=2, mma_m_axis=1, precision=1), mode=B.TT_MODE_STRICT)
+    assert st == B.TT_OK and info.tmem_cols == columns
+    st, info = W._dense(300, 480, 400).workload().check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=128, tile_k=32, stages=2, mma_m_axis=1, precision=1), mode=B.TT_MODE_STRICT)
+    assert st == B.TT_OK and info.tmem_cols == 128                 # a short reduction
+    wl.close()
