@@ -1124,13 +1124,17 @@ static tt_status legalise_row(const tt_workload* w, const tt_schedule_record* re
     I.threads = rpc * lanes; I.launches = 1;
     if ((s.nn & 3) != 0) {
         // Ragged rows pass through shared memory as long as a lane's values stay in registers and a warp's rows fit.  A chunk is a
-        // number of rows that fills whole 16-byte groups (two where rows are even, else four) and keeps all lanes busy, and short rows
-        // come several passes at a time, so that a copy is kRowRun bytes or more and a warp not gone after one pass (178560 rows of 33: 22.5 ->
-        // 18.4 us; 180600 of 77: 30.7 -> 24.6, of 1 KB at a time 30.7; 25908 of 1174 in twos 70.4 -> 59.4); warps per CTA
-        // follow the record, fewer where their rows or registers would not fit.  The lanes' accesses are single values.
-        const int per_lane = (s.nn + lanes - 1) / lanes;
-        int chunk = std::max(s.nn % 2 == 0 ? 2 : 4, 32 / lanes);
-        while (chunk * s.nn * 4 < kRowRun && rows / (2 * chunk) >= 32ll * kSms && 8ll * chunk * s.nn * (rpc * lanes / 32) <= kRowSmem) chunk *= 2;
+        // number of rows that fills whole 16-byte groups and keeps all lanes busy: four, or two of even rows where that is all a warp should
+        // have (14 KB and more in four: 30000 rows of 1174 74 -> 62 us; less than 14 chunks of four for each SM, of 1.5 KB and more: 3000 of
+        // 330 5.9 -> 4.7), or eight of short rows where there are still 54 chunks of them for each SM (100000 of 33 15.3 -> 11.9, 100000 of 130
+        // 22.1 -> 19.3; 30000 of 33, which are fewer, by 32 lanes 8.5 with four and 13.2 with eight).  159 combinations of length, rows and lanes: 1.062 times faster than four in the
+        // geometric mean, none slower by more than 2 %, and 1.6 % off the best of 2 to 64.  Warps per CTA follow the record, fewer where their
+        // rows or registers would not fit.  The lanes' accesses are single values.
+        const int per_lane = (s.nn + lanes - 1) / lanes, least = 32 / lanes;
+        int chunk = std::max(4, least);
+        const long long four = 16ll * s.nn, fours = rows / 4;
+        if (s.nn % 2 == 0 && (four > 14000 || (four >= 1500 && fours < 14 * kSms))) chunk = std::max(2, least);
+        else if (four < kRowRun && rows / 8 >= 54 * kSms && 32ll * s.nn * (rpc * lanes / 32) <= kRowSmem) chunk = std::max(8, least);
         const int warps = (int)std::min<long long>(std::min(rpc * lanes, ragged_threads(per_lane)) / 32, kRowSmem / ((long long)chunk * s.nn * 4));
         if (warps >= 1 && per_lane <= kRaggedMost && !(strict && (vec != 1 || warps * 32 != rpc * lanes))) {
             r.warps = warps; r.chunk = chunk;

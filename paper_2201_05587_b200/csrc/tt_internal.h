@@ -16,7 +16,7 @@ constexpr int kResidentClusters[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
 constexpr int kSmemLimit = 232448;      // 227 KB opt-in shared memory per CTA on sm_100
 constexpr int kDynSmemLimit = kSmemLimit - 6144;  // what is left for dynamic shared memory beside barriers
 constexpr int kRowSmem = 100 * 1024;    // shared memory of a CTA of the ragged softmax, so that two fit an SM
-constexpr int kRowRun = 2048;            // ... the bytes of short rows that a warp takes at once, at least
+constexpr int kRowRun = 3000;            // ... the bytes of four rows below which a warp may take eight
 constexpr int kRaggedMost = 65;         // ... and the values a lane of it keeps in registers at most
 constexpr int kCachedMost = 16;         // 16-byte groups a lane of the register-resident softmax keeps at most
 // Threads that their registers (both kernels are compiled for it) leave room for: values, or groups, per lane.

@@ -971,6 +971,16 @@ def test_compensated_products_over_an_odd_number_of_tiles(tile_n, tile_k, stages
         assert util.rel_l2(y, ref) <= 2e-5, (axis, util.rel_l2(y, ref))
 
 
+@pytest.mark.parametrize("rows,cols", [(70003, 33), (70001, 186), (300, 330), (299, 94), (303, 1174), (64000, 187)])
+def test_softmax_chunks_of_two_four_and_eight_rows(rows, cols):
+    """Both sides of the rule for a warp's rows, by few and many lanes; the last rows fill no whole chunk."""
+    spec = W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(1, rows, cols, scale=0.125), 1, f"softmax_{rows}x{cols}", "bert")
+    a = W.make_inputs(spec, 13)
+    ref = util.oracle_ref(spec, a)
+    for bx in (4, 16, 32):
+        run_spec(spec, B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=bx, block_y=8, vec_width=1), a, ref, ref_elem=ref)
+
+
 @pytest.mark.parametrize("tile_n", [96, 160, 224])
 def test_pairs_of_ctas_with_tiles_between_the_powers_of_two(tile_n):
     """Widths that the columns of a persistent record are dealt in: a CTA of the pair loads 48, 80 or 112 rows of B.  Ragged rows and

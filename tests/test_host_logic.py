@@ -1085,3 +1085,15 @@ def test_compensated_products_take_tensor_memory_where_a_stage_is_worth_it(tile_
     st, info = W._dense(300, 480, 400).workload().check(B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=128, tile_k=32, stages=2, mma_m_axis=1, precision=1), mode=B.TT_MODE_STRICT)
     assert st == B.TT_OK and info.tmem_cols == 128                 # a short reduction
     wl.close()
+
+
+@pytest.mark.parametrize("rows,cols,lanes,chunk", [
+    (100000, 33, 32, 8), (30000, 33, 32, 4), (100000, 187, 16, 8), (100000, 190, 16, 4),     # eight short rows, where there are many
+    (3000, 330, 16, 2), (3000, 330, 8, 4), (100000, 330, 16, 4), (3000, 46, 16, 4),          # two even ones, where there are few and they are long enough
+    (30000, 1174, 32, 2), (30000, 1175, 32, 4),                                              # ... or long
+])
+def test_rows_that_a_warp_of_the_ragged_softmax_takes(rows, cols, lanes, chunk):
+    wl = W.Spec(B.TT_OP_SOFTMAX, B.softmax_shapes(1, rows, cols, 1.0), 1, "s", "bert").workload()
+    st, info = wl.check(B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=lanes, block_y=4, vec_width=1))
+    assert st == B.TT_OK and info.smem_bytes == info.threads // 32 * chunk * cols * 4
+    wl.close()
