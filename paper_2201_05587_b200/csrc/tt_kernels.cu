@@ -482,7 +482,9 @@ enum GemmForm {
                         // MobileNetV2-shaped pass 256.5 us, 254.9 with one build)
     kFormX3 = 4,        // both K-major by TMA, error-compensated products, A and its remainders multiplied from shared memory ...
     kFormX3Tmem = 5,    // ... or from tensor memory
-    kFormGather = 3     // an operand gathered from global memory (the other one any way but by expansion)
+    kFormGather = 3,    // an operand gathered from global memory (the other one any way but by expansion)
+    kFormRaw = 7        // an operand of ragged rows by boxes (the other one any way but by expansion): its code in the form above cost short
+                        // launches there 0.2 to 0.5 us (132 heads of 21 x 64 over 21 4.4 us, 4.8 with it)
 };
 
 // CHAIN: a launch of a chained pass that does more than its layer (ChainArgs).
@@ -545,12 +547,12 @@ tt_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_cons
     const uint32_t stage_bytes = g.a_stage_bytes + g.b_stage_bytes + (x3 ? lo_off : 0u);
     // what the instantiation is made for (GemmForm); within it only the modes that its form leaves open are looked at
     constexpr bool slab_run = FORM == kFormIm2colRun, im2col = FORM == kFormIm2col || slab_run;
-    constexpr bool may_mn = FORM == kFormMn || FORM == kFormGather;
+    constexpr bool gathers = FORM == kFormGather || FORM == kFormRaw, may_mn = FORM == kFormMn || gathers;
     const bool a_mn = may_mn && g.a_mode == OPM_TMA_MN, b_mn = may_mn && g.b_mode == OPM_TMA_MN;
     const bool a_tma = FORM == kFormTma || x3 || FORM == kFormMn || g.a_mode == OPM_TMA || a_mn;
     const bool b_tma = FORM == kFormTma || x3 || FORM == kFormMn || g.b_mode == OPM_TMA || b_mn;
     const bool any_tma = a_tma || b_tma, any_gather = !a_tma || !b_tma;
-    const bool a_raw = FORM == kFormGather && g.a_mode == OPM_RAW, b_raw = FORM == kFormGather && g.b_mode == OPM_RAW;
+    const bool a_raw = FORM == kFormRaw && g.a_mode == OPM_RAW, b_raw = FORM == kFormRaw && g.b_mode == OPM_RAW;
     const bool any_raw = a_raw || b_raw;
     const int a_row0 = bz * g.M + m0, b_row0 = (g.b_tma_batched ? bz * g.N : 0) + n0;      // OPM_RAW: the tile's first row in the whole tensor
     const bool slab_tma = slab_run || (im2col && g.slab_tma != 0);
@@ -2640,8 +2642,9 @@ static bool gemm_two_per_sm(int smem_bytes, int tmem_cols) { return smem_bytes <
 typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs, const ChainParam<false>);
 // (compensated products from tensor memory have one CTA per SM)
 #define TT_GEMM_FORMS(CTAS, CL, X3_TMEM) {tt_gemm_tc_kernel<CTAS, kFormTma, CL>, tt_gemm_tc_kernel<CTAS, kFormMn, CL>, tt_gemm_tc_kernel<CTAS, kFormIm2col, CL>, \
-    tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>, X3_TMEM, tt_gemm_tc_kernel<CTAS, kFormIm2colRun, CL>}
-static const GemmKernel kGemmKernels[2][2][7] = {
+    tt_gemm_tc_kernel<CTAS, kFormGather, CL>, tt_gemm_tc_kernel<CTAS, kFormX3, CL>, X3_TMEM, tt_gemm_tc_kernel<CTAS, kFormIm2colRun, CL>, \
+    tt_gemm_tc_kernel<CTAS, kFormRaw, CL>}
+static const GemmKernel kGemmKernels[2][2][8] = {
     {TT_GEMM_FORMS(1, false, (tt_gemm_tc_kernel<1, kFormX3Tmem, false>)), TT_GEMM_FORMS(1, true, (tt_gemm_tc_kernel<1, kFormX3Tmem, true>))},
     {TT_GEMM_FORMS(2, false, nullptr), TT_GEMM_FORMS(2, true, nullptr)}};
 #undef TT_GEMM_FORMS
@@ -2650,14 +2653,14 @@ static int gemm_form(const GemmArgs& g) {
     if (g.x3) return g.x3_bufs > 0 ? kFormX3Tmem : kFormX3;
     if (g.a_mode == OPM_IM2COL || g.b_mode == OPM_IM2COL) return g.slab_tma == 2 ? kFormIm2colRun : kFormIm2col;
     const bool a = g.a_mode == OPM_TMA || g.a_mode == OPM_TMA_MN, b = g.b_mode == OPM_TMA || g.b_mode == OPM_TMA_MN;
-    if (!a || !b) return kFormGather;
+    if (!a || !b) return g.a_mode == OPM_RAW || g.b_mode == OPM_RAW ? kFormRaw : kFormGather;
     return g.a_mode == OPM_TMA && g.b_mode == OPM_TMA ? kFormTma : kFormMn;
 }
 
 // Which instantiation a plan runs; its shared-memory limit is raised once per device.  Which build (two CTAs per SM) is the
 // record's choice (ctas_per_sm), resolved by the legaliser.
 static cudaError_t gemm_kernel_for(const GemmArgs& g, int smem_bytes, GemmKernel* out) {
-    static OncePerDevice raised[2][2][7];
+    static OncePerDevice raised[2][2][8];
     const int two = g.two_per_sm && gemm_two_per_sm(smem_bytes, g.tmem_cols), form = gemm_form(g), cl = g.cluster > 0;
     *out = kGemmKernels[two][cl][form];
     return raised[two][cl][form]([&] { return cudaFuncSetAttribute(*out, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });

@@ -981,6 +981,16 @@ def test_softmax_chunks_of_two_four_and_eight_rows(rows, cols):
         run_spec(spec, B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=bx, block_y=8, vec_width=1), a, ref, ref_elem=ref)
 
 
+@pytest.mark.parametrize("k", [29, 31, 33])
+def test_ragged_rows_beside_a_gathered_operand(k):
+    """NN products whose x has ragged rows, on both sides of the reduction from which they come by TMA."""
+    spec = W.Spec(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(5, 45, 30, k, False), 1, f"nn_{k}", "bert")
+    a = W.make_inputs(spec, 18)
+    ref = util.oracle_ref(spec, a)
+    for axis in (1, 2):
+        run_spec(spec, tc(tile_n=32, tile_k=32, stages=2, mma_m_axis=axis), a, ref, ref_elem=elem_ref(spec, a, ref))
+
+
 @pytest.mark.parametrize("tile_n", [96, 160, 224])
 def test_pairs_of_ctas_with_tiles_between_the_powers_of_two(tile_n):
     """Widths that the columns of a persistent record are dealt in: a CTA of the pair loads 48, 80 or 112 rows of B.  Ragged rows and

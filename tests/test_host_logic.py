@@ -1097,3 +1097,17 @@ def test_rows_that_a_warp_of_the_ragged_softmax_takes(rows, cols, lanes, chunk):
     st, info = wl.check(B.make_record(B.TT_FAMILY_ROW_SIMT, block_x=lanes, block_y=4, vec_width=1))
     assert st == B.TT_OK and info.smem_bytes == info.threads // 32 * chunk * cols * 4
     wl.close()
+
+
+def test_short_reductions_beside_a_gathered_operand_come_without_boxes():
+    """Ragged rows of x in an NN product come by TMA from 33 of the reduction on; those of NT and dense products always do."""
+    rec = B.make_record(B.TT_FAMILY_GEMM_TC, tile_n=64, tile_k=32, stages=1, mma_m_axis=1)
+    for k, trans_b, boxes in ((31, False, 0), (33, False, 1), (31, True, 2)):
+        wl = B.Workload(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(4, 100, 64, k, trans_b), "b")
+        st, info = wl.check(rec)
+        plain = B.Workload(B.TT_OP_BATCH_MATMUL, B.bmm_shapes(4, 100, 64, 32 if k == 31 else 36, trans_b), "p")
+        st2, info2 = plain.check(rec)
+        box = lambda r: -(-36 * 4 * r // 128) * 128 * 4
+        assert st == st2 == B.TT_OK and info.smem_bytes - info2.smem_bytes == (0, box(32), box(32) + box(16))[boxes]
+        wl.close()
+        plain.close()
