@@ -29,16 +29,17 @@ constexpr int kAttnThreads = 512;
 constexpr int kAttnSoftmaxWarps = 4, kAttnStoreWarps = 10;
 constexpr uint32_t kAttnAtom = kAttnRows * 128u;         // bytes of a 32-column block of a tile of kAttnRows rows
 
-// Builds: FAR, more than 128 keys (two blocks of 32 a softmax warp); ANY, records of several accumulators, single values a lane or rows
-// of fewer than 16 lanes.  A launch meets a cold instruction cache, and what ANY adds costs it 0.5 us where nothing of it is run (the
-// 12-layer encoder on 128 tokens 385 -> 391 us, on 256 525 -> 531; without FAR 381).  80 or 128 registers and 512 threads: no CTA that
-// needs tensor memory, too, fits beside one that has not got its columns yet.
+// Builds: FAR, more than 128 keys (two blocks of 32 a softmax warp), and the order of the sums: rows of 16 or 32 lanes, of 8, or ORDER_ANY,
+// records of several accumulators, single values a lane or rows of 4 lanes too.  A launch meets a cold instruction cache, and code costs
+// it where nothing of it is run: 0.5 us what ORDER_ANY adds (the 12-layer encoder on 128 tokens 385 -> 391 us, on 256 525 -> 531), 0.3 FAR
+// (381).  80 or 128 registers and 512 threads: no CTA that needs tensor memory, too, fits beside one that has not got its columns yet.
+enum AttnOrder { ORDER_WIDE = 0, ORDER_EIGHT = 1, ORDER_ANY = 2 };
 
 // One product: its steps of 8 of the reduction go into the accumulators of its record, `pitch` columns apart: `per` steps to each in
 // turn (a record with splits), or dealt one by one (per = 0).
-template <bool ANY, typename Issue>
+template <int ORDER, typename Issue>
 __device__ __forceinline__ void attn_steps(uint32_t col, uint32_t pitch, int accs, int per, int steps, Issue issue) {
-    if (ANY && accs > 1) {
+    if (ORDER == ORDER_ANY && accs > 1) {
 #pragma unroll 1
         for (int a = 0; a < accs; ++a, col += pitch) {
             const int first = per > 0 ? a * per : a, end = per > 0 ? min(steps, first + per) : steps;
@@ -50,14 +51,14 @@ __device__ __forceinline__ void attn_steps(uint32_t col, uint32_t pitch, int acc
     for (int k8 = 0; k8 < steps; ++k8) issue(col, k8, k8 > 0 ? 1u : 0u);
 }
 // ... and 32 of its columns, read out in accumulator order.
-template <bool ANY>
+template <int ORDER>
 __device__ __forceinline__ void attn_read(uint32_t col, uint32_t pitch, int accs, float (&v)[32]) {
     uint32_t r[32];
     tmem_ld32(col, r);
     tmem_wait_ld();
 #pragma unroll
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-    if constexpr (ANY) {
+    if constexpr (ORDER == ORDER_ANY) {
 #pragma unroll 1
         for (int a = 1; a < accs; ++a) {
             tmem_ld32(col + (uint32_t)a * pitch, r);
@@ -70,21 +71,22 @@ __device__ __forceinline__ void attn_read(uint32_t col, uint32_t pitch, int accs
 
 // The sum of a row as 4 * m lanes come to it (m = 1, 2, 4, 8): lane l's share is the sum of values l, l + 4 m, ... of the line, the
 // shares are added in halves, l and l + 2 m first.  The line holds 8 groups of four values, or 16 (`far`).
-template <bool FAR, bool ANY>
+template <bool FAR, int ORDER>
 __device__ __forceinline__ float attn_row_sum(uint32_t line, bool far, int m) {
     const auto add = [](float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; };
     const auto at = [&](int q) { return ld_shared_v4f(line + 16u * (uint32_t)q); };
     float4 x[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) x[q] = at(q);
-    if (ANY && m < 4) {
+    if (ORDER == ORDER_EIGHT) m = 2;
+    if (ORDER == ORDER_EIGHT || (ORDER == ORDER_ANY && m < 4)) {
         // (m = 2: two shares of every second group; m = 1: one of all)
         const auto odd = [&](const float4& v) { if (m == 1) add(x[0], v); else add(x[1], v); };
         if (m == 1) add(x[0], x[1]);
 #pragma unroll
         for (int q = 2; q < 8; q += 2) { add(x[0], x[q]); odd(x[q + 1]); }
 #pragma unroll 1
-        for (int q = 8; q < (far ? 16 : 8); q += 2) { add(x[0], at(q)); odd(at(q + 1)); }
+        for (int q = 8; q < (FAR && far ? 16 : 8); q += 2) { add(x[0], at(q)); odd(at(q + 1)); }
         if (m == 2) add(x[0], x[1]);
     } else {
         if (FAR && far && m == 8) {
@@ -106,7 +108,7 @@ __device__ __forceinline__ float attn_row_sum(uint32_t line, bool far, int m) {
 __device__ __forceinline__ void attn_meet(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 __device__ __forceinline__ void attn_report(int id, int threads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
-template <bool FAR, bool ANY>
+template <bool FAR, int ORDER>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                     const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ AttnArgs g) {
@@ -177,7 +179,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
             if (ok) {
                 tc_fence_after();
                 const uint32_t a0 = lo + ((q_s & 0x3FFFFu) >> 4), b0 = lo + ((k_s & 0x3FFFFu) >> 4), b_atom = (uint32_t)g.n16 * 8u;
-                attn_steps<ANY>(tmem_base, (uint32_t)g.n_blocks * 32u, g.s_accs, g.s_per, g.d_steps, [&](uint32_t d, int k8, uint32_t accumulate) {
+                attn_steps<ORDER>(tmem_base, (uint32_t)g.n_blocks * 32u, g.s_accs, g.s_per, g.d_steps, [&](uint32_t d, int k8, uint32_t accumulate) {
                     const uint32_t at = (uint32_t)k8 >> 2, in = 2u * ((uint32_t)k8 & 3u);
                     mma_tf32(d, ((uint64_t)hi << 32) | (uint64_t)(a0 + at * (kAttnAtom >> 4) + in), ((uint64_t)hi << 32) | (uint64_t)(b0 + at * b_atom + in), g.idesc_s, accumulate);
                 });
@@ -190,7 +192,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
                 const uint32_t v_hi = (uint32_t)(v0 >> 32);
                 const uint32_t a0 = lo + ((p_s & 0x3FFFFu) >> 4);
                 const uint32_t b0 = (uint32_t)v0 + ((v_s & 0x3FFFFu) >> 4);
-                attn_steps<ANY>(tmem_base + (uint32_t)g.o_col, (uint32_t)g.v_boxes * 32u, g.o_accs, g.o_per, g.n8 >> 3, [&](uint32_t d, int k8, uint32_t accumulate) {
+                attn_steps<ORDER>(tmem_base + (uint32_t)g.o_col, (uint32_t)g.v_boxes * 32u, g.o_accs, g.o_per, g.n8 >> 3, [&](uint32_t d, int k8, uint32_t accumulate) {
                     const uint32_t a = a0 + ((uint32_t)k8 >> 2) * (kAttnAtom >> 4) + 2u * ((uint32_t)k8 & 3u);
                     mma_tf32(d, ((uint64_t)hi << 32) | (uint64_t)a, ((uint64_t)v_hi << 32) | (uint64_t)(b0 + 64u * (uint32_t)k8), g.idesc_o, accumulate);
                 });
@@ -212,7 +214,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
             for (int i = 0; i < kBlocks; ++i) {
                 const int blk = sw + i * kAttnSoftmaxWarps;
                 if (blk >= g.n_blocks) break;            // (warp-uniform)
-                attn_read<ANY>(tmem_base + (uint32_t)(blk * 32), (uint32_t)g.n_blocks * 32u, g.s_accs, v[i]);
+                attn_read<ORDER>(tmem_base + (uint32_t)(blk * 32), (uint32_t)g.n_blocks * 32u, g.s_accs, v[i]);
 #pragma unroll
                 for (int j = 0; j < 32; j += 4)
                     st_shared_v4(sc_s + (uint32_t)blk * kAttnAtom + line + ((((uint32_t)j >> 2) ^ swz) << 4), v[i][j], v[i][j + 1], v[i][j + 2], v[i][j + 3]);
@@ -242,7 +244,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
                 for (int j = 0; j < 32; ++j) v[i][j] = expf(v[i][j] - mx);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) t[j] = (v[i][4 * j] + v[i][4 * j + 1]) + (v[i][4 * j + 2] + v[i][4 * j + 3]);
-                if (ANY && !g.lane_groups) {
+                if (ORDER == ORDER_ANY && !g.lane_groups) {
 #pragma unroll
                     for (int j = 0; j < 32; j += 4)
                         st_shared_v4(p_s + (uint32_t)blk * kAttnAtom + line + ((((uint32_t)j >> 2) ^ swz) << 4), v[i][j], v[i][j + 1], v[i][j + 2], v[i][j + 3]);
@@ -252,7 +254,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
             st_shared_v4(sums + (uint32_t)blk * 32u + 16u, t[4], t[5], t[6], t[7]);
         }
         attn_meet(1, 32 * kAttnSoftmaxWarps);
-        if (ANY && !g.lane_groups) {
+        if (ORDER == ORDER_ANY && !g.lane_groups) {
             // ... or single values, every lane's 4 m apart: the warps add them up, four lanes' at a time
 #pragma unroll 1
             for (int q = sw; q < 8; q += kAttnSoftmaxWarps) {
@@ -266,7 +268,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
             }
             attn_meet(1, 32 * kAttnSoftmaxWarps);
         }
-        const float inv = 1.f / attn_row_sum<FAR, ANY>(sums, far && g.lane_groups, g.lanes4);
+        const float inv = 1.f / attn_row_sum<FAR, ORDER>(sums, far && g.lane_groups, g.lanes4);
 #pragma unroll
         for (int i = 0; i < kBlocks; ++i) {
             const int blk = sw + i * kAttnSoftmaxWarps;
@@ -287,7 +289,7 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
             if (lane == 0) for (unsigned* word : g.status_more) atomicCAS(word, 0u, (unsigned)TT_ERR_TIMEOUT | (20u << 8));
         } else if (sw * 32 < g.dv) {
             float r[32];
-            attn_read<ANY>(tmem_base + (uint32_t)(g.o_col + sw * 32), (uint32_t)g.v_boxes * 32u, g.o_accs, r);
+            attn_read<ORDER>(tmem_base + (uint32_t)(g.o_col + sw * 32), (uint32_t)g.v_boxes * 32u, g.o_accs, r);
             if (row < g.m) {
                 float* y = g.ctx + ((long long)head * g.m + row) * g.dv + sw * 32;
                 const int left = g.dv - sw * 32;         // (a multiple of 4)
@@ -332,10 +334,13 @@ tt_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
 }
 
 cudaError_t launch_attention(const AttnArgs& g, int heads, const void* tmap_q, const void* tmap_k, const void* tmap_v, cudaStream_t st) {
-    static OncePerDevice raised[3];
-    const bool any = g.s_accs > 1 || g.o_accs > 1 || !g.lane_groups || g.lanes4 < 4;
-    const int build = any ? 2 : g.n > 128 ? 1 : 0;
-    const auto kern = any ? tt_attention_kernel<true, true> : g.n > 128 ? tt_attention_kernel<true, false> : tt_attention_kernel<false, false>;
+    typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const AttnArgs);
+    static const Kernel kernels[] = {tt_attention_kernel<false, ORDER_WIDE>, tt_attention_kernel<true, ORDER_WIDE>, tt_attention_kernel<false, ORDER_EIGHT>,
+                                     tt_attention_kernel<true, ORDER_EIGHT>, tt_attention_kernel<true, ORDER_ANY>};
+    static OncePerDevice raised[5];
+    const bool any = g.s_accs > 1 || g.o_accs > 1 || !g.lane_groups || g.lanes4 < 2;
+    const int build = any ? 4 : 2 * (g.lanes4 == 2) + (g.n > 128);
+    const Kernel kern = kernels[build];
     const cudaError_t ready = raised[build]([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit); });
     if (ready != cudaSuccess) return ready;
     CUtensorMap tq, tk, tv;

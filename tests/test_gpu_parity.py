@@ -1578,6 +1578,8 @@ _PLAIN = dict(tile_n=64, tile_k=64, stages=2, mma_m_axis=1)
     (255, 32, dict(_PLAIN, tile_k=8), 32, dict(_PLAIN, tile_k=32, split_k=4), 1),
     (256, 64, _PLAIN, 16, dict(_PLAIN, split_k=4), 1),
     (256, 64, _PLAIN, 32, dict(_PLAIN, acc_split=2), 1),
+    (100, 64, _PLAIN, 8, _PLAIN, 1),
+    (128, 32, _PLAIN, 8, _PLAIN, 1),
     (129, 64, _PLAIN, 2, _PLAIN, 3),                                                                       # rows of two lanes
     (96, 64, _PLAIN, 16, dict(_PLAIN, tile_k=32, split_k=2, acc_split=2), 3),                               # splits of two accumulators
 ])
